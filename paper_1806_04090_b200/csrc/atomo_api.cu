@@ -38,12 +38,13 @@ struct TableWays {
 struct atomo_ctx {
   int device = 0;
   TableWays tab_sp, tab_dec, tab_avg;
-  TableCache tab_ew;
   int64_t table_uploads = 0, table_reuses = 0;
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
   uint32_t* h_flag = nullptr;        // pinned: convergence flag / state mirror
-  EwState* h_state = nullptr;        // pinned
+  EwLqPart* h_lq = nullptr;          // pinned: results of the l_q sums, written by the GPU
+  uint32_t* ew_words = nullptr;      // device: two sets of barrier counters of the entry-wise encode, the ticket of the l_q sums
+  int ew_set = 0;                    // the set the next launch takes (each launch zeroes the other one)
   cudaEvent_t ev_sync = nullptr;
   // stage timers: one set of events per API call, a ring of kEvRing sets (a set is read out -- its call is long
   // finished by then -- before it is used again), sums since profiling was switched on
@@ -94,6 +95,9 @@ int fail_cuda(atomo_ctx* ctx, cudaError_t e, const char* what) {
   ctx->err = std::string(what) + ": " + cudaGetErrorString(e);
   return ATOMO_ERR_CUDA;
 }
+constexpr int kLqResults = 64;                                 // vectors per round of the l_q sums
+constexpr int kEwSetWords = kEwBatch * kEwBarrierStride;
+constexpr int kEwWords = 2 * kEwSetWords + 32;
 #define CK(call)                                                            \
   do {                                                                      \
     cudaError_t e__ = (call);                                               \
@@ -252,6 +256,29 @@ uint64_t layout_entrywise(const int64_t* n, int n_vecs, int64_t k_cap, bool comp
   return align_up(off, 16);
 }
 
+// The vectors of an entry-wise decode in launches of up to kEwBatch of them (one tile per CTA); returns their number
+template <typename F>
+int for_each_ew_decode(const uint8_t* payload, const int64_t* cols, float* const* out, int n_layers, F launch) {
+  const int tile = ew_tile_elems();
+  auto fill = [&](auto& B, int first, int count) {
+    uint32_t tiles = 0;
+    for (int i = 0; i < count; ++i) {
+      B.v[i] = EwDecode{out[first + i], cols[first + i], first + i, tiles};
+      tiles += (uint32_t)((cols[first + i] + tile - 1) / tile);
+    }
+    B.n = count; B.payload = payload;
+    launch(B, tiles);
+  };
+  int n_launch = 0;
+  for (int l = 0; l < n_layers; ++n_launch) {
+    // a vector has fewer than 2^20 tiles, so a batch stays far below the grid limit
+    const int count = std::min(n_layers - l, kEwBatch);
+    if (count == 1) { EwDecodeBatch<1> B{}; fill(B, l, 1); } else { EwDecodeBatch<kEwBatch> B{}; fill(B, l, count); }
+    l += count;
+  }
+  return n_launch;
+}
+
 bool bad_budget(double s) { return !(s > 0.0) || !std::isfinite(s); }
 
 }  // namespace
@@ -265,11 +292,14 @@ int atomo_create(atomo_ctx** out, int device) {
   *out = ctx;
   CK(cudaSetDevice(device));
   CK(cudaMallocHost(&ctx->h_flag, 256));
-  CK(cudaMallocHost(&ctx->h_state, sizeof(EwState)));
+  CK(cudaMallocHost(&ctx->h_lq, kLqResults * sizeof(EwLqPart)));
+  CK(cudaMalloc(&ctx->ew_words, kEwWords * sizeof(uint32_t)));
+  CK(cudaMemset(ctx->ew_words, 0, kEwWords * sizeof(uint32_t)));
   CK(cudaEventCreateWithFlags(&ctx->ev_sync, cudaEventDisableTiming));
   for (int r = 0; r < atomo_ctx::kEvRing; ++r)
     for (int i = 0; i < ATOMO_N_STAGES; ++i) { CK(cudaEventCreate(&ctx->ev[r][i][0])); CK(cudaEventCreate(&ctx->ev[r][i][1])); }
-  const int e = sp_configure();
+  int e = sp_configure();
+  if (e == 0) e = ew_configure();
   if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaFuncSetAttribute(max dynamic shared memory)");
   ctx->tc_ok = sp_tc_configure() == 0;
   ctx->configured = true;
@@ -281,9 +311,10 @@ int atomo_destroy(atomo_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
   if (ctx->ws) cudaFree(ctx->ws);
-  table_free(ctx->tab_sp); table_free(ctx->tab_dec); table_free(ctx->tab_avg); table_free(ctx->tab_ew);
+  if (ctx->ew_words) cudaFree(ctx->ew_words);
+  table_free(ctx->tab_sp); table_free(ctx->tab_dec); table_free(ctx->tab_avg);
   if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
-  if (ctx->h_state) cudaFreeHost(ctx->h_state);
+  if (ctx->h_lq) cudaFreeHost(ctx->h_lq);
   if (ctx->ev_sync) cudaEventDestroy(ctx->ev_sync);
   for (int r = 0; r < atomo_ctx::kEvRing; ++r)
     for (int i = 0; i < ATOMO_N_STAGES; ++i) for (int j = 0; j < 2; ++j) if (ctx->ev[r][i][j]) cudaEventDestroy(ctx->ev[r][i][j]);
@@ -729,7 +760,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     put(d_given, ptrs.data(), ptrs.size() * sizeof(const float*));
   }
   { const int rc = table_commit(ctx, tab, tables.data(), table_bytes, st); if (rc != ATOMO_OK) return rc; }
-  launch_sp_begin(pay, gh, d_hdr_tmpl, n_layers, d_flag, nullptr, 0, st);          // payload header, layer headers, flags
+  launch_sp_begin(pay, gh, d_hdr_tmpl, n_layers, d_flag, st);          // payload header, layer headers, flags
   CK(cudaMemsetAsync(zero_beg, 0, zero_bytes, st));
 
   // ---- S1: Gram matrix, scaling ----
@@ -916,124 +947,123 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs
   atomo_layer_header* d_hdr = reinterpret_cast<atomo_layer_header*>(pay + sizeof(atomo_payload_header));
   const int tile = ew_tile_elems();
 
+  // Launches: runs of consecutive vectors (at most kEwBatch, their chunks one wave of resident CTAs) go through one
+  // launch of the one-kernel form; a vector too long for that takes the two-kernel form on its own.
+  struct Run { int first, count, solve_ctas; bool list; };       // solve_ctas > 0: two-kernel form
+  std::vector<Run> runs;
   std::vector<EwVec> V(n_vecs);
-  std::vector<char> fused(n_vecs, 0);
-  size_t need = 0;
-  uint8_t* ew_zero_beg = nullptr; size_t ew_zero_bytes = 0;
-  const int max_blocks = ew_solve_max_blocks();
-  if (max_blocks <= 0) return fail_cuda(ctx, cudaGetLastError(), "occupancy query for the cooperative solve");
+  const bool want_list = ctx->ew_launch == 0 && !(dbg && dbg->prob);   // asking for the probabilities means a second read
+  for (int l = 0; l < n_vecs; ++l) {
+    EwVec& v = V[l];
+    v = EwVec{};
+    v.g = vecs[l].data; v.n = vecs[l].n; v.n_tiles = (v.n + tile - 1) / tile;
+    v.pay = pay; v.hdr = d_hdr + l;
+    v.off_idx = lay[l].off_idx; v.off_val = lay[l].off_val; v.off_tiles = lay[l].off_tiles; v.off_sat = lay[l].off_sat;
+    v.layer = (uint32_t)l; v.k_cap = lay[l].kc; v.sat_cap = lay[l].sc; v.compact = compact ? 1 : 0;
+  }
+  auto two_kernels = [&](int l) {
+    const int ctas = ew_solve_ctas(V[l].n_tiles);
+    V[l].n_ctas = std::max(ctas, ew_pack_ctas(V[l].n_tiles));    // what the workspace has to hold
+    V[l].candidates = 0;
+    return ctas;
+  };
+  for (int l = 0; l < n_vecs;) {
+    int count = ctx->ew_launch == 1 ? 0 : std::min(n_vecs - l, kEwBatch);
+    bool list = want_list;
+    for (; count > 0; --count) {
+      if (list && ew_plan(&V[l], count, true) > 0) break;
+      if (ew_plan(&V[l], count, false) > 0) { list = false; break; }   // longer chunks fit without the list's slots
+    }
+    if (count == 0) {
+      const int ctas = two_kernels(l);
+      if (ctas <= 0) return fail_cuda(ctx, cudaGetLastError(), "occupancy query for the cooperative solve");
+      runs.push_back({l, 1, ctas, false});
+      ++l;
+      continue;
+    }
+    if (list) {
+      list = false;
+      for (int i = l; i < l + count; ++i) {
+        V[i].candidates = V[i].n_tiles > V[i].n_ctas && ew_list_pays(V[i].n, V[i].n_tiles, V[i].n_ctas, s) ? 1 : 0;
+        list |= V[i].candidates != 0;
+      }
+      if (!list && ew_plan(&V[l], count, false) == 0) return fail_cuda(ctx, cudaErrorInvalidConfiguration, "entry-wise launch plan");
+    }
+    runs.push_back({l, count, 0, list});
+    l += count;
+  }
   for (int pass = 0; pass < 2; ++pass) {
     Arena A(pass ? ctx->ws : nullptr);
     size_t dbg_atoms = 0, dbg_words = 0;
     for (int l = 0; l < n_vecs; ++l) {
       EwVec& v = V[l];
-      v.g = vecs[l].data; v.n = vecs[l].n; v.layer = (uint32_t)l; v.k_cap = lay[l].kc;
-      v.n_tiles = (v.n + tile - 1) / tile;
-      int fused_ctas = 0;
-      v.candidates = 0;
-      if (ctx->ew_launch != 1) {
-        // the one-kernel form, with the candidate list where the caller does not ask for the probabilities and the
-        // budget is small enough for the list to pay
-        const bool want_list = ctx->ew_launch == 0 && !(dbg && dbg->prob);
-        const int with_list = want_list ? ew_encode_ctas(v.n_tiles, compact, true) : 0;
-        if (with_list > 0 && ew_list_pays(v.n, v.n_tiles, with_list, s)) { fused_ctas = with_list; v.candidates = 1; }
-        else fused_ctas = ew_encode_ctas(v.n_tiles, compact, false);
-      }
-      fused[l] = fused_ctas > 0;
-      v.n_ctas = fused[l] ? fused_ctas : ew_sample_pack_ctas(v.n_tiles, compact);
-      v.compact = compact ? 1 : 0; v.sat_cap = lay[l].sc;
-      v.ent = reinterpret_cast<uint16_t*>(pay + lay[l].off_idx);
-      v.sat_idx = reinterpret_cast<uint32_t*>(pay + lay[l].off_sat);
-      v.sat_val = reinterpret_cast<float*>(pay + lay[l].off_val);
       const int64_t n_words = (v.n + 31) / 32;
       const bool want_mask = dbg && dbg->mask_words;           // the mask words leave the kernel only when asked for
       v.n_words = want_mask ? n_words : 0;
-      const int64_t want_chunks = std::min<int64_t>(max_blocks, (v.n + 4095) / 4096);
-      v.chunk = (int64_t)align_up((uint64_t)((v.n + want_chunks - 1) / want_chunks), 4);
-      v.n_chunks = (int)((v.n + v.chunk - 1) / v.chunk);
-      v.hdr = d_hdr + l;
-      v.idx = reinterpret_cast<uint32_t*>(pay + lay[l].off_idx);
-      v.val = reinterpret_cast<float*>(pay + lay[l].off_val);
-      v.tile_table = reinterpret_cast<uint32_t*>(pay + lay[l].off_tiles);
-      v.partials = A.take<EwPartial>((size_t)3 * std::max(v.n_chunks, v.n_ctas));
-      v.state = A.take<EwState>(1);
       v.mask_words = want_mask ? dbg->mask_words + dbg_words : nullptr;
       v.prob_out = (dbg && dbg->prob) ? dbg->prob + dbg_atoms : nullptr;
       dbg_atoms += v.n; dbg_words += n_words;
+      v.partials = A.take<EwPartial>((size_t)3 * v.n_ctas);
+      v.state = A.take<EwState>(1);
+      v.chunk_status = A.take<uint64_t>((size_t)std::max(v.n_ctas, ew_pack_ctas(v.n_tiles)));
+      v.ticket = A.take<uint32_t>(1);
     }
-    // zero-filled per call: look-back status words and tile tickets of all vectors, one contiguous region
-    uint8_t* zb = reinterpret_cast<uint8_t*>(A.take<uint32_t>(0));
-    const size_t z0 = A.off;
-    for (int l = 0; l < n_vecs; ++l) { V[l].tile_status = A.take<uint64_t>(V[l].n_ctas); V[l].ticket = A.take<uint32_t>(1); }
-    ew_zero_beg = zb; ew_zero_bytes = A.off - z0;
-    need = A.off + 256;
-    if (pass == 0) { const int rc = ensure_ws(ctx, need); if (rc != ATOMO_OK) return rc; }
+    if (pass == 0) { const int rc = ensure_ws(ctx, A.off + 256); if (rc != ATOMO_OK) return rc; }
   }
 
-  atomo_payload_header gh{};
+  EwBegin begin{};
+  begin.on = 1;
+  atomo_payload_header& gh = begin.gh;
   gh.magic = ATOMO_MAGIC; gh.version = ATOMO_VERSION; gh.kind = ATOMO_KIND_ENTRYWISE; gh.n_layers = (uint32_t)n_vecs;
   gh.total_bytes = total; gh.seed = seed; gh.step = step; gh.s = s;
   gh.ew_format = (uint64_t)ctx->ew_format; gh.ew_sat_cap = compact ? (uint64_t)ctx->ew_sat_cap : 0;
-  {
-    // layer header templates through the table cache; the headers themselves are written by a kernel
-    std::vector<atomo_layer_header> tmpl(n_vecs);
-    for (int l = 0; l < n_vecs; ++l) {
-      atomo_layer_header h{};
-      h.rows = 1; h.cols = ns[l]; h.k_cap = lay[l].kc; h.status = ATOMO_OK;
-      h.off_idx = lay[l].off_idx; h.off_val = lay[l].off_val; h.off_short = lay[l].off_tiles;
-      h.off_long = compact ? lay[l].off_sat : 0;
-      tmpl[l] = h;
-    }
-    const size_t tb = tmpl.size() * sizeof(atomo_layer_header);
-    { const int rc = table_reserve(ctx, ctx->tab_ew, tb); if (rc != ATOMO_OK) return rc; }
-    { const int rc = table_commit(ctx, ctx->tab_ew, reinterpret_cast<const uint8_t*>(tmpl.data()), tb, st); if (rc != ATOMO_OK) return rc; }
-  }
-  // ... and the look-back status words and tickets of the sample / pack kernels start at zero.  A call with one vector
-  // in the one-kernel form does all of this inside that kernel: one launch less.
-  auto begin = [&]() {
-    launch_sp_begin(pay, gh, reinterpret_cast<const atomo_layer_header*>(ctx->tab_ew.d), n_vecs, nullptr,
-                    reinterpret_cast<uint32_t*>(ew_zero_beg), (int64_t)((ew_zero_bytes + 3) / 4), st);
+  auto fill = [&](auto& B, int first, int count) {
+    uint32_t* const set = ctx->ew_words + ctx->ew_set * kEwSetWords;
+    for (int i = 0; i < count; ++i) { B.v[i] = V[first + i]; B.v[i].barrier = set + i * kEwBarrierStride; }
+    B.n = count; B.s = s; B.key = philox_round_keys(PhiloxKey{(uint32_t)seed, (uint32_t)(seed >> 32)});
+    B.kind_step = kind_step_word(ATOMO_KIND_ENTRYWISE, step);
+    B.begin = begin; B.begin.on = first == 0 ? 1 : 0;
+    ctx->ew_set ^= 1;
+    B.next_barriers = ctx->ew_words + ctx->ew_set * kEwSetWords;
   };
-  const bool begin_inside = n_vecs == 1 && fused[0];
-  EwBegin eb{};
-  eb.pay = pay; eb.tmpl = reinterpret_cast<const atomo_layer_header*>(ctx->tab_ew.d); eb.gh = gh; eb.on = begin_inside ? 1 : 0;
-  if (!begin_inside) begin();
-
-  const PhiloxKey key{(uint32_t)seed, (uint32_t)(seed >> 32)};
-  const uint32_t ks = kind_step_word(ATOMO_KIND_ENTRYWISE, step);
-  // probabilities: one cooperative launch per vector (pass 1 and the water-filling rounds); a vector that fits one
-  // wave of resident chunks goes on to sampling and packing inside the same launch (timed with the pack stage)
-  int n_two = 0, n_one = 0;
-  stage_begin(ctx, ATOMO_STAGE_EW_REDUCE, st);
-  for (int l = 0; l < n_vecs; ++l) {
-    if (fused[l]) continue;
-    const int e = launch_ew_solve(V[l], s, st);
-    if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(ew_solve)");
-    ++n_two;
-  }
-  stage_end(ctx, ATOMO_STAGE_EW_REDUCE, st, n_two);
-  stage_begin(ctx, ATOMO_STAGE_EW_PACK, st);
-  for (int l = 0; l < n_vecs; ++l) {
-    if (!fused[l]) { launch_ew_sample_pack(V[l], key, ks, st); continue; }
-    const int e = launch_ew_encode(V[l], s, key, ks, eb, st);
-    if (e == (int)cudaErrorCooperativeLaunchTooLarge) {
-      // fewer CTAs fit the GPU at once than the occupancy query promised: the two-kernel form takes the same chunks
-      cudaGetLastError();
-      fused[l] = 0;
-      if (begin_inside) begin();
-      const int e2 = launch_ew_solve(V[l], s, st);
-      if (e2 != 0) return fail_cuda(ctx, (cudaError_t)e2, "cudaLaunchCooperativeKernel(ew_solve)");
-      launch_ew_sample_pack(V[l], key, ks, st);
-      n_one += 2;
-      continue;
-    }
-    if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(ew_encode)");
-    ++n_one;
-  }
-  stage_end(ctx, ATOMO_STAGE_EW_PACK, st, (int64_t)(n_two + n_one));
-  CK(cudaGetLastError());
+  auto run_two = [&](int l, int solve_ctas) {
+    EwBatch<1> B{};
+    fill(B, l, 1);
+    return launch_ew_two_kernels(B, solve_ctas, ew_pack_ctas(V[l].n_tiles), st);
+  };
   ctx->ew_last_state.resize(n_vecs); ctx->ew_last_chunks.resize(n_vecs);
-  for (int l = 0; l < n_vecs; ++l) { ctx->ew_last_state[l] = V[l].state; ctx->ew_last_chunks[l] = fused[l] ? V[l].n_ctas : 0; }
+  for (int l = 0; l < n_vecs; ++l) { ctx->ew_last_state[l] = V[l].state; ctx->ew_last_chunks[l] = V[l].n_ctas; }
+  int64_t n_launch = 0;
+  stage_begin(ctx, ATOMO_STAGE_EW_PACK, st);
+  for (const Run& r : runs) {
+    int e = 0;
+    if (r.solve_ctas > 0) {
+      e = run_two(r.first, r.solve_ctas);
+      ctx->ew_last_chunks[r.first] = 0;
+      n_launch += 2;
+    } else {
+      if (r.count == 1) { EwBatch<1> B{}; fill(B, r.first, 1); e = launch_ew_encode(B, r.list, st); }
+      else { EwBatch<kEwBatch> B{}; fill(B, r.first, r.count); e = launch_ew_encode(B, r.list, st); }
+      ++n_launch;
+      if (e == (int)cudaErrorCooperativeLaunchTooLarge) {
+        // fewer CTAs fit the GPU at once than the occupancy query promised: the two-kernel form, vector by vector (the
+        // launch that did not happen zeroed no counters)
+        cudaGetLastError();
+        CK(cudaMemsetAsync(ctx->ew_words, 0, 2 * kEwSetWords * sizeof(uint32_t), st));
+        e = 0;
+        for (int l = r.first; l < r.first + r.count && e == 0; ++l) {
+          V[l].candidates = 0;
+          const int ctas = std::min(ew_solve_ctas(V[l].n_tiles), V[l].n_ctas);   // the workspace was carved for that many
+          e = ctas > 0 ? run_two(l, ctas) : (int)cudaErrorCooperativeLaunchTooLarge;
+          ctx->ew_last_chunks[l] = 0;
+          n_launch += 2;
+        }
+      }
+    }
+    if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "launch of the entry-wise encode");
+  }
+  stage_end(ctx, ATOMO_STAGE_EW_PACK, st, n_launch);
+  CK(cudaGetLastError());
   return ATOMO_OK;
 }
 
@@ -1064,39 +1094,40 @@ int atomo_lq_budget(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs, doubl
   }
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
-  const int n_ctas = 148 * 8;
-  double* d_sum = nullptr; float* d_max = nullptr;
+  const int max_ctas = 148 * 8;
+  EwLqPart* d_part = nullptr;
   for (int pass = 0; pass < 2; ++pass) {
     Arena A(pass ? ctx->ws : nullptr);
-    d_sum = A.take<double>(n_ctas);
-    d_max = A.take<float>(n_ctas);
+    d_part = A.take<EwLqPart>(max_ctas);
     if (pass == 0) { const int rc = ensure_ws(ctx, A.off + 256); if (rc != ATOMO_OK) return rc; }
   }
-  std::vector<double> h_sum(n_ctas);
-  std::vector<float> h_max(n_ctas);
-  for (int l = 0; l < n_vecs; ++l) {
-    launch_ew_lq(vecs[l].data, vecs[l].n, 0, q, 0.0, d_sum, d_max, n_ctas, st);
-    CK(cudaMemcpyAsync(h_sum.data(), d_sum, n_ctas * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(h_max.data(), d_max, n_ctas * sizeof(float), cudaMemcpyDeviceToHost, st));
+  uint32_t* const ticket = ctx->ew_words + 2 * kEwSetWords;
+  // the sums of up to kLqResults vectors arrive in pinned memory; one wait for all of them
+  for (int l0 = 0; l0 < n_vecs; l0 += kLqResults) {
+    const int n = std::min(n_vecs - l0, kLqResults);
+    for (int i = 0; i < n; ++i) launch_ew_lq(vecs[l0 + i].data, vecs[l0 + i].n, 0, q, 0.0, d_part, ticket, ctx->h_lq + i, max_ctas, st);
+    CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));
-    double l1 = 0.0, amax = 0.0;
-    for (int i = 0; i < n_ctas; ++i) { l1 += h_sum[i]; amax = std::max(amax, (double)h_max[i]); }
-    if (!(amax <= 3.0e38) || !(l1 == l1)) { s_out[l] = std::nan(""); continue; }
-    if (amax == 0.0) { s_out[l] = 0.0; continue; }
-    double norm_q;
-    if (std::isinf(q)) norm_q = amax;
-    else if (q == 1.0) norm_q = l1;
-    else {
-      launch_ew_lq(vecs[l].data, vecs[l].n, 1, q, 1.0 / amax, d_sum, d_max, n_ctas, st);
-      CK(cudaMemcpyAsync(h_sum.data(), d_sum, n_ctas * sizeof(double), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      double t = 0.0;
-      for (int i = 0; i < n_ctas; ++i) t += h_sum[i];
-      norm_q = amax * std::pow(t, 1.0 / q);
+    bool more = false;
+    std::vector<double> l1(n), amax(n);
+    for (int i = 0; i < n; ++i) {
+      const EwLqPart r = ctx->h_lq[i];
+      l1[i] = r.sum; amax[i] = r.amax;
+      double& out = s_out[l0 + i];
+      if (!(r.amax <= 3.0e38) || !(r.sum == r.sum)) { out = std::nan(""); l1[i] = -1.0; }
+      else if (r.amax == 0.0) { out = 0.0; l1[i] = -1.0; }
+      else if (std::isinf(q)) out = r.sum / r.amax;
+      else if (q == 1.0) out = 1.0;
+      else if (q == 2.0) out = r.sum / std::sqrt(r.sq);
+      else { launch_ew_lq(vecs[l0 + i].data, vecs[l0 + i].n, 1, q, 1.0 / r.amax, d_part, ticket, ctx->h_lq + i, max_ctas, st); more = true; continue; }
+      l1[i] = -1.0;
     }
-    s_out[l] = l1 / norm_q;
+    if (!more) continue;
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(st));
+    for (int i = 0; i < n; ++i)
+      if (l1[i] >= 0.0) s_out[l0 + i] = l1[i] / (amax[i] * std::pow(ctx->h_lq[i].sum, 1.0 / q));
   }
-  CK(cudaGetLastError());
   return ATOMO_OK;
 }
 
@@ -1110,16 +1141,12 @@ int atomo_decode(atomo_ctx* ctx, int32_t kind, const void* payload, const int64_
   cudaStream_t st = (cudaStream_t)stream;
   stage_reset(ctx);
   const uint8_t* pay = static_cast<const uint8_t*>(payload);
-  const atomo_payload_header* d_gh = reinterpret_cast<const atomo_payload_header*>(pay);
   const atomo_layer_header* d_hdr = reinterpret_cast<const atomo_layer_header*>(pay + sizeof(atomo_payload_header));
   stage_begin(ctx, ATOMO_STAGE_DECODE, st);
   if (kind == ATOMO_KIND_ENTRYWISE) {
-    for (int l = 0; l < n_layers; ++l) {
-      if (rows[l] != 1) return ATOMO_ERR_INVALID_ARG;
-      EwDecode d{pay, d_gh, d_hdr + l, out[l], cols[l]};
-      launch_ew_decode(d, st);
-    }
-    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_layers);
+    for (int l = 0; l < n_layers; ++l) if (rows[l] != 1) return ATOMO_ERR_INVALID_ARG;
+    const int n_launch = for_each_ew_decode(pay, cols, out, n_layers, [&](const auto& B, uint32_t tiles) { launch_ew_decode(B, tiles, st); });
+    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   } else {
     std::vector<SpDecodeLayer> D(n_layers);
     std::vector<TileRef> tiles;
@@ -1202,8 +1229,10 @@ int atomo_decode_average(atomo_ctx* ctx, int32_t kind, const void* const* payloa
     launch_sp_decode_average(d_pay, n_payloads, d_layers, d_tiles, (int)tiles.size(), st);
     stage_end(ctx, ATOMO_STAGE_DECODE, st, 1);
   } else {
-    for (int l = 0; l < n_layers; ++l) launch_ew_decode_average(d_pay, n_payloads, l, out[l], cols[l], st);
-    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_layers);
+    const int n_launch = for_each_ew_decode(nullptr, cols, out, n_layers, [&](const auto& B, uint32_t n_tiles) {
+      launch_ew_decode_average(B, n_tiles, d_pay, n_payloads, st);
+    });
+    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   }
   CK(cudaGetLastError());
   return ATOMO_OK;

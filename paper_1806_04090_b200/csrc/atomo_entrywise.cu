@@ -1,49 +1,45 @@
 // Entry-wise ATOMO on flat gradients: atoms e_i, lambda_i = g_i (Section 3 of the paper; the
 // QSGD / TernGrad family of Section 4 are the budgets s = ||g||_1/||g||_2 and ||g||_1/||g||_inf).
 //
-//   ew_solve (cooperative)     : pass 1: ||g||_1 (fp64 accumulation), ||g||_inf, non-finite scan; then the
-//                                water-filling form of Algorithm 1 -- every atom with
-//                                |g_i| (s - n_s) > sum_{unsaturated} |g_j| gets p = 1; repeated
-//                                until no new atom saturates (zero rounds when g is s-balanced,
-//                                Lemma 3); grid barriers instead of host round trips
-//   pass 2   ew_sample_pack    : per chunk of tiles: p_i = |g_i| (s-n_s)/T, Philox word, keep bit -> mask words
-//                                and counts; the counts of the earlier chunks are added (one bounded wait, no
-//                                chain); ordered compaction from the mask words: idx ascending, val = g_i / p_i;
-//                                the last chunk writes k, the capacity check and the header.  Compact format
-//                                (the ternary form of Section 4): a kept atom with p < 1 weighs sign(g_i) c, so
-//                                it travels as a 16-bit entry (index inside its tile, sign bit); the atoms with
-//                                p = 1 keep (idx, val) in a list of their own
-//   decode   ew_decode         : zero-fill with vector stores, then the tile's kept values (per-tile
-//                                offsets travel in the payload), either format
+//   ew_encode (cooperative)    : all vectors of a call (up to kEwBatch) in one launch; a CTA owns a chunk of consecutive
+//                                tiles of one vector.
+//     pass 1                     ||g||_1 (fp64 accumulation), ||g||_inf, non-finite scan; then the water-filling form
+//                                of Algorithm 1 -- every atom with |g_i| (s - n_s) > sum_{unsaturated} |g_j| gets
+//                                p = 1; repeated until no new atom saturates (zero rounds when g is s-balanced,
+//                                Lemma 3).  The CTAs of a vector meet at a barrier of their own.
+//     pass 2                     p_i = |g_i| (s-n_s)/T, Philox word, keep decision -> code bytes in shared memory; the
+//                                counts of the earlier chunks are added (one bounded wait, no chain); ordered
+//                                compaction from the code bytes: idx ascending, val = g_i / p_i; the last chunk writes
+//                                k, the capacity check and the header.  Compact format (the ternary form of Section 4):
+//                                a kept atom with p < 1 weighs sign(g_i) c, so it travels as a 16-bit entry (index
+//                                inside its tile, sign bit); the atoms with p = 1 keep (idx, val) in a list of their own
+//   ew_solve + ew_sample_pack  : the same two passes as two kernels, for vectors whose code bytes do not fit the shared
+//                                memory of one wave of resident CTAs
+//   ew_decode                  : a tile is put together in shared memory and leaves as one bulk copy, either format
 #include <algorithm>
-
-#include <cooperative_groups.h>
 
 #include "atomo_kernels.cuh"
 
-namespace cg = cooperative_groups;
-
-// development builds (-DEW_PROFILE) print the phase times of a few CTAs of the one-kernel form
-#ifdef EW_PROFILE
-#include <cstdio>
-__device__ __forceinline__ unsigned long long ew_now() { unsigned long long t; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)); return t; }
-#define EW_STAMP(k) if (threadIdx.x == 0) ew_t[k] = ew_now();
-#else
-#define EW_STAMP(k)
-#endif
-
 namespace atomo {
 
-constexpr int kEwThreads = 256;
-constexpr int kEwTile = 4096;                 // elements per tile of the sample / pack / decode passes
-#ifndef EW_MIN_BLOCKS
-#define EW_MIN_BLOCKS 5
-#endif
-constexpr int kEwMinBlocks = EW_MIN_BLOCKS;   // resident CTAs per SM the sample / pack kernel is compiled for
-#ifndef EW_ENCODE_BLOCKS
-#define EW_ENCODE_BLOCKS 4
-#endif
-constexpr int kEwEncodeBlocks = EW_ENCODE_BLOCKS;   // ... and the one-kernel form (64 registers: two tiles' loads per thread)
+namespace {
+
+// One CTA per SM: the warps of an SM share one chunk.  (Four CTAs of 256 threads with a chunk each took as long as the
+// slowest of them: the scheduler favours the oldest warps, so that of four equal chunks on an SM the first was done after 104 us
+// and the last, by then alone with eight warps, after 200.)
+constexpr int kEwThreads = 1024;
+constexpr int kEwWarps = kEwThreads / kWarp;
+constexpr int kEwTile = ATOMO_EW_TILE;        // elements per tile
+constexpr int kEwUnits = 8;                   // units per tile: what a warp takes at a time, 16 atoms per lane
+// The keep decisions of a block of four atoms (one Philox call) are a byte: K_j in bit j, S_j in bit 4 + j.
+// (K, S) = (1, sign bit of g): kept with p < 1; (0, 1): kept with p = 1 (saturated); (0, 0): not kept.
+constexpr int kEwBlocks = kEwTile / 4;        // blocks (code bytes) per tile
+constexpr int kEwPrefixes = kEwTile / 32;     // list form: prefix words per tile
+constexpr int kEwRegTiles = kEwWarps / kEwUnits;   // chunks of at most this many tiles stay in registers: a unit per warp
+constexpr int kEwBig = 8192;                  // entries of the list of runs with atoms that may saturate
+constexpr int kEwStage = 256;                 // kept atoms per staging window (one per warp) of the compaction
+constexpr uint32_t kEwPollLimit = 1u << 22;   // polls of a bounded wait (with a sleep between them)
+constexpr uint64_t kFlagReady = 1ull << 63;
 
 __device__ __forceinline__ float4 load4(const float* __restrict__ g, int64_t i, int64_t n, bool aligned) {
   if (aligned && i + 3 < n) return __ldg(reinterpret_cast<const float4*>(g + i));
@@ -55,238 +51,324 @@ __device__ __forceinline__ float4 load4(const float* __restrict__ g, int64_t i, 
   return v;
 }
 
-// ---- probabilities: one cooperative kernel (pass 1 + water-filling rounds, no host round trip) ----
-// Every CTA owns one contiguous chunk.  After each pass all CTAs meet at a grid barrier and each of them
-// reduces the per-chunk partials in the same fixed order, so every CTA holds the same state and takes the
-// same decision without a broadcast.  Partials are double-buffered: one barrier per pass.
-struct EwAcc { double sum; float amax; uint32_t cnt; uint32_t bad; };
+// The chunk of a CTA: n_my tiles of the vector from tile0 on, elements [beg, end)
+struct EwChunk {
+  int64_t tile0, beg, end;
+  int n_my, n_full, n_units;    // n_full: tiles that lie inside the vector and can be read with 16-byte loads
+  uint32_t index;               // position among the vector's chunks
+  bool aligned;
+};
+__device__ __forceinline__ EwChunk ew_chunk(const EwVec& v, uint32_t index) {
+  EwChunk c;
+  const int64_t q = v.n_tiles / v.n_ctas, rem = v.n_tiles % v.n_ctas;    // the first `rem` chunks have q + 1 tiles
+  c.index = index;
+  c.tile0 = (int64_t)index * q + min((int64_t)index, rem);
+  c.n_my = (int)(q + ((int64_t)index < rem ? 1 : 0));
+  c.beg = c.tile0 * kEwTile;
+  c.end = min(v.n, c.beg + (int64_t)c.n_my * kEwTile);
+  c.aligned = (reinterpret_cast<uintptr_t>(v.g) & 15u) == 0;
+  c.n_full = c.aligned ? (int)((c.end - c.beg) / kEwTile) : 0;
+  c.n_units = c.n_my * kEwUnits;
+  return c;
+}
+// number of a lane's first float4 of a unit inside the chunk; its other three are 256 apart
+__device__ __forceinline__ uint32_t ew_unit_block(int unit) {
+  return (uint32_t)(unit / kEwUnits) * kEwBlocks + (uint32_t)(unit % kEwUnits) * kWarp + threadIdx.x % kWarp;
+}
+// float4 number u = 0 .. 3 of a lane's 16 atoms of a unit; zeros past the end
+__device__ __forceinline__ float4 ew_load_unit(const EwVec& v, const EwChunk& c, int unit, int u) {
+  const int64_t i = c.beg + 4 * (int64_t)ew_unit_block(unit) + 1024 * u;
+  if (unit / kEwUnits < c.n_full) return __ldg(reinterpret_cast<const float4*>(v.g + i));
+  return i < c.end ? load4(v.g, i, c.end, c.aligned) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ void ew_load_unit(const EwVec& v, const EwChunk& c, int unit, float4 (&x)[4]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) x[u] = unit >= 0 && unit < c.n_units ? ew_load_unit(v, c, unit, u) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
 
-template <bool kRound>
-__device__ __forceinline__ EwAcc ew_chunk_pass(const EwVec& v, float theta, const int64_t beg, const int64_t end) {
-  const bool aligned = (reinterpret_cast<uintptr_t>(v.g) & 15u) == 0;
-  EwAcc acc{0.0, 0.0f, 0u, 0u};
-  constexpr int kU = 4;
-  for (int64_t base = beg + (int64_t)threadIdx.x * 4; base < end; base += (int64_t)kEwThreads * 4 * kU) {
-    float4 x[kU];
+// f(blk, x) for the four blocks (blk: number inside the chunk) and end(blk) with the first one's for every unit of the chunk,
+// each warp its own in ascending order.  kAhead units' loads are on their way: a float4's registers are loaded again as soon
+// as it has been used.  Two where the work per unit is small and the pass is bound by HBM; one where it is bound by
+// instruction issue (a second set of registers spilled), and there a barrier every few rounds keeps the warps abreast: left
+// alone the oldest ones run ahead and the last ones end alone.
+template <int kAhead, typename F, typename E>
+__device__ __forceinline__ void ew_for_units(const EwVec& v, const EwChunk& c, float4 (&x)[kAhead][4], F f, E end) {
+  constexpr int kStep = kEwWarps / kEwUnits * kEwBlocks;   // blocks from a warp's unit to its next
+  const int n = c.n_units, n_full = c.n_full * kEwUnits;
+  int unit = (int)(threadIdx.x / kWarp);
+  uint32_t blk = ew_unit_block(unit);
+  const float4* src = reinterpret_cast<const float4*>(v.g + c.beg) + blk + kAhead * kStep;
+  for (int u0 = 0, round = 0; u0 < n; u0 += kAhead * kEwWarps, ++round) {
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {                       // all loads first: kU requests in flight per thread
-      const int64_t i = base + (int64_t)u * kEwThreads * 4;
-      x[u] = i < end ? load4(v.g, i, end, aligned) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    float fsum = 0.0f;                                   // short fp32 run (<= 16 terms), then into fp64
+    for (int h = 0; h < kAhead; ++h) {
+      if (unit < n) {
+        const int next = unit + kAhead * kEwWarps;
+        if (next < n_full) {
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const float a[4] = {fabsf(x[u].x), fabsf(x[u].y), fabsf(x[u].z), fabsf(x[u].w)};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (!kRound) {
-          fsum += a[j];
-          acc.amax = fmaxf(acc.amax, a[j]);
-          acc.bad |= !(a[j] <= 3.402823466e38f);         // NaN or Inf
+          for (int u = 0; u < 4; ++u) { f(blk + (uint32_t)(256 * u), x[h][u]); x[h][u] = __ldg(src + 256 * u); }
         } else {
-          if (a[j] > theta) ++acc.cnt; else fsum += a[j];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) { f(blk + (uint32_t)(256 * u), x[h][u]); if (next < n) x[h][u] = ew_load_unit(v, c, next, u); }
         }
+        end(blk);
       }
+      unit += kEwWarps; blk += kStep; src += kStep;
     }
+    if (kAhead == 1 && (round & 3) == 3) __syncthreads();
+  }
+}
+template <int kAhead>
+__device__ __forceinline__ void ew_load_ahead(const EwVec& v, const EwChunk& c, float4 (&x)[kAhead][4]) {
+#pragma unroll
+  for (int h = 0; h < kAhead; ++h) ew_load_unit(v, c, (int)(threadIdx.x / kWarp) + h * kEwWarps, x[h]);
+}
+
+struct EwAcc { double sum; float amax; uint32_t cnt; };
+
+struct EwShared {                 // static shared memory of the encode and solve kernels
+  double sum[kEwWarps];
+  float mx[kEwWarps], est[kEwWarps];
+  uint32_t cnt[kEwWarps];
+  unsigned long long scan[kEwWarps], before[kEwWarps];
+  uint32_t n_big, stop, fail, next_unit;
+};
+
+// block reduction in a fixed order, result valid in every thread
+__device__ __forceinline__ EwAcc ew_block_reduce(EwAcc a, EwShared& sh) {
+  const int w = threadIdx.x / kWarp, l = threadIdx.x % kWarp;
+  a.sum = warp_sum(a.sum); a.amax = warp_max(a.amax); a.cnt = __reduce_add_sync(0xffffffffu, a.cnt);
+  __syncthreads();
+  if (l == 0) { sh.sum[w] = a.sum; sh.mx[w] = a.amax; sh.cnt[w] = a.cnt; }
+  __syncthreads();
+  return EwAcc{warp_sum(sh.sum[l]), warp_max(sh.mx[l]), __reduce_add_sync(0xffffffffu, sh.cnt[l])};
+}
+// sum of one float per thread, valid in every thread
+__device__ __forceinline__ float ew_block_sum(float x, EwShared& sh) {
+  x = warp_sum(x);
+  if (threadIdx.x % kWarp == 0) sh.est[threadIdx.x / kWarp] = x;
+  __syncthreads();
+  return warp_sum(sh.est[threadIdx.x % kWarp]);
+}
+
+// Barrier among the CTAs of one vector (all resident: cooperative launch).  `target` is the number of arrivals since
+// the counter was zeroed; the wait is bounded and a wait that runs out is reported in the layer's status word.
+__device__ __forceinline__ void ew_barrier(const EwVec& v, uint32_t target, EwShared& sh) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(v.barrier, 1u);
+    uint32_t polls = 0;
+    while (*(volatile uint32_t*)v.barrier < target) {
+      if (++polls > kEwPollLimit) { sh.fail = 1u; break; }
+      __nanosleep(20);
+    }
+    __threadfence();
+  }
+  __syncthreads();
+}
+
+// ---- pass 1 -------------------------------------------------------------------------------------------------------
+// Sums in short fp32 runs (16 terms per lane and unit), then fp64.  amax ignores NaN (and the sum keeps it), so "some
+// entry is NaN" is "the sum is NaN" and "some entry is infinite" is "amax is infinite": no test per entry.
+__device__ __forceinline__ float max4(const float4& x) {
+  return fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w)));
+}
+__device__ __forceinline__ void ew_sums(const float4& x, float& fsum, float& amax) {
+  fsum += fabsf(x.x); fsum += fabsf(x.y); fsum += fabsf(x.z); fsum += fabsf(x.w);
+  amax = fmaxf(amax, max4(x));
+}
+// the warps' first units (x): sum of |g| over them, scaled to the vector
+__device__ __forceinline__ double ew_estimate_l1(const EwVec& v, const EwChunk& c, const float4 (&x)[4], EwShared& sh) {
+  float ts = 0.0f, m = 0.0f;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) ew_sums(x[u], ts, m);
+  ts = ew_block_sum(ts, sh);
+  const double seen = (double)min((int64_t)kEwRegTiles * kEwTile, c.end - c.beg);
+  return (double)ts * (double)v.n / seen;
+}
+// Runs (a lane's 16 atoms of a unit) with an atom above a lower bound of the saturation threshold, listed during pass 1 so
+// that the water-filling rounds read those alone and not the whole vector (a round over 100 million elements costs 65 us,
+// the listed runs of 100 M Laplace entries at s = 10 % are 0.5 % of it).  The bound is 0.8 l1_est / s with l1_est the sum over
+// the chunk's first tiles scaled to the vector; the rounds lower the threshold a little (there: by half a per cent).  A round
+// forms the listed runs anew without the saturated atoms, exactly as a round over the whole chunk would.
+struct EwBigList {
+  uint32_t* run;                // [kEwBig] the run's first block inside the chunk, shared memory
+  float lo;                     // runs with an atom above lo are listed; inf: no list
+  double rest;                  // this thread's sum over the runs not listed
+};
+
+// pass 1 with that list; the caller has zeroed sh.n_big
+__device__ __forceinline__ EwAcc ew_pass_big(const EwVec& v, const EwChunk& c, const double s, EwBigList& B, EwShared& sh) {
+  double sum = 0.0, rest = 0.0;
+  float amax = 0.0f;
+  float4 x[2][4];
+  ew_load_ahead(v, c, x);
+  {
+    const float lo = (float)(0.8 * ew_estimate_l1(v, c, x[0], sh) / s);
+    // a zero or non-finite estimate, or a budget that keeps every atom (threshold 0): no list
+    B.lo = (lo > 0.0f && s < (double)v.n) ? lo : __int_as_float(0x7f800000);
+  }
+  float fsum = 0.0f, m = 0.0f;
+  ew_for_units(v, c, x, [&](uint32_t, const float4& y) { ew_sums(y, fsum, m); }, [&](uint32_t blk) {
+    amax = fmaxf(amax, m);
+    sum += (double)fsum;
+    if (!(m > B.lo)) rest += (double)fsum;
+    else if (*(volatile uint32_t*)&sh.n_big <= (uint32_t)kEwBig) {       // (a list that overflowed is not used: no more appends)
+      const uint32_t at = atomicAdd(&sh.n_big, 1u);
+      if (at < (uint32_t)kEwBig) B.run[at] = blk;
+    }
+    fsum = 0.0f; m = 0.0f;
+  });
+  B.rest = rest;
+  return EwAcc{sum, amax, 0u};
+}
+// one water-filling round over the chunk: unsaturated sum and saturated count at threshold theta, from memory
+__device__ __forceinline__ void ew_round_sums(const float4& x, const float theta, float& fsum, uint32_t& cnt) {
+  const float a[4] = {fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w)};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) { if (a[j] > theta) ++cnt; else fsum += a[j]; }
+}
+__device__ __forceinline__ EwAcc ew_round_memory(const EwVec& v, const EwChunk& c, const float theta) {
+  EwAcc acc{0.0, 0.0f, 0u};
+  float4 x[2][4];
+  ew_load_ahead(v, c, x);
+  float fsum = 0.0f;
+  ew_for_units(v, c, x, [&](uint32_t, const float4& y) { ew_round_sums(y, theta, fsum, acc.cnt); }, [&](uint32_t) { acc.sum += (double)fsum; fsum = 0.0f; });
+  return acc;
+}
+// ... and from the list, where it holds every run with an atom above theta
+__device__ __forceinline__ EwAcc ew_round_list(const EwVec& v, const EwChunk& c, const EwBigList& B, const uint32_t n_big, const float theta) {
+  EwAcc acc{B.rest, 0.0f, 0u};
+  for (uint32_t i = threadIdx.x; i < n_big; i += kEwThreads) {
+    const int64_t base = c.beg + 4 * (int64_t)B.run[i];
+    float4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t at = base + (int64_t)u * 1024;
+      x[u] = at < c.end ? load4(v.g, at, c.end, c.aligned) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float fsum = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ew_round_sums(x[u], theta, fsum, acc.cnt);
     acc.sum += (double)fsum;
   }
   return acc;
 }
 
-// block reduction in a fixed order, result valid in every thread
-__device__ __forceinline__ EwAcc ew_block_reduce(EwAcc a, double* s_sum, float* s_max, uint32_t* s_cnt, uint32_t* s_bad) {
-  a.sum = warp_sum(a.sum); a.amax = warp_max(a.amax); a.cnt = warp_sum(a.cnt);
-  a.bad = __any_sync(0xffffffffu, a.bad) ? 1u : 0u;
-  const int w = threadIdx.x / kWarp, l = threadIdx.x % kWarp;
-  __syncthreads();
-  if (l == 0) { s_sum[w] = a.sum; s_max[w] = a.amax; s_cnt[w] = a.cnt; s_bad[w] = a.bad; }
-  __syncthreads();
-  EwAcc r{0.0, 0.0f, 0u, 0u};
-  for (int i = 0; i < kEwThreads / kWarp; ++i) { r.sum += s_sum[i]; r.amax = fmaxf(r.amax, s_max[i]); r.cnt += s_cnt[i]; r.bad |= s_bad[i]; }
-  return r;
-}
-
-// ---- the first pass of the one-kernel form, with a list of candidates --------------------------------------------
+// ---- pass 1 with a list of candidates (small budgets) ----------------------------------------------------------------
 // The keep decision of an atom needs ||g||_1, which only the end of the first pass knows; but the Philox word of an
-// atom depends on its index alone.  So the first pass already draws the words and keeps a list of the few atoms that
-// can still be kept: an atom is kept (Eq. 2 with p < 1) iff word < floor(|g| scale 2^32), and the pass tests
-// word <= |g| M with M = 1.25 scale_est 2^32, where scale_est comes from the sum over the chunk's first tile, scaled to
-// the vector's length.  A thread keeps its candidates (index, value) in slots of its own, so the list needs neither
-// atomics nor votes.  After the grid barrier the true scale is known.  If M >= scale 2^32 (1 + 2^-22) (the slack
-// covers the roundings of both products), the vector is s-balanced (no atom with p = 1) and no thread ran out of
-// slots, the list holds every kept atom of the chunk and the exact decision is taken on its entries alone (their
-// words are drawn again): the chunk is read once.  Otherwise the CTA reads its chunk a second time as the two-kernel form does.  Either way
-// the decision is the same integer comparison on the same operands, so the payload does not depend on which way a
-// chunk went.  The sums are formed exactly as in ew_chunk_pass (same terms per thread, same order).
+// atom depends on its index alone.  So the first pass already draws the words and lists the few blocks of four atoms
+// (one Philox call) that can still hold a kept one: an atom is kept (Eq. 2 with p < 1) iff word < floor(|g| scale 2^32),
+// and the pass tests word <= |g| M with M = 1.25 scale_est 2^32, where scale_est comes from the sum over the chunk's
+// first tiles, scaled to the vector's length.  The test of a block is one fused multiply-add per atom (its sign is exact),
+// a maximum and one predicated store; a thread keeps its blocks in slots of its own, so the list needs neither atomics
+// nor votes.  After the barrier the true scale is known.  If M >= scale 2^32 (1 + 2^-22) (the slack covers the
+// rounding of the decision's product), the vector is s-balanced (no atom with p = 1) and no thread ran out of slots,
+// the list covers every kept atom of the chunk and the exact decision is taken on its blocks alone (their words are
+// drawn and their entries read again, mostly from the L2): the chunk is read once.  Otherwise the CTA reads its chunk
+// a second time.  Either way the decision is the same integer comparison on the same operands, so the payload does not
+// depend on which way a chunk went.
+// Bound: instruction issue (Philox4x32-10 is 40 of about 75 instructions per four atoms).  Listing single atoms with
+// their values, two stores and a test each, took 171 instructions per four atoms and 38 us for the pass over 25.6 M
+// elements.
 constexpr int kEwCandPerThread = 16;             // list entries per thread; 1.25 s (atoms per thread) / n are expected
-constexpr int kEwCandSlots = (kEwCandPerThread + 1) * kEwThreads;   // one more row takes what does not fit (never read)
+constexpr int kEwCandBytes = (kEwCandPerThread + 1) * kEwThreads * 4;   // one more row takes what does not fit (never read)
 struct EwCands {
-  uint32_t* idx;      // [kEwCandPerThread + 1][kEwThreads] atom index inside the chunk, then (same layout) its gradient entry
-  uint32_t* stop;     // set by the first thread that runs out of slots: the CTA stops listing
+  uint32_t* blk;      // [kEwCandPerThread + 1][kEwThreads] Philox blocks
   float m32;          // the multiplier M the list was made with (0: no list)
   uint32_t addr;      // shared-memory address of this thread's next slot: rows of kEwThreads 4-byte entries
   uint32_t addr0;     // ... of its first slot
 };
 __device__ __forceinline__ uint32_t ew_cand_count(const EwCands& C) { return (C.addr - C.addr0) / (4u * kEwThreads); }
 
-// One tile of the pass: 16 atoms per thread (float4 number tid + 256 u of the tile, u = 0 .. 3).  local0: index of
-// x[0].x inside the chunk; blk0: its Philox block (atom index / 4); left: elements of the chunk from x[0].x on
-// (FULL: the whole tile lies inside the chunk).  amax ignores NaN (and the sum keeps it), so "some entry is NaN" is
-// "the sum is NaN" and "some entry is infinite" is "amax is infinite": no test per entry.
-template <bool FULL>
-__device__ __forceinline__ void ew_cand_tile(const float4 (&x)[4], const uint32_t local0, const uint32_t blk0, const int64_t left,
-                                             const uint32_t layer, const PhiloxKey key, const uint32_t kind_step,
-                                             const bool listing, float& fsum, float& amax, EwCands& C) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const float a[4] = {fabsf(x[u].x), fabsf(x[u].y), fabsf(x[u].z), fabsf(x[u].w)};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      fsum += a[j];
-      amax = fmaxf(amax, a[j]);
-    }
-  }
-  if (!listing) return;
+// one block (blk: its Philox block, atom / 4); entries past the chunk's end are zeros, which are listed only where the word is
+// zero (and the exact decision drops them)
+__device__ __forceinline__ void ew_cand_block(const float4& x, const uint32_t blk, const uint32_t layer,
+                                              const PhiloxRoundKeys& key, const uint32_t kind_step, EwCands& C) {
   const float m32 = C.m32;
   const uint32_t spill = C.addr0 + (uint32_t)(kEwCandPerThread * kEwThreads * 4);   // this thread's slot in the extra row
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (!FULL && (int64_t)u * kEwThreads * 4 >= left) continue;
-    const uint4 wd = philox4x32_10(make_uint4(blk0 + (uint32_t)(u * kEwThreads), 0u, layer, kind_step), key);
-    const float gg[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-    const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      // candidate: two predicated stores (index, value) to the thread's next slot and the slot moves on; no branch
-      const uint32_t o = min(C.addr, spill);
-      const uint32_t li = local0 + (uint32_t)(u * kEwThreads * 4 + j);
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t.reg .f32 t, wf;\n\t"
-          "cvt.rz.f32.u32 wf, %3;\n\t"
-          "abs.f32 t, %2;\n\t"
-          "mul.f32 t, t, %4;\n\t"
-          "setp.ge.f32 p, t, wf;\n\t"
-          "@p st.shared.u32 [%1], %5;\n\t"
-          "@p st.shared.f32 [%1 + %6], %2;\n\t"
-          "@p add.u32 %0, %0, %7;\n\t}"
-          : "+r"(C.addr)
-          : "r"(o), "f"(gg[j]), "r"(ww[j]), "f"(m32), "r"(li), "n"(kEwCandSlots * 4), "n"(kEwThreads * 4)
-          : "memory");
-    }
-  }
-  if (C.addr > spill) *(volatile uint32_t*)C.stop = 1u;    // more candidates than slots: this chunk will be read twice
+  const uint4 wd = philox4x32_10(make_uint4(blk, 0u, layer, kind_step), key);
+  const float d0 = fmaf(fabsf(x.x), m32, -__uint2float_rz(wd.x)), d1 = fmaf(fabsf(x.y), m32, -__uint2float_rz(wd.y));
+  const float d2 = fmaf(fabsf(x.z), m32, -__uint2float_rz(wd.z)), d3 = fmaf(fabsf(x.w), m32, -__uint2float_rz(wd.w));
+  const float d = fmaxf(fmaxf(d0, d1), fmaxf(d2, d3));
+  const uint32_t o = min(C.addr, spill);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ge.f32 p, %2, 0f00000000;\n\t"
+      "@p st.shared.u32 [%1], %3;\n\t"
+      "@p add.u32 %0, %0, %4;\n\t}"
+      : "+r"(C.addr)
+      : "r"(o), "f"(d), "r"(blk), "n"(kEwThreads * 4)
+      : "memory");
 }
 
-__device__ __forceinline__ EwAcc ew_chunk_pass_cand(const EwVec& v, const PhiloxKey key, const uint32_t kind_step, const double s,
-                                                    const int64_t beg, const int64_t end, const int n_my, EwCands& C,
-                                                    float* s_red) {
-  const bool aligned = (reinterpret_cast<uintptr_t>(v.g) & 15u) == 0;
-  const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
-  constexpr int kU = 4;
+__device__ __forceinline__ EwAcc ew_pass_cand(const EwVec& v, const EwChunk& c, const double s, const PhiloxRoundKeys& key,
+                                              const uint32_t kind_step, EwCands& C, EwShared& sh) {
   double sum = 0.0;
   float amax = 0.0f;
-  C.m32 = 0.0f; C.addr = C.addr0;
-  // tiles that lie inside the chunk and can be read with 16-byte loads; the next tile's loads are issued before this
-  // tile's words are drawn, so a warp always has requests in flight
-  const int n_full = aligned ? (int)((end - beg) / kEwTile) : 0;
-  auto load_tile = [&](int tl, float4 (&x)[kU]) {
-    const int64_t base = beg + (int64_t)tl * kEwTile + (int64_t)tid * 4;
-    if (tl < n_full) {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) x[u] = __ldg(reinterpret_cast<const float4*>(v.g + base) + u * kEwThreads);
-    } else {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int64_t i = base + (int64_t)u * kEwThreads * 4;
-        x[u] = i < end ? load4(v.g, i, end, aligned) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-  };
-  // one tile: its sums, and its candidates while the CTA is still listing
-  auto do_tile = [&](int tl, const float4 (&x)[kU]) {
-    const uint32_t local0 = (uint32_t)(tl * kEwTile + tid * 4);
-    const uint32_t blk0 = (uint32_t)(beg >> 2) + (uint32_t)(tl * (kEwTile / 4) + tid);
-    float fsum = 0.0f;                                     // short fp32 run (16 terms), then into fp64: as in ew_chunk_pass
-    if (tl == 0) {                                         // the estimate: this tile's sum, scaled to the vector
-      ew_cand_tile<false>(x, local0, blk0, 0, v.layer, key, kind_step, false, fsum, amax, C);
-      const float ws = warp_sum(fsum);
-      if (lane == 0) s_red[w] = ws;
-      __syncthreads();
-      float ts = 0.0f;
-      for (int i2 = 0; i2 < kEwThreads / kWarp; ++i2) ts += s_red[i2];
-      const double in_tile = (double)min((int64_t)kEwTile, end - beg);
-      // M = 1.25 (s / l1_est) 2^32 with l1_est = ts n / in_tile.  A zero or non-finite ts gives inf or NaN: the threads'
-      // lists overflow or stay empty and the check after the barrier sends the chunk the other way.  No list either
-      // where a thread would expect more than a quarter of its slots to fill (budgets above about 1.5 % of the length:
-      // the list would cost more than the second read)
-      float m32 = (float)(1.25 * s * in_tile * 4294967296.0 / ((double)ts * (double)v.n));
-      const double expect = 1.25 * s * (double)(end - beg) / ((double)v.n * kEwThreads);
-      if (!(m32 > 0.0f) || expect > 0.25 * kEwCandPerThread) m32 = 0.0f;
-      C.m32 = m32;
-      float f2 = 0.0f, u2 = 0.0f;                          // the tile again, for its candidates (sums discarded)
-      if (m32 != 0.0f) ew_cand_tile<false>(x, local0, blk0, end - beg - (int64_t)local0, v.layer, key, kind_step, true, f2, u2, C);
-    } else {
-      const bool listing = C.m32 != 0.0f && *(volatile uint32_t*)C.stop == 0u;
-      if (tl < n_full) ew_cand_tile<true>(x, local0, blk0, 0, v.layer, key, kind_step, listing, fsum, amax, C);
-      else ew_cand_tile<false>(x, local0, blk0, end - beg - (int64_t)local0, v.layer, key, kind_step, listing, fsum, amax, C);
-    }
-    sum += (double)fsum;
-  };
-  float4 x[kU], xn[kU];
-  load_tile(0, x);
-  for (int tl = 0; tl < n_my; ++tl) {
-    if (tl + 1 < n_my) load_tile(tl + 1, xn);
-    do_tile(tl, x);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) x[u] = xn[u];
+  float4 x[1][4];
+  ew_load_ahead(v, c, x);
+  {
+    // M = 1.25 (s / l1_est) 2^32.  A zero or non-finite estimate gives inf or NaN: the threads' lists overflow or stay
+    // empty and the check after the barrier sends the chunk the other way
+    const float m32 = (float)(1.25 * s * 4294967296.0 / ew_estimate_l1(v, c, x[0], sh));
+    C.m32 = m32 > 0.0f ? m32 : 0.0f;
   }
-  EwAcc acc;
-  acc.sum = sum; acc.cnt = 0u; acc.amax = amax;
-  acc.bad = (!(sum == sum) || !(amax <= 3.402823466e38f)) ? 1u : 0u;   // an entry is NaN or infinite
-  return acc;
+  const uint32_t blk_beg = (uint32_t)(c.beg >> 2);
+  float fsum = 0.0f;
+  ew_for_units(v, c, x, [&](uint32_t blk, const float4& y) {
+    ew_sums(y, fsum, amax);
+    ew_cand_block(y, blk_beg + blk, v.layer, key, kind_step, C);
+  }, [&](uint32_t) {
+    sum += (double)fsum;
+    fsum = 0.0f;
+    if (C.addr > C.addr0 + (uint32_t)(kEwCandPerThread * kEwThreads * 4)) {   // no slot left: this chunk will be read twice
+      sh.stop = 1u;
+      C.m32 = -1.0f;                                       // nothing more to list
+    }
+  });
+  return EwAcc{sum, amax, 0u};
 }
 
-// what the probability solve leaves for the sampling pass (every CTA computes the same values)
-struct EwSolved { double T0; float scale, theta, c; uint32_t n_sat, rounds; bool nonfinite; };
+// ---- the solve --------------------------------------------------------------------------------------------------------
+// what the probability solve leaves for the sampling pass (every CTA of the vector computes the same values)
+struct EwSolved { double T0; float scale, theta, c, amax; uint32_t n_sat, rounds; bool nonfinite; };
 
-// The solve over this CTA's elements [beg, end) (a multiple of 4 from the start of the vector); all CTAs of the grid
-// call it together (cooperative launch).  `first`: the sums of the first pass, if the caller has made it already.
-__device__ __forceinline__ EwSolved ew_solve_body(const EwVec& v, const double s, const int64_t beg, const int64_t end,
-                                                  const EwAcc* first = nullptr) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ double s_sum[kEwThreads / kWarp];
-  __shared__ float s_max[kEwThreads / kWarp];
-  __shared__ uint32_t s_cnt[kEwThreads / kWarp], s_bad[kEwThreads / kWarp];
-  const int nb = gridDim.x;
-  // ---- pass 1: ||g||_1, ||g||_inf, non-finite scan ----
-  EwAcc mine = ew_block_reduce(first != nullptr ? *first : ew_chunk_pass<false>(v, 0.0f, beg, end), s_sum, s_max, s_cnt, s_bad);
-  if (threadIdx.x == 0) v.partials[blockIdx.x] = EwPartial{mine.sum, mine.amax, mine.cnt, mine.bad};
-  grid.sync();
-  EwAcc tot{0.0, 0.0f, 0u, 0u};
-  for (int i = threadIdx.x; i < nb; i += kEwThreads) {
-    const EwPartial p = v.partials[i];
-    tot.sum += p.sum; tot.amax = fmaxf(tot.amax, p.amax); tot.cnt += p.cnt; tot.bad |= p.nonfinite;
-  }
-  tot = ew_block_reduce(tot, s_sum, s_max, s_cnt, s_bad);
+// `first`: this thread's part of pass 1; `round(theta)`: this thread's part of a water-filling round over the chunk
+template <typename Round>
+__device__ __forceinline__ EwSolved ew_solve(const EwVec& v, const EwChunk& c, const double s, const EwAcc& first, Round round, EwShared& sh) {
+  const int nb = v.n_ctas;
+  uint32_t arrivals = 0;
+  // every chunk's partial sums out, those of all chunks in; each CTA adds them in the same order
+  auto exchange = [&](EwAcc mine, int buf) {
+    mine = ew_block_reduce(mine, sh);
+    if (nb == 1) return mine;
+    EwPartial* const part = v.partials + (size_t)buf * nb;
+    if (threadIdx.x == 0) part[c.index] = EwPartial{mine.sum, mine.amax, mine.cnt};
+    arrivals += (uint32_t)nb;
+    ew_barrier(v, arrivals, sh);
+    EwAcc tot{0.0, 0.0f, 0u};
+    for (int i = threadIdx.x; i < nb; i += kEwThreads) {
+      static_assert(sizeof(EwPartial) == 16, "one 16-byte load");
+      const int4 raw = __ldcg(reinterpret_cast<const int4*>(part + i));
+      tot.sum += __hiloint2double(raw.y, raw.x); tot.amax = fmaxf(tot.amax, __int_as_float(raw.z)); tot.cnt += (uint32_t)raw.w;
+    }
+    return ew_block_reduce(tot, sh);
+  };
+  EwAcc tot = exchange(first, 0);
   const double T0 = tot.sum;
   const float amax = tot.amax;
-  const bool nonfinite = tot.bad != 0;
+  const bool nonfinite = !(T0 == T0) || !(amax <= 3.402823466e38f);     // an entry is NaN or infinite
   double T = T0, s_cur = s;
   uint32_t n_sat = 0, rounds = 0;
   // atoms with |g| > theta are unbalanced (Definition 1) for the current (T, s_cur); Lemma 3: none if
   // s <= ||g||_1 / ||g||_inf.  The comparison is made in fp32 everywhere so that every kernel agrees on
-  // which atoms are saturated.
-  float theta = (float)(T0 / s);
+  // which atoms are saturated.  A budget of n or more keeps every non-zero atom: threshold 0 at once.
+  float theta = s >= (double)v.n ? 0.0f : (float)(T0 / s);
   bool done = nonfinite || !(amax > theta);
-  // ---- water-filling rounds ----
   while (!done && rounds < kEwMaxRounds) {
-    EwPartial* buf = v.partials + (size_t)((rounds & 1) + 1) * nb;
-    mine = ew_block_reduce(ew_chunk_pass<true>(v, theta, beg, end), s_sum, s_max, s_cnt, s_bad);
-    if (threadIdx.x == 0) buf[blockIdx.x] = EwPartial{mine.sum, 0.0f, mine.cnt, 0u};
-    grid.sync();
-    tot = EwAcc{0.0, 0.0f, 0u, 0u};
-    for (int i = threadIdx.x; i < nb; i += kEwThreads) { const EwPartial p = buf[i]; tot.sum += p.sum; tot.cnt += p.cnt; }
-    tot = ew_block_reduce(tot, s_sum, s_max, s_cnt, s_bad);
+    // buffers alternate: a chunk may still read the previous exchange while others write this one
+    tot = exchange(round(theta), (int)(rounds & 1) + 1);
     ++rounds;
     if (tot.cnt == n_sat) { done = true; }             // no new saturated atom: (T, s_cur) stand
     else {
@@ -297,390 +379,551 @@ __device__ __forceinline__ EwSolved ew_solve_body(const EwVec& v, const double s
   }
   const bool live = T > 0.0 && s_cur > 0.0 && !nonfinite;
   EwSolved r;
-  r.T0 = T0; r.theta = theta; r.n_sat = n_sat; r.rounds = rounds; r.nonfinite = nonfinite;
+  r.T0 = T0; r.theta = theta; r.n_sat = n_sat; r.rounds = rounds; r.nonfinite = nonfinite; r.amax = amax;
   r.scale = live ? (float)(s_cur / T) : 0.0f;            // p_i = |g_i| * scale
   r.c = live ? (float)(T / s_cur) : 0.0f;                // weight of kept unsaturated atoms
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    EwState* st = v.state;
-    st->T0 = T0; st->T = T; st->s_cur = s_cur; st->theta = (double)theta; st->theta_f = theta; st->amax = amax;
-    st->n_sat = n_sat; st->rounds = rounds; st->done = 1; st->nonfinite = nonfinite ? 1u : 0u;
-    st->scale = r.scale; st->c = r.c;
-  }
   return r;
 }
-
-__global__ void __launch_bounds__(kEwThreads) ew_solve_kernel(EwVec v, double s) {
-  const int64_t beg = (int64_t)blockIdx.x * v.chunk;
-  ew_solve_body(v, s, beg, min(v.n, beg + v.chunk));
+__device__ __forceinline__ void ew_store_state(const EwVec& v, const EwSolved& S) {
+  EwState* st = v.state;
+  st->T0 = S.T0; st->theta = S.theta; st->amax = S.amax; st->n_sat = S.n_sat; st->rounds = S.rounds;
+  st->nonfinite = S.nonfinite ? 1u : 0u; st->scale = S.scale; st->c = S.c;
 }
 
-// ---- sampling + ordered compaction, one kernel -----------------------------------------------------
-// A CTA takes the next chunk of consecutive tiles (the tiles are spread evenly over the chunks) (a ticket, so that every chunk it will wait for
-// is already running).  Phase 1: the keep bit of every atom of the chunk (Eq. 2: p_i = 1 on the saturated set,
-// |g_i| (s - n_s) / T elsewhere; Philox word against floor(p 2^32)); mask words go to shared memory (and to the
-// mask output), kept atoms are counted per tile.  The chunk's count is published; the CTA then waits (bounded)
-// until every earlier chunk has published and adds their counts -- all chunks of a wave finish phase 1 together,
-// so nobody waits on a chain.  Phase 2: ordered compaction of the chunk from the mask words in shared memory;
-// only the kept atoms' values are read again (they are still in L2).  The last chunk writes k, the capacity
-// check and the layer header.  A wait that runs out raises ATOMO_ERR_TIMEOUT in the layer header.
-constexpr uint64_t kFlagReady = 1ull << 63;
-constexpr uint32_t kChunkSpinLimit = 1u << 20;
-constexpr int kEwMaxTilesPerCta = 64;
-constexpr int kEwWordsPerTile = kEwTile / 32;
-
-// Phase 1 of the sample / pack kernel over the chunk's tiles: keep bits into the mask words, kept atoms counted per
-// tile.  A thread takes 16 consecutive atoms of a tile (four Philox blocks), so two neighbouring lanes hold a mask
-// word between them.  SAT also records which kept atoms are saturated (a second mask and count; the compact format
-// of a vector that is not s-balanced needs them); UNBAL: the vector is not s-balanced, so some atoms have p = 1 (an
-// s-balanced vector, Lemma 3, skips that test); FULL: the tile lies inside the vector and is 16-byte aligned;
-// PROB: the probabilities are wanted too (debug output).  The tiles are taken from the chunk's last to its first:
-// the reduction kernel read them in ascending order just before, so the end of the chunk is what the L2 still holds.
-template <bool SAT, bool UNBAL, bool FULL, bool PROB>
-__device__ __forceinline__ void ew_tile_bits(const EwVec& v, const PhiloxKey key, const uint32_t kind_step, const uint32_t tile,
-                                             const float scale, const float scale32, const float theta, const bool dead,
-                                             const bool aligned, uint32_t& nb_out, uint32_t& sb_out) {
-  const int tid = threadIdx.x;
-  const int64_t i0 = (int64_t)tile * kEwTile + 16 * tid;
+// ---- the keep decisions -------------------------------------------------------------------------------------------------
+// p = 1 on the saturated set, min(|g| scale, 1) elsewhere; keep iff p >= 1 or word < floor(p 2^32).  t = |g| scale32 is the
+// same product times 2^32 (exact).  word < floor(t) is word <= t - 1 in whole numbers, and rz(word) <= rd(t - 1) in fp32 says
+// exactly that: below 2^24 both sides are exact (t is a multiple of its last place, at most 1); above, rd(t - 1) is the
+// largest fp32 number below t, and rz(word) is below t iff word is.  (The conversion of t to an integer would go through
+// the pipe that converts 16 numbers per clock: 46 us for 100 M atoms.)
+struct EwDecide { float scale, scale32, theta, below_one; bool dead; };   // atoms with |g| < below_one have p < 1
+__device__ __forceinline__ EwDecide ew_decide_of(const EwSolved& S) {
+  EwDecide d;
+  d.scale = S.scale; d.scale32 = S.scale * 4294967296.0f; d.theta = S.theta; d.dead = S.nonfinite;
+  // |g| scale is below 1 by more than the rounding of the product, and |g| below theta.  (The fast path also wants a kept
+  // atom's entry to be a normal number: t >= 1 means |g| >= 1 / scale32.)
+  d.below_one = d.scale32 > 0.0f && d.scale32 < 1.0e27f && !d.dead ? fminf(d.theta, 0.999f / S.scale) : 0.0f;
+  return d;
+}
+// code byte of a block, any case; i: index of its first atom
+__device__ __noinline__ uint32_t ew_code_any(const float4 x, const uint4 wd, const EwDecide d, const int64_t i, const int64_t end) {
+  const float g[4] = {x.x, x.y, x.z, x.w};
+  const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
+  uint32_t code = 0;
+  for (int j = 0; j < 4; ++j) {
+    const float a = fabsf(g[j]), t = a * d.scale32;
+    const bool sat = a > d.theta;
+    if (d.dead || i + j >= end || !(sat || t >= 4294967296.0f || __uint2float_rz(ww[j]) <= __fadd_rd(t, -1.0f))) continue;
+    if (!sat) code |= 1u << j;
+    if (sat || __float_as_int(g[j]) < 0) code |= 16u << j;
+  }
+  return code;
+}
+// ... where every |g| of the block is below below_one and inside the chunk.  What bounds pass 2 is the pipe for logic, compares
+// and votes (half the rate of multiply-adds, and the rounds of Philox need it for 20 instructions per block), so the byte is
+// put together by multiply-adds: saturated to [0, 1] they are the indicators of "kept" and "negative", and the sum at 2^23
+// has the byte as its last bits.  (A compare and a vote per bit: 143 instructions per block, 65 of them in that pipe.)
+__device__ __forceinline__ uint32_t ew_code_plain(const float4& x, const uint4& wd, const EwDecide& d) {
+  const float g[4] = {x.x, x.y, x.z, x.w};
+  const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
+  float acc = 8388608.0f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float over = __fsub_rn(__fadd_rd(__fmul_rn(fabsf(g[j]), d.scale32), -1.0f), __uint2float_rz(ww[j]));   // kept iff >= 0; else at most -2^-24
+    const float kept = __saturatef(fmaf(over, 1.152921504606846976e18f, 1.0f));
+    const float neg = __saturatef(g[j] * -8.507059173023462e37f);                     // (of a kept atom: |g| >= 2^-90)
+    acc = fmaf(kept, fmaf(neg, (float)(16 << j), (float)(1 << j)), acc);
+  }
+  return __float_as_uint(acc) & 255u;
+}
+__device__ __forceinline__ uint4 ew_block_words(const EwVec& v, const EwChunk& c, const int unit, const int u, const PhiloxRoundKeys& key,
+                                                const uint32_t kind_step) {
+  // block of 4 atoms = atom >> 2 < 2^30 (n < 2^32): the high counter word is zero
+  return philox4x32_10(make_uint4((uint32_t)(c.beg >> 2) + ew_unit_block(unit) + (uint32_t)(256 * u), 0u, v.layer, kind_step), key);
+}
+__device__ __forceinline__ void ew_block_decide(const EwChunk& c, const int unit, const int u, const float4& x, const uint4& wd, const EwDecide& d, uint8_t* code) {
+  const uint32_t blk = ew_unit_block(unit) + (uint32_t)(256 * u);
+  const bool plain = unit / kEwUnits < c.n_full && max4(x) < d.below_one;      // almost always
+  code[blk] = (uint8_t)(plain ? ew_code_plain(x, wd, d) : ew_code_any(x, wd, d, c.beg + 4 * (int64_t)blk, c.end));
+}
+// the probabilities (debug output)
+__device__ __forceinline__ void ew_block_prob(const EwVec& v, const EwChunk& c, const int unit, const int u, const float4& x, const EwDecide& d) {
+  const int64_t i = c.beg + 4 * (int64_t)ew_unit_block(unit) + 1024 * u;
+  const float a[4] = {fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w)};
+  for (int j = 0; j < 4 && i + j < c.end; ++j)
+    v.prob_out[i + j] = d.dead ? 0.0f : ((a[j] > d.theta) ? 1.0f : fminf(a[j] * d.scale, 1.0f));
+}
+// pass 2 over the chunk, read (again) from memory.  The warps take the units as they become free, from the chunk's last to its
+// first: pass 1 read them in ascending order just before, so the end of the chunk is what the L2 still holds.
+__device__ __forceinline__ void ew_decide_memory(const EwVec& v, const EwChunk& c, const EwDecide& d, const PhiloxRoundKeys& key,
+                                                 const uint32_t kind_step, EwShared& sh, uint8_t* code) {
+  const int lane = threadIdx.x % kWarp;
+  if (threadIdx.x == 0) sh.next_unit = 0u;
+  __syncthreads();
+  auto take = [&]() -> int {                               // next unit, or a negative number
+    uint32_t t = 0;
+    if (lane == 0) t = atomicAdd(&sh.next_unit, 1u);
+    return c.n_units - 1 - (int)__shfl_sync(0xffffffffu, t, 0);
+  };
   float4 x[4];
+  int unit = take();
+  ew_load_unit(v, c, unit, x);
+  const uint32_t blk_beg = (uint32_t)(c.beg >> 2);
+  while (unit >= 0) {
+    const int next = take();
+    const uint32_t blk = ew_unit_block(unit);
+    if (unit / kEwUnits < c.n_full && next / kEwUnits < c.n_full && next >= 0 && v.prob_out == nullptr) {
+      const float4* const src = reinterpret_cast<const float4*>(v.g + c.beg) + ew_unit_block(next);
+      float m = 0.0f;
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int64_t i = i0 + 4 * it;
-    x[it] = FULL ? __ldg(reinterpret_cast<const float4*>(v.g + i))
-                 : (i < v.n ? load4(v.g, i, v.n, aligned) : make_float4(0.f, 0.f, 0.f, 0.f));
-  }
-  uint32_t nb = 0, sb = 0;
+      for (int u = 0; u < 4; ++u) {
+        const uint4 wd = philox4x32_10(make_uint4(blk_beg + blk + (uint32_t)(256 * u), 0u, v.layer, kind_step), key);
+        code[blk + (uint32_t)(256 * u)] = (uint8_t)ew_code_plain(x[u], wd, d);
+        m = fmaxf(m, max4(x[u]));
+        x[u] = __ldg(src + 256 * u);
+      }
+      if (!(m < d.below_one)) {                            // rare: a lane's blocks again, with the tests for p = 1
+        for (int u = 0; u < 4; ++u) {
+          const float4 y = ew_load_unit(v, c, unit, u);
+          const uint4 wd = philox4x32_10(make_uint4(blk_beg + blk + (uint32_t)(256 * u), 0u, v.layer, kind_step), key);
+          code[blk + (uint32_t)(256 * u)] = (uint8_t)ew_code_any(y, wd, d, c.beg + 4 * (int64_t)(blk + 256 * u), c.end);
+        }
+      }
+    } else {
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    // block of 4 atoms = atom >> 2 < 2^30 (n < 2^32): the high counter word is zero
-    const uint4 wd = philox4x32_10(make_uint4(tile * (uint32_t)(kEwTile / 4) + (uint32_t)(4 * tid + it), 0u, v.layer, kind_step), key);
-    const float a[4] = {fabsf(x[it].x), fabsf(x[it].y), fabsf(x[it].z), fabsf(x[it].w)};
-    const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      // p = 1 if saturated, else min(a scale, 1); keep iff p >= 1 or word < floor(p 2^32).  a scale32 is the
-      // same product times 2^32 (exact), and the truncating conversion gives the floor.
-      const float t = a[j] * scale32;
-      const bool sat = UNBAL && a[j] > theta;
-      bool keep = sat || t >= 4294967296.0f || ww[j] < __float2uint_rz(t);
-      if (!FULL) keep = keep && i0 + 4 * it + j < v.n;
-      if (keep) { nb |= 1u << (4 * it + j); if (SAT && sat) sb |= 1u << (4 * it + j); }
-    }
-    if (PROB) {
-      const int64_t i = i0 + 4 * it;
-      if (i < v.n) {
-        float pp[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) pp[j] = dead ? 0.0f : ((a[j] > theta) ? 1.0f : fminf(a[j] * scale, 1.0f));
-        if (i + 3 < v.n && (reinterpret_cast<uintptr_t>(v.prob_out) & 15u) == 0)
-          *reinterpret_cast<float4*>(v.prob_out + i) = make_float4(pp[0], pp[1], pp[2], pp[3]);
-        else
-          for (int j = 0; j < 4 && i + j < v.n; ++j) v.prob_out[i + j] = pp[j];
+      for (int u = 0; u < 4; ++u) {
+        ew_block_decide(c, unit, u, x[u], ew_block_words(v, c, unit, u, key, kind_step), d, code);
+        if (v.prob_out != nullptr) ew_block_prob(v, c, unit, u, x[u], d);
+        if (next >= 0) x[u] = ew_load_unit(v, c, next, u);
       }
     }
-  }
-  if (dead) { nb = 0; sb = 0; }
-  nb_out = nb; sb_out = sb;
-}
-
-template <bool SAT, bool UNBAL>
-__device__ __forceinline__ void ew_keep_bits(const EwVec& v, const PhiloxKey key, const uint32_t kind_step,
-                                             const int64_t tile0, const int n_my, const float scale, const float theta,
-                                             const bool dead, const bool aligned, uint32_t* s_mask, uint32_t* s_sat,
-                                             uint32_t* s_tcnt, uint32_t* s_tsat) {
-  const int tid = threadIdx.x, lane = tid % kWarp;
-  const float scale32 = scale * 4294967296.0f;    // exact: a power-of-two factor
-  for (int tl = n_my - 1; tl >= 0; --tl) {
-    const uint32_t tile = (uint32_t)(tile0 + tl);
-    const int64_t tile_base = (int64_t)tile * kEwTile;
-    const bool full = aligned && tile_base + kEwTile <= v.n;
-    uint32_t nb, sb;
-    if (v.prob_out != nullptr) ew_tile_bits<SAT, UNBAL, false, true>(v, key, kind_step, tile, scale, scale32, theta, dead, aligned, nb, sb);
-    else if (full) ew_tile_bits<SAT, UNBAL, true, false>(v, key, kind_step, tile, scale, scale32, theta, dead, aligned, nb, sb);
-    else ew_tile_bits<SAT, UNBAL, false, false>(v, key, kind_step, tile, scale, scale32, theta, dead, aligned, nb, sb);
-    // two neighbouring lanes hold the 32 bits of one mask word; the even lane stores it
-    const uint32_t other = __shfl_xor_sync(0xffffffffu, nb, 1);
-    const uint32_t word = nb | (other << 16);
-    uint32_t sword = 0;
-    if (SAT) sword = sb | (__shfl_xor_sync(0xffffffffu, sb, 1) << 16);
-    uint32_t kept = 0, kept_sat = 0;
-    if ((lane & 1) == 0) {
-      const int wl = tid >> 1;
-      s_mask[tl * kEwWordsPerTile + wl] = word;
-      if (SAT) s_sat[tl * kEwWordsPerTile + wl] = sword;
-      const int64_t widx = (tile_base >> 5) + wl;
-      if (widx < v.n_words) v.mask_words[widx] = word;
-      kept = __popc(word);
-      if (SAT) kept_sat = __popc(sword);
-    }
-    kept = warp_sum(kept);
-    if (lane == 0 && kept) atomicAdd(&s_tcnt[tl], kept);
-    if (SAT) {
-      kept_sat = warp_sum(kept_sat);
-      if (lane == 0 && kept_sat) atomicAdd(&s_tsat[tl], kept_sat);
-    }
+    unit = next;
   }
 }
+// pass 2 on the candidate blocks alone; the code bytes start at zero.  A warp first closes up its lanes' lists in place, row by
+// row (an entry never moves past one that is still to be read), so that every lane decides on the same number of blocks: the
+// fullest lane has three times the average.  What was decided on a block goes back to its place: code byte << 24 | block inside
+// the chunk.  Returns the warp's number of blocks.
+__device__ __forceinline__ uint32_t ew_decide_list(const EwVec& v, const EwChunk& c, const EwDecide& d, const PhiloxRoundKeys& key,
+                                                   const uint32_t kind_step, const EwCands& C, uint8_t* __restrict__ code) {
+  const int lane = threadIdx.x % kWarp;
+  uint32_t* const mine = C.blk + (threadIdx.x - lane);     // entry p of the warp: row p / 32, column p % 32
+  const uint32_t n_c = ew_cand_count(C), blk_beg = (uint32_t)(c.beg >> 2), rows = __reduce_max_sync(0xffffffffu, n_c);
+  uint32_t total = 0;
+  for (uint32_t e = 0; e < rows; ++e) {
+    const bool have = e < n_c;
+    const uint32_t b = have ? mine[e * kEwThreads + lane] : 0u, votes = __ballot_sync(0xffffffffu, have);
+    const uint32_t p = total + __popc(votes & ((1u << lane) - 1u));
+    __syncwarp();
+    if (have) mine[(p >> 5) * kEwThreads + (p & 31u)] = b;
+    total += __popc(votes);
+  }
+  __syncwarp();
+  for (uint32_t e0 = lane; e0 < total; e0 += 4 * kWarp) {
+    uint32_t b[4];
+    float4 x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {                          // four blocks' entries in flight
+      const uint32_t e = e0 + q * kWarp;
+      b[q] = e < total ? mine[(e >> 5) * kEwThreads + lane] : 0xFFFFFFFFu;
+      if (b[q] != 0xFFFFFFFFu) x[q] = load4(v.g, 4 * (int64_t)b[q], c.end, c.aligned);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (b[q] == 0xFFFFFFFFu) break;
+      const uint4 wd = philox4x32_10(make_uint4(b[q], 0u, v.layer, kind_step), key);
+      const uint32_t local = b[q] - blk_beg;
+      const uint32_t said = max4(x[q]) < d.below_one ? ew_code_plain(x[q], wd, d) : ew_code_any(x[q], wd, d, 4 * (int64_t)b[q], c.end);
+      if (said) atomicOr(reinterpret_cast<uint32_t*>(code) + (local >> 2), said << (8u * (local & 3u)));
+      mine[((e0 + q * kWarp) >> 5) * kEwThreads + lane] = (said << 24) | local;
+    }
+  }
+  return total;
+}
 
-// COMPACT: the payload takes, per kept atom with p < 1, a 16-bit entry (index inside the tile, sign bit) and, per
-// atom with p = 1, index and value in a list of its own; both ascending.  The chunk's status word then carries the
-// saturated count in bits 32..62 beside the total, and the kernel keeps a second bit mask (saturated and kept).
-template <bool COMPACT>
-__device__ __forceinline__ void ew_sample_pack_chunk(const EwVec& v, const PhiloxKey key, const uint32_t kind_step,
-                                                     const uint32_t chunk, const EwSolved& S, uint32_t* s_mask,
-                                                     const EwCands* cands = nullptr
-#ifdef EW_PROFILE
-                                                     , unsigned long long* ew_t = nullptr
-#endif
-                                                     ) {
-  constexpr int kWarps = kEwThreads / kWarp;
-  __shared__ uint32_t s_tcnt[kEwMaxTilesPerCta];  // kept atoms per tile, then their exclusive prefix
-  __shared__ uint32_t s_tsat[kEwMaxTilesPerCta];  // the same for the saturated kept atoms (COMPACT)
-  __shared__ uint32_t s_chunk, s_chunk_sat;
-  __shared__ unsigned long long s_base;           // kept atoms before this chunk (COMPACT: saturated ones in bits 32..62)
-  __shared__ int s_fail;
-  const float scale = S.scale, theta = S.theta, c = S.c;
-  const bool dead = S.nonfinite;
-  const bool any_sat = COMPACT && S.n_sat != 0;     // an s-balanced vector (Lemma 3) skips the saturated bookkeeping
-  const bool aligned = (reinterpret_cast<uintptr_t>(v.g) & 15u) == 0;
+// ---- counts of the earlier chunks, ordered compaction, headers -----------------------------------------------------------
+struct EwLists {                  // where a chunk's kept atoms go
+  uint32_t* idx; float* val; uint16_t* ent; uint32_t* sat_idx; uint32_t* table;
+  bool compact;
+  // position in the entry list (explicit: every kept atom; compact: those with p < 1) for counts as below
+  __device__ __forceinline__ uint64_t list_of(unsigned long long x) const { return compact ? (x & 0xFFFFFFFFull) - (x >> 32) : x & 0xFFFFFFFFull; }
+};
+__device__ __forceinline__ EwLists ew_lists(const EwVec& v) {
+  EwLists o;
+  o.idx = reinterpret_cast<uint32_t*>(v.pay + v.off_idx); o.ent = reinterpret_cast<uint16_t*>(v.pay + v.off_idx);
+  o.val = reinterpret_cast<float*>(v.pay + v.off_val); o.table = reinterpret_cast<uint32_t*>(v.pay + v.off_tiles);
+  o.sat_idx = reinterpret_cast<uint32_t*>(v.pay + v.off_sat);
+  o.compact = v.compact != 0;
+  return o;
+}
+// The chunk's counts (kept atoms, saturated ones in bits 32 ..) go out; the CTA then waits (bounded) until every earlier chunk of
+// the vector has published and adds their counts -- all chunks of a wave finish their decisions together, so nobody waits
+// on a chain.  Returns the counts before this chunk.  The last chunk writes k, the capacity check and the layer header; a
+// wait that runs out raises ATOMO_ERR_TIMEOUT.  Every thread of the CTA passes the same `total`.
+__device__ __forceinline__ unsigned long long ew_publish(const EwVec& v, const EwChunk& c, const EwSolved& S, const EwLists& o,
+                                                         const unsigned long long total, EwShared& sh) {
   const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
-  const int64_t q = v.n_tiles / v.n_ctas, rem = v.n_tiles % v.n_ctas;   // the first `rem` chunks have q + 1 tiles
-  if (tid == 0) { s_base = 0ull; s_fail = 0; }
-  if (tid < kEwMaxTilesPerCta) { s_tcnt[tid] = 0u; s_tsat[tid] = 0u; }
-  __syncthreads();
-  const int64_t tile0 = (int64_t)chunk * q + min((int64_t)chunk, rem);
-  const int n_my = (int)(q + ((int64_t)chunk < rem ? 1 : 0));
-  uint32_t* s_sat = s_mask + (size_t)(q + (rem ? 1 : 0)) * kEwWordsPerTile;   // COMPACT: saturated masks; one-kernel form deciding on its list: the kept atoms' sign bits
-
-  // ---- phase 1 ----
-  // the candidate list of the first pass holds every kept atom of the chunk if it was made with a multiplier that
-  // covers the true scale, did not overflow and no atom has p = 1
-  bool from_list = cands != nullptr && cands->m32 > 0.0f && S.n_sat == 0 && !dead && scale > 0.0f &&
-                   cands->m32 >= scale * 4294967296.0f * (1.0f + 2.384185791015625e-07f);
-  if (cands != nullptr) from_list = __syncthreads_or(ew_cand_count(*cands) > (uint32_t)kEwCandPerThread ? 1 : 0) == 0 && from_list;
-  if (from_list) {
-    if (tid == 0) atomicAdd(&v.state->list_chunks, 1u);
-    const float scale32 = scale * 4294967296.0f;
-    const int n_w = n_my * kEwWordsPerTile;
-    for (int wi = tid; wi < n_w; wi += kEwThreads) { s_mask[wi] = 0u; s_sat[wi] = 0u; }
-    __syncthreads();
-    const uint32_t n_c = ew_cand_count(*cands);
-    const uint32_t blk_beg = (uint32_t)(tile0 * (kEwTile / 4));
-    for (uint32_t e = 0; e < n_c; ++e) {                   // this thread's own entries; their words are drawn again
-      const uint32_t li = cands->idx[e * kEwThreads + tid];
-      const uint4 wd = philox4x32_10(make_uint4(blk_beg + (li >> 2), 0u, v.layer, kind_step), key);
-      const uint32_t j = li & 3u;
-      const uint32_t word = j == 0 ? wd.x : j == 1 ? wd.y : j == 2 ? wd.z : wd.w;
-      const uint32_t gbits = cands->idx[kEwCandSlots + e * kEwThreads + tid];
-      const float t = fabsf(__uint_as_float(gbits)) * scale32;           // the same product and comparison as ew_tile_bits
-      if (t >= 4294967296.0f || word < __float2uint_rz(t)) {
-        atomicOr(&s_mask[li >> 5], 1u << (li & 31u));
-        if (gbits >> 31) atomicOr(&s_sat[li >> 5], 1u << (li & 31u));    // the value of a kept atom is sign(g) c: its sign is all that phase 2 needs
-        atomicAdd(&s_tcnt[li / kEwTile], 1u);
+  unsigned long long base = 0;
+  if (v.n_ctas > 1) {
+    if (tid == 0) *(volatile unsigned long long*)(v.chunk_status + c.index) = kFlagReady | total;
+    unsigned long long before = 0;
+    for (uint32_t ci = tid; ci < c.index; ci += kEwThreads) {
+      unsigned long long sv;
+      uint32_t polls = 0;
+      for (;;) {
+        sv = *(volatile const unsigned long long*)(v.chunk_status + ci);
+        if ((sv & kFlagReady) || ++polls > kEwPollLimit) break;
+        __nanosleep(40);
       }
+      if (!(sv & kFlagReady)) sh.fail = 1u;
+      before += sv & ~kFlagReady;                          // totals < 2^32 in all: the two fields never mix
     }
-    if (v.n_words > 0) {
-      __syncthreads();
-      for (int wi = tid; wi < n_w; wi += kEwThreads) {
-        const int64_t widx = tile0 * kEwWordsPerTile + wi;
-        if (widx < v.n_words) v.mask_words[widx] = s_mask[wi];
-      }
-    }
-  } else
-  if (any_sat) ew_keep_bits<true, true>(v, key, kind_step, tile0, n_my, scale, theta, dead, aligned, s_mask, s_sat, s_tcnt, s_tsat);
-  else if (S.n_sat != 0) ew_keep_bits<false, true>(v, key, kind_step, tile0, n_my, scale, theta, dead, aligned, s_mask, s_sat, s_tcnt, s_tsat);
-  else ew_keep_bits<false, false>(v, key, kind_step, tile0, n_my, scale, theta, dead, aligned, s_mask, s_sat, s_tcnt, s_tsat);
-  __syncthreads();
-#ifdef EW_PROFILE
-  if (ew_t != nullptr) { EW_STAMP(2) }
-#endif
-
-  // ---- chunk count out, counts of the earlier chunks in ----
-  if (w == 0) {
-    uint32_t total = 0, total_sat = 0;
-    for (int t = lane; t < n_my; t += kWarp) { total += s_tcnt[t]; total_sat += s_tsat[t]; }
-    total = warp_sum(total); total_sat = warp_sum(total_sat);
-    if (lane == 0) {
-      *(volatile unsigned long long*)(v.tile_status + chunk) =
-          kFlagReady | ((unsigned long long)total_sat << 32) | (unsigned long long)total;
-      uint32_t run = 0, run_sat = 0;                      // exclusive prefixes over the chunk's tiles
-      for (int t = 0; t < n_my; ++t) {
-        const uint32_t cnt = s_tcnt[t]; s_tcnt[t] = run; run += cnt;
-        const uint32_t cs = s_tsat[t]; s_tsat[t] = run_sat; run_sat += cs;
-      }
-      s_chunk = total;                                    // reuse: the chunk's counts
-      s_chunk_sat = total_sat;
-    }
-  }
-  unsigned long long before = 0;
-  int fail = 0;
-  for (uint32_t cidx = tid; cidx < chunk; cidx += kEwThreads) {
-    unsigned long long sv;
-    uint32_t spins = 0;
-    for (;;) {
-      sv = *(volatile const unsigned long long*)(v.tile_status + cidx);
-      if ((sv & kFlagReady) || ++spins > kChunkSpinLimit) break;
-      __nanosleep(200);                                   // leave the issue slots to the CTAs that are still sampling
-    }
-    if (!(sv & kFlagReady)) fail = 1;
-    before += sv & ~kFlagReady;                           // totals < 2^32 in all: the two fields never mix
-  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-  if (lane == 0 && before) atomicAdd(&s_base, before);
-  if (fail) s_fail = 1;
-  __syncthreads();
-#ifdef EW_PROFILE
-  if (ew_t != nullptr) { EW_STAMP(3) }
-#endif
-  const uint64_t base_all = s_base & 0xFFFFFFFFull;       // kept atoms before this chunk
-  const uint64_t base_sat = s_base >> 32;                 // of them saturated (0 unless COMPACT)
-  const uint64_t base = COMPACT ? base_all - base_sat : base_all;   // position of the chunk's first list entry
-  const uint32_t total = s_chunk;
+    for (int q = 16; q > 0; q >>= 1) before += __shfl_xor_sync(0xffffffffu, before, q);
+    if (lane == 0) sh.before[w] = before;
+    __syncthreads();
+    base = sh.before[lane];
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) base += __shfl_xor_sync(0xffffffffu, base, q);
+  }
   if (tid == 0) {
-    if (s_fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
-    for (int t = 0; t < n_my; ++t)
-      v.tile_table[tile0 + t] = (uint32_t)min(base + s_tcnt[t] - (COMPACT ? s_tsat[t] : 0u), (uint64_t)0xFFFFFFFFull);
-    if (tile0 + n_my == v.n_tiles) {                      // the last chunk knows k: capacity check, layer header
-      const uint64_t k = base_all + total;
-      const uint64_t k_sat = base_sat + s_chunk_sat;
-      const uint64_t k_list = COMPACT ? k - k_sat : k;    // entries of the idx / entry list
+    if (sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
+    if (c.tile0 + c.n_my == v.n_tiles) {                   // the last chunk knows k: capacity check, layer header
+      const unsigned long long all = base + total;
+      const uint64_t k = all & 0xFFFFFFFFull, k_sat = all >> 32, k_list = o.list_of(all);
       atomo_layer_header* h = v.hdr;
       h->n_sat = S.n_sat; h->c = S.c; h->l1 = S.T0; h->sweeps = S.rounds;
       if (S.nonfinite) raise_status(h, ATOMO_ERR_NONFINITE);
-      else if (k_list > (uint64_t)v.k_cap || (COMPACT && k_sat > (uint64_t)v.sat_cap)) raise_status(h, ATOMO_ERR_CAPACITY);
+      else if (k_list > (uint64_t)v.k_cap || (o.compact && k_sat > (uint64_t)v.sat_cap)) raise_status(h, ATOMO_ERR_CAPACITY);
       const bool ok = *(volatile uint32_t*)&h->status == ATOMO_OK;
       h->k = ok ? (uint32_t)k : 0u;
-      if (COMPACT) h->n_sat = ok ? (uint32_t)k_sat : 0u;  // the length of the saturated list
-      v.tile_table[v.n_tiles] = ok ? (uint32_t)k_list : 0u;
+      if (o.compact) h->n_sat = ok ? (uint32_t)k_sat : 0u; // the length of the saturated list
+      o.table[v.n_tiles] = ok ? (uint32_t)k_list : 0u;
     }
   }
-  if (total == 0) return;
-
-  // ---- phase 2: ordered compaction, indices ascending, value = g_i / p_i ----
-  // A thread takes a run of consecutive mask words of the chunk; one scan over the threads' counts gives every run
-  // its place in the lists.  COMPACT scans two counts at once (list entries in the low half of a 64-bit word,
-  // saturated atoms in the high half).
-  const int n_w = n_my * kEwWordsPerTile;
-  const int wpt = (n_w + kEwThreads - 1) / kEwThreads;                       // words per thread
-  const int w_beg = min(tid * wpt, n_w), w_end = min(w_beg + wpt, n_w);
-  unsigned long long cnt = 0;
-  for (int wi = w_beg; wi < w_end; ++wi) {
-    const uint32_t word = s_mask[wi];
-    const uint32_t sword = any_sat ? s_sat[wi] : 0u;
-    cnt += COMPACT ? ((unsigned long long)__popc(word & ~sword) | ((unsigned long long)__popc(sword) << 32)) : (unsigned long long)__popc(word);
+  return base;
+}
+// the low nibbles of eight code bytes as 32 bits in the order of the atoms
+__device__ __forceinline__ uint32_t ew_nibbles(uint32_t lo, uint32_t hi) {
+  lo &= 0x0F0F0F0Fu; hi &= 0x0F0F0F0Fu;
+  lo = (lo | (lo >> 4)) & 0x00FF00FFu; hi = (hi | (hi >> 4)) & 0x00FF00FFu;
+  return __byte_perm(lo, hi, 0x6420);
+}
+// K and S bits of 32 consecutive atoms: word `at` of the chunk
+__device__ __forceinline__ void ew_word(const uint8_t* __restrict__ code, const int at, uint32_t& kk, uint32_t& ss) {
+  const uint2 b = reinterpret_cast<const uint2*>(code)[at];
+  kk = ew_nibbles(b.x, b.y); ss = ew_nibbles(b.x >> 4, b.y >> 4);
+}
+// debug output: the kept atoms as a plain bit mask
+__device__ __forceinline__ void ew_mask_out(const EwVec& v, const EwChunk& c, const uint8_t* __restrict__ code) {
+  for (int wi = threadIdx.x; wi < c.n_my * (kEwTile / 32); wi += kEwThreads) {
+    const int64_t widx = c.tile0 * (kEwTile / 32) + wi;
+    uint32_t kk, ss;
+    ew_word(code, wi, kk, ss);
+    if (widx < v.n_words) v.mask_words[widx] = kk | ss;
   }
-  unsigned long long inc = cnt;
+}
+
+// Compaction of the decisions taken on the list: a scan over the counts of 32 atoms each, then every kept atom finds its own
+// place from the prefix and the bits before it, and stores its entry directly.  `n_blocks`: what ew_decide_list returned;
+// pref: kEwPrefixes words per tile of the chunk.
+__device__ __forceinline__ void ew_pack_list(const EwVec& v, const EwChunk& c, const EwSolved& S, const EwCands& C, const uint32_t n_blocks,
+                                             const uint8_t* __restrict__ code, uint32_t* __restrict__ pref, EwShared& sh) {
+  const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
+  const EwLists o = ew_lists(v);
+  const int n = c.n_my * kEwPrefixes, per = (n + kEwThreads - 1) / kEwThreads;   // consecutive words per thread
+  const int g0 = min(tid * per, n), g1 = min(g0 + per, n);
+  auto count = [&](int at) -> uint32_t {                   // no atom has p = 1: the K bits alone
+    const uint2 b = reinterpret_cast<const uint2*>(code)[at];
+    return (uint32_t)(__popc(b.x & 0x0F0F0F0Fu) + __popc(b.y & 0x0F0F0F0Fu));
+  };
+  uint32_t cnt = 0;
+  for (int at = g0; at < g1; ++at) { pref[at] = cnt; cnt += count(at); }
+  uint32_t inc = cnt;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) { const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-  __shared__ unsigned long long s_wsum2[kWarps];
-  if (lane == 31) s_wsum2[w] = inc;
+  for (int q = 1; q < 32; q <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, q); if (lane >= q) inc += t; }
+  if (lane == 31) sh.cnt[w] = inc;
   __syncthreads();
-  unsigned long long off = inc - cnt;
-  for (int i = 0; i < w; ++i) off += s_wsum2[i];
-  uint64_t pos = base + (off & 0xFFFFFFFFull);
-  uint64_t pos_sat = base_sat + (off >> 32);
-  for (int wi = w_beg; wi < w_end; ++wi) {
-    uint32_t m = s_mask[wi];
-    const uint32_t sword = any_sat ? s_sat[wi] : 0u;
-    const int tl = wi / kEwWordsPerTile;
-    const uint32_t off0 = (uint32_t)(wi % kEwWordsPerTile) * 32u;            // first atom of the word inside its tile
-    const int64_t tile_base = (tile0 + tl) * (int64_t)kEwTile;
-    while (m) {
-      const int bpos = __ffs(m) - 1;
-      m &= m - 1;
-      const uint32_t o = off0 + (uint32_t)bpos;
-      // from the list: no atom has p = 1, so only the sign is needed, and the list left it in the second mask
-      const float g = from_list ? (((s_sat[wi] >> bpos) & 1u) ? -1.0f : 1.0f) : __ldg(v.g + tile_base + o);
-      if (!COMPACT) {
-        if (pos < (uint64_t)v.k_cap) {
-          // kept atom: saturated (p = 1) keeps g; otherwise g / p = sign(g) T / (s - n_s)
-          v.idx[pos] = (uint32_t)(tile_base + o);
-          v.val[pos] = (!from_list && fabsf(g) > theta) ? g : copysignf(c, g);
+  const uint32_t part = sh.cnt[lane];
+  const uint32_t total = __reduce_add_sync(0xffffffffu, part);
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < w ? part : 0u) + inc - cnt;
+  for (int at = g0; at < g1; ++at) pref[at] += before;
+  const uint64_t base = ew_publish(v, c, S, o, total, sh);
+  __syncthreads();                                         // pref is complete
+  if (v.n_words > 0) ew_mask_out(v, c, code);
+  for (int t = tid; t < c.n_my; t += kEwThreads) o.table[c.tile0 + t] = (uint32_t)min(base + pref[t * kEwPrefixes], (uint64_t)0xFFFFFFFFull);
+  const uint32_t* const mine = C.blk + (tid - lane);
+  const float cw = S.c;
+  for (uint32_t e = lane; e < n_blocks; e += kWarp) {
+    const uint32_t said = mine[(e >> 5) * kEwThreads + lane];
+    uint32_t nib = (said >> 24) & 15u;
+    if (nib == 0) continue;
+    const uint32_t b = said & 0xFFFFFFu, byte = b & 7u;
+    const uint2 eight = reinterpret_cast<const uint2*>(code)[b >> 3];
+    const uint32_t below = (1u << (8u * (byte & 3u))) - 1u;    // the earlier bytes of the block's own word
+    const uint32_t lo = eight.x & 0x0F0F0F0Fu & (byte < 4u ? below : 0xFFFFFFFFu), hi = eight.y & 0x0F0F0F0Fu & (byte < 4u ? 0u : below);
+    uint64_t pos = base + pref[b >> 3] + (uint32_t)(__popc(lo) + __popc(hi));
+    const uint32_t i0 = (uint32_t)(c.beg + 4 * (int64_t)b);
+    for (; nib; nib &= nib - 1, ++pos) {
+      const uint32_t j = (uint32_t)(__ffs(nib) - 1), neg = (said >> (28 + j)) & 1u;
+      if (pos >= (uint64_t)v.k_cap) continue;
+      // the value of a kept atom with p < 1 is sign(g) c
+      if (o.compact) o.ent[pos] = (uint16_t)(((i0 + j) & (uint32_t)(kEwTile - 1)) | (neg << 15));
+      else { o.idx[pos] = i0 + j; o.val[pos] = neg ? -cw : cw; }
+    }
+  }
+}
+
+// Compaction of the code bytes.  A warp takes a run of strips of 1024 atoms, 32 consecutive atoms per lane; a scan over the
+// lanes gives every lane its place in the lists, the kept atoms are put into the warp's window in shared memory in order and
+// the window leaves with coalesced stores (direct 4-byte stores from every thread's own run cost an L2 request each).  A
+// strip with more kept atoms than the window holds is written 32 atoms at a time, an atom per lane.  The signs in the code
+// bytes make a second read of the kept atoms' values unnecessary, except for saturated ones.
+__device__ __forceinline__ void ew_pack(const EwVec& v, const EwChunk& c, const EwSolved& S, const uint8_t* __restrict__ code,
+                                        uint32_t* __restrict__ stage, EwShared& sh) {
+  const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
+  const EwLists o = ew_lists(v);
+  const bool compact = o.compact;
+  const int n_strips = c.n_my * (kEwTile / 1024), u_lo = n_strips * w / kEwWarps, u_hi = n_strips * (w + 1) / kEwWarps;
+  unsigned long long mine = 0;                             // kept atoms of the warp's run; saturated ones in bits 32 ..
+  for (int u = u_lo; u < u_hi; ++u) {
+    uint32_t kk, ss;
+    ew_word(code, u * 32 + lane, kk, ss);                  // this lane's 32 atoms of the strip
+    mine += ((unsigned long long)__popc(ss & ~kk) << 32) | (unsigned long long)__popc(kk | ss);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+  if (lane == 0) sh.scan[w] = mine;
+  __syncthreads();
+  unsigned long long total = sh.scan[lane], run = lane < w ? total : 0ull;   // of the chunk; of the earlier warps
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) { total += __shfl_xor_sync(0xffffffffu, total, q); run += __shfl_xor_sync(0xffffffffu, run, q); }
+  run += ew_publish(v, c, S, o, total, sh);
+  if (v.n_words > 0) ew_mask_out(v, c, code);
+  // the warp's window: atom inside the strip | saturated << 14 | sign << 15
+  uint16_t* const win = reinterpret_cast<uint16_t*>(stage) + w * kEwStage;
+  const float cw = S.c;
+  const uint64_t k_cap = v.k_cap, sat_cap = v.sat_cap;
+  for (int u = u_lo; u < u_hi; ++u) {
+    uint32_t kk, ss;
+    ew_word(code, u * 32 + lane, kk, ss);                  // this lane's 32 atoms of the strip
+    const uint32_t sat_bits = ss & ~kk, list_bits = compact ? kk : kk | ss;
+    const uint32_t cnt = (uint32_t)__popc(list_bits) | ((uint32_t)__popc(sat_bits) << 16);   // at most 1024 each per strip
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+    const uint32_t all = __shfl_sync(0xffffffffu, inc, 31);
+    const uint32_t n_list = all & 0xFFFFu, n_sat = all >> 16;
+    const uint64_t list0 = o.list_of(run);                   // list position of the strip's first entry
+    if (u % (kEwTile / 1024) == 0 && lane == 0) o.table[c.tile0 + u / (kEwTile / 1024)] = (uint32_t)min(list0, (uint64_t)0xFFFFFFFFull);
+    const uint32_t atom0 = (uint32_t)((c.tile0 * (kEwTile / 1024) + u) * 1024);
+    if (n_list <= (uint32_t)kEwStage) {
+      uint32_t pos = (inc - cnt) & 0xFFFFu;
+      const uint32_t at0 = 32u * (uint32_t)lane;
+      if (n_sat == 0) {
+        for (uint32_t left = list_bits; left; left &= left - 1) {
+          const uint32_t b = (uint32_t)(__ffs(left) - 1);
+          win[pos++] = (uint16_t)((at0 + b) | (((ss >> b) & 1u) << 15));
         }
-        ++pos;
-      } else if ((sword >> bpos) & 1u) {
-        if (pos_sat < (uint64_t)v.sat_cap) { v.sat_idx[pos_sat] = (uint32_t)(tile_base + o); v.sat_val[pos_sat] = g; }
-        ++pos_sat;
       } else {
-        // value sign(g) c: the entry carries g's sign bit (what copysignf reads in the explicit format)
-        if (pos < (uint64_t)v.k_cap) v.ent[pos] = (uint16_t)(o | ((__float_as_uint(g) >> 31) << 15));
-        ++pos;
+        for (uint32_t left = list_bits; left; left &= left - 1) {
+          const uint32_t b = (uint32_t)(__ffs(left) - 1);
+          win[pos++] = (uint16_t)((at0 + b) | (((ss >> b) & 1u) << 15) | (((sat_bits >> b) & 1u) << 14));
+        }
+      }
+      __syncwarp();
+      for (uint32_t e = lane; e < n_list; e += kWarp) {
+        if (list0 + e >= k_cap) continue;
+        const uint32_t en = win[e], i = atom0 + (en & 1023u);
+        if (compact) { o.ent[list0 + e] = (uint16_t)((i & (uint32_t)(kEwTile - 1)) | (en & 0x8000u)); continue; }
+        // kept atom: saturated (p = 1) keeps g; otherwise g / p = sign(g) T / (s - n_s)
+        o.idx[list0 + e] = i;
+        o.val[list0 + e] = (en & 0x4000u) ? __ldg(v.g + i) : (en & 0x8000u) ? -cw : cw;
+      }
+      __syncwarp();
+    } else {
+      uint64_t at = list0;
+      for (int t = 0; t < 32; ++t) {
+        const bool in = (__shfl_sync(0xffffffffu, list_bits, t) >> lane) & 1u;
+        const bool neg = (__shfl_sync(0xffffffffu, ss, t) >> lane) & 1u, sat = (__shfl_sync(0xffffffffu, sat_bits, t) >> lane) & 1u;
+        const uint32_t have = __ballot_sync(0xffffffffu, in);
+        const uint64_t pos = at + __popc(have & ((1u << lane) - 1u));
+        const uint32_t i = atom0 + 32u * (uint32_t)t + (uint32_t)lane;
+        if (in && pos < k_cap) {
+          if (compact) o.ent[pos] = (uint16_t)((i & (uint32_t)(kEwTile - 1)) | (neg ? 0x8000u : 0u));
+          else { o.idx[pos] = i; o.val[pos] = sat ? __ldg(v.g + i) : neg ? -cw : cw; }
+        }
+        at += __popc(have);
       }
     }
+    if (compact && n_sat) {                                // the saturated atoms' own list
+      uint64_t at = run >> 32;
+      for (int t = 0; t < 32; ++t) {
+        const bool in = (__shfl_sync(0xffffffffu, sat_bits, t) >> lane) & 1u;
+        const uint32_t have = __ballot_sync(0xffffffffu, in);
+        const uint64_t pos = at + __popc(have & ((1u << lane) - 1u));
+        const uint32_t i = atom0 + 32u * (uint32_t)t + (uint32_t)lane;
+        if (in && pos < sat_cap) { o.sat_idx[pos] = i; o.val[pos] = __ldg(v.g + i); }
+        at += __popc(have);
+      }
+    }
+    run += compact ? ((unsigned long long)n_sat << 32) + n_list + n_sat : ((unsigned long long)n_sat << 32) + n_list;
   }
 }
 
-// The two-kernel form: the solve has left its result in the state record; a CTA takes the next chunk of consecutive
-// tiles by ticket, so that every chunk it will wait for is already running, however many waves the grid takes.
-template <bool COMPACT>
-__global__ void __launch_bounds__(kEwThreads, kEwMinBlocks) ew_sample_pack_kernel(EwVec v, PhiloxKey key, uint32_t kind_step) {
-  extern __shared__ uint32_t s_mask[];            // [tiles_per_cta][128] mask words of the chunk (COMPACT: then the saturated masks)
+// payload header (by the first vector's first CTA) and the layer header as it stands before the counts are known
+__device__ __forceinline__ void ew_write_headers(const EwVec& v, const EwBegin& b, const bool first_vec) {
+  if (threadIdx.x != 0) return;
+  if (b.on && first_vec) *reinterpret_cast<atomo_payload_header*>(v.pay) = b.gh;
+  atomo_layer_header h{};
+  h.rows = 1; h.cols = v.n; h.k_cap = v.k_cap; h.status = ATOMO_OK;
+  h.off_idx = v.off_idx; h.off_val = v.off_val; h.off_short = v.off_tiles; h.off_long = v.compact ? v.off_sat : 0;
+  *v.hdr = h;
+}
+
+// a value the compiler cannot trace: what is worked out from it after a pass is worked out anew instead of being kept in
+// registers (and spilled) through the pass
+__device__ __forceinline__ uint32_t ew_opaque(uint32_t x) { asm volatile("" : "+r"(x)); return x; }
+
+template <int N>
+__device__ __forceinline__ int ew_vec_of(const EwVec (&vecs)[N], const int n, const int cta) {
+  int i = 0;
+  if (N > 1) while (i + 1 < n && cta >= vecs[i + 1].cta0) ++i;
+  return i;
+}
+
+// The one-kernel form.  Dynamic shared memory: [scratch: candidate slots, or list of large atoms, later the staging window]
+// [code bytes of the chunk] [list form: prefix words].  A chunk of at most kEwRegTiles tiles keeps its entries in
+// registers and draws its words before the barrier: nothing is read twice and no list is kept.
+template <int N>
+__global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_constant__ EwBatch<N> B) {
+  extern __shared__ __align__(16) uint32_t ew_smem[];
+  __shared__ EwShared sh;
+  const int tid = threadIdx.x;
+  const int vi = ew_vec_of(B.v, B.n, (int)blockIdx.x);
+  const EwVec& v = B.v[vi];
+  EwChunk c = ew_chunk(v, blockIdx.x - (uint32_t)v.cta0);
+  uint32_t* const scratch = ew_smem;
+  uint8_t* const code = reinterpret_cast<uint8_t*>(ew_smem + B.scratch_words);
+  if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
+  if (blockIdx.x == 0 && tid < kEwBatch) B.next_barriers[tid * kEwBarrierStride] = 0u;   // for the next launch: nobody uses that set now
+  if (c.index == 0) {
+    ew_write_headers(v, B.begin, vi == 0);
+    if (tid == 0) v.state->list_chunks = 0u;               // counted after the barrier
+  }
+  if (tid == 0) v.chunk_status[c.index] = 0ull;            // ordered before its first use by the barrier after pass 1
+  __syncthreads();
+  if (c.n_my <= kEwRegTiles && v.prob_out == nullptr && !v.candidates) {
+    float4 x[4];
+    uint4 wd[4];
+    const int unit = tid / kWarp;
+    ew_load_unit(v, c, (int)(threadIdx.x / kWarp), x);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) wd[u] = ew_block_words(v, c, unit, u, B.key, B.kind_step);
+    float fsum = 0.0f, amax = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ew_sums(x[u], fsum, amax);
+    const EwSolved S = ew_solve(v, c, B.s, EwAcc{(double)fsum, amax, 0u}, [&](float theta) {
+      EwAcc a{0.0, 0.0f, 0u};
+      float f = 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ew_round_sums(x[u], theta, f, a.cnt);
+      a.sum = (double)f;
+      return a;
+    }, sh);
+    if (c.index == 0 && tid == 0) ew_store_state(v, S);
+    const EwDecide d = ew_decide_of(S);
+    if (unit < c.n_units) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ew_block_decide(c, unit, u, x[u], wd[u], d, code);
+    }
+    __syncthreads();
+    ew_pack(v, c, S, code, scratch, sh);
+    return;
+  }
+  if (v.candidates) {
+    const uint32_t cand0 = (uint32_t)__cvta_generic_to_shared(scratch) + 4u * tid;
+    EwCands cands{scratch, 0.0f, cand0, cand0};
+    for (int i = tid; i < c.n_my * (kEwBlocks / 16); i += kEwThreads) reinterpret_cast<uint4*>(code)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const EwAcc first = ew_pass_cand(v, c, B.s, B.key, B.kind_step, cands, sh);
+    c = ew_chunk(v, ew_opaque(blockIdx.x) - (uint32_t)v.cta0);
+    const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) { return ew_round_memory(v, c, theta); }, sh);
+    if (c.index == 0 && tid == 0) ew_store_state(v, S);
+    const EwDecide d = ew_decide_of(S);
+    // the list covers every kept atom of the chunk if it was made with a multiplier that covers the true scale, did not
+    // overflow and no atom has p = 1
+    bool from_list = cands.m32 > 0.0f && S.n_sat == 0 && !d.dead && S.scale > 0.0f &&
+                     cands.m32 >= d.scale32 * (1.0f + 2.384185791015625e-07f);
+    from_list = __syncthreads_or(ew_cand_count(cands) > (uint32_t)kEwCandPerThread || sh.stop != 0u ? 1 : 0) == 0 && from_list;
+    if (from_list) {
+      if (tid == 0) atomicAdd(&v.state->list_chunks, 1u);
+      const uint32_t n_blocks = ew_decide_list(v, c, d, B.key, B.kind_step, cands, code);
+      __syncthreads();
+      ew_pack_list(v, c, S, cands, n_blocks, code, reinterpret_cast<uint32_t*>(code + c.n_my * kEwBlocks), sh);
+    } else {
+      ew_decide_memory(v, c, d, B.key, B.kind_step, sh, code);
+      __syncthreads();
+      ew_pack(v, c, S, code, scratch, sh);
+    }
+    return;
+  }
+  EwBigList big{scratch, 0.0f, 0.0};
+  const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
+  c = ew_chunk(v, ew_opaque(blockIdx.x) - (uint32_t)v.cta0);
+  const float lo = big.lo;
+  const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
+    const uint32_t nb = *(volatile uint32_t*)&sh.n_big;    // complete: a barrier has passed since the last append
+    return nb <= (uint32_t)kEwBig && theta >= lo ? ew_round_list(v, c, big, nb, theta) : ew_round_memory(v, c, theta);
+  }, sh);
+  if (c.index == 0 && tid == 0) ew_store_state(v, S);
+  ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
+  __syncthreads();
+  ew_pack(v, c, S, code, scratch, sh);
+}
+
+// The two-kernel form: the solve leaves its result in the state record; a CTA of the second kernel takes the next chunk of
+// consecutive tiles by ticket, so that every chunk it will wait for is already running, however many waves the grid takes.
+__global__ void __launch_bounds__(kEwThreads, 1) ew_solve_kernel(const __grid_constant__ EwBatch<1> B, int n_pack_chunks) {
+  __shared__ EwShared sh;
+  __shared__ uint32_t s_big[kEwBig];
+  const EwVec& v = B.v[0];
+  const EwChunk c = ew_chunk(v, blockIdx.x);
+  const int tid = threadIdx.x;
+  if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
+  if (blockIdx.x == 0) {
+    if (tid < kEwBatch) B.next_barriers[tid * kEwBarrierStride] = 0u;
+    ew_write_headers(v, B.begin, true);
+    if (tid == 0) { *v.ticket = 0u; v.state->list_chunks = 0u; }
+  }
+  for (int i = blockIdx.x * kEwThreads + tid; i < n_pack_chunks; i += gridDim.x * kEwThreads) v.chunk_status[i] = 0ull;   // for the second kernel
+  __syncthreads();
+  EwBigList big{s_big, 0.0f, 0.0};
+  const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
+  const float lo = big.lo;
+  const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
+    const uint32_t nb = *(volatile uint32_t*)&sh.n_big;
+    return nb <= (uint32_t)kEwBig && theta >= lo ? ew_round_list(v, c, big, nb, theta) : ew_round_memory(v, c, theta);
+  }, sh);
+  if (blockIdx.x == 0 && tid == 0) ew_store_state(v, S);
+  if (tid == 0 && sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
+}
+
+__global__ void __launch_bounds__(kEwThreads, 1) ew_sample_pack_kernel(const __grid_constant__ EwBatch<1> B) {
+  extern __shared__ __align__(16) uint32_t ew_smem[];
+  __shared__ EwShared sh;
   __shared__ uint32_t s_ticket;
+  const EwVec& v = B.v[0];
   const EwState* st = v.state;
   EwSolved S;
-  S.T0 = st->T0; S.scale = st->scale; S.theta = st->theta_f; S.c = st->c; S.n_sat = st->n_sat; S.rounds = st->rounds;
+  S.T0 = st->T0; S.scale = st->scale; S.theta = st->theta; S.c = st->c; S.n_sat = st->n_sat; S.rounds = st->rounds; S.amax = st->amax;
   S.nonfinite = st->nonfinite != 0;
-  if (threadIdx.x == 0) s_ticket = atomicAdd(v.ticket, 1u);
+  if (threadIdx.x == 0) { s_ticket = atomicAdd(v.ticket, 1u); sh.fail = 0u; }
   __syncthreads();
-  ew_sample_pack_chunk<COMPACT>(v, key, kind_step, s_ticket, S, s_mask);
-}
-
-// The one-kernel form (cooperative launch, every chunk resident): a CTA solves over its own chunk of tiles and then
-// samples and packs the same chunk: from the candidate list of its first pass where that holds every kept atom,
-// else from a second read of the chunk, which it finds in the L2 on its own side of the chip.
-// LIST: the form with the candidate list (64 registers, four CTAs per SM); without it the kernel is compiled for five.
-template <bool COMPACT, bool LIST>
-__global__ void __launch_bounds__(kEwThreads, LIST ? kEwEncodeBlocks : kEwMinBlocks)
-ew_encode_kernel(EwVec v, double s, PhiloxKey key, uint32_t kind_step, EwBegin begin) {
-  extern __shared__ uint32_t s_mask[];
-  if (blockIdx.x == 0 && threadIdx.x == 0) v.state->list_chunks = 0u;   // counted after the grid barrier
-  if (begin.on) {
-    // a call with one vector: the payload header, the layer header and the chunks' status words are set here instead of
-    // by a kernel of their own; the grid barrier after the first pass orders them before their first use
-    if (blockIdx.x == 0) {
-      if (threadIdx.x == 0) *reinterpret_cast<atomo_payload_header*>(begin.pay) = begin.gh;
-      if (threadIdx.x < sizeof(atomo_layer_header) / 16)
-        reinterpret_cast<uint4*>(v.hdr)[threadIdx.x] = reinterpret_cast<const uint4*>(begin.tmpl + v.layer)[threadIdx.x];
-    }
-    if (threadIdx.x == 0) v.tile_status[blockIdx.x] = 0ull;
-  }
-  const int64_t q = v.n_tiles / v.n_ctas, rem = v.n_tiles % v.n_ctas;
-  const int64_t chunk = blockIdx.x;
-  const int64_t tile0 = chunk * q + min(chunk, rem);
-  const int64_t n_my = q + (chunk < rem ? 1 : 0);
-#ifdef EW_PROFILE
-  unsigned long long ew_t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#endif
-  EW_STAMP(0)
-  const int64_t beg = tile0 * kEwTile, end = min(v.n, (tile0 + n_my) * kEwTile);
-  if constexpr (LIST) {
-    __shared__ uint32_t s_cand[2 * kEwCandSlots], s_cstop;   // indices, then values
-    __shared__ float s_red[kEwThreads / kWarp];
-    const uint32_t cand0 = (uint32_t)__cvta_generic_to_shared(s_cand) + 4u * threadIdx.x;
-    EwCands cands{s_cand, &s_cstop, 0.0f, cand0, cand0};
-    const bool with_list = v.prob_out == nullptr;
-    EwAcc first;
-    if (with_list) {
-      if (threadIdx.x == 0) s_cstop = 0u;                    // ordered before its first use by the barrier inside the first tile
-      first = ew_chunk_pass_cand(v, key, kind_step, s, beg, end, (int)n_my, cands, s_red);
-      EW_STAMP(6)
-    }
-    const EwSolved S = ew_solve_body(v, s, beg, end, with_list ? &first : nullptr);
-    EW_STAMP(1)
-#ifdef EW_PROFILE
-    ew_sample_pack_chunk<COMPACT>(v, key, kind_step, (uint32_t)chunk, S, s_mask, &cands, ew_t);
-    EW_STAMP(5)
-    if (threadIdx.x == 0 && (blockIdx.x == 0 || blockIdx.x == gridDim.x / 2 || blockIdx.x == gridDim.x - 1))
-      printf("cta %d tiles %d: first pass with list %llu ns (%u candidates in thread 0), solve %llu, keep bits %llu, publish+wait %llu, scan+pack %llu, total %llu\n",
-             (int)blockIdx.x, (int)n_my, ew_t[6] ? ew_t[6] - ew_t[0] : 0ull, ew_cand_count(cands), ew_t[1] - ew_t[0], ew_t[2] - ew_t[1], ew_t[3] - ew_t[2],
-             ew_t[5] - ew_t[3], ew_t[5] - ew_t[0]);
-#else
-    ew_sample_pack_chunk<COMPACT>(v, key, kind_step, (uint32_t)chunk, S, s_mask, &cands);
-#endif
-  } else {
-    const EwSolved S = ew_solve_body(v, s, beg, end);
-    ew_sample_pack_chunk<COMPACT>(v, key, kind_step, (uint32_t)chunk, S, s_mask);
-  }
+  const EwChunk c = ew_chunk(v, s_ticket);
+  uint8_t* const code = reinterpret_cast<uint8_t*>(ew_smem + B.scratch_words);
+  ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
+  __syncthreads();
+  ew_pack(v, c, S, code, ew_smem, sh);
 }
 
 // ---- decode -------------------------------------------------------------------------------------
@@ -690,184 +933,365 @@ __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* __restrict__
   return lo;
 }
 
-__global__ void __launch_bounds__(kEwThreads) ew_decode_kernel(EwDecode d) {
-  const atomo_layer_header* h = d.hdr;
-  const bool compact = d.ghdr->ew_format == ATOMO_EW_COMPACT;
-  const uint32_t sat_cap = compact ? (uint32_t)min(d.ghdr->ew_sat_cap, (uint64_t)0xFFFFFFFFull) : 0u;
-  bool ok = d.ghdr->magic == ATOMO_MAGIC && d.ghdr->kind == ATOMO_KIND_ENTRYWISE && d.ghdr->ew_format <= ATOMO_EW_COMPACT &&
-            h->rows == 1 && h->cols == d.n;
-  if (compact) ok = ok && h->n_sat <= h->k && h->n_sat <= sat_cap && h->k - h->n_sat <= h->k_cap;
-  else ok = ok && h->k <= h->k_cap;
-  if (!ok && blockIdx.x == 0 && threadIdx.x == 0) raise_status(const_cast<atomo_layer_header*>(h), ATOMO_ERR_PAYLOAD);
-  const uint32_t n_sat = (ok && compact) ? h->n_sat : 0u;
-  const uint32_t k = ok ? h->k - n_sat : 0u;               // entries of the idx / entry list
-  const float c = h->c;
-  const uint32_t* idx = reinterpret_cast<const uint32_t*>(d.payload + h->off_idx);
-  const uint16_t* ent = reinterpret_cast<const uint16_t*>(d.payload + h->off_idx);
-  const float* val = reinterpret_cast<const float*>(d.payload + h->off_val);
-  const uint32_t* table = reinterpret_cast<const uint32_t*>(d.payload + h->off_short);   // list entries before each tile
-  const uint32_t* sat_idx = reinterpret_cast<const uint32_t*>(d.payload + h->off_long);
-  const int64_t n_tiles = (d.n + kEwTile - 1) / kEwTile;
-  const bool vec = (reinterpret_cast<uintptr_t>(d.out) & 15u) == 0;
-  // a CTA walks over tiles: zero-fill with vector stores, barrier, then the tile's few kept values
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t tile_base = tile * kEwTile;
-    float* out = d.out + tile_base;
-    const int64_t left = d.n - tile_base;
-    if (left >= kEwTile && vec) {
+// What a decoder needs of one vector of a payload; nothing is kept where the header does not fit the shapes
+struct EwSource {
+  const uint32_t* idx; const uint16_t* ent; const float* val; const uint32_t* table; const uint32_t* sat_idx;
+  uint32_t k, n_sat; float c; bool compact, ok;
+};
+__device__ __forceinline__ EwSource ew_source(const uint8_t* payload, const int layer, const int64_t n) {
+  const atomo_payload_header* gh = reinterpret_cast<const atomo_payload_header*>(payload);
+  const atomo_layer_header* h = reinterpret_cast<const atomo_layer_header*>(payload + sizeof(atomo_payload_header)) + layer;
+  EwSource r;
+  r.compact = gh->ew_format == ATOMO_EW_COMPACT;
+  const uint32_t sat_cap = r.compact ? (uint32_t)min(gh->ew_sat_cap, (uint64_t)0xFFFFFFFFull) : 0u;
+  r.ok = gh->magic == ATOMO_MAGIC && gh->kind == ATOMO_KIND_ENTRYWISE && gh->ew_format <= ATOMO_EW_COMPACT &&
+         h->rows == 1 && h->cols == n;
+  if (r.compact) r.ok = r.ok && h->n_sat <= h->k && h->n_sat <= sat_cap && h->k - h->n_sat <= h->k_cap;
+  else r.ok = r.ok && h->k <= h->k_cap;
+  r.n_sat = (r.ok && r.compact) ? h->n_sat : 0u;
+  r.k = r.ok ? h->k - r.n_sat : 0u;                        // entries of the idx / entry list
+  r.c = h->c;
+  r.idx = reinterpret_cast<const uint32_t*>(payload + h->off_idx);
+  r.ent = reinterpret_cast<const uint16_t*>(payload + h->off_idx);
+  r.val = reinterpret_cast<const float*>(payload + h->off_val);
+  r.table = reinterpret_cast<const uint32_t*>(payload + h->off_short);   // list entries before each tile
+  r.sat_idx = reinterpret_cast<const uint32_t*>(payload + h->off_long);
+  return r;
+}
+__device__ __forceinline__ void ew_raise_payload(const uint8_t* payload, const int layer) {
+  raise_status(reinterpret_cast<atomo_layer_header*>(const_cast<uint8_t*>(payload) + sizeof(atomo_payload_header)) + layer, ATOMO_ERR_PAYLOAD);
+}
+
+// A tile from shared memory to the output: one bulk copy where the output allows it (16-byte base), plain stores for the
+// rest.  Called by every thread of the CTA after its last write to the tile.
+__device__ __forceinline__ void ew_tile_out(float* __restrict__ out, const float* __restrict__ s_tile, const int64_t left, const int threads) {
+  const bool bulk = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  const int n = (int)min(left, (int64_t)kEwTile), n_bulk = bulk ? n & ~3 : 0;
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && n_bulk > 0) {
+    const uint32_t src = (uint32_t)__cvta_generic_to_shared(s_tile);
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out), "r"(src), "r"(n_bulk * 4) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  }
+  for (int i = n_bulk + threadIdx.x; i < n; i += threads) out[i] = s_tile[i];
+  if (threadIdx.x == 0 && n_bulk > 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the tile may go now
+}
+
+// One tile per CTA, all vectors of the call in one launch.  Bound: HBM writes.  The tile is zeroed and filled in shared
+// memory and leaves as one 16 KB bulk copy, so the L2 sees whole lines only (zero stores followed by the kept values as
+// 4-byte stores of their own, behind a barrier, took 21.4 us for 25.6 M elements at 1 % and 106 us for 100 M at 10 %).
+// Small CTAs, so that a dozen tiles per SM overlap their chains header -> tile table -> entries.
+constexpr int kEwDecThreads = 128;
+template <int N>
+__global__ void __launch_bounds__(kEwDecThreads) ew_decode_kernel(const __grid_constant__ EwDecodeBatch<N> B) {
+  __shared__ __align__(128) float s_tile[kEwTile];
+  int vi = 0;
+  if (N > 1) while (vi + 1 < B.n && blockIdx.x >= B.v[vi + 1].tile0) ++vi;
+  const EwDecode& d = B.v[vi];
+  const int64_t tile = blockIdx.x - d.tile0, tile_base = tile * kEwTile, left = d.n - tile_base;
+  const int tid = threadIdx.x;
+  const EwSource s = ew_source(B.payload, d.layer, d.n);
+  if (!s.ok && tile == 0 && tid == 0) ew_raise_payload(B.payload, d.layer);
+  uint32_t lo = 0, hi = 0;
+  if (s.k) { lo = min(__ldg(s.table + tile), s.k); hi = min(__ldg(s.table + tile + 1), s.k); }
 #pragma unroll
-      for (int i = 0; i < kEwTile / 4 / kEwThreads; ++i)
-        reinterpret_cast<float4*>(out)[threadIdx.x + i * kEwThreads] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-      for (int i = threadIdx.x; i < kEwTile && i < left; i += kEwThreads) out[i] = 0.0f;
-    }
-    uint32_t lo = 0, hi = 0;
-    if (k) { lo = min(__ldg(table + tile), k); hi = min(__ldg(table + tile + 1), k); }
-    __syncthreads();                                     // zeros are ordered before the values below
-    if (!compact) {
-      for (uint32_t j = lo + threadIdx.x; j < hi; j += kEwThreads) {
-        const uint32_t i = __ldg(idx + j);
-        if ((int64_t)i >= tile_base && (int64_t)i < tile_base + kEwTile && (int64_t)i < d.n) d.out[i] = __ldg(val + j);
-      }
-    } else {
-      for (uint32_t j = lo + threadIdx.x; j < hi; j += kEwThreads) {
-        const uint32_t e = __ldg(ent + j);
-        const int64_t off = e & (uint32_t)(kEwTile - 1);
-        if (off < left) out[off] = (e & 0x8000u) ? -c : c;
-      }
-      if (n_sat) {                                       // the saturated atoms of this tile (ascending list)
-        const uint32_t s_lo = lower_bound_u32(sat_idx, n_sat, (uint64_t)tile_base);
-        for (uint32_t j = s_lo + threadIdx.x; j < n_sat; j += kEwThreads) {
-          const int64_t off = (int64_t)__ldg(sat_idx + j) - tile_base;
-          if (off >= kEwTile) break;
-          if (off >= 0 && off < left) out[off] = __ldg(val + j);
-        }
-      }
+  for (int i = 0; i < kEwTile / 4 / kEwDecThreads; ++i) reinterpret_cast<float4*>(s_tile)[tid + i * kEwDecThreads] = make_float4(0.f, 0.f, 0.f, 0.f);
+  // the first entries are on their way while the zeros settle
+  uint32_t j = lo + tid, i0 = 0;
+  float v0 = 0.0f;
+  if (j < hi) {
+    if (!s.compact) { i0 = __ldg(s.idx + j) - (uint32_t)tile_base; v0 = __ldg(s.val + j); }
+    else { const uint32_t e = __ldg(s.ent + j); i0 = e & (uint32_t)(kEwTile - 1); v0 = (e & 0x8000u) ? -s.c : s.c; }
+  }
+  __syncthreads();
+  while (j < hi) {
+    if (i0 < (uint32_t)kEwTile) s_tile[i0] = v0;
+    j += kEwDecThreads;
+    if (j < hi) {
+      if (!s.compact) { i0 = __ldg(s.idx + j) - (uint32_t)tile_base; v0 = __ldg(s.val + j); }
+      else { const uint32_t e = __ldg(s.ent + j); i0 = e & (uint32_t)(kEwTile - 1); v0 = (e & 0x8000u) ? -s.c : s.c; }
     }
   }
+  if (s.n_sat) {                                           // compact: the saturated atoms of this tile (ascending list)
+    for (uint32_t q = lower_bound_u32(s.sat_idx, s.n_sat, (uint64_t)tile_base) + tid; q < s.n_sat; q += kEwDecThreads) {
+      const int64_t off = (int64_t)__ldg(s.sat_idx + q) - tile_base;
+      if (off >= kEwTile) break;
+      if (off >= 0) s_tile[off] = __ldg(s.val + q);
+    }
+  }
+  ew_tile_out(d.out + tile_base, s_tile, left, kEwDecThreads);
+}
+
+// ---- decode and average ---------------------------------------------------------------------------
+// out = (1/P) sum over the payloads (combine step of data-parallel training, Section 2): a tile per CTA in shared memory
+// receives payload 0's kept values, then payload 1's, ... (indices are unique inside a payload, so no two threads meet
+// between barriers) and leaves once; explicit and compact payloads may be mixed.  Bound: HBM writes.  The payloads'
+// headers and table entries are fetched by one thread each, then the entries of all of them, as one sequence of up to
+// 2048 at a time, before the first is added: the chain of dependent loads is paid once per tile instead of once per
+// payload (88 us for eight payloads of 25.6 M elements at 1 % with a payload at a time).
+constexpr int kAvgThreads = 256, kAvgPer = 8, kAvgPayloads = 64;     // payloads per round: their ranges sit in shared memory
+struct AvgSource { const void* idx; const float* val; const uint32_t* sat_idx; uint32_t lo, sat_begin, n_sat, compact; float c; };
+template <int N>
+__global__ void __launch_bounds__(kAvgThreads) ew_decode_average_kernel(const __grid_constant__ EwDecodeBatch<N> B,
+                                                                        const uint8_t* const* __restrict__ payloads,
+                                                                        const int n_payloads, const float inv_p) {
+  __shared__ __align__(128) float s_tile[kEwTile];
+  __shared__ AvgSource s_src[kAvgPayloads];
+  __shared__ uint32_t s_begin[kAvgPayloads + 1];             // entries of the earlier payloads of the round
+  int vi = 0;
+  if (N > 1) while (vi + 1 < B.n && blockIdx.x >= B.v[vi + 1].tile0) ++vi;
+  const EwDecode& d = B.v[vi];
+  const int64_t tile = blockIdx.x - d.tile0, tile_base = tile * kEwTile, left = d.n - tile_base;
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < kEwTile / 4 / kAvgThreads; ++i) reinterpret_cast<float4*>(s_tile)[tid + i * kAvgThreads] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int p0 = 0; p0 < n_payloads; p0 += kAvgPayloads) {
+    const int np = min(kAvgPayloads, n_payloads - p0);
+    __syncthreads();                                       // the previous round has used the ranges
+    if (tid < np) {
+      const uint8_t* payload = payloads[p0 + tid];
+      const EwSource s = ew_source(payload, d.layer, d.n);
+      if (!s.ok && tile == 0) ew_raise_payload(payload, d.layer);
+      uint32_t lo = 0, hi = 0;
+      if (s.k) { lo = min(__ldg(s.table + tile), s.k); hi = min(__ldg(s.table + tile + 1), s.k); }
+      const uint32_t sat0 = s.n_sat ? lower_bound_u32(s.sat_idx, s.n_sat, (uint64_t)tile_base) : 0u;
+      s_src[tid] = AvgSource{s.idx, s.val, s.sat_idx, lo, sat0, s.n_sat, s.compact ? 1u : 0u, s.c};
+      s_begin[tid + 1] = hi > lo ? hi - lo : 0u;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      uint32_t run = 0;
+      s_begin[0] = 0;
+      for (int p = 0; p < np; ++p) { run += s_begin[p + 1]; s_begin[p + 1] = run; }
+    }
+    __syncthreads();
+    const uint32_t total = s_begin[np];
+    int p_next = 0;                                        // payloads before it are complete
+    auto add_saturated = [&](int p) {                      // compact: the atoms with p = 1, none of them in the entry list
+      const AvgSource& s = s_src[p];
+      for (uint32_t q = s.sat_begin + tid; q < s.n_sat; q += kAvgThreads) {
+        const int64_t off = (int64_t)__ldg(s.sat_idx + q) - tile_base;
+        if (off >= kEwTile) break;
+        if (off >= 0) s_tile[off] += __ldg(s.val + q);
+      }
+    };
+    for (uint32_t e0 = 0; e0 < total; e0 += kAvgThreads * kAvgPer) {
+      // this thread's entries of the window: element, value, payload
+      uint32_t el[kAvgPer]; float vl[kAvgPer]; int pl[kAvgPer];
+      int p = 0;
+#pragma unroll
+      for (int q = 0; q < kAvgPer; ++q) {
+        const uint32_t e = e0 + (uint32_t)(q * kAvgThreads) + tid;
+        el[q] = kEwTile; vl[q] = 0.0f; pl[q] = np;
+        if (e < total) {
+          while (e >= s_begin[p + 1]) ++p;
+          const AvgSource& s = s_src[p];
+          const uint32_t j = s.lo + (e - s_begin[p]);
+          pl[q] = p;
+          if (!s.compact) {
+            el[q] = __ldg(reinterpret_cast<const uint32_t*>(s.idx) + j) - (uint32_t)tile_base;
+            vl[q] = __ldg(s.val + j);
+          } else {
+            const uint32_t en = __ldg(reinterpret_cast<const uint16_t*>(s.idx) + j);
+            el[q] = en & (uint32_t)(kEwTile - 1);
+            vl[q] = (en & 0x8000u) ? -s.c : s.c;
+          }
+        }
+      }
+      const uint32_t e_end = min(e0 + (uint32_t)(kAvgThreads * kAvgPer), total);
+      for (int pp = p_next; pp < np && s_begin[pp] < e_end; ++pp) {     // payload by payload, in array order
+#pragma unroll
+        for (int q = 0; q < kAvgPer; ++q) if (pl[q] == pp && el[q] < (uint32_t)kEwTile) s_tile[el[q]] += vl[q];
+        if (s_begin[pp + 1] <= e_end) { add_saturated(pp); p_next = pp + 1; }
+        __syncthreads();
+      }
+    }
+    for (; p_next < np; ++p_next) if (s_src[p_next].n_sat) { add_saturated(p_next); __syncthreads(); }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kEwTile / 4 / kAvgThreads; ++i) {
+    float4& t = reinterpret_cast<float4*>(s_tile)[tid + i * kAvgThreads];
+    t = make_float4(t.x * inv_p, t.y * inv_p, t.z * inv_p, t.w * inv_p);
+  }
+  ew_tile_out(d.out + tile_base, s_tile, left, kAvgThreads);
 }
 
 // ---- l_q budget (Section 4: the budget s = ||g||_1 / ||g||_q turns entry-wise ATOMO into QSGD for q = 2 and
 //      into TernGrad for q = infinity) --------------------------------------------------------------------
-// pass 0: per-CTA sum |g| and max |g|; pass 1 (finite q > 1 only): per-CTA sum (|g| / amax)^q.  fp64 sums.
-__global__ void __launch_bounds__(kEwThreads) ew_lq_kernel(const float* __restrict__ g, int64_t n, int pass, double q,
-                                                           double inv_amax, double* __restrict__ part_sum,
-                                                           float* __restrict__ part_max) {
-  __shared__ double s_sum[kEwThreads / kWarp];
-  __shared__ float s_max[kEwThreads / kWarp];
-  double sum = 0.0;
+// pass 0: sum |g|, max |g| and sum g^2 (fp64: the squares of fp32 numbers neither overflow nor vanish there, so q = 2 needs
+// no scaling and one read of the vector); pass 1 (other finite q > 1): sum (|g| / amax)^q.  fp64 sums, added up by the last
+// CTA in a fixed order into host memory.  Bound: HBM (two passes with 4-byte loads and a host-side sum of the CTAs' parts
+// took 2 x 85 us for 25.6 M elements, where one read is 16 us).
+constexpr int kLqThreads = 256, kLqWarps = kLqThreads / kWarp;
+__global__ void __launch_bounds__(kLqThreads) ew_lq_kernel(const float* __restrict__ g, int64_t n, int pass, double q,
+                                                           double inv_amax, EwLqPart* __restrict__ part, uint32_t* __restrict__ ticket,
+                                                           EwLqPart* __restrict__ result) {
+  __shared__ double s_sum[kLqWarps], s_sq[kLqWarps];
+  __shared__ float s_max[kLqWarps];
+  __shared__ uint32_t s_last;
+  const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
+  const bool aligned = (reinterpret_cast<uintptr_t>(g) & 15u) == 0;
+  double sum = 0.0, sq = 0.0;
   float amax = 0.0f;
-  for (int64_t i = (int64_t)blockIdx.x * kEwThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kEwThreads) {
-    const float a = fabsf(__ldg(g + i));
-    if (pass == 0) { sum += (double)a; amax = fmaxf(amax, a); if (!(a <= 3.0e38f)) amax = __int_as_float(0x7f800000); }
-    else if (a > 0.0f) sum += (q == 2.0) ? ((double)a * inv_amax) * ((double)a * inv_amax) : pow((double)a * inv_amax, q);
+  auto one = [&](float x) {
+    const float a = fabsf(x);
+    if (pass == 0) {
+      const double d = (double)a;
+      sum += d; sq = fma(d, d, sq); amax = fmaxf(amax, a);
+      if (!(a <= 3.0e38f)) amax = __int_as_float(0x7f800000);
+    } else if (a > 0.0f) sum += pow((double)a * inv_amax, q);
+  };
+  const int64_t n4 = aligned ? n / 4 : 0, stride = (int64_t)gridDim.x * kLqThreads;
+  for (int64_t i = (int64_t)blockIdx.x * kLqThreads + tid; i < n4; i += 4 * stride) {
+    float4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = i + u * stride < n4 ? __ldg(reinterpret_cast<const float4*>(g) + i + u * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { one(x[u].x); one(x[u].y); one(x[u].z); one(x[u].w); }
   }
-  sum = warp_sum(sum); amax = warp_max(amax);
-  const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
-  if (lane == 0) { s_sum[w] = sum; s_max[w] = amax; }
+  for (int64_t i = 4 * n4 + (int64_t)blockIdx.x * kLqThreads + tid; i < n; i += stride) one(__ldg(g + i));
+  auto reduce = [&]() {
+    sum = warp_sum(sum); sq = warp_sum(sq); amax = warp_max(amax);
+    __syncthreads();
+    if (lane == 0) { s_sum[w] = sum; s_sq[w] = sq; s_max[w] = amax; }
+    __syncthreads();
+    sum = 0.0; sq = 0.0; amax = 0.0f;
+    for (int i = 0; i < kLqWarps; ++i) { sum += s_sum[i]; sq += s_sq[i]; amax = fmaxf(amax, s_max[i]); }   // fixed order
+  };
+  reduce();
+  if (tid == 0) {
+    part[blockIdx.x] = EwLqPart{sum, sq, (double)amax};
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0; float m = 0.0f;
-    for (int i = 0; i < kEwThreads / kWarp; ++i) { t += s_sum[i]; m = fmaxf(m, s_max[i]); }   // fixed order
-    part_sum[blockIdx.x] = t;
-    if (pass == 0) part_max[blockIdx.x] = m;
+  if (!s_last) return;
+  __threadfence();
+  sum = 0.0; sq = 0.0; amax = 0.0f;
+  for (int i = tid; i < (int)gridDim.x; i += kLqThreads) {
+    sum += __ldcg(&part[i].sum); sq += __ldcg(&part[i].sq); amax = fmaxf(amax, (float)__ldcg(&part[i].amax));
   }
+  reduce();
+  if (tid == 0) { *ticket = 0u; *result = EwLqPart{sum, sq, (double)amax}; }
 }
 
-void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax, double* part_sum, float* part_max,
-                  int n_ctas, cudaStream_t st) {
-  ew_lq_kernel<<<n_ctas, kEwThreads, 0, st>>>(g, n, pass, q, inv_amax, part_sum, part_max);
-}
+}  // namespace
 
 // ---- host-side launchers --------------------------------------------------------------------------
-int ew_solve_max_blocks() {
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ew_solve_kernel, kEwThreads, 0) != cudaSuccess) return 0;
-  return sms * per_sm;
+void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax, EwLqPart* part, uint32_t* ticket,
+                  EwLqPart* result, int max_ctas, cudaStream_t st) {
+  const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>(max_ctas, (n + 16 * kLqThreads - 1) / (16 * kLqThreads)));
+  ew_lq_kernel<<<ctas, kLqThreads, 0, st>>>(g, n, pass, q, inv_amax, part, ticket, result);
 }
 
-int launch_ew_solve(const EwVec& v, double s, cudaStream_t st) {
-  EwVec vv = v; double ss = s;
-  void* args[] = {&vv, &ss};
-  return (int)cudaLaunchCooperativeKernel((const void*)ew_solve_kernel, dim3(v.n_chunks), dim3(kEwThreads), args, 0, st);
-}
 namespace {
-// co-resident CTAs of a sample / pack style kernel with its largest chunk in shared memory
-template <typename K> int64_t ew_wave(K kernel, int dyn_tiles) {
-  int dev = 0, sms = 148, per_sm = 4;
+int ew_sms() {
+  int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kEwThreads, (size_t)dyn_tiles * kEwWordsPerTile * sizeof(uint32_t));
-  if (e != cudaSuccess || per_sm < 1) { cudaGetLastError(); per_sm = 4; }
-  return (int64_t)sms * per_sm;
+  return sms;
 }
+// the slots of the candidate list; else the staging windows (or the list of runs with large atoms)
+size_t ew_scratch_bytes(bool list) { return list ? (size_t)kEwCandBytes : std::max((size_t)kEwWarps * kEwStage * sizeof(uint16_t), kEwBig * sizeof(uint32_t)); }
+static_assert(kEwCandBytes >= kEwWarps * kEwStage * 2 && kEwCandBytes >= kEwBig * 4, "the scratch area serves in turn");
+size_t ew_dyn_bytes(int tiles, bool list) {
+  return ew_scratch_bytes(list) + (size_t)tiles * (kEwBlocks + (list ? kEwPrefixes * sizeof(uint32_t) : 0));
+}
+constexpr size_t kEwMaxDyn = 225 * 1024;            // dynamic shared memory of a CTA (227 KB less the static part)
+constexpr int kEwPackTiles = 64;                    // tiles per chunk of the two-kernel form
 }  // namespace
 
-int ew_sample_pack_ctas(int64_t n_tiles, bool compact) {
-  // one wave of chunks when it fits (at most 64 tiles per chunk, 32 for the compact format): tiles spread evenly, sizes differ by at most one
-  const int64_t wave = compact ? ew_wave(ew_sample_pack_kernel<true>, 32) : ew_wave(ew_sample_pack_kernel<false>, 16);
-  const int max_tiles = compact ? kEwMaxTilesPerCta / 2 : kEwMaxTilesPerCta;   // compact: two masks per tile in shared memory
-  const int64_t min_ctas = (n_tiles + max_tiles - 1) / max_tiles;
-  return (int)std::max<int64_t>(1, std::max(min_ctas, std::min(n_tiles, wave)));
-}
-namespace {
-const void* ew_encode_fn(bool compact, bool list) {
-  if (list) return compact ? (const void*)ew_encode_kernel<true, true> : (const void*)ew_encode_kernel<false, true>;
-  return compact ? (const void*)ew_encode_kernel<true, false> : (const void*)ew_encode_kernel<false, false>;
-}
-}  // namespace
-// CTAs of the one-kernel form, or 0 if the vector does not fit one wave of resident chunks.  `list`: the form that
-// keeps a candidate list during its first pass.
-int ew_encode_ctas(int64_t n_tiles, bool compact, bool list) {
-  static int64_t waves[2][2] = {{0, 0}, {0, 0}};
-  // chunks of at most 12 tiles with the list: with the two masks (12 KB) and the list a CTA stays below 48 KB, so that
-  // four CTAs per SM fit the 196 KB carve-out a cooperative launch is checked against; 16 without (8 or 16 KB of masks)
-  const int64_t fit_tiles = list ? 12 : 16;
-  if (waves[compact][list] == 0) {
-    int dev = 0, sms = 148, per_sm = 4;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t dyn = (size_t)fit_tiles * kEwWordsPerTile * sizeof(uint32_t) * ((compact || list) ? 2 : 1);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ew_encode_fn(compact, list), kEwThreads, dyn) != cudaSuccess || per_sm < 1) {
-      cudaGetLastError(); per_sm = 4;
-    }
-    waves[compact][list] = (int64_t)sms * per_sm;
+int ew_configure() {
+  const void* fns[] = {(const void*)ew_encode_kernel<1>, (const void*)ew_encode_kernel<kEwBatch>, (const void*)ew_sample_pack_kernel};
+  for (const void* f : fns) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEwMaxDyn);
+    if (e != cudaSuccess) return (int)e;
   }
-  const int max_tiles = compact ? kEwMaxTilesPerCta / 2 : kEwMaxTilesPerCta;
-  const int64_t ctas = std::min(n_tiles, waves[compact][list]);
-  if (ctas < 1 || (n_tiles + ctas - 1) / ctas > std::min<int64_t>(max_tiles, fit_tiles)) return 0;
-  return (int)ctas;
-}
-// Whether the list pays for a vector of n elements in `ctas` chunks at budget s: a thread expects 1.25 s (its atoms) / n
-// candidates and has kEwCandPerThread slots; beyond a quarter of them (budgets above about 1.5 % of the length) the
-// appends cost more than the second read saves and overflows become likely.
-bool ew_list_pays(int64_t n, int64_t n_tiles, int ctas, double s) {
-  if (ctas < 1) return false;
-  const double chunk = (double)((n_tiles + ctas - 1) / ctas) * kEwTile;
-  return 1.25 * s * chunk / ((double)n * kEwThreads) <= 0.25 * kEwCandPerThread;
-}
-void launch_ew_sample_pack(const EwVec& v, PhiloxKey key, uint32_t kind_step, cudaStream_t st) {
-  const int64_t most = (v.n_tiles + v.n_ctas - 1) / v.n_ctas;
-  const size_t smem = (size_t)most * kEwWordsPerTile * sizeof(uint32_t);
-  if (v.compact) {
-    // two masks per tile; chunks of at most 32 tiles keep them inside the default 48 KB of dynamic shared memory
-    ew_sample_pack_kernel<true><<<(unsigned)v.n_ctas, kEwThreads, 2 * smem, st>>>(v, key, kind_step);
-  } else {
-    ew_sample_pack_kernel<false><<<(unsigned)v.n_ctas, kEwThreads, smem, st>>>(v, key, kind_step);
+  for (const void* f : {(const void*)ew_decode_kernel<1>, (const void*)ew_decode_kernel<kEwBatch>, (const void*)ew_decode_average_kernel<1>,
+                        (const void*)ew_decode_average_kernel<kEwBatch>}) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return (int)e;
   }
+  return 0;
 }
-int launch_ew_encode(const EwVec& v, double s, PhiloxKey key, uint32_t kind_step, const EwBegin& begin, cudaStream_t st) {
-  const int64_t most = (v.n_tiles + v.n_ctas - 1) / v.n_ctas;
-  // mask words; a second mask for the saturated atoms (compact format) or the sign bits (list)
-  const size_t smem = (size_t)most * kEwWordsPerTile * sizeof(uint32_t) * ((v.compact || v.candidates) ? 2 : 1);
-  EwVec vv = v; double ss = s; PhiloxKey kk = key; uint32_t ks = kind_step; EwBegin bb = begin;
-  void* args[] = {&vv, &ss, &kk, &ks, &bb};
-  return (int)cudaLaunchCooperativeKernel(ew_encode_fn(v.compact != 0, v.candidates != 0), dim3((unsigned)v.n_ctas), dim3(kEwThreads), args, smem, st);
+
+// Chunks of equal size (in tiles) over all vectors, as small as one wave of resident CTAs allows: the fewer tiles a CTA
+// walks over, the shorter the chain between two barriers.  Sets n_ctas and cta0; 0 if the vectors do not fit one wave.
+int ew_plan(EwVec* v, int n_vecs, bool list) {
+  const int sms = ew_sms();
+  int64_t total = 0;
+  for (int i = 0; i < n_vecs; ++i) total += v[i].n_tiles;
+  for (int64_t t = std::max<int64_t>(1, total / sms); ew_dyn_bytes((int)std::min<int64_t>(t, 4096), list) <= kEwMaxDyn; ++t) {
+    int64_t ctas = 0;
+    for (int i = 0; i < n_vecs; ++i) ctas += (v[i].n_tiles + t - 1) / t;
+    if (ctas > sms) continue;
+    int at = 0;
+    for (int i = 0; i < n_vecs; ++i) { v[i].n_ctas = (int)((v[i].n_tiles + t - 1) / t); v[i].cta0 = at; at += v[i].n_ctas; }
+    return at;
+  }
+  return 0;
 }
-void launch_ew_decode(const EwDecode& d, cudaStream_t st) {
-  const int64_t tiles = (d.n + kEwTile - 1) / kEwTile;
-  ew_decode_kernel<<<(unsigned)std::min<int64_t>(tiles, 1 << 20), kEwThreads, 0, st>>>(d);   // a tile per CTA: the CTAs of a wave hide one another's barriers
+// Whether the candidate list pays for a vector of n elements at budget s in n_ctas chunks.  A thread expects 1.25 s (its
+// atoms) / n candidates and has kEwCandPerThread slots: beyond a quarter of them overflows become likely; and with more
+// than a quarter of the blocks listed (budgets above 5 % of the length) the decisions on the list cost what the second
+// read does.  A chunk that fits the registers needs no list.
+bool ew_list_pays(int64_t n, int64_t n_tiles, int n_ctas, double s) {
+  const int64_t tiles = (n_tiles + n_ctas - 1) / n_ctas;
+  if (tiles <= kEwRegTiles || 1.25 * s * 4.0 > 0.25 * (double)n) return false;
+  return 1.25 * s * (double)(tiles * kEwTile) / ((double)n * kEwThreads) <= 0.25 * kEwCandPerThread;
 }
+
+template <int N>
+int launch_ew_encode(EwBatch<N>& B, bool list, cudaStream_t st) {
+  int64_t most = 1;
+  int ctas = 0;
+  bool waits = false;                                // CTAs that wait for one another have to be resident together
+  for (int i = 0; i < B.n; ++i) {
+    most = std::max(most, (B.v[i].n_tiles + B.v[i].n_ctas - 1) / B.v[i].n_ctas);
+    ctas += B.v[i].n_ctas;
+    waits |= B.v[i].n_ctas > 1;
+  }
+  B.scratch_words = (int)(ew_scratch_bytes(list) / sizeof(uint32_t));
+  const size_t smem = ew_dyn_bytes((int)most, list);
+  if (!waits) { ew_encode_kernel<N><<<ctas, kEwThreads, smem, st>>>(B); return (int)cudaGetLastError(); }
+  void* args[] = {&B};
+  return (int)cudaLaunchCooperativeKernel((const void*)ew_encode_kernel<N>, dim3((unsigned)ctas), dim3(kEwThreads), args, smem, st);
+}
+template int launch_ew_encode<1>(EwBatch<1>&, bool, cudaStream_t);
+template int launch_ew_encode<kEwBatch>(EwBatch<kEwBatch>&, bool, cudaStream_t);
+
+int ew_solve_ctas(int64_t n_tiles) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ew_solve_kernel, kEwThreads, 0) != cudaSuccess || per_sm < 1) { cudaGetLastError(); return 0; }
+  return (int)std::min<int64_t>(n_tiles, (int64_t)ew_sms() * per_sm);
+}
+int ew_pack_ctas(int64_t n_tiles) {
+  return (int)std::max<int64_t>((n_tiles + kEwPackTiles - 1) / kEwPackTiles, std::min<int64_t>(n_tiles, (int64_t)ew_sms()));
+}
+int launch_ew_two_kernels(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st) {
+  B.v[0].n_ctas = solve_ctas; B.v[0].cta0 = 0;
+  void* args[] = {&B, &pack_ctas};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)ew_solve_kernel, dim3((unsigned)solve_ctas), dim3(kEwThreads), args, 0, st);
+  if (e != cudaSuccess) return (int)e;
+  B.v[0].n_ctas = pack_ctas;
+  B.scratch_words = (int)(ew_scratch_bytes(false) / sizeof(uint32_t));
+  const int64_t most = (B.v[0].n_tiles + pack_ctas - 1) / pack_ctas;
+  ew_sample_pack_kernel<<<(unsigned)pack_ctas, kEwThreads, ew_dyn_bytes((int)most, false), st>>>(B);
+  return (int)cudaGetLastError();
+}
+template <int N>
+void launch_ew_decode(const EwDecodeBatch<N>& B, uint32_t n_tiles, cudaStream_t st) {
+  ew_decode_kernel<N><<<n_tiles, kEwDecThreads, 0, st>>>(B);
+}
+template void launch_ew_decode<1>(const EwDecodeBatch<1>&, uint32_t, cudaStream_t);
+template void launch_ew_decode<kEwBatch>(const EwDecodeBatch<kEwBatch>&, uint32_t, cudaStream_t);
+template <int N>
+void launch_ew_decode_average(const EwDecodeBatch<N>& B, uint32_t n_tiles, const uint8_t* const* d_payloads, int n_payloads, cudaStream_t st) {
+  ew_decode_average_kernel<N><<<n_tiles, kAvgThreads, 0, st>>>(B, d_payloads, n_payloads, 1.0f / (float)n_payloads);
+}
+template void launch_ew_decode_average<1>(const EwDecodeBatch<1>&, uint32_t, const uint8_t* const*, int, cudaStream_t);
+template void launch_ew_decode_average<kEwBatch>(const EwDecodeBatch<kEwBatch>&, uint32_t, const uint8_t* const*, int, cudaStream_t);
 int ew_tile_elems() { return kEwTile; }
 
 }  // namespace atomo

@@ -8,58 +8,58 @@ namespace atomo {
 constexpr int kEwMaxRounds = 64;      // water-filling rounds; Algorithm 1 saturates < ceil(s) atoms,
                                       // a round usually takes many at once
 
-struct EwPartial { double sum; float amax; uint32_t cnt; uint32_t nonfinite; };
+constexpr int kEwBatch = 24;          // vectors per launch (their descriptors travel as a kernel argument)
+constexpr int kEwBarrierStride = 32;  // words between the barrier counters of two vectors (a line each)
+
+struct EwPartial { double sum; float amax; uint32_t cnt; };
 
 struct EwState {
   double T0;        // ||g||_1
-  double T;         // sum of |g| over unsaturated atoms
-  double s_cur;     // s - n_sat
-  double theta;     // atoms with |g| > theta have p = 1
-  float scale;      // p_i = |g_i| * scale for the rest
-  float c;          // T / s_cur
-  float theta_f, amax;
-  uint32_t n_sat, rounds, done, nonfinite;
+  float scale;      // p_i = |g_i| * scale for atoms with |g| <= theta
+  float c;          // weight of the kept atoms with p < 1
+  float theta, amax;// atoms with |g| > theta have p = 1; max |g|
+  uint32_t n_sat, rounds, nonfinite;
   uint32_t list_chunks; // one-kernel form: chunks whose keep decisions were taken on the candidate list (test introspection)
 };
 
 struct EwVec {
-  const float* g; int64_t n;
-  uint32_t layer; uint32_t k_cap;
-  int64_t chunk; int n_chunks;            // reduction split (chunk is a multiple of 4)
-  int64_t n_tiles; int64_t n_words;
-  atomo_layer_header* hdr; uint32_t* idx; float* val;          // payload
-  EwPartial* partials; EwState* state;                         // workspace
-  uint32_t* mask_words;
-  int n_ctas;                                                  // chunks (CTAs) of the sample / pack kernel
-  uint64_t* tile_status;                                       // [chunks] ready flag (bit 63) | kept atoms of the chunk; zeroed per call
-  uint32_t* ticket;                                            // next chunk to hand out; zeroed per call
-  uint32_t* tile_table;                                        // payload: kept atoms before each tile
-  float* prob_out;                                             // debug or nullptr
-  // compact payload format (else compact = 0 and the rest unused)
-  int compact; uint32_t sat_cap;
-  int candidates;                                              // one-kernel form: keep a candidate list during the first pass (else read the chunk twice)
-  uint16_t* ent;                                               // [k_cap] tile-local index | sign << 15 of kept atoms with p < 1
-  uint32_t* sat_idx; float* sat_val;                           // [sat_cap] atoms with p = 1
+  const float* g; int64_t n, n_tiles;
+  uint8_t* pay; atomo_layer_header* hdr;                       // payload
+  uint64_t off_idx, off_val, off_tiles, off_sat;
+  uint32_t layer, k_cap, sat_cap;
+  int compact, candidates;                                     // payload format; keep a candidate list during the first pass (else read the chunk twice)
+  int n_ctas, cta0;                                            // chunks (CTAs) of this vector, its first CTA in the launch
+  EwPartial* partials; EwState* state;                         // workspace: [3][n_ctas], one record
+  uint64_t* chunk_status;                                      // [chunks] ready flag (bit 63) | saturated << 32 | kept atoms of the chunk
+  uint32_t* barrier; uint32_t* ticket;                         // arrivals at the vector's barriers; next chunk (two-kernel form)
+  uint32_t* mask_words; float* prob_out; int64_t n_words;      // debug outputs or nullptr / 0
+};
+struct EwBegin { atomo_payload_header gh; int on; };           // the payload header, written by the call's first launch
+template <int N> struct EwBatch {
+  EwVec v[N];
+  int n, scratch_words;
+  double s; PhiloxRoundKeys key; uint32_t kind_step;
+  EwBegin begin;
+  uint32_t* next_barriers;                                     // the counters of the next launch: zeroed by this one
 };
 
-struct EwDecode {
-  const uint8_t* payload; const atomo_payload_header* ghdr; const atomo_layer_header* hdr;
-  float* out; int64_t n;
-};
+struct EwDecode { float* out; int64_t n; int layer; uint32_t tile0; };
+template <int N> struct EwDecodeBatch { EwDecode v[N]; int n; const uint8_t* payload; };
+struct EwLqPart { double sum, sq, amax; };
 
-int ew_solve_max_blocks();                                     // co-resident CTAs of the cooperative solve
-int launch_ew_solve(const EwVec& v, double s, cudaStream_t st); // returns a cudaError_t
-void launch_ew_sample_pack(const EwVec& v, PhiloxKey key, uint32_t kind_step, cudaStream_t st);
-void launch_ew_decode(const EwDecode& d, cudaStream_t st);
+int ew_configure();                                            // shared memory opt-in; cudaError_t
+int ew_plan(EwVec* v, int n_vecs, bool list);                  // CTAs of the one-kernel form (sets n_ctas, cta0), 0: does not fit one wave
+bool ew_list_pays(int64_t n, int64_t n_tiles, int n_ctas, double s);   // whether the candidate list is worth keeping at this budget
+template <int N> int launch_ew_encode(EwBatch<N>& B, bool list, cudaStream_t st);       // cudaError_t
+int ew_solve_ctas(int64_t n_tiles);                            // two-kernel form: CTAs of the solve, chunks of the sampling
+int ew_pack_ctas(int64_t n_tiles);
+int launch_ew_two_kernels(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st);   // cudaError_t
+template <int N> void launch_ew_decode(const EwDecodeBatch<N>& B, uint32_t n_tiles, cudaStream_t st);
+template <int N> void launch_ew_decode_average(const EwDecodeBatch<N>& B, uint32_t n_tiles, const uint8_t* const* d_payloads,
+                                               int n_payloads, cudaStream_t st);
 int ew_tile_elems();
-void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax, double* part_sum, float* part_max,
-                  int n_ctas, cudaStream_t st);
-int ew_sample_pack_ctas(int64_t n_tiles, bool compact);
-int ew_encode_ctas(int64_t n_tiles, bool compact, bool list);  // CTAs of the one-kernel form (with or without the candidate list); 0 = the vector needs the two-kernel form
-bool ew_list_pays(int64_t n, int64_t n_tiles, int ctas, double s);   // whether the candidate list is worth keeping at this budget
-// what the header kernel would do for a call with one vector, done by the one-kernel form itself (on = 0: not asked for)
-struct EwBegin { uint8_t* pay; const atomo_layer_header* tmpl; atomo_payload_header gh; int on; };
-int launch_ew_encode(const EwVec& v, double s, PhiloxKey key, uint32_t kind_step, const EwBegin& begin, cudaStream_t st);   // cudaError_t
+void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax, EwLqPart* part, uint32_t* ticket,
+                  EwLqPart* result, int max_ctas, cudaStream_t st);
 
 // ================================= spectral path =================================================
 constexpr int kMaxShort = 4096;       // largest short side (atoms per layer)
@@ -123,12 +123,10 @@ struct TileRef { int32_t layer, a, b, c; };
 // averaging decode of several payloads (combine step of data-parallel training)
 void launch_sp_decode_average(const uint8_t* const* d_payloads, int n_payloads, const SpDecodeLayer* d_layers,
                               const TileRef* d_tiles, int n_tiles, cudaStream_t st);
-void launch_ew_decode_average(const uint8_t* const* d_payloads, int n_payloads, int layer, float* out, int64_t n,
-                              cudaStream_t st);
 
-// payload header (by value), layer headers from a device template, the call's four flag words (may be null)
+// payload header (by value), layer headers from a device template, the call's four flag words
 void launch_sp_begin(uint8_t* pay, const atomo_payload_header& gh, const atomo_layer_header* d_tmpl, int n_layers,
-                     uint32_t* d_flags, uint32_t* d_zero, int64_t n_zero, cudaStream_t st);
+                     uint32_t* d_flags, cudaStream_t st);
 void launch_sp_init(const SpLayer* d_layers, int n_layers, const TileRef* d_diag_tiles, int n_diag_tiles, cudaStream_t st);
 void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
 void launch_sp_scale(const SpLayer* d_layers, int n_layers, cudaStream_t st);   // trace, then scaling
