@@ -66,7 +66,8 @@ struct atomo_ctx {
   bool tc_ok = false;                // tensor-map entry point found
   int eig_scheme = 3;                // eigen-solve: 0 = Jacobi, one launch per step, 1 = persistent (cooperative), 2 = clusters first, 3 = tridiagonal route first
   int tri_clusters = -1;             // co-resident clusters of the tridiagonal reduction (-1 = not asked yet, 0 = unavailable)
-  int tri_big_ok = -1;               // blocked tridiagonal reduction for short sides above 512 (-1 = not asked yet)
+  int tri_big_ok = -1;               // two-stage tridiagonal reduction for short sides above 512 (-1 = not asked yet)
+  int band_capacity[13];             // co-resident CTAs of its first stage, by ceil(log2(short side)) (-1 = not asked yet)
   int tri_big_ctas = 0;              // CTAs per layer of that reduction: 0 = chosen per batch, else 1, 2, 4, 8 or 16
   int eig_scheme_used = -1;          // what the last spectral encode actually ran
   int ew_format = ATOMO_EW_EXPLICIT; // payload format of entry-wise encodes
@@ -76,6 +77,7 @@ struct atomo_ctx {
   int64_t ew_sat_cap = 0;            // compact format: capacity of the saturated list
   int cluster_capacity[16] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};   // by log2(rp_max), -1 = not asked yet
   std::string err;
+  atomo_ctx() { for (int& c : band_capacity) c = -1; }
 };
 
 namespace {
@@ -545,8 +547,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     if (ctx->tri_clusters < 1) tri_form = false;
   }
   if (tri_form && any_big) {
-    if (ctx->tri_big_ok < 0) ctx->tri_big_ok = (sp_configure_tridiag_big() == 0 && sp_configure_bisect() == 0) ? 1 : 0;
-    if (ctx->tri_big_ok < 1 || r_max > sp_tridiag_big_max_r()) tri_form = false;
+    if (ctx->tri_big_ok < 0) ctx->tri_big_ok = (sp_configure_band() == 0 && sp_configure_eigvec_big() == 0 && sp_configure_bisect() == 0) ? 1 : 0;
+    if (ctx->tri_big_ok < 1 || r_max > sp_band_max_r()) tri_form = false;
   }
   std::vector<int> big_layers;
   for (int l = 0; l < n_layers; ++l) {
@@ -626,6 +628,50 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     }
     n_clusters = (int)used.size();
   }
+  // two-stage reduction of the large layers, largest first: CTAs of the first stage dealt in proportion to the work (r^3); a
+  // launch holds as many as are resident together (they wait for one another), further layers take another launch
+  struct BandRun { int first, count, r_max; };
+  std::vector<BandRun> band_runs;
+  std::vector<ClusterCta> band_ctas;
+  if (tri_form && any_big) {
+    std::stable_sort(big_layers.begin(), big_layers.end(), [&](int a, int b) { return L[a].r > L[b].r; });
+    for (size_t i = 0; i < big_layers.size();) {
+      const int rm = L[big_layers[i]].r;
+      int lg = 0;
+      while ((1 << lg) < rm) ++lg;
+      if (ctx->band_capacity[lg] < 0) ctx->band_capacity[lg] = sp_band_capacity(1 << lg);
+      const int room = ctx->band_capacity[lg];
+      if (room < 1) { tri_form = false; break; }
+      const int fixed = ctx->tri_big_ctas;                           // CTAs per layer asked for (0: chosen here)
+      size_t n = 0;
+      int used = 0;
+      double work = 0.0;
+      while (i + n < big_layers.size()) {
+        const int want = fixed > 0 ? std::min(fixed, sp_band_strips(L[big_layers[i + n]].r)) : 1;
+        if (used + want > room) break;
+        used += want;
+        const double rr = L[big_layers[i + n]].r;
+        work += rr * rr * rr;
+        ++n;
+      }
+      if (n == 0) { tri_form = false; break; }
+      std::vector<int> g(n);
+      int total = 0;
+      for (size_t q = 0; q < n; ++q) {
+        const double rr = L[big_layers[i + q]].r;
+        const int strips = sp_band_strips(L[big_layers[i + q]].r);
+        g[q] = fixed > 0 ? std::min(fixed, strips) : std::max(1, std::min(strips, (int)(room * (rr * rr * rr / work))));
+        total += g[q];
+      }
+      for (size_t q = n; total > room; q = q > 1 ? q - 1 : n) if (g[q - 1] > 1) { --g[q - 1]; --total; }   // the minimum of one each went over
+      BandRun run{(int)band_ctas.size(), 0, rm};
+      for (size_t q = 0; q < n; ++q) for (int c = 0; c < g[q]; ++c) band_ctas.push_back(ClusterCta{big_layers[i + q], c, 0, g[q]});
+      run.count = (int)band_ctas.size() - run.first;
+      band_runs.push_back(run);
+      i += n;
+    }
+    if (!tri_form) { for (int l = 0; l < n_layers; ++l) L[l].tri = 0; return fail_cuda(ctx, cudaErrorInvalidConfiguration, "occupancy query for the band reduction"); }
+  }
   // the tables go to the table cache (device buffer tab_sp, host mirror `tables` with the same offsets), everything
   // the kernels write to the workspace
   SpLayer* d_layers = nullptr; TileRef *d_gram = nullptr, *d_pairs = nullptr, *d_bp = nullptr, *d_chol = nullptr, *d_ref = nullptr, *d_tc = nullptr;
@@ -633,6 +679,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   uint32_t* d_flag = nullptr;
   ClusterCta* d_ctas = nullptr;
   int* d_big = nullptr;
+  ClusterCta* d_band = nullptr;
   const float** d_given = nullptr;
   atomo_layer_header* d_hdr_tmpl = nullptr;
   std::vector<uint8_t> tables;
@@ -654,6 +701,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     d_maps = T.take<uint8_t>(maps_blob.size());
     d_ctas = T.take<ClusterCta>(ctas.size());
     d_big = T.take<int>(big_layers.size());
+    d_band = T.take<ClusterCta>(band_ctas.size());
     d_given = T.take<const float*>(given ? (size_t)2 * n_layers : 0);
     d_hdr_tmpl = T.take<atomo_layer_header>(n_layers);
     table_bytes = T.off + 256;
@@ -693,13 +741,16 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.td_tau = A.take<double>(d.tri ? d.rp : 0); d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
       d.td_V = A.take<float>(d.tri ? (size_t)d.r * d.td_ldv : 0);
-      d.tb_fp64 = 0;
-      d.tb_ldw = (d.r + 3) / 4 * 4;
-      d.tb_W = A.take<float>(d.tri == 2 ? (size_t)sp_tridiag_big_panel() * d.tb_ldw : 0);
       d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);
       {
-        const size_t nb = (size_t)(d.r + 31) / 32;
-        d.tb_At = A.take<float>(d.tri == 2 && d.r <= 1024 ? nb * (nb + 1) / 2 * 1024 : 0);
+        const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
+        d.bd_parts = sp_band_parts(d.r);
+        d.bd_U = A.take<float>(on * rows * kBandWidth); d.bd_W = A.take<float>(on * rows * kBandWidth);
+        d.bd_X = A.take<float>(on * kBandWidth * ((d.r + 3) / 4 * 4));
+        d.bd_part = A.take<double>(on * d.bd_parts * rows * kBandWidth);
+        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<double>(on * sp_band_strips(d.r) * kBandWidth * kBandWidth);
+        d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
+        d.bd_V2 = A.take<float>(on * d.r * sp_band_steps(d.r) * kBandWidth);
       }
       d.chol_dd = A.take<float>(32 * 32 + 32);
       d.row_inv = A.take<float>(d.rp);
@@ -713,7 +764,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     // zero-filled region: rotation counters and the X matrices
     uint8_t* zb = reinterpret_cast<uint8_t*>(A.take<uint32_t>(0));
     size_t z0 = A.off;
-    for (int l = 0; l < n_layers; ++l) { L[l].rot_count = A.take<uint32_t>(max_sweeps); L[l].step_bar = A.take<uint32_t>(1); L[l].vec_ticket = A.take<uint32_t>(1); }
+    for (int l = 0; l < n_layers; ++l) { L[l].rot_count = A.take<uint32_t>(max_sweeps); L[l].step_bar = A.take<uint32_t>(1); L[l].vec_ticket = A.take<uint32_t>(1); L[l].bd_bar = A.take<uint32_t>(1); }
     for (int l = 0; l < n_layers; ++l) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       L[l].gram_ticket = A.take<uint32_t>(L[l].tc && L[l].gram_split > 1 ? (size_t)tt * (tt + 1) / 2 : 0);
@@ -723,7 +774,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     for (int l = 0; l < n_layers; ++l) {
       SpLayer& d = L[l];
       if (d.acc) { d.A = d.X; d.lda = d.ldx; }
-      else if (d.tri == 2) { d.lda = (d.r + 3) / 4 * 4; d.A = A.take<float>((size_t)d.r * d.lda); d.tb_A = d.A; }   // 16-byte rows
+      else if (d.tri == 2) { d.lda = (d.r + 3) / 4 * 4; d.A = A.take<float>((size_t)d.r * d.lda); }   // 16-byte rows
       else { d.A = A.take<float>((size_t)d.r * d.r); d.lda = d.r; }
     }
     need = A.off + 256;
@@ -754,6 +805,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   put(d_maps, maps_blob.data(), maps_blob.size());
   put(d_ctas, ctas.data(), ctas.size() * sizeof(ClusterCta));
   put(d_big, big_layers.data(), big_layers.size() * sizeof(int));
+  put(d_band, band_ctas.data(), band_ctas.size() * sizeof(ClusterCta));
   if (given) {
     std::vector<const float*> ptrs(2 * (size_t)n_layers);
     for (int l = 0; l < n_layers; ++l) { ptrs[l] = given_sigma[l]; ptrs[n_layers + l] = given_short[l]; }
@@ -797,28 +849,17 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(tridiagonal reduction)");
       ++n_eig_launch;
     }
-    if (!big_layers.empty()) {
-      // larger layers: a cluster of C CTAs each.  C is the smallest that holds the rows; it is doubled while the
-      // batch still leaves SMs idle (the result does not depend on C)
-      int sms = 148, dev = 0;
-      if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      int cmin = 1, rb = 0;
-      for (int l : big_layers) { cmin = std::max(cmin, sp_tridiag_big_min_ctas(L[l].r)); rb = std::max(rb, L[l].r); }
-      int cc = cmin;
-      if (ctx->tri_big_ctas > 0) cc = std::max(cmin, ctx->tri_big_ctas);
-      else {
-        // (clusters sit inside one GPC each: the GPU holds fewer of them than SMs / CTAs, so ask)
-        auto fits = [&](int c2) {
-          const int mc = sp_tridiag_big_max_clusters(c2, rb);
-          return mc > 0 ? (int)big_layers.size() <= mc : (int)big_layers.size() * c2 <= sms;
-        };
-        while (cc < 16 && fits(cc * 2)) cc *= 2;
-        // up to a short side of 1024 one CTA per layer runs the triangle-only kernel, which beats a pair of CTAs on full
-        // rows (40 layers: 25 ms against 36 ms); clusters pay from four CTAs per layer on
-        if (cc == 2 && rb <= 1024) cc = 1;
-      }
-      const int e = launch_sp_tridiag_big(d_layers, d_big, (int)big_layers.size(), rb, cc, 0, st);
-      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(blocked tridiagonal reduction)");
+    for (const BandRun& b : band_runs) {                             // larger layers: to a band, then to tridiagonal form
+      const int e = launch_sp_band(d_layers, d_band + b.first, b.count, b.r_max, d_flag + 1, st);
+      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(band reduction)");
+      ++n_eig_launch;
+    }
+    for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one cluster size are neighbours)
+      const int c = sp_chase_ctas(L[big_layers[i]].r);
+      n = 1;
+      while (i + n < big_layers.size() && sp_chase_ctas(L[big_layers[i + n]].r) == c) ++n;
+      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
+      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(bulge chase)");
       ++n_eig_launch;
     }
     // the eigenvalues (bisection) are timed with the sampling stage.  No host wait on this route: a bounded wait of

@@ -63,6 +63,7 @@ void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax
 
 // ================================= spectral path =================================================
 constexpr int kMaxShort = 4096;       // largest short side (atoms per layer)
+constexpr int kBandWidth = 8;         // sub-diagonals between the two stages of the large layers' reduction
 constexpr int kSmemRowsMaxRp = 4096;  // largest padded short side the shared-memory Jacobi kernel holds
 
 struct SpLayer {
@@ -104,14 +105,15 @@ struct SpLayer {
   float* td_V;                 // r x td_ldv: row k = v_k / ||v_k|| (zero up to index k), fp32 for the back-transformation: H_k = I - 2 u u^T
   double* lam64;               // rp: eigenvalues of T, ascending (scaled units); lam holds the same in fp32
   uint32_t* vec_ticket;        // CTAs of the vector kernel that finished this layer; zeroed per call
-  // tridiagonal route for short sides above 512 (tri = 2): blocked Householder reduction with A in global memory
-  void* tb_A;                  // r x lda matrix the reduction works on: float (= A) or double (tb_fp64)
-  void* tb_W;                  // [panel][tb_ldw] the panel's w vectors, same type as tb_A
-  int64_t tb_ldw;
-  int tb_fp64;                 // matrix and panel vectors in fp64
+  // tridiagonal route for short sides above 512 (tri = 2): dense -> band -> tridiagonal
+  float* bd_U; float* bd_W;    // [rows padded to strips][8] panel vectors of the panel before
+  float* bd_X;                 // [8][lda] entries of the next panel
+  double* bd_part; int bd_parts; // [parts][rows padded to strips][8] partial products, tasks per strip
+  double* bd_P; double* bd_S;  // [rows padded to strips][8] product A U; [strips][64] U^T A U per strip
+  double* bd_band;             // [r][9] the band, by column
+  float* bd_V2;                // [r][steps][8] reflectors of the chase: sweep, step
+  uint32_t* bd_bar;            // arrivals at the layer's barriers; zeroed per call
   double* tb_vecwork;          // [slots][5][rp] work vectors of the twisted factorisation
-  float* tb_At;                // short side <= 1024: the lower triangle in tile-major order (32 x 32 sub-tiles of 4 KB), the
-                               // working copy of the one-CTA-per-layer kernel
 };
 
 struct SpDecodeLayer {
@@ -155,15 +157,19 @@ int sp_configure_tridiag();                                       // co-resident
 int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_clusters, int rp_max, cudaStream_t st);  // cudaError_t
 void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t n_eigenvalues, cudaStream_t st);
 void launch_sp_eigvec(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st);
-// tridiagonal route for short sides above 512 (atomo_tridiag_big.cu)
-int sp_tridiag_big_max_r();
-int sp_tridiag_big_panel();
-int sp_tridiag_big_min_ctas(int r);                               // fewest CTAs per layer that hold r rows
+// tridiagonal route for short sides above 512 (atomo_band.cu, vectors in atomo_tridiag_big.cu)
+int sp_band_max_r();
+int sp_band_strips(int r);
+int sp_band_parts(int r);
+int sp_band_steps(int r);
+int sp_band_capacity(int r_max);                                  // co-resident CTAs of the band reduction (0: not available)
+int sp_configure_band();                                          // 0 if available
+int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int r_max, uint32_t* d_timeout, cudaStream_t st);  // cudaError_t
+int sp_chase_ctas(int r);                                         // CTAs per layer of the chase
+int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st);   // cudaError_t
 int sp_eigvec_big_slots();                                        // warps per layer of the vector kernel (work vectors)
-int sp_configure_tridiag_big();                                   // 0 if available
-int sp_tridiag_big_max_clusters(int ctas, int r_max);              // co-resident clusters of that many CTAs (0: unknown)
+int sp_configure_eigvec_big();                                    // 0 if available
 int sp_configure_bisect();                                        // 0 if the eigenvalue kernel got its shared memory
-int launch_sp_tridiag_big(const SpLayer* d_layers, const int* d_big, int n_big, int r_max, int ctas, int fp64, cudaStream_t st);  // cudaError_t
 void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rp_max, cudaStream_t st);
 int launch_sp_cholesky(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st);
 int launch_sp_cholesky_big(const SpLayer* d_layers, const TileRef* d_ctas, int n_ctas, int max_panels, cudaStream_t st);
