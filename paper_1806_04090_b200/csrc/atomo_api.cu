@@ -67,7 +67,7 @@ struct atomo_ctx {
   int eig_scheme = 3;                // eigen-solve: 0 = Jacobi, one launch per step, 1 = persistent (cooperative), 2 = clusters first, 3 = tridiagonal route first
   int tri_clusters = -1;             // co-resident clusters of the tridiagonal reduction (-1 = not asked yet, 0 = unavailable)
   int tri_big_ok = -1;               // two-stage tridiagonal reduction for short sides above 512 (-1 = not asked yet)
-  int band_capacity[13];             // co-resident CTAs of its first stage, by ceil(log2(short side)) (-1 = not asked yet)
+  int band_capacity[2][13];          // co-resident CTAs of its first stage, by instance and ceil(log2(short side)) (-1 = not asked yet)
   int tri_big_ctas = 0;              // CTAs per layer of that reduction: 0 = chosen per batch, else 1, 2, 4, 8 or 16
   int eig_scheme_used = -1;          // what the last spectral encode actually ran
   int ew_format = ATOMO_EW_EXPLICIT; // payload format of entry-wise encodes
@@ -77,7 +77,7 @@ struct atomo_ctx {
   int64_t ew_sat_cap = 0;            // compact format: capacity of the saturated list
   int cluster_capacity[16] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};   // by log2(rp_max), -1 = not asked yet
   std::string err;
-  atomo_ctx() { for (int& c : band_capacity) c = -1; }
+  atomo_ctx() { for (auto& f : band_capacity) for (int& c : f) c = -1; }
 };
 
 namespace {
@@ -630,17 +630,22 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   }
   // two-stage reduction of the large layers, largest first: CTAs of the first stage dealt in proportion to the work (r^3); a
   // launch holds as many as are resident together (they wait for one another), further layers take another launch
-  struct BandRun { int first, count, r_max; };
+  struct BandRun { int first, count, form, r_max; };
   std::vector<BandRun> band_runs;
   std::vector<ClusterCta> band_ctas;
+  int band_form = 0;
   if (tri_form && any_big) {
     std::stable_sort(big_layers.begin(), big_layers.end(), [&](int a, int b) { return L[a].r > L[b].r; });
+    int64_t strips = 0;
+    for (int l : big_layers) strips += sp_band_strips(L[l].r);
+    band_form = sp_band_form(L[big_layers[0]].r, strips);
     for (size_t i = 0; i < big_layers.size();) {
       const int rm = L[big_layers[i]].r;
       int lg = 0;
       while ((1 << lg) < rm) ++lg;
-      if (ctx->band_capacity[lg] < 0) ctx->band_capacity[lg] = sp_band_capacity(1 << lg);
-      const int room = ctx->band_capacity[lg];
+      int& room_known = ctx->band_capacity[band_form][lg];
+      if (room_known < 0) room_known = sp_band_capacity(band_form, 1 << lg);
+      const int room = room_known;
       if (room < 1) { tri_form = false; break; }
       const int fixed = ctx->tri_big_ctas;                           // CTAs per layer asked for (0: chosen here)
       size_t n = 0;
@@ -664,7 +669,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         total += g[q];
       }
       for (size_t q = n; total > room; q = q > 1 ? q - 1 : n) if (g[q - 1] > 1) { --g[q - 1]; --total; }   // the minimum of one each went over
-      BandRun run{(int)band_ctas.size(), 0, rm};
+      BandRun run{(int)band_ctas.size(), 0, band_form, rm};
       for (size_t q = 0; q < n; ++q) for (int c = 0; c < g[q]; ++c) band_ctas.push_back(ClusterCta{big_layers[i + q], c, 0, g[q]});
       run.count = (int)band_ctas.size() - run.first;
       band_runs.push_back(run);
@@ -744,11 +749,11 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);
       {
         const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
-        d.bd_parts = sp_band_parts(d.r);
         d.bd_U = A.take<float>(on * rows * kBandWidth); d.bd_W = A.take<float>(on * rows * kBandWidth);
-        d.bd_X = A.take<float>(on * kBandWidth * ((d.r + 3) / 4 * 4));
-        d.bd_part = A.take<double>(on * d.bd_parts * rows * kBandWidth);
-        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<double>(on * sp_band_strips(d.r) * kBandWidth * kBandWidth);
+        d.bd_X = A.take<float>(on * rows * kBandWidth);
+        d.bd_part = A.take<double>(on * sp_band_parts(band_form) * rows * kBandWidth);
+        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<long long>(on * sp_band_strips(d.r) * kBandWidth * kBandWidth);
+        d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
         d.bd_V2 = A.take<float>(on * d.r * sp_band_steps(d.r) * kBandWidth);
       }
@@ -774,7 +779,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     for (int l = 0; l < n_layers; ++l) {
       SpLayer& d = L[l];
       if (d.acc) { d.A = d.X; d.lda = d.ldx; }
-      else if (d.tri == 2) { d.lda = (d.r + 3) / 4 * 4; d.A = A.take<float>((size_t)d.r * d.lda); }   // 16-byte rows
+      else if (d.tri == 2) { d.lda = (int64_t)sp_band_strips(d.r) * 64; d.A = A.take<float>((size_t)d.r * d.lda); }   // whole strips
       else { d.A = A.take<float>((size_t)d.r * d.r); d.lda = d.r; }
     }
     need = A.off + 256;
@@ -850,7 +855,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       ++n_eig_launch;
     }
     for (const BandRun& b : band_runs) {                             // larger layers: to a band, then to tridiagonal form
-      const int e = launch_sp_band(d_layers, d_band + b.first, b.count, b.r_max, d_flag + 1, st);
+      const int e = launch_sp_band(d_layers, d_band + b.first, b.count, b.form, b.r_max, d_flag + 1, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(band reduction)");
       ++n_eig_launch;
     }

@@ -37,24 +37,31 @@ static_assert(kBw == 8, "the operand vectors are two float4");
 // layer's G CTAs take the strips in turn.  A[j][i] with i in the strip is read as row j, two neighbouring entries per lane
 // (256 bytes per warp), so a lane keeps everything of its two rows -- their entries of U and W of the panel before, and
 // their eight sums of the product -- in registers and walks over the columns j, whose U, W and new U entries are broadcast
-// from shared memory: 48 multiply-adds per 8 bytes read and written and six 16-byte broadcasts, no exchange between lanes.
-// The columns of a strip are split into `parts` tasks for the warps; the parts of a sum are added in fp64 in a fixed order
-// that depends on neither G nor the batch.
+// from shared memory: 48 multiply-adds per 8 bytes read and written and six 16-byte broadcasts, no exchange between lanes
+// (17 cycles per column and warp on an SM, 70 % of the FMA rate, when the data is at hand).  The columns of a strip are split
+// into PARTS tasks for the warps; the parts of a sum are added in fp64.
+// The panel's QR is a Householder QR worked out on 8 x 8 matrices: the reflectors' norms and products follow from the panel's
+// Gram matrix (downdated as rows of R split off) and its first eight rows, and below those rows V = X K with an 8 x 8 matrix
+// K.  A column whose remainder is below 3e-8 of it is left alone (the fp32 panel has no more digits).  However inexact V is
+// for an ill-conditioned panel, Q stays orthogonal: T comes from the actual dots of the rounded U.
 // A panel has two barriers among the layer's CTAs:
-//   every CTA: QR of the whole panel (redundant: its entries are exchanged anyway, and the chain of eight column steps is
-//              what a panel costs when little of the matrix is left)
-//   pass:      own strips: update with the panel before, product with this panel's U; S = U^T A U per strip      -> barrier
-//   every CTA: T^T S T; own rows: W = (A U) T - 1/2 U (T^T S T), entries of the next panel                     -> barrier
-// With two CTAs per SM, which belong to different layers, one's chains and barriers overlap with the other's pass.
+//   every CTA: Gram matrix and first rows of the panel in, 8 x 8 factorisation (one warp), U = X K for all rows
+//   pass:      own strips: update with the panel before, product with this panel's U; U^T A U and U^T U        -> barrier
+//   every CTA: T, T^T (U^T A U) T; own rows: W = (A U) T - 1/2 U T^T (U^T A U) T, entries of the next panel and their Gram
+//              matrix                                                                                          -> barrier
+// Sums over rows are formed per strip (or half strip) in an order of their own and added up in strip order, U^T A U in fixed
+// point, so the result does not depend on G.  With two CTAs per SM, which belong to different layers, one's chains and
+// barriers overlap with the other's pass.
 namespace {
 
+constexpr double kFix = 1125899906842624.0;   // 2^50: U^T A U in fixed point (|entries| <= 1)
+
 struct BandShared {
-  double red[2][16][8];           // per warp: parts of the panel's dots (alternating buffers)
-  double m[16][36];               // per warp: parts of U^T U
   double T[8][8], S[8][8], Y[8][8], X[8][8];
-  float Wc[8][8];                 // W of the next panel's pivot rows
-  double piv[2][8];               // entries of the pivot row (alternating buffers)
-  double M[36];
+  double K[8][8], vtop[8][8];     // K scaled to unit vectors; the reflectors' entries in the panel's first eight rows
+  double M[36], G[36], sum[16][36];
+  double top[8][8];
+  double Wc[8][8], Uc[8][8];      // W and U of the next panel's pivot rows
   uint32_t fail;
 };
 
@@ -71,6 +78,28 @@ __device__ __forceinline__ double band_scatter8(const double (&v)[8], int lane) 
   c += __shfl_xor_sync(0xffffffffu, c, 1);
   return c;
 }
+// the 36 dots of the columns of a 32 x 8 block, one row (a, b) per lane, to dst (lower triangle by rows).  (Out of line: what runs
+// once per panel has to stay small.  A panel is a walk through the whole kernel, and straight-line code that no longer fits
+// the instruction cache costs its misses every time: the 8 x 8 factorisation unrolled took 52 k cycles, rolled up 7 k.)
+__device__ __noinline__ void band_gram32(const float4 a, const float4 b, double* __restrict__ dst, int lane) {
+  const double d[8] = {(double)a.x, (double)a.y, (double)a.z, (double)a.w, (double)b.x, (double)b.y, (double)b.z, (double)b.w};
+  double acc[40];
+  int e = 0;
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+#pragma unroll
+    for (int q = 0; q <= p; ++q, ++e) acc[e] = d[p] * d[q];
+#pragma unroll
+  for (int q = 36; q < 40; ++q) acc[q] = 0.0;
+#pragma unroll
+  for (int e0 = 0; e0 < 40; e0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = acc[e0 + q];
+    const double s = band_scatter8(v, lane);
+    if ((lane & 3) == 0 && e0 + (lane >> 2) < 36) dst[e0 + (lane >> 2)] = s;
+  }
+}
 
 // barrier among the layer's CTAs (co-resident: cooperative launch), bounded; a wait that runs out shows as
 // ATOMO_ERR_TIMEOUT in the layers' status words
@@ -85,13 +114,88 @@ __device__ __forceinline__ void band_barrier(uint32_t* ctr, uint32_t target, Ban
     }
     __threadfence();
   }
+  __syncwarp();                                              // (without it the polling thread's warp may stay divided past the barrier)
   __syncthreads();
+}
+
+// sums of 36 values over `n` blocks of global memory, in an order that depends on THREADS alone; complete after the caller's
+// next barrier but one (this function has one inside)
+template <int THREADS>
+__device__ __forceinline__ void band_sum36(const double* __restrict__ src, int first, int n, double (*part)[36], double* __restrict__ dst) {
+  constexpr int kGroups = THREADS / 36 < 16 ? THREADS / 36 : 16;
+  const int tid = threadIdx.x, gr = tid / 36, e = tid % 36;
+  if (gr < kGroups) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = first / kGroups * kGroups + gr; b < n; b += kGroups) if (b >= first) s += __ldcg(src + (int64_t)b * 36 + e);
+    part[gr][e] = s;
+  }
+  __syncthreads();
+  if (tid < 36) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < kGroups; ++q) s += part[q][tid];
+    dst[tid] = s;
+  }
+}
+
+// Householder QR of the panel on its Gram matrix (lower triangle in sh.G) and first eight rows (sh.top), one warp.  Lane:
+// column l = lane % 8, rows lane / 8 and lane / 8 + 4.  Leaves R in sh.top, the unit reflectors' entries in the first eight rows
+// in sh.vtop (zero above the diagonal) and K, scaled likewise.
+__device__ __noinline__ void band_small_qr(BandShared& sh, const int n_ref, const int lane) {
+  // The warp has to be whole here: left divided by an earlier branch it takes 52 k cycles instead of 6 k
+  __syncwarp();
+  const int l = lane & 7, i0 = lane >> 3;
+  double top[2], g[2], k[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = i0 + 4 * h;
+    top[h] = sh.top[i][l];
+    g[h] = sh.G[i >= l ? i * (i + 1) / 2 + l : l * (l + 1) / 2 + i];
+    k[h] = i == l ? 1.0 : 0.0;
+  }
+  const double orig = sh.G[l * (l + 1) / 2 + l];             // squared norm of column l as given
+#pragma unroll 1
+  for (int t = 0; t < 8; ++t) {
+    const bool up = t >= 4;                                  // row t: register up of the lanes tl ..
+    const int tl = (t & 3) * 8;
+    const double g_of = up ? g[1] : g[0], top_of = up ? top[1] : top[0];
+    const double gt = __shfl_sync(0xffffffffu, g_of, tl + l), tt = __shfl_sync(0xffffffffu, top_of, tl + l);
+    const double nx2 = __shfl_sync(0xffffffffu, gt, t), x0 = __shfl_sync(0xffffffffu, tt, t), o = __shfl_sync(0xffffffffu, orig, t);
+    double alpha = x0, beta = 0.0, un = 0.0;
+    const bool act = t < n_ref && nx2 > 1.0e-290 && nx2 > 1.0e-15 * o;   // else H = I: a zero column, or no digits left
+    if (act) {
+      const double nx = nx2 * rsqrt(nx2);
+      alpha = -copysign(nx, x0);
+      const double half = fma(fabs(x0), nx, nx2);            // v^T v / 2
+      un = rsqrt(2.0 * half);
+      beta = 2.0 * un * un;
+    }
+    const double gl = l > t ? beta * (gt - alpha * tt) : 0.0;   // beta v^T x_l
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + 4 * h;
+      const double xi = __shfl_sync(0xffffffffu, top[h], (lane & 24) + t), ki = __shfl_sync(0xffffffffu, k[h], (lane & 24) + t);
+      const double v = i > t ? xi : i == t ? x0 - alpha : 0.0;
+      if (l > t) { top[h] = fma(-gl, v, top[h]); k[h] = fma(-gl, ki, k[h]); }
+      if (l == t) {
+        sh.vtop[i][t] = v * un;
+        sh.K[i][t] = ki * un;
+        if (act) top[h] = i == t ? alpha : i > t ? 0.0 : top[h];
+      }
+    }
+    const double r_of = up ? top[1] : top[0], rl = __shfl_sync(0xffffffffu, r_of, tl + l);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) g[h] = fma(-__shfl_sync(0xffffffffu, r_of, tl + i0 + 4 * h), rl, g[h]);   // row t of R leaves the Gram matrix
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) sh.top[i0 + 4 * h][l] = top[h];
 }
 
 }  // namespace
 
-// THREADS threads hold RPT panel rows each (as type PT); MINB CTAs per SM
-template <int THREADS, int RPT, typename PT, int MINB>
+// A CTA of THREADS threads, MINB per SM
+template <int THREADS, int MINB, int PARTS>
 __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* __restrict__ layers, const ClusterCta* __restrict__ ctas,
                                                                 const int cap, uint32_t* __restrict__ timeout_flag) {
   constexpr int kWarps = THREADS / 32;
@@ -102,163 +206,120 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int r = L.r, g = me.slot, G = me.pad;
   const int n_strips = (r + kStrip - 1) / kStrip;
-  float* const A = L.A; const int64_t lda = L.lda;
+  float* const A = L.A; const int64_t lda = L.lda;           // lda is a multiple of the strip: whole strips may be read and written
   float* const gU = L.bd_U; float* const gW = L.bd_W; float* const gX = L.bd_X;
-  double* const gPart = L.bd_part; double* const gP = L.bd_P; double* const gS = L.bd_S; double* const gB = L.bd_band;
+  double* const gPart = L.bd_part; double* const gP = L.bd_P; long long* const gS = L.bd_S; double* const gB = L.bd_band;
+  double* const gG = L.bd_G; double* const gM = L.bd_M;
   float* const gV = L.td_V; const int64_t ldv = L.td_ldv;
   float* const s_u = band_smem;                              // [r][8] this panel's U, by row
   float* const s_ops = band_smem + (size_t)r * 8;            // [cap][16] U and W of the panel before, columns col0 ..
   if (tid == 0) sh.fail = 0u;
   uint32_t arrivals = 0;
-  // the first panel as it stands: entries A[t][i] of the own strips
-  for (int s = g; s < n_strips; s += G)
-    for (int q = tid; q < kStrip * 8; q += THREADS) {
-      const int t = q / kStrip, i = s * kStrip + q % kStrip;
-      if (i < r && t < r) gX[(int64_t)t * lda + i] = A[(int64_t)t * lda + i];
-    }
-  arrivals += (uint32_t)G;
-  band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
-
   for (int c = 0; c < r; c += kBw) {
+    // ---- own rows: U and W of the panel before out, entries of this panel (columns c .. c+7) and the Gram matrix of those
+    // below the band; half a strip per warp ----
+    {
+      const int s_lo = c / kStrip, s_own = s_lo + ((g - s_lo % G) % G + G) % G;
+      for (int n = w;; n += kWarps) {
+        const int half = 2 * (s_own + n / 2 * G) + (n & 1);
+        if (half >= 2 * n_strips) break;
+        const int i = half * 32 + lane;
+        const bool in = i >= c && i < r;
+        float x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = in && c + t < r ? __ldcg(A + (int64_t)(c + t) * lda + i) : 0.0f;
+        if (c > 0) {
+          float uu[8], ww[8];
+          double p[8];
+          const double2* src = reinterpret_cast<const double2*>(gP + (int64_t)i * 8);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) { const double2 d = in ? src[t] : make_double2(0.0, 0.0); p[2 * t] = d.x; p[2 * t + 1] = d.y; }
+#pragma unroll
+          for (int t = 0; t < 8; ++t) uu[t] = in ? s_u[(size_t)i * 8 + t] : 0.0f;
+          double z[8];                                       // W[i][t] = sum_s P[i][s] T[s][t] - 1/2 sum_s U[i][s] (T^T S T)[s][t]
+#pragma unroll
+          for (int t = 0; t < 8; ++t) z[t] = 0.0;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { if (q <= t) z[t] = fma(p[q], sh.T[q][t], z[t]); z[t] = fma((double)uu[q], sh.X[q][t], z[t]); }
+          }
+#pragma unroll
+          for (int t = 0; t < 8; ++t) { ww[t] = (float)z[t]; z[t] = (double)x[t]; }
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const double uq = (double)uu[q], wq = (double)ww[q];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) z[t] -= fma(uq, sh.Wc[t][q], wq * sh.Uc[t][q]);
+          }
+#pragma unroll
+          for (int t = 0; t < 8; ++t) x[t] = in && c + t < r ? (float)z[t] : 0.0f;
+          float4* du = reinterpret_cast<float4*>(gU + (int64_t)i * 8);
+          float4* dw = reinterpret_cast<float4*>(gW + (int64_t)i * 8);
+          du[0] = make_float4(uu[0], uu[1], uu[2], uu[3]); du[1] = make_float4(uu[4], uu[5], uu[6], uu[7]);
+          dw[0] = make_float4(ww[0], ww[1], ww[2], ww[3]); dw[1] = make_float4(ww[4], ww[5], ww[6], ww[7]);
+        }
+        float4 lo = make_float4(x[0], x[1], x[2], x[3]), hi = make_float4(x[4], x[5], x[6], x[7]);
+        float4* dx = reinterpret_cast<float4*>(gX + (int64_t)i * 8);
+        dx[0] = lo; dx[1] = hi;
+        if (i < c + kBw) { lo = make_float4(0.f, 0.f, 0.f, 0.f); hi = lo; }
+        band_gram32(lo, hi, gG + (int64_t)half * 36, lane);
+      }
+    }
+    arrivals += (uint32_t)G;
+    band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
+    if (sh.fail) break;
     const int row0 = c + kBw;                                // first row below the band of the panel
     const int m = r - row0;                                  // panel rows
+    const int c_strip = c / kStrip, first_strip = row0 / kStrip;
     // ---- diagonal block, QR of the panel (every CTA) ----
     if (g == 0 && tid < kBw * kBw) {
       const int a = tid / kBw, b = tid % kBw;                // entry (c + a, c + b), a >= b
-      if (a >= b && c + a < r) gB[(int64_t)(c + b) * (kBw + 1) + a - b] = (double)__ldcg(gX + (int64_t)b * lda + c + a);
+      if (a >= b && c + a < r) gB[(int64_t)(c + b) * (kBw + 1) + a - b] = (double)__ldcg(gX + (int64_t)(c + a) * 8 + b);
     }
     if (m <= 0) break;
-    PT x[RPT][8];
-#pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-      const int i = row0 + tid + q * THREADS;
-#pragma unroll
-      for (int t = 0; t < 8; ++t) x[q][t] = i < r ? (PT)__ldcg(gX + (int64_t)t * lda + i) : (PT)0;
+    if (tid >= THREADS - 64) {
+      const int q = tid - (THREADS - 64), a = q / 8, b = q % 8;
+      sh.top[a][b] = row0 + a < r ? (double)__ldcg(gX + (int64_t)(row0 + a) * 8 + b) : 0.0;
     }
-    const int n_ref = min(kBw, m - 1);                       // reflectors of this panel: rows row0 + t .. r-1, at least two of them
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      if (t < n_ref) {
-        // dots of column t with the columns t .. 7 over the rows row0 + t .. (rows above carry zeros in column t: see below)
-        double d[8];
-#pragma unroll
-        for (int l = 0; l < 8; ++l) {
-          d[l] = 0.0;
-          if (l >= t) {
-            PT acc = (PT)0;
-#pragma unroll
-            for (int q = 0; q < RPT; ++q) {
-              const bool in = q > 0 || tid >= t;
-              acc = in ? fma(x[q][t], x[q][l], acc) : acc;
-            }
-            d[l] = (double)acc;
-          }
-        }
-        const double part = band_scatter8(d, lane);
-        if ((lane & 3) == 0) sh.red[t & 1][w][lane >> 2] = part;
-        if (tid == t) {
-#pragma unroll
-          for (int l = 0; l < 8; ++l) sh.piv[t & 1][l] = (double)x[0][l];
-        }
-        __syncthreads();
-        double tot = 0.0;
-#pragma unroll
-        for (int ww = 0; ww < kWarps / 4; ++ww) tot += sh.red[t & 1][4 * ww + (lane >> 3)][lane & 7];
-        tot += __shfl_xor_sync(0xffffffffu, tot, 8);
-        tot += __shfl_xor_sync(0xffffffffu, tot, 16);        // lane: the dot with column lane & 7
-        const double nx2 = __shfl_sync(0xffffffffu, tot, t), x0 = sh.piv[t & 1][t];
-        double alpha = 0.0, beta = 0.0, un = 0.0;
-        if (nx2 > 1.0e-290) {                                // below: a zero column (H = I)
-          const double nx = nx2 * rsqrt(nx2);
-          alpha = -copysign(nx, x0);
-          const double half = fma(fabs(x0), nx, nx2);        // v^T v / 2
-          un = rsqrt(2.0 * half);
-          beta = 2.0 * un * un;
-        }
-        const double gl = beta * (tot - alpha * sh.piv[t & 1][lane & 7]);    // beta v^T x_l for l = lane & 7
-        PT gc[8];
-#pragma unroll
-        for (int l = 0; l < 8; ++l) gc[l] = l > t ? (PT)__shfl_sync(0xffffffffu, gl, l) : (PT)0;
-        const PT al = (PT)alpha, us = (PT)un;
-#pragma unroll
-        for (int q = 0; q < RPT; ++q) {
-          const bool below = q > 0 || tid > t, pivot = q == 0 && tid == t;
-          const PT v = below ? x[q][t] : pivot ? x[q][t] - al : (PT)0;
-#pragma unroll
-          for (int l = 0; l < 8; ++l) if (l > t) x[q][l] = fma(-gc[l], v, x[q][l]);
-          const int i = row0 + tid + q * THREADS;
-          if (i < r) s_u[(size_t)i * 8 + t] = (float)(v * us);
-          if (pivot) x[q][t] = al;
-          // (column t of the rows below is not needed any more)
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < RPT; ++q) { const int i = row0 + tid + q * THREADS; if (i < r) s_u[(size_t)i * 8 + t] = 0.0f; }
-      }
-    }
-    // R: rows row0 + a (held by thread a), columns c + t, t >= a (all columns where no reflector acted)
-    if (g == 0 && tid < kBw && row0 + tid < r) {
-#pragma unroll
-      for (int t = 0; t < 8; ++t) if (t >= tid) gB[(int64_t)(c + t) * (kBw + 1) + row0 + tid - (c + t)] = (double)x[0][t];
-    }
+    band_sum36<THREADS>(gG, 2 * c_strip, 2 * n_strips, sh.sum, sh.G);
     __syncthreads();
-    // U^T U of the rounded U, 36 dots; then T (I - U T U^T is the product of the I - tau u u^T with tau = 2 / u^T u)
-    {
-      double acc[36];
+    const int n_ref = min(kBw, m - 1);                       // reflectors of this panel: rows row0 + t .. r-1, at least two of them
+    if (w == 0) band_small_qr(sh, n_ref, lane);
+    __syncthreads();
+    for (int i = row0 + tid; i < r; i += THREADS) {
+      float u[8];
+      if (i < row0 + kBw) {
 #pragma unroll
-      for (int e = 0; e < 36; ++e) acc[e] = 0.0;
-      for (int i = row0 + tid; i < r; i += THREADS) {
-        const float4 a = *reinterpret_cast<const float4*>(s_u + (size_t)i * 8), b = *reinterpret_cast<const float4*>(s_u + (size_t)i * 8 + 4);
-        const double u[8] = {(double)a.x, (double)a.y, (double)a.z, (double)a.w, (double)b.x, (double)b.y, (double)b.z, (double)b.w};
-        int e = 0;
+        for (int t = 0; t < 8; ++t) u[t] = (float)sh.vtop[i - row0][t];
+      } else {
+        const float4 a = __ldcg(reinterpret_cast<const float4*>(gX + (int64_t)i * 8)), b = __ldcg(reinterpret_cast<const float4*>(gX + (int64_t)i * 8) + 1);
+        const double x[8] = {(double)a.x, (double)a.y, (double)a.z, (double)a.w, (double)b.x, (double)b.y, (double)b.z, (double)b.w};
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-#pragma unroll
-          for (int q = 0; q <= p; ++q, ++e) acc[e] = fma(u[p], u[q], acc[e]);
-      }
-#pragma unroll
-      for (int e0 = 0; e0 < 36; e0 += 8) {
-        double v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = e0 + e < 36 ? acc[e0 + e < 36 ? e0 + e : 0] : 0.0;
-        const double sum = band_scatter8(v, lane);
-        if ((lane & 3) == 0 && e0 + (lane >> 2) < 36) sh.m[w][e0 + (lane >> 2)] = sum;
-      }
-      __syncthreads();
-      if (w == 0) {
-        for (int e = lane; e < 36; e += 32) {
-          double s = 0.0;
-          for (int ww = 0; ww < kWarps; ++ww) s += sh.m[ww][e];
-          sh.M[e] = s;
-        }
-        __syncwarp();
-        // column t of T: tau_t in place t, -tau_t T[0:t, 0:t] M[0:t, t] above
         for (int t = 0; t < 8; ++t) {
-          const double mtt = sh.M[t * (t + 1) / 2 + t], tau = mtt > 0.5 ? 2.0 / mtt : 0.0;
           double z = 0.0;
-          if (lane < t) for (int q = lane; q < t; ++q) z = fma(sh.T[lane][q], sh.M[t * (t + 1) / 2 + q], z);
-          __syncwarp();
-          if (lane < 8) sh.T[lane][t] = lane < t ? -tau * z : lane == t ? tau : 0.0;
-          __syncwarp();
+#pragma unroll
+          for (int q = 0; q <= t; ++q) z = fma(x[q], sh.K[q][t], z);
+          u[t] = (float)z;
         }
       }
+      float4* d = reinterpret_cast<float4*>(s_u + (size_t)i * 8);
+      d[0] = make_float4(u[0], u[1], u[2], u[3]); d[1] = make_float4(u[4], u[5], u[6], u[7]);
     }
-    // the reflectors' rows for the back-transformation, own strips (zero above row0 + t)
-    for (int s = g; s < n_strips; s += G)
-      for (int q = tid; q < kStrip * 8; q += THREADS) {
-        const int t = q / kStrip, i = s * kStrip + q % kStrip;
-        if (i < r && c + t < r) gV[(int64_t)(c + t) * ldv + i] = i >= row0 + t ? s_u[(size_t)i * 8 + t] : 0.0f;
-      }
-    // ---- pass over the own strips ----
+    // R: rows row0 + a, columns c + t, t >= a
+    if (g == 0 && tid < 64) {
+      const int a = tid / 8, t = tid % 8;
+      if (t >= a && row0 + a < r) gB[(int64_t)(c + t) * (kBw + 1) + kBw + a - t] = sh.top[a][t];
+    }
     const bool first = c == 0;
-    const int first_strip = row0 / kStrip;
     const int s0 = first_strip + ((g - first_strip % G) % G + G) % G;      // first active strip of this CTA
-    const int parts = L.bd_parts;
-    const int per = ((m + parts - 1) / parts + 3) & ~3;                    // columns per task, a multiple of 4
+    const int n_own = s0 < n_strips ? (n_strips - 1 - s0) / G + 1 : 0;
+    // ---- pass over the own strips ----
+    const int per = ((m + PARTS - 1) / PARTS + 3) & ~3;      // columns per task, a multiple of 4
     for (int col0 = row0; col0 < r; col0 += cap) {
       const int col1 = min(r, col0 + cap);
       if (!first) {
-        __syncthreads();                                     // the block before has been used
+        if (col0 > row0) __syncthreads();                    // the block before has been used
         for (int q = tid; q < (col1 - col0) * 4; q += THREADS) {
           const int j = col0 + q / 4, h = q % 4;
           const float4* src = reinterpret_cast<const float4*>((h < 2 ? gU : gW) + (int64_t)j * 8) + (h & 1);
@@ -266,16 +327,15 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         }
       }
       __syncthreads();
-      // tasks (strip, part) of this block of columns, dealt to the warps; the strips of this CTA are s0, s0 + G, ...
-      const int n_own = s0 < n_strips ? (n_strips - 1 - s0) / G + 1 : 0;
-      for (int task = w; task < n_own * parts; task += kWarps) {
-        const int s = s0 + task / parts * G, part = task % parts;
-        const int jb = max(row0 + part * per, col0), je = min(min(row0 + (part + 1) * per, r), col1);
+      // tasks (strip, part), dealt to the warps
+      for (int task = w; task < n_own * PARTS; task += kWarps) {
+        const int s = s0 + task / PARTS * G, part = task % PARTS;
+        const int p_lo = row0 + part * per;
+        const int jb = max(p_lo, col0), je = min(min(p_lo + per, r), col1);
         const int i = s * kStrip + 2 * lane;
-        const bool in = i < r;
-        double* const dst = gPart + ((int64_t)part * n_strips * kStrip + (int64_t)s * kStrip + 2 * lane) * 8;
+        double* const dst = gPart + ((int64_t)part * n_strips * kStrip + i) * 8;
         if (jb >= je) {
-          if (row0 + part * per >= r && col0 == row0 && in) {      // an empty part
+          if (p_lo >= r && col0 == row0) {                   // an empty part
 #pragma unroll
             for (int t = 0; t < 16; t += 2) *reinterpret_cast<double2*>(dst + t) = make_double2(0.0, 0.0);
           }
@@ -285,18 +345,18 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         double p0[8], p1[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) { up0[t] = wp0[t] = up1[t] = wp1[t] = 0.0f; p0[t] = p1[t] = 0.0; }
-        if (in && !first) {
+        if (!first) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const float4 a = __ldcg(reinterpret_cast<const float4*>(gU + (int64_t)i * 8) + h), b = __ldcg(reinterpret_cast<const float4*>(gW + (int64_t)i * 8) + h);
             const float4 d = __ldcg(reinterpret_cast<const float4*>(gU + (int64_t)i * 8 + 8) + h), e = __ldcg(reinterpret_cast<const float4*>(gW + (int64_t)i * 8 + 8) + h);
-            up0[4 * h] = a.x; up0[4 * h + 1] = a.y; up0[4 * h + 2] = a.z; up0[4 * h + 3] = a.w;
-            wp0[4 * h] = b.x; wp0[4 * h + 1] = b.y; wp0[4 * h + 2] = b.z; wp0[4 * h + 3] = b.w;
-            up1[4 * h] = d.x; up1[4 * h + 1] = d.y; up1[4 * h + 2] = d.z; up1[4 * h + 3] = d.w;
-            wp1[4 * h] = e.x; wp1[4 * h + 1] = e.y; wp1[4 * h + 2] = e.z; wp1[4 * h + 3] = e.w;
+            up0[4 * h] = -a.x; up0[4 * h + 1] = -a.y; up0[4 * h + 2] = -a.z; up0[4 * h + 3] = -a.w;
+            wp0[4 * h] = -b.x; wp0[4 * h + 1] = -b.y; wp0[4 * h + 2] = -b.z; wp0[4 * h + 3] = -b.w;
+            up1[4 * h] = -d.x; up1[4 * h + 1] = -d.y; up1[4 * h + 2] = -d.z; up1[4 * h + 3] = -d.w;
+            wp1[4 * h] = -e.x; wp1[4 * h + 1] = -e.y; wp1[4 * h + 2] = -e.z; wp1[4 * h + 3] = -e.w;
           }
         }
-        if (jb > row0 + part * per && in) {                  // the part began in an earlier block of columns
+        if (jb > p_lo) {                                     // the part began in an earlier block of columns
 #pragma unroll
           for (int t = 0; t < 8; t += 2) {
             const double2 a = *reinterpret_cast<const double2*>(dst + t), b = *reinterpret_cast<const double2*>(dst + 8 + t);
@@ -309,99 +369,132 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         float* ap = A + (int64_t)jb * lda + i;
         const float4* ops = reinterpret_cast<const float4*>(s_ops) + (size_t)(jb - col0) * 4;
         const float4* un = reinterpret_cast<const float4*>(s_u) + (size_t)jb * 2;
-        constexpr int kU = 4;
-        float2 a[kU], an[kU];
-        auto fetch = [&](float2 (&buf)[kU], int j, const float* p) {
+        // one column: update, store, product
+        auto column = [&](float2 v, const float4* o, const float4* n, float* p) {
+          if (!first) {
+            const float4 cu0 = o[0], cu1 = o[1], cw0 = o[2], cw1 = o[3];
+            const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
+            const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
 #pragma unroll
-          for (int u = 0; u < kU; ++u) buf[u] = in && j + u < je ? *reinterpret_cast<const float2*>(p + (int64_t)u * lda) : make_float2(0.f, 0.f);
-        };
-        auto columns = [&](float2 (&buf)[kU], int j, float* p) {
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            if (j + u < je) {
-              float2 v = buf[u];
-              if (!first) {
-                const float4 cu0 = ops[4 * u], cu1 = ops[4 * u + 1], cw0 = ops[4 * u + 2], cw1 = ops[4 * u + 3];
-                const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
-                const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
-                float d0 = 0.0f, d1 = 0.0f;
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                  d0 = fmaf(up0[t], cw[t], d0); d1 = fmaf(up1[t], cw[t], d1);
-                  d0 = fmaf(wp0[t], cu[t], d0); d1 = fmaf(wp1[t], cu[t], d1);
-                }
-                v.x -= d0; v.y -= d1;
-                if (in) *reinterpret_cast<float2*>(p + (int64_t)u * lda) = v;
-              }
-              const float4 n0 = un[2 * u], n1 = un[2 * u + 1];
-              const float cn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-#pragma unroll
-              for (int t = 0; t < 8; ++t) { q0[t] = fmaf(v.x, cn[t], q0[t]); q1[t] = fmaf(v.y, cn[t], q1[t]); }
+            for (int t = 0; t < 8; ++t) {
+              v.x = fmaf(up0[t], cw[t], v.x); v.y = fmaf(up1[t], cw[t], v.y);
+              v.x = fmaf(wp0[t], cu[t], v.x); v.y = fmaf(wp1[t], cu[t], v.y);
             }
+            *reinterpret_cast<float2*>(p) = v;
           }
-        };
-        auto flush = [&]() {
+          const float4 n0 = n[0], n1 = n[1];
+          const float cn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
 #pragma unroll
-          for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; q0[t] = q1[t] = 0.0f; }
+          for (int t = 0; t < 8; ++t) { q0[t] = fmaf(v.x, cn[t], q0[t]); q1[t] = fmaf(v.y, cn[t], q1[t]); }
         };
-        fetch(a, jb, ap);
-        for (int j = jb, n = 0; j < je; j += 2 * kU, n += 2 * kU) {
-          fetch(an, j + kU, ap + (int64_t)kU * lda);
-          columns(a, j, ap);
-          ops += 4 * kU; un += 2 * kU; ap += (int64_t)kU * lda;
-          fetch(a, j + 2 * kU, ap + (int64_t)kU * lda);
-          columns(an, j + kU, ap);
-          ops += 4 * kU; un += 2 * kU; ap += (int64_t)kU * lda;
-          if ((n & 31) == 24) flush();
+        // groups of four columns, the next group's entries on their way; further ahead a prefetch asks the L2 for 16 columns
+        // at a time (two 128-byte lines each), so that a load waits for the L2 and not for DRAM
+        constexpr int kU = 4;
+        float2 a[kU];
+        const int whole = (je - jb) / kU;
+        const float* pre = A + (int64_t)(jb + lane / 2) * lda + s * kStrip + (lane & 1) * 32;
+        auto ask = [&](int j) { if (j + lane / 2 < je) asm volatile("prefetch.global.L2 [%0];" ::"l"(pre)); pre += (int64_t)16 * lda; };
+        ask(jb); ask(jb + 16);
+        if (whole > 0) {
+#pragma unroll
+          for (int u = 0; u < kU; ++u) a[u] = *reinterpret_cast<const float2*>(ap + (int64_t)u * lda);
         }
-        flush();
-        if (in) {
+        for (int q = 0; q < whole; ++q) {
+          float2 b[kU];
+          const float* nx = ap + (int64_t)kU * lda;
+          if (q + 1 < whole) {
 #pragma unroll
-          for (int t = 0; t < 8; t += 2) {
-            *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t], p0[t + 1]);
-            *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t], p1[t + 1]);
+            for (int u = 0; u < kU; ++u) b[u] = *reinterpret_cast<const float2*>(nx + (int64_t)u * lda);
           }
+          if ((q & 3) == 0) ask(jb + 4 * q + 32);
+#pragma unroll
+          for (int u = 0; u < kU; ++u) column(a[u], ops + 4 * u, un + 2 * u, ap + (int64_t)u * lda);
+          if ((q & 7) == 7) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; q0[t] = q1[t] = 0.0f; }
+          }
+#pragma unroll
+          for (int u = 0; u < kU; ++u) a[u] = b[u];
+          ops += 4 * kU; un += 2 * kU; ap += (int64_t)kU * lda;
+        }
+        for (int j = jb + whole * kU; j < je; ++j, ops += 4, un += 2, ap += lda) column(*reinterpret_cast<const float2*>(ap), ops, un, ap);
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) {
+          *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t] + (double)q0[t], p0[t + 1] + (double)q0[t + 1]);
+          *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t] + (double)q1[t], p1[t + 1] + (double)q1[t + 1]);
         }
       }
     }
     __syncthreads();
-    // ---- P = A U of the own rows (parts added in order), S = U^T P per strip ----
-    for (int s = s0; s < n_strips; s += G) {
-      double acc[8];
+    // ---- P = A U of the own rows (parts added in order), U^T P and U^T U; eight rows per warp at a time ----
+    {
+      long long acc[8];
 #pragma unroll
-      for (int a = 0; a < 8; ++a) acc[a] = 0.0;
-      for (int q = tid; q < kStrip * 8; q += THREADS) {      // lane: row q / 8, column q % 8
-        const int i = s * kStrip + q / 8;
-        double p = 0.0;
-        if (i < r && i >= row0) {
-          for (int part = 0; part < parts; ++part) p += gPart[((int64_t)part * n_strips * kStrip + i) * 8 + q % 8];
-          gP[(int64_t)i * 8 + q % 8] = p;
+      for (int a = 0; a < 8; ++a) acc[a] = 0;
+      for (int q = w; q < n_own * (kStrip / 8); q += kWarps) {
+        const int i0 = (s0 + q / (kStrip / 8) * G) * kStrip + q % (kStrip / 8) * 8;
 #pragma unroll
-          for (int a = 0; a < 8; ++a) acc[a] = fma((double)s_u[(size_t)i * 8 + a], p, acc[a]);
+        for (int h = 0; h < 2; ++h) {                        // lane: row i0 + 4 h + lane / 8, column lane % 8
+          const int i = i0 + 4 * h + lane / 8;
+          double pp[PARTS];
+#pragma unroll
+          for (int part = 0; part < PARTS; ++part) pp[part] = gPart[((int64_t)part * n_strips * kStrip + i) * 8 + lane % 8];
+          double p = 0.0;
+#pragma unroll
+          for (int part = 0; part < PARTS; ++part) p += pp[part];
+          gP[(int64_t)i * 8 + lane % 8] = p;
+          if (i >= row0 && i < r) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) acc[a] += __double2ll_rn((double)s_u[(size_t)i * 8 + a] * p * kFix);
+          }
         }
       }
 #pragma unroll
       for (int a = 0; a < 8; ++a) { acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 8); acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 16); }
-      double* const part_s = &sh.m[0][0];                    // [warp][64] does not fit: one value of a at a time
+      long long* const part_s = reinterpret_cast<long long*>(s_ops);       // [warp][64]: the operands have been used
+      if (lane < 8) {
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        if (lane < 8) part_s[w * 8 + lane] = acc[a];
-        __syncthreads();
-        if (tid < 8) {
-          double t = 0.0;
-          for (int ww = 0; ww < kWarps; ++ww) t += part_s[ww * 8 + tid];
-          gS[(int64_t)s * 64 + a * 8 + tid] = t;
-        }
-        __syncthreads();
+        for (int a = 0; a < 8; ++a) part_s[w * 64 + a * 8 + lane] = acc[a];
+      }
+      for (int q = w; q < 2 * n_own; q += kWarps) {          // half strips
+        const int half = 2 * (s0 + q / 2 * G) + (q & 1), i = half * 32 + lane;
+        const bool in = i >= row0 && i < r;
+        const float4* src = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : row0) * 8);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        band_gram32(in ? src[0] : zero, in ? src[1] : zero, gM + (int64_t)half * 36, lane);
+      }
+      __syncthreads();
+      if (tid < 64) {
+        long long t = 0;
+#pragma unroll
+        for (int ww = 0; ww < kWarps; ++ww) t += part_s[ww * 64 + tid];
+        gS[(int64_t)g * 64 + tid] = t;
       }
     }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
-    // ---- T^T S T; W of the next panel's pivot rows (every CTA) ----
-    if (tid < 64) {
-      double t = 0.0;
-      for (int s = first_strip; s < n_strips; ++s) t += __ldcg(gS + (int64_t)s * 64 + tid);
-      sh.S[tid / 8][tid % 8] = t;
+    // ---- T, T^T S T, W of the next panel's pivot rows (every CTA) ----
+    if (tid >= THREADS - 64) {
+      const int q = tid - (THREADS - 64);
+      long long t = 0;
+#pragma unroll 4
+      for (int s = 0; s < G; ++s) t += __ldcg(gS + (int64_t)s * 64 + q);
+      sh.S[q / 8][q % 8] = (double)t * (1.0 / kFix);
+    }
+    band_sum36<THREADS>(gM, 2 * first_strip, 2 * n_strips, sh.sum, sh.M);
+    __syncthreads();
+    if (w == 0) {
+      // T: tau_t in place t, -tau_t T[0:t, 0:t] M[0:t, t] above (lane: row)
+#pragma unroll 1
+      for (int t = 0; t < 8; ++t) {
+        const double* mt = sh.M + t * (t + 1) / 2;
+        const double tau = mt[t] > 0.5 ? 2.0 / mt[t] : 0.0;
+        double z0 = 0.0, z1 = 0.0;                           // (T is zero below its diagonal)
+#pragma unroll
+        for (int q = 0; q < 7; ++q) if (q < t && lane < 8) { if (q & 1) z1 = fma(sh.T[lane][q], mt[q], z1); else z0 = fma(sh.T[lane][q], mt[q], z0); }
+        if (lane < 8) sh.T[lane][t] = lane < t ? -tau * (z0 + z1) : lane == t ? tau : 0.0;
+        __syncwarp();
+      }
     }
     __syncthreads();
     if (tid < 64) {
@@ -412,57 +505,31 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       sh.Y[a][b] = t;
     }
     __syncthreads();
-    if (tid < 64) {
+    if (tid < 64) {                                          // X = -1/2 T^T S T
       const int a = tid / 8, b = tid % 8;
       double t = 0.0;
 #pragma unroll
       for (int q = 0; q < 8; ++q) t = fma(sh.T[q][a], sh.Y[q][b], t);
-      sh.X[a][b] = t;
+      sh.X[a][b] = -0.5 * t;
     }
     __syncthreads();
-    auto w_of = [&](const double* p, int i, int t) {         // W[i][t] = sum_s P[i][s] T[s][t] - 1/2 sum_s U[i][s] X[s][t]
-      double z = 0.0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) z = fma(p[q], sh.T[q][t], fma(-0.5 * (double)s_u[(size_t)i * 8 + q], sh.X[q][t], z));
-      return z;
-    };
     if (tid < 64) {
-      const int a = tid / 8, i = row0 + a;
-      double p[8];
+      const int a = tid / 8, t = tid % 8, i = row0 + a;
+      double z = 0.0;
+      if (i < r) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) p[q] = i < r ? __ldcg(gP + (int64_t)i * 8 + q) : 0.0;
-      sh.Wc[a][tid % 8] = i < r ? (float)w_of(p, i, tid % 8) : 0.0f;
+        for (int q = 0; q < 8; ++q) { z = fma(__ldcg(gP + (int64_t)i * 8 + q), sh.T[q][t], z); z = fma((double)s_u[(size_t)i * 8 + q], sh.X[q][t], z); }
+      }
+      sh.Wc[a][t] = (double)(float)z;
+      sh.Uc[a][t] = i < r ? (double)s_u[(size_t)i * 8 + t] : 0.0;
     }
     __syncthreads();
-    // ---- own rows: U, W out, entries of the next panel ----
-    for (int s = s0; s < n_strips; s += G)
-      for (int q = tid; q < kStrip * 8; q += THREADS) {      // entry (row, t): rows along the lanes for the panel's rows of A
-        const int i = s * kStrip + q % kStrip, t = q / kStrip;
-        if (i < row0 || i >= r) {
-          if (i < r) { gU[(int64_t)i * 8 + t] = 0.0f; gW[(int64_t)i * 8 + t] = 0.0f; }
-          continue;
-        }
-        double p[8];
-#pragma unroll
-        for (int h = 0; h < 8; ++h) p[h] = gP[(int64_t)i * 8 + h];
-        const float wi = (float)w_of(p, i, t);
-        gU[(int64_t)i * 8 + t] = s_u[(size_t)i * 8 + t];
-        gW[(int64_t)i * 8 + t] = wi;
-      }
-    __syncthreads();
-    for (int s = s0; s < n_strips; s += G)
+    // the reflectors' rows for the back-transformation (zero above row0 + t)
+    for (int s = g; s < n_strips; s += G)
       for (int q = tid; q < kStrip * 8; q += THREADS) {
-        const int i = s * kStrip + q % kStrip, t = q / kStrip;
-        if (i < row0 || i >= r || row0 + t >= r) continue;
-        double v = (double)__ldcg(A + (int64_t)(row0 + t) * lda + i);
-#pragma unroll
-        for (int h = 0; h < 8; ++h)
-          v -= fma((double)s_u[(size_t)i * 8 + h], (double)sh.Wc[t][h], (double)gW[(int64_t)i * 8 + h] * (double)s_u[(size_t)(row0 + t) * 8 + h]);
-        gX[(int64_t)t * lda + i] = (float)v;
+        const int t = q / kStrip, i = s * kStrip + q % kStrip;
+        if (i < r && c + t < r) gV[(int64_t)(c + t) * ldv + i] = i >= row0 + t ? s_u[(size_t)i * 8 + t] : 0.0f;
       }
-    arrivals += (uint32_t)G;
-    band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
-    if (sh.fail) break;
   }
 }
 
@@ -473,19 +540,32 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
 // columns R_{t-1} from the left (step 0: column j), the diagonal block R_t from both sides, rows R_{t+1} x columns R_t from
 // the right.  Step t of sweep j+1 needs step t+2 of sweep j, so sweep j runs step tick - 3 j: all active sweeps (one in 23
 // columns) advance together, separated by a barrier per tick, 3 r ticks in all.  No flags, no waits.
-// The band sits in shared memory as fp64, 15 sub-diagonals (eight and the fill) per column; sixteen lanes take a step (a lane
-// holds row l mod 8 and every other column of the blocks), so that a warp advances two sweeps.
-// Bound: the latency of a tick (two dependent reductions over eight lanes, two reciprocal square roots, an update), times
-// 3 r.  Short sides above 1024 are spread over a cluster, 1024 columns per CTA; only steps at the edge of a CTA's columns
-// touch the next CTA's memory, and the barrier per tick is the cluster's.
+// The band sits in shared memory as fp64, 15 sub-diagonals (eight and the fill) per column; sixteen lanes take a step, so that a
+// warp advances two sweeps.  Lane (k, h) holds column k, rows 4h .. 4h+3 of the left and of the diagonal block and row k,
+// columns 4h .. 4h+3 of the lower one: every product with the reflector is four multiply-adds and one exchange (only u^T D u
+// takes three more), and all addresses are one base plus offsets that never change.  What lies outside the matrix is stored
+// as zeros, lanes without a step work on a dummy block of zeros: no bounds tests.
+// Bound: instruction issue (a step is about 170 instructions, 23 warps) and, close behind, the latency of the step's chain.
+// Short sides above 1024 are spread over a cluster, 1024 columns per CTA.  A cluster barrier and the reads of a
+// neighbour's memory in every tick took 4.4 us per tick, three times the step itself; so a CTA also keeps copies of the
+// columns next to its own, works on them as well, and fetches them afresh every kChTicks ticks.  What it lacks spoils these
+// columns from their outer ends inwards: by eight columns a tick from above (a sweep moves down by a block), by fifteen from
+// below (a sweep that misses its predecessor's work spoils its own block, 15 columns further up), hence the widths.
 namespace {
-constexpr int kChThreads = 736;               // 46 half-warps: 1024 columns hold at most 45 active sweeps
 constexpr int kChCols = 1024;                 // columns per CTA
 constexpr int kChLd = 20;                     // doubles per column: 16 in use; 19 between neighbours of a row spreads the banks
+constexpr int kChTicks = 8;                   // ticks between two exchanges
+template <int C> struct ChForm {
+  static constexpr int kAbove = C > 1 ? 8 * kChTicks + 8 : 0, kBelow = C > 1 ? 15 * kChTicks + 16 : 16;
+  static constexpr int kLocal = kAbove + kChCols + kBelow;   // columns in shared memory, then 24 of zeros
+  static constexpr int kThreads = ((kLocal + 22) / 23 + 2) / 2 * 32;   // two half-warps per 46 columns
+  static constexpr size_t kSmem = (size_t)(kLocal + 24) * kChLd * sizeof(double);
+};
 }  // namespace
 
 template <int C>
-__global__ void __launch_bounds__(kChThreads, 1) sp_chase_kernel(const SpLayer* __restrict__ layers, const int* __restrict__ list) {
+__global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const SpLayer* __restrict__ layers, const int* __restrict__ list) {
+  constexpr int kAbove = ChForm<C>::kAbove, kLocal = ChForm<C>::kLocal, kThreads = ChForm<C>::kThreads;
   extern __shared__ __align__(16) double ch_smem[];
   const SpLayer& L = layers[list[blockIdx.x / C]];
   const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
@@ -494,98 +574,94 @@ __global__ void __launch_bounds__(kChThreads, 1) sp_chase_kernel(const SpLayer* 
   const double* const gB = L.bd_band;
   float* const gV2 = L.bd_V2;
   const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that gV2 has room for
-  const int col0 = rank * kChCols;
-  double* peer[2] = {ch_smem, ch_smem};                      // this CTA's columns, the next one's
+  const int col0 = rank * kChCols, lo = col0 - kAbove;       // first own column, first column in shared memory
+  const double *above = ch_smem, *below = ch_smem;           // the neighbours' shared memory
   if (C > 1) {
     cg::cluster_group cluster = cg::this_cluster();
-    peer[1] = cluster.map_shared_rank(ch_smem, min(rank + 1, C - 1));
+    above = cluster.map_shared_rank(ch_smem, max(rank - 1, 0));
+    below = cluster.map_shared_rank(ch_smem, min(rank + 1, C - 1));
   }
-  for (int q = tid; q < kChCols * 16; q += kChThreads) {
-    const int j = col0 + q / 16, d = q % 16;
-    ch_smem[(q / 16) * kChLd + d] = j < r && d <= kBw && j + d < r ? gB[(int64_t)j * (kBw + 1) + d] : 0.0;
+  for (int q = tid; q < (kLocal + 24) * kChLd; q += kThreads) {
+    const int j = lo + q / kChLd, d = q % kChLd;
+    ch_smem[q] = q / kChLd < kLocal && j >= 0 && j < r && d <= kBw && j + d < r ? gB[(int64_t)j * (kBw + 1) + d] : 0.0;
   }
-  auto sync = [&]() { if (C > 1) cg::this_cluster().sync(); else __syncthreads(); };
-  sync();
-  // entry (i, j), i >= j, of this CTA's or the next one's columns (zero where it is outside the matrix or the stored diagonals)
-  auto at = [&](int i, int j) -> double* {
-    const int jl = j - col0;
-    double* const base = C > 1 && jl >= kChCols ? peer[1] + (size_t)(jl - kChCols) * kChLd : ch_smem + (size_t)jl * kChLd;
-    return base + (i - j);
-  };
-  const int half = tid / 16, hl = tid % 16, row = hl & 7, par = hl >> 3;   // a lane's columns of a block: par, par + 2, par + 4, par + 6
+  if (C > 1) cg::this_cluster().sync(); else __syncthreads();
+  const int half = tid / 16, k = tid & 7, h = (tid >> 3) & 1, base_lane = lane & 16;
+  // offsets of this lane's entries: left block from (first column, first row), diagonal and lower block from (start, start)
+  int od[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { const int e = 4 * h + q; od[q] = e >= k ? 19 * k + e : 19 * e + k; }
+  const int ob = 19 * k + 4 * h, on = 19 * 4 * h + 8 + k;
   const int ticks = 3 * (r - 3) + 1;                         // (no sweep for r < 3)
   for (int tick = 0; tick < ticks; ++tick) {
-    // sweep j's step t = tick - 3 j starts at row j + 1 + 8 t = 8 tick + 1 - 23 j; this CTA takes the steps whose first column
-    // is one of its own
-    const int top = 8 * tick + 1;
-    const int hi = col0 + kChCols - 1;                       // last column of this CTA
-    const int j_lo = top - kBw > hi ? (top - kBw - hi + 22) / 23 : 0;
-    const int j = j_lo + half;
+    if (C > 1 && tick % kChTicks == 0 && tick > 0) {
+      cg::cluster_group cluster = cg::this_cluster();
+      cluster.sync();                                        // every CTA's own columns are up to date
+      if (rank > 0)
+        for (int q = tid; q < kAbove * 16; q += kThreads) ch_smem[(q / 16) * kChLd + q % 16] = above[(kChCols + q / 16) * kChLd + q % 16];
+      if (rank < C - 1)
+        for (int q = tid; q < (kLocal - kAbove - kChCols) * 16; q += kThreads)
+          ch_smem[(kAbove + kChCols + q / 16) * kChLd + q % 16] = below[(kAbove + q / 16) * kChLd + q % 16];
+      cluster.sync();                                        // copies taken before anybody goes on
+    }
+    // sweep j's step t = tick - 3 j starts at row j + 1 + 8 t = 8 tick + 1 - 23 j
+    const int top = 8 * tick + 1, last = lo + kLocal - kBw;  // last start whose columns are all here
+    const int j = (top > last ? (top - last + 22) / 23 : 0) + half;
     const int start = top - 23 * j, t = tick - 3 * j;
     const int prev = t > 0 ? start - kBw : j;                // first column of the block to the left
-    const bool active = j <= r - 3 && t >= 0 && prev >= col0 && prev <= hi && start <= r - 2;
+    const bool active = j <= r - 3 && t >= 0 && prev >= lo && start <= r - 2;
     if (__any_sync(0xffffffffu, active)) {
-      const int i = start + row;                             // this lane's row in R_t; in R_{t+1}: i + 8
-      const bool in = active && i < r, in2 = active && i + kBw < r;
+      double* const pd = ch_smem + (active ? start - lo : kLocal + 8) * kChLd;
+      // step 0 has a left block of one column; its other lanes take the zeros
+      double* const pb = active && (t > 0 || k == 0) ? ch_smem + (prev - lo) * kChLd + (start - prev) + ob : ch_smem + kLocal * kChLd + 8 + ob;
       double bl[4], dd[4], bn[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int cq = par + 2 * q;
-        bl[q] = in && (t > 0 || cq == 0) ? *at(i, prev + cq) : 0.0;
-        const int jc = start + cq;
-        dd[q] = in && jc < r ? (i >= jc ? *at(i, jc) : *at(jc, i)) : 0.0;
-        bn[q] = in2 && jc < r ? *at(i + kBw, jc) : 0.0;
-      }
-      // reflector of the first column of the left block (lanes par == 0, q == 0)
-      const double xr = __shfl_sync(0xffffffffu, bl[0], (lane & 16) | row);
-      double nx2 = xr * xr;
+      for (int q = 0; q < 4; ++q) { bl[q] = pb[q]; dd[q] = pd[od[q]]; bn[q] = pd[on + 19 * q]; }
+      // reflector of the left block's first column (lanes k == 0)
+      double u[4];
 #pragma unroll
-      for (int o = 1; o < 8; o <<= 1) nx2 += __shfl_xor_sync(0xffffffffu, nx2, o);
-      const double x0 = __shfl_sync(0xffffffffu, xr, lane & 16);
+      for (int q = 0; q < 4; ++q) u[q] = __shfl_sync(0xffffffffu, bl[q], lane & 24);
+      double nx2 = fma(u[0], u[0], u[1] * u[1]) + fma(u[2], u[2], u[3] * u[3]);
+      const double x0 = __shfl_sync(0xffffffffu, u[0], base_lane);
+      nx2 += __shfl_xor_sync(0xffffffffu, nx2, 8);
       double alpha = 0.0, us = 0.0;
       if (nx2 > 1.0e-290) {
         const double nx = nx2 * rsqrt(nx2);
         alpha = -copysign(nx, x0);
         us = rsqrt(2.0 * fma(fabs(x0), nx, nx2));            // 1 / ||v||
       }
-      const double u = (row == 0 ? xr - alpha : xr) * us;    // unit vector; 0 for a zero column (H = I)
-      double uc[4];
+      if (h == 0) u[0] -= alpha;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) uc[q] = __shfl_sync(0xffffffffu, u, (lane & 16) | (par + 2 * q));
-      // y = D u and p = Bn u (rows), z = u^T Bl (columns)
-      double y = 0.0, p = 0.0, z[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { y = fma(dd[q], uc[q], y); p = fma(bn[q], uc[q], p); z[q] = u * bl[q]; }
+      for (int q = 0; q < 4; ++q) u[q] *= us;                // entries 4h .. 4h+3 of the unit vector; 0 for a zero column (H = I)
+      const double mine = (k & 2) ? ((k & 1) ? u[3] : u[2]) : ((k & 1) ? u[1] : u[0]), theirs = __shfl_xor_sync(0xffffffffu, mine, 8);
+      const double uk = (k >> 2) == h ? mine : theirs;       // entry k
+      double z = fma(u[0], bl[0], u[1] * bl[1]) + fma(u[2], bl[2], u[3] * bl[3]);     // u^T Bl, column k
+      double y = fma(u[0], dd[0], u[1] * dd[1]) + fma(u[2], dd[2], u[3] * dd[3]);     // D u, entry k
+      double p = fma(u[0], bn[0], u[1] * bn[1]) + fma(u[2], bn[2], u[3] * bn[3]);     // Bn u, row k
+      z += __shfl_xor_sync(0xffffffffu, z, 8);
       y += __shfl_xor_sync(0xffffffffu, y, 8);
       p += __shfl_xor_sync(0xffffffffu, p, 8);
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) z[q] += __shfl_xor_sync(0xffffffffu, z[q], o);
-      }
-      double s = u * y;
+      double s = uk * y;
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const double wr = 2.0 * fma(-s, u, y);                 // D - u w^T - w u^T, w = 2 (y - s u)
-      double wc[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) wc[q] = __shfl_sync(0xffffffffu, wr, (lane & 16) | (par + 2 * q));
+      const double wk = 2.0 * fma(-s, uk, y);                // D - u w^T - w u^T, w = 2 (y - s u)
+      z *= -2.0; p *= -2.0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int cq = par + 2 * q, jc = start + cq;
-        if (in && (t > 0 || cq == 0)) *at(i, prev + cq) = cq == 0 ? (row == 0 ? alpha : 0.0) : fma(-2.0 * u, z[q], bl[q]);
-        if (in && jc <= i) *at(i, jc) = fma(-u, wc[q], fma(-wr, uc[q], dd[q]));
-        if (in2 && jc < r) *at(i + kBw, jc) = fma(-2.0 * p, uc[q], bn[q]);
+        const double we = __shfl_sync(0xffffffffu, wk, base_lane + 4 * h + q);
+        pb[q] = k == 0 ? (h == 0 && q == 0 ? alpha : 0.0) : fma(u[q], z, bl[q]);
+        if (4 * h + q >= k) pd[od[q]] = fma(-u[q], wk, fma(-we, uk, dd[q]));
+        pd[on + 19 * q] = fma(p, u[q], bn[q]);
       }
-      if (active && par == 0) gV2[((int64_t)j * ns + t) * kBw + row] = (float)u;
+      if (active && h == 0 && prev >= col0 && prev < col0 + kChCols) gV2[((int64_t)j * ns + t) * kBw + k] = (float)uk;
     }
-    sync();
+    __syncthreads();
   }
-  for (int q = tid; q < kChCols; q += kChThreads) {
+  for (int q = tid; q < kChCols; q += kThreads) {
     const int j = col0 + q;
-    if (j < r) { L.td_d[j] = ch_smem[(size_t)q * kChLd]; L.td_e[j] = j + 1 < r ? ch_smem[(size_t)q * kChLd + 1] : 0.0; }
+    if (j < r) { L.td_d[j] = ch_smem[(size_t)(kAbove + q) * kChLd]; L.td_e[j] = j + 1 < r ? ch_smem[(size_t)(kAbove + q) * kChLd + 1] : 0.0; }
   }
-  if (C > 1) cg::this_cluster().sync();                      // nobody leaves while a neighbour may still reach into its memory
+  if (C > 1) cg::this_cluster().sync();                      // nobody leaves while a neighbour may still read its memory
 }
 
 // ---- host side ----------------------------------------------------------------------------------------------------------------
@@ -595,31 +671,30 @@ int band_sms() {
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms;
 }
-// the instances of the band kernel, by the largest short side of the batch
-struct BandForm { int max_r, threads, per_sm, cap; const void* fn; };
+// The instances of the band kernel.  Many layers up to 1024 rows: two small CTAs per SM (96 KB: U of the panel, all columns' U
+// and W of the panel before).  Few layers, or larger ones: one CTA of sixteen warps per SM, a strip each, its columns split
+// over the warps; the operands of 1024 columns at a time.
+struct BandForm { int max_r, threads, per_sm, cap, parts; const void* fn; };
 const BandForm kBandForms[] = {
-    // two CTAs per SM hold U of the panel (32 B per row) and all columns' U and W of the panel before (64 B) twice over
-    {1024, 256, 2, 1024, (const void*)sp_band_kernel<256, 4, double, 2>},
-    {2048, 512, 1, 1024, (const void*)sp_band_kernel<512, 4, double, 1>},
-    {4096, 512, 1, 1024, (const void*)sp_band_kernel<512, 8, float, 1>},
+    {1024, 256, 2, 1024, 4, (const void*)sp_band_kernel<256, 2, 4>},
+    {4096, 512, 1, 1024, 16, (const void*)sp_band_kernel<512, 1, 16>},
 };
-const BandForm& band_form(int r_max) { for (const BandForm& f : kBandForms) if (r_max <= f.max_r) return f; return kBandForms[2]; }
 size_t band_smem(const BandForm& f, int r_max) { return ((size_t)r_max * 8 + (size_t)std::min(f.cap, r_max) * 16) * sizeof(float); }
-size_t chase_smem() { return (size_t)kChCols * kChLd * sizeof(double); }
 template <int C> int chase_configure() {
-  if (cudaFuncSetAttribute(sp_chase_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chase_smem()) != cudaSuccess) return 1;
+  if (cudaFuncSetAttribute(sp_chase_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ChForm<C>::kSmem) != cudaSuccess) return 1;
   return 0;
 }
 }  // namespace
 
 int sp_band_max_r() { return 4096; }
 int sp_band_strips(int r) { return (r + kStrip - 1) / kStrip; }
-// tasks that a strip's columns are split into: enough for the warps of a CTA that has few strips
-int sp_band_parts(int r) { return r <= 1024 ? 4 : 16; }
 int sp_band_steps(int r) { return (r + kBw - 1) / kBw; }
-// CTAs that one launch can hold together, for a batch of layers of at most r_max rows (0: not available)
-int sp_band_capacity(int r_max) {
-  const BandForm& f = band_form(r_max);
+// which instance a batch takes whose layers have `strips` strips in all and at most r_max rows
+int sp_band_form(int r_max, int64_t strips) { return r_max <= kBandForms[0].max_r && strips > band_sms() ? 0 : 1; }
+int sp_band_parts(int form) { return kBandForms[form].parts; }
+// CTAs that one launch can hold together (0: not available)
+int sp_band_capacity(int form, int r_max) {
+  const BandForm& f = kBandForms[form];
   int per = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f.fn, f.threads, band_smem(f, r_max)) != cudaSuccess) { cudaGetLastError(); return 0; }
   return band_sms() * std::min(per, f.per_sm);
@@ -636,8 +711,8 @@ int sp_configure_band() {
   return bad;
 }
 
-int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int r_max, uint32_t* d_timeout, cudaStream_t st) {
-  const BandForm& f = band_form(r_max);
+int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int form, int r_max, uint32_t* d_timeout, cudaStream_t st) {
+  const BandForm& f = kBandForms[form];
   int cap = std::min(f.cap, r_max);
   void* args[] = {&d_layers, &d_ctas, &cap, &d_timeout};
   return (int)cudaLaunchCooperativeKernel(f.fn, dim3((unsigned)n_ctas), dim3(f.threads), args, band_smem(f, r_max), st);
@@ -646,7 +721,7 @@ int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas
 namespace {
 template <int C> int chase_launch(const SpLayer* d_layers, const int* d_list, int n, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n * C); cfg.blockDim = dim3(kChThreads); cfg.dynamicSmemBytes = chase_smem(); cfg.stream = st;
+  cfg.gridDim = dim3(n * C); cfg.blockDim = dim3(ChForm<C>::kThreads); cfg.dynamicSmemBytes = ChForm<C>::kSmem; cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;

@@ -107,9 +107,10 @@ struct SpLayer {
   uint32_t* vec_ticket;        // CTAs of the vector kernel that finished this layer; zeroed per call
   // tridiagonal route for short sides above 512 (tri = 2): dense -> band -> tridiagonal
   float* bd_U; float* bd_W;    // [rows padded to strips][8] panel vectors of the panel before
-  float* bd_X;                 // [8][lda] entries of the next panel
-  double* bd_part; int bd_parts; // [parts][rows padded to strips][8] partial products, tasks per strip
-  double* bd_P; double* bd_S;  // [rows padded to strips][8] product A U; [strips][64] U^T A U per strip
+  float* bd_X;                 // [rows padded to strips][8] entries of the next panel
+  double* bd_part;             // [parts][rows padded to strips][8] partial products
+  double* bd_P; long long* bd_S; // [rows padded to strips][8] product A U; [CTAs][64] U^T A U, fixed point
+  double* bd_G; double* bd_M;  // [half strips][36] dots of the next panel's columns, of U's
   double* bd_band;             // [r][9] the band, by column
   float* bd_V2;                // [r][steps][8] reflectors of the chase: sweep, step
   uint32_t* bd_bar;            // arrivals at the layer's barriers; zeroed per call
@@ -160,11 +161,12 @@ void launch_sp_eigvec(const SpLayer* d_layers, int n_layers, int rp_max, cudaStr
 // tridiagonal route for short sides above 512 (atomo_band.cu, vectors in atomo_tridiag_big.cu)
 int sp_band_max_r();
 int sp_band_strips(int r);
-int sp_band_parts(int r);
 int sp_band_steps(int r);
-int sp_band_capacity(int r_max);                                  // co-resident CTAs of the band reduction (0: not available)
+int sp_band_form(int r_max, int64_t strips);                      // instance of the band kernel for a batch
+int sp_band_parts(int form);                                      // tasks that a strip's columns are split into
+int sp_band_capacity(int form, int r_max);                        // co-resident CTAs of the band reduction (0: not available)
 int sp_configure_band();                                          // 0 if available
-int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int r_max, uint32_t* d_timeout, cudaStream_t st);  // cudaError_t
+int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int form, int r_max, uint32_t* d_timeout, cudaStream_t st);  // cudaError_t
 int sp_chase_ctas(int r);                                         // CTAs per layer of the chase
 int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st);   // cudaError_t
 int sp_eigvec_big_slots();                                        // warps per layer of the vector kernel (work vectors)
