@@ -860,10 +860,11 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       ++n_eig_launch;
     }
     for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one cluster size are neighbours)
-      const int c = sp_chase_ctas(L[big_layers[i]].r);
+      const int n_big = (int)big_layers.size(), rm = L[big_layers[i]].r, c = sp_chase_ctas(rm, n_big);
+      auto same = [&](int l) { return sp_chase_ctas(L[l].r, n_big) == c && (L[l].r > 1024) == (rm > 1024); };
       n = 1;
-      while (i + n < big_layers.size() && sp_chase_ctas(L[big_layers[i + n]].r) == c) ++n;
-      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
+      while (i + n < big_layers.size() && same(big_layers[i + n])) ++n;
+      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, rm, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(bulge chase)");
       ++n_eig_launch;
     }

@@ -78,9 +78,8 @@ __device__ __forceinline__ double band_scatter8(const double (&v)[8], int lane) 
   c += __shfl_xor_sync(0xffffffffu, c, 1);
   return c;
 }
-// the 36 dots of the columns of a 32 x 8 block, one row (a, b) per lane, to dst (lower triangle by rows).  (Out of line: what runs
-// once per panel has to stay small.  A panel is a walk through the whole kernel, and straight-line code that no longer fits
-// the instruction cache costs its misses every time: the 8 x 8 factorisation unrolled took 52 k cycles, rolled up 7 k.)
+// the 36 dots of the columns of a 32 x 8 block, one row (a, b) per lane, to dst (lower triangle by rows).  (Out of line, as the
+// 8 x 8 factorisation below: a panel is a walk through the whole kernel, and what runs once per panel should stay small.)
 __device__ __noinline__ void band_gram32(const float4 a, const float4 b, double* __restrict__ dst, int lane) {
   const double d[8] = {(double)a.x, (double)a.y, (double)a.z, (double)a.w, (double)b.x, (double)b.y, (double)b.z, (double)b.w};
   double acc[40];
@@ -143,7 +142,6 @@ __device__ __forceinline__ void band_sum36(const double* __restrict__ src, int f
 // column l = lane % 8, rows lane / 8 and lane / 8 + 4.  Leaves R in sh.top, the unit reflectors' entries in the first eight rows
 // in sh.vtop (zero above the diagonal) and K, scaled likewise.
 __device__ __noinline__ void band_small_qr(BandShared& sh, const int n_ref, const int lane) {
-  // The warp has to be whole here: left divided by an earlier branch it takes 52 k cycles instead of 6 k
   __syncwarp();
   const int l = lane & 7, i0 = lane >> 3;
   double top[2], g[2], k[2];
@@ -541,31 +539,32 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
 // the right.  Step t of sweep j+1 needs step t+2 of sweep j, so sweep j runs step tick - 3 j: all active sweeps (one in 23
 // columns) advance together, separated by a barrier per tick, 3 r ticks in all.  No flags, no waits.
 // The band sits in shared memory as fp64, 15 sub-diagonals (eight and the fill) per column; sixteen lanes take a step, so that a
-// warp advances two sweeps.  Lane (k, h) holds column k, rows 4h .. 4h+3 of the left and of the diagonal block and row k,
-// columns 4h .. 4h+3 of the lower one: every product with the reflector is four multiply-adds and one exchange (only u^T D u
+// warp advances two sweeps.  Lane (k, h) holds column k, rows h, h+2, h+4, h+6 of the left and of the diagonal block and row k,
+// those columns of the lower one: every product with the reflector is four multiply-adds and one exchange (only u^T D u
 // takes three more), and all addresses are one base plus offsets that never change.  What lies outside the matrix is stored
 // as zeros, lanes without a step work on a dummy block of zeros: no bounds tests.
-// Bound: instruction issue (a step is about 170 instructions, 23 warps) and, close behind, the latency of the step's chain.
-// Short sides above 1024 are spread over a cluster, 1024 columns per CTA.  A cluster barrier and the reads of a
+// Bound: shared memory where a CTA has 1024 columns (23 warps), else the latency of the step's chain.
+// (The shared-memory pipe, which the exchanges use too, takes about 110 cycles per warp and tick: 24 loads and stores of
+// eight bytes, 36 shuffles.)  Larger short sides, and batches that leave SMs idle, are spread over a cluster, down to 256
+// columns per CTA.  A cluster barrier and the reads of a
 // neighbour's memory in every tick took 4.4 us per tick, three times the step itself; so a CTA also keeps copies of the
 // columns next to its own, works on them as well, and fetches them afresh every kChTicks ticks.  What it lacks spoils these
 // columns from their outer ends inwards: by eight columns a tick from above (a sweep moves down by a block), by fifteen from
 // below (a sweep that misses its predecessor's work spoils its own block, 15 columns further up), hence the widths.
 namespace {
-constexpr int kChCols = 1024;                 // columns per CTA
-constexpr int kChLd = 20;                     // doubles per column: 16 in use; 19 between neighbours of a row spreads the banks
+constexpr int kChLd = 19;                     // doubles per column, 16 in use: a half-warp's loads of a left block meet 16 different banks
 constexpr int kChTicks = 8;                   // ticks between two exchanges
-template <int C> struct ChForm {
+template <int C, int COLS> struct ChForm {     // CTAs per layer, columns per CTA
   static constexpr int kAbove = C > 1 ? 8 * kChTicks + 8 : 0, kBelow = C > 1 ? 15 * kChTicks + 16 : 16;
-  static constexpr int kLocal = kAbove + kChCols + kBelow;   // columns in shared memory, then 24 of zeros
+  static constexpr int kLocal = kAbove + COLS + kBelow;   // columns in shared memory, then 24 of zeros
   static constexpr int kThreads = ((kLocal + 22) / 23 + 2) / 2 * 32;   // two half-warps per 46 columns
   static constexpr size_t kSmem = (size_t)(kLocal + 24) * kChLd * sizeof(double);
 };
 }  // namespace
 
-template <int C>
-__global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const SpLayer* __restrict__ layers, const int* __restrict__ list) {
-  constexpr int kAbove = ChForm<C>::kAbove, kLocal = ChForm<C>::kLocal, kThreads = ChForm<C>::kThreads;
+template <int C, int COLS>
+__global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(const SpLayer* __restrict__ layers, const int* __restrict__ list) {
+  constexpr int kAbove = ChForm<C, COLS>::kAbove, kLocal = ChForm<C, COLS>::kLocal, kThreads = ChForm<C, COLS>::kThreads;
   extern __shared__ __align__(16) double ch_smem[];
   const SpLayer& L = layers[list[blockIdx.x / C]];
   const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
@@ -574,7 +573,7 @@ __global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const 
   const double* const gB = L.bd_band;
   float* const gV2 = L.bd_V2;
   const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that gV2 has room for
-  const int col0 = rank * kChCols, lo = col0 - kAbove;       // first own column, first column in shared memory
+  const int col0 = rank * COLS, lo = col0 - kAbove;       // first own column, first column in shared memory
   const double *above = ch_smem, *below = ch_smem;           // the neighbours' shared memory
   if (C > 1) {
     cg::cluster_group cluster = cg::this_cluster();
@@ -590,18 +589,18 @@ __global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const 
   // offsets of this lane's entries: left block from (first column, first row), diagonal and lower block from (start, start)
   int od[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) { const int e = 4 * h + q; od[q] = e >= k ? 19 * k + e : 19 * e + k; }
-  const int ob = 19 * k + 4 * h, on = 19 * 4 * h + 8 + k;
+  for (int q = 0; q < 4; ++q) { const int e = 2 * q + h; od[q] = e >= k ? (kChLd - 1) * k + e : (kChLd - 1) * e + k; }
+  const int ob = (kChLd - 1) * k + h, on = (kChLd - 1) * h + 8 + k;
   const int ticks = 3 * (r - 3) + 1;                         // (no sweep for r < 3)
   for (int tick = 0; tick < ticks; ++tick) {
     if (C > 1 && tick % kChTicks == 0 && tick > 0) {
       cg::cluster_group cluster = cg::this_cluster();
       cluster.sync();                                        // every CTA's own columns are up to date
       if (rank > 0)
-        for (int q = tid; q < kAbove * 16; q += kThreads) ch_smem[(q / 16) * kChLd + q % 16] = above[(kChCols + q / 16) * kChLd + q % 16];
+        for (int q = tid; q < kAbove * 16; q += kThreads) ch_smem[(q / 16) * kChLd + q % 16] = above[(COLS + q / 16) * kChLd + q % 16];
       if (rank < C - 1)
-        for (int q = tid; q < (kLocal - kAbove - kChCols) * 16; q += kThreads)
-          ch_smem[(kAbove + kChCols + q / 16) * kChLd + q % 16] = below[(kAbove + q / 16) * kChLd + q % 16];
+        for (int q = tid; q < (kLocal - kAbove - COLS) * 16; q += kThreads)
+          ch_smem[(kAbove + COLS + q / 16) * kChLd + q % 16] = below[(kAbove + q / 16) * kChLd + q % 16];
       cluster.sync();                                        // copies taken before anybody goes on
     }
     // sweep j's step t = tick - 3 j starts at row j + 1 + 8 t = 8 tick + 1 - 23 j
@@ -616,7 +615,7 @@ __global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const 
       double* const pb = active && (t > 0 || k == 0) ? ch_smem + (prev - lo) * kChLd + (start - prev) + ob : ch_smem + kLocal * kChLd + 8 + ob;
       double bl[4], dd[4], bn[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { bl[q] = pb[q]; dd[q] = pd[od[q]]; bn[q] = pd[on + 19 * q]; }
+      for (int q = 0; q < 4; ++q) { bl[q] = pb[2 * q]; dd[q] = pd[od[q]]; bn[q] = pd[on + 2 * (kChLd - 1) * q]; }
       // reflector of the left block's first column (lanes k == 0)
       double u[4];
 #pragma unroll
@@ -632,9 +631,9 @@ __global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const 
       }
       if (h == 0) u[0] -= alpha;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) u[q] *= us;                // entries 4h .. 4h+3 of the unit vector; 0 for a zero column (H = I)
-      const double mine = (k & 2) ? ((k & 1) ? u[3] : u[2]) : ((k & 1) ? u[1] : u[0]), theirs = __shfl_xor_sync(0xffffffffu, mine, 8);
-      const double uk = (k >> 2) == h ? mine : theirs;       // entry k
+      for (int q = 0; q < 4; ++q) u[q] *= us;                // entries h, h+2, h+4, h+6 of the unit vector; 0 for a zero column (H = I)
+      const double mine = (k & 4) ? ((k & 2) ? u[3] : u[2]) : ((k & 2) ? u[1] : u[0]), theirs = __shfl_xor_sync(0xffffffffu, mine, 8);
+      const double uk = (k & 1) == h ? mine : theirs;       // entry k
       double z = fma(u[0], bl[0], u[1] * bl[1]) + fma(u[2], bl[2], u[3] * bl[3]);     // u^T Bl, column k
       double y = fma(u[0], dd[0], u[1] * dd[1]) + fma(u[2], dd[2], u[3] * dd[3]);     // D u, entry k
       double p = fma(u[0], bn[0], u[1] * bn[1]) + fma(u[2], bn[2], u[3] * bn[3]);     // Bn u, row k
@@ -648,16 +647,16 @@ __global__ void __launch_bounds__(ChForm<C>::kThreads, 1) sp_chase_kernel(const 
       z *= -2.0; p *= -2.0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const double we = __shfl_sync(0xffffffffu, wk, base_lane + 4 * h + q);
-        pb[q] = k == 0 ? (h == 0 && q == 0 ? alpha : 0.0) : fma(u[q], z, bl[q]);
-        if (4 * h + q >= k) pd[od[q]] = fma(-u[q], wk, fma(-we, uk, dd[q]));
-        pd[on + 19 * q] = fma(p, u[q], bn[q]);
+        const double we = __shfl_sync(0xffffffffu, wk, base_lane + 2 * q + h);
+        pb[2 * q] = k == 0 ? (h == 0 && q == 0 ? alpha : 0.0) : fma(u[q], z, bl[q]);
+        if (2 * q + h >= k) pd[od[q]] = fma(-u[q], wk, fma(-we, uk, dd[q]));
+        pd[on + 2 * (kChLd - 1) * q] = fma(p, u[q], bn[q]);
       }
-      if (active && h == 0 && prev >= col0 && prev < col0 + kChCols) gV2[((int64_t)j * ns + t) * kBw + k] = (float)uk;
+      if (active && h == 0 && prev >= col0 && prev < col0 + COLS) gV2[((int64_t)j * ns + t) * kBw + k] = (float)uk;
     }
     __syncthreads();
   }
-  for (int q = tid; q < kChCols; q += kThreads) {
+  for (int q = tid; q < COLS; q += kThreads) {
     const int j = col0 + q;
     if (j < r) { L.td_d[j] = ch_smem[(size_t)(kAbove + q) * kChLd]; L.td_e[j] = j + 1 < r ? ch_smem[(size_t)(kAbove + q) * kChLd + 1] : 0.0; }
   }
@@ -680,8 +679,10 @@ const BandForm kBandForms[] = {
     {4096, 512, 1, 1024, 16, (const void*)sp_band_kernel<512, 1, 16>},
 };
 size_t band_smem(const BandForm& f, int r_max) { return ((size_t)r_max * 8 + (size_t)std::min(f.cap, r_max) * 16) * sizeof(float); }
-template <int C> int chase_configure() {
-  if (cudaFuncSetAttribute(sp_chase_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ChForm<C>::kSmem) != cudaSuccess) return 1;
+template <int C, int COLS> int chase_configure() {
+  auto* fn = sp_chase_kernel<C, COLS>;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ChForm<C, COLS>::kSmem) != cudaSuccess) return 1;
+  if (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 1;
   return 0;
 }
 }  // namespace
@@ -706,7 +707,8 @@ int sp_configure_band() {
     bad |= cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)band_smem(f, f.max_r)) != cudaSuccess;
     bad |= cudaFuncSetAttribute(f.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess;
   }
-  bad |= chase_configure<1>() | chase_configure<2>() | chase_configure<4>();
+  bad |= chase_configure<1, 1024>() | chase_configure<2, 1024>() | chase_configure<4, 1024>() | chase_configure<4, 256>() |
+         chase_configure<8, 256>() | chase_configure<16, 256>();
   if (bad) cudaGetLastError();
   return bad;
 }
@@ -719,24 +721,31 @@ int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas
 }
 
 namespace {
-template <int C> int chase_launch(const SpLayer* d_layers, const int* d_list, int n, cudaStream_t st) {
+template <int C, int COLS> int chase_launch(const SpLayer* d_layers, const int* d_list, int n, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n * C); cfg.blockDim = dim3(ChForm<C>::kThreads); cfg.dynamicSmemBytes = ChForm<C>::kSmem; cfg.stream = st;
+  cfg.gridDim = dim3(n * C); cfg.blockDim = dim3(ChForm<C, COLS>::kThreads); cfg.dynamicSmemBytes = ChForm<C, COLS>::kSmem; cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = C > 1 ? 1 : 0;
-  return (int)cudaLaunchKernelEx(&cfg, sp_chase_kernel<C>, d_layers, d_list);
+  return (int)cudaLaunchKernelEx(&cfg, sp_chase_kernel<C, COLS>, d_layers, d_list);
 }
 }  // namespace
-int sp_chase_ctas(int r) { return r <= kChCols ? 1 : r <= 2 * kChCols ? 2 : 4; }
-// d_list: n layers that take `ctas` CTAs each
-int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st) {
+// CTAs per layer of the chase for a layer of r rows in a batch of n large layers: 256 columns each (half the time of 1024
+// columns per CTA) while the batch's clusters fit the GPU side by side, else as few as hold the layer
+int sp_chase_ctas(int r, int n) {
+  const int few = r <= 1024 ? 1 : r <= 2048 ? 2 : 4, many = 4 * few;
+  return n * many <= band_sms() / 2 ? many : few;
+}
+// d_list: n layers of at most r_max rows that take `ctas` CTAs each
+int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, int r_max, cudaStream_t st) {
   if (n <= 0) return 0;
   switch (ctas) {
-    case 1: return chase_launch<1>(d_layers, d_list, n, st);
-    case 2: return chase_launch<2>(d_layers, d_list, n, st);
-    default: return chase_launch<4>(d_layers, d_list, n, st);
+    case 1: return chase_launch<1, 1024>(d_layers, d_list, n, st);
+    case 2: return chase_launch<2, 1024>(d_layers, d_list, n, st);
+    case 4: return r_max <= 1024 ? chase_launch<4, 256>(d_layers, d_list, n, st) : chase_launch<4, 1024>(d_layers, d_list, n, st);
+    case 8: return chase_launch<8, 256>(d_layers, d_list, n, st);
+    default: return chase_launch<16, 256>(d_layers, d_list, n, st);
   }
 }
 
