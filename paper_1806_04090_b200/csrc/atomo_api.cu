@@ -850,7 +850,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // the other; a single layer with more block pairs than the GPU holds CTAs falls back to one launch per step.
   if (tri_form) {
     if (n_clusters > 0) {
-      const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, rp_max_small, st);
+      const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, d_flag + 1, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(tridiagonal reduction)");
       ++n_eig_launch;
     }

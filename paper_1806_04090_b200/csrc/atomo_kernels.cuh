@@ -155,7 +155,7 @@ int sp_tridiag_max_rp();
 int sp_tridiag_cluster_ctas();
 int sp_tridiag_ctas_of(int rp);                                   // CTAs a layer of padded short side rp takes
 int sp_configure_tridiag();                                       // co-resident clusters (0: route not available)
-int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_clusters, int rp_max, cudaStream_t st);  // cudaError_t
+int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_clusters, uint32_t* d_timeout, cudaStream_t st);  // cudaError_t
 void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t n_eigenvalues, cudaStream_t st);
 void launch_sp_eigvec(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st);
 // tridiagonal route for short sides above 512 (atomo_band.cu, vectors in atomo_tridiag_big.cu)

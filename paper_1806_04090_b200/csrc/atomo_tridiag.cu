@@ -4,10 +4,9 @@
 //
 //   sp_tridiag_cluster_kernel : Householder reduction of the scaled Gram matrix A (r x r) to a symmetric
 //                               tridiagonal T = Q^T A Q, in fp64.  A layer's rows sit in blocks of 32 on rp/32 CTAs
-//                               of a 16-CTA cluster and stay in registers; per step the product A v, the next
-//                               pivot column's ingredients and the parts of p^T v travel through distributed
-//                               shared memory (one cluster barrier per step).  The reflectors go to global memory
-//                               as fp32 unit vectors for the back-transformation.
+//                               of a 16-CTA cluster and stay in registers; per step the product A v and the next
+//                               pivot column's ingredients travel through distributed shared memory.  The
+//                               reflectors go to global memory as fp32 unit vectors for the back-transformation.
 //   sp_bisect_kernel          : all eigenvalues of T, eight lanes per eigenvalue: 13 rounds of 9-section on Sturm
 //                               counts (division-free three-term recurrence with power-of-two rescaling).
 //   (sp_finalize_sample_kernel sorts, solves Algorithm 1 and draws, as for the other routes)
@@ -32,291 +31,240 @@ namespace atomo {
 namespace {
 
 constexpr int kTriCtas = 16;          // CTAs per cluster
-constexpr int kTriThreads = 512;
+constexpr int kTriThreads = 256;
 constexpr int kTriWarps = kTriThreads / 32;
-constexpr int kTriRows = 32;          // rows of A per CTA
+constexpr int kTriRows = 32;          // rows of A per CTA, four per warp
 constexpr int kTriMaxRp = 512;        // largest padded short side
 constexpr int kTriCols = kTriMaxRp / 32;   // columns per lane
+constexpr uint32_t kTriWaitLimit = 1u << 18;
 
 }  // namespace
 
 // ---- Householder tridiagonalisation ------------------------------------------------------------------------
 // Step k (k = 0 .. r-3) with x = A[k+1.., k]:  alpha = -sign(x_0) ||x||,  v = x - alpha e_1,  beta = 2 / v^T v,
-// H = I - beta v v^T;  p = beta A22 v,  K = beta/2 p^T v,  w = p - K v,  A22 -= v w^T + w v^T;  d_k = A[k][k],
+// H = I - beta v v^T;  q = A22 v,  K = beta^2/2 q^T v,  w = beta q - K v,  A22 -= v w^T + w v^T;  d_k = A[k][k],
 // e_k = alpha.
-// Layout: CTA g of a layer's nc = rp / 32 CTAs holds the rows 32 g .. 32 g + 31, two per warp, in registers for the
-// whole reduction; a lane holds the columns j = lane + 32 m.  The 32 entries of a vector that a CTA produces are
-// contiguous: one warp sends them to a peer as one 256-byte store into the peer's shared memory.  The trailing
-// block shrinks from the top left: column slots m < (k+1)/32 are dead and skipped, so a step costs in proportion
-// to the columns that are left (the CTAs of the dead rows only keep the barriers).
-// One cluster barrier per step: with p_i the owners also send c_i = A[i][k+1] as it is after update k-1, from which
-// every CTA forms the next pivot column x_i = c_i - v_i w_{k+1} - w_i v_{k+1} itself, hence v_{k+1}; the update of
-// step k and the product A v_{k+1} then share one pass over the rows.
-__device__ __forceinline__ double tri_block_sum(double x, double* s_red, int lane, int w) {
-  x = warp_sum(x);
-  if (lane == 0) s_red[w] = x;
-  __syncthreads();
-  double t = s_red[lane & (kTriWarps - 1)];
-#pragma unroll
-  for (int o = kTriWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;                                                   // the same bits in every thread of the CTA
+// Layout: CTA g of a layer's nc = rp / 32 CTAs holds the rows 32 g .. 32 g + 31, four per warp, in registers for the
+// whole reduction; a lane holds the columns lane + 32 (nc-1-m) in slot m, so that the columns still alive are the
+// first slots.  The trailing block shrinks from the top left: a step works on the live slots only, and a CTA whose
+// rows are all done leaves the exchange.
+// A step is a chain of short dependent pieces (the fp64 work of 512 rows is 770 cycles at most, on average half of
+// that), so the pieces are few: with q_i the owners also send c_i = A[i][k+1] as it is after update k-1, from which
+// every CTA forms the next pivot column x_i = c_i - v_i w_{k+1} - w_i v_{k+1} itself; the update of step k and the
+// product of A with that column, its first entry left out, share one pass over the rows, while the norm of the column
+// is still being summed up; the reflector's first entry v_0 = x_0 - alpha is added as v_0 A[i][k+2] afterwards.  The
+// entries travel as asynchronous stores into the peers' shared memory that count down a barrier there (980 cycles for
+// 16 CTAs, against 1660 for stores and a cluster barrier).  Eight warps: every exchange between lanes is paid once
+// per warp, and the fp64 chains of two warps per scheduler do not get in each other's way.
+// 512 rows: 1408 -> 749 us, 64 rows: 148 -> 75 us (before: sixteen warps of two rows, stores and a cluster barrier, the
+// reflector ahead of the pass).
+__device__ __forceinline__ uint32_t tri_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t tri_map(uint32_t a, int rank) {
+  uint32_t o;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(rank));
+  return o;
 }
-
-// alpha, beta and the first entry of v from ||x||^2 and x_0.  The square root comes from the reciprocal square root
-// and beta from a reciprocal: two short dependent sequences instead of a square root and a division (the chain sits
-// on the critical path of every step); v^T v / 2 = alpha (alpha - x_0) = ||x||^2 + |x_0| ||x||.
-__device__ __forceinline__ void tri_reflector(double nx2, double x0, double& alpha, double& beta, double& v0) {
-  alpha = 0.0; beta = 0.0; v0 = 0.0;
-  if (nx2 > 1.0e-290) {                                       // below: treated as a zero column (H = I)
-    const double nx = nx2 * rsqrt(nx2);
-    alpha = -copysign(nx, x0);
-    v0 = x0 - alpha;
-    const double den = fma(fabs(x0), nx, nx2);
-    beta = __drcp_rn(den);
+// bounded wait for a phase of a barrier in shared memory; false if it ran out
+__device__ __forceinline__ bool tri_wait(uint32_t bar, uint32_t phase) {
+  for (uint32_t n = 0; n < kTriWaitLimit; ++n) {
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(bar), "r"(phase) : "memory");
+    if (ok) return true;
   }
+  return false;
+}
+// sum of eight doubles in shared memory, the same bits in every thread
+__device__ __forceinline__ double tri_sum8(const double* s) {
+  const double2* q = reinterpret_cast<const double2*>(s);
+  const double2 a = q[0], b = q[1], c = q[2], d = q[3];
+  return ((a.x + a.y) + (b.x + b.y)) + ((c.x + c.y) + (d.x + d.y));
 }
 
-// one entry of each of the two register rows, slot chosen at run time (uniform over the warp): a jump, not 16 selects
-#define TRI_PICK(slot, out0, out1)                                                                       \
-  switch (slot) {                                                                                        \
-    case 0: out0 = row0[0]; out1 = row1[0]; break;    case 1: out0 = row0[1]; out1 = row1[1]; break;     \
-    case 2: out0 = row0[2]; out1 = row1[2]; break;    case 3: out0 = row0[3]; out1 = row1[3]; break;     \
-    case 4: out0 = row0[4]; out1 = row1[4]; break;    case 5: out0 = row0[5]; out1 = row1[5]; break;     \
-    case 6: out0 = row0[6]; out1 = row1[6]; break;    case 7: out0 = row0[7]; out1 = row1[7]; break;     \
-    case 8: out0 = row0[8]; out1 = row1[8]; break;    case 9: out0 = row0[9]; out1 = row1[9]; break;     \
-    case 10: out0 = row0[10]; out1 = row1[10]; break; case 11: out0 = row0[11]; out1 = row1[11]; break;  \
-    case 12: out0 = row0[12]; out1 = row1[12]; break; case 13: out0 = row0[13]; out1 = row1[13]; break;  \
-    case 14: out0 = row0[14]; out1 = row1[14]; break; default: out0 = row0[15]; out1 = row1[15]; break;  \
+// an entry of each of the four register rows, slot chosen at run time (uniform over the warp): a jump, not 64 selects
+#define TRI_CASE(M) case M: c[0] = row[0][M]; c[1] = row[1][M]; c[2] = row[2][M]; c[3] = row[3][M]; break;
+#define TRI_PICK(slot)                                                                                    \
+  switch (slot) {                                                                                         \
+    TRI_CASE(0) TRI_CASE(1) TRI_CASE(2) TRI_CASE(3) TRI_CASE(4) TRI_CASE(5) TRI_CASE(6) TRI_CASE(7)       \
+    TRI_CASE(8) TRI_CASE(9) TRI_CASE(10) TRI_CASE(11) TRI_CASE(12) TRI_CASE(13) TRI_CASE(14)              \
+    default: c[0] = row[0][15]; c[1] = row[1][15]; c[2] = row[2][15]; c[3] = row[3][15]; break;           \
   }
 
 __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(const SpLayer* __restrict__ layers,
-                                                                            const ClusterCta* __restrict__ ctas) {
-  static_assert(kTriCols == 16, "TRI_PICK lists 16 slots");
+                                                                            const ClusterCta* __restrict__ ctas,
+                                                                            uint32_t* __restrict__ timeout_flag) {
+  static_assert(kTriCols == 16 && kTriWarps == 8 && kTriRows == 4 * kTriWarps, "TRI_PICK lists 16 slots, four rows per warp");
   cg::cluster_group cluster = cg::this_cluster();
-  __shared__ double s_p[2][kTriMaxRp];                        // beta A22 v of step k in s_p[k & 1] (written by the row owners)
-  __shared__ double s_c[2][kTriMaxRp];                        // column k+1 after update k-1, likewise
-  __shared__ double s_v[2][kTriMaxRp];                        // v of step k in s_v[k & 1]
-  __shared__ double s_w[kTriMaxRp];
-  __shared__ double s_stage[2][kTriRows];                     // this CTA's 32 entries of p and c on their way out
-  __shared__ double s_pk[2][kTriCtas];                        // the CTAs' parts of p^T v, sent along with p (same parity)
-  __shared__ double s_red2[kTriWarps];
-  __shared__ double s_x0, s_scal[3];                          // first entry of the next pivot column; alpha, beta, v_0 of the next reflector
+  // the vectors' entries start at [32]: a pass over an even number of slots may run into the 32 zeros before them
+  __shared__ __align__(16) double2 s_qc[2][kTriMaxRp];        // (q, c) of step k in s_qc[(k + 1) & 1] (written by the row owners)
+  __shared__ __align__(16) double s_v[2][32 + kTriMaxRp];     // v of step k, likewise
+  __shared__ __align__(16) double s_w[32 + kTriMaxRp];
+  __shared__ __align__(16) double s_k[kTriWarps], s_n[kTriWarps];
+  __shared__ __align__(16) double s_c2[kTriRows];
+  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ double s_x0;
   const ClusterCta me = ctas[blockIdx.x];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  // every CTA of the cluster keeps the same number of barriers: the longest reduction among the cluster's layers
-  int steps = 0;
-  {
-    const int c0 = blockIdx.x / kTriCtas * kTriCtas;
-    for (int c = 0; c < kTriCtas; ++c) { const int l = ctas[c0 + c].layer; if (l >= 0) steps = max(steps, layers[l].r - 2); }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tri_smem(&s_bar[0])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tri_smem(&s_bar[1])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = tid; i < 32 + kTriMaxRp; i += kTriThreads) { s_v[0][i] = s_v[1][i] = s_w[i] = 0.0; }
+  for (int i = tid; i < kTriMaxRp; i += kTriThreads) { s_qc[0][i] = s_qc[1][i] = make_double2(0.0, 0.0); }
   cluster.sync();                                             // every CTA of the cluster runs: remote stores may start
-  if (me.layer < 0) {
-    for (int k = 0; k <= steps; ++k) cluster.sync();
-    cluster.sync();
-    return;
-  }
+  if (me.layer < 0) { cluster.sync(); return; }
   const SpLayer& L = layers[me.layer];
   const int r = L.r, nc = me.pad, g = me.slot, base = me.base_rank;
   // the layer's pointers in registers: a field read through `layers` inside a loop would be a global load each time
   double* const td_d = L.td_d; double* const td_e = L.td_e; double* const td_tau = L.td_tau; float* const td_V = L.td_V;
   const float* const gA = L.A; const int64_t lda = L.lda; const int ldv = L.td_ldv;
   const int my_steps = max(r - 2, 0);
-  const int li0 = w, li1 = w + kTriWarps;                     // this warp's two rows
-  const int i0 = 32 * g + li0, i1 = 32 * g + li1;
-  double row0[kTriCols], row1[kTriCols];
+  const int row_lo = 32 * g + 4 * w;                          // this warp's rows
+  double row[4][kTriCols];
 #pragma unroll
   for (int m = 0; m < kTriCols; ++m) {
-    const int j = lane + 32 * m;
-    const bool in = m < nc && j < r;
-    row0[m] = (in && i0 < r) ? (double)gA[(int64_t)i0 * lda + j] : 0.0;
-    row1[m] = (in && i1 < r) ? (double)gA[(int64_t)i1 * lda + j] : 0.0;
-  }
-  const int sq = w * 32 + lane;                               // this thread's entry of the vectors (warps < nc)
-  const int sj = sq;                                          // its index
-  const bool slice = w < nc;
-  // ---- the first reflector and A v_0 ----
-  double beta = 0.0, v0 = 0.0;
-  if (my_steps > 0) {
-    const double xq = (slice && sj > 0 && sj < r) ? (double)gA[sj] : 0.0;   // column 0 = row 0 (symmetric)
-    if (slice) s_v[0][sq] = xq;
-    const double nx2 = tri_block_sum(xq * xq, s_red2, lane, w);
-    const int q1 = 1;
-    if (tid == 0) {
-      double alpha;
-      tri_reflector(nx2, (double)gA[1], alpha, beta, v0);
-      s_scal[0] = alpha; s_scal[1] = beta; s_scal[2] = v0;
-      s_v[0][q1] = v0;
-      if (g == 0) { td_d[0] = (double)gA[0]; td_e[0] = alpha; td_tau[0] = beta; }
-    }
-    __syncthreads();
-    beta = s_scal[1]; v0 = s_scal[2];
-    {
-      // reflectors are filed as unit vectors (H = I - 2 u u^T, u = v sqrt(beta / 2)): no range trouble in fp32
-      const double un = sqrt(0.5 * beta);
-      if (g == 0) for (int j = tid; j < r; j += kTriThreads) td_V[j] = (float)(s_v[0][j] * un);   // row 0
-    }
-    double a0 = 0.0, a1 = 0.0;
+    const int j = lane + 32 * (nc - 1 - m);
 #pragma unroll
-    for (int m = 0; m < kTriCols; ++m) {
-      if (m < nc) {
-        const double vq = s_v[0][lane + 32 * m];
-        a0 = fma(row0[m], vq, a0); a1 = fma(row1[m], vq, a1);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { a0 += __shfl_xor_sync(0xffffffffu, a0, o); a1 += __shfl_xor_sync(0xffffffffu, a1, o); }
-    double c0 = 0.0, c1 = 0.0;
-    TRI_PICK(q1 >> 5, c0, c1);
-    if (lane == (q1 & 31)) { s_stage[1][li0] = c0; s_stage[1][li1] = c1; }
-    if (lane == 0) {
-      s_stage[0][li0] = (i0 > 0 && i0 < r) ? a0 * beta : 0.0;
-      s_stage[0][li1] = (i1 > 0 && i1 < r) ? a1 * beta : 0.0;
-    }
+    for (int e = 0; e < 4; ++e) row[e][m] = m < nc && j < r && row_lo + e < r ? (double)gA[(int64_t)(row_lo + e) * lda + j] : 0.0;
   }
+  const int jA = tid, jB = tid + kTriThreads;                 // this thread's entries of the vectors
+  // step -1: no update, the pivot column is column 0
+  if (jA < r) s_qc[0][jA] = make_double2(0.0, (double)gA[jA]);
+  if (jB < r) s_qc[0][jB] = make_double2(0.0, (double)gA[jB]);
   __syncthreads();
-  if (my_steps > 0 && w < nc) {                               // warp w carries this CTA's 32 entries to peer w
-    const double pl = s_stage[0][lane];
-    cluster.map_shared_rank(&s_p[0][0], base + w)[g * 32 + lane] = pl;
-    cluster.map_shared_rank(&s_c[0][0], base + w)[g * 32 + lane] = s_stage[1][lane];
-    // ... and this CTA's part of p^T v (its 32 rows), from which every CTA forms K without a reduction of its own
-    const double part = warp_sum(pl * s_v[0][g * 32 + lane]);
-    if (lane == 0) cluster.map_shared_rank(&s_pk[0][0], base + w)[g] = part;
-  }
-  cluster.sync();
-  // warp w < nc talks to peer w: that CTA's copies of the three arrays, mapped once
-  const int peer = base + min(w, nc - 1);
-  double* const peer_p = cluster.map_shared_rank(&s_p[0][0], peer);
-  double* const peer_c = cluster.map_shared_rank(&s_c[0][0], peer);
-  double* const peer_pk = cluster.map_shared_rank(&s_pk[0][0], peer);
-  // A layer that fills its cluster finishes alone: once every live row sits in the CTA of the last rows, that CTA runs
-  // the remaining steps (at most 31) by itself, with stores into its own shared memory and __syncthreads in place of
-  // the cluster barrier, and the other CTAs leave the loop.
-  const int g_last = (max(r, 1) - 1) >> 5;
-  const int k_tail = nc == kTriCtas ? 32 * g_last - 1 : 0x7fffffff;
-  // instances: with the cluster (a layer that fills it, or a smaller one) and alone; for the layers that fill the
-  // cluster also one per first live column slot, so that the pass over the rows is straight-line code
-  auto step = [&](auto solo_tag, auto full_tag, auto mlo_tag, const int k) {
-    constexpr bool solo = decltype(solo_tag)::value;
-    constexpr int kMlo = decltype(mlo_tag)::value;            // first live column slot, or -1: taken from k at run time
-    constexpr bool full = decltype(full_tag)::value;          // the layer has all kTriCtas CTAs: loop bounds known at compile time
-    const int ncc = full ? kTriCtas : nc;
-    const bool active = k < my_steps;
-    const bool last = k + 1 == my_steps;                      // no reflector follows
-    const int par = k & 1, nxt = par ^ 1;
+  double vA = 0.0, vB = 0.0, beta = 0.0, v0 = 0.0;            // v, beta and the first entry of v of step k
+  const int e_own = lane >> 3;                                // the row whose sum this lane ends up with
+  const bool files = g == (max(r, 1) - 1) >> 5;               // the CTA of the last rows, alive to the end, files T and the reflectors
+  const uint32_t dst0 = tri_map(tri_smem(&s_qc[0][row_lo + e_own]), base + min(lane & 7, nc - 1));
+  const uint32_t dst1 = tri_map(tri_smem(&s_qc[0][row_lo + e_own]), base + min((lane & 7) + 8, nc - 1));
+  const uint32_t bar0 = tri_map(tri_smem(&s_bar[0]), base + min(lane & 7, nc - 1));
+  const uint32_t bar1 = tri_map(tri_smem(&s_bar[0]), base + min((lane & 7) + 8, nc - 1));
+  for (int k = -1; k < my_steps && 32 * g + 31 >= k + 2; ++k) {
+    const int par = (k + 1) & 1, nxt = par ^ 1;
     const int q1 = k + 1, q2 = k + 2;
-    const int m_lo = kMlo >= 0 ? kMlo : (k + 1) >> 5;         // first column slot that is still alive
-    double beta_n = 0.0, v0_n = 0.0;
-    if (active) {
-      // K = beta/2 p^T v: the CTAs' parts arrived with p; every thread adds them in the same order
-      const double vq = slice ? s_v[par][sq] : 0.0;
-      const double pq = slice ? s_p[par][sq] : 0.0;
-      const int kc = lane & (kTriCtas - 1);                   // (alone, only this CTA's part is there)
-      double ksum = (solo ? kc == g : kc < ncc) ? s_pk[par][kc] : 0.0;
+    const bool last = q1 == my_steps;                         // no reflector follows
+    const int g_lo = q2 >> 5;                                 // first CTA, and first block of columns, that is still alive
+    if (k >= 0 && !tri_wait(tri_smem(&s_bar[par]), (uint32_t)(k >> 1) & 1u)) { *timeout_flag = 1u; break; }
+    const double2 qcA = s_qc[par][jA], qcB = s_qc[par][jB];
+    const double2 qc1 = s_qc[par][min(q1, kTriMaxRp - 1)];
+    // K = beta^2/2 q^T v (v is zero outside the live rows)
+    const double part = warp_sum(fma(qcA.x, vA, qcB.x * vB));
+    if (lane == 0) s_k[w] = part;
+    __syncthreads();
+    const double K = 0.5 * beta * beta * tri_sum8(s_k);
+    const double w1 = fma(-K, v0, beta * qc1.x);              // w_{k+1}
+    const bool inA = jA > q1 && jA < r, inB = jB > q1 && jB < r;
+    const double wA = inA ? fma(-K, vA, beta * qcA.x) : 0.0, wB = inB ? fma(-K, vB, beta * qcB.x) : 0.0;
+    const double xA = inA ? qcA.y - fma(vA, w1, wA * v0) : 0.0, xB = inB ? qcB.y - fma(vB, w1, wB * v0) : 0.0;
+    s_w[32 + jA] = wA; s_w[32 + jB] = wB;
+    s_v[nxt][32 + jA] = jA == q2 ? 0.0 : xA; s_v[nxt][32 + jB] = jB == q2 ? 0.0 : xB;
+    if (jA == q2) s_x0 = xA;
+    if (jB == q2) s_x0 = xB;
+    if (files) {
+      if (tid == (q1 & (kTriThreads - 1))) td_d[q1] = qc1.y - 2.0 * v0 * w1;
+      if (last && r > 1 && tid == ((r - 1) & (kTriThreads - 1))) td_e[r - 2] = r - 1 < kTriThreads ? xA : xB;
+    }
+    __syncthreads();
+    if (tid == 0 && !last) {
+      const uint32_t bytes = (uint32_t)(nc - g_lo) * kTriRows * sizeof(double2);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tri_smem(&s_bar[nxt])), "r"(bytes) : "memory");
+    }
+    // update of the rows with (v, w), fused with their products with the next v; meanwhile the norm of the next column
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    double nsq = fma(xA, xA, xB * xB);
+    auto pass = [&](auto n_tag) {
+      constexpr int kN = decltype(n_tag)::value;
+      nsq = warp_sum(nsq);
+      double vi[4], wi[4];
 #pragma unroll
-      for (int o = kTriCtas / 2; o > 0; o >>= 1) ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
-      const double K = 0.5 * beta * ksum;
-      const double w1 = fma(-K, v0, s_p[par][q1]);            // w_{k+1}
-      // w, and the next pivot column x_j = c_j - v_j w_{k+1} - w_j v_{k+1} for j > k+1
-      const double wq = fma(-K, vq, pq);
-      double xn = 0.0;
-      if (slice) {
-        s_w[sq] = wq;
-        if (sj > k + 1 && sj < r && !last) xn = s_c[par][sq] - fma(vq, w1, wq * v0);
-        s_v[nxt][sq] = xn;
-        if (sq == q2) s_x0 = xn;
+      for (int e = 0; e < 4; e += 2) {
+        const double2 v2 = *reinterpret_cast<const double2*>(&s_v[par][32 + row_lo + e]), w2 = *reinterpret_cast<const double2*>(&s_w[32 + row_lo + e]);
+        vi[e] = -v2.x; vi[e + 1] = -v2.y; wi[e] = -w2.x; wi[e + 1] = -w2.y;
       }
-      const double nx2 = tri_block_sum(xn * xn, s_red2, lane, w);
-      if (tid == 0) {                                         // one thread forms the reflector; a zero column gives v = 0
-        double alpha_n;
-        tri_reflector(nx2, s_x0, alpha_n, beta_n, v0_n);
-        s_scal[0] = alpha_n; s_scal[1] = beta_n; s_scal[2] = v0_n;
-        if (!last) s_v[nxt][q2] = v0_n;
-      }
-      __syncthreads();
-      beta_n = s_scal[1]; v0_n = s_scal[2];
-      // update of the two rows with (v, w), fused with their products with the next v
-      const double vi0 = s_v[par][g * 32 + li0], vi1 = s_v[par][g * 32 + li1];
-      const double wi0 = s_w[g * 32 + li0], wi1 = s_w[g * 32 + li1];
-      const double* __restrict__ pv = &s_v[par][lane];
-      const double* __restrict__ pn = &s_v[nxt][lane];
-      const double* __restrict__ pw = &s_w[lane];
-      double a0 = 0.0, a1 = 0.0;
+      const int at = 32 * nc + lane;                          // slot m: [at - 32 m]
 #pragma unroll
-      for (int m = 0; m < kTriCols; ++m) {
-        if (m >= m_lo && m < ncc) {
-          const double vq2 = pv[32 * m], wq2 = pw[32 * m], vn = pn[32 * m];
-          row0[m] = fma(-vi0, wq2, fma(-wi0, vq2, row0[m]));
-          row1[m] = fma(-vi1, wq2, fma(-wi1, vq2, row1[m]));
-          a0 = fma(row0[m], vn, a0); a1 = fma(row1[m], vn, a1);
+      for (int m = 0; m < kN; ++m) {
+        const double vq = s_v[par][at - 32 * m], wq = s_w[at - 32 * m], vn = s_v[nxt][at - 32 * m];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          row[e][m] = fma(vi[e], wq, fma(wi[e], vq, row[e][m]));
+          a[e] = fma(row[e][m], vn, a[e]);
         }
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) { a0 += __shfl_xor_sync(0xffffffffu, a0, o); a1 += __shfl_xor_sync(0xffffffffu, a1, o); }
-      // column k+2 of the two rows goes out with the products; column k+1 holds the entries of T that are final now
-      double c20 = 0.0, c21 = 0.0;
-      TRI_PICK(q2 >> 5, c20, c21);
+    };
+#define TRI_PASS(N) pass(std::integral_constant<int, N>{})
+    switch (nc - g_lo) {
+      case 0: case 1: TRI_PASS(1); break;
+      case 2: TRI_PASS(2); break;
+      case 3: case 4: TRI_PASS(4); break;
+      case 5: case 6: TRI_PASS(6); break;
+      case 7: case 8: TRI_PASS(8); break;
+      case 9: case 10: TRI_PASS(10); break;
+      case 11: case 12: TRI_PASS(12); break;
+      case 13: case 14: TRI_PASS(14); break;
+      default: TRI_PASS(16); break;
+    }
+#undef TRI_PASS
+    if (lane == 0) s_n[w] = nsq;
+    {                                                         // column k+2 of the rows
+      double c[4];
+      TRI_PICK(nc - 1 - g_lo)
       if (lane == (q2 & 31)) {
-        s_stage[1][li0] = c20; s_stage[1][li1] = c21;
-        if (last) { if (i0 == r - 1) td_d[r - 1] = c20; if (i1 == r - 1) td_d[r - 1] = c21; }
-      }
-      if (i0 == k + 1 || i1 == k + 1 || (last && (i0 == r - 1 || i1 == r - 1))) {
-        double c10 = 0.0, c11 = 0.0;
-        TRI_PICK(q1 >> 5, c10, c11);
-        if (lane == (q1 & 31)) {
-          if (i0 == k + 1) td_d[k + 1] = c10;
-          if (i1 == k + 1) td_d[k + 1] = c11;
-          if (last) { if (i0 == r - 1) td_e[r - 2] = c10; if (i1 == r - 1) td_e[r - 2] = c11; }
-        }
-      }
-      if (lane == 0) {
-        s_stage[0][li0] = (i0 > k + 1 && i0 < r) ? a0 * beta_n : 0.0;
-        s_stage[0][li1] = (i1 > k + 1 && i1 < r) ? a1 * beta_n : 0.0;
+        *reinterpret_cast<double2*>(&s_c2[4 * w]) = make_double2(c[0], c[1]);
+        *reinterpret_cast<double2*>(&s_c2[4 * w + 2]) = make_double2(c[2], c[3]);
       }
     }
     __syncthreads();
-    if (active && !last && (solo ? w == 0 : w < ncc)) {        // alone: the same entries into this CTA's own arrays
-      double* const to_p = solo ? &s_p[0][0] : peer_p;
-      double* const to_c = solo ? &s_c[0][0] : peer_c;
-      double* const to_pk = solo ? &s_pk[0][0] : peer_pk;
-      const double pl = s_stage[0][lane];
-      to_p[nxt * kTriMaxRp + g * 32 + lane] = pl;
-      to_c[nxt * kTriMaxRp + g * 32 + lane] = s_stage[1][lane];
-      const double part = warp_sum(pl * s_v[nxt][g * 32 + lane]);
-      if (lane == 0) to_pk[nxt * kTriCtas + g] = part;
+    const double nx2 = tri_sum8(s_n), x0 = s_x0, c2 = s_c2[4 * w + e_own];
+    if (last) {                                               // order 1 and 2 as they are: only the last diagonal entry is left
+      if (r > 1 && (lane & 7) == 0 && row_lo + e_own == r - 1) td_d[r - 1] = c2;
+      break;
     }
-    if (!solo) cluster.barrier_arrive();                      // (release) the entries above are on their way
-    if (active && !last && (solo || g == 0)) {                // meanwhile the CTA of the first rows (dead after 31 steps) files the reflector
-      if (tid == 0) { td_e[k + 1] = s_scal[0]; td_tau[k + 1] = beta_n; }
-      const double un = sqrt(0.5 * beta_n);                   // filed as a unit vector: H = I - 2 u u^T
-      for (int j = tid; j < r; j += kTriThreads) td_V[(int64_t)(k + 1) * ldv + j] = (float)(s_v[nxt][j] * un);
+    // the sums of the four rows over the lanes: lane ends with row lane / 8
+    double sum;
+    {
+      const bool h4 = lane & 16, h3 = lane & 8;
+      const double b0 = (h4 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h4 ? a[0] : a[2], 16);
+      const double b1 = (h4 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h4 ? a[1] : a[3], 16);
+      sum = (h3 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h3 ? b0 : b1, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     }
-    beta = beta_n; v0 = v0_n;
-    if (solo) __syncthreads(); else cluster.barrier_wait();
-  };
-  const int k_mid = min(steps, k_tail);
-  using Dyn = std::integral_constant<int, -1>;
-  if (nc == kTriCtas) {
-#define TRI_SLOT(M) case M: step(std::false_type{}, std::true_type{}, std::integral_constant<int, M>{}, k); break;
-    for (int k = 0; k < k_mid; ++k) {
-      switch ((k + 1) >> 5) {
-        TRI_SLOT(0) TRI_SLOT(1) TRI_SLOT(2) TRI_SLOT(3) TRI_SLOT(4) TRI_SLOT(5) TRI_SLOT(6) TRI_SLOT(7)
-        TRI_SLOT(8) TRI_SLOT(9) TRI_SLOT(10) TRI_SLOT(11) TRI_SLOT(12) TRI_SLOT(13) TRI_SLOT(14)
-        default: step(std::false_type{}, std::true_type{}, std::integral_constant<int, 15>{}, k); break;
-      }
+    // the square root comes from the reciprocal square root; v^T v / 2 = ||x||^2 + |x_0| ||x||
+    double alpha = 0.0, half = 0.0;
+    v0 = 0.0;
+    if (nx2 > 1.0e-290) {                                     // below: treated as a zero column (H = I)
+      const double nx = nx2 * rsqrt(nx2);
+      alpha = -copysign(nx, x0);
+      v0 = x0 - alpha;
+      half = fma(fabs(x0), nx, nx2);
     }
-#undef TRI_SLOT
-    if (g == g_last) for (int k = k_mid; k < steps; ++k) step(std::true_type{}, std::true_type{}, Dyn{}, k);
-  } else {
-    for (int k = 0; k < steps; ++k) step(std::false_type{}, std::false_type{}, Dyn{}, k);
-  }
-  // matrices of order 1 and 2 are tridiagonal as they are
-  if (my_steps == 0 && g == 0 && tid == 0) {
-    td_d[0] = (double)gA[0];
-    if (r == 2) { td_d[1] = (double)gA[lda + 1]; td_e[0] = (double)gA[lda]; }
+    // (q, c) of the rows to the CTAs that are alive in the next step; two peers per lane
+    {
+      const double q = fma(v0, c2, sum);
+      const int peer_lo = (q2 + 1) >> 5, t = lane & 7;
+      const uint32_t off = nxt * (uint32_t)sizeof(s_qc[0]), offb = nxt * (uint32_t)sizeof(s_bar[0]);
+      if (t >= peer_lo && t < nc)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(dst0 + off), "d"(q), "d"(c2), "r"(bar0 + offb) : "memory");
+      if (t + 8 >= peer_lo && t + 8 < nc)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(dst1 + off), "d"(q), "d"(c2), "r"(bar1 + offb) : "memory");
+    }
+    const double un = half > 0.0 ? rsqrt(2.0 * half) : 0.0;   // 1 / ||v||
+    beta = 2.0 * un * un;
+    vA = jA == q2 ? v0 : xA; vB = jB == q2 ? v0 : xB;
+    if (jA == q2) s_v[nxt][32 + jA] = v0;
+    if (jB == q2) s_v[nxt][32 + jB] = v0;
+    if (files) {                                              // reflectors as unit vectors (H = I - 2 u u^T): no range trouble in fp32
+      if (jA < r) td_V[(int64_t)q1 * ldv + jA] = (float)(vA * un);
+      if (jB < r) td_V[(int64_t)q1 * ldv + jB] = (float)(vB * un);
+      if (tid == 0) { td_e[q1] = alpha; td_tau[q1] = beta; }
+    }
   }
   cluster.sync();                                             // nobody leaves while a peer may still write here
 }
 #undef TRI_PICK
+#undef TRI_CASE
 
 // ---- eigenvalues of T: Sturm counts -------------------------------------------------------------------------
 // count(x) = number of eigenvalues below x = sign changes of p_0 = 1, p_1 = d_0 - x, p_{i+1} = (d_i - x) p_i -
@@ -577,7 +525,6 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
 }
 
 // ---- host side ---------------------------------------------------------------------------------------------------
-static size_t tri_smem_bytes(int) { return 0; }             // rows in registers, vectors in static shared memory
 static size_t vec_smem_bytes(int rp_max) {
   return (size_t)(2 + kVecWork * kVecWarps) * rp_max * sizeof(double) + (size_t)kVecStages * kVecGroup * rp_max * sizeof(float);
 }
@@ -601,15 +548,14 @@ int sp_configure_bisect() {
 
 int sp_configure_tridiag() {
   // optional route: a GPU that refuses the cluster size or the shared memory simply reports it as unavailable
-  if (cudaFuncSetAttribute(sp_tridiag_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem_bytes(kTriMaxRp)) != cudaSuccess ||
-      cudaFuncSetAttribute(sp_tridiag_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+  if (cudaFuncSetAttribute(sp_tridiag_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
       cudaFuncSetAttribute(sp_eigvec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_smem_bytes(kTriMaxRp)) != cudaSuccess ||
       sp_configure_bisect() != 0) {
     cudaGetLastError();
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kTriCtas); cfg.blockDim = dim3(kTriThreads); cfg.dynamicSmemBytes = tri_smem_bytes(kTriMaxRp);
+  cfg.gridDim = dim3(kTriCtas); cfg.blockDim = dim3(kTriThreads);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = kTriCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -619,15 +565,15 @@ int sp_configure_tridiag() {
   return n;
 }
 
-int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_clusters, int rp_max, cudaStream_t st) {
+int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_clusters, uint32_t* d_timeout, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_clusters * kTriCtas); cfg.blockDim = dim3(kTriThreads);
-  cfg.dynamicSmemBytes = tri_smem_bytes(rp_max); cfg.stream = st;
+  cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = kTriCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return (int)cudaLaunchKernelEx(&cfg, sp_tridiag_cluster_kernel, d_layers, d_ctas);
+  return (int)cudaLaunchKernelEx(&cfg, sp_tridiag_cluster_kernel, d_layers, d_ctas, d_timeout);
 }
 
 void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t n_eigenvalues, cudaStream_t st) {
