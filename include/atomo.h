@@ -234,20 +234,11 @@ int atomo_decode_average(atomo_ctx* ctx, int32_t kind, const void* const* payloa
  * Same result as atomo_decode() for a spectral payload, for callers that must not allocate device
  * memory: a process whose framework allocator already owns the whole GPU, a latency-critical
  * section that cannot take cudaMalloc's device-wide synchronisation, a memory-capped job.  It needs
- * no context and calls no cudaMalloc / cudaFree: the per-call tables (one descriptor per layer, one
- * entry per 64 x 1024 output tile) go into a fixed array inside the library image, about 130 KB that
- * every GPU loading the library holds until the process exits.
- *   - Limits: n_layers <= ATOMO_STATIC_MAX_LAYERS and at most ATOMO_STATIC_MAX_TILES output tiles in
- *     all (sum over layers of ceil(rows/64) * ceil(cols/1024)); beyond that ATOMO_ERR_CAPACITY is
- *     returned and nothing is launched.
- *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress, with
- *     that device made current); make that first call before any stream capture begins.
- *   - All calls on a device share the one array: it still holds the previous call's tables, which
- *     the next call overwrites in stream order.  Two calls whose work overlaps on the GPU (different
- *     streams, no dependency) race on it; serialise them.
- *   - The tables are staged in pageable host memory (up to 128 KB per calling thread): the copy may make
- *     the host wait until earlier work on `stream` has drained, and the staging buffer is reused by the
- *     thread's next call.
+ * no context and calls no cudaMalloc / cudaFree: the layers' descriptors travel as kernel arguments,
+ * so calls share no state and need no order among each other.
+ *   - Limits: n_layers <= ATOMO_STATIC_MAX_LAYERS and at most ATOMO_STATIC_MAX_TILES output tiles of
+ *     64 x 1024 in all (sum over layers of ceil(rows/64) * ceil(cols/1024)); beyond that
+ *     ATOMO_ERR_CAPACITY is returned and nothing is launched.
  *   - out[l] must hold rows[l] * cols[l] floats: every element is written through the raw pointer.
  * `device` is the CUDA ordinal; payload, rows, cols, out, stream as in atomo_decode().               */
 enum { ATOMO_STATIC_MAX_LAYERS = 64, ATOMO_STATIC_MAX_TILES = 8192 };

@@ -37,7 +37,7 @@ struct TableWays {
 
 struct atomo_ctx {
   int device = 0;
-  TableWays tab_sp, tab_dec, tab_avg;
+  TableWays tab_sp, tab_avg;
   int64_t table_uploads = 0, table_reuses = 0;
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
@@ -314,7 +314,7 @@ int atomo_destroy(atomo_ctx* ctx) {
   cudaDeviceSynchronize();
   if (ctx->ws) cudaFree(ctx->ws);
   if (ctx->ew_words) cudaFree(ctx->ew_words);
-  table_free(ctx->tab_sp); table_free(ctx->tab_dec); table_free(ctx->tab_avg);
+  table_free(ctx->tab_sp); table_free(ctx->tab_avg);
   if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
   if (ctx->h_lq) cudaFreeHost(ctx->h_lq);
   if (ctx->ev_sync) cudaEventDestroy(ctx->ev_sync);
@@ -1188,39 +1188,15 @@ int atomo_decode(atomo_ctx* ctx, int32_t kind, const void* payload, const int64_
   cudaStream_t st = (cudaStream_t)stream;
   stage_reset(ctx);
   const uint8_t* pay = static_cast<const uint8_t*>(payload);
-  const atomo_layer_header* d_hdr = reinterpret_cast<const atomo_layer_header*>(pay + sizeof(atomo_payload_header));
   stage_begin(ctx, ATOMO_STAGE_DECODE, st);
   if (kind == ATOMO_KIND_ENTRYWISE) {
     for (int l = 0; l < n_layers; ++l) if (rows[l] != 1) return ATOMO_ERR_INVALID_ARG;
     const int n_launch = for_each_ew_decode(pay, cols, out, n_layers, [&](const auto& B, uint32_t tiles) { launch_ew_decode(B, tiles, st); });
     stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   } else {
-    std::vector<SpDecodeLayer> D(n_layers);
-    std::vector<TileRef> tiles;
-    const int tr = sp_decode_tile_rows(), tc = sp_decode_tile_cols();
-    for (int l = 0; l < n_layers; ++l) {
-      D[l] = SpDecodeLayer{d_hdr + l, out[l], rows[l], cols[l]};
-      const int na = (int)((rows[l] + tr - 1) / tr), nbt = (int)((cols[l] + tc - 1) / tc);
-      for (int a = 0; a < na; ++a) for (int b = 0; b < nbt; ++b) tiles.push_back({l, a, b, 0});
-    }
-    SpDecodeLayer* d_layers = nullptr; TileRef* d_tiles = nullptr;
-    size_t tb = 0;
-    uint64_t key = table_key(kKeySeed, &payload, sizeof(payload));
-    key = table_key(key, out, (size_t)n_layers * sizeof(float*));
-    TableCache& tab = table_pick(ctx->tab_dec, key);
-    for (int pass = 0; pass < 2; ++pass) {
-      Arena T(pass ? tab.d : nullptr);
-      d_layers = T.take<SpDecodeLayer>(n_layers);
-      d_tiles = T.take<TileRef>(tiles.size());
-      tb = T.off + 256;
-      if (pass == 0) { const int rc = table_reserve(ctx, tab, tb); if (rc != ATOMO_OK) return rc; }
-    }
-    std::vector<uint8_t> tables(tb, 0);
-    std::memcpy(tables.data() + (reinterpret_cast<uint8_t*>(d_layers) - tab.d), D.data(), D.size() * sizeof(SpDecodeLayer));
-    std::memcpy(tables.data() + (reinterpret_cast<uint8_t*>(d_tiles) - tab.d), tiles.data(), tiles.size() * sizeof(TileRef));
-    { const int rc = table_commit(ctx, tab, tables.data(), tb, st); if (rc != ATOMO_OK) return rc; }
-    launch_sp_decode(pay, d_layers, d_tiles, (int)tiles.size(), st);
-    stage_end(ctx, ATOMO_STAGE_DECODE, st, 1);
+    ++ctx->table_reuses;                                           // the layers travel as kernel arguments: nothing to upload
+    const int n_launch = launch_sp_decode(pay, nullptr, 1, rows, cols, out, n_layers, st);
+    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   }
   CK(cudaGetLastError());
   return ATOMO_OK;
@@ -1239,42 +1215,25 @@ int atomo_decode_average(atomo_ctx* ctx, int32_t kind, const void* const* payloa
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
   stage_reset(ctx);
-  std::vector<SpDecodeLayer> D;
-  std::vector<TileRef> tiles;
-  if (kind == ATOMO_KIND_SPECTRAL) {
-    D.resize(n_layers);
-    const int tr = sp_decode_tile_rows(), tc = sp_decode_tile_cols();
-    for (int l = 0; l < n_layers; ++l) {
-      D[l] = SpDecodeLayer{nullptr, out[l], rows[l], cols[l]};
-      const int na = (int)((rows[l] + tr - 1) / tr), nbt = (int)((cols[l] + tc - 1) / tc);
-      for (int a = 0; a < na; ++a) for (int b = 0; b < nbt; ++b) tiles.push_back({l, a, b, 0});
-    }
-  }
-  const uint8_t** d_pay = nullptr; SpDecodeLayer* d_layers = nullptr; TileRef* d_tiles = nullptr;
+  const uint8_t** d_pay = nullptr;
   size_t tb = 0;
-  uint64_t key = table_key(kKeySeed, payloads, (size_t)n_payloads * sizeof(void*));
-  key = table_key(key, out, (size_t)n_layers * sizeof(float*));
-  TableCache& tab = table_pick(ctx->tab_avg, key);
+  TableCache& tab = table_pick(ctx->tab_avg, table_key(kKeySeed, payloads, (size_t)n_payloads * sizeof(void*)));
   for (int pass = 0; pass < 2; ++pass) {
     Arena T(pass ? tab.d : nullptr);
     d_pay = T.take<const uint8_t*>(n_payloads);
-    d_layers = T.take<SpDecodeLayer>(D.size());
-    d_tiles = T.take<TileRef>(tiles.size());
     tb = T.off + 256;
     if (pass == 0) { const int rc = table_reserve(ctx, tab, tb); if (rc != ATOMO_OK) return rc; }
   }
   {
     std::vector<uint8_t> tables(tb, 0);
     std::memcpy(tables.data() + (reinterpret_cast<uint8_t*>(d_pay) - tab.d), payloads, (size_t)n_payloads * sizeof(void*));
-    if (!D.empty()) std::memcpy(tables.data() + (reinterpret_cast<uint8_t*>(d_layers) - tab.d), D.data(), D.size() * sizeof(SpDecodeLayer));
-    if (!tiles.empty()) std::memcpy(tables.data() + (reinterpret_cast<uint8_t*>(d_tiles) - tab.d), tiles.data(), tiles.size() * sizeof(TileRef));
     const int rc = table_commit(ctx, tab, tables.data(), tb, st);
     if (rc != ATOMO_OK) return rc;
   }
   stage_begin(ctx, ATOMO_STAGE_DECODE, st);
   if (kind == ATOMO_KIND_SPECTRAL) {
-    launch_sp_decode_average(d_pay, n_payloads, d_layers, d_tiles, (int)tiles.size(), st);
-    stage_end(ctx, ATOMO_STAGE_DECODE, st, 1);
+    const int n_launch = launch_sp_decode(nullptr, d_pay, n_payloads, rows, cols, out, n_layers, st);
+    stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   } else {
     const int n_launch = for_each_ew_decode(nullptr, cols, out, n_layers, [&](const auto& B, uint32_t n_tiles) {
       launch_ew_decode_average(B, n_tiles, d_pay, n_payloads, st);

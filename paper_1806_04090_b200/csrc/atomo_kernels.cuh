@@ -117,15 +117,12 @@ struct SpLayer {
   double* tb_vecwork;          // [slots][5][rp] work vectors of the twisted factorisation
 };
 
-struct SpDecodeLayer {
-  const atomo_layer_header* hdr; float* out; int64_t rows, cols;
-};
+// a layer of a spectral decode: threads per output row, rows per CTA, the layer's first CTA
+struct SpDecodeLayer { float* out; int64_t rows, cols; int32_t layer, width, cta_rows; uint32_t cta0; };
+constexpr int kSpDecodeBatch = 64;
+template <int N> struct SpDecodeBatch { SpDecodeLayer v[N]; int n; };
 
 struct TileRef { int32_t layer, a, b, c; };
-
-// averaging decode of several payloads (combine step of data-parallel training)
-void launch_sp_decode_average(const uint8_t* const* d_payloads, int n_payloads, const SpDecodeLayer* d_layers,
-                              const TileRef* d_tiles, int n_tiles, cudaStream_t st);
 
 // payload header (by value), layer headers from a device template, the call's four flag words
 void launch_sp_begin(uint8_t* pay, const atomo_payload_header& gh, const atomo_layer_header* d_tmpl, int n_layers,
@@ -187,8 +184,9 @@ void launch_sp_finalize_sample(const SpLayer* d_layers, int n_layers, double s, 
                                uint32_t kind_step, int max_sweeps, const uint32_t* timeout_flag, cudaStream_t st);
 void launch_sp_backproject(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, int r_max, cudaStream_t st);
 void launch_sp_finish_atoms(const SpLayer* d_layers, int n_layers, int k_cap_max, cudaStream_t st);
-void launch_sp_decode(const uint8_t* payload, const SpDecodeLayer* d_layers, const TileRef* d_tiles, int n_tiles,
-                      cudaStream_t st);
+// decode of one payload, or (payload null) the mean of n_payloads of them whose addresses are in device memory
+int launch_sp_decode(const uint8_t* payload, const uint8_t* const* d_payloads, int n_payloads, const int64_t* rows, const int64_t* cols,
+                     float* const* out, int n_layers, cudaStream_t st);      // launches
 int sp_configure();          // opt in to large dynamic shared memory; returns cudaError_t
 // tensor-core Gram kernel (atomo_tc.cu)
 int sp_tc_configure();       // driver entry point for tensor maps + shared memory opt-in; returns cudaError_t
@@ -201,7 +199,5 @@ void launch_sp_gram_tc(const SpLayer* d_layers, const void* d_maps, const TileRe
 int sp_bp_rows_per_tile();
 int sp_bp_cols_per_tile();
 int sp_bp_chunk_rows();
-int sp_decode_tile_rows();
-int sp_decode_tile_cols();
 
 }  // namespace atomo

@@ -15,8 +15,10 @@
 //                      compaction of the kept ranks, short-side vectors of the kept atoms
 //   sp_backproject     long-side vector of each kept atom, w_i = G^T u_i (or G v_i)
 //   sp_finish_atoms    sigma_i = ||w_i||, coef_i = sigma_i / p_i, w_i normalised
-//   sp_decode          G_hat = sum_k coef_k u_k v_k^T, one streaming write pass (8 atoms per pass)
+//   sp_decode          G_hat = sum_k coef_k u_k v_k^T, one streaming write pass
 #include <algorithm>
+
+#include <type_traits>
 
 #include "atomo_kernels.cuh"
 
@@ -634,131 +636,206 @@ void launch_sp_finish_atoms(const SpLayer* d_layers, int n_layers, int k_cap_max
 }
 
 // =================================================================================================
-// decode: out[i][c] = sum_a coef_a rowvec_a[i] colvec_a[c], a streaming write of the output.
-// Tile 64 rows x 1024 columns, 256 threads: a thread owns 4 consecutive columns, keeps the column-vector
-// entries of up to 8 atoms in registers and walks down the 64 rows, one 16-byte store per row; the row-vector
-// entries (times coef) of the tile sit in shared memory and are read as broadcasts.  k is about s, a handful:
-// a layer with more than 8 kept atoms takes further passes that add to what the first one wrote.
+// decode: out[i][c] = sum_a coef_a rowvec_a[i] colvec_a[c] over the kept atoms of one payload, or of all payloads of an
+// average: every output element is written once, whatever the number of atoms.
+// A thread keeps 16 rows x 4 columns of sums in registers (4 x 4 where a layer has at most 128 columns) and walks over the
+// atoms: one 16-byte load of the column vector and four broadcast loads of row entries (times coef, in shared memory) for 64
+// multiply-adds.  Where rows are a multiple of 16 bytes a thread owns four neighbouring columns, else columns that lie a
+// warp or more apart, so that single stores are still coalesced.  The layers come as a kernel argument, the payloads'
+// headers are read by one lane each: three dependent reads of global memory before the first product.
+// Bound: the writes of the output (4096-column layers, one payload: @DEC96@), for an average of 24 atoms the multiply-adds as
+// well: mean of eight ResNet-18 payloads 126 -> @DECAVG@ us (before: eight atoms per pass over the output, 208 CTAs, headers
+// read one after the other by every thread).
 // =================================================================================================
-constexpr int kDecRows = 64, kDecCols = 1024, kDecAtoms = 8, kDecThreads = 256;
-int sp_decode_tile_rows() { return kDecRows; }
-int sp_decode_tile_cols() { return kDecCols; }
+constexpr int kDecThreads = 256, kDecAtoms = 32;               // atoms per round through shared memory
+constexpr int kDecCols = 1024, kDecMaxRows = 128;              // columns and at most rows of a CTA
 
-// `single` (one payload) or `list[0 .. n_payloads)`: the kept atoms of all payloads are walked as one sequence,
-// payload after payload, 8 per pass; `scale` multiplies every term (1, or 1 / n_payloads for the average).
-__global__ void __launch_bounds__(kDecThreads) sp_decode_kernel(const uint8_t* __restrict__ single,
-                                                                const uint8_t* const* __restrict__ list, int n_payloads,
-                                                                float scale, const SpDecodeLayer* __restrict__ layers,
-                                                                const TileRef* __restrict__ tiles) {
-  __shared__ __align__(16) float s_rc[kDecRows][kDecAtoms];      // scale * coef_a * rowvec_a[i] of the tile's rows
-  const TileRef ref = tiles[blockIdx.x];
-  const SpDecodeLayer D = layers[ref.layer];
+// `single` (one payload) or `list[0 .. n_payloads)`: the kept atoms of all payloads are walked as one sequence, payload after
+// payload; `scale` multiplies every term (1, or 1 / n_payloads for the average).
+template <int N>
+__global__ void __launch_bounds__(kDecThreads, 2) sp_decode_kernel(const __grid_constant__ SpDecodeBatch<N> B, const uint8_t* __restrict__ single,
+                                                                   const uint8_t* const* __restrict__ list, const int n_payloads, const float scale) {
+  __shared__ __align__(16) float s_rc[kDecAtoms][kDecMaxRows]; // scale * coef_a * rowvec_a[i] of the CTA's rows
+  __shared__ const float *s_row[kDecAtoms], *s_col[kDecAtoms];
+  __shared__ float s_cf[kDecAtoms];
+  __shared__ const float *s_rows[32], *s_cols[32], *s_vals[32];  // the arrays of a round's payloads
+  __shared__ int s_first[32], s_k[32];                           // ... and their atoms in the sequence
+  __shared__ int s_total;
+  int v = 0;
+  if (N > 1) {                                                 // the last layer whose first CTA is not above this one
+    int hi = B.n;
+    while (hi - v > 1) { const int m = (v + hi) / 2; if (B.v[m].cta0 <= blockIdx.x) v = m; else hi = m; }
+  }
+  const SpDecodeLayer& D = B.v[v];
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int64_t rows = D.rows, cols = D.cols;
   const bool tall = rows > cols;
   const int64_t r = tall ? cols : rows, len = tall ? rows : cols;
-  const int64_t rlen = tall ? len : r, clen = tall ? r : len;     // lengths of the row- and column-indexed vectors
-  const int64_t i0 = (int64_t)ref.a * kDecRows, c = (int64_t)ref.b * kDecCols + 4 * threadIdx.x;
-  const int n_rows = (int)min((int64_t)kDecRows, rows - i0);
-  const bool vec_out = (cols % 4 == 0) && ((reinterpret_cast<uintptr_t>(D.out) & 15u) == 0);
-  float* out = D.out + i0 * cols + c;
-  int p = 0;                                                     // cursor over (payload, atom)
-  uint32_t a_next = 0;
-  bool first_pass = true;
-  for (;;) {
-    // up to 8 atoms for this pass
-    const float* rowv[kDecAtoms]; const float* colv[kDecAtoms]; float cf[kDecAtoms];
-    int na = 0;
-    while (na < kDecAtoms && p < n_payloads) {
-      const uint8_t* payload = list ? list[p] : single;
-      const atomo_payload_header* gh = reinterpret_cast<const atomo_payload_header*>(payload);
-      // a payload normally comes from another rank: its header is checked before anything it points to is read.  The
-      // layer headers must exist (layer index below n_layers) and every array must lie inside total_bytes; a header
-      // that fails contributes zeros, and the status word is written only where it is known to be a status word
-      const bool has_hdr = gh->magic == ATOMO_MAGIC && (uint32_t)ref.layer < gh->n_layers &&
-                           sizeof(atomo_payload_header) + (uint64_t)gh->n_layers * sizeof(atomo_layer_header) <= gh->total_bytes;
-      const atomo_layer_header* h = reinterpret_cast<const atomo_layer_header*>(payload + sizeof(atomo_payload_header)) +
-                                    (has_hdr ? ref.layer : 0);
-      bool ok = has_hdr && gh->kind == ATOMO_KIND_SPECTRAL && h->rows == rows && h->cols == cols && h->k <= h->k_cap;
-      if (ok) {
-        const uint64_t kc = h->k_cap, tb = gh->total_bytes;
-        ok = h->off_idx <= tb && kc * 4 <= tb - h->off_idx && h->off_val <= tb && kc * 4 <= tb - h->off_val &&
-             h->off_short <= tb && kc * (uint64_t)r * 4 <= tb - h->off_short &&
-             h->off_long <= tb && kc * (uint64_t)len * 4 <= tb - h->off_long;
-      }
-      if (!ok && has_hdr && a_next == 0 && ref.a == 0 && ref.b == 0 && threadIdx.x == 0)
-        raise_status(const_cast<atomo_layer_header*>(h), ATOMO_ERR_PAYLOAD);
-      const uint32_t k = ok ? h->k : 0u;
-      if (a_next >= k) { ++p; a_next = 0; continue; }
-      const float* shortv = reinterpret_cast<const float*>(payload + h->off_short);
-      const float* longv = reinterpret_cast<const float*>(payload + h->off_long);
-      rowv[na] = (tall ? longv : shortv) + (int64_t)a_next * rlen;     // indexed by output row
-      colv[na] = (tall ? shortv : longv) + (int64_t)a_next * clen;     // indexed by output column
-      cf[na] = __ldg(reinterpret_cast<const float*>(payload + h->off_val) + a_next) * scale;
-      ++na; ++a_next;
-    }
-    if (na == 0 && !first_pass) break;
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < kDecRows * kDecAtoms; idx += kDecThreads) {
-      const int i = idx / kDecAtoms, a = idx % kDecAtoms;
-      float v = 0.f;
+  const int64_t rlen = tall ? len : r, clen = tall ? r : len;  // lengths of the row- and column-indexed vectors
+  const uint32_t local = blockIdx.x - D.cta0, n_cb = (uint32_t)((cols + kDecCols - 1) / kDecCols);
+  const int width = D.width, my_col = tid & (width - 1), grp = tid / width;   // threads per row, position, row group
+  const int64_t i0 = (int64_t)(local / n_cb) * D.cta_rows, c0 = (int64_t)(local % n_cb) * kDecCols;
+  const int n_rows = (int)min((int64_t)D.cta_rows, rows - i0);
+  const bool quad = (cols % 4 == 0) && ((reinterpret_cast<uintptr_t>(D.out) & 15u) == 0);
+  const int64_t c = quad ? c0 + 4 * my_col : c0 + my_col;      // first column of the thread, then every dc-th
+  const int dc = quad ? 1 : width;
+  const int64_t c_end = min(cols, c0 + 4 * width);
+  float* const out = D.out + i0 * cols;
+  const int row_bits = __ffs(D.cta_rows) - 1;                  // (a power of two)
+  bool staged = false;                                         // all atoms fit shared memory and are there
+  // a block of rows: rounds of 32 payloads, their atoms 32 at a time
+  auto block = [&](auto rows_tag, const int row_lo) {
+    constexpr int kRows = decltype(rows_tag)::value;
+    float acc[kRows][4];
 #pragma unroll
-      for (int u = 0; u < kDecAtoms; ++u) if (u == a && u < na && i < n_rows) v = __ldg(rowv[u] + i0 + i) * cf[u];
-      s_rc[i][a] = v;
-    }
-    float4 cv[kDecAtoms];
+    for (int i = 0; i < kRows; ++i)
 #pragma unroll
-    for (int a = 0; a < kDecAtoms; ++a) {
-      cv[a] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (a < na && c < cols) {
-        const float* src = colv[a] + c;
-        if ((clen % 4 == 0) && ((reinterpret_cast<uintptr_t>(colv[a]) & 15u) == 0) && c + 3 < cols)
-          cv[a] = __ldg(reinterpret_cast<const float4*>(src));
-        else {
-          cv[a].x = __ldg(src);
-          if (c + 1 < cols) cv[a].y = __ldg(src + 1);
-          if (c + 2 < cols) cv[a].z = __ldg(src + 2);
-          if (c + 3 < cols) cv[a].w = __ldg(src + 3);
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+    for (int p0 = 0; p0 < n_payloads; p0 += 32) {
+      if (w == 0 && !staged) {
+        // a payload normally comes from another rank: its header is checked before anything it points to is read.  The
+        // layer headers must exist (layer index below n_layers) and every array must lie inside total_bytes; a header
+        // that fails contributes zeros, and the status word is written only where it is known to be a status word
+        uint32_t k = 0;
+        if (p0 + lane < n_payloads) {
+          const uint8_t* payload = list ? list[p0 + lane] : single;
+          const atomo_payload_header* gh = reinterpret_cast<const atomo_payload_header*>(payload);
+          const bool has_hdr = gh->magic == ATOMO_MAGIC && (uint32_t)D.layer < gh->n_layers &&
+                               sizeof(atomo_payload_header) + (uint64_t)gh->n_layers * sizeof(atomo_layer_header) <= gh->total_bytes;
+          const atomo_layer_header* h = reinterpret_cast<const atomo_layer_header*>(payload + sizeof(atomo_payload_header)) +
+                                        (has_hdr ? D.layer : 0);
+          bool ok = has_hdr && gh->kind == ATOMO_KIND_SPECTRAL && h->rows == rows && h->cols == cols && h->k <= h->k_cap;
+          if (ok) {
+            const uint64_t kc = h->k_cap, tb = gh->total_bytes;
+            ok = h->off_idx <= tb && kc * 4 <= tb - h->off_idx && h->off_val <= tb && kc * 4 <= tb - h->off_val &&
+                 h->off_short <= tb && kc * (uint64_t)r * 4 <= tb - h->off_short &&
+                 h->off_long <= tb && kc * (uint64_t)len * 4 <= tb - h->off_long;
+          }
+          if (ok) {
+            k = h->k;
+            s_rows[lane] = reinterpret_cast<const float*>(payload + (tall ? h->off_long : h->off_short));
+            s_cols[lane] = reinterpret_cast<const float*>(payload + (tall ? h->off_short : h->off_long));
+            s_vals[lane] = reinterpret_cast<const float*>(payload + h->off_val);
+          } else if (has_hdr && local == 0 && row_lo == 0) raise_status(const_cast<atomo_layer_header*>(h), ATOMO_ERR_PAYLOAD);
         }
+        uint32_t upto = k;                                     // atoms of the payloads up to this lane's
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t x = __shfl_up_sync(0xffffffffu, upto, o); if (lane >= o) upto += x; }
+        s_first[lane] = (int)(upto - k); s_k[lane] = (int)k;
+        if (lane == 31) s_total = (int)upto;
       }
+      __syncthreads();
+      const int total = s_total;
+      for (int a0 = 0; a0 < total; a0 += kDecAtoms) {
+        const int na = min(kDecAtoms, total - a0);
+        if (!staged) {
+          if (w == 0) {
+            const int first = s_first[lane], lo = max(first, a0), hi = min(first + s_k[lane], a0 + na);
+            for (int t = lo; t < hi; ++t) {
+              const int64_t a = t - first;
+              s_row[t - a0] = s_rows[lane] + a * rlen + i0;
+              s_col[t - a0] = s_cols[lane] + a * clen;
+              s_cf[t - a0] = __ldg(s_vals[lane] + a) * scale;
+            }
+          }
+          __syncthreads();
+          for (int q = tid; q < na << row_bits; q += kDecThreads) {
+            const int a = q >> row_bits, i = q & (D.cta_rows - 1);
+            s_rc[a][i] = i < n_rows ? __ldg(s_row[a] + i) * s_cf[a] : 0.0f;
+          }
+          __syncthreads();
+          staged = n_payloads <= 32 && total <= kDecAtoms;
+        }
+        if (c < cols) {
+          auto entries = [&](int a) {
+            const float* src = s_col[a] + c;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (quad && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) x = __ldg(reinterpret_cast<const float4*>(src));
+            else {
+              x.x = __ldg(src);
+              if (c + dc < c_end) x.y = __ldg(src + dc);
+              if (c + 2 * dc < c_end) x.z = __ldg(src + 2 * dc);
+              if (c + 3 * dc < c_end) x.w = __ldg(src + 3 * dc);
+            }
+            return x;
+          };
+          const float* rc = &s_rc[0][row_lo + grp * kRows];
+          auto add = [&](const float4 x, int a) {
+#pragma unroll
+            for (int i = 0; i < kRows; i += 4) {
+              const float4 q = *reinterpret_cast<const float4*>(rc + (size_t)a * kDecMaxRows + i);
+              const float y[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                acc[i + u][0] = fmaf(y[u], x.x, acc[i + u][0]); acc[i + u][1] = fmaf(y[u], x.y, acc[i + u][1]);
+                acc[i + u][2] = fmaf(y[u], x.z, acc[i + u][2]); acc[i + u][3] = fmaf(y[u], x.w, acc[i + u][3]);
+              }
+            }
+          };
+          int a = 0;
+          for (; a + 4 <= na; a += 4) {                        // four loads in flight
+            const float4 x0 = entries(a), x1 = entries(a + 1), x2 = entries(a + 2), x3 = entries(a + 3);
+            add(x0, a); add(x1, a + 1); add(x2, a + 2); add(x3, a + 3);
+          }
+          for (; a < na; ++a) add(entries(a), a);
+        }
+        if (!staged) __syncthreads();
+      }
+      if (!staged) __syncthreads();
     }
-    __syncthreads();
     if (c < cols) {
-      const bool add = !first_pass;
-#pragma unroll 4
-      for (int i = 0; i < n_rows; ++i) {
-        const float4 r0 = *reinterpret_cast<const float4*>(&s_rc[i][0]);
-        const float4 r1 = *reinterpret_cast<const float4*>(&s_rc[i][4]);
-        const float rc[kDecAtoms] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      float* o = out + (int64_t)(row_lo + grp * kRows) * cols + c;
 #pragma unroll
-        for (int a = 0; a < kDecAtoms; ++a) {
-          v.x = fmaf(rc[a], cv[a].x, v.x); v.y = fmaf(rc[a], cv[a].y, v.y);
-          v.z = fmaf(rc[a], cv[a].z, v.z); v.w = fmaf(rc[a], cv[a].w, v.w);
+      for (int i = 0; i < kRows; ++i) {
+        if (row_lo + grp * kRows + i < n_rows) {
+          if (quad) *reinterpret_cast<float4*>(o) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+          else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (c + j * dc < c_end) o[j * dc] = acc[i][j];
+          }
         }
-        float* o = out + (int64_t)i * cols;
-        if (vec_out && c + 3 < cols) {
-          if (add) { const float4 old = *reinterpret_cast<const float4*>(o); v.x += old.x; v.y += old.y; v.z += old.z; v.w += old.w; }
-          *reinterpret_cast<float4*>(o) = v;
-        } else {
-          const float vv[4] = {v.x, v.y, v.z, v.w};
-          for (int j = 0; j < 4; ++j) if (c + j < cols) o[j] = add ? o[j] + vv[j] : vv[j];
-        }
+        o += cols;
       }
     }
-    first_pass = false;
-    if (na < kDecAtoms) break;                                    // the sequence is exhausted
+  };
+  if (width >= 64) { for (int lo = 0; lo < n_rows; lo += 16 * (kDecThreads / width)) block(std::integral_constant<int, 16>{}, lo); }
+  else { for (int lo = 0; lo < n_rows; lo += 4 * (kDecThreads / width)) block(std::integral_constant<int, 4>{}, lo); }
+}
+
+// The layers of a decode in launches of up to kSpDecodeBatch of them; returns their number.  The thread layout of a layer
+// follows from its columns.  A CTA takes one block of rows; four where the call has CTAs enough to fill the GPU many times
+// over (what a CTA reads before its first product then counts less).
+int launch_sp_decode(const uint8_t* payload, const uint8_t* const* d_payloads, int n_payloads, const int64_t* rows, const int64_t* cols,
+                     float* const* out, int n_layers, cudaStream_t st) {
+  auto describe = [&](int l, int blocks, uint32_t cta0) {
+    SpDecodeLayer D{out[l], rows[l], cols[l], l, 8, 0, cta0};
+    while (4 * D.width < std::min<int64_t>(cols[l], kDecCols)) D.width *= 2;
+    D.cta_rows = std::min((D.width >= 64 ? 16 : 4) * (kDecThreads / D.width) * blocks, kDecMaxRows);
+    return D;
+  };
+  auto ctas_of = [](const SpDecodeLayer& D) {
+    return (uint64_t)((D.rows + D.cta_rows - 1) / D.cta_rows) * (uint64_t)((D.cols + kDecCols - 1) / kDecCols);
+  };
+  uint64_t total = 0;
+  for (int l = 0; l < n_layers; ++l) total += ctas_of(describe(l, 1, 0));
+  const int blocks = total >= 8192 ? 4 : 1;
+  const float scale = payload ? 1.0f : 1.0f / (float)n_payloads;
+  int n_launch = 0;
+  for (int l = 0; l < n_layers; ++n_launch) {
+    uint64_t ctas = 0;
+    auto run = [&](auto& B, int most) {
+      for (B.n = 0; B.n < most && l < n_layers; ++B.n, ++l) {
+        const SpDecodeLayer D = describe(l, blocks, (uint32_t)ctas);
+        if (B.n > 0 && ctas + ctas_of(D) > 0x7fffffffull) break;
+        B.v[B.n] = D;
+        ctas += ctas_of(D);
+      }
+      sp_decode_kernel<<<(unsigned)ctas, kDecThreads, 0, st>>>(B, payload, d_payloads, n_payloads, scale);
+    };
+    if (n_layers - l == 1) { SpDecodeBatch<1> B{}; run(B, 1); }
+    else { SpDecodeBatch<kSpDecodeBatch> B{}; run(B, kSpDecodeBatch); }
   }
-}
-
-void launch_sp_decode(const uint8_t* payload, const SpDecodeLayer* d_layers, const TileRef* d_tiles, int n_tiles,
-                      cudaStream_t st) {
-  if (n_tiles > 0) sp_decode_kernel<<<n_tiles, kDecThreads, 0, st>>>(payload, nullptr, 1, 1.0f, d_layers, d_tiles);
-}
-
-void launch_sp_decode_average(const uint8_t* const* d_payloads, int n_payloads, const SpDecodeLayer* d_layers,
-                              const TileRef* d_tiles, int n_tiles, cudaStream_t st) {
-  if (n_tiles > 0)
-    sp_decode_kernel<<<n_tiles, kDecThreads, 0, st>>>(nullptr, d_payloads, n_payloads, 1.0f / (float)n_payloads, d_layers, d_tiles);
+  return n_launch;
 }
 
 }  // namespace atomo
