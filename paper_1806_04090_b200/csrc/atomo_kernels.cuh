@@ -119,7 +119,7 @@ struct SpLayer {
 
 // a layer of a spectral decode: threads per output row, rows per CTA, the layer's first CTA
 struct SpDecodeLayer { float* out; int64_t rows, cols; int32_t layer, width, cta_rows; uint32_t cta0; };
-constexpr int kSpDecodeBatch = 64;
+constexpr int kSpDecodeBatch = 128;
 template <int N> struct SpDecodeBatch { SpDecodeLayer v[N]; int n; };
 
 struct TileRef { int32_t layer, a, b, c; };

@@ -643,8 +643,8 @@ void launch_sp_finish_atoms(const SpLayer* d_layers, int n_layers, int k_cap_max
 // multiply-adds.  Where rows are a multiple of 16 bytes a thread owns four neighbouring columns, else columns that lie a
 // warp or more apart, so that single stores are still coalesced.  The layers come as a kernel argument, the payloads'
 // headers are read by one lane each: three dependent reads of global memory before the first product.
-// Bound: the writes of the output (4096-column layers, one payload: @DEC96@), for an average of 24 atoms the multiply-adds as
-// well: mean of eight ResNet-18 payloads 126 -> @DECAVG@ us (before: eight atoms per pass over the output, 208 CTAs, headers
+// Bound: the writes of the output (96 layers of 1024 x 4096, one payload: 340 us, 4.7 TB/s), for an average of 24 atoms the multiply-adds as
+// well: mean of eight ResNet-18 payloads 126 -> 42 us (before: eight atoms per pass over the output, 208 CTAs, headers
 // read one after the other by every thread).
 // =================================================================================================
 constexpr int kDecThreads = 256, kDecAtoms = 32;               // atoms per round through shared memory
@@ -833,6 +833,7 @@ int launch_sp_decode(const uint8_t* payload, const uint8_t* const* d_payloads, i
       sp_decode_kernel<<<(unsigned)ctas, kDecThreads, 0, st>>>(B, payload, d_payloads, n_payloads, scale);
     };
     if (n_layers - l == 1) { SpDecodeBatch<1> B{}; run(B, 1); }
+    else if (n_layers - l <= 24) { SpDecodeBatch<24> B{}; run(B, 24); }   // (a kilobyte of arguments)
     else { SpDecodeBatch<kSpDecodeBatch> B{}; run(B, kSpDecodeBatch); }
   }
   return n_launch;
