@@ -749,10 +749,10 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);
       {
         const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
-        d.bd_U = A.take<float>(on * rows * kBandWidth); d.bd_W = A.take<float>(on * rows * kBandWidth);
+        d.bd_UW = A.take<float>(on * rows * 2 * kBandWidth);
         d.bd_X = A.take<float>(on * rows * kBandWidth);
         d.bd_part = A.take<double>(on * sp_band_parts(band_form) * rows * kBandWidth);
-        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<long long>(on * sp_band_strips(d.r) * kBandWidth * kBandWidth);
+        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<long long>(on * 3 * kBandWidth * kBandWidth);
         d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
         d.bd_V2 = A.take<float>(on * d.r * sp_band_steps(d.r) * kBandWidth);

@@ -54,6 +54,8 @@ static_assert(kBw == 8, "the operand vectors are two float4");
 // barriers overlap with the other's pass.
 namespace {
 
+constexpr int kGroup = 4;                     // columns that travel together through a warp's ring
+constexpr int kGroupFloats = kGroup * (kStrip + 16);
 constexpr double kFix = 1125899906842624.0;   // 2^50: U^T A U in fixed point (|entries| <= 1)
 
 struct BandShared {
@@ -193,9 +195,9 @@ __device__ __noinline__ void band_small_qr(BandShared& sh, const int n_ref, cons
 }  // namespace
 
 // A CTA of THREADS threads, MINB per SM
-template <int THREADS, int MINB, int PARTS>
+template <int THREADS, int MINB, int PARTS, int STAGES>
 __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* __restrict__ layers, const ClusterCta* __restrict__ ctas,
-                                                                const int cap, uint32_t* __restrict__ timeout_flag) {
+                                                                uint32_t* __restrict__ timeout_flag) {
   constexpr int kWarps = THREADS / 32;
   extern __shared__ __align__(16) float band_smem[];
   __shared__ BandShared sh;
@@ -205,13 +207,14 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   const int r = L.r, g = me.slot, G = me.pad;
   const int n_strips = (r + kStrip - 1) / kStrip;
   float* const A = L.A; const int64_t lda = L.lda;           // lda is a multiple of the strip: whole strips may be read and written
-  float* const gU = L.bd_U; float* const gW = L.bd_W; float* const gX = L.bd_X;
+  float* const gUW = L.bd_UW; float* const gX = L.bd_X;
   double* const gPart = L.bd_part; double* const gP = L.bd_P; long long* const gS = L.bd_S; double* const gB = L.bd_band;
   double* const gG = L.bd_G; double* const gM = L.bd_M;
   float* const gV = L.td_V; const int64_t ldv = L.td_ldv;
   float* const s_u = band_smem;                              // [r][8] this panel's U, by row
-  float* const s_ops = band_smem + (size_t)r * 8;            // [cap][16] U and W of the panel before, columns col0 ..
+  float* const s_ring = band_smem + (size_t)(r + kGroup) * 8; // [warps][STAGES] groups of columns on their way
   if (tid == 0) sh.fail = 0u;
+  if (tid < kGroup * 8) s_u[(size_t)r * 8 + tid] = 0.0f;     // rows past the end, of a last group that is not full
   uint32_t arrivals = 0;
   for (int c = 0; c < r; c += kBw) {
     // ---- own rows: U and W of the panel before out, entries of this panel (columns c .. c+7) and the Gram matrix of those
@@ -252,8 +255,8 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
           }
 #pragma unroll
           for (int t = 0; t < 8; ++t) x[t] = in && c + t < r ? (float)z[t] : 0.0f;
-          float4* du = reinterpret_cast<float4*>(gU + (int64_t)i * 8);
-          float4* dw = reinterpret_cast<float4*>(gW + (int64_t)i * 8);
+          float4* du = reinterpret_cast<float4*>(gUW + (int64_t)i * 16);
+          float4* dw = du + 2;
           du[0] = make_float4(uu[0], uu[1], uu[2], uu[3]); du[1] = make_float4(uu[4], uu[5], uu[6], uu[7]);
           dw[0] = make_float4(ww[0], ww[1], ww[2], ww[3]); dw[1] = make_float4(ww[4], ww[5], ww[6], ww[7]);
         }
@@ -264,6 +267,10 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         band_gram32(lo, hi, gG + (int64_t)half * 36, lane);
       }
     }
+    // U^T A U is added up in one of three sets of 64 words in turn; the next panel's is cleared here: its last readers are
+    // past the barrier before this one, its adders wait for the one after it
+    long long* const s_sum = gS + c / kBw % 3 * 64;
+    if (g == 0 && tid < 64) { gS[(c / kBw + 1) % 3 * 64 + tid] = 0; if (c == 0) s_sum[tid] = 0; }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
     if (sh.fail) break;
@@ -313,63 +320,70 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
     const int s0 = first_strip + ((g - first_strip % G) % G + G) % G;      // first active strip of this CTA
     const int n_own = s0 < n_strips ? (n_strips - 1 - s0) / G + 1 : 0;
     // ---- pass over the own strips ----
-    const int per = ((m + PARTS - 1) / PARTS + 3) & ~3;      // columns per task, a multiple of 4
-    for (int col0 = row0; col0 < r; col0 += cap) {
-      const int col1 = min(r, col0 + cap);
+    const int per = ((m + PARTS - 1) / PARTS + 3) & ~3;      // columns per task, a multiple of the group
+    __syncthreads();
+    // tasks (strip, part), dealt to the warps
+    for (int task = w; task < n_own * PARTS; task += kWarps) {
+      const int s = s0 + task / PARTS * G, part = task % PARTS;
+      const int jb = row0 + part * per, je = min(jb + per, r);
+      const int i = s * kStrip + 2 * lane;
+      double* const dst = gPart + ((int64_t)part * n_strips * kStrip + i) * 8;
+      if (jb >= je) {                                        // an empty part
+#pragma unroll
+        for (int t = 0; t < 16; t += 2) *reinterpret_cast<double2*>(dst + t) = make_double2(0.0, 0.0);
+        continue;
+      }
+      // a group of four columns: 64 entries of A each (16 bytes per lane, half a warp per column), then their U and W
+      const int groups = (je - jb + kGroup - 1) / kGroup;
+      float* const ring = s_ring + (size_t)w * STAGES * kGroupFloats;
+      const float* src = A + (int64_t)(jb + lane / 16) * lda + s * kStrip + (lane & 15) * 4;
+      const float* src_uw = gUW + (int64_t)jb * 16 + lane * 4;
+      auto issue = [&](int q) {
+        if (q < groups) {
+          const uint32_t d = (uint32_t)__cvta_generic_to_shared(ring + (q % STAGES) * kGroupFloats + lane * 4);
+          const int j = jb + q * kGroup;
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(j + lane / 16 < je ? src : A), "r"(j + lane / 16 < je ? 16 : 0) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 512), "l"(j + 2 + lane / 16 < je ? src + 2 * lda : A),
+                       "r"(j + 2 + lane / 16 < je ? 16 : 0) : "memory");
+          if (!first && lane < 16)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 1024), "l"(j + lane / 4 < je ? src_uw : gUW), "r"(j + lane / 4 < je ? 16 : 0) : "memory");
+          src += (int64_t)kGroup * lda; src_uw += kGroup * 16;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory"); // one group per call, empty or not: the counting stays uniform
+      };
+#pragma unroll
+      for (int q = 0; q < STAGES - 1; ++q) issue(q);
+      float up0[8], wp0[8], up1[8], wp1[8];
+      double p0[8], p1[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) { up0[t] = wp0[t] = up1[t] = wp1[t] = 0.0f; p0[t] = p1[t] = 0.0; }
       if (!first) {
-        if (col0 > row0) __syncthreads();                    // the block before has been used
-        for (int q = tid; q < (col1 - col0) * 4; q += THREADS) {
-          const int j = col0 + q / 4, h = q % 4;
-          const float4* src = reinterpret_cast<const float4*>((h < 2 ? gU : gW) + (int64_t)j * 8) + (h & 1);
-          reinterpret_cast<float4*>(s_ops)[(size_t)(j - col0) * 4 + h] = __ldcg(src);
+        const float4* own = reinterpret_cast<const float4*>(gUW + (int64_t)i * 16);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 a = __ldcg(own + h), b = __ldcg(own + 2 + h), d = __ldcg(own + 4 + h), e = __ldcg(own + 6 + h);
+          up0[4 * h] = -a.x; up0[4 * h + 1] = -a.y; up0[4 * h + 2] = -a.z; up0[4 * h + 3] = -a.w;
+          wp0[4 * h] = -b.x; wp0[4 * h + 1] = -b.y; wp0[4 * h + 2] = -b.z; wp0[4 * h + 3] = -b.w;
+          up1[4 * h] = -d.x; up1[4 * h + 1] = -d.y; up1[4 * h + 2] = -d.z; up1[4 * h + 3] = -d.w;
+          wp1[4 * h] = -e.x; wp1[4 * h + 1] = -e.y; wp1[4 * h + 2] = -e.z; wp1[4 * h + 3] = -e.w;
         }
       }
-      __syncthreads();
-      // tasks (strip, part), dealt to the warps
-      for (int task = w; task < n_own * PARTS; task += kWarps) {
-        const int s = s0 + task / PARTS * G, part = task % PARTS;
-        const int p_lo = row0 + part * per;
-        const int jb = max(p_lo, col0), je = min(min(p_lo + per, r), col1);
-        const int i = s * kStrip + 2 * lane;
-        double* const dst = gPart + ((int64_t)part * n_strips * kStrip + i) * 8;
-        if (jb >= je) {
-          if (p_lo >= r && col0 == row0) {                   // an empty part
+      float q0[8], q1[8];                                    // fp32 runs of up to 32 columns
 #pragma unroll
-            for (int t = 0; t < 16; t += 2) *reinterpret_cast<double2*>(dst + t) = make_double2(0.0, 0.0);
-          }
-          continue;
-        }
-        float up0[8], wp0[8], up1[8], wp1[8];
-        double p0[8], p1[8];
+      for (int t = 0; t < 8; ++t) q0[t] = q1[t] = 0.0f;
+      float* ap = A + (int64_t)jb * lda + i;
+      const float4* un = reinterpret_cast<const float4*>(s_u) + (size_t)jb * 2;
+      int left = je - jb;
+      for (int q = 0; q < groups; ++q, left -= kGroup) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncwarp();                                        // group q has landed for the warp; the stage of group q - 1 is free
+        issue(q + STAGES - 1);
+        const float* const st = ring + (q % STAGES) * kGroupFloats;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) { up0[t] = wp0[t] = up1[t] = wp1[t] = 0.0f; p0[t] = p1[t] = 0.0; }
-        if (!first) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float4 a = __ldcg(reinterpret_cast<const float4*>(gU + (int64_t)i * 8) + h), b = __ldcg(reinterpret_cast<const float4*>(gW + (int64_t)i * 8) + h);
-            const float4 d = __ldcg(reinterpret_cast<const float4*>(gU + (int64_t)i * 8 + 8) + h), e = __ldcg(reinterpret_cast<const float4*>(gW + (int64_t)i * 8 + 8) + h);
-            up0[4 * h] = -a.x; up0[4 * h + 1] = -a.y; up0[4 * h + 2] = -a.z; up0[4 * h + 3] = -a.w;
-            wp0[4 * h] = -b.x; wp0[4 * h + 1] = -b.y; wp0[4 * h + 2] = -b.z; wp0[4 * h + 3] = -b.w;
-            up1[4 * h] = -d.x; up1[4 * h + 1] = -d.y; up1[4 * h + 2] = -d.z; up1[4 * h + 3] = -d.w;
-            wp1[4 * h] = -e.x; wp1[4 * h + 1] = -e.y; wp1[4 * h + 2] = -e.z; wp1[4 * h + 3] = -e.w;
-          }
-        }
-        if (jb > p_lo) {                                     // the part began in an earlier block of columns
-#pragma unroll
-          for (int t = 0; t < 8; t += 2) {
-            const double2 a = *reinterpret_cast<const double2*>(dst + t), b = *reinterpret_cast<const double2*>(dst + 8 + t);
-            p0[t] = a.x; p0[t + 1] = a.y; p1[t] = b.x; p1[t + 1] = b.y;
-          }
-        }
-        float q0[8], q1[8];                                  // fp32 runs of up to 32 columns
-#pragma unroll
-        for (int t = 0; t < 8; ++t) q0[t] = q1[t] = 0.0f;
-        float* ap = A + (int64_t)jb * lda + i;
-        const float4* ops = reinterpret_cast<const float4*>(s_ops) + (size_t)(jb - col0) * 4;
-        const float4* un = reinterpret_cast<const float4*>(s_u) + (size_t)jb * 2;
-        // one column: update, store, product
-        auto column = [&](float2 v, const float4* o, const float4* n, float* p) {
+        for (int u = 0; u < kGroup; ++u) {                   // one column: update, store, product
+          float2 v = *reinterpret_cast<const float2*>(st + u * kStrip + 2 * lane);
           if (!first) {
+            const float4* o = reinterpret_cast<const float4*>(st + kGroup * kStrip + u * 16);
             const float4 cu0 = o[0], cu1 = o[1], cw0 = o[2], cw1 = o[3];
             const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
             const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
@@ -378,49 +392,24 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
               v.x = fmaf(up0[t], cw[t], v.x); v.y = fmaf(up1[t], cw[t], v.y);
               v.x = fmaf(wp0[t], cu[t], v.x); v.y = fmaf(wp1[t], cu[t], v.y);
             }
-            *reinterpret_cast<float2*>(p) = v;
+            if (u < left) *reinterpret_cast<float2*>(ap + (int64_t)u * lda) = v;
           }
-          const float4 n0 = n[0], n1 = n[1];
+          const float4 n0 = un[2 * u], n1 = un[2 * u + 1];
           const float cn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
 #pragma unroll
           for (int t = 0; t < 8; ++t) { q0[t] = fmaf(v.x, cn[t], q0[t]); q1[t] = fmaf(v.y, cn[t], q1[t]); }
-        };
-        // groups of four columns, the next group's entries on their way; further ahead a prefetch asks the L2 for 16 columns
-        // at a time (two 128-byte lines each), so that a load waits for the L2 and not for DRAM
-        constexpr int kU = 4;
-        float2 a[kU];
-        const int whole = (je - jb) / kU;
-        const float* pre = A + (int64_t)(jb + lane / 2) * lda + s * kStrip + (lane & 1) * 32;
-        auto ask = [&](int j) { if (j + lane / 2 < je) asm volatile("prefetch.global.L2 [%0];" ::"l"(pre)); pre += (int64_t)16 * lda; };
-        ask(jb); ask(jb + 16);
-        if (whole > 0) {
-#pragma unroll
-          for (int u = 0; u < kU; ++u) a[u] = *reinterpret_cast<const float2*>(ap + (int64_t)u * lda);
         }
-        for (int q = 0; q < whole; ++q) {
-          float2 b[kU];
-          const float* nx = ap + (int64_t)kU * lda;
-          if (q + 1 < whole) {
+        if ((q & 7) == 7) {
 #pragma unroll
-            for (int u = 0; u < kU; ++u) b[u] = *reinterpret_cast<const float2*>(nx + (int64_t)u * lda);
-          }
-          if ((q & 3) == 0) ask(jb + 4 * q + 32);
-#pragma unroll
-          for (int u = 0; u < kU; ++u) column(a[u], ops + 4 * u, un + 2 * u, ap + (int64_t)u * lda);
-          if ((q & 7) == 7) {
-#pragma unroll
-            for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; q0[t] = q1[t] = 0.0f; }
-          }
-#pragma unroll
-          for (int u = 0; u < kU; ++u) a[u] = b[u];
-          ops += 4 * kU; un += 2 * kU; ap += (int64_t)kU * lda;
+          for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; q0[t] = q1[t] = 0.0f; }
         }
-        for (int j = jb + whole * kU; j < je; ++j, ops += 4, un += 2, ap += lda) column(*reinterpret_cast<const float2*>(ap), ops, un, ap);
+        un += 2 * kGroup; ap += (int64_t)kGroup * lda;
+      }
+      __syncwarp();                                          // the ring is free for the warp's next task
 #pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-          *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t] + (double)q0[t], p0[t + 1] + (double)q0[t + 1]);
-          *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t] + (double)q1[t], p1[t + 1] + (double)q1[t + 1]);
-        }
+      for (int t = 0; t < 8; t += 2) {
+        *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t] + (double)q0[t], p0[t + 1] + (double)q0[t + 1]);
+        *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t] + (double)q1[t], p1[t + 1] + (double)q1[t + 1]);
       }
     }
     __syncthreads();
@@ -449,7 +438,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       }
 #pragma unroll
       for (int a = 0; a < 8; ++a) { acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 8); acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 16); }
-      long long* const part_s = reinterpret_cast<long long*>(s_ops);       // [warp][64]: the operands have been used
+      long long* const part_s = reinterpret_cast<long long*>(s_ring);      // [warp][64]: the ring is empty
       if (lane < 8) {
 #pragma unroll
         for (int a = 0; a < 8; ++a) part_s[w * 64 + a * 8 + lane] = acc[a];
@@ -466,7 +455,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         long long t = 0;
 #pragma unroll
         for (int ww = 0; ww < kWarps; ++ww) t += part_s[ww * 64 + tid];
-        gS[(int64_t)g * 64 + tid] = t;
+        atomicAdd(reinterpret_cast<unsigned long long*>(s_sum) + tid, (unsigned long long)t);
       }
     }
     arrivals += (uint32_t)G;
@@ -474,10 +463,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
     // ---- T, T^T S T, W of the next panel's pivot rows (every CTA) ----
     if (tid >= THREADS - 64) {
       const int q = tid - (THREADS - 64);
-      long long t = 0;
-#pragma unroll 4
-      for (int s = 0; s < G; ++s) t += __ldcg(gS + (int64_t)s * 64 + q);
-      sh.S[q / 8][q % 8] = (double)t * (1.0 / kFix);
+      sh.S[q / 8][q % 8] = (double)__ldcg(s_sum + q) * (1.0 / kFix);
     }
     band_sum36<THREADS>(gM, 2 * first_strip, 2 * n_strips, sh.sum, sh.M);
     __syncthreads();
@@ -670,15 +656,14 @@ int band_sms() {
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms;
 }
-// The instances of the band kernel.  Many layers up to 1024 rows: two small CTAs per SM (96 KB: U of the panel, all columns' U
-// and W of the panel before).  Few layers, or larger ones: one CTA of sixteen warps per SM, a strip each, its columns split
-// over the warps; the operands of 1024 columns at a time.
-struct BandForm { int max_r, threads, per_sm, cap, parts; const void* fn; };
+// The instances of the band kernel.  Many layers up to 1024 rows: two small CTAs per SM.  Few layers, or larger ones: one CTA of
+// sixteen warps per SM, a strip each, its columns split over the warps.  Shared memory: U of the panel and the warps' rings.
+struct BandForm { int max_r, threads, per_sm, parts, stages; const void* fn; };
 const BandForm kBandForms[] = {
-    {1024, 256, 2, 1024, 4, (const void*)sp_band_kernel<256, 2, 4>},
-    {4096, 512, 1, 1024, 16, (const void*)sp_band_kernel<512, 1, 16>},
+    {1024, 256, 2, 4, 6, (const void*)sp_band_kernel<256, 2, 4, 6>},
+    {4096, 512, 1, 16, 4, (const void*)sp_band_kernel<512, 1, 16, 4>},
 };
-size_t band_smem(const BandForm& f, int r_max) { return ((size_t)r_max * 8 + (size_t)std::min(f.cap, r_max) * 16) * sizeof(float); }
+size_t band_smem(const BandForm& f, int r_max) { return ((size_t)(r_max + kGroup) * 8 + (size_t)f.threads / 32 * f.stages * kGroupFloats) * sizeof(float); }
 template <int C, int COLS> int chase_configure() {
   auto* fn = sp_chase_kernel<C, COLS>;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ChForm<C, COLS>::kSmem) != cudaSuccess) return 1;
@@ -715,8 +700,7 @@ int sp_configure_band() {
 
 int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int form, int r_max, uint32_t* d_timeout, cudaStream_t st) {
   const BandForm& f = kBandForms[form];
-  int cap = std::min(f.cap, r_max);
-  void* args[] = {&d_layers, &d_ctas, &cap, &d_timeout};
+  void* args[] = {&d_layers, &d_ctas, &d_timeout};
   return (int)cudaLaunchCooperativeKernel(f.fn, dim3((unsigned)n_ctas), dim3(f.threads), args, band_smem(f, r_max), st);
 }
 
