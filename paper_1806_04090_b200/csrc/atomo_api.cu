@@ -660,12 +660,14 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         ++n;
       }
       if (n == 0) { tri_form = false; break; }
+      // (a strip's columns are dealt to CTAs as well: four warps' worth of a strip are enough for one)
+      const int band_spread = std::max(1, sp_band_parts(band_form) / 4);
       std::vector<int> g(n);
       int total = 0;
       for (size_t q = 0; q < n; ++q) {
         const double rr = L[big_layers[i + q]].r;
         const int strips = sp_band_strips(L[big_layers[i + q]].r);
-        g[q] = fixed > 0 ? std::min(fixed, strips) : std::max(1, std::min(strips, (int)(room * (rr * rr * rr / work))));
+        g[q] = fixed > 0 ? std::min(fixed, strips) : std::max(1, std::min(strips * band_spread, (int)(room * (rr * rr * rr / work))));
         total += g[q];
       }
       for (size_t q = n; total > room; q = q > 1 ? q - 1 : n) if (g[q - 1] > 1) { --g[q - 1]; --total; }   // the minimum of one each went over
@@ -752,7 +754,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.bd_UW = A.take<float>(on * rows * 2 * kBandWidth);
         d.bd_X = A.take<float>(on * rows * kBandWidth);
         d.bd_part = A.take<double>(on * sp_band_parts(band_form) * rows * kBandWidth);
-        d.bd_P = A.take<double>(on * rows * kBandWidth); d.bd_S = A.take<long long>(on * 3 * kBandWidth * kBandWidth);
+        d.bd_S = A.take<double>(on * 3 * kBandWidth * kBandWidth);
         d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
         d.bd_V2 = A.take<float>(on * d.r * sp_band_steps(d.r) * kBandWidth);

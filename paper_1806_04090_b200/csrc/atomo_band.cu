@@ -56,14 +56,17 @@ namespace {
 
 constexpr int kGroup = 4;                     // columns that travel together through a warp's ring
 constexpr int kGroupFloats = kGroup * (kStrip + 16);
-constexpr double kFix = 1125899906842624.0;   // 2^50: U^T A U in fixed point (|entries| <= 1)
+// U^T A U is rounded to multiples of 2^-50 (the last place of 4 .. 8) as it is added up: sums below 8 are then exact in any order.
+// (A has trace one at most and U unit columns, so that no partial sum passes one.)
+constexpr double kFix = 6.0;
 
 struct BandShared {
   double T[8][8], S[8][8], Y[8][8], X[8][8];
   double K[8][8], vtop[8][8];     // K scaled to unit vectors; the reflectors' entries in the panel's first eight rows
   double M[36], G[36], sum[16][36];
+  double s_part[16][64];          // the warps' parts of U^T A U
   double top[8][8];
-  double Wc[8][8], Uc[8][8];      // W and U of the next panel's pivot rows
+  double Wc[8][8], Uc[8][8], Pc[8][8];   // W, U and A U of the next panel's pivot rows
   uint32_t fail;
 };
 
@@ -208,7 +211,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   const int n_strips = (r + kStrip - 1) / kStrip;
   float* const A = L.A; const int64_t lda = L.lda;           // lda is a multiple of the strip: whole strips may be read and written
   float* const gUW = L.bd_UW; float* const gX = L.bd_X;
-  double* const gPart = L.bd_part; double* const gP = L.bd_P; long long* const gS = L.bd_S; double* const gB = L.bd_band;
+  double* const gPart = L.bd_part; double* const gS = L.bd_S; double* const gB = L.bd_band;
   double* const gG = L.bd_G; double* const gM = L.bd_M;
   float* const gV = L.td_V; const int64_t ldv = L.td_ldv;
   float* const s_u = band_smem;                              // [r][8] this panel's U, by row
@@ -216,14 +219,12 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   if (tid == 0) sh.fail = 0u;
   if (tid < kGroup * 8) s_u[(size_t)r * 8 + tid] = 0.0f;     // rows past the end, of a last group that is not full
   uint32_t arrivals = 0;
+  auto own_from = [&](int row) { const int h = row / 32; return h + ((g - h % G) % G + G) % G; };   // this CTA's first half strip, then every G-th
   for (int c = 0; c < r; c += kBw) {
     // ---- own rows: U and W of the panel before out, entries of this panel (columns c .. c+7) and the Gram matrix of those
     // below the band; half a strip per warp ----
     {
-      const int s_lo = c / kStrip, s_own = s_lo + ((g - s_lo % G) % G + G) % G;
-      for (int n = w;; n += kWarps) {
-        const int half = 2 * (s_own + n / 2 * G) + (n & 1);
-        if (half >= 2 * n_strips) break;
+      for (int half = own_from(c) + w * G; half < 2 * n_strips; half += kWarps * G) {
         const int i = half * 32 + lane;
         const bool in = i >= c && i < r;
         float x[8];
@@ -231,10 +232,15 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         for (int t = 0; t < 8; ++t) x[t] = in && c + t < r ? __ldcg(A + (int64_t)(c + t) * lda + i) : 0.0f;
         if (c > 0) {
           float uu[8], ww[8];
-          double p[8];
-          const double2* src = reinterpret_cast<const double2*>(gP + (int64_t)i * 8);
+          double p[8];                                       // the product A U: the parts added in order
 #pragma unroll
-          for (int t = 0; t < 4; ++t) { const double2 d = in ? src[t] : make_double2(0.0, 0.0); p[2 * t] = d.x; p[2 * t + 1] = d.y; }
+          for (int t = 0; t < 8; ++t) p[t] = 0.0;
+          const double2* src = reinterpret_cast<const double2*>(gPart + (int64_t)i * 8);
+#pragma unroll 4
+          for (int part = 0; part < PARTS; ++part, src += (int64_t)n_strips * kStrip * 4) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) { const double2 d = in ? __ldcg(src + t) : make_double2(0.0, 0.0); p[2 * t] += d.x; p[2 * t + 1] += d.y; }
+          }
 #pragma unroll
           for (int t = 0; t < 8; ++t) uu[t] = in ? s_u[(size_t)i * 8 + t] : 0.0f;
           double z[8];                                       // W[i][t] = sum_s P[i][s] T[s][t] - 1/2 sum_s U[i][s] (T^T S T)[s][t]
@@ -269,14 +275,14 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
     }
     // U^T A U is added up in one of three sets of 64 words in turn; the next panel's is cleared here: its last readers are
     // past the barrier before this one, its adders wait for the one after it
-    long long* const s_sum = gS + c / kBw % 3 * 64;
-    if (g == 0 && tid < 64) { gS[(c / kBw + 1) % 3 * 64 + tid] = 0; if (c == 0) s_sum[tid] = 0; }
+    double* const s_sum = gS + c / kBw % 3 * 64;
+    if (g == 0 && tid < 64) { gS[(c / kBw + 1) % 3 * 64 + tid] = 0.0; if (c == 0) s_sum[tid] = 0.0; }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
     if (sh.fail) break;
     const int row0 = c + kBw;                                // first row below the band of the panel
     const int m = r - row0;                                  // panel rows
-    const int c_strip = c / kStrip, first_strip = row0 / kStrip;
+    const int first_strip = row0 / kStrip;
     // ---- diagonal block, QR of the panel (every CTA) ----
     if (g == 0 && tid < kBw * kBw) {
       const int a = tid / kBw, b = tid % kBw;                // entry (c + a, c + b), a >= b
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       const int q = tid - (THREADS - 64), a = q / 8, b = q % 8;
       sh.top[a][b] = row0 + a < r ? (double)__ldcg(gX + (int64_t)(row0 + a) * 8 + b) : 0.0;
     }
-    band_sum36<THREADS>(gG, 2 * c_strip, 2 * n_strips, sh.sum, sh.G);
+    band_sum36<THREADS>(gG, c / 32, 2 * n_strips, sh.sum, sh.G);
     __syncthreads();
     const int n_ref = min(kBw, m - 1);                       // reflectors of this panel: rows row0 + t .. r-1, at least two of them
     if (w == 0) band_small_qr(sh, n_ref, lane);
@@ -317,14 +323,14 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       if (t >= a && row0 + a < r) gB[(int64_t)(c + t) * (kBw + 1) + kBw + a - t] = sh.top[a][t];
     }
     const bool first = c == 0;
-    const int s0 = first_strip + ((g - first_strip % G) % G + G) % G;      // first active strip of this CTA
-    const int n_own = s0 < n_strips ? (n_strips - 1 - s0) / G + 1 : 0;
-    // ---- pass over the own strips ----
+    // ---- pass ----
     const int per = ((m + PARTS - 1) / PARTS + 3) & ~3;      // columns per task, a multiple of the group
     __syncthreads();
-    // tasks (strip, part), dealt to the warps
-    for (int task = w; task < n_own * PARTS; task += kWarps) {
-      const int s = s0 + task / PARTS * G, part = task % PARTS;
+    sh.s_part[w][lane] = sh.s_part[w][lane + 32] = 0.0;
+    __syncwarp();
+    // tasks (strip, part), dealt to the warps of all CTAs
+    for (int task = g + w * G; task < (n_strips - first_strip) * PARTS; task += kWarps * G) {
+      const int s = first_strip + task / PARTS, part = task % PARTS;
       const int jb = row0 + part * per, je = min(jb + per, r);
       const int i = s * kStrip + 2 * lane;
       double* const dst = gPart + ((int64_t)part * n_strips * kStrip + i) * 8;
@@ -407,65 +413,55 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       }
       __syncwarp();                                          // the ring is free for the warp's next task
 #pragma unroll
+      for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; }
+#pragma unroll
       for (int t = 0; t < 8; t += 2) {
-        *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t] + (double)q0[t], p0[t + 1] + (double)q0[t + 1]);
-        *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t] + (double)q1[t], p1[t + 1] + (double)q1[t + 1]);
+        *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t], p0[t + 1]);
+        *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t], p1[t + 1]);
+      }
+      const bool in0 = i >= row0 && i < r, in1 = i + 1 >= row0 && i + 1 < r;
+#pragma unroll 1
+      for (int a = 0; a < 8; ++a) {                          // row a of U^T (A U): this task's rows and columns
+        const double ua = in0 ? (double)s_u[(size_t)i * 8 + a] : 0.0, ub = in1 ? (double)s_u[(size_t)(i + 1) * 8 + a] : 0.0;
+        double x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = fma(ub, p1[t], fma(ua, p0[t], kFix)) - kFix;
+        const double sum = band_scatter8(x, lane);
+        if ((lane & 3) == 0) sh.s_part[w][a * 8 + (lane >> 2)] += sum;
       }
     }
+    for (int half = own_from(row0) + w * G; half < 2 * n_strips; half += kWarps * G) {   // U^T U of the own half strips
+      const int i = half * 32 + lane;
+      const bool in = i >= row0 && i < r;
+      const float4* src = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : row0) * 8);
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      band_gram32(in ? src[0] : zero, in ? src[1] : zero, gM + (int64_t)half * 36, lane);
+    }
     __syncthreads();
-    // ---- P = A U of the own rows (parts added in order), U^T P and U^T U; eight rows per warp at a time ----
-    {
-      long long acc[8];
+    if (tid < 64) {
+      double t = 0.0;
 #pragma unroll
-      for (int a = 0; a < 8; ++a) acc[a] = 0;
-      for (int q = w; q < n_own * (kStrip / 8); q += kWarps) {
-        const int i0 = (s0 + q / (kStrip / 8) * G) * kStrip + q % (kStrip / 8) * 8;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {                        // lane: row i0 + 4 h + lane / 8, column lane % 8
-          const int i = i0 + 4 * h + lane / 8;
-          double pp[PARTS];
-#pragma unroll
-          for (int part = 0; part < PARTS; ++part) pp[part] = gPart[((int64_t)part * n_strips * kStrip + i) * 8 + lane % 8];
-          double p = 0.0;
-#pragma unroll
-          for (int part = 0; part < PARTS; ++part) p += pp[part];
-          gP[(int64_t)i * 8 + lane % 8] = p;
-          if (i >= row0 && i < r) {
-#pragma unroll
-            for (int a = 0; a < 8; ++a) acc[a] += __double2ll_rn((double)s_u[(size_t)i * 8 + a] * p * kFix);
-          }
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < 8; ++a) { acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 8); acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 16); }
-      long long* const part_s = reinterpret_cast<long long*>(s_ring);      // [warp][64]: the ring is empty
-      if (lane < 8) {
-#pragma unroll
-        for (int a = 0; a < 8; ++a) part_s[w * 64 + a * 8 + lane] = acc[a];
-      }
-      for (int q = w; q < 2 * n_own; q += kWarps) {          // half strips
-        const int half = 2 * (s0 + q / 2 * G) + (q & 1), i = half * 32 + lane;
-        const bool in = i >= row0 && i < r;
-        const float4* src = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : row0) * 8);
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        band_gram32(in ? src[0] : zero, in ? src[1] : zero, gM + (int64_t)half * 36, lane);
-      }
-      __syncthreads();
-      if (tid < 64) {
-        long long t = 0;
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) t += part_s[ww * 64 + tid];
-        atomicAdd(reinterpret_cast<unsigned long long*>(s_sum) + tid, (unsigned long long)t);
-      }
+      for (int ww = 0; ww < kWarps; ++ww) t += sh.s_part[ww][tid];
+      atomicAdd(s_sum + tid, t);
     }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
     // ---- T, T^T S T, W of the next panel's pivot rows (every CTA) ----
     if (tid >= THREADS - 64) {
       const int q = tid - (THREADS - 64);
-      sh.S[q / 8][q % 8] = (double)__ldcg(s_sum + q) * (1.0 / kFix);
+      sh.S[q / 8][q % 8] = __ldcg(s_sum + q);
     }
-    band_sum36<THREADS>(gM, 2 * first_strip, 2 * n_strips, sh.sum, sh.M);
+    band_sum36<THREADS>(gM, row0 / 32, 2 * n_strips, sh.sum, sh.M);
+    if (tid >= THREADS - 128 && tid < THREADS - 64) {         // the product's next pivot rows
+      const int q = tid - (THREADS - 128), i = row0 + q / 8;
+      double p = 0.0;
+      if (i < r) {
+        const double* src = gPart + (int64_t)i * 8 + q % 8;
+#pragma unroll
+        for (int part = 0; part < PARTS; ++part) p += __ldcg(src + (int64_t)part * n_strips * kStrip * 8);
+      }
+      sh.Pc[q / 8][q % 8] = p;
+    }
     __syncthreads();
     if (w == 0) {
       // T: tau_t in place t, -tau_t T[0:t, 0:t] M[0:t, t] above (lane: row)
@@ -502,7 +498,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
       double z = 0.0;
       if (i < r) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { z = fma(__ldcg(gP + (int64_t)i * 8 + q), sh.T[q][t], z); z = fma((double)s_u[(size_t)i * 8 + q], sh.X[q][t], z); }
+        for (int q = 0; q < 8; ++q) { z = fma(sh.Pc[a][q], sh.T[q][t], z); z = fma((double)s_u[(size_t)i * 8 + q], sh.X[q][t], z); }
       }
       sh.Wc[a][t] = (double)(float)z;
       sh.Uc[a][t] = i < r ? (double)s_u[(size_t)i * 8 + t] : 0.0;
@@ -660,7 +656,7 @@ int band_sms() {
 // sixteen warps per SM, a strip each, its columns split over the warps.  Shared memory: U of the panel and the warps' rings.
 struct BandForm { int max_r, threads, per_sm, parts, stages; const void* fn; };
 const BandForm kBandForms[] = {
-    {1024, 256, 2, 4, 6, (const void*)sp_band_kernel<256, 2, 4, 6>},
+    {1024, 256, 2, 4, 4, (const void*)sp_band_kernel<256, 2, 4, 4>},
     {4096, 512, 1, 16, 4, (const void*)sp_band_kernel<512, 1, 16, 4>},
 };
 size_t band_smem(const BandForm& f, int r_max) { return ((size_t)(r_max + kGroup) * 8 + (size_t)f.threads / 32 * f.stages * kGroupFloats) * sizeof(float); }

@@ -109,7 +109,7 @@ struct SpLayer {
   float* bd_UW;                // [rows padded to strips][16] U and W of the panel before
   float* bd_X;                 // [rows padded to strips][8] entries of the next panel
   double* bd_part;             // [parts][rows padded to strips][8] partial products
-  double* bd_P; long long* bd_S; // [rows padded to strips][8] product A U; [3][64] U^T A U, fixed point, of three panels in turn
+  double* bd_S;                // [3][64] U^T A U of three panels in turn
   double* bd_G; double* bd_M;  // [half strips][36] dots of the next panel's columns, of U's
   double* bd_band;             // [r][9] the band, by column
   float* bd_V2;                // [r][steps][8] reflectors of the chase: sweep, step
