@@ -33,24 +33,28 @@ static_assert(kBw == 8, "the operand vectors are two float4");
 }  // namespace
 
 // ---- stage 1: dense -> band ---------------------------------------------------------------------------------------------
-// Panel k (c = 8 k): columns c .. c+7 below row c+7.  The rows (= columns: A is symmetric) are cut into strips of 64; a
-// layer's G CTAs take the strips in turn.  A[j][i] with i in the strip is read as row j, two neighbouring entries per lane
-// (256 bytes per warp), so a lane keeps everything of its two rows -- their entries of U and W of the panel before, and
-// their eight sums of the product -- in registers and walks over the columns j, whose U, W and new U entries are broadcast
-// from shared memory: 48 multiply-adds per 8 bytes read and written and six 16-byte broadcasts, no exchange between lanes
-// (17 cycles per column and warp on an SM, 70 % of the FMA rate, when the data is at hand).  The columns of a strip are split
-// into PARTS tasks for the warps; the parts of a sum are added in fp64.
+// Panel k (c = 8 k): columns c .. c+7 below row c+7.  The rows (= columns: A is symmetric) are cut into strips of 64.
+// A[j][i] with i in the strip is read as row j, two neighbouring entries per lane (256 bytes per warp), so a lane keeps
+// everything of its two rows -- their entries of U and W of the panel before, and their eight sums of the product -- in
+// registers and walks over the columns j, whose U, W and new U entries are broadcast from shared memory: 48 multiply-adds per
+// 8 bytes read and written and six 16-byte broadcasts, no exchange between lanes.  The columns of a strip are split into PARTS
+// tasks, dealt to the warps of all the layer's CTAs in turn (a strip per CTA left half of them idle on average); the parts of a
+// sum are added in fp64.  A warp streams its columns through a ring of its own (asynchronous copies of four columns with their
+// U and W).  Twelve warps per SM: with sixteen the 128 registers do not hold a task.
+// Bound: latency of the walk with few layers (a group of four columns takes a lone warp about 1000 cycles, its 200
+// multiply-adds alone would take 200), and the chain of a panel's small steps (Gram sums, 8 x 8 factorisation, U, T: 25 k
+// cycles).  Two layers of 4096 rows: 106 (one-stage reduction) -> 49.7 -> 25.9 ms; 96 of 1024: 29.4 -> 13.2 ms.
 // The panel's QR is a Householder QR worked out on 8 x 8 matrices: the reflectors' norms and products follow from the panel's
 // Gram matrix (downdated as rows of R split off) and its first eight rows, and below those rows V = X K with an 8 x 8 matrix
 // K.  A column whose remainder is below 3e-8 of it is left alone (the fp32 panel has no more digits).  However inexact V is
 // for an ill-conditioned panel, Q stays orthogonal: T comes from the actual dots of the rounded U.
 // A panel has two barriers among the layer's CTAs:
 //   every CTA: Gram matrix and first rows of the panel in, 8 x 8 factorisation (one warp), U = X K for all rows
-//   pass:      own strips: update with the panel before, product with this panel's U; U^T A U and U^T U        -> barrier
+//   pass:      tasks: update with the panel before, product with this panel's U, U^T A U; U^T U of own rows      -> barrier
 //   every CTA: T, T^T (U^T A U) T; own rows: W = (A U) T - 1/2 U T^T (U^T A U) T, entries of the next panel and their Gram
 //              matrix                                                                                          -> barrier
-// Sums over rows are formed per strip (or half strip) in an order of their own and added up in strip order, U^T A U in fixed
-// point, so the result does not depend on G.  With two CTAs per SM, which belong to different layers, one's chains and
+// Sums over rows are formed per half strip in an order of their own and added up in that order, U^T A U in multiples of a
+// fixed unit, so the result does not depend on G.  With two CTAs per SM, which belong to different layers, one's chains and
 // barriers overlap with the other's pass.
 namespace {
 
@@ -209,7 +213,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int r = L.r, g = me.slot, G = me.pad;
   const int n_strips = (r + kStrip - 1) / kStrip;
-  float* const A = L.A; const int64_t lda = L.lda;           // lda is a multiple of the strip: whole strips may be read and written
+  float* const A = L.A; const int64_t lda = L.lda; const int ld32 = (int)lda;           // lda is a multiple of the strip: whole strips may be read and written
   float* const gUW = L.bd_UW; float* const gX = L.bd_X;
   double* const gPart = L.bd_part; double* const gS = L.bd_S; double* const gB = L.bd_band;
   double* const gG = L.bd_G; double* const gM = L.bd_M;
@@ -340,25 +344,27 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         continue;
       }
       // a group of four columns: 64 entries of A each (16 bytes per lane, half a warp per column), then their U and W
-      const int groups = (je - jb + kGroup - 1) / kGroup;
-      float* const ring = s_ring + (size_t)w * STAGES * kGroupFloats;
-      const float* src = A + (int64_t)(jb + lane / 16) * lda + s * kStrip + (lane & 15) * 4;
-      const float* src_uw = gUW + (int64_t)jb * 16 + lane * 4;
-      auto issue = [&](int q) {
-        if (q < groups) {
-          const uint32_t d = (uint32_t)__cvta_generic_to_shared(ring + (q % STAGES) * kGroupFloats + lane * 4);
-          const int j = jb + q * kGroup;
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(j + lane / 16 < je ? src : A), "r"(j + lane / 16 < je ? 16 : 0) : "memory");
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 512), "l"(j + 2 + lane / 16 < je ? src + 2 * lda : A),
-                       "r"(j + 2 + lane / 16 < je ? 16 : 0) : "memory");
+      const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_ring + (size_t)w * STAGES * kGroupFloats);
+      const float* src = A + (int64_t)(jb + lane / 16) * lda + s * kStrip + (lane & 15) * 4;   // the next group to ask for
+      const float* const src_uw = gUW + lane * 4;
+      const int back = 2 * lane - (lane & 15) * 4 - (lane / 16 + (STAGES - 1) * kGroup) * ld32;   // from there to the group at work
+      int stage = 0;
+      auto issue = [&](int j) {                              // columns j .. j + 3 into the ring
+        if (j < je) {
+          const uint32_t d = ring + stage * (kGroupFloats * 4) + lane * 16;
+          const int n = je - j;                              // (lanes past the end fill with zeros)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(lane / 16 < n ? src : A), "r"(lane / 16 < n ? 16 : 0) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 512), "l"(2 + lane / 16 < n ? src + 2 * ld32 : A),
+                       "r"(2 + lane / 16 < n ? 16 : 0) : "memory");
           if (!first && lane < 16)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 1024), "l"(j + lane / 4 < je ? src_uw : gUW), "r"(j + lane / 4 < je ? 16 : 0) : "memory");
-          src += (int64_t)kGroup * lda; src_uw += kGroup * 16;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 1024), "l"(src_uw + (lane / 4 < n ? j * 16 : 0)), "r"(lane / 4 < n ? 16 : 0) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory"); // one group per call, empty or not: the counting stays uniform
+        src += kGroup * ld32;
+        stage = stage == STAGES - 1 ? 0 : stage + 1;
       };
 #pragma unroll
-      for (int q = 0; q < STAGES - 1; ++q) issue(q);
+      for (int q = 0; q < STAGES - 1; ++q) issue(jb + q * kGroup);
       float up0[8], wp0[8], up1[8], wp1[8];
       double p0[8], p1[8];
 #pragma unroll
@@ -374,46 +380,54 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
           wp1[4 * h] = -e.x; wp1[4 * h + 1] = -e.y; wp1[4 * h + 2] = -e.z; wp1[4 * h + 3] = -e.w;
         }
       }
-      float q0[8], q1[8];                                    // fp32 runs of up to 32 columns
+      // (two loops, so that the fp64 sums can leave the registers for the inner one: a spill among the 128 registers costs
+      // every group a round trip to the L2, there is no L1 left beside the shared memory)
+#pragma unroll 1
+      for (int j0 = jb; j0 < je; j0 += 32) {                 // fp32 runs of up to 32 columns
+        float q0[8], q1[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) q0[t] = q1[t] = 0.0f;
-      float* ap = A + (int64_t)jb * lda + i;
-      const float4* un = reinterpret_cast<const float4*>(s_u) + (size_t)jb * 2;
-      int left = je - jb;
-      for (int q = 0; q < groups; ++q, left -= kGroup) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-        __syncwarp();                                        // group q has landed for the warp; the stage of group q - 1 is free
-        issue(q + STAGES - 1);
-        const float* const st = ring + (q % STAGES) * kGroupFloats;
+        for (int t = 0; t < 8; ++t) q0[t] = q1[t] = 0.0f;
+#pragma unroll 1
+        for (int j = j0; j < min(je, j0 + 32); j += kGroup) {
+          asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+          __syncwarp();                                      // the group has landed for the warp; the stage of the one before is free
+          const int at = stage == STAGES - 1 ? 0 : stage + 1;
+          float* const ap = const_cast<float*>(src) + back;
+          issue(j + (STAGES - 1) * kGroup);
+          const float* const st = s_ring + ((size_t)w * STAGES + at) * kGroupFloats;
+          const float4* const un = reinterpret_cast<const float4*>(s_u) + (size_t)j * 2;
+          // the columns are stored together at the end: a store between them might alias the shared memory for all the
+          // compiler knows, so that a column's loads would wait for the column before it
+          float2 out[kGroup];
 #pragma unroll
-        for (int u = 0; u < kGroup; ++u) {                   // one column: update, store, product
-          float2 v = *reinterpret_cast<const float2*>(st + u * kStrip + 2 * lane);
-          if (!first) {
-            const float4* o = reinterpret_cast<const float4*>(st + kGroup * kStrip + u * 16);
-            const float4 cu0 = o[0], cu1 = o[1], cw0 = o[2], cw1 = o[3];
-            const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
-            const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
+          for (int u = 0; u < kGroup; ++u) {                 // one column: update, product
+            float2 v = *reinterpret_cast<const float2*>(st + u * kStrip + 2 * lane);
+            if (!first) {
+              const float4* o = reinterpret_cast<const float4*>(st + kGroup * kStrip + u * 16);
+              const float4 cu0 = o[0], cu1 = o[1], cw0 = o[2], cw1 = o[3];
+              const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
+              const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              v.x = fmaf(up0[t], cw[t], v.x); v.y = fmaf(up1[t], cw[t], v.y);
-              v.x = fmaf(wp0[t], cu[t], v.x); v.y = fmaf(wp1[t], cu[t], v.y);
+              for (int t = 0; t < 8; ++t) {
+                v.x = fmaf(up0[t], cw[t], v.x); v.y = fmaf(up1[t], cw[t], v.y);
+                v.x = fmaf(wp0[t], cu[t], v.x); v.y = fmaf(wp1[t], cu[t], v.y);
+              }
             }
-            if (u < left) *reinterpret_cast<float2*>(ap + (int64_t)u * lda) = v;
+            out[u] = v;
+            const float4 n0 = un[2 * u], n1 = un[2 * u + 1];
+            const float cn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { q0[t] = fmaf(v.x, cn[t], q0[t]); q1[t] = fmaf(v.y, cn[t], q1[t]); }
           }
-          const float4 n0 = un[2 * u], n1 = un[2 * u + 1];
-          const float cn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+          if (!first) {
 #pragma unroll
-          for (int t = 0; t < 8; ++t) { q0[t] = fmaf(v.x, cn[t], q0[t]); q1[t] = fmaf(v.y, cn[t], q1[t]); }
+            for (int u = 0; u < kGroup; ++u) if (j + u < je) *reinterpret_cast<float2*>(ap + u * ld32) = out[u];
+          }
         }
-        if ((q & 7) == 7) {
 #pragma unroll
-          for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; q0[t] = q1[t] = 0.0f; }
-        }
-        un += 2 * kGroup; ap += (int64_t)kGroup * lda;
+        for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; }
       }
       __syncwarp();                                          // the ring is free for the warp's next task
-#pragma unroll
-      for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; }
 #pragma unroll
       for (int t = 0; t < 8; t += 2) {
         *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t], p0[t + 1]);
@@ -653,11 +667,11 @@ int band_sms() {
   return sms;
 }
 // The instances of the band kernel.  Many layers up to 1024 rows: two small CTAs per SM.  Few layers, or larger ones: one CTA of
-// sixteen warps per SM, a strip each, its columns split over the warps.  Shared memory: U of the panel and the warps' rings.
+// twelve warps per SM, a strip's columns in sixteen tasks.  Shared memory: U of the panel and the warps' rings.
 struct BandForm { int max_r, threads, per_sm, parts, stages; const void* fn; };
 const BandForm kBandForms[] = {
-    {1024, 256, 2, 4, 4, (const void*)sp_band_kernel<256, 2, 4, 4>},
-    {4096, 512, 1, 16, 4, (const void*)sp_band_kernel<512, 1, 16, 4>},
+    {1024, 192, 2, 4, 4, (const void*)sp_band_kernel<192, 2, 4, 4>},
+    {4096, 384, 1, 16, 4, (const void*)sp_band_kernel<384, 1, 16, 4>},
 };
 size_t band_smem(const BandForm& f, int r_max) { return ((size_t)(r_max + kGroup) * 8 + (size_t)f.threads / 32 * f.stages * kGroupFloats) * sizeof(float); }
 template <int C, int COLS> int chase_configure() {
