@@ -61,7 +61,7 @@ namespace {
 constexpr int kGroup = 4;                     // columns that travel together through a warp's ring
 constexpr int kGroupFloats = kGroup * (kStrip + 16);
 // U^T A U is rounded to multiples of 2^-50 (the last place of 4 .. 8) as it is added up: sums below 8 are then exact in any order.
-// (A has trace one at most and U unit columns, so that no partial sum passes one.)
+// (A's trace is about one and U's columns are unit vectors, so that no partial sum passes two.)
 constexpr double kFix = 6.0;
 
 struct BandShared {
@@ -428,12 +428,15 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         for (int t = 0; t < 8; ++t) { p0[t] += (double)q0[t]; p1[t] += (double)q1[t]; }
       }
       __syncwarp();                                          // the ring is free for the warp's next task
+      // rows outside the trailing block (past the end A holds whatever the workspace held) count as zeros
+      const bool in0 = i >= row0 && i < r, in1 = i + 1 >= row0 && i + 1 < r;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) { if (!in0) p0[t] = 0.0; if (!in1) p1[t] = 0.0; }
 #pragma unroll
       for (int t = 0; t < 8; t += 2) {
         *reinterpret_cast<double2*>(dst + t) = make_double2(p0[t], p0[t + 1]);
         *reinterpret_cast<double2*>(dst + 8 + t) = make_double2(p1[t], p1[t + 1]);
       }
-      const bool in0 = i >= row0 && i < r, in1 = i + 1 >= row0 && i + 1 < r;
 #pragma unroll 1
       for (int a = 0; a < 8; ++a) {                          // row a of U^T (A U): this task's rows and columns
         const double ua = in0 ? (double)s_u[(size_t)i * 8 + a] : 0.0, ub = in1 ? (double)s_u[(size_t)(i + 1) * 8 + a] : 0.0;
