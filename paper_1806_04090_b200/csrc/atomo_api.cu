@@ -509,7 +509,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
     } else {
-      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) gram_tiles.push_back({l, a, b, 0});
+      d.gram_split = given ? 1 : sp_gram_split(d.r, d.L);
+      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.gram_split; ++c) gram_tiles.push_back({l, a, b, c});
     }
     for (int p = 0; p < d.nb / 2; ++p) block_pairs.push_back({l, p, 0, 0});
     row_floats_max = std::max(row_floats_max, d.ldx); steps_max = std::max(steps_max, d.nb - 1);
@@ -537,7 +538,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       for (int a = 0; a < gt; ++a) for (int b = 0; b < d.refine_tiles; ++b) refine_tiles.push_back({l, a, b, 0});
   }
   // Tridiagonal routes first: eigenvalues of every atom from T = Q^T A Q, vectors for the kept atoms only -- in the
-  // registers of a cluster for short sides up to 512, blocked with A in global memory above (no per-atom refinement,
+  // registers of a cluster for short sides up to 512, in two stages with A in global memory above (no per-atom refinement,
   // no request for the whole short-side basis).  Otherwise the Jacobi routes, the cluster form first.
   bool tri_form = !given && ctx->eig_scheme == 3 && ctx->eig_mode != 0 && !(dbg && dbg->short_vecs);
   bool any_small = false, any_big = false;
@@ -744,6 +745,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.gram_part = A.take<float>(d.tc && d.gram_split > 1
                                         ? (size_t)tt * (tt + 1) / 2 * d.gram_split * sp_tc_tile() * sp_tc_tile() : 0);
       }
+      d.gram_sums = A.take<double>(d.tc ? 0 : (size_t)sp_gram_sums(d.r, d.gram_split));
       d.td_d = A.take<double>(d.tri ? d.rp : 0); d.td_e = A.take<double>(d.tri ? d.rp : 0);
       d.td_tau = A.take<double>(d.tri ? d.rp : 0); d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
@@ -774,7 +776,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     for (int l = 0; l < n_layers; ++l) { L[l].rot_count = A.take<uint32_t>(max_sweeps); L[l].step_bar = A.take<uint32_t>(1); L[l].vec_ticket = A.take<uint32_t>(1); L[l].bd_bar = A.take<uint32_t>(1); }
     for (int l = 0; l < n_layers; ++l) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
-      L[l].gram_ticket = A.take<uint32_t>(L[l].tc && L[l].gram_split > 1 ? (size_t)tt * (tt + 1) / 2 : 0);
+      const int tf = (L[l].r + 63) / 64;
+      L[l].gram_ticket = A.take<uint32_t>(L[l].gram_split > 1 ? (size_t)(L[l].tc ? tt * (tt + 1) / 2 : tf * (tf + 1) / 2) : 0);
     }
     for (int l = 0; l < n_layers; ++l) L[l].X = A.take<float>(L[l].tri ? 0 : (size_t)L[l].rp * L[l].ldx);
     zero_beg = zb; zero_bytes = A.off - z0;
@@ -831,7 +834,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if (ctx->eig_mode == 0) launch_sp_init(d_layers, n_layers, nullptr, 0, st);   // the identity half of [A | I]
   launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), st);
   launch_sp_gram_tc(d_layers, d_maps, d_tc, (int)tc_tiles.size(), d_flag + 1, st);
-  launch_sp_scale(d_layers, n_layers, st);
+  launch_sp_scale(d_layers, n_layers, r_max, st);
   }
   if (!given && ctx->eig_mode != 0 && !tri_form) {
     const int ec = launch_sp_cholesky(d_layers, n_layers, rp_max, st);

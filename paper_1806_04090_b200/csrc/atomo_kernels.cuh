@@ -91,14 +91,15 @@ struct SpLayer {
   float* chol_dd;              // 32 x 32 + 32 floats: diagonal block of the current Cholesky panel, published by its owner
   float* dbg_short;            // r x r or nullptr
   int tc;                      // Gram matrix came from the tensor-core kernel (see sp_scale_kernel)
-  int gram_split;              // tensor-core Gram: CTAs per output tile (parts of the K range), 1 = no split
+  int gram_split;              // Gram matrix: CTAs per output tile (parts of the K range), 1 = no split
   float* gram_part;            // [tiles][gram_split][128 x 128] partial tiles (column-major) when gram_split > 1
+  double* gram_sums;           // FMA kernel: [tiles][gram_split][64 x 64] partial tiles
   uint32_t* gram_ticket;       // [tiles] parts finished; zeroed per call
   int refine, refine_tiles;    // singular values from the projection norms; tiles along the long side
   float* row_inv;              // rp: 1 / norm of each short-side vector as stored in X
   float* refine_partials;      // [refine_tiles][rp] partial squared norms
   // tridiagonal route (short side <= 512): T = Q^T A Q, eigenvalues by bisection, vectors of the kept atoms only
-  int tri;                     // this layer takes the tridiagonal route: 1 = registers of a cluster (rp <= 512), 2 = blocked, A in global memory
+  int tri;                     // this layer takes the tridiagonal route: 1 = registers of a cluster (rp <= 512), 2 = two stages, A in global memory
   double* td_d; double* td_e;  // rp each: diagonal and off-diagonal of T
   double* td_tau;              // rp: beta_k of the reflectors H_k = I - beta_k v_k v_k^T
   int td_ldv;                  // floats per row of td_V: r rounded up to a multiple of 4 (16-byte rows)
@@ -128,8 +129,10 @@ struct TileRef { int32_t layer, a, b, c; };
 void launch_sp_begin(uint8_t* pay, const atomo_payload_header& gh, const atomo_layer_header* d_tmpl, int n_layers,
                      uint32_t* d_flags, cudaStream_t st);
 void launch_sp_init(const SpLayer* d_layers, int n_layers, const TileRef* d_diag_tiles, int n_diag_tiles, cudaStream_t st);
+int sp_gram_split(int r, int len);                               // FMA kernel: parts of the K range, doubles for their sums
+int64_t sp_gram_sums(int r, int split);
 void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
-void launch_sp_scale(const SpLayer* d_layers, int n_layers, cudaStream_t st);   // trace, then scaling
+void launch_sp_scale(const SpLayer* d_layers, int n_layers, int r_max, cudaStream_t st);   // trace, then scaling
 void launch_sp_load_svd(const SpLayer* d_layers, int n_layers, const float* const* d_sigma, const float* const* d_vecs,
                         cudaStream_t st);                                       // a decomposition given by the caller
 // one Jacobi step (global step index t) for every layer of the batch

@@ -41,9 +41,17 @@ void launch_sp_init(const SpLayer* d_layers, int n_layers, const TileRef*, int, 
 
 // =================================================================================================
 // Gram matrix of the short side.  64 x 64 output tile per CTA, 16 x 16 threads, 4 x 4 per thread.
-// Short-side vector i is row i of G (rows <= cols) or column i of G (rows > cols).
+// Short-side vector i is row i of G (rows <= cols) or column i of G (rows > cols).  A layer with a short side of up to 1024 has
+// its K range cut into parts (ref.c: which part) of 512, or 2048 above 256, where they have more tiles (a 16384 x 18 layer was one CTA walking over 16384 rows: 1340 -> 235 us for a set with
+// some); above there are tiles enough, and the parts' sums would cost more than they bring.
 // =================================================================================================
 constexpr int kGramTile = 64, kGramK = 16;
+__host__ __device__ inline int gram_part(int r) { return r <= 256 ? 512 : 2048; }
+int sp_gram_split(int r, int len) { return r <= 1024 ? (len + gram_part(r) - 1) / gram_part(r) : 1; }
+int64_t sp_gram_sums(int r, int split) {
+  const int64_t gt = (r + kGramTile - 1) / kGramTile;
+  return split > 1 ? gt * (gt + 1) / 2 * split * kGramTile * kGramTile : 0;
+}
 
 __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict__ layers,
                                                       const TileRef* __restrict__ tiles) {
@@ -55,8 +63,10 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
   const bool diag = ref.a == ref.b;
   const float* __restrict__ G = L.G;
   const int64_t ld = L.ld;
-  const int r = L.r, len = L.L;
+  const int r = L.r, len = L.L, n_split = L.gram_split;
+  const bool tall = L.tall;
   const int t = threadIdx.x, ty = t / 16, tx = t % 16;
+  __shared__ bool s_last;
   float acc[4][4];
   double acc64[4][4];
 #pragma unroll
@@ -64,28 +74,29 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) { acc[a][b] = 0.0f; acc64[a][b] = 0.0; }
 
-  int flush = 0;
-  for (int c0 = 0; c0 < len; c0 += kGramK) {
-    // stage As[kk][i] = x_{i0+i}[c0+kk], Bs likewise for j0
-    if (!L.tall) {
-      const int row = t / 4, k4 = (t % 4) * 4;
+  // the K range of a tile is cut into parts of kGramPart where a layer has few tiles
+  const int c_lo = n_split > 1 ? ref.c * gram_part(r) : 0, c_hi = n_split > 1 ? min(len, c_lo + gram_part(r)) : len;
+  // this thread's entries of the next stage, fetched while the stage before is multiplied
+  const int row = tall ? t / 16 : t / 4, col = (tall ? t % 16 : t % 4) * 4;
+  float fa[4], fb[4];
+  auto fetch = [&](int c0) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = c0 + k4 + j;
-        const int ia = i0 + row, ib = j0 + row;
-        As[k4 + j][row] = (ia < r && c < len) ? __ldg(G + (int64_t)ia * ld + c) : 0.0f;
-        if (!diag) Bs[k4 + j][row] = (ib < r && c < len) ? __ldg(G + (int64_t)ib * ld + c) : 0.0f;
-      }
-    } else {
-      const int kk = t / 16, i4 = (t % 16) * 4;
-      const int c = c0 + kk;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int ia = i0 + i4 + j, ib = j0 + i4 + j;
-        As[kk][i4 + j] = (ia < r && c < len) ? __ldg(G + (int64_t)c * ld + ia) : 0.0f;
-        if (!diag) Bs[kk][i4 + j] = (ib < r && c < len) ? __ldg(G + (int64_t)c * ld + ib) : 0.0f;
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int c = tall ? c0 + row : c0 + col + j, ia = tall ? i0 + col + j : i0 + row, ib = tall ? j0 + col + j : j0 + row;
+      fa[j] = ia < r && c < c_hi ? __ldg(G + (tall ? (int64_t)c * ld + ia : (int64_t)ia * ld + c)) : 0.0f;
+      if (!diag) fb[j] = ib < r && c < c_hi ? __ldg(G + (tall ? (int64_t)c * ld + ib : (int64_t)ib * ld + c)) : 0.0f;
     }
+  };
+  fetch(c_lo);
+  int flush = 0;
+  for (int c0 = c_lo; c0 < c_hi; c0 += kGramK) {
+    // As[kk][i] = x_{i0+i}[c0+kk], Bs likewise for j0
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (tall) { As[row][col + j] = fa[j]; if (!diag) Bs[row][col + j] = fb[j]; }
+      else { As[col + j][row] = fa[j]; if (!diag) Bs[col + j][row] = fb[j]; }
+    }
+    if (c0 + kGramK < c_hi) fetch(c0 + kGramK);
     __syncthreads();
     const float(*Bp)[kGramTile + 4] = diag ? As : Bs;
 #pragma unroll
@@ -107,6 +118,30 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
         for (int q = 0; q < 4; ++q) { acc64[p][q] += (double)acc[p][q]; acc[p][q] = 0.0f; }
     }
   }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc64[p][q] += (double)acc[p][q];
+  if (n_split > 1) {                                          // the last part to finish adds them up, in order
+    const int gt = (r + kGramTile - 1) / kGramTile, tile = ref.a * gt - ref.a * (ref.a - 1) / 2 + ref.b - ref.a;
+    double* const parts = L.gram_sums + (int64_t)tile * n_split * (kGramTile * kGramTile);
+    double* const mine = parts + (int64_t)ref.c * (kGramTile * kGramTile) + t;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) mine[e * 256] = acc64[e / 4][e % 4];
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(L.gram_ticket + tile, 1u) == (uint32_t)(n_split - 1);
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] = 0.0;
+    for (int s = 0; s < n_split; ++s) {
+      const double* part = parts + (int64_t)s * (kGramTile * kGramTile) + t;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] += __ldcg(part + e * 256);
+    }
+  }
   const int64_t lda = L.lda;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
@@ -114,7 +149,7 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
     for (int q = 0; q < 4; ++q) {
       const int i = i0 + ty * 4 + p, j = j0 + tx * 4 + q;
       if (i < r && j < r) {
-        const float v = (float)(acc64[p][q] + (double)acc[p][q]);
+        const float v = (float)acc64[p][q];
         L.A[(int64_t)i * lda + j] = v;
         if (!diag) L.A[(int64_t)j * lda + i] = v;
       }
@@ -195,9 +230,10 @@ void launch_sp_load_svd(const SpLayer* d_layers, int n_layers, const float* cons
   sp_load_svd_kernel<<<dim3(n_layers, 32), 256, 0, st>>>(d_layers, d_sigma, d_vecs);
 }
 
-void launch_sp_scale(const SpLayer* d_layers, int n_layers, cudaStream_t st) {
+void launch_sp_scale(const SpLayer* d_layers, int n_layers, int r_max, cudaStream_t st) {
   sp_trace_kernel<<<n_layers, 256, 0, st>>>(d_layers);
-  sp_scale_kernel<<<dim3(n_layers, 32), 256, 0, st>>>(d_layers);
+  // (a 4096-row layer on 32 CTAs took 300 us)
+  sp_scale_kernel<<<dim3(n_layers, std::min(std::max(r_max / 8, 32), 512)), 256, 0, st>>>(d_layers);
 }
 
 // =================================================================================================
