@@ -31,8 +31,6 @@ L2_BYTES = 126 * 1024 * 1024
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant kernel, from the ncu captures
 # summarised under profiles/ (None: no capture on file for that kernel and workload)
 NCU_TRAFFIC = {("sp_tridiag_cluster_kernel", "c2"): 5638912,
-               # profiles/sp_tridiag_big1_c5.txt: 1.706 TB/s of DRAM traffic over the 29.52 ms of the captured launch
-               ("sp_tridiag_big_kernel", "c5"): 50_400_000_000,
                # profiles/entrywise_c4.txt: the encode kernel (2.09 TB/s over 51.9 us) plus the decode kernel (3.74 TB/s over
                # 24.4 us) of one step at s = 1 %
                ("entrywise", "c4"): 200_000_000}
@@ -341,6 +339,11 @@ def tridiag_big_bytes(shapes):
     return tot
 
 
+def band_bytes(shapes):
+    """Bytes of the first stage of the two-stage reduction: the trailing block read and written once per eight columns."""
+    return float(sum(8.0 * (min(sh) - c) ** 2 for sh in shapes if min(sh) > 512 for c in range(8, min(sh), 8)))
+
+
 def roofline_for(run, eig_ms_per_step, eig_launches_per_step, scheme, peaks, fma_peaks, step_ms):
     """Roofline of the dominant kernel of a spectral workload (the eigen stage)."""
     shapes = run.shapes
@@ -348,14 +351,14 @@ def roofline_for(run, eig_ms_per_step, eig_launches_per_step, scheme, peaks, fma
     out = {"share_of_step": eig_ms_per_step / step_ms, "launches_per_step": eig_launches_per_step,
            "avg_launch_us": eig_ms_per_step * 1e3 / max(eig_launches_per_step, 1.0)}
     if scheme == 3 and big:
-        # the blocked reduction dominates whenever it runs (config 3: also one launch of the small-layer kernel in the stage)
-        b = tridiag_big_bytes(shapes)
+        # the two-stage reduction dominates whenever it runs (config 3: also one launch of the small-layer kernel in the stage)
+        b = band_bytes(shapes)
         ach = b / (eig_ms_per_step * 1e-3) / 1e9
-        out.update(bound="hbm", kernel="sp_tridiag_big1_kernel (one CTA per layer)" if max(min(sh) for sh in shapes) <= 1024 and sum(1 for sh in shapes if min(sh) > 512) >= 38 else "sp_tridiag_big_kernel (clusters)", achieved=ach, peak=peaks["hbm_gbs"], unit="GB/s",
-                   frac=ach / peaks["hbm_gbs"], traffic=NCU_TRAFFIC.get(("sp_tridiag_big_kernel", run.name)),
+        out.update(bound="hbm", kernel="sp_band_kernel, then sp_chase_kernel", achieved=ach, peak=peaks["hbm_gbs"], unit="GB/s",
+                   frac=ach / peaks["hbm_gbs"], traffic=None,
                    peak_source=f"{peaks['source']} copy bandwidth (MEASURED_PEAKS.json)",
-                   algorithmic="one triangle of the trailing block per Householder step, 4-byte entries: (2/3) r^3 bytes per layer",
-                   arithmetic="f32 storage and products, f64 sums and scalars")
+                   algorithmic="the trailing block read and written once per panel of eight columns: r^3 / 3 bytes per layer, over the time of both stages",
+                   arithmetic="f32 storage and products, f64 sums and scalars; chase in f64")
     elif scheme == 3:
         f = tridiag_small_flops(shapes)
         ach = f / (eig_ms_per_step * 1e-3) / 1e12

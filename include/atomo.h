@@ -181,16 +181,16 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs /*HOST array*/,
  * on the format.  A vector whose kept unsaturated atoms exceed k_cap or whose saturated atoms exceed sat_cap
  * gets ATOMO_ERR_CAPACITY in its status word and k = 0.  Decoders read the format from the payload.       */
 int atomo_set_entrywise_format(atomo_ctx* ctx, int32_t format, int64_t sat_cap);
-/* Launch form of the context's later atomo_encode_entrywise calls.  two_kernels = 0 (default): a vector whose tiles
- * fit one wave of resident CTAs (up to about 48 million elements on a B200, 29 million with the list below) is encoded by ONE cooperative kernel -- a CTA
- * computes its part of sum |g| and max |g| (Algorithm 1's inputs), all CTAs meet at a grid barrier, and the same CTA
- * then samples and packs its part.  The Philox word of an atom depends on its index alone, so the first pass already
- * draws the words and lists the atoms that an estimate of sum |g| (with a factor of two to spare) cannot rule out; where
- * the true sum confirms the estimate and no atom has p = 1, the exact keep decision (the same integer comparison) is
- * taken on the list and the vector is read once.  Otherwise a CTA reads its part a second time (from the L2 cache).
- * Longer vectors take the two-kernel form.  two_kernels = 1: always a solve kernel followed by a sample / pack kernel
- * whose chunks are handed out by ticket.  two_kernels = 2: the one-kernel form without the list (every part read
- * twice).  Payloads, masks and decoded gradients are bit-identical in all forms.  Other values:
+/* Launch form of the context's later atomo_encode_entrywise calls.  two_kernels = 0 (default): the vectors of a call, up
+ * to 24 at a time, are encoded by ONE kernel with one CTA per SM, dealt to the vectors in proportion to their lengths -- a
+ * CTA computes its chunk's part of sum |g| and max |g| (Algorithm 1's inputs), a vector's CTAs meet at a barrier, and the
+ * same CTA then samples and packs its chunk.  Short chunks stay in registers between the two.  The Philox word of an atom
+ * depends on its index alone, so on longer chunks and at small budgets the first pass already draws the words and lists the
+ * atoms that an estimate of sum |g| cannot rule out; where the true sum confirms the estimate and no atom has p = 1, the
+ * exact keep decision (the same integer comparison) is taken on the list and the vector is read once.  Otherwise a CTA
+ * reads its part a second time.  Vectors that do not fit take the two-kernel form.  two_kernels = 1: always a solve kernel
+ * followed by a sample / pack kernel whose chunks are handed out by ticket.  two_kernels = 2: the one-kernel form without
+ * the list.  Payloads, masks and decoded gradients are bit-identical in all forms.  Other values:
  * ATOMO_ERR_INVALID_ARG.     */
 int atomo_set_entrywise_launch(atomo_ctx* ctx, int32_t two_kernels);
 /* Test introspection, for vector `vec` of the context's last atomo_encode_entrywise call: the number of chunks (CTAs)
@@ -299,9 +299,9 @@ int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores);
  *     kept atoms only (twisted factorisation, back-transformation with the reflectors): only the singular values of
  *     all atoms enter the probabilities, the vectors of atoms that are not kept are never formed.  Short sides up to
  *     512: the rows sit in the registers of the CTAs of a 16-CTA cluster and are exchanged through distributed shared
- *     memory, fp64 arithmetic, one cluster barrier per step.  Short sides above 512 (up to 4096): the matrix stays in
- *     global memory (fp32) and the reduction is blocked in panels of 32 columns, a cluster of 1 to 16 CTAs per layer
- *     (atomo_set_tridiag_ctas); sums and scalars in fp64.  Both kinds of layer can share one call.  A batch takes
+ *     memory, fp64 arithmetic.  Short sides above 512 (up to 4096): the matrix stays in global memory (fp32) and is
+ *     reduced in two stages, first to a band of eight sub-diagonals by any number of CTAs per layer
+ *     (atomo_set_tridiag_ctas), then by bulge chasing in fp64.  Both kinds of layer can share one call.  A batch takes
  *     scheme 2 instead when eigen-solver route 0 or the whole short-side basis (atomo_debug.short_vecs) is asked
  *     for, or when the GPU cannot place the clusters;
  * 2 = one-sided Jacobi in thread-block clusters where they apply: when every layer of the batch has at most 16 block
@@ -317,13 +317,9 @@ int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores);
  * fp32 throughout and resolve the probabilities of layers with a short side of 1024 only to a few 1e-5; they are
  * kept as a fallback and as an independent cross-check of scheme 3.                                              */
 int atomo_set_persistent_eig(atomo_ctx* ctx, int32_t enabled);
-/* CTAs per layer of the blocked tridiagonal reduction that scheme 3 runs for short sides above 512: 0 (default) =
- * chosen per batch (the fewest that hold the layer's rows, doubled while SMs would stay idle; never 2 up to a short side
- * of 1024, where one CTA per layer is faster than a pair), else 1, 2, 4, 8 or 16 (raised to the fewest that hold the rows).  With 2 to 16 CTAs a layer runs the cluster kernel, every sum of which has
- * an order that does not depend on this number: the payload is bit-identical for 2, 4, 8 and 16 (the knob exists for
- * tuning and for checking exactly that).  With 1 CTA per layer (short sides up to 1024; what a batch of 38 layers or
- * more gets) another kernel runs (triangle-only products, panels of 16 columns): same kept atoms, values equal to
- * rounding.                                                                                                    */
+/* CTAs per layer of the band reduction that scheme 3 runs for short sides above 512: 0 (default) = dealt to the layers
+ * of the batch in proportion to their work, else 1, 2, 4, 8 or 16 (at most one per 64 rows).  The payload does not
+ * depend on it bit for bit (the knob exists for tuning and for checking exactly that).                          */
 int atomo_set_tridiag_ctas(atomo_ctx* ctx, int32_t ctas_per_layer);
 /* The scheme (0 to 3 as above) that the last atomo_encode_spectral() of this context actually ran; -1 before
  * the first call.  Host only.                                                                                */

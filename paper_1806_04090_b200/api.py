@@ -7,6 +7,7 @@ device is present, the calls raise.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from dataclasses import dataclass, field
 from typing import List, Optional, Sequence
@@ -129,6 +130,22 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     if path == LIB_PATH:
         _lib = lib
     return lib
+
+
+@functools.lru_cache(maxsize=256)
+def _dims(shapes: tuple):
+    """(rows, cols) of the layers as the C arrays a decode takes; nobody writes to them."""
+    n = len(shapes)
+    return (ctypes.c_int64 * n)(*[int(r) for r, _ in shapes]), (ctypes.c_int64 * n)(*[int(c) for _, c in shapes])
+
+
+@functools.lru_cache(maxsize=256)
+def _payload_bytes(kind: int, shapes: tuple, k_cap: int, compact: bool, sat_cap: int) -> int:
+    """The payload sizes below for shapes seen before (a training step encodes the same shapes every time)."""
+    if kind == KIND_SPECTRAL:
+        return payload_bytes_spectral(shapes, k_cap)
+    lengths = [c for _, c in shapes]
+    return payload_bytes_entrywise_compact(lengths, k_cap, sat_cap) if compact else payload_bytes_entrywise(lengths, k_cap)
 
 
 def payload_bytes_spectral(shapes: Sequence[Sequence[int]], k_cap: int) -> int:
@@ -327,9 +344,9 @@ class Atomo:
             raise AtomoError(rc, where, self._cuda_error() if rc == 7 else "")
 
     @staticmethod
-    def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
-        s = stream if stream is not None else torch.cuda.current_stream()
-        return ctypes.c_void_p(s.cuda_stream)
+    def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
+        # (the stream's handle without a Stream object, which takes as long as a kernel launch)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
     def _make_debug(self, n_atoms: Sequence[int], spectral: bool, want_short: bool, dev, want_prob: bool = True) -> Debug:
         a_off = np.concatenate([[0], np.cumsum(n_atoms)]).astype(np.int64)
@@ -359,16 +376,17 @@ class Atomo:
                               stream: Optional[torch.cuda.Stream] = None):
         """Spectral ATOMO over a batch of 2-D fp32 CUDA tensors.  Returns (Payload, Debug | None)."""
         n = len(layers)
-        mats = (_Mat * n)()
-        shapes = []
-        for i, g in enumerate(layers):
+        desc, shapes = [], []
+        for g in layers:
             if not (g.is_cuda and g.dtype == torch.float32 and g.dim() == 2 and g.stride(1) == 1):
                 raise ValueError("layers must be 2-D fp32 CUDA tensors with unit column stride")
-            mats[i] = _Mat(g.data_ptr(), g.shape[0], g.shape[1], g.stride(0) if g.shape[0] > 1 else g.shape[1])
-            shapes.append((int(g.shape[0]), int(g.shape[1])))
+            m, c = g.shape
+            desc.append((g.data_ptr(), m, c, g.stride(0) if m > 1 else c))
+            shapes.append((m, c))
+        mats = (_Mat * n)(*desc)
         if k_cap is None:
             k_cap = default_k_cap(s, max(min(r, c) for r, c in shapes))
-        nbytes = payload_bytes_spectral(shapes, k_cap)
+        nbytes = _payload_bytes(KIND_SPECTRAL, tuple(shapes), int(k_cap), False, 0)
         if nbytes < 0:
             raise AtomoError(1, "atomo_payload_bytes_spectral")
         dev = layers[0].device
@@ -377,7 +395,7 @@ class Atomo:
         dbg = self._make_debug([min(r, c) for r, c in shapes], True, debug_short, dev) if (debug or debug_short) else None
         ds = self._debug_struct(dbg)
         rc = self.lib.atomo_encode_spectral(self._h, mats, n, float(s), int(seed), int(step), int(k_cap),
-                                            ctypes.c_void_p(payload.data_ptr()), payload.numel(),
+                                            payload.data_ptr(), payload.numel(),
                                             ctypes.byref(ds) if ds is not None else None, self._stream_ptr(stream))
         self._check(rc, "atomo_encode_spectral")
         return Payload(payload, KIND_SPECTRAL, shapes, int(k_cap), self), dbg
@@ -408,7 +426,7 @@ class Atomo:
         sp = (ctypes.c_void_p * n)(*[t.data_ptr() for t in sigma])
         vp_ = (ctypes.c_void_p * n)(*[t.data_ptr() for t in short_vecs])
         rc = self.lib.atomo_encode_spectral_from_svd(self._h, mats, n, sp, vp_, float(s), int(seed), int(step), int(k_cap),
-                                                     ctypes.c_void_p(payload.data_ptr()), payload.numel(),
+                                                     payload.data_ptr(), payload.numel(),
                                                      ctypes.byref(ds) if ds is not None else None, self._stream_ptr(stream))
         self._check(rc, "atomo_encode_spectral_from_svd")
         return Payload(payload, KIND_SPECTRAL, shapes, int(k_cap), self), dbg
@@ -421,32 +439,29 @@ class Atomo:
         debug: True = probabilities and mask words, "mask" = the mask words alone (asking for the probabilities makes
         the one-kernel form read every vector twice)."""
         n = len(vecs)
-        arr = (_Vec * n)()
-        lengths = []
-        for i, g in enumerate(vecs):
+        desc, shapes = [], []
+        for g in vecs:
             if not (g.is_cuda and g.dtype == torch.float32 and g.is_contiguous()):
                 raise ValueError("vectors must be contiguous fp32 CUDA tensors")
-            arr[i] = _Vec(g.data_ptr(), g.numel())
-            lengths.append(int(g.numel()))
+            length = g.numel()
+            desc.append((g.data_ptr(), length))
+            shapes.append((1, length))
+        arr = (_Vec * n)(*desc)
         if k_cap is None:
-            k_cap = default_k_cap(s, max(lengths))
-        if self._ew_format == EW_COMPACT:
-            nbytes = payload_bytes_entrywise_compact(lengths, k_cap, self._ew_sat_cap)
-        else:
-            nbytes = payload_bytes_entrywise(lengths, k_cap)
+            k_cap = default_k_cap(s, max(c for _, c in shapes))
+        nbytes = _payload_bytes(KIND_ENTRYWISE, tuple(shapes), int(k_cap), self._ew_format == EW_COMPACT, self._ew_sat_cap)
         if nbytes < 0:
             raise AtomoError(1, "atomo_payload_bytes_entrywise")
         dev = vecs[0].device
         if payload is None:
             payload = torch.empty(nbytes, dtype=torch.uint8, device=dev)
-        dbg = self._make_debug(lengths, False, False, dev, want_prob=(debug != "mask")) if debug else None
+        dbg = self._make_debug([c for _, c in shapes], False, False, dev, want_prob=(debug != "mask")) if debug else None
         ds = self._debug_struct(dbg)
         rc = self.lib.atomo_encode_entrywise(self._h, arr, n, float(s), int(seed), int(step), int(k_cap),
-                                             ctypes.c_void_p(payload.data_ptr()), payload.numel(),
+                                             payload.data_ptr(), payload.numel(),
                                              ctypes.byref(ds) if ds is not None else None, self._stream_ptr(stream))
         self._check(rc, "atomo_encode_entrywise")
-        return Payload(payload, KIND_ENTRYWISE, [(1, x) for x in lengths], int(k_cap), self,
-                       ew_format=self._ew_format, sat_cap=self._ew_sat_cap), dbg
+        return Payload(payload, KIND_ENTRYWISE, shapes, int(k_cap), self, self._ew_format, self._ew_sat_cap), dbg
 
     def atomo_decode(self, payload: Payload, out: Optional[Sequence[torch.Tensor]] = None,
                      stream: Optional[torch.cuda.Stream] = None) -> List[torch.Tensor]:
@@ -456,10 +471,9 @@ class Atomo:
         if out is None:
             out = [torch.empty(r * c, dtype=torch.float32, device=dev).view((c,) if payload.kind == KIND_ENTRYWISE else (r, c))
                    for r, c in payload.shapes]
-        rows = (ctypes.c_int64 * n)(*[r for r, _ in payload.shapes])
-        cols = (ctypes.c_int64 * n)(*[c for _, c in payload.shapes])
+        rows, cols = _dims(tuple(payload.shapes))
         ptrs = (ctypes.c_void_p * n)(*[o.data_ptr() for o in out])
-        rc = self.lib.atomo_decode(self._h, payload.kind, ctypes.c_void_p(payload.buf.data_ptr()), rows, cols, ptrs, n,
+        rc = self.lib.atomo_decode(self._h, payload.kind, payload.buf.data_ptr(), rows, cols, ptrs, n,
                                    self._stream_ptr(stream))
         self._check(rc, "atomo_decode")
         return list(out)
@@ -480,8 +494,7 @@ class Atomo:
         if out is None:
             out = [torch.empty(r * c, dtype=torch.float32, device=dev).view((c,) if first.kind == KIND_ENTRYWISE else (r, c))
                    for r, c in first.shapes]
-        rows = (ctypes.c_int64 * n)(*[r for r, _ in first.shapes])
-        cols = (ctypes.c_int64 * n)(*[c for _, c in first.shapes])
+        rows, cols = _dims(tuple(first.shapes))
         ptrs = (ctypes.c_void_p * n)(*[o.data_ptr() for o in out])
         pays = (ctypes.c_void_p * len(payloads))(*[p.buf.data_ptr() for p in payloads])
         rc = self.lib.atomo_decode_average(self._h, first.kind, pays, len(payloads), rows, cols, ptrs, n,
@@ -567,7 +580,7 @@ class Atomo:
         return int(up.value), int(re.value)
 
     def set_tridiag_ctas(self, ctas_per_layer: int):
-        """CTAs per layer of the blocked tridiagonal reduction (short sides above 512): 0 = chosen per batch, else 1,
+        """CTAs per layer of the band reduction (short sides above 512): 0 = chosen per batch, else 1,
         2, 4, 8 or 16.  The payload does not depend on it."""
         self._check(self.lib.atomo_set_tridiag_ctas(self._h, int(ctas_per_layer)), "atomo_set_tridiag_ctas")
 
