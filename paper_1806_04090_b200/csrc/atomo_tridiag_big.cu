@@ -22,7 +22,7 @@ namespace {
 constexpr int kVbThreads = 512;
 constexpr int kVbWarps = kVbThreads / 32;
 constexpr int kVbSlots = 16;                 // work-vector sets per layer (phase A: 16 atoms at a time over the layer's CTAs)
-constexpr int kVbMaxCtas = 4;                // CTAs per layer (the kept atoms are dealt to them)
+constexpr int kVbMaxCtas = 16;               // CTAs per layer (the kept atoms are dealt to them)
 constexpr int kVbBatch = 4;                  // atoms per pass over the reflectors
 constexpr int kVbSums = 4 * kVbBatch + 6;    // products summed per group
 constexpr double kVbSameEig = 1.0e-9;        // as on the small route
@@ -190,18 +190,31 @@ __device__ __forceinline__ void vb_chase_back(const float* __restrict__ gV2, con
     const int th = f / (2 * BPT), c = f % (2 * BPT);
     return th * 2 * BPT + (c ^ (BPT == 1 ? (th >> 2) & 1 : th & (2 * BPT - 1)));
   };
+  // this thread's chunks of a sweep: where they go, the last sweep that has them, where they come from (sweep by sweep upwards)
+  constexpr int kMine = (kChunks + THREADS - 1) / THREADS;
+  uint32_t to[kMine];
+  int last[kMine];
+  const float* from[kMine];
+#pragma unroll
+  for (int c = 0; c < kMine; ++c) {
+    const int f = tid + c * THREADS, t = f / 2;
+    to[c] = (uint32_t)__cvta_generic_to_shared(s_ring + place(f));
+    last[c] = f < kChunks ? min(r - 3, r - 3 - 8 * t) : -1;
+    from[c] = gV2 + ((int64_t)(sweeps - 1) * ns + t) * 8 + (f & 1) * 4;
+  }
+  int fill = 0, use = 0;                                       // stages
   auto issue = [&](int j) {                                    // sweep j (none below 0: an empty group keeps the count)
     if (j >= 0) {
-      float4* const dst = s_ring + (size_t)((sweeps - 1 - j) % kBackStages) * kChunks;
-      for (int f = tid; f < kChunks; f += THREADS) {
-        const int t = f / 2;
-        const bool ok = j <= r - 3 && j + 1 + 8 * t <= r - 2;
-        const float* src = ok ? gV2 + ((int64_t)j * ns + t) * 8 + (f & 1) * 4 : gV2;
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + place(f));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+#pragma unroll
+      for (int c = 0; c < kMine; ++c) {
+        const bool ok = j <= last[c];
+        if (kChunks % THREADS == 0 || tid + c * THREADS < kChunks)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[c] + fill * (uint32_t)(kChunks * sizeof(float4))), "l"(ok ? from[c] : gV2), "r"(ok ? 16 : 0) : "memory");
+        from[c] -= (int64_t)ns * 8;
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    fill = fill == kBackStages - 1 ? 0 : fill + 1;
   };
   float x[kW];
 #pragma unroll
@@ -220,7 +233,8 @@ __device__ __forceinline__ void vb_chase_back(const float* __restrict__ gV2, con
         if (lane == 0) in = me == 0 ? (j + 1 < r ? z[j + 1] : 0.0f) : s_edge[(j + 1) & 1][w - 1];
         x[(kW - s) % kW] = in;
       }
-      const float4* const st = s_ring + (size_t)((sweeps - 1 - j) % kBackStages) * kChunks;
+      const float4* const st = s_ring + use * kChunks;
+      use = use == kBackStages - 1 ? 0 : use + 1;
 #pragma unroll
       for (int b = 0; b < BPT; ++b) {
         const float4 u0 = st[place((me * BPT + b) * 2)], u1 = st[place((me * BPT + b) * 2 + 1)];
@@ -377,7 +391,10 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
     }
     for (int b = nb; b < kVbBatch; ++b) for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = 0.0f;
     __syncthreads();
-    vb_chase_back<kVbThreads, 4, kVbBatch>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+    // one atom: a run per thread and a turn of eight sweeps; the turn of 32 that four atoms share the reflectors in is more
+    // code than the instruction cache holds (one of 4096 entries: 9.0 -> 7.3 ms with the rest of the kernel)
+    if (nb == 1) vb_chase_back<kVbThreads, 1, 1>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+    else vb_chase_back<kVbThreads, 4, kVbBatch>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
     if (rp <= 4 * kVbThreads) vb_apply_reflectors<kVbThreads, kVbBatch, 4, true>(gV, ldv, r, rp, nref, nb, s_z, s_part, s_tot);
     else vb_apply_reflectors<kVbThreads, kVbBatch, 8, true>(gV, ldv, r, rp, nref, nb, s_z, s_part, s_tot);
     // normalise and file
@@ -423,7 +440,7 @@ void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, 
   // and the other way round)
   sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(rp_max), st>>>(d_layers, d_big);
   if (rp_max <= kVcMaxRp) return;
-  // larger layers: CTAs per layer (1, 2 or 4; the kept atoms are dealt to them), as many as keep the launch within one wave
+  // larger layers: CTAs per layer (1 to 16; the kept atoms are dealt to them), as many as keep the launch within one wave
   static int sms = 0;
   if (sms == 0) { int dev = 0; if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 1; }
   int per = 1;
