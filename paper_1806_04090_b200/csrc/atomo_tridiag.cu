@@ -301,9 +301,9 @@ constexpr int kBisThreads = 64;           // small CTAs: the warps of a large la
 // round) and rounds, chosen so that the final interval is below 1e-12 of the spectrum's extent: 8 lanes and 13 rounds
 // (9^13 = 2.5e12) where the batch has few eigenvalues and the chain of rounds is what takes the time; 2 lanes and 26
 // rounds (3^26 = 2.5e12) where it has many: half the Sturm counts per eigenvalue, and enough eigenvalues to fill the GPU.
-template <int kBisLanes, int kBisRounds>
-__global__ void __launch_bounds__(kBisThreads) sp_bisect_kernel(const SpLayer* __restrict__ layers, int bis_stride) {
-  constexpr int kBisPerCta = kBisThreads / kBisLanes;
+template <int kBisLanes, int kBisRounds, int THREADS = kBisThreads>
+__global__ void __launch_bounds__(THREADS) sp_bisect_kernel(const SpLayer* __restrict__ layers, int bis_stride) {
+  constexpr int kBisPerCta = THREADS / kBisLanes;
   const SpLayer& L = layers[blockIdx.y];
   if (!L.tri) return;
   const int r = L.r;
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kBisThreads) sp_bisect_kernel(const SpLayer* _
   extern __shared__ __align__(16) double bis_smem[];           // d and e^2, r_max + 8 entries each
   double* const s_d = bis_smem;
   double* const s_e2 = bis_smem + bis_stride;
-  for (int i = tid; i < r + 8; i += kBisThreads) {
+  for (int i = tid; i < r + 8; i += THREADS) {
     s_d[i] = i < r ? L.td_d[i] : kSturmPad;
     const double e = i + 1 < r ? L.td_e[i] : 0.0;
     s_e2[i] = e * e;
@@ -539,6 +539,7 @@ int sp_configure_bisect() {
   const int bytes = (int)(2 * (kMaxShort + 10) * sizeof(double));
   if (cudaFuncSetAttribute(sp_bisect_kernel<1, 41>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
       cudaFuncSetAttribute(sp_bisect_kernel<8, 13>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(sp_bisect_kernel<8, 13, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
       cudaFuncSetAttribute(sp_bisect_kernel<2, 26>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
     cudaGetLastError();
     return 1;
@@ -587,6 +588,10 @@ void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t 
   } else if (n_eigenvalues >= 16384) {
     constexpr int per = kBisThreads / 2;
     sp_bisect_kernel<2, 26><<<dim3((r_max + per - 1) / per, n_layers), kBisThreads, smem, st>>>(d_layers, stride);
+  } else if (r_max > 2048) {
+    // 64 KB of d and e^2 per CTA at 4096 rows: three CTAs per SM, so they have to be larger to fill it (2 x 4096: 2.60 -> 2.11 ms)
+    constexpr int per = 256 / 8;
+    sp_bisect_kernel<8, 13, 256><<<dim3((r_max + per - 1) / per, n_layers), 256, smem, st>>>(d_layers, stride);
   } else {
     constexpr int per = kBisThreads / 8;
     sp_bisect_kernel<8, 13><<<dim3((r_max + per - 1) / per, n_layers), kBisThreads, smem, st>>>(d_layers, stride);
