@@ -43,8 +43,7 @@ struct atomo_ctx {
   size_t ws_bytes = 0;
   uint32_t* h_flag = nullptr;        // pinned: convergence flag / state mirror
   EwLqPart* h_lq = nullptr;          // pinned: results of the l_q sums, written by the GPU
-  uint32_t* ew_words = nullptr;      // device: two sets of barrier counters of the entry-wise encode, the ticket of the l_q sums
-  int ew_set = 0;                    // the set the next launch takes (each launch zeroes the other one)
+  uint32_t* ew_words = nullptr;      // device: barrier counters of the entry-wise encode (zero between launches), the ticket of the l_q sums
   cudaEvent_t ev_sync = nullptr;
   // stage timers: one set of events per API call, a ring of kEvRing sets (a set is read out -- its call is long
   // finished by then -- before it is used again), sums since profiling was switched on
@@ -98,8 +97,8 @@ int fail_cuda(atomo_ctx* ctx, cudaError_t e, const char* what) {
   return ATOMO_ERR_CUDA;
 }
 constexpr int kLqResults = 64;                                 // vectors per round of the l_q sums
-constexpr int kEwSetWords = kEwBatch * kEwBarrierStride;
-constexpr int kEwWords = 2 * kEwSetWords + 32;
+constexpr int kEwBarrierWords = kEwBatch * kEwBarrierStride;
+constexpr int kEwWords = kEwBarrierWords + 32;
 #define CK(call)                                                            \
   do {                                                                      \
     cudaError_t e__ = (call);                                               \
@@ -1070,13 +1069,10 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs
   gh.total_bytes = total; gh.seed = seed; gh.step = step; gh.s = s;
   gh.ew_format = (uint64_t)ctx->ew_format; gh.ew_sat_cap = compact ? (uint64_t)ctx->ew_sat_cap : 0;
   auto fill = [&](auto& B, int first, int count) {
-    uint32_t* const set = ctx->ew_words + ctx->ew_set * kEwSetWords;
-    for (int i = 0; i < count; ++i) { B.v[i] = V[first + i]; B.v[i].barrier = set + i * kEwBarrierStride; }
+    for (int i = 0; i < count; ++i) { B.v[i] = V[first + i]; B.v[i].barrier = ctx->ew_words + i * kEwBarrierStride; }
     B.n = count; B.s = s; B.key = philox_round_keys(PhiloxKey{(uint32_t)seed, (uint32_t)(seed >> 32)});
     B.kind_step = kind_step_word(ATOMO_KIND_ENTRYWISE, step);
     B.begin = begin; B.begin.on = first == 0 ? 1 : 0;
-    ctx->ew_set ^= 1;
-    B.next_barriers = ctx->ew_words + ctx->ew_set * kEwSetWords;
   };
   auto run_two = [&](int l, int solve_ctas) {
     EwBatch<1> B{};
@@ -1098,10 +1094,8 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs
       else { EwBatch<kEwBatch> B{}; fill(B, r.first, r.count); e = launch_ew_encode(B, r.list, st); }
       ++n_launch;
       if (e == (int)cudaErrorCooperativeLaunchTooLarge) {
-        // fewer CTAs fit the GPU at once than the occupancy query promised: the two-kernel form, vector by vector (the
-        // launch that did not happen zeroed no counters)
+        // fewer CTAs fit the GPU at once than the occupancy query promised: the two-kernel form, vector by vector
         cudaGetLastError();
-        CK(cudaMemsetAsync(ctx->ew_words, 0, 2 * kEwSetWords * sizeof(uint32_t), st));
         e = 0;
         for (int l = r.first; l < r.first + r.count && e == 0; ++l) {
           V[l].candidates = 0;
@@ -1153,7 +1147,7 @@ int atomo_lq_budget(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs, doubl
     d_part = A.take<EwLqPart>(max_ctas);
     if (pass == 0) { const int rc = ensure_ws(ctx, A.off + 256); if (rc != ATOMO_OK) return rc; }
   }
-  uint32_t* const ticket = ctx->ew_words + 2 * kEwSetWords;
+  uint32_t* const ticket = ctx->ew_words + kEwBarrierWords;
   // the sums of up to kLqResults vectors arrive in pinned memory; one wait for all of them
   for (int l0 = 0; l0 < n_vecs; l0 += kLqResults) {
     const int n = std::min(n_vecs - l0, kLqResults);

@@ -166,6 +166,14 @@ __device__ __forceinline__ void ew_barrier(const EwVec& v, uint32_t target, EwSh
   }
   __syncthreads();
 }
+// At the end of a CTA: it will not look at the vector's barrier again.  The last CTA of the vector leaves both counters at zero, so
+// every launch that runs finds zeros and leaves zeros: a launch that never happened, a replayed graph or a wait that ran out
+// changes nothing for the next one, and the host keeps no count of launches.  (No fence: nothing is handed on but the counters,
+// and a CTA's last poll has returned before its atomic is issued.)
+__device__ __forceinline__ void ew_leave(const EwVec& v) {
+  if (v.n_ctas == 1 || threadIdx.x != kEwThreads - 1) return;
+  if (atomicAdd(v.barrier + 1, 1u) == (uint32_t)v.n_ctas - 1u) { v.barrier[0] = 0u; v.barrier[1] = 0u; }
+}
 
 // ---- pass 1 -------------------------------------------------------------------------------------------------------
 // Sums in short fp32 runs (16 terms per lane and unit), then fp64.  amax ignores NaN (and the sum keeps it), so "some
@@ -806,7 +814,6 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
   uint32_t* const scratch = ew_smem;
   uint8_t* const code = reinterpret_cast<uint8_t*>(ew_smem + B.scratch_words);
   if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
-  if (blockIdx.x == 0 && tid < kEwBatch) B.next_barriers[tid * kEwBarrierStride] = 0u;   // for the next launch: nobody uses that set now
   if (c.index == 0) {
     ew_write_headers(v, B.begin, vi == 0);
     if (tid == 0) v.state->list_chunks = 0u;               // counted after the barrier
@@ -839,6 +846,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
     }
     __syncthreads();
     ew_pack(v, c, S, code, scratch, sh);
+    ew_leave(v);
     return;
   }
   if (v.candidates) {
@@ -865,6 +873,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
       __syncthreads();
       ew_pack(v, c, S, code, scratch, sh);
     }
+    ew_leave(v);
     return;
   }
   EwBigList big{scratch, 0.0f, 0.0};
@@ -879,6 +888,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
   ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
   __syncthreads();
   ew_pack(v, c, S, code, scratch, sh);
+  ew_leave(v);
 }
 
 // The two-kernel form: the solve leaves its result in the state record; a CTA of the second kernel takes the next chunk of
@@ -891,7 +901,6 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_solve_kernel(const __grid_co
   const int tid = threadIdx.x;
   if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
   if (blockIdx.x == 0) {
-    if (tid < kEwBatch) B.next_barriers[tid * kEwBarrierStride] = 0u;
     ew_write_headers(v, B.begin, true);
     if (tid == 0) { *v.ticket = 0u; v.state->list_chunks = 0u; }
   }
@@ -906,6 +915,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_solve_kernel(const __grid_co
   }, sh);
   if (blockIdx.x == 0 && tid == 0) ew_store_state(v, S);
   if (tid == 0 && sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
+  ew_leave(v);
 }
 
 __global__ void __launch_bounds__(kEwThreads, 1) ew_sample_pack_kernel(const __grid_constant__ EwBatch<1> B) {
