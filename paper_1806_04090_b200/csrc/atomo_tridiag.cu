@@ -103,12 +103,14 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
   __shared__ __align__(16) double s_c2[kTriRows];
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ double s_x0;
+  __shared__ uint32_t s_late;                                 // a thread's wait ran out
   const ClusterCta me = ctas[blockIdx.x];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tri_smem(&s_bar[0])) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tri_smem(&s_bar[1])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_late = 0u;
   }
   for (int i = tid; i < 32 + kTriMaxRp; i += kTriThreads) { s_v[0][i] = s_v[1][i] = s_w[i] = 0.0; }
   for (int i = tid; i < kTriMaxRp; i += kTriThreads) { s_qc[0][i] = s_qc[1][i] = make_double2(0.0, 0.0); }
@@ -145,7 +147,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
     const int q1 = k + 1, q2 = k + 2;
     const bool last = q1 == my_steps;                         // no reflector follows
     const int g_lo = q2 >> 5;                                 // first CTA, and first block of columns, that is still alive
-    if (k >= 0 && !tri_wait(tri_smem(&s_bar[par]), (uint32_t)(k >> 1) & 1u)) { *timeout_flag = 1u; break; }
+    // every thread polls, but the CTA gives up as one (below, where the answer is not waited for): a thread that left alone would
+    // meet the others in different barriers
+    if (k >= 0 && !tri_wait(tri_smem(&s_bar[par]), (uint32_t)(k >> 1) & 1u)) s_late = 1u;
     const double2 qcA = s_qc[par][jA], qcB = s_qc[par][jB];
     const double2 qc1 = s_qc[par][min(q1, kTriMaxRp - 1)];
     // K = beta^2/2 q^T v (v is zero outside the live rows)
@@ -166,6 +170,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
       if (last && r > 1 && tid == ((r - 1) & (kTriThreads - 1))) td_e[r - 2] = r - 1 < kTriThreads ? xA : xB;
     }
     __syncthreads();
+    const bool late = s_late != 0u;
     if (tid == 0 && !last) {
       const uint32_t bytes = (uint32_t)(nc - g_lo) * kTriRows * sizeof(double2);
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tri_smem(&s_bar[nxt])), "r"(bytes) : "memory");
@@ -217,6 +222,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
     }
     __syncthreads();
     const double nx2 = tri_sum8(s_n), x0 = s_x0, c2 = s_c2[4 * w + e_own];
+    if (late) { *timeout_flag = 1u; break; }
     if (last) {                                               // order 1 and 2 as they are: only the last diagonal entry is left
       if (r > 1 && (lane & 7) == 0 && row_lo + e_own == r - 1) td_d[r - 1] = c2;
       break;
