@@ -46,16 +46,16 @@ __device__ __forceinline__ void tc_mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void tc_mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// bounded wait for the phase with the given parity; also gives up when another role has set the abort word
+// bounded wait for the phase with the given parity; also gives up when another role has set the abort word (null: no other role)
 __device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_word) {
   for (int it = 0; it < kTcSpin; ++it) {
     uint32_t ok;
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     if (ok) return true;
-    if ((it & 63) == 63 && *abort_word) return false;
+    if (abort_word != nullptr && (it & 63) == 63 && *abort_word) return false;
   }
-  *abort_word = 1u;
+  if (abort_word != nullptr) *abort_word = 1u;
   return false;
 }
 __device__ __forceinline__ void tc_tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_d = *s_tmem;
 
+  int issued = 0;                                              // (thread 0) stages asked for
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
         tc_mbar_expect_tx(full_bar(s), diag ? kTcTileBytes : 2 * kTcTileBytes);
         tc_tma_load_2d(stage, map, full_bar(s), (kb_lo + kb) * kTcKBlk, ti * kTcTile);
         if (!diag) tc_tma_load_2d(stage + 2 * kTcTileBytes, map, full_bar(s), (kb_lo + kb) * kTcKBlk, tj * kTcTile);
+        issued = kb + 1;
       }
     }
   } else if (warp == 1) {
@@ -203,7 +205,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
     bool ok = true;
     for (int kb = 0; kb < num_kb && ok; ++kb) {
       const int buf = kb & 1;
-      if (!tc_mbar_wait(tfull_bar(buf), (uint32_t)(kb >> 1) & 1u, s_abort)) { ok = false; break; }
+      // (a warp stays together: the loads below are the whole warp's)
+      ok = __all_sync(0xffffffffu, tc_mbar_wait(tfull_bar(buf), (uint32_t)(kb >> 1) & 1u, s_abort)) != 0;
+      if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
       for (int c0 = 0; c0 < kTcTile; c0 += 32) {
@@ -225,6 +229,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       tc_mbar_arrive(tempty_bar(buf));
     }
+    // the four warps meet, and what they do next depends on the abort word alone: it is set before a warp whose wait ran out gets
+    // here, and if no wait of theirs ran out then every other role's have been answered too
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+    ok = *s_abort == 0u;
     // Epilogue.  The stage buffers are free now (every load has landed and every MMA has completed): the tile goes
     // through shared memory (row stride 129 floats, conflict-free both ways) so that both triangles of A are written
     // with consecutive lanes on consecutive addresses.
@@ -273,6 +281,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (*s_abort) {                                              // given up: the copies on their way land first (bounded, too)
+    if (tid == 0)
+      for (int kb = max(0, issued - kTcStages); kb < issued; ++kb) tc_mbar_wait(full_bar(kb % kTcStages), (uint32_t)(kb / kTcStages) & 1u, nullptr);
+    __syncthreads();
+  }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(kTcTmemCols) : "memory");

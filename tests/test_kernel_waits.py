@@ -25,3 +25,14 @@ def test_tridiagonal_reduction_gives_up_as_a_block():
     assert after.index("__syncthreads()") < read.start()
     assert "break" not in after[:read.start()] and "return" not in after[:read.start()]
     assert re.search(r"if \(%s\) \{[^}]*break;" % read.group(1), after[read.start():])
+
+
+def test_gram_drain_gives_up_as_a_group():
+    src = _source("atomo_tc.cu")
+    drain = src[src.index("tfull_bar(buf), (uint32_t)(kb >> 1) & 1u"):]
+    # a warp decides as one (the TMEM loads are warp-wide) ...
+    assert "__all_sync(0xffffffffu, tc_mbar_wait(tfull_bar" in src
+    # ... and the four warps meet before the abort word says what they do next
+    group = drain.index('"bar.sync 2, 128;"')
+    decide = drain.index("ok = *s_abort == 0u;")
+    assert group < decide < drain.index("bool write_tile = ok;")
