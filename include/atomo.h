@@ -190,7 +190,9 @@ int atomo_set_entrywise_format(atomo_ctx* ctx, int32_t format, int64_t sat_cap);
  * exact keep decision (the same integer comparison) is taken on the list and the vector is read once.  Otherwise a CTA
  * reads its part a second time.  Vectors that do not fit take the two-kernel form.  two_kernels = 1: always a solve kernel
  * followed by a sample / pack kernel whose chunks are handed out by ticket.  two_kernels = 2: the one-kernel form without
- * the list.  Payloads, masks and decoded gradients are bit-identical in all forms.  Other values:
+ * the list.  In every form a call gives the same bits each time.  The forms take the same decisions by the same comparison and
+ * differ only in the order of their fp64 sums, so that payloads, masks and decoded gradients are the same in all of them too unless
+ * a sum lies within an fp64 rounding of where its fp32 result would round the other way.  Other values:
  * ATOMO_ERR_INVALID_ARG.     */
 int atomo_set_entrywise_launch(atomo_ctx* ctx, int32_t two_kernels);
 /* Test introspection, for vector `vec` of the context's last atomo_encode_entrywise call: the number of chunks (CTAs)

@@ -36,7 +36,7 @@ constexpr int kEwUnits = 8;                   // units per tile: what a warp tak
 constexpr int kEwBlocks = kEwTile / 4;        // blocks (code bytes) per tile
 constexpr int kEwPrefixes = kEwTile / 32;     // list form: prefix words per tile
 constexpr int kEwRegTiles = kEwWarps / kEwUnits;   // chunks of at most this many tiles stay in registers: a unit per warp
-constexpr int kEwBig = 8192;                  // entries of the list of runs with atoms that may saturate
+constexpr int kEwBig = 8;                     // a thread's entries of the list of runs with atoms that may saturate
 constexpr int kEwStage = 256;                 // kept atoms per staging window (one per warp) of the compaction
 constexpr uint32_t kEwPollLimit = 1u << 22;   // polls of a bounded wait (with a sleep between them)
 constexpr uint64_t kFlagReady = 1ull << 63;
@@ -130,7 +130,8 @@ struct EwShared {                 // static shared memory of the encode and solv
   float mx[kEwWarps], est[kEwWarps];
   uint32_t cnt[kEwWarps];
   unsigned long long scan[kEwWarps], before[kEwWarps];
-  uint32_t n_big, stop, fail, next_unit;
+  uint32_t big[kEwWarps];       // runs on the warps' lists, closed up
+  uint32_t big_over, stop, fail, next_unit;
 };
 
 // block reduction in a fixed order, result valid in every thread
@@ -199,16 +200,24 @@ __device__ __forceinline__ double ew_estimate_l1(const EwVec& v, const EwChunk& 
 // the listed runs of 100 M Laplace entries at s = 10 % are 0.5 % of it).  The bound is 0.8 l1_est / s with l1_est the sum over
 // the chunk's first tiles scaled to the vector; the rounds lower the threshold a little (there: by half a per cent).  A round
 // forms the listed runs anew without the saturated atoms, exactly as a round over the whole chunk would.
+// Every thread lists its own runs in slots of its own and the warps close them up before the first round, so that the sums have a
+// fixed order; a thread without a slot left sends the rounds to memory (a chunk of up to 32 tiles has a slot for every run).
+// (One list of the CTA, filled through an atomic counter and dealt to the threads by position, gave fp64 sums that depended on
+// which warp came first.  25 M elements at 13 %: 94.6 us with it, 96.9 so, 99.0 where a round goes through a thread's own slots; a
+// list per warp, placed by ballot, doubled the spills of this pass: 100 M elements at 10 % 341 -> 358 us, so 342.)
+constexpr uint32_t kEwClosed = 0xFFFFFFFFu;
 struct EwBigList {
-  uint32_t* run;                // [kEwBig] the run's first block inside the chunk, shared memory
+  uint32_t* run;                // [kEwBig][kEwThreads] the runs' first blocks inside the chunk, shared memory
+  uint32_t n;                   // this thread's; kEwClosed: closed up
   float lo;                     // runs with an atom above lo are listed; inf: no list
   double rest;                  // this thread's sum over the runs not listed
 };
 
-// pass 1 with that list; the caller has zeroed sh.n_big
+// pass 1 with that list; the caller has zeroed sh.big_over
 __device__ __forceinline__ EwAcc ew_pass_big(const EwVec& v, const EwChunk& c, const double s, EwBigList& B, EwShared& sh) {
   double sum = 0.0, rest = 0.0;
   float amax = 0.0f;
+  uint32_t at = threadIdx.x;
   float4 x[2][4];
   ew_load_ahead(v, c, x);
   {
@@ -221,13 +230,12 @@ __device__ __forceinline__ EwAcc ew_pass_big(const EwVec& v, const EwChunk& c, c
     amax = fmaxf(amax, m);
     sum += (double)fsum;
     if (!(m > B.lo)) rest += (double)fsum;
-    else if (*(volatile uint32_t*)&sh.n_big <= (uint32_t)kEwBig) {       // (a list that overflowed is not used: no more appends)
-      const uint32_t at = atomicAdd(&sh.n_big, 1u);
-      if (at < (uint32_t)kEwBig) B.run[at] = blk;
-    }
+    else if (at < (uint32_t)(kEwBig * kEwThreads)) { B.run[at] = blk; at += kEwThreads; }
+    else sh.big_over = 1u;
     fsum = 0.0f; m = 0.0f;
   });
   B.rest = rest;
+  B.n = at / kEwThreads;
   return EwAcc{sum, amax, 0u};
 }
 // one water-filling round over the chunk: unsaturated sum and saturated count at threshold theta, from memory
@@ -244,11 +252,45 @@ __device__ __forceinline__ EwAcc ew_round_memory(const EwVec& v, const EwChunk& 
   ew_for_units(v, c, x, [&](uint32_t, const float4& y) { ew_round_sums(y, theta, fsum, acc.cnt); }, [&](uint32_t) { acc.sum += (double)fsum; fsum = 0.0f; });
   return acc;
 }
-// ... and from the list, where it holds every run with an atom above theta
-__device__ __forceinline__ EwAcc ew_round_list(const EwVec& v, const EwChunk& c, const EwBigList& B, const uint32_t n_big, const float theta) {
+// The warp's lists in place, row by row, without the gaps (an entry never moves past one that is still to be read): entry p of the
+// warp is in row p / 32, column p % 32 of its part.  Returns their number.
+__device__ __forceinline__ uint32_t ew_close_up(uint32_t* const mine, const uint32_t n_mine, const int lane) {
+  const uint32_t rows = __reduce_max_sync(0xffffffffu, n_mine);
+  uint32_t total = 0;
+  for (uint32_t e = 0; e < rows; ++e) {
+    const bool have = e < n_mine;
+    const uint32_t b = have ? mine[e * kEwThreads + lane] : 0u, votes = __ballot_sync(0xffffffffu, have);
+    const uint32_t p = total + __popc(votes & ((1u << lane) - 1u));
+    __syncwarp();
+    if (have) mine[(p >> 5) * kEwThreads + (p & 31u)] = b;
+    total += __popc(votes);
+  }
+  __syncwarp();
+  return total;
+}
+// ... and from the list, where it holds every run with an atom above theta: run i of all the warps' lists one after the other goes to
+// thread i (mod the CTA).  Called by every thread of the CTA.
+__device__ __forceinline__ EwAcc ew_round_list(const EwVec& v, const EwChunk& c, EwBigList& B, const float theta, EwShared& sh) {
   EwAcc acc{B.rest, 0.0f, 0u};
-  for (uint32_t i = threadIdx.x; i < n_big; i += kEwThreads) {
-    const int64_t base = c.beg + 4 * (int64_t)B.run[i];
+  const int w = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
+  if (B.n != kEwClosed) {
+    const uint32_t n = ew_close_up(B.run + w * kWarp, B.n, lane);
+    if (lane == 0) sh.big[w] = n;
+    B.n = kEwClosed;
+    __syncthreads();
+  }
+  uint32_t upto = sh.big[lane];                            // lane: runs of the warps up to this one
+#pragma unroll
+  for (int q = 1; q < kWarp; q <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, upto, q); if (lane >= q) upto += t; }
+  const uint32_t total = __shfl_sync(0xffffffffu, upto, kWarp - 1);
+  for (uint32_t i0 = w * kWarp; i0 < total; i0 += kEwThreads) {
+    const uint32_t i = i0 + lane;
+    int of = 0;                                            // the warp whose list holds it
+#pragma unroll
+    for (int q = kWarp / 2; q > 0; q >>= 1) if (__shfl_sync(0xffffffffu, upto, of + q - 1) <= i) of += q;
+    const uint32_t before = __shfl_sync(0xffffffffu, upto, max(of - 1, 0)), e = i - (of > 0 ? before : 0u);
+    if (i >= total) continue;
+    const int64_t base = c.beg + 4 * (int64_t)B.run[(e >> 5) * kEwThreads + of * kWarp + (e & 31u)];
     float4 x[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -508,25 +550,14 @@ __device__ __forceinline__ void ew_decide_memory(const EwVec& v, const EwChunk& 
     unit = next;
   }
 }
-// pass 2 on the candidate blocks alone; the code bytes start at zero.  A warp first closes up its lanes' lists in place, row by
-// row (an entry never moves past one that is still to be read), so that every lane decides on the same number of blocks: the
-// fullest lane has three times the average.  What was decided on a block goes back to its place: code byte << 24 | block inside
+// pass 2 on the candidate blocks alone; the code bytes start at zero.  A warp first closes up its lanes' lists, so that every lane
+// decides on the same number of blocks: the fullest lane has three times the average.  What was decided on a block goes back to its place: code byte << 24 | block inside
 // the chunk.  Returns the warp's number of blocks.
 __device__ __forceinline__ uint32_t ew_decide_list(const EwVec& v, const EwChunk& c, const EwDecide& d, const PhiloxRoundKeys& key,
                                                    const uint32_t kind_step, const EwCands& C, uint8_t* __restrict__ code) {
   const int lane = threadIdx.x % kWarp;
   uint32_t* const mine = C.blk + (threadIdx.x - lane);     // entry p of the warp: row p / 32, column p % 32
-  const uint32_t n_c = ew_cand_count(C), blk_beg = (uint32_t)(c.beg >> 2), rows = __reduce_max_sync(0xffffffffu, n_c);
-  uint32_t total = 0;
-  for (uint32_t e = 0; e < rows; ++e) {
-    const bool have = e < n_c;
-    const uint32_t b = have ? mine[e * kEwThreads + lane] : 0u, votes = __ballot_sync(0xffffffffu, have);
-    const uint32_t p = total + __popc(votes & ((1u << lane) - 1u));
-    __syncwarp();
-    if (have) mine[(p >> 5) * kEwThreads + (p & 31u)] = b;
-    total += __popc(votes);
-  }
-  __syncwarp();
+  const uint32_t blk_beg = (uint32_t)(c.beg >> 2), total = ew_close_up(mine, ew_cand_count(C), lane);
   for (uint32_t e0 = lane; e0 < total; e0 += 4 * kWarp) {
     uint32_t b[4];
     float4 x[4];
@@ -813,7 +844,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
   EwChunk c = ew_chunk(v, blockIdx.x - (uint32_t)v.cta0);
   uint32_t* const scratch = ew_smem;
   uint8_t* const code = reinterpret_cast<uint8_t*>(ew_smem + B.scratch_words);
-  if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
+  if (tid == 0) { sh.big_over = 0u; sh.stop = 0u; sh.fail = 0u; }
   if (c.index == 0) {
     ew_write_headers(v, B.begin, vi == 0);
     if (tid == 0) v.state->list_chunks = 0u;               // counted after the barrier
@@ -876,13 +907,13 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
     ew_leave(v);
     return;
   }
-  EwBigList big{scratch, 0.0f, 0.0};
+  EwBigList big{scratch, 0u, 0.0f, 0.0};
   const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
   c = ew_chunk(v, ew_opaque(blockIdx.x) - (uint32_t)v.cta0);
   const float lo = big.lo;
   const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
-    const uint32_t nb = *(volatile uint32_t*)&sh.n_big;    // complete: a barrier has passed since the last append
-    return nb <= (uint32_t)kEwBig && theta >= lo ? ew_round_list(v, c, big, nb, theta) : ew_round_memory(v, c, theta);
+    // (a barrier has passed since the pass)
+    return *(volatile uint32_t*)&sh.big_over == 0u && theta >= lo ? ew_round_list(v, c, big, theta, sh) : ew_round_memory(v, c, theta);
   }, sh);
   if (c.index == 0 && tid == 0) ew_store_state(v, S);
   ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
@@ -895,23 +926,22 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
 // consecutive tiles by ticket, so that every chunk it will wait for is already running, however many waves the grid takes.
 __global__ void __launch_bounds__(kEwThreads, 1) ew_solve_kernel(const __grid_constant__ EwBatch<1> B, int n_pack_chunks) {
   __shared__ EwShared sh;
-  __shared__ uint32_t s_big[kEwBig];
+  __shared__ uint32_t s_big[kEwBig * kEwThreads];
   const EwVec& v = B.v[0];
   const EwChunk c = ew_chunk(v, blockIdx.x);
   const int tid = threadIdx.x;
-  if (tid == 0) { sh.n_big = 0u; sh.stop = 0u; sh.fail = 0u; }
+  if (tid == 0) { sh.big_over = 0u; sh.stop = 0u; sh.fail = 0u; }
   if (blockIdx.x == 0) {
     ew_write_headers(v, B.begin, true);
     if (tid == 0) { *v.ticket = 0u; v.state->list_chunks = 0u; }
   }
   for (int i = blockIdx.x * kEwThreads + tid; i < n_pack_chunks; i += gridDim.x * kEwThreads) v.chunk_status[i] = 0ull;   // for the second kernel
   __syncthreads();
-  EwBigList big{s_big, 0.0f, 0.0};
+  EwBigList big{s_big, 0u, 0.0f, 0.0};
   const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
   const float lo = big.lo;
   const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
-    const uint32_t nb = *(volatile uint32_t*)&sh.n_big;
-    return nb <= (uint32_t)kEwBig && theta >= lo ? ew_round_list(v, c, big, nb, theta) : ew_round_memory(v, c, theta);
+    return *(volatile uint32_t*)&sh.big_over == 0u && theta >= lo ? ew_round_list(v, c, big, theta, sh) : ew_round_memory(v, c, theta);
   }, sh);
   if (blockIdx.x == 0 && tid == 0) ew_store_state(v, S);
   if (tid == 0 && sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
@@ -1203,8 +1233,8 @@ int ew_sms() {
   return sms;
 }
 // the slots of the candidate list; else the staging windows (or the list of runs with large atoms)
-size_t ew_scratch_bytes(bool list) { return list ? (size_t)kEwCandBytes : std::max((size_t)kEwWarps * kEwStage * sizeof(uint16_t), kEwBig * sizeof(uint32_t)); }
-static_assert(kEwCandBytes >= kEwWarps * kEwStage * 2 && kEwCandBytes >= kEwBig * 4, "the scratch area serves in turn");
+size_t ew_scratch_bytes(bool list) { return list ? (size_t)kEwCandBytes : std::max((size_t)kEwWarps * kEwStage * sizeof(uint16_t), (size_t)kEwBig * kEwThreads * sizeof(uint32_t)); }
+static_assert(kEwCandBytes >= kEwWarps * kEwStage * 2 && kEwCandBytes >= kEwBig * kEwThreads * 4, "the scratch area serves in turn");
 size_t ew_dyn_bytes(int tiles, bool list) {
   return ew_scratch_bytes(list) + (size_t)tiles * (kEwBlocks + (list ? kEwPrefixes * sizeof(uint32_t) : 0));
 }
