@@ -478,7 +478,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // ---- host descriptors, tiles, workspace carving (two passes: size, then pointers) ----
   std::vector<SpLayer> L(n_layers);
   std::vector<int> tc_layers;
-  std::vector<TileRef> gram_tiles, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles;
+  std::vector<TileRef> gram_tiles, gram_parts, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles;
   const int map_bytes = sp_tc_map_bytes();
   std::vector<uint8_t> maps_blob((size_t)n_layers * map_bytes, 0);
   int chol_panels = 0;
@@ -499,7 +499,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     k_cap_max = std::max(k_cap_max, (int)d.k_cap);
     r_max = std::max(r_max, d.r); rp_max = std::max(rp_max, d.rp);
     const int gt = (d.r + 63) / 64;
-    d.tc = 0; d.gram_split = 1;
+    d.tc = 0; d.gram_split = 1; d.gram_part_len = d.L;
     // The tensor core's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the
     // fp32 FMA kernel, whose sums round to nearest (their Gram matrix is a small part of their cost)
@@ -509,7 +509,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       tc_layers.push_back(l);
     } else {
       d.gram_split = given ? 1 : sp_gram_split(d.r, d.L);
-      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.gram_split; ++c) gram_tiles.push_back({l, a, b, c});
+      d.gram_part_len = sp_gram_part(d.r, d.L);
+      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.gram_split; ++c) (d.r > 1024 ? gram_tiles : gram_parts).push_back({l, a, b, c});
     }
     for (int p = 0; p < d.nb / 2; ++p) block_pairs.push_back({l, p, 0, 0});
     row_floats_max = std::max(row_floats_max, d.ldx); steps_max = std::max(steps_max, d.nb - 1);
@@ -536,6 +537,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     if (d.refine)
       for (int a = 0; a < gt; ++a) for (int b = 0; b < d.refine_tiles; ++b) refine_tiles.push_back({l, a, b, 0});
   }
+  gram_tiles.insert(gram_tiles.end(), gram_parts.begin(), gram_parts.end());   // (an instance of the kernel each)
   // Tridiagonal routes first: eigenvalues of every atom from T = Q^T A Q, vectors for the kept atoms only -- in the
   // registers of a cluster for short sides up to 512, in two stages with A in global memory above (no per-atom refinement,
   // no request for the whole short-side basis).  Otherwise the Jacobi routes, the cluster form first.
@@ -831,7 +833,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     launch_sp_load_svd(d_layers, n_layers, d_given, d_given + n_layers, st);
   } else {
   if (ctx->eig_mode == 0) launch_sp_init(d_layers, n_layers, nullptr, 0, st);   // the identity half of [A | I]
-  launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), st);
+  launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), (int)gram_parts.size(), st);
   launch_sp_gram_tc(d_layers, d_maps, d_tc, (int)tc_tiles.size(), d_flag + 1, st);
   launch_sp_scale(d_layers, n_layers, r_max, st);
   }

@@ -92,7 +92,8 @@ struct SpLayer {
   int tc;                      // Gram matrix came from the tensor-core kernel (see sp_scale_kernel)
   int gram_split;              // Gram matrix: CTAs per output tile (parts of the K range), 1 = no split
   float* gram_part;            // [tiles][gram_split][128 x 128] partial tiles (column-major) when gram_split > 1
-  double* gram_sums;           // FMA kernel: [tiles][gram_split][64 x 64] partial tiles
+  int gram_part_len;           // FMA kernel: length of a part of the K range
+  double* gram_sums;           // FMA kernel: [tiles][gram_split][16][threads that hold entries] partial tiles
   uint32_t* gram_ticket;       // [tiles] parts finished; zeroed per call
   int refine, refine_tiles;    // singular values from the projection norms; tiles along the long side
   float* row_inv;              // rp: 1 / norm of each short-side vector as stored in X
@@ -128,9 +129,10 @@ struct TileRef { int32_t layer, a, b, c; };
 void launch_sp_begin(uint8_t* pay, const atomo_payload_header& gh, const atomo_layer_header* d_tmpl, int n_layers,
                      uint32_t* d_flags, cudaStream_t st);
 void launch_sp_init(const SpLayer* d_layers, int n_layers, const TileRef* d_diag_tiles, int n_diag_tiles, cudaStream_t st);
-int sp_gram_split(int r, int len);                               // FMA kernel: parts of the K range, doubles for their sums
+int sp_gram_part(int r, int len);                                // FMA kernel: length of a part of the K range, parts, doubles for their sums
+int sp_gram_split(int r, int len);
 int64_t sp_gram_sums(int r, int split);
-void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
+void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, int n_parts, cudaStream_t st);
 void launch_sp_scale(const SpLayer* d_layers, int n_layers, int r_max, cudaStream_t st);   // trace, then scaling
 void launch_sp_load_svd(const SpLayer* d_layers, int n_layers, const float* const* d_sigma, const float* const* d_vecs,
                         cudaStream_t st);                                       // a decomposition given by the caller

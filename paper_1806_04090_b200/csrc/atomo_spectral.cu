@@ -42,17 +42,28 @@ void launch_sp_init(const SpLayer* d_layers, int n_layers, const TileRef*, int, 
 // =================================================================================================
 // Gram matrix of the short side.  64 x 64 output tile per CTA, 16 x 16 threads, 4 x 4 per thread.
 // Short-side vector i is row i of G (rows <= cols) or column i of G (rows > cols).  A layer with a short side of up to 1024 has
-// its K range cut into parts (ref.c: which part) of 512, or 2048 above 256, where they have more tiles (a 16384 x 18 layer was one CTA walking over 16384 rows: 1340 -> 235 us for a set with
-// some); above there are tiles enough, and the parts' sums would cost more than they bring.
+// its K range cut into parts (ref.c: which part) of 512, or 2048 above 256, where they have more tiles (a 16384 x 18 layer was
+// one CTA walking over 16384 rows: 1340 -> 235 us for a set with some); above there are tiles enough, and the parts' sums would
+// cost more than they bring.  A layer gets at most kGramCtas CTAs, four per SM: more fill no idle SM, and the parts' sums, of which
+// only the short side's own entries are kept, would outgrow the gradient (64 bytes per element of a 1 x n layer).  The parts
+// depend on the layer alone, so that its sums do not change with the batch.
 // =================================================================================================
-constexpr int kGramTile = 64, kGramK = 16;
-__host__ __device__ inline int gram_part(int r) { return r <= 256 ? 512 : 2048; }
-int sp_gram_split(int r, int len) { return r <= 1024 ? (len + gram_part(r) - 1) / gram_part(r) : 1; }
+constexpr int kGramTile = 64, kGramK = 16, kGramCtas = 4 * 148;
+int sp_gram_part(int r, int len) {
+  const int gt = (r + kGramTile - 1) / kGramTile, most = std::max(1, kGramCtas / (gt * (gt + 1) / 2)), part = r <= 256 ? 512 : 2048;
+  if (r > 1024) return len;
+  const int64_t even = ((int64_t)len + most - 1) / most;
+  return (int)std::max<int64_t>(part, (even + 31) / 32 * 32);           // whole fp32 runs of 32 products
+}
+int sp_gram_split(int r, int len) { return (int)(((int64_t)len + sp_gram_part(r, len) - 1) / sp_gram_part(r, len)); }
 int64_t sp_gram_sums(int r, int split) {
-  const int64_t gt = (r + kGramTile - 1) / kGramTile;
-  return split > 1 ? gt * (gt + 1) / 2 * split * kGramTile * kGramTile : 0;
+  const int64_t gt = (r + kGramTile - 1) / kGramTile, side = std::min((r + 3) / 4, 16);   // threads along a tile's side that hold entries
+  return split > 1 ? gt * (gt + 1) / 2 * split * side * side * 16 : 0;
 }
 
+// kParts: short sides up to 1024, whose K range may be cut.  Larger layers have an instance of their own: with the code that adds
+// parts up in the same kernel, the loop took 6.9 ms on two layers of 4096 x 4096, without it 6.5.
+template <bool kParts>
 __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict__ layers,
                                                       const TileRef* __restrict__ tiles) {
   __shared__ __align__(16) float As[kGramK][kGramTile + 4];
@@ -63,10 +74,9 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
   const bool diag = ref.a == ref.b;
   const float* __restrict__ G = L.G;
   const int64_t ld = L.ld;
-  const int r = L.r, len = L.L, n_split = L.gram_split;
+  const int r = L.r, len = L.L;
   const bool tall = L.tall;
   const int t = threadIdx.x, ty = t / 16, tx = t % 16;
-  __shared__ bool s_last;
   float acc[4][4];
   double acc64[4][4];
 #pragma unroll
@@ -74,8 +84,8 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) { acc[a][b] = 0.0f; acc64[a][b] = 0.0; }
 
-  // the K range of a tile is cut into parts of kGramPart where a layer has few tiles
-  const int c_lo = n_split > 1 ? ref.c * gram_part(r) : 0, c_hi = n_split > 1 ? min(len, c_lo + gram_part(r)) : len;
+  // the K range of a tile is cut into parts where a layer has few tiles
+  const int c_lo = kParts ? ref.c * L.gram_part_len : 0, c_hi = kParts ? c_lo + min(len - c_lo, L.gram_part_len) : len;
   // this thread's entries of the next stage, fetched while the stage before is multiplied
   const int row = tall ? t / 16 : t / 4, col = (tall ? t % 16 : t % 4) * 4;
   float fa[4], fb[4];
@@ -122,12 +132,18 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
   for (int p = 0; p < 4; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc64[p][q] += (double)acc[p][q];
-  if (n_split > 1) {                                          // the last part to finish adds them up, in order
+  __shared__ bool s_last;
+  if (kParts && L.gram_split > 1) {                           // the last part to finish adds them up, in order
+    const int n_split = L.gram_split;
     const int gt = (r + kGramTile - 1) / kGramTile, tile = ref.a * gt - ref.a * (ref.a - 1) / 2 + ref.b - ref.a;
-    double* const parts = L.gram_sums + (int64_t)tile * n_split * (kGramTile * kGramTile);
-    double* const mine = parts + (int64_t)ref.c * (kGramTile * kGramTile) + t;
+    const int side = min((r + 3) / 4, 16), n_t = side * side; // threads whose 4 x 4 entries hold some of the matrix (short sides below 64: not all)
+    const bool holds = ty < side && tx < side;
+    double* const parts = L.gram_sums + (int64_t)tile * n_split * (16 * n_t) + ty * side + tx;
+    double* const mine = parts + (int64_t)ref.c * (16 * n_t);
+    if (holds) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) mine[e * 256] = acc64[e / 4][e % 4];
+      for (int e = 0; e < 16; ++e) mine[e * n_t] = acc64[e / 4][e % 4];
+    }
     __threadfence();
     __syncthreads();
     if (t == 0) s_last = atomicAdd(L.gram_ticket + tile, 1u) == (uint32_t)(n_split - 1);
@@ -136,10 +152,10 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
     __threadfence();
 #pragma unroll
     for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] = 0.0;
-    for (int s = 0; s < n_split; ++s) {
-      const double* part = parts + (int64_t)s * (kGramTile * kGramTile) + t;
+    for (int s = 0; s < n_split && holds; ++s) {
+      const double* part = parts + (int64_t)s * (16 * n_t);
 #pragma unroll
-      for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] += __ldcg(part + e * 256);
+      for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] += __ldcg(part + e * n_t);
     }
   }
   const int64_t lda = L.lda;
@@ -156,8 +172,10 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
     }
 }
 
-void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, cudaStream_t st) {
-  if (n_tiles > 0) sp_gram_kernel<<<n_tiles, 256, 0, st>>>(d_layers, d_tiles);
+// d_tiles: n_tiles tiles, the last n_parts of them of short sides up to 1024 (or parts of such)
+void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, int n_parts, cudaStream_t st) {
+  if (n_tiles > n_parts) sp_gram_kernel<false><<<n_tiles - n_parts, 256, 0, st>>>(d_layers, d_tiles);
+  if (n_parts > 0) sp_gram_kernel<true><<<n_parts, 256, 0, st>>>(d_layers, d_tiles + (n_tiles - n_parts));
 }
 
 // =================================================================================================
