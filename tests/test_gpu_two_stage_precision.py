@@ -1,0 +1,44 @@
+"""What the two-stage route (short sides above 512) adds to the rounding of its inputs, against 64 bits, on the spectra where it shows:
+a broad noise bulk with little above it.  The bars are 1.5 times what the one-stage reduction that was here before it measured on
+the same matrices (blocked Householder form, one rounding of the matrix per 32 columns)."""
+import math
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(m, n, seed):
+    """16 directions with singular values 1 / i under noise of four times their norm"""
+    import torch
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(seed)
+    sigma = torch.arange(1, 17, dtype=torch.float32, device=dev) ** -1.0
+    u = torch.randn(m, 16, device=dev, generator=gen) / math.sqrt(m)
+    v = torch.randn(n, 16, device=dev, generator=gen) / math.sqrt(n)
+    g = torch.randn(m, n, device=dev, generator=gen)
+    g *= 4.0 * float(torch.linalg.norm(sigma)) / math.sqrt(m * n)
+    return g.addmm_(u * sigma, v.T)
+
+
+@pytest.fixture(scope="module")
+def atomo():
+    from paper_1806_04090_b200 import api
+    a = api.Atomo(0)
+    yield a
+    a.close()
+
+
+# nearly square: the smallest singular values are a few thousandths of the largest and magnify what reached the matrix
+@pytest.mark.parametrize("m,n,bar", [(2000, 2048, 9e-8), (3000, 3100, 8e-8)])
+def test_singular_values(atomo, m, n, bar):
+    import torch
+    G = _layer(m, n, m + 1)
+    pay, dbg = atomo.atomo_encode_spectral([G], 8.0, 5, step=1, k_cap=64, debug=True)
+    assert pay.headers()[1][0].status == 0
+    want = torch.linalg.eigvalsh(G.double() @ G.double().T).clamp(min=0).sqrt().flip(0)
+    got = torch.from_numpy(dbg.layer_sigma(0, m)).to(want)
+    err = float((got - want).norm() / want.norm())
+    print(f"{m} x {n}: sigma relative l2 error {err:.2e}")
+    assert err <= bar
