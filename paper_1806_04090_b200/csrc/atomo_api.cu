@@ -752,6 +752,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.td_ldv = (d.r + 3) / 4 * 4;
       d.td_V = A.take<float>(d.tri ? (size_t)d.r * d.td_ldv : 0);
       d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);
+      d.tb_z = A.take<double>(d.tri == 2 && d.rp > 1024 ? (size_t)d.k_cap * d.rp : 0);
       {
         const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
         d.bd_UW = A.take<float>(on * rows * 2 * kBandWidth);
@@ -760,7 +761,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.bd_S = A.take<double>(on * 3 * kBandWidth * kBandWidth);
         d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
-        d.bd_V2 = A.take<float>(on * d.r * sp_band_steps(d.r) * kBandWidth);
+        d.bd_T = A.take<double>(on * sp_band_steps(d.r) * kBandWidth * kBandWidth);
+        d.bd_V2 = A.take<double>(on * d.r * sp_band_steps(d.r) * kBandWidth);
       }
       d.chol_dd = A.take<float>(32 * 32 + 32);
       d.row_inv = A.take<float>(d.rp);
@@ -946,7 +948,9 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   stage_begin(ctx, ATOMO_STAGE_BACKPROJECT, st);
   if (tri_form) {                                                   // short-side vectors of the kept atoms
     if (any_small) launch_sp_eigvec(d_layers, n_layers, rp_max_small, st);
-    launch_sp_eigvec_big(d_layers, d_big, (int)big_layers.size(), rp_max, st);
+    int rps = 0;
+    for (int l : big_layers) rps |= L[l].rp <= 1024 ? 1 : L[l].rp <= 2048 ? 2 : 4;
+    launch_sp_eigvec_big(d_layers, d_big, (int)big_layers.size(), rps, st);
   }
   launch_sp_backproject(d_layers, d_bp, (int)bp_tiles.size(), std::max(r_max_tall, 1), st);
   launch_sp_finish_atoms(d_layers, n_layers, k_cap_max, st);

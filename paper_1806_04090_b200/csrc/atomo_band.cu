@@ -9,8 +9,8 @@
 //                    side of 1024, a cluster above), all sweeps in flight at once.
 //
 // Then the eigenvalues of T by bisection and vectors for the kept atoms only, as on the small route; a vector of T goes
-// through the chase's reflectors (sp_chase_back, used by the vector kernels of atomo_tridiag_big.cu) and then through the
-// panels' (unit vectors u, H = I - 2 u u^T, rows of td_V).
+// through the chase's reflectors and then through the panels' (I - U T U^T, the columns of U as rows of td_V) in the vector
+// kernels of atomo_tridiag_big.cu.
 //
 // Precision: the matrix, the panel vectors U and W and the panel itself are fp32; products run in fp32 over 32 terms and are
 // added up in fp64; panel dots, scalars and the whole chase are fp64.  Q1 is applied as I - U T U^T with T formed from the
@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   double* const gPart = L.bd_part; double* const gS = L.bd_S; double* const gB = L.bd_band;
   double* const gG = L.bd_G; double* const gM = L.bd_M;
   float* const gV = L.td_V; const int64_t ldv = L.td_ldv;
+  double* const gT = L.bd_T;
   float* const s_u = band_smem;                              // [r][8] this panel's U, by row
   float* const s_ring = band_smem + (size_t)(r + kGroup) * 8; // [warps][STAGES] groups of columns on their way
   if (tid == 0) sh.fail = 0u;
@@ -506,6 +507,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
 #pragma unroll
       for (int q = 0; q < 8; ++q) t = fma(sh.S[a][q], sh.T[q][b], t);
       sh.Y[a][b] = t;
+      if (g == 0) gT[(int64_t)(c / kBw) * 64 + tid] = sh.T[a][b];   // for the back-transformation, as the reflectors' rows below
     }
     __syncthreads();
     if (tid < 64) {                                          // X = -1/2 T^T S T
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(
   const int tid = threadIdx.x, lane = tid % 32;
   const int r = L.r;
   const double* const gB = L.bd_band;
-  float* const gV2 = L.bd_V2;
+  double* const gV2 = L.bd_V2;
   const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that gV2 has room for
   const int col0 = rank * COLS, lo = col0 - kAbove;       // first own column, first column in shared memory
   const double *above = ch_smem, *below = ch_smem;           // the neighbours' shared memory
@@ -657,7 +659,7 @@ __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(
         if (2 * q + h >= k) pd[od[q]] = fma(-u[q], wk, fma(-we, uk, dd[q]));
         pd[on + 2 * (kChLd - 1) * q] = fma(p, u[q], bn[q]);
       }
-      if (active && h == 0 && prev >= col0 && prev < col0 + COLS) gV2[((int64_t)j * ns + t) * kBw + k] = (float)uk;
+      if (active && h == 0 && prev >= col0 && prev < col0 + COLS) gV2[((int64_t)j * ns + t) * kBw + k] = uk;
     }
     __syncthreads();
   }

@@ -113,9 +113,11 @@ struct SpLayer {
   double* bd_S;                // [3][64] U^T A U of three panels in turn
   double* bd_G; double* bd_M;  // [half strips][36] dots of the next panel's columns, of U's
   double* bd_band;             // [r][9] the band, by column
-  float* bd_V2;                // [r][steps][8] reflectors of the chase: sweep, step
+  double* bd_T;                // [panels][64] T of the panels: Q1 is the product of I - U T U^T
+  double* bd_V2;               // [r][steps][8] reflectors of the chase: sweep, step
   uint32_t* bd_bar;            // arrivals at the layer's barriers; zeroed per call
   double* tb_vecwork;          // [slots][5][rp] work vectors of the twisted factorisation
+  double* tb_z;                // [k_cap][rp] short sides above 1024: the kept atoms' eigenvectors of T
 };
 
 // a layer of a spectral decode: threads per output row, rows per CTA, the layer's first CTA
@@ -173,7 +175,8 @@ int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas,
 int sp_eigvec_big_slots();                                        // warps per layer of the vector kernel (work vectors)
 int sp_configure_eigvec_big();                                    // 0 if available
 int sp_configure_bisect();                                        // 0 if the eigenvalue kernel got its shared memory
-void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rp_max, cudaStream_t st);
+// rps: which padded short sides are among them (bit 0: up to 1024, bit 1: up to 2048, bit 2: above)
+void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, cudaStream_t st);
 int launch_sp_cholesky(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st);
 int launch_sp_cholesky_big(const SpLayer* d_layers, const TileRef* d_ctas, int n_ctas, int max_panels, cudaStream_t st);
 int sp_cholesky_big_rows_per_cta();

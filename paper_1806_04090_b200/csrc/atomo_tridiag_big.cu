@@ -10,21 +10,24 @@ namespace atomo {
 
 // ---- vectors of the kept atoms ------------------------------------------------------------------------------------
 // Two phases per CTA.  (A) one warp per kept atom: the eigenvector of T by the twisted factorisation of the small
-// route (work vectors in global memory), normalised, filed in the payload's slot of the atom.  (B) the whole CTA
-// applies the reflectors to up to four of its atoms at once, u = H_0 H_1 ... H_{r-3} z with H = I - 2 v v^T, from the
-// last reflector to the first, four at a time: a thread owns the columns tid, tid + 512, ... of the four reflector rows
-// (read once per group, kept in registers between the dot products and the update) and of every z (in shared memory;
-// no other thread touches them), so the only exchange per group is the block-wide sum of the products: v_i.z for
-// every atom and the six v_i.v_j.  For a group applied in the order 0, 1, 2, 3:  c_0 = 2 v_0.z,
-// c_i = 2 (v_i.z - sum_{j<i} c_j v_i.v_j),  z -= sum c_i v_i.  The matrix of reflectors is read once per four atoms
-// instead of once per atom, by 512 threads instead of 32.
+// route (work vectors in global memory), normalised.  (B) the whole CTA takes up to four of its atoms at once through the
+// reflectors, all in fp64 (the reflectors of the panels are fp32 numbers, and Q1 is exactly what the band reduction
+// applied): first the chase's (vb_chase_back), then the panels', four reflectors at a time.  There a thread owns the columns
+// tid, tid + 512, ... of the four reflector rows (read once per group, kept in registers between the dot products and the
+// update) and of every z (in shared memory; no other thread touches them), so the only exchange per group is the
+// block-wide sum of the products p_i = u_i.z; with the group's 4 x 4 block T of the panel's triangular factor,
+// z -= sum_i u_i (T p)_i.  The matrix of reflectors is read once per batch of atoms.
+// In fp32 (reflectors of the chase rounded, every application rounded) a kept atom's residual |A u - lambda u| / lambda_1 was
+// 2.7e-8 instead of 1.0e-8 on 1024 x 4096 noise, its vectors orthogonal to 2.4e-7 instead of 4e-9: the eigenvector of the band
+// fills eight times as many entries as one of a one-stage T, and each of its reflectors rounds them.  Cost: two layers of 4096 rows 7.5 -> 8.3 ms for this and
+// the back-projection, 96 of 1024 rows 1.7 -> 2.1.
 namespace {
 constexpr int kVbThreads = 512;
 constexpr int kVbWarps = kVbThreads / 32;
 constexpr int kVbSlots = 16;                 // work-vector sets per layer (phase A: 16 atoms at a time over the layer's CTAs)
 constexpr int kVbMaxCtas = 16;               // CTAs per layer (the kept atoms are dealt to them)
-constexpr int kVbBatch = 4;                  // atoms per pass over the reflectors
-constexpr int kVbSums = 4 * kVbBatch + 6;    // products summed per group
+constexpr int kVbBatch = 4;                  // atoms per pass over the reflectors; two above a short side of 2048 (shared memory)
+constexpr int kVbHalf = 2048;
 constexpr double kVbSameEig = 1.0e-9;        // as on the small route
 }  // namespace
 
@@ -72,97 +75,93 @@ __device__ __forceinline__ void vb_orthogonalise_equal(const SpLayer& L, uint32_
 
 
 namespace {
-// the columns tid, tid + THREADS, ... of the four reflector rows top, top - 1, top - 2, top - 3 (rows below 0: zeros)
+// the columns tid, tid + THREADS, ... of the four reflector rows base .. base + 3
 template <int THREADS, int COLS>
-__device__ __forceinline__ void vb_load_rows(const float* __restrict__ gV, int64_t ldv, int r, int top, float (&q)[4][COLS]) {
+__device__ __forceinline__ void vb_load_rows(const float* __restrict__ gV, int64_t ldv, int r, int base, float (&q)[4][COLS]) {
   const int tid = threadIdx.x;
-  const float* v0 = gV + (int64_t)top * ldv;
-  const float* v1 = gV + (int64_t)max(top - 1, 0) * ldv;
-  const float* v2 = gV + (int64_t)max(top - 2, 0) * ldv;
-  const float* v3 = gV + (int64_t)max(top - 3, 0) * ldv;
-  const bool e1 = top - 1 >= 0, e2 = top - 2 >= 0, e3 = top - 3 >= 0;
-  const int h0 = max(top - 3, 0) + kBandWidth;                 // reflector kk is zero below index kk + 8
+  const float* v = gV + (int64_t)base * ldv;
 #pragma unroll
   for (int m = 0; m < COLS; ++m) {
     const int h = tid + m * THREADS;
-    const bool in = h >= h0 && h < r;
-    q[0][m] = in ? __ldcg(v0 + h) : 0.0f;
-    q[1][m] = in && e1 ? __ldcg(v1 + h) : 0.0f;
-    q[2][m] = in && e2 ? __ldcg(v2 + h) : 0.0f;
-    q[3][m] = in && e3 ? __ldcg(v3 + h) : 0.0f;
+    const bool in = h >= base + kBandWidth && h < r;           // reflector kk is zero below index kk + 8
+#pragma unroll
+    for (int x = 0; x < 4; ++x) q[x][m] = in ? __ldcg(v + x * ldv + h) : 0.0f;
   }
 }
 
-// z_b <- H_0 ... H_{nref-1} z_b for the nb vectors in s_z, the whole CTA.  PREFETCH: the next group's rows are on their
-// way while this group's sums are added up (needs twice the registers for the rows: short sides up to 2048).
-template <int THREADS, int BATCH, int COLS, bool PREFETCH>
-__device__ __forceinline__ void vb_apply_reflectors(const float* __restrict__ gV, int64_t ldv, int r, int rp, int nref, int nb,
-                                                    float* s_z, float (*s_part)[4 * BATCH + 6], float* s_tot) {
-  constexpr int kSums = 4 * BATCH + 6, kWarps = THREADS / 32;
+// z_b <- Q1 z_b for the nb vectors in s_z, the whole CTA; the next group's rows are on their way while this group's sums are
+// added up.  Reflectors kk >= nref of the last group are rows of zeros.
+template <int THREADS, int BATCH, int COLS>
+__device__ __forceinline__ void vb_apply_reflectors(const float* __restrict__ gV, int64_t ldv, const double* __restrict__ gT, int r, int rp, int nref,
+                                                    int nb, double* s_z, double (*s_part)[4 * BATCH], double* s_tot) {
+  constexpr int kSums = 4 * BATCH, kWarps = THREADS / 32;
+  static_assert(kSums <= 32, "one warp adds the warps' parts");
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  float q[4][COLS], qn[4][PREFETCH ? COLS : 1];
-  if (PREFETCH && nref > 0) vb_load_rows<THREADS, COLS>(gV, ldv, r, nref - 1, q);
-  for (int top = nref - 1; top >= 0; top -= 4) {
-    if (!PREFETCH) vb_load_rows<THREADS, COLS>(gV, ldv, r, top, q);
-    float acc[kSums];
+  float q[4][COLS], qn[4][COLS];
+  const int top = (nref - 1) / 4 * 4;                          // the last group's first reflector
+  if (nref > 0) vb_load_rows<THREADS, COLS>(gV, ldv, r, top, q);
+  for (int base = nref > 0 ? top : -1; base >= 0; base -= 4) {
+    double2 t01 = make_double2(0.0, 0.0), t23 = t01;           // row lane % 4 of the group's block of T
+    if (w == 0) {
+      const double* t = gT + (int64_t)(base / 8) * 64 + (base % 8 + lane % 4) * 8 + base % 8;
+      t01 = __ldcg(reinterpret_cast<const double2*>(t)); t23 = __ldcg(reinterpret_cast<const double2*>(t) + 1);
+    }
+    double acc[kSums];
 #pragma unroll
-    for (int x = 0; x < kSums; ++x) acc[x] = 0.0f;
+    for (int x = 0; x < kSums; ++x) acc[x] = 0.0;
 #pragma unroll
     for (int m = 0; m < COLS; ++m) {
       const int h = tid + m * THREADS;
       if (h < r) {
-        acc[0] = fmaf(q[1][m], q[0][m], acc[0]); acc[1] = fmaf(q[2][m], q[0][m], acc[1]); acc[2] = fmaf(q[2][m], q[1][m], acc[2]);
-        acc[3] = fmaf(q[3][m], q[0][m], acc[3]); acc[4] = fmaf(q[3][m], q[1][m], acc[4]); acc[5] = fmaf(q[3][m], q[2][m], acc[5]);
 #pragma unroll
         for (int b = 0; b < BATCH; ++b) {
           if (b < nb) {
-            const float zh = s_z[(size_t)b * rp + h];
-            acc[6 + 4 * b + 0] = fmaf(q[0][m], zh, acc[6 + 4 * b + 0]); acc[6 + 4 * b + 1] = fmaf(q[1][m], zh, acc[6 + 4 * b + 1]);
-            acc[6 + 4 * b + 2] = fmaf(q[2][m], zh, acc[6 + 4 * b + 2]); acc[6 + 4 * b + 3] = fmaf(q[3][m], zh, acc[6 + 4 * b + 3]);
+            const double zh = s_z[(size_t)b * rp + h];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) acc[4 * b + x] = fma((double)q[x][m], zh, acc[4 * b + x]);
           }
         }
       }
     }
-    if (PREFETCH && top - 4 >= 0) vb_load_rows<THREADS, COLS>(gV, ldv, r, top - 4, reinterpret_cast<float (&)[4][COLS]>(qn));
-    const int n_sums = 6 + 4 * nb;
+    if (base >= 4) vb_load_rows<THREADS, COLS>(gV, ldv, r, base - 4, qn);
 #pragma unroll
     for (int x = 0; x < kSums; ++x) {
-      if (x < n_sums) {
-        const float t = warp_sum(acc[x]);
+      if (x < 4 * nb) {
+        const double t = warp_sum(acc[x]);
         if (lane == 0) s_part[w][x] = t;
       }
     }
     __syncthreads();
-    if (tid < n_sums) {
-      float t = 0.0f;
+    if (w == 0) {                                              // lane 4 b + i: (T p)_i of vector b
+      double p = 0.0;
+      if (lane < 4 * nb) {
 #pragma unroll
-      for (int ww = 0; ww < kWarps; ++ww) t += s_part[ww][tid];
-      s_tot[tid] = t;
+        for (int ww = 0; ww < kWarps; ++ww) p += s_part[ww][lane];
+      }
+      const int l0 = lane & ~3;
+      double s = t01.x * __shfl_sync(0xffffffffu, p, l0);      // (T is zero below its diagonal)
+      s = fma(t01.y, __shfl_sync(0xffffffffu, p, l0 + 1), s);
+      s = fma(t23.x, __shfl_sync(0xffffffffu, p, l0 + 2), s);
+      s = fma(t23.y, __shfl_sync(0xffffffffu, p, l0 + 3), s);
+      if (lane < 4 * nb) s_tot[lane] = s;
     }
     __syncthreads();
-    const float g10 = s_tot[0], g20 = s_tot[1], g21 = s_tot[2], g30 = s_tot[3], g31 = s_tot[4], g32 = s_tot[5];
 #pragma unroll
     for (int b = 0; b < BATCH; ++b) {
       if (b < nb) {
-        const float c0 = 2.0f * s_tot[6 + 4 * b];
-        const float c1 = 2.0f * (s_tot[6 + 4 * b + 1] - c0 * g10);
-        const float c2 = 2.0f * (s_tot[6 + 4 * b + 2] - c0 * g20 - c1 * g21);
-        const float c3 = 2.0f * (s_tot[6 + 4 * b + 3] - c0 * g30 - c1 * g31 - c2 * g32);
+        const double c0 = s_tot[4 * b], c1 = s_tot[4 * b + 1], c2 = s_tot[4 * b + 2], c3 = s_tot[4 * b + 3];
 #pragma unroll
         for (int m = 0; m < COLS; ++m) {
           const int h = tid + m * THREADS;
-          if (h < r) s_z[(size_t)b * rp + h] -= fmaf(c0, q[0][m], fmaf(c1, q[1][m], fmaf(c2, q[2][m], c3 * q[3][m])));
+          if (h < r) s_z[(size_t)b * rp + h] -= fma(c0, (double)q[0][m], fma(c1, (double)q[1][m], fma(c2, (double)q[2][m], c3 * (double)q[3][m])));
         }
       }
     }
-    // (the next group's partial sums go to s_part only after the barrier that follows them in program order for the
-    // slowest reader of s_tot: two barriers separate a write from the reads of the group before)
-    if (PREFETCH) {
+    // (two barriers separate a write to s_part or s_tot from the reads of the group before)
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+    for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int m = 0; m < COLS; ++m) q[x][m] = qn[x][PREFETCH ? m : 0];
-    }
+      for (int m = 0; m < COLS; ++m) q[x][m] = qn[x][m];
   }
 }
 }  // namespace
@@ -175,32 +174,32 @@ __device__ __forceinline__ void vb_apply_reflectors(const float* __restrict__ gV
 // ahead, read once for all ATOMS vectors.  One block barrier per sweep.
 namespace {
 constexpr int kBackStages = 5;
-template <int THREADS, int BPT, int ATOMS> constexpr size_t vb_ring_bytes() { return (size_t)kBackStages * (THREADS / ATOMS) * BPT * 8 * sizeof(float); }
+template <int THREADS, int BPT, int ATOMS> constexpr size_t vb_ring_bytes() { return (size_t)kBackStages * (THREADS / ATOMS) * BPT * 8 * sizeof(double); }
 
 template <int THREADS, int BPT, int ATOMS>
-__device__ __forceinline__ void vb_chase_back(const float* __restrict__ gV2, const int ns, const int r, float* s_z, const int z_stride,
-                                              float4* s_ring, float (*s_edge)[THREADS / 32]) {
+__device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, const int ns, const int r, double* s_z, const int z_stride,
+                                              double2* s_ring, double (*s_edge)[THREADS / 32]) {
   constexpr int kPer = THREADS / ATOMS;                        // threads per vector
-  constexpr int kChunks = kPer * BPT * 2;                      // float4 per sweep
+  constexpr int kChunks = kPer * BPT * 4;                      // double2 per sweep
   constexpr int kW = 8 * BPT;                                  // entries per thread = sweeps per turn
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32, me = tid % kPer;
-  float* const z = s_z + (size_t)(tid / kPer) * z_stride;
+  double* const z = s_z + (size_t)(tid / kPer) * z_stride;
   const int sweeps = ((r - 2 + kW - 1) / kW) * kW;             // the first ones of a partial turn act on nothing
   auto place = [](int f) -> int {                              // chunk f of a sweep inside its stage (spread over the banks)
-    const int th = f / (2 * BPT), c = f % (2 * BPT);
-    return th * 2 * BPT + (c ^ (BPT == 1 ? (th >> 2) & 1 : th & (2 * BPT - 1)));
+    const int th = f / (4 * BPT), c = f % (4 * BPT);
+    return th * 4 * BPT + (c ^ (BPT == 1 ? (th >> 1) & 3 : th & 7));
   };
   // this thread's chunks of a sweep: where they go, the last sweep that has them, where they come from (sweep by sweep upwards)
   constexpr int kMine = (kChunks + THREADS - 1) / THREADS;
   uint32_t to[kMine];
   int last[kMine];
-  const float* from[kMine];
+  const double* from[kMine];
 #pragma unroll
   for (int c = 0; c < kMine; ++c) {
-    const int f = tid + c * THREADS, t = f / 2;
+    const int f = tid + c * THREADS, t = f / 4;
     to[c] = (uint32_t)__cvta_generic_to_shared(s_ring + place(f));
     last[c] = f < kChunks ? min(r - 3, r - 3 - 8 * t) : -1;
-    from[c] = gV2 + ((int64_t)(sweeps - 1) * ns + t) * 8 + (f & 1) * 4;
+    from[c] = gV2 + ((int64_t)(sweeps - 1) * ns + t) * 8 + (f & 3) * 2;
   }
   int fill = 0, use = 0;                                       // stages
   auto issue = [&](int j) {                                    // sweep j (none below 0: an empty group keeps the count)
@@ -209,16 +208,16 @@ __device__ __forceinline__ void vb_chase_back(const float* __restrict__ gV2, con
       for (int c = 0; c < kMine; ++c) {
         const bool ok = j <= last[c];
         if (kChunks % THREADS == 0 || tid + c * THREADS < kChunks)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[c] + fill * (uint32_t)(kChunks * sizeof(float4))), "l"(ok ? from[c] : gV2), "r"(ok ? 16 : 0) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[c] + fill * (uint32_t)(kChunks * sizeof(double2))), "l"(ok ? from[c] : gV2), "r"(ok ? 16 : 0) : "memory");
         from[c] -= (int64_t)ns * 8;
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     fill = fill == kBackStages - 1 ? 0 : fill + 1;
   };
-  float x[kW];
+  double x[kW];
 #pragma unroll
-  for (int e = 0; e < kW; ++e) { const int at = sweeps + me * kW + e; x[e] = at < r ? z[at] : 0.0f; }
+  for (int e = 0; e < kW; ++e) { const int at = sweeps + me * kW + e; x[e] = at < r ? z[at] : 0.0; }
   __syncthreads();
   for (int s = 0; s < kBackStages - 1; ++s) issue(sweeps - 1 - s);
   for (int j0 = sweeps - 1; j0 >= 0; j0 -= kW) {
@@ -229,22 +228,23 @@ __device__ __forceinline__ void vb_chase_back(const float* __restrict__ gV2, con
       __syncthreads();                                         // sweep j has landed for everybody; the stage of j + 1 is free
       issue(j - (kBackStages - 1));
       if (j < sweeps - 1) {                                    // the window moves up by one entry
-        float in = __shfl_up_sync(0xffffffffu, x[(kW - s) % kW], 1);        // what was the last entry of the thread before
-        if (lane == 0) in = me == 0 ? (j + 1 < r ? z[j + 1] : 0.0f) : s_edge[(j + 1) & 1][w - 1];
+        double in = __shfl_up_sync(0xffffffffu, x[(kW - s) % kW], 1);        // what was the last entry of the thread before
+        if (lane == 0) in = me == 0 ? (j + 1 < r ? z[j + 1] : 0.0) : s_edge[(j + 1) & 1][w - 1];
         x[(kW - s) % kW] = in;
       }
-      const float4* const st = s_ring + use * kChunks;
+      const double2* const st = s_ring + use * kChunks;
       use = use == kBackStages - 1 ? 0 : use + 1;
 #pragma unroll
       for (int b = 0; b < BPT; ++b) {
-        const float4 u0 = st[place((me * BPT + b) * 2)], u1 = st[place((me * BPT + b) * 2 + 1)];
-        const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-        float d0 = 0.0f, d1 = 0.0f;
+        double u[8];
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) { d0 = fmaf(u[e], x[(8 * b + e - s + 2 * kW) % kW], d0); d1 = fmaf(u[e + 1], x[(8 * b + e + 1 - s + 2 * kW) % kW], d1); }
-        const float d = -2.0f * (d0 + d1);
+        for (int c = 0; c < 4; ++c) { const double2 v = st[place((me * BPT + b) * 4 + c)]; u[2 * c] = v.x; u[2 * c + 1] = v.y; }
+        double d0 = 0.0, d1 = 0.0;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[(8 * b + e - s + 2 * kW) % kW] = fmaf(d, u[e], x[(8 * b + e - s + 2 * kW) % kW]);
+        for (int e = 0; e < 8; e += 2) { d0 = fma(u[e], x[(8 * b + e - s + 2 * kW) % kW], d0); d1 = fma(u[e + 1], x[(8 * b + e + 1 - s + 2 * kW) % kW], d1); }
+        const double d = -2.0 * (d0 + d1);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[(8 * b + e - s + 2 * kW) % kW] = fma(d, u[e], x[(8 * b + e - s + 2 * kW) % kW]);
       }
       if (lane == 31) s_edge[j & 1][w] = x[(2 * kW - 1 - s) % kW];
     }
@@ -275,11 +275,11 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
   const int r = L.r, rp = L.rp;
   double* s_d = reinterpret_cast<double*>(vb_smem);            // [rp]
   double* s_e = s_d + rp;                                      // [rp]
-  float* s_z = reinterpret_cast<float*>(s_e + rp);             // [rp]
-  float4* s_ring = reinterpret_cast<float4*>(s_z + rp);
-  __shared__ float s_part[kVcWarps][10];
-  __shared__ float s_tot[10];
-  __shared__ float s_edge[2][kVcWarps];
+  double* s_z = s_e + rp;                                      // [rp]
+  double2* s_ring = reinterpret_cast<double2*>(s_z + rp);
+  __shared__ double s_part[kVcWarps][4];
+  __shared__ double s_tot[4];
+  __shared__ double s_edge[2][kVcWarps];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const uint32_t k = L.hdr->k;
   const float* const gV = L.td_V; const int64_t ldv = L.td_ldv; const double* const gLam = L.lam64;
@@ -310,46 +310,50 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
         }
         __syncwarp();
         const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
-        for (int i = lane; i < r; i += 32) s_z[i] = (float)(zz[i] * inv);
+        for (int i = lane; i < r; i += 32) s_z[i] = zz[i] * inv;
       }
       __syncthreads();
       vb_chase_back<kVcThreads, 1, 1>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
-      vb_apply_reflectors<kVcThreads, 1, kVcMaxRp / kVcThreads, true>(gV, ldv, r, rp, nref, 1, s_z, s_part, s_tot);
-      float n2f = 0.0f;
-      for (int i = tid; i < r; i += kVcThreads) n2f = fmaf(s_z[i], s_z[i], n2f);
-      n2f = warp_sum(n2f);
+      vb_apply_reflectors<kVcThreads, 1, kVcMaxRp / kVcThreads>(gV, ldv, L.bd_T, r, rp, nref, 1, s_z, s_part, s_tot);
+      double n2 = 0.0;
+      for (int i = tid; i < r; i += kVcThreads) n2 = fma(s_z[i], s_z[i], n2);
+      n2 = warp_sum(n2);
       __syncthreads();
-      if (lane == 0) s_part[w][0] = n2f;
+      if (lane == 0) s_part[w][0] = n2;
       __syncthreads();
-      float tot = 0.0f;
+      double tot = 0.0;
 #pragma unroll
       for (int ww = 0; ww < kVcWarps; ++ww) tot += s_part[ww][0];
-      const float invf = tot > 0.0f ? rsqrtf(tot) : 0.0f;
-      for (int i = tid; i < r; i += kVcThreads) gShort[(int64_t)a * r + i] = s_z[i] * invf;
+      const double inv = tot > 0.0 ? rsqrt(tot) : 0.0;
+      for (int i = tid; i < r; i += kVcThreads) gShort[(int64_t)a * r + i] = (float)(s_z[i] * inv);
       __syncthreads();
     }
   }
   vb_orthogonalise_equal(L, k, kVcCtas);
 }
 
+// BATCH atoms at a time, COLS columns per thread: up to a short side of 2048, or above
+template <int BATCH, int COLS>
 __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLayer* __restrict__ layers,
                                                                       const int* __restrict__ big_layers) {
+  constexpr int kRp = COLS * kVbThreads, kFew = kVbThreads * 8 / kRp;
   const SpLayer& L = layers[big_layers[blockIdx.x]];
-  if (L.rp <= 1024) return;                                    // smaller layers: sp_eigvec_big_cta_kernel
+  if (L.rp <= kVcMaxRp || (L.rp <= kVbHalf) != (kRp <= kVbHalf)) return;   // another kernel's
   extern __shared__ __align__(16) unsigned char vb_smem[];
   const int r = L.r, rp = L.rp;
-  double* s_d = reinterpret_cast<double*>(vb_smem);            // [rp]
+  double* s_z = reinterpret_cast<double*>(vb_smem);            // [BATCH][rp]
+  double* s_d = s_z + (size_t)BATCH * rp;                      // [rp], phase A
   double* s_e = s_d + rp;                                      // [rp]
-  float* s_z = reinterpret_cast<float*>(s_e + rp);             // [kVbBatch][rp]
-  float4* s_ring = reinterpret_cast<float4*>(s_z + (size_t)kVbBatch * rp);
-  __shared__ float s_edge[2][kVbWarps];
-  __shared__ float s_part[kVbWarps][kVbSums];
-  __shared__ float s_tot[kVbSums];
+  double2* s_ring = reinterpret_cast<double2*>(s_d);           // phase B
+  __shared__ double s_edge[2][kVbWarps];
+  __shared__ double s_part[kVbWarps][4 * BATCH];
+  __shared__ double s_tot[4 * BATCH];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int n_ctas = gridDim.y, cy = blockIdx.y;
   const uint32_t k = L.hdr->k;
   const float* const gV = L.td_V; const int64_t ldv = L.td_ldv; const double* const gLam = L.lam64;
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
+  double* const gZ = L.tb_z;
   const int nref = max(r - kBandWidth - 1, 0);
   for (int i = tid; i < r; i += kVbThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
   __syncthreads();
@@ -376,41 +380,38 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
       }
       __syncwarp();
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
-      for (int i = lane; i < r; i += 32) gShort[(int64_t)a * r + i] = (float)(zz[i] * inv);
+      for (int i = lane; i < r; i += 32) gZ[(int64_t)a * rp + i] = zz[i] * inv;
       __syncwarp();
     }
   }
   __syncthreads();
-  // ---- (B) back-transformation, kVbBatch of this CTA's atoms per pass over the reflectors ----
+  // ---- (B) back-transformation, BATCH of this CTA's atoms per pass over the reflectors ----
   const uint32_t n_mine = k > (uint32_t)cy ? (k - (uint32_t)cy + (uint32_t)n_ctas - 1u) / (uint32_t)n_ctas : 0u;
-  for (uint32_t b0 = 0; b0 < n_mine; b0 += kVbBatch) {
-    const int nb = (int)min((uint32_t)kVbBatch, n_mine - b0);
-    for (int b = 0; b < nb; ++b) {
-      const float* src = gShort + (int64_t)(cy + (b0 + b) * n_ctas) * r;
-      for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = src[i];
+  for (uint32_t b0 = 0; b0 < n_mine; b0 += BATCH) {
+    const int nb = (int)min((uint32_t)BATCH, n_mine - b0);
+    for (int b = 0; b < BATCH; ++b) {
+      const double* src = gZ + (int64_t)(cy + (b0 + b) * n_ctas) * rp;
+      for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = b < nb ? __ldcg(src + i) : 0.0;
     }
-    for (int b = nb; b < kVbBatch; ++b) for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = 0.0f;
     __syncthreads();
-    // one atom: a run per thread and a turn of eight sweeps; the turn of 32 that four atoms share the reflectors in is more
-    // code than the instruction cache holds (one of 4096 entries: 9.0 -> 7.3 ms with the rest of the kernel)
-    if (nb == 1) vb_chase_back<kVbThreads, 1, 1>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
-    else vb_chase_back<kVbThreads, 4, kVbBatch>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
-    if (rp <= 4 * kVbThreads) vb_apply_reflectors<kVbThreads, kVbBatch, 4, true>(gV, ldv, r, rp, nref, nb, s_z, s_part, s_tot);
-    else vb_apply_reflectors<kVbThreads, kVbBatch, 8, true>(gV, ldv, r, rp, nref, nb, s_z, s_part, s_tot);
+    // few atoms: a run per thread and a turn of eight sweeps
+    if (nb <= kFew) vb_chase_back<kVbThreads, 1, kFew>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+    else vb_chase_back<kVbThreads, COLS * BATCH / 8, BATCH>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+    vb_apply_reflectors<kVbThreads, BATCH, COLS>(gV, ldv, L.bd_T, r, rp, nref, nb, s_z, s_part, s_tot);
     // normalise and file
     for (int b = 0; b < nb; ++b) {
-      float n2f = 0.0f;
-      for (int i = tid; i < r; i += kVbThreads) n2f = fmaf(s_z[(size_t)b * rp + i], s_z[(size_t)b * rp + i], n2f);
-      n2f = warp_sum(n2f);
+      double n2 = 0.0;
+      for (int i = tid; i < r; i += kVbThreads) n2 = fma(s_z[(size_t)b * rp + i], s_z[(size_t)b * rp + i], n2);
+      n2 = warp_sum(n2);
       __syncthreads();
-      if (lane == 0) s_part[w][0] = n2f;
+      if (lane == 0) s_part[w][0] = n2;
       __syncthreads();
-      float tot = 0.0f;
+      double tot = 0.0;
 #pragma unroll
       for (int ww = 0; ww < kVbWarps; ++ww) tot += s_part[ww][0];
-      const float invf = tot > 0.0f ? rsqrtf(tot) : 0.0f;
+      const double inv = tot > 0.0 ? rsqrt(tot) : 0.0;
       float* dst = gShort + (int64_t)(cy + (b0 + b) * n_ctas) * r;
-      for (int i = tid; i < r; i += kVbThreads) dst[i] = s_z[(size_t)b * rp + i] * invf;
+      for (int i = tid; i < r; i += kVbThreads) dst[i] = (float)(s_z[(size_t)b * rp + i] * inv);
     }
     __syncthreads();
   }
@@ -419,33 +420,38 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
 
 // ---- host side ---------------------------------------------------------------------------------------------------
 namespace {
-size_t vb_smem_bytes(int rp_max) {
-  return (size_t)rp_max * (2 * sizeof(double) + kVbBatch * sizeof(float)) + vb_ring_bytes<kVbThreads, 4, kVbBatch>();
+// shared memory of the kernel with BATCH atoms and COLS columns per thread for a short side of rp: the vectors, then the diagonals of
+// T or the ring of reflectors (the larger of its two forms)
+template <int BATCH, int COLS> size_t vb_smem_bytes(int rp) {
+  const size_t ring = std::max(vb_ring_bytes<kVbThreads, 1, 8 / COLS>(), vb_ring_bytes<kVbThreads, COLS * BATCH / 8, BATCH>());
+  return (size_t)rp * BATCH * sizeof(double) + std::max(ring, (size_t)rp * 2 * sizeof(double));
 }
-size_t vc_smem_bytes(int rp_max) { return (size_t)std::min(rp_max, kVcMaxRp) * (2 * sizeof(double) + sizeof(float)) + vb_ring_bytes<kVcThreads, 1, 1>(); }
+size_t vc_smem_bytes(int rp_max) { return (size_t)std::min(rp_max, kVcMaxRp) * 3 * sizeof(double) + vb_ring_bytes<kVcThreads, 1, 1>(); }
 }  // namespace
 
 int sp_eigvec_big_slots() { return kVbSlots; }
 
 // 0 if the kernels got their shared memory
 int sp_configure_eigvec_big() {
-  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes(kMaxShort)) != cudaSuccess;
+  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbBatch, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch, 4>(kVbHalf)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<2, 8>(kMaxShort)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vc_smem_bytes(kVcMaxRp)) != cudaSuccess;
   if (bad) cudaGetLastError();
   return bad;
 }
 
-void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rp_max, cudaStream_t st) {
+void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, cudaStream_t st) {
   if (n_big <= 0) return;
-  // layers up to a short side of 1024: a four-warp CTA per kept atom (the other kernel's CTAs leave such layers at once,
-  // and the other way round)
-  sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(rp_max), st>>>(d_layers, d_big);
-  if (rp_max <= kVcMaxRp) return;
+  // layers up to a short side of 1024: a four-warp CTA per kept atom (each kernel's CTAs leave the others' layers at once)
+  if (rps & 1) sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(kVcMaxRp), st>>>(d_layers, d_big);
+  if (!(rps & 6)) return;
   // larger layers: CTAs per layer (1 to 16; the kept atoms are dealt to them), as many as keep the launch within one wave
-  static int sms = 0;
-  if (sms == 0) { int dev = 0; if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 1; }
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int per = 1;
   while (per < kVbMaxCtas && n_big * per * 2 <= sms) per *= 2;
-  sp_eigvec_big_kernel<<<dim3(n_big, per), kVbThreads, vb_smem_bytes(rp_max), st>>>(d_layers, d_big);
+  if (rps & 2) sp_eigvec_big_kernel<kVbBatch, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<kVbBatch, 4>(kVbHalf), st>>>(d_layers, d_big);
+  if (rps & 4) sp_eigvec_big_kernel<2, 8><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<2, 8>(kMaxShort), st>>>(d_layers, d_big);
 }
 
 }  // namespace atomo

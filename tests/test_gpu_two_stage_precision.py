@@ -42,3 +42,29 @@ def test_singular_values(atomo, m, n, bar):
     err = float((got - want).norm() / want.norm())
     print(f"{m} x {n}: sigma relative l2 error {err:.2e}")
     assert err <= bar
+
+
+# one layer, or so many that a CTA takes several atoms at a time; residual bar: 1.5 times the one-stage route's
+@pytest.mark.parametrize("m,n,count,bar", [(520, 1500, 1, 2.6e-8), (1024, 4096, 1, 1.6e-8), (777, 3001, 9, 1.9e-8), (1100, 2048, 24, 1.7e-8),
+                                           (2048, 4096, 1, 1.2e-8), (3000, 3100, 1, 1.1e-8), (2049, 2300, 10, 1.5e-8)])
+def test_vectors_of_kept_atoms(atomo, m, n, count, bar):
+    """Residuals |A u - (u.A u) u| / lambda_1 of the kept short-side vectors, and their dots with one another.  The stored vectors are
+    fp32: rounding alone gives dots of 2^-24.5 / sqrt(r) (r.m.s.), some four times that for the largest of a thousand pairs."""
+    import torch
+    import numpy as np
+    G = _layer(m, n, m + 3)
+    pay, _ = atomo.atomo_encode_spectral([G] * count, 24.0, 6, step=1, k_cap=96)
+    hdrs = pay.headers()
+    A = G.double() @ G.double().T
+    top = float(torch.linalg.eigvalsh(A)[-1])
+    for l in range(count):
+        assert hdrs[1][l].status == 0 and hdrs[1][l].k > 8
+        U = torch.from_numpy(pay.layer_arrays(l, hdrs)["U"].astype(np.float64)).cuda()
+        AU = A @ U
+        res = (AU - U * ((U * AU).sum(0) / (U * U).sum(0))).norm(dim=0) / top
+        dots = U.T @ U
+        off = float((dots - torch.diag(torch.diag(dots))).abs().max())
+        rms = float(res.square().mean().sqrt())
+        if l == 0:
+            print(f"{m} x {n}: residual {rms:.2e} (worst {float(res.max()):.2e}), dots {off:.2e}")
+        assert rms <= bar and off <= 2e-8 and float((torch.diag(dots) - 1).abs().max()) <= 4e-7
