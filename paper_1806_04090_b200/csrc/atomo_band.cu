@@ -41,8 +41,8 @@ static_assert(kBw == 8, "the operand vectors are two float4");
 // tasks, dealt to the warps of all the layer's CTAs in turn (a strip per CTA left half of them idle on average); the parts of a
 // sum are added in fp64.  A warp streams its columns through a ring of its own (asynchronous copies of four columns with their
 // U and W).  Twelve warps per SM: with sixteen the 128 registers do not hold a task.
-// (The sixteen products that update an entry are summed first and added to it once: added one by one they rounded the matrix
-// sixteen times per panel, and the singular values of 2000 x 2048 noise were off by 1.7e-7 instead of 5.5e-8.)
+// (The sixteen products that update an entry are summed before they are added to it: added one by one they rounded the matrix
+// sixteen times per panel, and the singular values of 2000 x 2048 noise were off by 1.6e-7 instead of 5.4e-8.)
 // Bound: latency of the walk with few layers (a group of four columns takes a lone warp about 1000 cycles, its 200
 // multiply-adds alone would take 200), and the chain of a panel's small steps (Gram sums, 8 x 8 factorisation, U, T: 25 k
 // cycles).  Two layers of 4096 rows: 106 (one-stage reduction) -> 49.7 -> 25.9 ms; 96 of 1024: 29.4 -> 13.2 ms.
@@ -410,14 +410,21 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
               const float4 cu0 = o[0], cu1 = o[1], cw0 = o[2], cw1 = o[3];
               const float cu[8] = {cu0.x, cu0.y, cu0.z, cu0.w, cu1.x, cu1.y, cu1.z, cu1.w};
               const float cw[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
-              // the sixteen products are summed before they meet the entry: one rounding at the entry's scale per panel
-              float dx = up0[0] * cw[0], dy = up1[0] * cw[0];
-              dx = fmaf(wp0[0], cu[0], dx); dy = fmaf(wp1[0], cu[0], dy);
+              // the sixteen products are summed before they meet the entry: one rounding at the entry's scale per panel.  The last
+              // reflectors' first: what the first ones take away is the largest where few directions outweigh the rest (with the
+              // first ones first sigma of 2000 x 2048 at noise 0.05 was off by 8.1e-6 instead of 3.9e-6); in two chains (one:
+              // VGG-11 58.6 ms, two 58.4)
+              float dx = up0[7] * cw[7], dy = up1[7] * cw[7], ex = up0[6] * cw[6], ey = up1[6] * cw[6];
+              dx = fmaf(wp0[7], cu[7], dx); dy = fmaf(wp1[7], cu[7], dy);
+              ex = fmaf(wp0[6], cu[6], ex); ey = fmaf(wp1[6], cu[6], ey);
 #pragma unroll
-              for (int t = 1; t < 8; ++t) {
+              for (int t = 5; t >= 0; t -= 2) {
                 dx = fmaf(up0[t], cw[t], dx); dy = fmaf(up1[t], cw[t], dy);
                 dx = fmaf(wp0[t], cu[t], dx); dy = fmaf(wp1[t], cu[t], dy);
+                ex = fmaf(up0[t - 1], cw[t - 1], ex); ey = fmaf(up1[t - 1], cw[t - 1], ey);
+                ex = fmaf(wp0[t - 1], cu[t - 1], ex); ey = fmaf(wp1[t - 1], cu[t - 1], ey);
               }
+              dx += ex; dy += ey;
               v.x += dx; v.y += dy;
             }
             out[u] = v;

@@ -8,8 +8,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def _layer(m, n, seed):
-    """16 directions with singular values 1 / i under noise of four times their norm"""
+def _layer(m, n, seed, noise=4.0):
+    """16 directions with singular values 1 / i under noise of `noise` times their norm"""
     import torch
     dev = torch.device("cuda", 0)
     gen = torch.Generator(device=dev)
@@ -18,7 +18,7 @@ def _layer(m, n, seed):
     u = torch.randn(m, 16, device=dev, generator=gen) / math.sqrt(m)
     v = torch.randn(n, 16, device=dev, generator=gen) / math.sqrt(n)
     g = torch.randn(m, n, device=dev, generator=gen)
-    g *= 4.0 * float(torch.linalg.norm(sigma)) / math.sqrt(m * n)
+    g *= noise * float(torch.linalg.norm(sigma)) / math.sqrt(m * n)
     return g.addmm_(u * sigma, v.T)
 
 
@@ -42,6 +42,19 @@ def test_singular_values(atomo, m, n, bar):
     err = float((got - want).norm() / want.norm())
     print(f"{m} x {n}: sigma relative l2 error {err:.2e}")
     assert err <= bar
+
+
+# few directions that outweigh the rest: the first reflectors' products are the largest.  The bar is 1.5 times what the update measured
+# that added its products one by one to the entry (the entry shrinks with them, and so do their roundings)
+def test_singular_values_under_strong_directions(atomo):
+    import torch
+    G = _layer(2000, 2048, 77, noise=0.05)
+    pay, dbg = atomo.atomo_encode_spectral([G], 8.0, 5, step=1, k_cap=64, debug=True)
+    assert pay.headers()[1][0].status == 0
+    want = torch.linalg.eigvalsh(G.double() @ G.double().T).clamp(min=0).sqrt().flip(0)
+    err = float((torch.from_numpy(dbg.layer_sigma(0, 2000)).to(want) - want).norm() / want.norm())
+    print(f"2000 x 2048, strong directions: sigma relative l2 error {err:.2e}")
+    assert err <= 5e-6
 
 
 # one layer, or so many that a CTA takes several atoms at a time; residual bar: 1.5 times the one-stage route's
