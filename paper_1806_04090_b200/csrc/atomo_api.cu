@@ -67,6 +67,7 @@ struct atomo_ctx {
   int tri_clusters = -1;             // co-resident clusters of the tridiagonal reduction (-1 = not asked yet, 0 = unavailable)
   int tri_big_ok = -1;               // two-stage tridiagonal reduction for short sides above 512 (-1 = not asked yet)
   int band_capacity[2][13];          // co-resident CTAs of its first stage, by instance and ceil(log2(short side)) (-1 = not asked yet)
+  int chase_capacity[5] = {-1, -1, -1, -1, -1};   // clusters of its second stage side by side, by log2(CTAs)
   int tri_big_ctas = 0;              // CTAs per layer of that reduction: 0 = chosen per batch, else 1, 2, 4, 8 or 16
   int eig_scheme_used = -1;          // what the last spectral encode actually ran
   int ew_format = ATOMO_EW_EXPLICIT; // payload format of entry-wise encodes
@@ -278,6 +279,14 @@ int for_each_ew_decode(const uint8_t* payload, const int64_t* cols, float* const
     l += count;
   }
   return n_launch;
+}
+
+// clusters of the bulge chase that run side by side, asked for once per context
+int chase_room(atomo_ctx* ctx, int ctas) {
+  int lg = 0;
+  while ((1 << lg) < ctas) ++lg;
+  if (ctx->chase_capacity[lg] < 0) ctx->chase_capacity[lg] = sp_chase_capacity(ctas);
+  return ctx->chase_capacity[lg];
 }
 
 bool bad_budget(double s) { return !(s > 0.0) || !std::isfinite(s); }
@@ -867,12 +876,13 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(band reduction)");
       ++n_eig_launch;
     }
-    for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one cluster size are neighbours)
-      const int n_big = (int)big_layers.size(), rm = L[big_layers[i]].r, c = sp_chase_ctas(rm, n_big);
-      auto same = [&](int l) { return sp_chase_ctas(L[l].r, n_big) == c && (L[l].r > 1024) == (rm > 1024); };
+    auto chase_class = [&](int l) { return L[l].r <= 1024 ? 1024 : L[l].r <= 2048 ? 2048 : 4096; };
+    for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one class are neighbours)
+      const int of = chase_class(big_layers[i]);
       n = 1;
-      while (i + n < big_layers.size() && same(big_layers[i + n])) ++n;
-      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, rm, st);
+      while (i + n < big_layers.size() && chase_class(big_layers[i + n]) == of) ++n;
+      const int c = sp_chase_ctas(of, (int)n, of > 1024 ? chase_room(ctx, of / 256) : 0);
+      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(bulge chase)");
       ++n_eig_launch;
     }

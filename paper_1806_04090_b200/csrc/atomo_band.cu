@@ -559,8 +559,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
 // as zeros, lanes without a step work on a dummy block of zeros: no bounds tests.
 // Bound: shared memory where a CTA has 1024 columns (23 warps), else the latency of the step's chain.
 // (The shared-memory pipe, which the exchanges use too, takes about 110 cycles per warp and tick: 24 loads and stores of
-// eight bytes, 36 shuffles.)  Larger short sides, and batches that leave SMs idle, are spread over a cluster, down to 256
-// columns per CTA.  A cluster barrier and the reads of a
+// eight bytes, 36 shuffles.)  Larger short sides are spread over a cluster, down to 256 columns per CTA.  A cluster barrier and the reads of a
 // neighbour's memory in every tick took 4.4 us per tick, three times the step itself; so a CTA also keeps copies of the
 // columns next to its own, works on them as well, and fetches them afresh every kChTicks ticks.  What it lacks spoils these
 // columns from their outer ends inwards: by eight columns a tick from above (a sweep moves down by a block), by fifteen from
@@ -692,9 +691,11 @@ const BandForm kBandForms[] = {
     {4096, 384, 1, 16, 4, (const void*)sp_band_kernel<384, 1, 16, 4>},
 };
 size_t band_smem(const BandForm& f, int r_max) { return ((size_t)(r_max + kGroup) * 8 + (size_t)f.threads / 32 * f.stages * kGroupFloats) * sizeof(float); }
+constexpr size_t kChAlone = 120 * 1024;       // more than half an SM's shared memory: a CTA on its own
 template <int C, int COLS> int chase_configure() {
   auto* fn = sp_chase_kernel<C, COLS>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ChForm<C, COLS>::kSmem) != cudaSuccess) return 1;
+  const size_t smem = std::max(ChForm<C, COLS>::kSmem, C >= 8 ? kChAlone : (size_t)0);   // (the capacity is asked for with that much)
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 1;
   if (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 1;
   return 0;
 }
@@ -720,7 +721,7 @@ int sp_configure_band() {
     bad |= cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)band_smem(f, f.max_r)) != cudaSuccess;
     bad |= cudaFuncSetAttribute(f.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess;
   }
-  bad |= chase_configure<1, 1024>() | chase_configure<2, 1024>() | chase_configure<4, 1024>() | chase_configure<4, 256>() |
+  bad |= chase_configure<1, 1024>() | chase_configure<2, 1024>() | chase_configure<4, 1024>() |
          chase_configure<8, 256>() | chase_configure<16, 256>();
   if (bad) cudaGetLastError();
   return bad;
@@ -743,19 +744,40 @@ template <int C, int COLS> int chase_launch(const SpLayer* d_layers, const int* 
   return (int)cudaLaunchKernelEx(&cfg, sp_chase_kernel<C, COLS>, d_layers, d_list);
 }
 }  // namespace
-// CTAs per layer of the chase for a layer of r rows in a batch of n large layers: 256 columns each (half the time of 1024
-// columns per CTA) while the batch's clusters fit the GPU side by side, else as few as hold the layer
-int sp_chase_ctas(int r, int n) {
-  const int few = r <= 1024 ? 1 : r <= 2048 ? 2 : 4, many = 4 * few;
-  return n * many <= band_sms() / 2 ? many : few;
+// Clusters of `ctas` CTAs that run side by side with an SM for each CTA (0: not available).  (The instances of 256 columns leave
+// room for a second CTA on an SM; asked for as if they did not.)
+int sp_chase_capacity(int ctas) {
+  if (ctas == 1) return band_sms();
+  const bool wide = ctas >= 8;
+  const void* fn = ctas == 2 ? (const void*)sp_chase_kernel<2, 1024> : ctas == 4 ? (const void*)sp_chase_kernel<4, 1024>
+                 : ctas == 8 ? (const void*)sp_chase_kernel<8, 256> : (const void*)sp_chase_kernel<16, 256>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3(wide ? ChForm<8, 256>::kThreads : ChForm<2, 1024>::kThreads);
+  cfg.dynamicSmemBytes = wide ? kChAlone : ChForm<2, 1024>::kSmem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
 }
-// d_list: n layers of at most r_max rows that take `ctas` CTAs each
-int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, int r_max, cudaStream_t st) {
+// CTAs per layer of the chase for n layers of r rows (up to 1024, 2048 or 4096): 256 columns each while the clusters run side by
+// side with an SM per CTA, else 1024 columns.  Both stages of the reduction, 256 | 1024 columns, ms: 9 of 2048 rows 21.5 | 24.3, 14
+// 27.4 | 30.2, 16 35.9 | 32.1; of 4096 rows 1 33.9 | 43.2, 7 73.7 | 83.0, 8 95.4 | 90.8 (14 and 7 clusters fit).  Up to 1024 rows a
+// single CTA takes what a cluster of four takes (1 layer 6.05 | 6.08, 20 layers 7.85 | 7.92) and leaves the others their SMs (36:
+// 9.5 | 12.7).
+int sp_chase_ctas(int r, int n, int wide_capacity) {
+  const int few = r <= 1024 ? 1 : r <= 2048 ? 2 : 4;
+  return few > 1 && n <= wide_capacity ? 4 * few : few;
+}
+// d_list: n layers that take `ctas` CTAs each
+int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st) {
   if (n <= 0) return 0;
   switch (ctas) {
     case 1: return chase_launch<1, 1024>(d_layers, d_list, n, st);
     case 2: return chase_launch<2, 1024>(d_layers, d_list, n, st);
-    case 4: return r_max <= 1024 ? chase_launch<4, 256>(d_layers, d_list, n, st) : chase_launch<4, 1024>(d_layers, d_list, n, st);
+    case 4: return chase_launch<4, 1024>(d_layers, d_list, n, st);
     case 8: return chase_launch<8, 256>(d_layers, d_list, n, st);
     default: return chase_launch<16, 256>(d_layers, d_list, n, st);
   }

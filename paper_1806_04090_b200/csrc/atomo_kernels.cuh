@@ -170,8 +170,9 @@ int sp_band_parts(int form);                                      // tasks that 
 int sp_band_capacity(int form, int r_max);                        // co-resident CTAs of the band reduction (0: not available)
 int sp_configure_band();                                          // 0 if available
 int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas, int form, int r_max, uint32_t* d_timeout, cudaStream_t st);  // cudaError_t
-int sp_chase_ctas(int r, int n);                                  // CTAs per layer of the chase, in a batch of n large layers
-int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, int r_max, cudaStream_t st);   // cudaError_t
+int sp_chase_capacity(int ctas);                                  // clusters of that many CTAs side by side (0: not available)
+int sp_chase_ctas(int r, int n, int wide_capacity);               // CTAs per layer of the chase, for n layers of its size
+int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st);   // cudaError_t
 int sp_eigvec_big_slots();                                        // warps per layer of the vector kernel (work vectors)
 int sp_configure_eigvec_big();                                    // 0 if available
 int sp_configure_bisect();                                        // 0 if the eigenvalue kernel got its shared memory
