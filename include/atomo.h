@@ -323,6 +323,10 @@ int atomo_set_persistent_eig(atomo_ctx* ctx, int32_t enabled);
  * of the batch in proportion to their work, else 1, 2, 4, 8 or 16 (at most one per 64 rows).  The payload does not
  * depend on it bit for bit (the knob exists for tuning and for checking exactly that).                          */
 int atomo_set_tridiag_ctas(atomo_ctx* ctx, int32_t ctas_per_layer);
+/* Test hook for scheme 3 above a short side of 512: the occupancy queries count as if they reported at most `band_ctas`
+ * co-resident CTAs of the band reduction and `chase_clusters` clusters of the bulge chase (-1, the default: no limit).  With 0 of
+ * either a batch that needs it takes scheme 2 as on a GPU that cannot place it.                                              */
+int atomo_limit_tridiag_route(atomo_ctx* ctx, int32_t band_ctas, int32_t chase_clusters);
 /* The scheme (0 to 3 as above) that the last atomo_encode_spectral() of this context actually ran; -1 before
  * the first call.  Host only.                                                                                */
 int atomo_last_eig_scheme(atomo_ctx* ctx);

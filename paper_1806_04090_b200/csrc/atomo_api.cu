@@ -68,6 +68,7 @@ struct atomo_ctx {
   int tri_big_ok = -1;               // two-stage tridiagonal reduction for short sides above 512 (-1 = not asked yet)
   int band_capacity[2][13];          // co-resident CTAs of its first stage, by instance and ceil(log2(short side)) (-1 = not asked yet)
   int chase_capacity[5] = {-1, -1, -1, -1, -1};   // clusters of its second stage side by side, by log2(CTAs)
+  int band_limit = -1, chase_limit = -1;          // at most that many of either, whatever the queries say (-1: no limit)
   int tri_big_ctas = 0;              // CTAs per layer of that reduction: 0 = chosen per batch, else 1, 2, 4, 8 or 16
   int eig_scheme_used = -1;          // what the last spectral encode actually ran
   int ew_format = ATOMO_EW_EXPLICIT; // payload format of entry-wise encodes
@@ -281,13 +282,23 @@ int for_each_ew_decode(const uint8_t* payload, const int64_t* cols, float* const
   return n_launch;
 }
 
-// clusters of the bulge chase that run side by side, asked for once per context
+// What the occupancy queries say of the two-stage reduction, asked for once per context: CTAs of the band reduction that are
+// resident together (layers of at most r rows), clusters of the bulge chase that run side by side
+int band_room(atomo_ctx* ctx, int form, int r) {
+  int lg = 0;
+  while ((1 << lg) < r) ++lg;
+  int& known = ctx->band_capacity[form][lg];
+  if (known < 0) known = sp_band_capacity(form, 1 << lg);
+  return ctx->band_limit >= 0 ? std::min(known, ctx->band_limit) : known;
+}
 int chase_room(atomo_ctx* ctx, int ctas) {
   int lg = 0;
   while ((1 << lg) < ctas) ++lg;
-  if (ctx->chase_capacity[lg] < 0) ctx->chase_capacity[lg] = sp_chase_capacity(ctas);
-  return ctx->chase_capacity[lg];
+  int& known = ctx->chase_capacity[lg];
+  if (known < 0) known = sp_chase_capacity(ctas);
+  return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
+int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
 bool bad_budget(double s) { return !(s > 0.0) || !std::isfinite(s); }
 
@@ -440,6 +451,13 @@ int atomo_set_tridiag_ctas(atomo_ctx* ctx, int32_t ctas_per_layer) {
   return ATOMO_OK;
 }
 
+int atomo_limit_tridiag_route(atomo_ctx* ctx, int32_t band_ctas, int32_t chase_clusters) {
+  if (!ctx || band_ctas < -1 || chase_clusters < -1) return ATOMO_ERR_INVALID_ARG;
+  ctx->band_limit = band_ctas;
+  ctx->chase_limit = chase_clusters;
+  return ATOMO_OK;
+}
+
 int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores) {
   if (!ctx) return ATOMO_ERR_INVALID_ARG;
   ctx->tc_gram = tensor_cores != 0;
@@ -561,11 +579,22 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     if (ctx->tri_big_ok < 0) ctx->tri_big_ok = (sp_configure_band() == 0 && sp_configure_eigvec_big() == 0 && sp_configure_bisect() == 0) ? 1 : 0;
     if (ctx->tri_big_ok < 1 || r_max > sp_band_max_r()) tri_form = false;
   }
+  // the large layers, largest first; a GPU that cannot hold a CTA of their band reduction or a cluster of their chase takes the
+  // Jacobi routes
   std::vector<int> big_layers;
+  int band_form = 0;
+  if (tri_form && any_big) {
+    int64_t strips = 0;
+    for (int l = 0; l < n_layers; ++l) if (L[l].rp > sp_tridiag_max_rp()) { big_layers.push_back(l); strips += sp_band_strips(L[l].r); }
+    std::stable_sort(big_layers.begin(), big_layers.end(), [&](int a, int b) { return L[a].r > L[b].r; });
+    band_form = sp_band_form(r_max, strips);
+    bool can = band_room(ctx, band_form, r_max) >= 1;
+    for (int l : big_layers) { const int few = sp_chase_ctas(chase_class(L[l].r), 1, 0); can &= chase_room(ctx, few) >= 1; }
+    if (!can) { tri_form = false; big_layers.clear(); }
+  }
   for (int l = 0; l < n_layers; ++l) {
     L[l].tri = !tri_form ? 0 : (L[l].rp <= sp_tridiag_max_rp() ? 1 : 2);
     if (L[l].tri) { L[l].refine = 0; }
-    if (L[l].tri == 2) big_layers.push_back(l);
   }
   if (tri_form) refine_tiles.clear();
   bool cluster_form = !given && !tri_form && ctx->eig_scheme >= 2 && ctx->eig_mode != 0;
@@ -644,33 +673,21 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   struct BandRun { int first, count, form, r_max; };
   std::vector<BandRun> band_runs;
   std::vector<ClusterCta> band_ctas;
-  int band_form = 0;
   if (tri_form && any_big) {
-    std::stable_sort(big_layers.begin(), big_layers.end(), [&](int a, int b) { return L[a].r > L[b].r; });
-    int64_t strips = 0;
-    for (int l : big_layers) strips += sp_band_strips(L[l].r);
-    band_form = sp_band_form(L[big_layers[0]].r, strips);
     for (size_t i = 0; i < big_layers.size();) {
-      const int rm = L[big_layers[i]].r;
-      int lg = 0;
-      while ((1 << lg) < rm) ++lg;
-      int& room_known = ctx->band_capacity[band_form][lg];
-      if (room_known < 0) room_known = sp_band_capacity(band_form, 1 << lg);
-      const int room = room_known;
-      if (room < 1) { tri_form = false; break; }
+      const int rm = L[big_layers[i]].r, room = band_room(ctx, band_form, rm);   // (at least what the largest layer was given above)
       const int fixed = ctx->tri_big_ctas;                           // CTAs per layer asked for (0: chosen here)
       size_t n = 0;
       int used = 0;
       double work = 0.0;
       while (i + n < big_layers.size()) {
-        const int want = fixed > 0 ? std::min(fixed, sp_band_strips(L[big_layers[i + n]].r)) : 1;
+        const int want = fixed > 0 ? std::min({fixed, sp_band_strips(L[big_layers[i + n]].r), room}) : 1;
         if (used + want > room) break;
         used += want;
         const double rr = L[big_layers[i + n]].r;
         work += rr * rr * rr;
         ++n;
       }
-      if (n == 0) { tri_form = false; break; }
       // (a strip's columns are dealt to CTAs as well: four warps' worth of a strip are enough for one)
       const int band_spread = std::max(1, sp_band_parts(band_form) / 4);
       std::vector<int> g(n);
@@ -678,7 +695,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       for (size_t q = 0; q < n; ++q) {
         const double rr = L[big_layers[i + q]].r;
         const int strips = sp_band_strips(L[big_layers[i + q]].r);
-        g[q] = fixed > 0 ? std::min(fixed, strips) : std::max(1, std::min(strips * band_spread, (int)(room * (rr * rr * rr / work))));
+        g[q] = fixed > 0 ? std::min({fixed, strips, room}) : std::max(1, std::min(strips * band_spread, (int)(room * (rr * rr * rr / work))));
         total += g[q];
       }
       for (size_t q = n; total > room; q = q > 1 ? q - 1 : n) if (g[q - 1] > 1) { --g[q - 1]; --total; }   // the minimum of one each went over
@@ -688,7 +705,6 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       band_runs.push_back(run);
       i += n;
     }
-    if (!tri_form) { for (int l = 0; l < n_layers; ++l) L[l].tri = 0; return fail_cuda(ctx, cudaErrorInvalidConfiguration, "occupancy query for the band reduction"); }
   }
   // the tables go to the table cache (device buffer tab_sp, host mirror `tables` with the same offsets), everything
   // the kernels write to the workspace
@@ -876,11 +892,10 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(band reduction)");
       ++n_eig_launch;
     }
-    auto chase_class = [&](int l) { return L[l].r <= 1024 ? 1024 : L[l].r <= 2048 ? 2048 : 4096; };
     for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one class are neighbours)
-      const int of = chase_class(big_layers[i]);
+      const int of = chase_class(L[big_layers[i]].r);
       n = 1;
-      while (i + n < big_layers.size() && chase_class(big_layers[i + n]) == of) ++n;
+      while (i + n < big_layers.size() && chase_class(L[big_layers[i + n]].r) == of) ++n;
       const int c = sp_chase_ctas(of, (int)n, of > 1024 ? chase_room(ctx, of / 256) : 0);
       const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(bulge chase)");
