@@ -122,7 +122,8 @@ typedef struct { float* sigma; float* prob; uint32_t* mask_words; float* short_v
 /* Stage timers (milliseconds of device time, CUDA events on the call's stream) filled while
  * profiling is on.  `launches[i]` counts the kernels of stage i in the last call.  On the
  * tridiagonal route EIG is the Householder reduction alone; the bisection for the eigenvalues
- * is timed with SAMPLE and the vectors of the kept atoms with BACKPROJECT.                    */
+ * is timed with SAMPLE and the vectors of the kept atoms with BACKPROJECT.  EW_REDUCE is the solve
+ * kernel of vectors that take the two-kernel form; the one-kernel form is timed as EW_PACK.  */
 enum { ATOMO_STAGE_GRAM = 0, ATOMO_STAGE_EIG, ATOMO_STAGE_SAMPLE, ATOMO_STAGE_BACKPROJECT,
        ATOMO_STAGE_EW_REDUCE, ATOMO_STAGE_EW_PACK, ATOMO_STAGE_DECODE, ATOMO_N_STAGES };
 

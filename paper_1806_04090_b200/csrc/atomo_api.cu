@@ -1105,21 +1105,37 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs
     B.kind_step = kind_step_word(ATOMO_KIND_ENTRYWISE, step);
     B.begin = begin; B.begin.on = first == 0 ? 1 : 0;
   };
-  auto run_two = [&](int l, int solve_ctas) {
+  auto solve = [&](int l, int solve_ctas) {
     EwBatch<1> B{};
     fill(B, l, 1);
-    return launch_ew_two_kernels(B, solve_ctas, ew_pack_ctas(V[l].n_tiles), st);
+    return launch_ew_solve(B, solve_ctas, ew_pack_ctas(V[l].n_tiles), st);
+  };
+  auto sample_pack = [&](int l) {
+    EwBatch<1> B{};
+    fill(B, l, 1);
+    return launch_ew_sample_pack(B, ew_pack_ctas(V[l].n_tiles), st);
   };
   ctx->ew_last_state.resize(n_vecs); ctx->ew_last_chunks.resize(n_vecs);
   for (int l = 0; l < n_vecs; ++l) { ctx->ew_last_state[l] = V[l].state; ctx->ew_last_chunks[l] = V[l].n_ctas; }
-  int64_t n_launch = 0;
+  // the probabilities of the vectors that take two kernels are a stage of their own; all other encoding is timed as packing
+  int64_t n_launch = 0, n_solve = 0;
+  for (const Run& r : runs) n_solve += r.solve_ctas > 0 ? 1 : 0;
+  if (n_solve > 0) {
+    stage_begin(ctx, ATOMO_STAGE_EW_REDUCE, st);
+    for (const Run& r : runs) {
+      if (r.solve_ctas == 0) continue;
+      const int e = solve(r.first, r.solve_ctas);
+      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(entry-wise solve)");
+      ctx->ew_last_chunks[r.first] = 0;
+    }
+    stage_end(ctx, ATOMO_STAGE_EW_REDUCE, st, n_solve);
+  }
   stage_begin(ctx, ATOMO_STAGE_EW_PACK, st);
   for (const Run& r : runs) {
     int e = 0;
     if (r.solve_ctas > 0) {
-      e = run_two(r.first, r.solve_ctas);
-      ctx->ew_last_chunks[r.first] = 0;
-      n_launch += 2;
+      e = sample_pack(r.first);
+      ++n_launch;
     } else {
       if (r.count == 1) { EwBatch<1> B{}; fill(B, r.first, 1); e = launch_ew_encode(B, r.list, st); }
       else { EwBatch<kEwBatch> B{}; fill(B, r.first, r.count); e = launch_ew_encode(B, r.list, st); }
@@ -1131,7 +1147,8 @@ int atomo_encode_entrywise(atomo_ctx* ctx, const atomo_vec* vecs, int32_t n_vecs
         for (int l = r.first; l < r.first + r.count && e == 0; ++l) {
           V[l].candidates = 0;
           const int ctas = std::min(ew_solve_ctas(V[l].n_tiles), V[l].n_ctas);   // the workspace was carved for that many
-          e = ctas > 0 ? run_two(l, ctas) : (int)cudaErrorCooperativeLaunchTooLarge;
+          e = ctas > 0 ? solve(l, ctas) : (int)cudaErrorCooperativeLaunchTooLarge;
+          if (e == 0) e = sample_pack(l);
           ctx->ew_last_chunks[l] = 0;
           n_launch += 2;
         }

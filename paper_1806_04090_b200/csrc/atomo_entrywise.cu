@@ -1309,12 +1309,14 @@ int ew_solve_ctas(int64_t n_tiles) {
 int ew_pack_ctas(int64_t n_tiles) {
   return (int)std::max<int64_t>((n_tiles + kEwPackTiles - 1) / kEwPackTiles, std::min<int64_t>(n_tiles, (int64_t)ew_sms()));
 }
-int launch_ew_two_kernels(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st) {
+// (the two take the same batch, one after the other)
+int launch_ew_solve(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st) {
   B.v[0].n_ctas = solve_ctas; B.v[0].cta0 = 0;
   void* args[] = {&B, &pack_ctas};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)ew_solve_kernel, dim3((unsigned)solve_ctas), dim3(kEwThreads), args, 0, st);
-  if (e != cudaSuccess) return (int)e;
-  B.v[0].n_ctas = pack_ctas;
+  return (int)cudaLaunchCooperativeKernel((const void*)ew_solve_kernel, dim3((unsigned)solve_ctas), dim3(kEwThreads), args, 0, st);
+}
+int launch_ew_sample_pack(EwBatch<1>& B, int pack_ctas, cudaStream_t st) {
+  B.v[0].n_ctas = pack_ctas; B.v[0].cta0 = 0;
   B.scratch_words = (int)(ew_scratch_bytes(false) / sizeof(uint32_t));
   const int64_t most = (B.v[0].n_tiles + pack_ctas - 1) / pack_ctas;
   ew_sample_pack_kernel<<<(unsigned)pack_ctas, kEwThreads, ew_dyn_bytes((int)most, false), st>>>(B);

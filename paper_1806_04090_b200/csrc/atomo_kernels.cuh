@@ -52,7 +52,8 @@ bool ew_list_pays(int64_t n, int64_t n_tiles, int n_ctas, double s);   // whethe
 template <int N> int launch_ew_encode(EwBatch<N>& B, bool list, cudaStream_t st);       // cudaError_t
 int ew_solve_ctas(int64_t n_tiles);                            // two-kernel form: CTAs of the solve, chunks of the sampling
 int ew_pack_ctas(int64_t n_tiles);
-int launch_ew_two_kernels(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st);   // cudaError_t
+int launch_ew_solve(EwBatch<1>& B, int solve_ctas, int pack_ctas, cudaStream_t st);     // cudaError_t, both
+int launch_ew_sample_pack(EwBatch<1>& B, int pack_ctas, cudaStream_t st);
 template <int N> void launch_ew_decode(const EwDecodeBatch<N>& B, uint32_t n_tiles, cudaStream_t st);
 template <int N> void launch_ew_decode_average(const EwDecodeBatch<N>& B, uint32_t n_tiles, const uint8_t* const* d_payloads,
                                                int n_payloads, cudaStream_t st);
