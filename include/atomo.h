@@ -262,8 +262,9 @@ int atomo_payload_status(atomo_ctx* ctx, const void* payload /*DEVICE*/, int32_t
 /* Descriptor tables (layer descriptors, tile lists, tensor maps, header templates) are kept in device buffers owned by
  * the context and uploaded only when they differ from the previous call's: a loop that calls with the same pointers
  * and shapes every step issues no host-to-device copy in steady state (the payload header travels as a kernel
- * argument).  Counts since atomo_create: calls that had to upload their tables, and calls that found them in place.
- * Host only; either pointer may be NULL.                                                              */
+ * argument).  Counts since atomo_create: calls that had to upload their tables, and calls that found them in place.  A spectral
+ * atomo_decode has no table any more (its layers travel as kernel arguments) and counts as one of the latter; entry-wise
+ * encodes and decodes have none either and are not counted.  Host only; either pointer may be NULL.                                                              */
 int atomo_get_table_uploads(atomo_ctx* ctx, int64_t* uploads /*HOST*/, int64_t* reuses /*HOST*/);
 
 /* --- profiling ------------------------------------------------------------------------------ */

@@ -1241,7 +1241,7 @@ int atomo_decode(atomo_ctx* ctx, int32_t kind, const void* payload, const int64_
     const int n_launch = for_each_ew_decode(pay, cols, out, n_layers, [&](const auto& B, uint32_t tiles) { launch_ew_decode(B, tiles, st); });
     stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   } else {
-    ++ctx->table_reuses;                                           // the layers travel as kernel arguments: nothing to upload
+    ++ctx->table_reuses;                                           // counted as a call with nothing to upload: the layers travel as kernel arguments
     const int n_launch = launch_sp_decode(pay, nullptr, 1, rows, cols, out, n_layers, st);
     stage_end(ctx, ATOMO_STAGE_DECODE, st, n_launch);
   }
