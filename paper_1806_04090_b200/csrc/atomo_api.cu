@@ -44,7 +44,6 @@ struct atomo_ctx {
   uint32_t* h_flag = nullptr;        // pinned: convergence flag / state mirror
   EwLqPart* h_lq = nullptr;          // pinned: results of the l_q sums, written by the GPU
   uint32_t* ew_words = nullptr;      // device: barrier counters of the entry-wise encode (zero between launches), the ticket of the l_q sums
-  cudaEvent_t ev_sync = nullptr;
   // stage timers: one set of events per API call, a ring of kEvRing sets (a set is read out -- its call is long
   // finished by then -- before it is used again), sums since profiling was switched on
   static constexpr int kEvRing = 32;
@@ -316,7 +315,6 @@ int atomo_create(atomo_ctx** out, int device) {
   CK(cudaMallocHost(&ctx->h_lq, kLqResults * sizeof(EwLqPart)));
   CK(cudaMalloc(&ctx->ew_words, kEwWords * sizeof(uint32_t)));
   CK(cudaMemset(ctx->ew_words, 0, kEwWords * sizeof(uint32_t)));
-  CK(cudaEventCreateWithFlags(&ctx->ev_sync, cudaEventDisableTiming));
   for (int r = 0; r < atomo_ctx::kEvRing; ++r)
     for (int i = 0; i < ATOMO_N_STAGES; ++i) { CK(cudaEventCreate(&ctx->ev[r][i][0])); CK(cudaEventCreate(&ctx->ev[r][i][1])); }
   int e = sp_configure();
@@ -336,7 +334,6 @@ int atomo_destroy(atomo_ctx* ctx) {
   table_free(ctx->tab_sp); table_free(ctx->tab_avg);
   if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
   if (ctx->h_lq) cudaFreeHost(ctx->h_lq);
-  if (ctx->ev_sync) cudaEventDestroy(ctx->ev_sync);
   for (int r = 0; r < atomo_ctx::kEvRing; ++r)
     for (int i = 0; i < ATOMO_N_STAGES; ++i) for (int j = 0; j < 2; ++j) if (ctx->ev[r][i][j]) cudaEventDestroy(ctx->ev[r][i][j]);
   delete ctx;
@@ -773,7 +770,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       }
       d.gram_sums = A.take<double>(d.tc ? 0 : (size_t)sp_gram_sums(d.r, d.gram_split));
       d.td_d = A.take<double>(d.tri ? d.rp : 0); d.td_e = A.take<double>(d.tri ? d.rp : 0);
-      d.td_tau = A.take<double>(d.tri ? d.rp : 0); d.lam64 = A.take<double>(d.tri ? d.rp : 0);
+      d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
       d.td_V = A.take<float>(d.tri ? (size_t)d.r * d.td_ldv : 0);
       d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);

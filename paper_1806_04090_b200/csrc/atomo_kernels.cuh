@@ -102,7 +102,6 @@ struct SpLayer {
   // tridiagonal route (short side <= 512): T = Q^T A Q, eigenvalues by bisection, vectors of the kept atoms only
   int tri;                     // this layer takes the tridiagonal route: 1 = registers of a cluster (rp <= 512), 2 = two stages, A in global memory
   double* td_d; double* td_e;  // rp each: diagonal and off-diagonal of T
-  double* td_tau;              // rp: beta_k of the reflectors H_k = I - beta_k v_k v_k^T
   int td_ldv;                  // floats per row of td_V: r rounded up to a multiple of 4 (16-byte rows)
   float* td_V;                 // r x td_ldv: row k = v_k / ||v_k|| (zero up to index k), fp32 for the back-transformation: H_k = I - 2 u u^T
   double* lam64;               // rp: eigenvalues of T, ascending (scaled units); lam holds the same in fp32

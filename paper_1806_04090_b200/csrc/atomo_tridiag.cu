@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
   const SpLayer& L = layers[me.layer];
   const int r = L.r, nc = me.pad, g = me.slot, base = me.base_rank;
   // the layer's pointers in registers: a field read through `layers` inside a loop would be a global load each time
-  double* const td_d = L.td_d; double* const td_e = L.td_e; double* const td_tau = L.td_tau; float* const td_V = L.td_V;
+  double* const td_d = L.td_d; double* const td_e = L.td_e; float* const td_V = L.td_V;
   const float* const gA = L.A; const int64_t lda = L.lda; const int ldv = L.td_ldv;
   const int my_steps = max(r - 2, 0);
   const int row_lo = 32 * g + 4 * w;                          // this warp's rows
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
     if (files) {                                              // reflectors as unit vectors (H = I - 2 u u^T): no range trouble in fp32
       if (jA < r) td_V[(int64_t)q1 * ldv + jA] = (float)(vA * un);
       if (jB < r) td_V[(int64_t)q1 * ldv + jB] = (float)(vB * un);
-      if (tid == 0) { td_e[q1] = alpha; td_tau[q1] = beta; }
+      if (tid == 0) td_e[q1] = alpha;
     }
   }
   cluster.sync();                                             // nobody leaves while a peer may still write here
