@@ -28,12 +28,9 @@ if ROOT not in sys.path:
 METRIC = "gradient elements encoded+decoded/sec"
 UNIT = "elements/s"
 L2_BYTES = 126 * 1024 * 1024
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant kernel, from the ncu captures
-# summarised under profiles/ (None: no capture on file for that kernel and workload)
-NCU_TRAFFIC = {("sp_tridiag_cluster_kernel", "c2"): 5638912,
-               # profiles/entrywise_c4.txt: the encode kernel (2.09 TB/s over 51.9 us) plus the decode kernel (3.74 TB/s over
-               # 24.4 us) of one step at s = 1 %
-               ("entrywise", "c4"): 200_000_000}
+# DRAM bytes of one launch of the dominant kernel (entry-wise: of encode and decode), from the captures summarised in
+# profiles/counters.txt (None: no capture on file for that kernel and workload)
+NCU_TRAFFIC = {("sp_tridiag_cluster_kernel", "c2"): 5_640_000, ("entrywise", "c4"): 161_000_000}
 
 
 def measured_peaks():
@@ -327,7 +324,8 @@ def tridiag_small_flops(shapes):
 
 
 def tridiag_big_bytes(shapes):
-    """Blocked Householder reduction with the matrix in global memory (short sides above 512), fp32 storage: every
+    """What a one-stage Householder reduction in global memory would read (short sides above 512; the two-stage route is measured
+    against band_bytes), fp32 storage: every
     step must read the trailing block once for its matrix-vector product; a symmetric matrix needs one triangle:
     sum over steps of m^2 / 2 entries of 4 bytes = (2/3) r^3 bytes per layer.  (A kernel that reads the full square
     shows twice this as DRAM traffic.)"""
