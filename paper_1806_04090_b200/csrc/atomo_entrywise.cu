@@ -167,15 +167,6 @@ __device__ __forceinline__ void ew_barrier(const EwVec& v, uint32_t target, EwSh
   }
   __syncthreads();
 }
-// At the end of a CTA: it will not look at the vector's barrier again.  The last CTA of the vector leaves both counters at zero, so
-// every launch that runs finds zeros and leaves zeros: a launch that never happened, a replayed graph or a wait that ran out
-// changes nothing for the next one, and the host keeps no count of launches.  (No fence: nothing is handed on but the counters,
-// and a CTA's last poll has returned before its atomic is issued.)
-__device__ __forceinline__ void ew_leave(const EwVec& v) {
-  if (v.n_ctas == 1 || threadIdx.x != kEwThreads - 1) return;
-  if (atomicAdd(v.barrier + 1, 1u) == (uint32_t)v.n_ctas - 1u) { v.barrier[0] = 0u; v.barrier[1] = 0u; }
-}
-
 // ---- pass 1 -------------------------------------------------------------------------------------------------------
 // Sums in short fp32 runs (16 terms per lane and unit), then fp64.  amax ignores NaN (and the sum keeps it), so "some
 // entry is NaN" is "the sum is NaN" and "some entry is infinite" is "amax is infinite": no test per entry.
@@ -434,6 +425,8 @@ __device__ __forceinline__ EwSolved ew_solve(const EwVec& v, const EwChunk& c, c
   r.c = live ? (float)(T / s_cur) : 0.0f;                // weight of kept unsaturated atoms
   return r;
 }
+// what the vector's barrier counts in a solve: every CTA once per exchange
+__device__ __forceinline__ uint32_t ew_arrivals(const EwVec& v, const EwSolved& S) { return v.n_ctas > 1 ? (uint32_t)v.n_ctas * (1u + S.rounds) : 0u; }
 __device__ __forceinline__ void ew_store_state(const EwVec& v, const EwSolved& S) {
   EwState* st = v.state;
   st->T0 = S.T0; st->theta = S.theta; st->amax = S.amax; st->n_sat = S.n_sat; st->rounds = S.rounds;
@@ -599,7 +592,12 @@ __device__ __forceinline__ EwLists ew_lists(const EwVec& v) {
 // the vector has published and adds their counts -- all chunks of a wave finish their decisions together, so nobody waits
 // on a chain.  Returns the counts before this chunk.  The last chunk writes k, the capacity check and the layer header; a
 // wait that runs out raises ATOMO_ERR_TIMEOUT.  Every thread of the CTA passes the same `total`.
-__device__ __forceinline__ unsigned long long ew_publish(const EwVec& v, const EwChunk& c, const EwSolved& S, const EwLists& o,
+//
+// One-kernel form: that CTA also leaves the vector's barrier counter at zero.  Every CTA has published, so nobody looks at the barrier
+// any more, and `arrivals` is what it must have counted.  So every launch finds a zero, whatever the host launched before it, in
+// a replayed graph too; a counter that was not zero (after a wait that ran out) shows as ATOMO_ERR_TIMEOUT, once.  (Counting the
+// CTAs out with an atomic each at their ends: 1.5 M elements 24.6 us instead of 23.9.)
+__device__ __forceinline__ unsigned long long ew_publish(const EwVec& v, const EwChunk& c, const EwSolved& S, const uint32_t arrivals, const EwLists& o,
                                                          const unsigned long long total, EwShared& sh) {
   const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
   unsigned long long base = 0;
@@ -628,13 +626,19 @@ __device__ __forceinline__ unsigned long long ew_publish(const EwVec& v, const E
   if (tid == 0) {
     if (sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
     if (c.tile0 + c.n_my == v.n_tiles) {                   // the last chunk knows k: capacity check, layer header
+      atomo_layer_header* h = v.hdr;
       const unsigned long long all = base + total;
       const uint64_t k = all & 0xFFFFFFFFull, k_sat = all >> 32, k_list = o.list_of(all);
-      atomo_layer_header* h = v.hdr;
+      uint32_t seen, status;                               // (both loads on their way before either is looked at)
+      asm volatile("ld.volatile.global.u32 %0, [%2];\n\tld.volatile.global.u32 %1, [%3];" : "=&r"(seen), "=r"(status) : "l"(v.barrier), "l"(&h->status) : "memory");
+      if (arrivals > 0) *(volatile uint32_t*)v.barrier = 0u;
       h->n_sat = S.n_sat; h->c = S.c; h->l1 = S.T0; h->sweeps = S.rounds;
-      if (S.nonfinite) raise_status(h, ATOMO_ERR_NONFINITE);
-      else if (k_list > (uint64_t)v.k_cap || (o.compact && k_sat > (uint64_t)v.sat_cap)) raise_status(h, ATOMO_ERR_CAPACITY);
-      const bool ok = *(volatile uint32_t*)&h->status == ATOMO_OK;
+      uint32_t bad = ATOMO_OK;
+      if (sh.fail || (arrivals > 0 && seen != arrivals)) bad = ATOMO_ERR_TIMEOUT;
+      else if (S.nonfinite) bad = ATOMO_ERR_NONFINITE;
+      else if (k_list > (uint64_t)v.k_cap || (o.compact && k_sat > (uint64_t)v.sat_cap)) bad = ATOMO_ERR_CAPACITY;
+      if (bad != ATOMO_OK) raise_status(h, bad);
+      const bool ok = bad == ATOMO_OK && status == ATOMO_OK;
       h->k = ok ? (uint32_t)k : 0u;
       if (o.compact) h->n_sat = ok ? (uint32_t)k_sat : 0u; // the length of the saturated list
       o.table[v.n_tiles] = ok ? (uint32_t)k_list : 0u;
@@ -666,7 +670,7 @@ __device__ __forceinline__ void ew_mask_out(const EwVec& v, const EwChunk& c, co
 // Compaction of the decisions taken on the list: a scan over the counts of 32 atoms each, then every kept atom finds its own
 // place from the prefix and the bits before it, and stores its entry directly.  `n_blocks`: what ew_decide_list returned;
 // pref: kEwPrefixes words per tile of the chunk.
-__device__ __forceinline__ void ew_pack_list(const EwVec& v, const EwChunk& c, const EwSolved& S, const EwCands& C, const uint32_t n_blocks,
+__device__ __forceinline__ void ew_pack_list(const EwVec& v, const EwChunk& c, const EwSolved& S, const uint32_t arrivals, const EwCands& C, const uint32_t n_blocks,
                                              const uint8_t* __restrict__ code, uint32_t* __restrict__ pref, EwShared& sh) {
   const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
   const EwLists o = ew_lists(v);
@@ -687,7 +691,7 @@ __device__ __forceinline__ void ew_pack_list(const EwVec& v, const EwChunk& c, c
   const uint32_t total = __reduce_add_sync(0xffffffffu, part);
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < w ? part : 0u) + inc - cnt;
   for (int at = g0; at < g1; ++at) pref[at] += before;
-  const uint64_t base = ew_publish(v, c, S, o, total, sh);
+  const uint64_t base = ew_publish(v, c, S, arrivals, o, total, sh);
   __syncthreads();                                         // pref is complete
   if (v.n_words > 0) ew_mask_out(v, c, code);
   for (int t = tid; t < c.n_my; t += kEwThreads) o.table[c.tile0 + t] = (uint32_t)min(base + pref[t * kEwPrefixes], (uint64_t)0xFFFFFFFFull);
@@ -718,7 +722,7 @@ __device__ __forceinline__ void ew_pack_list(const EwVec& v, const EwChunk& c, c
 // the window leaves with coalesced stores (direct 4-byte stores from every thread's own run cost an L2 request each).  A
 // strip with more kept atoms than the window holds is written 32 atoms at a time, an atom per lane.  The signs in the code
 // bytes make a second read of the kept atoms' values unnecessary, except for saturated ones.
-__device__ __forceinline__ void ew_pack(const EwVec& v, const EwChunk& c, const EwSolved& S, const uint8_t* __restrict__ code,
+__device__ __forceinline__ void ew_pack(const EwVec& v, const EwChunk& c, const EwSolved& S, const uint32_t arrivals, const uint8_t* __restrict__ code,
                                         uint32_t* __restrict__ stage, EwShared& sh) {
   const int tid = threadIdx.x, lane = tid % kWarp, w = tid / kWarp;
   const EwLists o = ew_lists(v);
@@ -737,7 +741,7 @@ __device__ __forceinline__ void ew_pack(const EwVec& v, const EwChunk& c, const 
   unsigned long long total = sh.scan[lane], run = lane < w ? total : 0ull;   // of the chunk; of the earlier warps
 #pragma unroll
   for (int q = 16; q > 0; q >>= 1) { total += __shfl_xor_sync(0xffffffffu, total, q); run += __shfl_xor_sync(0xffffffffu, run, q); }
-  run += ew_publish(v, c, S, o, total, sh);
+  run += ew_publish(v, c, S, arrivals, o, total, sh);
   if (v.n_words > 0) ew_mask_out(v, c, code);
   // the warp's window: atom inside the strip | saturated << 14 | sign << 15
   uint16_t* const win = reinterpret_cast<uint16_t*>(stage) + w * kEwStage;
@@ -876,8 +880,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
       for (int u = 0; u < 4; ++u) ew_block_decide(c, unit, u, x[u], wd[u], d, code);
     }
     __syncthreads();
-    ew_pack(v, c, S, code, scratch, sh);
-    ew_leave(v);
+    ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
     return;
   }
   if (v.candidates) {
@@ -898,13 +901,12 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
       if (tid == 0) atomicAdd(&v.state->list_chunks, 1u);
       const uint32_t n_blocks = ew_decide_list(v, c, d, B.key, B.kind_step, cands, code);
       __syncthreads();
-      ew_pack_list(v, c, S, cands, n_blocks, code, reinterpret_cast<uint32_t*>(code + c.n_my * kEwBlocks), sh);
+      ew_pack_list(v, c, S, ew_arrivals(v, S), cands, n_blocks, code, reinterpret_cast<uint32_t*>(code + c.n_my * kEwBlocks), sh);
     } else {
       ew_decide_memory(v, c, d, B.key, B.kind_step, sh, code);
       __syncthreads();
-      ew_pack(v, c, S, code, scratch, sh);
+      ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
     }
-    ew_leave(v);
     return;
   }
   EwBigList big{scratch, 0u, 0.0f, 0.0};
@@ -918,8 +920,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
   if (c.index == 0 && tid == 0) ew_store_state(v, S);
   ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
   __syncthreads();
-  ew_pack(v, c, S, code, scratch, sh);
-  ew_leave(v);
+  ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
 }
 
 // The two-kernel form: the solve leaves its result in the state record; a CTA of the second kernel takes the next chunk of
@@ -945,7 +946,8 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_solve_kernel(const __grid_co
   }, sh);
   if (blockIdx.x == 0 && tid == 0) ew_store_state(v, S);
   if (tid == 0 && sh.fail) raise_status(v.hdr, ATOMO_ERR_TIMEOUT);
-  ew_leave(v);
+  // nobody publishes here: the CTAs count themselves out, and the last one leaves both counters at zero
+  if (v.n_ctas > 1 && tid == 0 && atomicAdd(v.barrier + 1, 1u) == (uint32_t)v.n_ctas - 1u) { v.barrier[0] = 0u; v.barrier[1] = 0u; }
 }
 
 __global__ void __launch_bounds__(kEwThreads, 1) ew_sample_pack_kernel(const __grid_constant__ EwBatch<1> B) {
@@ -963,7 +965,7 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_sample_pack_kernel(const __g
   uint8_t* const code = reinterpret_cast<uint8_t*>(ew_smem + B.scratch_words);
   ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
   __syncthreads();
-  ew_pack(v, c, S, code, ew_smem, sh);
+  ew_pack(v, c, S, 0u, code, ew_smem, sh);
 }
 
 // ---- decode -------------------------------------------------------------------------------------

@@ -9,7 +9,7 @@ constexpr int kEwMaxRounds = 64;      // water-filling rounds; Algorithm 1 satur
                                       // a round usually takes many at once
 
 constexpr int kEwBatch = 24;          // vectors per launch (their descriptors travel as a kernel argument)
-constexpr int kEwBarrierStride = 32;  // words between the barrier counters of two vectors (a line each: arrivals, CTAs that are done with them)
+constexpr int kEwBarrierStride = 32;  // words between the barrier counters of two vectors (a line each: arrivals; two-kernel form: CTAs that are done with them)
 
 struct EwPartial { double sum; float amax; uint32_t cnt; };
 
@@ -31,7 +31,7 @@ struct EwVec {
   int n_ctas, cta0;                                            // chunks (CTAs) of this vector, its first CTA in the launch
   EwPartial* partials; EwState* state;                         // workspace: [3][n_ctas], one record
   uint64_t* chunk_status;                                      // [chunks] ready flag (bit 63) | saturated << 32 | kept atoms of the chunk
-  uint32_t* barrier; uint32_t* ticket;                         // arrivals at the vector's barriers, CTAs past the last one; next chunk (two-kernel form)
+  uint32_t* barrier; uint32_t* ticket;                         // arrivals at the vector's barriers; next chunk (two-kernel form)
   uint32_t* mask_words; float* prob_out; int64_t n_words;      // debug outputs or nullptr / 0
 };
 struct EwBegin { atomo_payload_header gh; int on; };           // the payload header, written by the call's first launch
