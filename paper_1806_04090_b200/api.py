@@ -279,9 +279,8 @@ def atomo_decode_spectral_static(payload: "Payload", out: Sequence[torch.Tensor]
                                  stream: Optional[torch.cuda.Stream] = None) -> List[torch.Tensor]:
     """Spectral decode that allocates nothing on the device: for processes whose framework
     allocator owns the whole GPU, or that cannot take cudaMalloc's device-wide synchronisation
-    where they decode.  The caller supplies the output tensors; the per-call tables live in a fixed
-    array inside the library (limits: 64 layers, 8192 output tiles of 64 x 1024).  Calls on one
-    device share that array, so they must not overlap on the GPU.  Every output must be a contiguous
+    where they decode.  The caller supplies the output tensors; the layers' descriptors travel as
+    kernel arguments (limits: 64 layers, 8192 output tiles of 64 x 1024), so calls share no state.  Every output must be a contiguous
     fp32 CUDA tensor on the payload's device with exactly rows * cols elements: the kernel writes all
     of them through the raw pointer, so anything else is refused here, before the C call."""
     lib = load_library()
@@ -303,7 +302,7 @@ def atomo_decode_spectral_static(payload: "Payload", out: Sequence[torch.Tensor]
                                           ctypes.c_void_p(s.cuda_stream))
     if rc != 0:
         raise AtomoError(rc, "atomo_decode_spectral_static",
-                         "batch exceeds the fixed table (64 layers / 8192 tiles)" if rc == 3 else "")
+                         "batch exceeds the limits (64 layers / 8192 tiles)" if rc == 3 else "")
     return list(out)
 
 

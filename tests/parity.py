@@ -22,8 +22,8 @@ GAP_MIN = 1e-3          # an atom's rank-one term is comparable across two SVDs 
 
 # Calibrated per route and size (tests/test_gpu_gap_certificate.py measures err <= floor + c / gap on seeds of its own):
 # on the tridiagonal routes the vectors come from an fp64 factorisation of T, and c is 2e-10 ... 4e-10 up to a short side
-# of 512 (fp64 reduction) and 9e-9 at 1024 (fp32 storage): a gap of 4e-6 resp. 9e-5 would do for the 1e-4 bar; the values
-# below keep a factor of 2.5 to 3 on top.  The Jacobi routes and short sides above 1024 keep the Gram matrix's own bound.
+# of 512 (fp64 reduction) and 6e-9 at 1024 (fp32 storage of the matrix): a gap of 4e-6 resp. 6e-5 would do for the 1e-4 bar; the
+# values below keep a factor of 2.5 to 5 on top.  The Jacobi routes and short sides above 1024 keep the Gram matrix's own bound.
 GAP_MIN_TRIDIAG_512 = 1e-5
 GAP_MIN_TRIDIAG_1024 = 3e-4
 
