@@ -546,132 +546,205 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
 }
 
 // ---- stage 2: band -> tridiagonal -----------------------------------------------------------------------------------------
-// Bulge chasing with reflectors of length eight.  Sweep j brings column j to tridiagonal form: step 0 reflects the rows
-// R_0 = j+1 .. j+8 of column j; applied from both sides this fills the block below (rows R_1, columns R_0), whose first column
-// step 1 reflects, and so on down the band (rows R_t = j+1+8t .. j+8+8t).  A step works on three 8 x 8 blocks: rows R_t x
-// columns R_{t-1} from the left (step 0: column j), the diagonal block R_t from both sides, rows R_{t+1} x columns R_t from
-// the right.  Step t of sweep j+1 needs step t+2 of sweep j, so sweep j runs step tick - 3 j: all active sweeps (one in 23
-// columns) advance together, separated by a barrier per tick, 3 r ticks in all.  No flags, no waits.
-// The band sits in shared memory as fp64, 15 sub-diagonals (eight and the fill) per column; sixteen lanes take a step, so that a
-// warp advances two sweeps.  Lane (k, h) holds column k, rows h, h+2, h+4, h+6 of the left and of the diagonal block and row k,
-// those columns of the lower one: every product with the reflector is four multiply-adds and one exchange (only u^T D u
-// takes three more), and all addresses are one base plus offsets that never change.  What lies outside the matrix is stored
-// as zeros, lanes without a step work on a dummy block of zeros: no bounds tests.
-// Bound: shared memory where a CTA has 1024 columns (23 warps), else the latency of the step's chain.
-// (The shared-memory pipe, which the exchanges use too, takes about 110 cycles per warp and tick: 24 loads and stores of
-// eight bytes, 36 shuffles.)  Larger short sides are spread over a cluster, down to 256 columns per CTA.  A cluster barrier and the reads of a
+// Bulge chasing with reflectors of length eight.  Sweep j brings column j to tridiagonal form: step -1 forms the reflector of
+// the column's rows R_0 = j+1 .. j+8; step t = 0, 1, .. applies the reflector of the rows R_t = j+1+8t .. j+8+8t from both sides
+// to their diagonal block D and from the right to the block Bn below it (rows R_{t+1}), which this fills, forms the reflector of
+// the first column of Bn and applies it to Bn from the left, so that the next step's block starts as the band does.  A step
+// therefore touches the columns R_t only, and step t of sweep j+1 needs step t+1 of sweep j and nothing later: sweep j runs step
+// tick - 2 j - 1, all active sweeps (one in 15 columns) advance together, separated by a barrier per tick, 2 r ticks in all.
+// (With the left product in the step after, each step reached into three blocks and the sweeps had to keep three ticks
+// apart, one in 23 columns.)  No flags, no waits.  Measured, before | now: two layers of 4096 rows 14.1 | 8.0 ms, one of 1023 2.12 |
+// 1.42, 96 of 1024 3.18 | 2.09; of the first, 4 ms come from the closer sweeps and 2 from the two halves below.
+// The band sits in shared memory as fp64, 15 sub-diagonals (eight and the fill) per column, and four more words: a reflector
+// waits for its step in those of the block's first two columns, those of the next two carry w between the lanes of D.  A step is
+// two independent halves, D and Bn, each taken by four lanes of different warps: what bounds a tick where few sweeps are at work
+// is the number of instructions that one warp issues one after the other (about four cycles each).  Lane k holds the rows k and
+// k + 4 of its block, products with the reflector from the right are its own, and all addresses are one base plus offsets that
+// never change.  (Eight lanes instead of four: half the instructions of a warp, but every vector is handed to twice as many
+// lanes, and shared memory bounds a CTA with 1024 columns at work.)  A sweep stays with its lanes.  What lies outside the
+// matrix is stored as zeros, lanes without a step work on a dummy block of zeros: no bounds tests.
+// Larger short sides are spread over a cluster, down to 256 columns per CTA.  A cluster barrier and the reads of a
 // neighbour's memory in every tick took 4.4 us per tick, three times the step itself; so a CTA also keeps copies of the
-// columns next to its own, works on them as well, and fetches them afresh every kChTicks ticks.  What it lacks spoils these
-// columns from their outer ends inwards: by eight columns a tick from above (a sweep moves down by a block), by fifteen from
-// below (a sweep that misses its predecessor's work spoils its own block, 15 columns further up), hence the widths.
+// columns next to its own, works on them as well, and gets them afresh every kChTicks ticks: its neighbours store them into
+// a buffer of its own, two in turn, so that one cluster barrier separates what is stored from what is read.  What it lacks spoils these
+// columns from their outer ends inwards: by eight columns a tick from above (a sweep moves down by a block), by seven from
+// below (a sweep that misses its predecessor's work spoils its own block, seven columns further up), hence the widths.
 namespace {
-constexpr int kChLd = 19;                     // doubles per column, 16 in use: a half-warp's loads of a left block meet 16 different banks
+constexpr int kChLd = 20;                     // doubles per column: 16 of the band and four more; a half-warp's loads of D and Bn meet 16 different banks
+constexpr int kChVec = 16;                    // where those start
 constexpr int kChTicks = 8;                   // ticks between two exchanges
 template <int C, int COLS> struct ChForm {     // CTAs per layer, columns per CTA
-  static constexpr int kAbove = C > 1 ? 8 * kChTicks + 8 : 0, kBelow = C > 1 ? 15 * kChTicks + 16 : 16;
-  static constexpr int kLocal = kAbove + COLS + kBelow;   // columns in shared memory, then 24 of zeros
-  static constexpr int kThreads = ((kLocal + 22) / 23 + 2) / 2 * 32;   // two half-warps per 46 columns
-  static constexpr size_t kSmem = (size_t)(kLocal + 24) * kChLd * sizeof(double);
+  static constexpr int kAbove = C > 1 ? 8 * kChTicks + 8 : 0, kBelow = C > 1 ? 7 * kChTicks + 8 : 16;
+  static constexpr int kLocal = kAbove + COLS + kBelow;   // columns in shared memory, then eight of zeros
+  static constexpr int kSteps = (kLocal - 3) / 15 + 1;    // sweeps that can be at work on them
+  static constexpr int kWarps = (kSteps + 7) / 8;         // of either half
+  static_assert(15 * 8 * kWarps >= kLocal - 2, "a sweep is taken up before its first step");
+  static constexpr int kThreads = 2 * 32 * kWarps;
+  static constexpr int kHalo = C > 1 ? kAbove + kBelow : 0;
+  // the neighbours' columns arrive in two buffers in turn where there is room for them
+  static constexpr bool kPush = (size_t)(kLocal + kBw + 2 * kHalo) * kChLd * sizeof(double) <= 227 * 1024;
+  static constexpr size_t kSmem = (size_t)(kLocal + kBw + (kPush ? 2 * kHalo : 0)) * kChLd * sizeof(double);
 };
+// sum over the four lanes of a step
+__device__ __forceinline__ double ch_sum(double x) {
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x + __shfl_xor_sync(0xffffffffu, x, 2);
+}
+__device__ __forceinline__ double ch_dot(const double (&a)[8], const double (&u)[8]) {
+  return (fma(a[0], u[0], a[1] * u[1]) + fma(a[2], u[2], a[3] * u[3])) + (fma(a[4], u[4], a[5] * u[5]) + fma(a[6], u[6], a[7] * u[7]));
+}
+// eight doubles from the spare words of two neighbouring columns
+__device__ __forceinline__ void ch_vec(const double* p, double (&u)[8]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const double2 a = *reinterpret_cast<const double2*>(p + h * kChLd), b = *reinterpret_cast<const double2*>(p + h * kChLd + 2);
+    u[4 * h] = a.x; u[4 * h + 1] = a.y; u[4 * h + 2] = b.x; u[4 * h + 3] = b.y;
+  }
+}
+// n double2 from src to dst, either of them perhaps in a neighbour's shared memory
+template <int THREADS, int N>
+__device__ __forceinline__ void ch_copy(double* dst, const double* src) {
+  constexpr int kMine = (N + THREADS - 1) / THREADS;
+#pragma unroll 8
+  for (int c = 0; c < kMine; ++c) {
+    const int q = threadIdx.x + c * THREADS;
+    if (q < N) reinterpret_cast<double2*>(dst)[q] = reinterpret_cast<const double2*>(src)[q];
+  }
+}
 }  // namespace
 
 template <int C, int COLS>
 __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(const SpLayer* __restrict__ layers, const int* __restrict__ list) {
-  constexpr int kAbove = ChForm<C, COLS>::kAbove, kLocal = ChForm<C, COLS>::kLocal, kThreads = ChForm<C, COLS>::kThreads;
+  using F = ChForm<C, COLS>;
+  constexpr int kAbove = F::kAbove, kBelow = F::kBelow, kLocal = F::kLocal, kThreads = F::kThreads, kSlots = 8 * F::kWarps;
   extern __shared__ __align__(16) double ch_smem[];
   const SpLayer& L = layers[list[blockIdx.x / C]];
   const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
   const int tid = threadIdx.x, lane = tid % 32;
   const int r = L.r;
   const double* const gB = L.bd_band;
-  double* const gV2 = L.bd_V2;
-  const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that gV2 has room for
+  const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that L.bd_V2 has room for
   const int col0 = rank * COLS, lo = col0 - kAbove;       // first own column, first column in shared memory
-  const double *above = ch_smem, *below = ch_smem;           // the neighbours' shared memory
+  double* const s_in = ch_smem + (kLocal + kBw) * kChLd;     // [2][kHalo] columns from the neighbours
+  double *above = ch_smem, *below = ch_smem;                 // the neighbours' shared memory
   if (C > 1) {
     cg::cluster_group cluster = cg::this_cluster();
     above = cluster.map_shared_rank(ch_smem, max(rank - 1, 0));
     below = cluster.map_shared_rank(ch_smem, min(rank + 1, C - 1));
   }
-  for (int q = tid; q < (kLocal + 24) * kChLd; q += kThreads) {
+  for (int q = tid; q < (kLocal + kBw) * kChLd; q += kThreads) {
     const int j = lo + q / kChLd, d = q % kChLd;
     ch_smem[q] = q / kChLd < kLocal && j >= 0 && j < r && d <= kBw && j + d < r ? gB[(int64_t)j * (kBw + 1) + d] : 0.0;
   }
   if (C > 1) cg::this_cluster().sync(); else __syncthreads();
-  const int half = tid / 16, k = tid & 7, h = (tid >> 3) & 1, base_lane = lane & 16;
-  // offsets of this lane's entries: left block from (first column, first row), diagonal and lower block from (start, start)
-  int od[4];
+  const bool diag = tid >= kThreads / 2;                     // this warp's half of a step: D, or Bn
+  const int k = tid & 3;
+  // offsets of the rows k and k + 4 of D from its first diagonal entry (rows of Bn: on + (kChLd - 1) e, four further down)
+  int od[2][8];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) { const int e = 2 * q + h; od[q] = e >= k ? (kChLd - 1) * k + e : (kChLd - 1) * e + k; }
-  const int ob = (kChLd - 1) * k + h, on = (kChLd - 1) * h + 8 + k;
-  const int ticks = 3 * (r - 3) + 1;                         // (no sweep for r < 3)
+  for (int e = 0; e < 8; ++e) {
+    od[0][e] = e <= k ? (kChLd - 1) * e + k : (kChLd - 1) * k + e;
+    od[1][e] = e <= k + 4 ? (kChLd - 1) * e + k + 4 : (kChLd - 1) * (k + 4) + e;
+  }
+  const int on = kBw + k;
+  const int ticks = max(2 * r - 4, 0);                       // (no sweep for r < 3)
+  constexpr int kLast = kLocal - kBw - 2;                    // last local start whose columns, and the next block's first two, are all here
+  // sweep j's step t = tick - 2 j - 1 starts at row j + 1 + 8 t = 8 tick - 7 - 15 j (step -1: column j, seven further down).
+  // Lanes go on with the sweep kSlots further when theirs has left the columns that are here.
+  int j = tid % (kThreads / 2) / 4, t = -2 * j - 1, start = -7 - lo - 15 * j;   // (start: local)
+  double* to2 = L.bd_V2 + ((int64_t)j * ns + t + 1) * kBw + k;   // where the reflector of step t + 1 goes
   for (int tick = 0; tick < ticks; ++tick) {
-    if (C > 1 && tick % kChTicks == 0 && tick > 0) {
+    if (C > 1 && tick % kChTicks == 0 && tick > 0) {         // every CTA's own columns are up to date
       cg::cluster_group cluster = cg::this_cluster();
-      cluster.sync();                                        // every CTA's own columns are up to date
-      if (rank > 0)
-        for (int q = tid; q < kAbove * 16; q += kThreads) ch_smem[(q / 16) * kChLd + q % 16] = above[(COLS + q / 16) * kChLd + q % 16];
-      if (rank < C - 1)
-        for (int q = tid; q < (kLocal - kAbove - COLS) * 16; q += kThreads)
-          ch_smem[(kAbove + COLS + q / 16) * kChLd + q % 16] = below[(kAbove + q / 16) * kChLd + q % 16];
-      cluster.sync();                                        // copies taken before anybody goes on
+      if (F::kPush) {
+        double* const in = s_in + (tick / kChTicks & 1) * (F::kHalo * kChLd);
+        const int64_t away = in - ch_smem;
+        if (rank > 0) ch_copy<kThreads, kBelow * kChLd / 2>(above + away + kAbove * kChLd, ch_smem + kAbove * kChLd);
+        if (rank < C - 1) ch_copy<kThreads, kAbove * kChLd / 2>(below + away, ch_smem + COLS * kChLd);
+        cluster.sync();
+        if (rank > 0) ch_copy<kThreads, kAbove * kChLd / 2>(ch_smem, in);
+        if (rank < C - 1) ch_copy<kThreads, kBelow * kChLd / 2>(ch_smem + (kAbove + COLS) * kChLd, in + kAbove * kChLd);
+        __syncthreads();
+      } else {
+        cluster.sync();
+        if (rank > 0) ch_copy<kThreads, kAbove * kChLd / 2>(ch_smem, above + COLS * kChLd);
+        if (rank < C - 1) ch_copy<kThreads, kBelow * kChLd / 2>(ch_smem + (kAbove + COLS) * kChLd, below + kAbove * kChLd);
+        cluster.sync();                                      // copies taken before anybody goes on
+      }
     }
-    // sweep j's step t = tick - 3 j starts at row j + 1 + 8 t = 8 tick + 1 - 23 j
-    const int top = 8 * tick + 1, last = lo + kLocal - kBw;  // last start whose columns are all here
-    const int j = (top > last ? (top - last + 22) / 23 : 0) + half;
-    const int start = top - 23 * j, t = tick - 3 * j;
-    const int prev = t > 0 ? start - kBw : j;                // first column of the block to the left
-    const bool active = j <= r - 3 && t >= 0 && prev >= lo && start <= r - 2;
-    if (__any_sync(0xffffffffu, active)) {
-      double* const pd = ch_smem + (active ? start - lo : kLocal + 8) * kChLd;
-      // step 0 has a left block of one column; its other lanes take the zeros
-      double* const pb = active && (t > 0 || k == 0) ? ch_smem + (prev - lo) * kChLd + (start - prev) + ob : ch_smem + kLocal * kChLd + 8 + ob;
-      double bl[4], dd[4], bn[4];
+    const bool first = t == -1;
+    const bool active = j <= r - 3 && t >= -1 && start <= kLast && (first ? start + 7 : start) >= 0 && start + lo <= r - 2;
+    if (diag) {
+      if (__any_sync(0xffffffffu, active && !first)) {       // D - u w^T - w u^T, w = 2 (y - s u), y = D u, s = u^T y
+        double* const pd = ch_smem + (active && !first ? start : kLocal) * kChLd;
+        double* const pu = pd + kChVec;
+        double u[8], dd[2][8], we[8];
+        ch_vec(pu, u);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { bl[q] = pb[2 * q]; dd[q] = pd[od[q]]; bn[q] = pd[on + 2 * (kChLd - 1) * q]; }
-      // reflector of the left block's first column (lanes k == 0)
-      double u[4];
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) u[q] = __shfl_sync(0xffffffffu, bl[q], lane & 24);
-      double nx2 = fma(u[0], u[0], u[1] * u[1]) + fma(u[2], u[2], u[3] * u[3]);
-      const double x0 = __shfl_sync(0xffffffffu, u[0], base_lane);
-      nx2 += __shfl_xor_sync(0xffffffffu, nx2, 8);
-      double alpha = 0.0, us = 0.0;
-      if (nx2 > 1.0e-290) {
-        const double nx = nx2 * rsqrt(nx2);
-        alpha = -copysign(nx, x0);
-        us = rsqrt(2.0 * fma(fabs(x0), nx, nx2));            // 1 / ||v||
+          for (int e = 0; e < 8; ++e) dd[h][e] = pd[od[h][e]];
+        const double uk[2] = {pu[k], pu[kChLd + k]};         // entries k and k + 4
+        const double y[2] = {ch_dot(dd[0], u), ch_dot(dd[1], u)};
+        const double s = ch_sum(fma(uk[0], y[0], uk[1] * y[1]));
+        const double wk[2] = {2.0 * fma(-s, uk[0], y[0]), 2.0 * fma(-s, uk[1], y[1])};
+        pu[2 * kChLd + k] = wk[0]; pu[3 * kChLd + k] = wk[1];
+        __syncwarp();
+        ch_vec(pu + 2 * kChLd, we);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int e = 0; e < 8; ++e) if (e <= k + 4 * h) pd[od[h][e]] = fma(-u[e], wk[h], fma(-we[e], uk[h], dd[h][e]));
       }
-      if (h == 0) u[0] -= alpha;
+    } else if (__any_sync(0xffffffffu, active)) {
+      double* const pd = ch_smem + (active && !first ? start : kLocal) * kChLd;
+      double* const pn = pd + on;
+      double* const pb = active && first ? ch_smem + (start + 7) * kChLd + 1 + k : pn;   // Bn's first column (step -1: column j)
+      double u[8], bn[2][8];
+      ch_vec(pd + kChVec, u);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) u[q] *= us;                // entries h, h+2, h+4, h+6 of the unit vector; 0 for a zero column (H = I)
-      const double mine = (k & 4) ? ((k & 2) ? u[3] : u[2]) : ((k & 2) ? u[1] : u[0]), theirs = __shfl_xor_sync(0xffffffffu, mine, 8);
-      const double uk = (k & 1) == h ? mine : theirs;       // entry k
-      double z = fma(u[0], bl[0], u[1] * bl[1]) + fma(u[2], bl[2], u[3] * bl[3]);     // u^T Bl, column k
-      double y = fma(u[0], dd[0], u[1] * dd[1]) + fma(u[2], dd[2], u[3] * dd[3]);     // D u, entry k
-      double p = fma(u[0], bn[0], u[1] * bn[1]) + fma(u[2], bn[2], u[3] * bn[3]);     // Bn u, row k
-      z += __shfl_xor_sync(0xffffffffu, z, 8);
-      y += __shfl_xor_sync(0xffffffffu, y, 8);
-      p += __shfl_xor_sync(0xffffffffu, p, 8);
-      double s = uk * y;
+      for (int h = 0; h < 2; ++h) {
+        bn[h][0] = pb[4 * h];
 #pragma unroll
-      for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const double wk = 2.0 * fma(-s, uk, y);                // D - u w^T - w u^T, w = 2 (y - s u)
-      z *= -2.0; p *= -2.0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double we = __shfl_sync(0xffffffffu, wk, base_lane + 2 * q + h);
-        pb[2 * q] = k == 0 ? (h == 0 && q == 0 ? alpha : 0.0) : fma(u[q], z, bl[q]);
-        if (2 * q + h >= k) pd[od[q]] = fma(-u[q], wk, fma(-we, uk, dd[q]));
-        pd[on + 2 * (kChLd - 1) * q] = fma(p, u[q], bn[q]);
+        for (int e = 1; e < 8; ++e) bn[h][e] = pn[(kChLd - 1) * e + 4 * h];
       }
-      if (active && h == 0 && prev >= col0 && prev < col0 + COLS) gV2[((int64_t)j * ns + t) * kBw + k] = uk;
+      // from the right, and the norm of what is now the first column
+      const double p[2] = {-2.0 * ch_dot(bn[0], u), -2.0 * ch_dot(bn[1], u)};
+      const double x[2] = {fma(p[0], u[0], bn[0][0]), fma(p[1], u[0], bn[1][0])};
+      const double nx2 = ch_sum(fma(x[0], x[0], x[1] * x[1])), x0 = __shfl_sync(0xffffffffu, x[0], lane & 28);
+#pragma unroll
+      for (int e = 1; e < 8; ++e) { bn[0][e] = fma(p[0], u[e], bn[0][e]); bn[1][e] = fma(p[1], u[e], bn[1][e]); }
+      // the next block's reflector (H = I for a zero column, or where it has one row only): v = x - alpha e_0, v^T v / 2 = half
+      const bool more = start + lo + kBw <= r - 2, act = nx2 > 1.0e-290 && more;
+      const double nx = nx2 * rsqrt(nx2);
+      const double alpha = act ? -copysign(nx, x0) : x0;
+      const double v[2] = {act ? (k == 0 ? x[0] - alpha : x[0]) : 0.0 * x[0], act ? x[1] : 0.0 * x[1]};
+      const double us = act ? rsqrt(2.0 * fma(fabs(x0), nx, nx2)) : 0.0;      // 1 / ||v||
+      double z[8];                                           // v^T Bn
+#pragma unroll
+      for (int e = 1; e < 8; ++e) z[e] = ch_sum(fma(v[0], bn[0][e], v[1] * bn[1][e]));
+      const double un[2] = {v[0] * us, v[1] * us};           // entries k and k + 4 of the unit vector
+      const double c[2] = {-2.0 * us * un[0], -2.0 * us * un[1]};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        pb[4 * h] = k == 0 && h == 0 ? alpha : 0.0;
+#pragma unroll
+        for (int e = 1; e < 8; ++e) pn[(kChLd - 1) * e + 4 * h] = fma(z[e], c[h], bn[h][e]);
+      }
+      if (active) {
+        double* const to = ch_smem + (start + kBw) * kChLd + kChVec + k;
+        to[0] = un[0]; to[kChLd] = un[1];
+        const int own = (first ? start + 7 : start) - kAbove;
+        if (more && own >= 0 && own < COLS) { to2[0] = un[0]; to2[4] = un[1]; }
+      }
     }
     __syncthreads();
+    ++t; start += kBw; to2 += kBw;
+    if (start > kLast) { j += kSlots; t -= 2 * kSlots; start -= 15 * kSlots; to2 += ((int64_t)ns - 2) * kSlots * kBw; }
   }
   for (int q = tid; q < COLS; q += kThreads) {
-    const int j = col0 + q;
-    if (j < r) { L.td_d[j] = ch_smem[(size_t)(kAbove + q) * kChLd]; L.td_e[j] = j + 1 < r ? ch_smem[(size_t)(kAbove + q) * kChLd + 1] : 0.0; }
+    const int jj = col0 + q;
+    if (jj < r) { L.td_d[jj] = ch_smem[(size_t)(kAbove + q) * kChLd]; L.td_e[jj] = jj + 1 < r ? ch_smem[(size_t)(kAbove + q) * kChLd + 1] : 0.0; }
   }
   if (C > 1) cg::this_cluster().sync();                      // nobody leaves while a neighbour may still read its memory
 }
@@ -765,10 +838,9 @@ int sp_chase_capacity(int ctas) {
   return n;
 }
 // CTAs per layer of the chase for n layers of r rows (up to 1024, 2048 or 4096): 256 columns each while the clusters run side by
-// side with an SM per CTA, else 1024 columns.  Both stages of the reduction, 256 | 1024 columns, ms: 9 of 2048 rows 21.5 | 24.3, 14
-// 27.4 | 30.2, 16 35.9 | 32.1; of 4096 rows 1 33.9 | 43.2, 7 73.7 | 83.0, 8 95.4 | 90.8 (14 and 7 clusters fit).  Up to 1024 rows a
-// single CTA takes what a cluster of four takes (1 layer 6.05 | 6.08, 20 layers 7.85 | 7.92) and leaves the others their SMs (36:
-// 9.5 | 12.7).
+// side with an SM per CTA, else 1024 columns.  A whole encode, 256 | 1024 columns, ms: 9 of 2048 rows 25.4 | 26.9, 14 32.7 | 34.2;
+// of 4096 rows 1 37.9 | 42.2, 7 100.5 | 104.8 (14 and 7 clusters fit).  Up to 1024 rows a single CTA is faster than a cluster of
+// four (the chase of 1023 rows 1.42 | 1.47, of 600 rows 1.01 | 1.12) and leaves the others their SMs.
 int sp_chase_ctas(int r, int n, int wide_capacity) {
   const int few = r <= 1024 ? 1 : r <= 2048 ? 2 : 4;
   return few > 1 && n <= wide_capacity ? 4 * few : few;
