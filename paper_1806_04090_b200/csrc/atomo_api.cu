@@ -773,7 +773,6 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
       d.td_V = A.take<float>(d.tri ? (size_t)d.r * d.td_ldv : 0);
-      d.tb_vecwork = A.take<double>(d.tri == 2 ? (size_t)sp_eigvec_big_slots() * 5 * d.rp : 0);
       d.tb_z = A.take<double>(d.tri == 2 && d.rp > 1024 ? (size_t)d.k_cap * d.rp : 0);
       {
         const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
@@ -784,7 +783,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
         d.bd_T = A.take<double>(on * sp_band_steps(d.r) * kBandWidth * kBandWidth);
-        d.bd_V2 = A.take<double>(on * d.r * sp_band_steps(d.r) * kBandWidth);
+        d.bd_V2 = A.take<double>(on * d.r * sp_chase_row(d.r));
       }
       d.chol_dd = A.take<float>(32 * 32 + 32);
       d.row_inv = A.take<float>(d.rp);

@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(
   const int tid = threadIdx.x, lane = tid % 32;
   const int r = L.r;
   const double* const gB = L.bd_band;
-  const int ns = (r + kBw - 1) / kBw;                        // steps per sweep that L.bd_V2 has room for
+  const int64_t row = sp_chase_row(r);                       // doubles per sweep in L.bd_V2
   const int col0 = rank * COLS, lo = col0 - kAbove;       // first own column, first column in shared memory
   double* const s_in = ch_smem + (kLocal + kBw) * kChLd;     // [2][kHalo] columns from the neighbours
   double *above = ch_smem, *below = ch_smem;                 // the neighbours' shared memory
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(
   // sweep j's step t = tick - 2 j - 1 starts at row j + 1 + 8 t = 8 tick - 7 - 15 j (step -1: column j, seven further down).
   // Lanes go on with the sweep kSlots further when theirs has left the columns that are here.
   int j = tid % (kThreads / 2) / 4, t = -2 * j - 1, start = -7 - lo - 15 * j;   // (start: local)
-  double* to2 = L.bd_V2 + ((int64_t)j * ns + t + 1) * kBw + k;   // where the reflector of step t + 1 goes
+  double* to2 = L.bd_V2 + j * row + k / 2 * 64 + k % 2;      // where the sweep's reflectors go: in groups of 32, entries by pairs
   for (int tick = 0; tick < ticks; ++tick) {
     if (C > 1 && tick % kChTicks == 0 && tick > 0) {         // every CTA's own columns are up to date
       cg::cluster_group cluster = cg::this_cluster();
@@ -735,12 +735,15 @@ __global__ void __launch_bounds__(ChForm<C, COLS>::kThreads, 1) sp_chase_kernel(
         double* const to = ch_smem + (start + kBw) * kChLd + kChVec + k;
         to[0] = un[0]; to[kChLd] = un[1];
         const int own = (first ? start + 7 : start) - kAbove;
-        if (more && own >= 0 && own < COLS) { to2[0] = un[0]; to2[4] = un[1]; }
+        if (more && own >= 0 && own < COLS) {
+          double* const to = to2 + (t + 1) / 32 * 256 + (t + 1) % 32 * 2;
+          to[0] = un[0]; to[128] = un[1];
+        }
       }
     }
     __syncthreads();
-    ++t; start += kBw; to2 += kBw;
-    if (start > kLast) { j += kSlots; t -= 2 * kSlots; start -= 15 * kSlots; to2 += ((int64_t)ns - 2) * kSlots * kBw; }
+    ++t; start += kBw;
+    if (start > kLast) { j += kSlots; t -= 2 * kSlots; start -= 15 * kSlots; to2 += kSlots * row; }
   }
   for (int q = tid; q < COLS; q += kThreads) {
     const int jj = col0 + q;

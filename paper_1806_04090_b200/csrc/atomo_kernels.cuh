@@ -64,6 +64,9 @@ void launch_ew_lq(const float* g, int64_t n, int pass, double q, double inv_amax
 // ================================= spectral path =================================================
 constexpr int kMaxShort = 4096;       // largest short side (atoms per layer)
 constexpr int kBandWidth = 8;         // sub-diagonals between the two stages of the large layers' reduction
+// doubles that a sweep of the chase takes in bd_V2: its steps in groups of 32, in a group the steps' entries 0 and 1, then 2 and
+// 3, .. (a warp of the back-transformation, a reflector per lane, reads whole lines)
+__host__ __device__ inline int64_t sp_chase_row(int r) { return (int64_t)((r + 255) / 256) * 256; }
 constexpr int kSmemRowsMaxRp = 4096;  // largest padded short side the shared-memory Jacobi kernel holds
 
 struct SpLayer {
@@ -114,9 +117,8 @@ struct SpLayer {
   double* bd_G; double* bd_M;  // [half strips][36] dots of the next panel's columns, of U's
   double* bd_band;             // [r][9] the band, by column
   double* bd_T;                // [panels][64] T of the panels: Q1 is the product of I - U T U^T
-  double* bd_V2;               // [r][steps][8] reflectors of the chase: sweep, step
+  double* bd_V2;               // [r][sp_chase_row] reflectors of the chase, by sweep
   uint32_t* bd_bar;            // arrivals at the layer's barriers; zeroed per call
-  double* tb_vecwork;          // [slots][5][rp] work vectors of the twisted factorisation
   double* tb_z;                // [k_cap][rp] short sides above 1024: the kept atoms' eigenvectors of T
 };
 
@@ -173,7 +175,6 @@ int launch_sp_band(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_ctas
 int sp_chase_capacity(int ctas);                                  // clusters of that many CTAs side by side (0: not available)
 int sp_chase_ctas(int r, int n, int wide_capacity);               // CTAs per layer of the chase, for n layers of its size
 int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas, cudaStream_t st);   // cudaError_t
-int sp_eigvec_big_slots();                                        // warps per layer of the vector kernel (work vectors)
 int sp_configure_eigvec_big();                                    // 0 if available
 int sp_configure_bisect();                                        // 0 if the eigenvalue kernel got its shared memory
 // rps: which padded short sides are among them (bit 0: up to 1024, bit 1: up to 2048, bit 2: above)

@@ -363,7 +363,7 @@ constexpr int kVecWarps = kVecThreads / 32;
 constexpr int kVecCtasPerLayer = 4;
 constexpr int kVecGroup = 4;          // reflectors applied together in the back-transformation
 constexpr int kVecStages = 4;         // groups in flight between global and shared memory
-constexpr int kVecWork = 5;           // work vectors of the twisted factorisation per warp
+constexpr int kVecWork = 3;           // work vectors of the twisted factorisation per warp
 constexpr double kSameEig = 1.0e-9;   // scaled units (largest eigenvalue below 1): eigenvalues this close share a subspace
 
 __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer* __restrict__ layers) {
@@ -388,9 +388,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
   __syncthreads();
   double* wa = s_work + (size_t)w * kVecWork * rp;
   double* wb = wa + rp;
-  double* wc = wb + rp;
-  double* wd = wc + rp;
-  double* z = wd + rp;
+  double* z = wb + rp;
   constexpr int kCols = kTriCols;
   for (uint32_t a0 = blockIdx.y * kVecWarps; a0 < k; a0 += kVecCtasPerLayer * kVecWarps) {
     const uint32_t a = a0 + w;
@@ -406,7 +404,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
       for (uint32_t b = lane; b < a; b += 32) skip += fabs(gLam[gPerm[gIdx[b]]] - lambda) <= kSameEig ? 1 : 0;
       skip = (int)warp_sum((uint32_t)skip);
       double n2 = 1.0;
-      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, z, lane, skip, &n2);
+      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, skip, &n2);
       // the vector's error is about |correction| / gap to the nearest other eigenvalue: well-separated atoms are done
       double gap = 1.0e300;
       if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
@@ -414,7 +412,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
       if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {   // one Rayleigh-quotient step, then the vector again
         lambda += corr;
         __syncwarp();
-        twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, z, lane, 0, &n2);
+        twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, 0, &n2);
       }
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
 #pragma unroll

@@ -24,7 +24,6 @@ namespace atomo {
 namespace {
 constexpr int kVbThreads = 512;
 constexpr int kVbWarps = kVbThreads / 32;
-constexpr int kVbSlots = 16;                 // work-vector sets per layer (phase A: 16 atoms at a time over the layer's CTAs)
 constexpr int kVbMaxCtas = 16;               // CTAs per layer (the kept atoms are dealt to them)
 constexpr int kVbBatch = 4;                  // atoms per pass over the reflectors; two above a short side of 2048 (shared memory)
 constexpr int kVbHalf = 2048;
@@ -75,183 +74,165 @@ __device__ __forceinline__ void vb_orthogonalise_equal(const SpLayer& L, uint32_
 
 
 namespace {
-// the columns tid, tid + THREADS, ... of the four reflector rows base .. base + 3
-template <int THREADS, int COLS>
-__device__ __forceinline__ void vb_load_rows(const float* __restrict__ gV, int64_t ldv, int r, int base, float (&q)[4][COLS]) {
-  const int tid = threadIdx.x;
-  const float* v = gV + (int64_t)base * ldv;
+// reduce-scatter of eight doubles over a warp: the lane ends with the sum of value lane / 4
+__device__ __forceinline__ double vb_scatter8(const double (&v)[8], int lane) {
+  double a[4], b[2], c;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
 #pragma unroll
-  for (int m = 0; m < COLS; ++m) {
-    const int h = tid + m * THREADS;
-    const bool in = h >= base + kBandWidth && h < r;           // reflector kk is zero below index kk + 8
+  for (int i = 0; i < 4; ++i) a[i] = (h4 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[4 + i], 16);
 #pragma unroll
-    for (int x = 0; x < 4; ++x) q[x][m] = in ? __ldcg(v + x * ldv + h) : 0.0f;
-  }
+  for (int i = 0; i < 2; ++i) b[i] = (h3 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[2 + i], 8);
+  c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
 }
 
-// z_b <- Q1 z_b for the nb vectors in s_z, the whole CTA; the next group's rows are on their way while this group's sums are
-// added up.  Reflectors kk >= nref of the last group are rows of zeros.
+// z_b <- Q1 z_b for the nb vectors in s_z, the whole CTA, a panel at a time: z -= U (T (U^T z)).  A thread owns the columns tid,
+// tid + THREADS, .. of the panel's eight rows, read once, in registers between the dots and the update; a column that has been
+// updated makes room for the next panel's.  Panels shrink towards the last: a warp whose columns lie outside skips them.
+// Reflectors kk >= nref of the last panel are rows of zeros.
 template <int THREADS, int BATCH, int COLS>
 __device__ __forceinline__ void vb_apply_reflectors(const float* __restrict__ gV, int64_t ldv, const double* __restrict__ gT, int r, int rp, int nref,
-                                                    int nb, double* s_z, double (*s_part)[4 * BATCH], double* s_tot) {
-  constexpr int kSums = 4 * BATCH, kWarps = THREADS / 32;
-  static_assert(kSums <= 32, "one warp adds the warps' parts");
+                                                    int nb, double* s_z, double (*s_part)[8 * BATCH], double* s_tot) {
+  constexpr int kWarps = THREADS / 32;
+  static_assert(BATCH <= kWarps, "a warp per vector adds the warps' parts");
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  float q[4][COLS], qn[4][COLS];
-  const int top = (nref - 1) / 4 * 4;                          // the last group's first reflector
-  if (nref > 0) vb_load_rows<THREADS, COLS>(gV, ldv, r, top, q);
-  for (int base = nref > 0 ? top : -1; base >= 0; base -= 4) {
-    double2 t01 = make_double2(0.0, 0.0), t23 = t01;           // row lane % 4 of the group's block of T
-    if (w == 0) {
-      const double* t = gT + (int64_t)(base / 8) * 64 + (base % 8 + lane % 4) * 8 + base % 8;
-      t01 = __ldcg(reinterpret_cast<const double2*>(t)); t23 = __ldcg(reinterpret_cast<const double2*>(t) + 1);
-    }
-    double acc[kSums];
+  if (nref <= 0) return;
+  float q[8][COLS];
+  auto load = [&](int base, int m) {
+    const int h = tid + m * THREADS;
+    const bool in = base >= 0 && h >= base + kBandWidth && h < r;   // reflector kk is zero below index kk + 8
+    const float* v = gV + (int64_t)base * ldv + h;
 #pragma unroll
-    for (int x = 0; x < kSums; ++x) acc[x] = 0.0;
+    for (int x = 0; x < 8; ++x) q[x][m] = in ? __ldcg(v + x * ldv) : 0.0f;
+  };
+  const int top = (nref - 1) / 8 * 8;                          // the last panel's first reflector
 #pragma unroll
-    for (int m = 0; m < COLS; ++m) {
-      const int h = tid + m * THREADS;
-      if (h < r) {
+  for (int m = 0; m < COLS; ++m) load(top, m);
+  for (int base = top; base >= 0; base -= 8) {
+    double2 t = make_double2(0.0, 0.0);                        // T[lane % 8][2 (lane / 8) ..]
+    if (w < nb) t = __ldcg(reinterpret_cast<const double2*>(gT + (int64_t)(base / 8) * 64 + (lane & 7) * 8 + (lane >> 3) * 2));
+    auto inside = [&](int m) { return 32 * w + 31 + m * THREADS >= base + kBandWidth && 32 * w + m * THREADS < r; };   // some of the warp's columns
 #pragma unroll
-        for (int b = 0; b < BATCH; ++b) {
-          if (b < nb) {
-            const double zh = s_z[(size_t)b * rp + h];
+    for (int b = 0; b < BATCH; ++b) {
+      if (b < nb) {
+        double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int x = 0; x < 4; ++x) acc[4 * b + x] = fma((double)q[x][m], zh, acc[4 * b + x]);
+        for (int m = 0; m < COLS; ++m) {
+          if (inside(m)) {
+            const int h = tid + m * THREADS;
+            const double zh = h < r ? s_z[(size_t)b * rp + h] : 0.0;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) acc[x] = fma((double)q[x][m], zh, acc[x]);
           }
         }
-      }
-    }
-    if (base >= 4) vb_load_rows<THREADS, COLS>(gV, ldv, r, base - 4, qn);
-#pragma unroll
-    for (int x = 0; x < kSums; ++x) {
-      if (x < 4 * nb) {
-        const double t = warp_sum(acc[x]);
-        if (lane == 0) s_part[w][x] = t;
+        const double sum = vb_scatter8(acc, lane);
+        if ((lane & 3) == 0) s_part[w][8 * b + (lane >> 2)] = sum;
       }
     }
     __syncthreads();
-    if (w == 0) {                                              // lane 4 b + i: (T p)_i of vector b
+    if (w < nb) {                                              // the vector of number w: lane's value lane % 8, of every fourth warp
       double p = 0.0;
-      if (lane < 4 * nb) {
 #pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) p += s_part[ww][lane];
-      }
-      const int l0 = lane & ~3;
-      double s = t01.x * __shfl_sync(0xffffffffu, p, l0);      // (T is zero below its diagonal)
-      s = fma(t01.y, __shfl_sync(0xffffffffu, p, l0 + 1), s);
-      s = fma(t23.x, __shfl_sync(0xffffffffu, p, l0 + 2), s);
-      s = fma(t23.y, __shfl_sync(0xffffffffu, p, l0 + 3), s);
-      if (lane < 4 * nb) s_tot[lane] = s;
+      for (int ww = 0; ww < kWarps; ww += 4) p += s_part[ww + (lane >> 3)][8 * w + (lane & 7)];
+      p += __shfl_xor_sync(0xffffffffu, p, 8);
+      p += __shfl_xor_sync(0xffffffffu, p, 16);
+      double c = t.x * __shfl_sync(0xffffffffu, p, (lane >> 3) * 2);
+      c = fma(t.y, __shfl_sync(0xffffffffu, p, (lane >> 3) * 2 + 1), c);
+      c += __shfl_xor_sync(0xffffffffu, c, 8);
+      c += __shfl_xor_sync(0xffffffffu, c, 16);
+      if (lane < 8) s_tot[8 * w + lane] = c;
     }
     __syncthreads();
 #pragma unroll
     for (int b = 0; b < BATCH; ++b) {
       if (b < nb) {
-        const double c0 = s_tot[4 * b], c1 = s_tot[4 * b + 1], c2 = s_tot[4 * b + 2], c3 = s_tot[4 * b + 3];
+        double c[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) c[x] = s_tot[8 * b + x];
 #pragma unroll
         for (int m = 0; m < COLS; ++m) {
-          const int h = tid + m * THREADS;
-          if (h < r) s_z[(size_t)b * rp + h] -= fma(c0, (double)q[0][m], fma(c1, (double)q[1][m], fma(c2, (double)q[2][m], c3 * (double)q[3][m])));
+          if (inside(m)) {
+            const int h = tid + m * THREADS;
+            double z0 = 0.0, z1 = 0.0;
+#pragma unroll
+            for (int x = 0; x < 8; x += 2) { z0 = fma(c[x], (double)q[x][m], z0); z1 = fma(c[x + 1], (double)q[x + 1][m], z1); }
+            if (h < r) s_z[(size_t)b * rp + h] -= z0 + z1;
+          }
+          if (b == nb - 1) load(base - 8, m);
         }
       }
     }
-    // (two barriers separate a write to s_part or s_tot from the reads of the group before)
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int m = 0; m < COLS; ++m) q[x][m] = qn[x][m];
+    // (two barriers separate a write to s_part or s_tot from the reads of the panel before)
   }
 }
 }  // namespace
 
 // ---- back-transformation through the bulge chase -----------------------------------------------------------------------
 // z <- H_first ... H_last z, the sweeps from the last to the first.  The reflectors of a sweep act on disjoint runs of eight
-// entries, and from one sweep to the one before all runs move up by one entry.  A thread holds BPT runs in registers; a
+// entries, and from one sweep to the one before all runs move up by one entry.  A thread holds a run in registers; a
 // move hands its last entry to the next thread (a shuffle, across warps through shared memory) and renames the others (the
-// loop is unrolled over a whole turn of the names).  The reflectors arrive through a ring in shared memory, kStages sweeps
-// ahead, read once for all ATOMS vectors.  One block barrier per sweep.
+// loop is unrolled over a whole turn of the names).  Entries only ever move towards the next warp, so warp w does the eight
+// sweeps of a turn while warp w + 1 does those of the turn before: a block barrier per turn, not per sweep, and a warp takes up
+// its work when its runs have come inside the matrix.  A lane's reflectors come straight into registers, DEPTH sweeps ahead.
+// Bound: the reflectors, 4 r^2 bytes of fp64 per vector through one SM.
 namespace {
-constexpr int kBackStages = 5;
-template <int THREADS, int BPT, int ATOMS> constexpr size_t vb_ring_bytes() { return (size_t)kBackStages * (THREADS / ATOMS) * BPT * 8 * sizeof(double); }
-
-template <int THREADS, int BPT, int ATOMS>
-__device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, const int ns, const int r, double* s_z, const int z_stride,
-                                              double2* s_ring, double (*s_edge)[THREADS / 32]) {
+template <int THREADS, int ATOMS, int DEPTH>
+__device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, const int r, double* s_z, const int z_stride,
+                                              double (*s_edge)[THREADS / 32][8]) {
   constexpr int kPer = THREADS / ATOMS;                        // threads per vector
-  constexpr int kChunks = kPer * BPT * 4;                      // double2 per sweep
-  constexpr int kW = 8 * BPT;                                  // entries per thread = sweeps per turn
-  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32, me = tid % kPer;
+  static_assert(8 % DEPTH == 0, "a sweep's registers are the same in every turn");
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32, me = tid % kPer, wv = me / 32;
   double* const z = s_z + (size_t)(tid / kPer) * z_stride;
-  const int sweeps = ((r - 2 + kW - 1) / kW) * kW;             // the first ones of a partial turn act on nothing
-  auto place = [](int f) -> int {                              // chunk f of a sweep inside its stage (spread over the banks)
-    const int th = f / (4 * BPT), c = f % (4 * BPT);
-    return th * 4 * BPT + (c ^ (BPT == 1 ? (th >> 1) & 3 : th & 7));
-  };
-  // this thread's chunks of a sweep: where they go, the last sweep that has them, where they come from (sweep by sweep upwards)
-  constexpr int kMine = (kChunks + THREADS - 1) / THREADS;
-  uint32_t to[kMine];
-  int last[kMine];
-  const double* from[kMine];
+  const int turns = max(r - 2 + 7, 0) / 8;                     // the first sweeps of a partial turn act on nothing
+  // the first turn in which one of the warp's entries is inside: before, they are all zeros
+  const int first = max(0, (8 * turns + 256 * wv - r) / 8);
+  const int j_first = 8 * (turns - first) - 1;
+  const int64_t row = sp_chase_row(r);
+  const double* from = gV2 + (j_first * row + wv * 256 + lane * 2);
+  const int last = r - 3 - 8 * me;                             // the last sweep that has this thread's reflector
+  double u[DEPTH][8];
+  auto load = [&](double (&v)[8], int j) {
+    const bool in = j >= 0 && j <= last;
 #pragma unroll
-  for (int c = 0; c < kMine; ++c) {
-    const int f = tid + c * THREADS, t = f / 4;
-    to[c] = (uint32_t)__cvta_generic_to_shared(s_ring + place(f));
-    last[c] = f < kChunks ? min(r - 3, r - 3 - 8 * t) : -1;
-    from[c] = gV2 + ((int64_t)(sweeps - 1) * ns + t) * 8 + (f & 3) * 2;
-  }
-  int fill = 0, use = 0;                                       // stages
-  auto issue = [&](int j) {                                    // sweep j (none below 0: an empty group keeps the count)
-    if (j >= 0) {
-#pragma unroll
-      for (int c = 0; c < kMine; ++c) {
-        const bool ok = j <= last[c];
-        if (kChunks % THREADS == 0 || tid + c * THREADS < kChunks)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[c] + fill * (uint32_t)(kChunks * sizeof(double2))), "l"(ok ? from[c] : gV2), "r"(ok ? 16 : 0) : "memory");
-        from[c] -= (int64_t)ns * 8;
-      }
+    for (int c = 0; c < 4; ++c) {
+      const double2 x = in ? __ldcg(reinterpret_cast<const double2*>(from + 64 * c)) : make_double2(0.0, 0.0);
+      v[2 * c] = x.x; v[2 * c + 1] = x.y;
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    fill = fill == kBackStages - 1 ? 0 : fill + 1;
+    from -= row;
   };
-  double x[kW];
+  double x[8], carry = 0.0;                                    // carry: what the next turn's first move brings from the warp before
 #pragma unroll
-  for (int e = 0; e < kW; ++e) { const int at = sweeps + me * kW + e; x[e] = at < r ? z[at] : 0.0; }
-  __syncthreads();
-  for (int s = 0; s < kBackStages - 1; ++s) issue(sweeps - 1 - s);
-  for (int j0 = sweeps - 1; j0 >= 0; j0 -= kW) {
+  for (int e = 0; e < 8; ++e) { const int at = j_first + 1 + me * 8 + e; x[e] = at < r ? z[at] : 0.0; }
 #pragma unroll
-    for (int s = 0; s < kW; ++s) {                             // entry e of the window sits in x[(e - s) mod kW]
-      const int j = j0 - s;
-      asm volatile("cp.async.wait_group %0;" ::"n"(kBackStages - 2) : "memory");
-      __syncthreads();                                         // sweep j has landed for everybody; the stage of j + 1 is free
-      issue(j - (kBackStages - 1));
-      if (j < sweeps - 1) {                                    // the window moves up by one entry
-        double in = __shfl_up_sync(0xffffffffu, x[(kW - s) % kW], 1);        // what was the last entry of the thread before
-        if (lane == 0) in = me == 0 ? (j + 1 < r ? z[j + 1] : 0.0) : s_edge[(j + 1) & 1][w - 1];
-        x[(kW - s) % kW] = in;
-      }
-      const double2* const st = s_ring + use * kChunks;
-      use = use == kBackStages - 1 ? 0 : use + 1;
+  for (int s = 0; s < DEPTH; ++s) load(u[s], first < turns ? j_first - s : -1);
+  for (int tick = 0; tick < turns + kPer / 32 - 1; ++tick) {
+    const int b = tick - wv;
+    if (b >= first && b < turns) {
 #pragma unroll
-      for (int b = 0; b < BPT; ++b) {
-        double u[8];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { const double2 v = st[place((me * BPT + b) * 4 + c)]; u[2 * c] = v.x; u[2 * c + 1] = v.y; }
+      for (int s = 0; s < 8; ++s) {                            // entry e of the window sits in x[(e - s) mod 8]
+        const int j = 8 * (turns - b) - 1 - s;
+        if (s > 0 || b > first) {                              // the window moves up by one entry
+          double in = __shfl_up_sync(0xffffffffu, x[(8 - s) % 8], 1);          // what was the last entry of the thread before
+          if (lane == 0) in = wv == 0 ? (j + 1 < r ? z[j + 1] : 0.0) : s == 0 ? carry : s_edge[b & 1][w - 1][s - 1];
+          x[(8 - s) % 8] = in;
+        }
+        double (&v)[8] = u[s % DEPTH];
         double d0 = 0.0, d1 = 0.0;
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) { d0 = fma(u[e], x[(8 * b + e - s + 2 * kW) % kW], d0); d1 = fma(u[e + 1], x[(8 * b + e + 1 - s + 2 * kW) % kW], d1); }
+        for (int e = 0; e < 8; e += 2) { d0 = fma(v[e], x[(e - s + 8) % 8], d0); d1 = fma(v[e + 1], x[(e + 1 - s + 8) % 8], d1); }
         const double d = -2.0 * (d0 + d1);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[(8 * b + e - s + 2 * kW) % kW] = fma(d, u[e], x[(8 * b + e - s + 2 * kW) % kW]);
+        for (int e = 0; e < 8; ++e) x[(e - s + 8) % 8] = fma(d, v[e], x[(e - s + 8) % 8]);
+        load(v, j - DEPTH);
+        if (lane == 31) s_edge[b & 1][w][s] = x[(15 - s) % 8];
       }
-      if (lane == 31) s_edge[j & 1][w] = x[(2 * kW - 1 - s) % kW];
+      if (wv > 0) carry = s_edge[b & 1][w - 1][7];
     }
+    __syncthreads();
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
-  for (int e = 0; e < kW; ++e) { const int at = 1 + me * kW + e; if (at < r) z[at] = x[(e + 1) % kW]; }   // after kW - 1 moves of the turn
+  for (int e = 0; e < 8; ++e) { const int at = 1 + me * 8 + e; if (at < r) z[at] = x[(e + 1) % 8]; }   // after the seven moves of the last turn
   __syncthreads();
 }
 }  // namespace
@@ -263,7 +244,7 @@ __device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, co
 namespace {
 constexpr int kVcThreads = 128;
 constexpr int kVcWarps = kVcThreads / 32;
-constexpr int kVcCtas = 16;                  // CTAs per layer = work-vector sets per layer
+constexpr int kVcCtas = 16;                  // CTAs per layer
 constexpr int kVcMaxRp = 1024;
 }  // namespace
 
@@ -276,10 +257,10 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
   double* s_d = reinterpret_cast<double*>(vb_smem);            // [rp]
   double* s_e = s_d + rp;                                      // [rp]
   double* s_z = s_e + rp;                                      // [rp]
-  double2* s_ring = reinterpret_cast<double2*>(s_z + rp);
-  __shared__ double s_part[kVcWarps][4];
-  __shared__ double s_tot[4];
-  __shared__ double s_edge[2][kVcWarps];
+  double* const s_work = s_z + rp;                              // [2][rp], work vectors
+  __shared__ double s_part[kVcWarps][8];
+  __shared__ double s_tot[8];
+  __shared__ double s_edge[2][kVcWarps][8];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const uint32_t k = L.hdr->k;
   const float* const gV = L.td_V; const int64_t ldv = L.td_ldv; const double* const gLam = L.lam64;
@@ -289,8 +270,8 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
   if ((uint32_t)slot < k) {
     for (int i = tid; i < r; i += kVcThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
     __syncthreads();
-    double* wa = L.tb_vecwork + (size_t)slot * 5 * rp;
-    double* wb = wa + rp; double* wc = wb + rp; double* wd = wc + rp; double* zz = wd + rp;
+    double* const wa = s_work;
+    double* const wb = wa + rp;
     for (uint32_t a = slot; a < k; a += kVcCtas) {
       if (w == 0) {
         const int ei = gPerm[gIdx[a]];                         // index of the atom's eigenvalue (ascending order)
@@ -299,21 +280,21 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
         for (uint32_t b2 = lane; b2 < a; b2 += 32) skip += fabs(gLam[gPerm[gIdx[b2]]] - lambda) <= kVbSameEig ? 1 : 0;
         skip = (int)warp_sum((uint32_t)skip);
         double n2 = 1.0;
-        const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, zz, lane, skip, &n2);
+        const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, skip, &n2);
         double gap = 1.0e300;
         if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
         if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
         if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {  // one Rayleigh-quotient step, then the vector again
           lambda += corr;
           __syncwarp();
-          twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, zz, lane, 0, &n2);
+          twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, 0, &n2);
         }
         __syncwarp();
         const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
-        for (int i = lane; i < r; i += 32) s_z[i] = zz[i] * inv;
+        for (int i = lane; i < r; i += 32) s_z[i] *= inv;
       }
       __syncthreads();
-      vb_chase_back<kVcThreads, 1, 1>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+      vb_chase_back<kVcThreads, 1, 8>(L.bd_V2, r, s_z, rp, s_edge);
       vb_apply_reflectors<kVcThreads, 1, kVcMaxRp / kVcThreads>(gV, ldv, L.bd_T, r, rp, nref, 1, s_z, s_part, s_tot);
       double n2 = 0.0;
       for (int i = tid; i < r; i += kVcThreads) n2 = fma(s_z[i], s_z[i], n2);
@@ -344,10 +325,10 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
   double* s_z = reinterpret_cast<double*>(vb_smem);            // [BATCH][rp]
   double* s_d = s_z + (size_t)BATCH * rp;                      // [rp], phase A
   double* s_e = s_d + rp;                                      // [rp]
-  double2* s_ring = reinterpret_cast<double2*>(s_d);           // phase B
-  __shared__ double s_edge[2][kVbWarps];
-  __shared__ double s_part[kVbWarps][4 * BATCH];
-  __shared__ double s_tot[4 * BATCH];
+  __shared__ double s_ex[kVbWarps * (BATCH > 2 ? 8 * BATCH : 16)];   // what the warps exchange: in the chase's turns, in the panels' sums
+  double (*const s_edge)[kVbWarps][8] = reinterpret_cast<double (*)[kVbWarps][8]>(s_ex);
+  double (*const s_part)[8 * BATCH] = reinterpret_cast<double (*)[8 * BATCH]>(s_ex);
+  __shared__ double s_tot[8 * BATCH];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int n_ctas = gridDim.y, cy = blockIdx.y;
   const uint32_t k = L.hdr->k;
@@ -357,26 +338,26 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
   const int nref = max(r - kBandWidth - 1, 0);
   for (int i = tid; i < r; i += kVbThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
   __syncthreads();
-  // ---- (A) this CTA's atoms are a = cy, cy + n_ctas, ...; warp w < slots-per-CTA takes every (slots-per-CTA)-th of them ----
-  const int spc = kVbSlots / n_ctas;                           // work-vector sets of this CTA
-  if (w < spc) {
-    double* wa = L.tb_vecwork + (size_t)(cy * spc + w) * 5 * rp;
-    double* wb = wa + rp; double* wc = wb + rp; double* wd = wc + rp; double* zz = wd + rp;
-    for (uint32_t a = cy + (uint32_t)n_ctas * w; a < k; a += (uint32_t)(n_ctas * spc)) {
+  // ---- (A) this CTA's atoms are a = cy, cy + n_ctas, ...; as many warps as there is room for work vectors beside T share them ----
+  constexpr int kWork = kRp <= kVbHalf ? 2 : 1;
+  if (w < kWork) {
+    double* const wa = s_e + rp + (size_t)w * 3 * rp;
+    double* const wb = wa + rp; double* const zz = wb + rp;
+    for (uint32_t a = cy + (uint32_t)n_ctas * w; a < k; a += (uint32_t)(n_ctas * kWork)) {
       const int ei = gPerm[gIdx[a]];                           // index of the atom's eigenvalue (ascending order)
       double lambda = gLam[ei];
       int skip = 0;                                            // earlier kept atoms with the same eigenvalue: another twist index each
       for (uint32_t b2 = lane; b2 < a; b2 += 32) skip += fabs(gLam[gPerm[gIdx[b2]]] - lambda) <= kVbSameEig ? 1 : 0;
       skip = (int)warp_sum((uint32_t)skip);
       double n2 = 1.0;
-      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, zz, lane, skip, &n2);
+      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, skip, &n2);
       double gap = 1.0e300;
       if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
       if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
       if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {    // one Rayleigh-quotient step, then the vector again
         lambda += corr;
         __syncwarp();
-        twisted_vector(s_d, s_e, r, lambda, wa, wb, wc, wd, zz, lane, 0, &n2);
+        twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, 0, &n2);
       }
       __syncwarp();
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
@@ -394,9 +375,8 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
       for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = b < nb ? __ldcg(src + i) : 0.0;
     }
     __syncthreads();
-    // few atoms: a run per thread and a turn of eight sweeps
-    if (nb <= kFew) vb_chase_back<kVbThreads, 1, kFew>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
-    else vb_chase_back<kVbThreads, COLS * BATCH / 8, BATCH>(L.bd_V2, (r + kBandWidth - 1) / kBandWidth, r, s_z, rp, s_ring, s_edge);
+    // a run per thread: one or two atoms at a time
+    for (int b = 0; b < nb; b += kFew) vb_chase_back<kVbThreads, kFew, 4>(L.bd_V2, r, s_z + (size_t)b * rp, rp, s_edge);
     vb_apply_reflectors<kVbThreads, BATCH, COLS>(gV, ldv, L.bd_T, r, rp, nref, nb, s_z, s_part, s_tot);
     // normalise and file
     for (int b = 0; b < nb; ++b) {
@@ -420,22 +400,17 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
 
 // ---- host side ---------------------------------------------------------------------------------------------------
 namespace {
-// shared memory of the kernel with BATCH atoms and COLS columns per thread for a short side of rp: the vectors, then the diagonals of
-// T or the ring of reflectors (the larger of its two forms)
-template <int BATCH, int COLS> size_t vb_smem_bytes(int rp) {
-  const size_t ring = std::max(vb_ring_bytes<kVbThreads, 1, 8 / COLS>(), vb_ring_bytes<kVbThreads, COLS * BATCH / 8, BATCH>());
-  return (size_t)rp * BATCH * sizeof(double) + std::max(ring, (size_t)rp * 2 * sizeof(double));
-}
-size_t vc_smem_bytes(int rp_max) { return (size_t)std::min(rp_max, kVcMaxRp) * 3 * sizeof(double) + vb_ring_bytes<kVcThreads, 1, 1>(); }
+// shared memory of the kernel with BATCH atoms and COLS columns per thread for a short side of rp: the vectors, T, the work
+// vectors of one or two atoms
+template <int BATCH> size_t vb_smem_bytes(int rp) { return (size_t)(BATCH + 2 + 3 * (rp <= kVbHalf ? 2 : 1)) * rp * sizeof(double); }
+size_t vc_smem_bytes() { return (size_t)kVcMaxRp * 5 * sizeof(double); }
 }  // namespace
-
-int sp_eigvec_big_slots() { return kVbSlots; }
 
 // 0 if the kernels got their shared memory
 int sp_configure_eigvec_big() {
-  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbBatch, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch, 4>(kVbHalf)) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<2, 8>(kMaxShort)) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(sp_eigvec_big_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vc_smem_bytes(kVcMaxRp)) != cudaSuccess;
+  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbBatch, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch>(kVbHalf)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<2>(kMaxShort)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vc_smem_bytes()) != cudaSuccess;
   if (bad) cudaGetLastError();
   return bad;
 }
@@ -443,15 +418,15 @@ int sp_configure_eigvec_big() {
 void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, cudaStream_t st) {
   if (n_big <= 0) return;
   // layers up to a short side of 1024: a four-warp CTA per kept atom (each kernel's CTAs leave the others' layers at once)
-  if (rps & 1) sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(kVcMaxRp), st>>>(d_layers, d_big);
+  if (rps & 1) sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(), st>>>(d_layers, d_big);
   if (!(rps & 6)) return;
   // larger layers: CTAs per layer (1 to 16; the kept atoms are dealt to them), as many as keep the launch within one wave
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int per = 1;
   while (per < kVbMaxCtas && n_big * per * 2 <= sms) per *= 2;
-  if (rps & 2) sp_eigvec_big_kernel<kVbBatch, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<kVbBatch, 4>(kVbHalf), st>>>(d_layers, d_big);
-  if (rps & 4) sp_eigvec_big_kernel<2, 8><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<2, 8>(kMaxShort), st>>>(d_layers, d_big);
+  if (rps & 2) sp_eigvec_big_kernel<kVbBatch, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<kVbBatch>(kVbHalf), st>>>(d_layers, d_big);
+  if (rps & 4) sp_eigvec_big_kernel<2, 8><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<2>(kMaxShort), st>>>(d_layers, d_big);
 }
 
 }  // namespace atomo

@@ -8,52 +8,83 @@ namespace atomo {
 __device__ __forceinline__ bool finite64(double x) { return fabs(x) <= 1.7e308; }
 constexpr double kPivMin = 1.0e-280;
 
-// Twisted factorisation of T - lambda I: forward pivots D+_i = p_i / p_{i-1} from the leading principal minors
+// power of two that brings a pair of running minors to about one
+__device__ __forceinline__ double minor_scale(double p, double pm) {
+  const int ex = ((__double2hiint(fabs(p) + fabs(pm)) >> 20) & 0x7ff) - 1023;
+  return __hiloint2double((1023 - max(min(ex, 1022), -1022)) << 20, 0);
+}
+// a zero or non-finite pivot is replaced, as a perturbed one would be
+__device__ __forceinline__ double safe_pivot(double x) {
+  if (!(fabs(x) >= kPivMin)) x = kPivMin;
+  return finite64(x) ? x : 1.0e300;
+}
+
+// Twisted factorisation of T - lambda I by one warp: forward pivots D+_i = p_i / p_{i-1} from the leading principal minors
 // p_i = (d_i - lambda) p_{i-1} - e_{i-1}^2 p_{i-2} (lane 0), backward pivots D- from the trailing ones (lane 1, the same
-// instructions on mirrored indices).  The recurrences carry no division: numerator and denominator of every pivot
-// are stored as a pair (the running pair is rescaled by a power of two every 8 steps, after it was stored) and the
+// instructions on mirrored addresses).  The recurrences carry no division: the minors are stored, the running pair is rescaled by a
+// power of two every 8 steps (after it was stored; who divides finds the factor again from the two minors), and the
 // quotients are taken by all lanes afterwards.  Twist index at the smallest |gamma_k| = |D+_k + D-_k - (d_k - lambda)|,
 // z_k = 1, z_i = -(e_i / D+_i) z_{i+1} above and z_{i+1} = -(e_i / D-_{i+1}) z_i below.  Returns gamma_k / z^T z, the
-// Rayleigh-quotient correction of lambda.  wa, wb, wc, wd, z: r doubles each, in shared or global memory.
+// Rayleigh-quotient correction of lambda.  na, nb, z: r doubles each, in shared memory.
+// Bound: the two serial loops.  Their operands are fetched eight steps at a time, so that a step is what the one warp issues (two
+// products, two loads and a store), not a round trip to memory.
 static __device__ __noinline__ double twisted_vector(const double* __restrict__ d, const double* __restrict__ e, int r, double lambda,
-                                 double* wa, double* wb, double* wc, double* wd, double* z, int lane, int skip,
-                                 double* znorm2) {
+                                                     double* na, double* nb, double* z, int lane, int skip,
+                                                     double* znorm2) {
+  constexpr int kStep = 8;
   if (lane < 2) {
     const bool back = lane == 1;
-    double* N = back ? wb : wa;                               // numerators
-    double* Q = back ? wd : wc;                               // denominators
-    int cur = back ? r - 1 : 0;
-    double pm = 1.0, p = d[cur] - lambda;
-    N[cur] = p; Q[cur] = pm;
-    double ee = r > 1 ? e[back ? r - 2 : 0] : 0.0;
-    double dn = r > 1 ? d[back ? r - 2 : 1] : 0.0;
-    for (int t = 0; t + 1 < r; ++t) {
-      const int nxt = back ? cur - 1 : cur + 1;
-      const int ie2 = back ? max(r - 3 - t, 0) : min(t + 1, r - 2);      // next step's off-diagonal and diagonal
-      const int in2 = back ? max(nxt - 1, 0) : min(nxt + 1, r - 1);
-      const double ee2 = e[ie2], dn2 = d[in2];
-      const double pn = fma(dn - lambda, p, -(ee * ee) * pm);
-      N[nxt] = pn; Q[nxt] = p;
-      pm = p; p = pn;
-      if ((t & 7) == 7) {
-        const int ex = ((__double2hiint(fabs(p) + fabs(pm)) >> 20) & 0x7ff) - 1023;
-        const double sc = __hiloint2double((1023 - max(min(ex, 1022), -1022)) << 20, 0);
-        p *= sc; pm *= sc;
+    const int s = back ? -1 : 1;
+    const double* pd = d + (back ? r - 1 : 0);
+    const double* pe = e + (back ? r - 2 : 0);
+    double* n = back ? nb + (r - 1) : na;
+    double pm = 1.0, p = *pd - lambda;
+    *n = p;
+    int t = 1;
+#pragma unroll 1
+    for (; t + kStep <= r; t += kStep) {
+      double dd[kStep], ee[kStep];
+#pragma unroll
+      for (int u = 0; u < kStep; ++u) { dd[u] = pd[s * (u + 1)]; ee[u] = pe[s * u]; }
+      pd += s * kStep; pe += s * kStep;
+#pragma unroll
+      for (int u = 0; u < kStep; ++u) {
+        const double pn = fma(dd[u] - lambda, p, -(ee[u] * ee[u]) * pm);
+        n[s * (u + 1)] = pn;
+        pm = p; p = pn;
       }
-      cur = nxt; ee = ee2; dn = dn2;
+      n += s * kStep;
+      const double sc = minor_scale(p, pm);
+      p *= sc; pm *= sc;
+    }
+    for (; t < r; ++t) {
+      pd += s; n += s;
+      const double pn = fma(*pd - lambda, p, -(*pe * *pe) * pm);
+      *n = pn;
+      pm = p; p = pn; pe += s;
     }
   }
   __syncwarp();
-  // pivots: wa <- D+, wb <- D- (a zero or non-finite quotient is replaced, as a perturbed pivot would be)
-  for (int i = lane; i < r; i += 32) {
-    double dp = wa[i] / wc[i], dm = wb[i] / wd[i];
-    if (!(fabs(dp) >= kPivMin)) dp = kPivMin;
-    if (!(fabs(dm) >= kPivMin)) dm = kPivMin;
-    if (!finite64(dp)) dp = 1.0e300;
-    if (!finite64(dm)) dm = 1.0e300;
-    wa[i] = dp; wb[i] = dm;
+  // pivots in place: na <- D+ (from the last index down: a quotient needs the two minors before it), nb <- D- (upwards)
+  const int top = (r - 1) / 32 * 32;
+#pragma unroll 2
+  for (int i0 = top; i0 >= 0; i0 -= 32) {
+    const int i = i0 + lane;
+    const double p = na[min(i, r - 1)], q1 = na[min(max(i - 1, 0), r - 1)], q2 = na[min(max(i - 2, 0), r - 1)];
+    const double q = i == 0 ? 1.0 : (i - 1) % kStep == 0 && i > 1 ? q1 * minor_scale(q1, q2) : q1;
+    __syncwarp();
+    if (i < r) na[i] = safe_pivot(p / q);
+    __syncwarp();
   }
-  __syncwarp();
+#pragma unroll 2
+  for (int i0 = 0; i0 <= top; i0 += 32) {
+    const int i = i0 + lane, t = r - 1 - i;                    // (mirrored index)
+    const double p = nb[min(i, r - 1)], q1 = nb[min(i + 1, r - 1)], q2 = nb[min(i + 2, r - 1)];
+    const double q = t <= 0 ? 1.0 : (t - 1) % kStep == 0 && t > 1 ? q1 * minor_scale(q1, q2) : q1;
+    __syncwarp();
+    if (i < r) nb[i] = safe_pivot(p / q);
+    __syncwarp();
+  }
   // twist index: the (skip+1)-th smallest |gamma| (lowest index on ties).  skip > 0 for the later members of a group
   // of kept atoms with coinciding eigenvalues: z = gamma_k (T - lambda I)^{-1} e_k, so another k is another start
   // vector of inverse iteration and gives another vector of the invariant subspace.
@@ -61,8 +92,9 @@ static __device__ __noinline__ double twisted_vector(const double* __restrict__ 
   for (int pick = 0; pick <= skip; ++pick) {
     const double pb = best; const int pk = bk;
     double cb = 1.0e300; int ck = 0x7fffffff;
+#pragma unroll 4
     for (int i = lane; i < r; i += 32) {
-      const double gam = fabs(wa[i] + wb[i] - (d[i] - lambda));
+      const double gam = fabs(na[i] + nb[i] - (d[i] - lambda));
       const bool after = gam > pb || (gam == pb && i > pk);   // not picked yet
       if (after && (gam < cb || (gam == cb && i < ck))) { cb = gam; ck = i; }
     }
@@ -76,31 +108,35 @@ static __device__ __noinline__ double twisted_vector(const double* __restrict__ 
     best = cb; bk = ck;
   }
   if (bk < 0) bk = 0;
-  const double gamma = wa[bk] + wb[bk] - (d[bk] - lambda);
+  const double gamma = na[bk] + nb[bk] - (d[bk] - lambda);
   __syncwarp();
-  // multipliers in place: wa[i] <- e_i / D+_i (i < r-1), wb[i] <- e_i / D-_{i+1}
-  for (int i0 = 0; i0 < r; i0 += 32) {
-    const int i = i0 + lane;
-    double l = 0.0, u = 0.0;
-    if (i + 1 < r) { l = e[i] / wa[i]; u = e[i] / wb[i + 1]; }
-    __syncwarp();
-    if (i < r) { wa[i] = l; wb[i] = u; }
-    __syncwarp();
-  }
+  // multipliers: na[i] <- e_i / D+_i above the twist, e_i / D-_{i+1} from there
+#pragma unroll 4
+  for (int i = lane; i < r - 1; i += 32) na[i] = e[i] / (i < bk ? na[i] : nb[i + 1]);
   if (lane == 0) z[bk] = 1.0;
   __syncwarp();
-  if (lane < 2) {
+  if (lane < 2) {                                             // lane 0 upwards from the twist, lane 1 downwards, in step
     const bool down = lane == 1;
+    const int s = down ? 1 : -1, n = down ? r - 1 - bk : bk, longer = max(bk, r - 1 - bk);
+    const double* pm = na + (down ? bk : bk - 1);
+    double* pz = z + (down ? bk + 1 : bk - 1);
     double zz = 1.0;
-    const int n = down ? r - 1 - bk : bk;
-    for (int t = 0; t < n; ++t) {
-      const int i = down ? bk + t : bk - 1 - t;               // multiplier index
-      zz = -(down ? wb[i] : wa[i]) * zz;
-      z[down ? i + 1 : i] = zz;
+#pragma unroll 1
+    for (int t = 0; t < longer; t += kStep) {
+      double m[kStep];
+#pragma unroll
+      for (int u = 0; u < kStep; ++u) m[u] = t + u < n ? pm[s * u] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kStep; ++u) {
+        zz = -m[u] * zz;
+        if (t + u < n) pz[s * u] = zz;
+      }
+      pm += s * kStep; pz += s * kStep;
     }
   }
   __syncwarp();
   double n2 = 0.0;
+#pragma unroll 4
   for (int i = lane; i < r; i += 32) n2 = fma(z[i], z[i], n2);
   n2 = warp_sum(n2);
   *znorm2 = n2;
