@@ -10,17 +10,19 @@ namespace atomo {
 
 // ---- vectors of the kept atoms ------------------------------------------------------------------------------------
 // Two phases per CTA.  (A) one warp per kept atom: the eigenvector of T by the twisted factorisation of the small
-// route (work vectors in global memory), normalised.  (B) the whole CTA takes up to four of its atoms at once through the
+// route (work vectors in shared memory), normalised.  (B) the whole CTA takes its atoms through the
 // reflectors, all in fp64 (the reflectors of the panels are fp32 numbers, and Q1 is exactly what the band reduction
-// applied): first the chase's (vb_chase_back), then the panels', four reflectors at a time.  There a thread owns the columns
-// tid, tid + 512, ... of the four reflector rows (read once per group, kept in registers between the dot products and the
-// update) and of every z (in shared memory; no other thread touches them), so the only exchange per group is the
-// block-wide sum of the products p_i = u_i.z; with the group's 4 x 4 block T of the panel's triangular factor,
-// z -= sum_i u_i (T p)_i.  The matrix of reflectors is read once per batch of atoms.
+// applied): first the chase's (vb_chase_back), one or two atoms at a time, then the panels' (vb_apply_reflectors), up to four at
+// a time, so that their rows are read once.
 // In fp32 (reflectors of the chase rounded, every application rounded) a kept atom's residual |A u - lambda u| / lambda_1 was
 // 2.7e-8 instead of 1.0e-8 on 1024 x 4096 noise, its vectors orthogonal to 2.4e-7 instead of 4e-9: the eigenvector of the band
-// fills eight times as many entries as one of a one-stage T, and each of its reflectors rounds them.  Cost: two layers of 4096 rows 7.5 -> 8.3 ms for this and
-// the back-projection, 96 of 1024 rows 1.7 -> 2.1.
+// fills eight times as many entries as one of a one-stage T, and each of its reflectors rounds them.
+// Measured, before (a block barrier per sweep, four panel reflectors at a time, work vectors in global memory) | now: two layers of 4096 rows
+// 8.0 | 3.7 ms, nine of 2048 rows 2.23 | 1.30, 96 of 1024 rows 1.66 | 1.02, one of 1023 rows 0.54 | 0.33.  What bounds it now:
+// the panels (sums over all warps and conversions to fp64: 3500 cycles each at 1024 rows, 8500 at 4096), then the sweeps of the chase
+// (290 and 640 cycles each).
+// Tried and dropped: what the moves bring fetched once per turn instead of a load per sweep (spills: 3.8 -> 4.5 ms); eight warps per atom up
+// to 1024 rows (1.02 -> 1.12 ms).
 namespace {
 constexpr int kVbThreads = 512;
 constexpr int kVbWarps = kVbThreads / 32;
@@ -178,7 +180,7 @@ __device__ __forceinline__ void vb_apply_reflectors(const float* __restrict__ gV
 // Bound: the reflectors, 4 r^2 bytes of fp64 per vector through one SM.
 namespace {
 template <int THREADS, int ATOMS, int DEPTH>
-__device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, const int r, double* s_z, const int z_stride,
+__device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, const int r, double* s_z, const int z_stride, const int n_vecs,
                                               double (*s_edge)[THREADS / 32][8]) {
   constexpr int kPer = THREADS / ATOMS;                        // threads per vector
   static_assert(8 % DEPTH == 0, "a sweep's registers are the same in every turn");
@@ -186,7 +188,7 @@ __device__ __forceinline__ void vb_chase_back(const double* __restrict__ gV2, co
   double* const z = s_z + (size_t)(tid / kPer) * z_stride;
   const int turns = max(r - 2 + 7, 0) / 8;                     // the first sweeps of a partial turn act on nothing
   // the first turn in which one of the warp's entries is inside: before, they are all zeros
-  const int first = max(0, (8 * turns + 256 * wv - r) / 8);
+  const int first = tid / kPer < n_vecs ? max(0, (8 * turns + 256 * wv - r) / 8) : turns;
   const int j_first = 8 * (turns - first) - 1;
   const int64_t row = sp_chase_row(r);
   const double* from = gV2 + (j_first * row + wv * 256 + lane * 2);
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
         for (int i = lane; i < r; i += 32) s_z[i] *= inv;
       }
       __syncthreads();
-      vb_chase_back<kVcThreads, 1, 8>(L.bd_V2, r, s_z, rp, s_edge);
+      vb_chase_back<kVcThreads, 1, 8>(L.bd_V2, r, s_z, rp, 1, s_edge);
       vb_apply_reflectors<kVcThreads, 1, kVcMaxRp / kVcThreads>(gV, ldv, L.bd_T, r, rp, nref, 1, s_z, s_part, s_tot);
       double n2 = 0.0;
       for (int i = tid; i < r; i += kVcThreads) n2 = fma(s_z[i], s_z[i], n2);
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
     }
     __syncthreads();
     // a run per thread: one or two atoms at a time
-    for (int b = 0; b < nb; b += kFew) vb_chase_back<kVbThreads, kFew, 4>(L.bd_V2, r, s_z + (size_t)b * rp, rp, s_edge);
+    for (int b = 0; b < nb; b += kFew) vb_chase_back<kVbThreads, kFew, 4>(L.bd_V2, r, s_z + (size_t)b * rp, rp, nb - b, s_edge);
     vb_apply_reflectors<kVbThreads, BATCH, COLS>(gV, ldv, L.bd_T, r, rp, nref, nb, s_z, s_part, s_tot);
     // normalise and file
     for (int b = 0; b < nb; ++b) {
