@@ -420,11 +420,22 @@ __global__ void __launch_bounds__(kFinThreads) sp_finalize_sample_kernel(const S
   }
   __syncthreads();
   const bool bad = s_bad != 0;
-  // rank by counting (descending, ties: lower row first); sigma = sqrt(lambda)
+  // rank (descending, ties: lower row first); sigma = sqrt(lambda).  The tridiagonal routes hand over ascending values, but for the
+  // last digits: then two binary searches find the rank, else it is counted (r^2 comparisons by one CTA: 0.5 ms at 4096 rows)
+  bool falls = false;
+  for (int i = tid; i + 1 < r; i += kFinThreads) falls |= !(s_lam[i] <= s_lam[i + 1]);
+  const bool ascending = !__syncthreads_or(falls);
   for (int i = tid; i < r; i += kFinThreads) {
     const float li = s_lam[i];
     int rank = 0;
-    for (int j = 0; j < r; ++j) { const float lj = s_lam[j]; rank += (lj > li) || (lj == li && j < i); }
+    if (ascending) {
+      int below = 0, upto = i;                                 // values below li, values up to li: [below, upto)
+      for (int n = i; n > 0;) { const int half = n / 2; if (s_lam[below + half] < li) { below += half + 1; n -= half + 1; } else n = half; }
+      for (int n = r - i; n > 0;) { const int half = n / 2; if (s_lam[upto + half] <= li) { upto += half + 1; n -= half + 1; } else n = half; }
+      rank = r - upto + i - below;
+    } else {
+      for (int j = 0; j < r; ++j) { const float lj = s_lam[j]; rank += (lj > li) || (lj == li && j < i); }
+    }
     s_sig[rank] = bad ? 0.0f : sqrtf(li);
     L.perm[rank] = i;
   }
