@@ -7,8 +7,8 @@
 //                               of a 16-CTA cluster and stay in registers; per step the product A v and the next
 //                               pivot column's ingredients travel through distributed shared memory.  The
 //                               reflectors go to global memory as fp32 unit vectors for the back-transformation.
-//   sp_bisect_kernel          : all eigenvalues of T, eight lanes per eigenvalue: 13 rounds of 9-section on Sturm
-//                               counts (division-free three-term recurrence with power-of-two rescaling).
+//   sp_bisect_kernel          : all eigenvalues of T from Sturm counts and determinants (division-free three-term
+//                               recurrence with power-of-two rescaling).
 //   (sp_finalize_sample_kernel sorts, solves Algorithm 1 and draws, as for the other routes)
 //   sp_eigvec_kernel          : for the kept atoms only: eigenvector of T by a twisted factorisation with one
 //                               Rayleigh-quotient correction, back-transformation u = Q z with the reflectors
@@ -16,7 +16,7 @@
 //                               nearly equal eigenvalues are orthogonalised against each other at the end.
 //
 // Work per layer: about 2 r^3 fp64 flops for the reduction (full symmetric storage: matrix-vector product and
-// rank-two update of the trailing block), r^2 * 13 * 8 recurrence steps for the eigenvalues, O(r^2) per kept atom.
+// rank-two update of the trailing block), about 11 r^2 to 32 r^2 recurrence steps for the eigenvalues, O(r^2) per kept atom.
 #include <type_traits>
 
 #include <cooperative_groups.h>
@@ -274,87 +274,157 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
 
 // ---- eigenvalues of T: Sturm counts -------------------------------------------------------------------------
 // count(x) = number of eigenvalues below x = sign changes of p_0 = 1, p_1 = d_0 - x, p_{i+1} = (d_i - x) p_i -
-// e_{i-1}^2 p_{i-1}.  The pair (p_i, p_{i-1}) is rescaled by a power of two every 8 steps (ratios and signs keep).
-__device__ __forceinline__ int sturm_count(const double* __restrict__ d, const double* __restrict__ e2, int r, double x) {
+// e_{i-1}^2 p_{i-1}.  The pair (p_i, p_{i-1}) is rescaled by a power of two every 8 steps (ratios and signs keep).  The last
+// term, |p_r| = |det(T - x I)| up to a constant factor, comes as val * 2^ex.
+struct SturmPoint { double x, val; int cnt, ex; };
+// (d + 1 and e2 on 16-byte boundaries, padded with kSturmPad, far above every eigenvalue, and 0 up to eight entries past the end: there
+// the step is p <- (pad - x) p, which keeps the sign.)  A step is one multiply-add in the serial chain: the operands of the next eight
+// steps are fetched, the sign bits gathered and the power of two taken (from a pair two steps back) beside it.
+__device__ __forceinline__ SturmPoint sturm_point(const double* __restrict__ d, const double* __restrict__ e2, int r, double x) {
   double pm = 1.0, p = d[0] - x;
-  int neg = __double2hiint(p);                                // sign bit of the previous term
-  int cnt = (uint32_t)neg >> 31;
-  // eight steps at a time: their operands are fetched together, so that only the multiply-add chain is serial.
-  // The caller pads d with kSturmPad (far above every eigenvalue) and e2 with 0 up to a multiple of 8 past the end:
-  // there the step is p <- (pad - x) p, which keeps the sign.
-  for (int i0 = 1; i0 < r; i0 += 8) {
-    double dd[8], ee[8];
+  uint32_t signs = (uint32_t)__double2hiint(p) >> 31;         // the newest in bit 0
+  int cnt = (int)signs, shift = 0;
+  auto fetch = [&](double (&dd)[8], double (&ee)[8], int i0) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) { dd[u] = d[i0 + u] - x; ee[u] = e2[i0 + u - 1]; }   // padded arrays: no bounds test
+    for (int u = 0; u < 8; u += 2) {
+      const double2 a = *reinterpret_cast<const double2*>(d + i0 + u), b = *reinterpret_cast<const double2*>(e2 + i0 + u - 1);
+      dd[u] = a.x; dd[u + 1] = a.y; ee[u] = b.x; ee[u + 1] = b.y;
+    }
+  };
+  double dd[8], ee[8];
+  if (r > 1) fetch(dd, ee, 1);
+#pragma unroll 2
+  for (int i0 = 1; i0 < r; i0 += 8) {
+    double nd[8], ne[8];
+    fetch(nd, ne, i0 + 8 < r ? i0 + 8 : i0);
+    int top = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const double pn = fma(dd[u], p, -ee[u] * pm);
-      const int hn = __double2hiint(pn);
-      cnt += (uint32_t)(hn ^ neg) >> 31;
-      neg = hn;
+      const double pn = fma(dd[u] - x, p, -ee[u] * pm);
+      signs = __funnelshift_l((uint32_t)__double2hiint(pn), signs, 1);
       pm = p; p = pn;
+      if (u == 5) top = max(__double2hiint(p) & 0x7fffffff, __double2hiint(pm) & 0x7fffffff) >> 20;
     }
-    const int ex = ((__double2hiint(fabs(p) + fabs(pm)) >> 20) & 0x7ff) - 1023;
-    const double sc = __hiloint2double((1023 - max(min(ex, 1022), -1022)) << 20, 0);
-    p *= sc; pm *= sc;
+    cnt += __popc((signs ^ (signs >> 1)) & 0xffu);
+    const int ex = max(min(top - 1023, 1022), -1022);
+    const double sc = __hiloint2double((1023 - ex) << 20, 0);
+    p *= sc; pm *= sc; shift += ex;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) { dd[u] = nd[u]; ee[u] = ne[u]; }
   }
-  return cnt;
+  return SturmPoint{x, fabs(p), cnt, shift};
+}
+// where the line through the two values crosses zero, as a part of the way from a to b (the values have opposite signs)
+__device__ __forceinline__ double sturm_part(const SturmPoint& a, const SturmPoint& b) {
+  const int top = max(a.ex, b.ex);
+  const double va = a.val * __hiloint2double((1023 + max(a.ex - top, -1022)) << 20, 0), vb = b.val * __hiloint2double((1023 + max(b.ex - top, -1022)) << 20, 0);
+  return va / fmax(va + vb, 1.0e-300);
+}
+__device__ __forceinline__ SturmPoint sturm_from(const SturmPoint& p, int lane) {
+  return SturmPoint{__shfl_sync(0xffffffffu, p.x, lane), __shfl_sync(0xffffffffu, p.val, lane), __shfl_sync(0xffffffffu, p.cnt, lane),
+                    __shfl_sync(0xffffffffu, p.ex, lane)};
 }
 
 constexpr double kSturmPad = 1.0e6;    // diagonal entries past the end (the matrices are scaled to trace <= 1)
-constexpr int kBisThreads = 64;           // small CTAs: the warps of a large layer spread over all SMs (the recurrences are latency-bound)
-// Points per round and eigenvalue (kBisLanes lanes work on one eigenvalue: the interval shrinks kBisLanes + 1 times per
-// round) and rounds, chosen so that the final interval is below 1e-12 of the spectrum's extent: 8 lanes and 13 rounds
-// (9^13 = 2.5e12) where the batch has few eigenvalues and the chain of rounds is what takes the time; 2 lanes and 26
-// rounds (3^26 = 2.5e12) where it has many: half the Sturm counts per eigenvalue, and enough eigenvalues to fill the GPU.
-template <int kBisLanes, int kBisRounds, int THREADS = kBisThreads>
+constexpr int kBisRounds = 100;        // bound of the loop (halving the brackets alone would take 30)
+
+// A CTA takes THREADS / LANES neighbouring eigenvalues.  Two rounds of THREADS counts bracket them: points over the whole
+// spectrum, then over the part that holds the CTA's eigenvalues, so that most brackets hold a single one.  Then two or four lanes per
+// eigenvalue: as long as a bracket holds several, it is cut in equal parts; after that the determinant, which the
+// counts yield for nothing, says where in the bracket the eigenvalue lies, and the lanes' points are set around that crossing, at a
+// distance delta (with four lanes 4 delta as well), a part of the bracket that is squared when the inner
+// pair has caught the eigenvalue.  Every bracket is one by the counts: the values only choose
+// the points.  Final brackets are below 4e-13 of the spectrum's extent, and the line through their values is exact to about 5e-14
+// of it (the midpoint where a bracket still holds several).
+// Bound: the serial chain of the recurrence with few eigenvalues (four lanes, 2 + 8 rounds), fp64 with many (two lanes, half the counts).
+// Before, with sections without the values (13 rounds of eight counts, 26 of two or 41 of one) and a recurrence that
+// waited for its operands | now, us: ResNet-18 set 118 | 74, one 64 x 64 layer 16.7 | 11.1, two layers of 4096 rows 2152 | 985, nine
+// of 2048 1022 | 601, 96 of 1024 1724 | 1026.  One lane with a regula falsi took 1035 us on the last: a warp waits for its slowest.
+template <int LANES, int THREADS>
 __global__ void __launch_bounds__(THREADS) sp_bisect_kernel(const SpLayer* __restrict__ layers, int bis_stride) {
-  constexpr int kBisPerCta = THREADS / kBisLanes;
+  static_assert(LANES == 2 || LANES == 4, "two lanes per eigenvalue or four");
+  constexpr int kPerCta = THREADS / LANES;
   const SpLayer& L = layers[blockIdx.y];
   if (!L.tri) return;
   const int r = L.r;
   const int tid = threadIdx.x, lane = tid % 32;
-  if ((int)blockIdx.x * kBisPerCta >= r) return;
+  const int j0 = (int)blockIdx.x * kPerCta;
+  if (j0 >= r) return;
   extern __shared__ __align__(16) double bis_smem[];           // d and e^2, r_max + 8 entries each
-  double* const s_d = bis_smem;
+  double* const s_d = bis_smem + 1;                            // (entry 1 on a 16-byte boundary)
   double* const s_e2 = bis_smem + bis_stride;
-  for (int i = tid; i < r + 8; i += THREADS) {
-    s_d[i] = i < r ? L.td_d[i] : kSturmPad;
-    const double e = i + 1 < r ? L.td_e[i] : 0.0;
-    s_e2[i] = e * e;
-  }
-  __syncthreads();
-  // Gershgorin interval (every warp the same), widened a little; a NaN or Inf anywhere poisons the result
+  __shared__ SturmPoint s_pt[THREADS];
+  __shared__ double s_lo[THREADS / 32], s_hi[THREADS / 32];
+  // Gershgorin interval, widened a little; a NaN or Inf anywhere poisons the result
   double gl = 1.0e300, gu = -1.0e300;
   bool bad = false;
-  for (int i = lane; i < r; i += 32) {
-    const double el = i > 0 ? sqrt(s_e2[i - 1]) : 0.0, er = sqrt(s_e2[i]);
-    gl = fmin(gl, s_d[i] - el - er); gu = fmax(gu, s_d[i] + el + er);
-    bad |= !finite64(s_d[i]) || !finite64(s_e2[i]);
+  for (int i = tid; i < r + 8; i += THREADS) {
+    const double d = i < r ? L.td_d[i] : kSturmPad, er = i + 1 < r ? L.td_e[i] : 0.0, el = i > 0 && i < r ? L.td_e[i - 1] : 0.0;
+    s_d[i] = d;
+    s_e2[i] = er * er;
+    if (i < r) {
+      gl = fmin(gl, d - fabs(el) - fabs(er)); gu = fmax(gu, d + fabs(el) + fabs(er));
+      bad |= !finite64(d) || !finite64(er * er);
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) { gl = fmin(gl, __shfl_xor_sync(0xffffffffu, gl, o)); gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, o)); }
-  bad = __any_sync(0xffffffffu, bad);
-  const int grp = lane / kBisLanes, t = lane % kBisLanes;     // 4 eigenvalues per warp, 8 lanes each
-  const int j = blockIdx.x * kBisPerCta + (tid / 32) * (32 / kBisLanes) + grp;   // ascending order
-  const int jj = min(j, r - 1);                               // lanes past the end follow the last eigenvalue
+  if (lane == 0) { s_lo[tid / 32] = gl; s_hi[tid / 32] = gu; }
+  bad = __syncthreads_or(bad);
+#pragma unroll
+  for (int w = 0; w < THREADS / 32; ++w) { gl = fmin(gl, s_lo[w]); gu = fmax(gu, s_hi[w]); }
+  const int j = j0 + tid / LANES, jj = min(j, r - 1);         // ascending order; lanes past the end follow the last eigenvalue
+  const bool files = tid % LANES == 0 && j < r;
   if (bad) {
-    if (t == 0 && j < r) { L.lam64[j] = __longlong_as_double(0x7ff8000000000000ll); L.lam[j] = __int_as_float(0x7fc00000); }
+    if (files) { L.lam64[j] = __longlong_as_double(0x7ff8000000000000ll); L.lam[j] = __int_as_float(0x7fc00000); }
     return;
   }
   const double pad = 1.0e-14 * fmax(fabs(gl), fabs(gu)) + 1.0e-300;
-  double lo = gl - pad, hi = gu + pad;
-  for (int it = 0; it < kBisRounds; ++it) {
-    const double h = (hi - lo) * (1.0 / (kBisLanes + 1));
-    const double x = fma((double)(t + 1), h, lo);
-    const int cnt = sturm_count(s_d, s_e2, r, x);
-    const uint32_t le = __ballot_sync(0xffffffffu, cnt <= jj);              // points not above lambda_j
-    const int nle = __popc((le >> (grp * kBisLanes)) & ((1u << kBisLanes) - 1u));
-    const double nlo = fma((double)nle, h, lo);
-    hi = fmin(hi, fma((double)(nle + 1), h, lo));
-    lo = nlo;
+  gl -= pad; gu += pad;
+  const double tol = fmax(4.0e-13 * (gu - gl), 1.0e-15 * fmax(fabs(gl), fabs(gu)));
+  SturmPoint lo, hi;
+  {
+    const double h = (gu - gl) * (1.0 / (THREADS + 1));
+    const int cnt = sturm_point(s_d, s_e2, r, fma((double)(tid + 1), h, gl)).cnt;
+    const int below = __syncthreads_count(cnt <= j0), upto = __syncthreads_count(cnt <= min(j0 + kPerCta, r) - 1);
+    const double a = fma((double)below, h, gl), b = upto == THREADS ? gu : fma((double)(upto + 1), h, gl);
+    s_pt[tid] = sturm_point(s_d, s_e2, r, tid == THREADS - 1 ? b : fma((double)tid, (b - a) * (1.0 / (THREADS - 1)), a));
+    __syncthreads();
+    int first = 0, n = THREADS;                               // points whose count is at most jj come first
+    while (n > 0) { const int half = n / 2; if (s_pt[first + half].cnt <= jj) { first += half + 1; n -= half + 1; } else n = half; }
+    first = max(1, min(first, THREADS - 1));
+    lo = s_pt[first - 1]; hi = s_pt[first];
   }
-  if (t == 0 && j < r) { const double lam = 0.5 * (lo + hi); L.lam64[j] = lam; L.lam[j] = (float)lam; }
+  double lam = 0.5 * (lo.x + hi.x);
+  const int t = lane % LANES, base = lane - t;
+  constexpr double kRho = 1.0 / 16.0, kRhoMost = LANES == 4 ? 0.125 : 0.25;
+  double rho = kRho;
+  bool done = false;
+  for (int it = 0; it < kBisRounds; ++it) {
+    const double w = hi.x - lo.x;
+    const bool single = hi.cnt - lo.cnt == 1;
+    const double s = fma(sturm_part(lo, hi), w, lo.x);
+    if (!done) lam = single ? s : 0.5 * (lo.x + hi.x);
+    done |= w <= tol;
+    if (__all_sync(0xffffffffu, done)) break;
+    const double delta = fmax(rho * w, 0.45 * tol);
+    // the inner point of this lane's side and the outer one, inside the bracket in this order
+    const bool left = t < LANES / 2, inner = LANES == 2 || t == 1 || t == 2;
+    const double way = left ? s - lo.x : hi.x - s;            // from the crossing to the end on this side
+    const double in = way > delta ? delta : 0.999 * way, out = way > 4.0 * delta ? 4.0 * delta : 0.5 * (in + way);
+    const double off = inner ? in : out;
+    const double x = single ? (left ? s - off : s + off) : fma((double)(t + 1), w * (1.0 / (LANES + 1)), lo.x);
+    const SturmPoint p = sturm_point(s_d, s_e2, r, x);
+    const int le = __popc(__ballot_sync(0xffffffffu, p.cnt <= jj) >> base & ((1u << LANES) - 1u));   // points not above the eigenvalue
+    const SturmPoint a = sturm_from(p, base + max(le - 1, 0)), b = sturm_from(p, base + min(le, LANES - 1));
+    if (!done) {
+      if (le > 0) lo = a;
+      if (le < LANES) hi = b;
+      const double now = hi.x - lo.x;
+      rho = !single ? kRho : now <= 2.01 * delta ? fmax(rho * rho, 3.8e-6) : LANES == 4 && now <= 3.03 * delta ? rho : fmin(sqrt(rho), kRhoMost);
+    }
+  }
+  if (files) { L.lam64[j] = lam; L.lam[j] = (float)lam; }
 }
 
 // ---- vectors of the kept atoms --------------------------------------------------------------------------------
@@ -540,11 +610,10 @@ int sp_tridiag_ctas_of(int rp) { return rp / kTriRows < 1 ? 1 : rp / kTriRows; }
 // the eigenvalue kernel keeps d and e^2 of a layer in shared memory: more than the default 48 KB above a short side of
 // about 3000.  Both tridiagonal routes need this (a batch may hold large layers only).  0 if it went through.
 int sp_configure_bisect() {
-  const int bytes = (int)(2 * (kMaxShort + 10) * sizeof(double));
-  if (cudaFuncSetAttribute(sp_bisect_kernel<1, 41>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(sp_bisect_kernel<8, 13>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(sp_bisect_kernel<8, 13, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(sp_bisect_kernel<2, 26>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+  const int bytes = (int)(2 * (kMaxShort + 12) * sizeof(double));
+  if (cudaFuncSetAttribute(sp_bisect_kernel<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(sp_bisect_kernel<4, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(sp_bisect_kernel<4, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
@@ -582,23 +651,17 @@ int launch_sp_tridiag(const SpLayer* d_layers, const ClusterCta* d_ctas, int n_c
 }
 
 void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t n_eigenvalues, cudaStream_t st) {
-  const int stride = (r_max + 8 + 1) & ~1;
+  const int stride = (r_max + 9 + 1) & ~1;
   const size_t smem = 2 * (size_t)stride * sizeof(double);
-  if (n_eigenvalues >= 65536) {
-    // enough eigenvalues to fill the fp64 pipes with one lane each: plain bisection gets one bit per Sturm count
-    // (3-section 0.79, 9-section 0.40), 41 rounds for the same final width as the other forms
-    constexpr int per = kBisThreads;
-    sp_bisect_kernel<1, 41><<<dim3((r_max + per - 1) / per, n_layers), kBisThreads, smem, st>>>(d_layers, stride);
-  } else if (n_eigenvalues >= 16384) {
-    constexpr int per = kBisThreads / 2;
-    sp_bisect_kernel<2, 26><<<dim3((r_max + per - 1) / per, n_layers), kBisThreads, smem, st>>>(d_layers, stride);
+  // two lanes per eigenvalue where there are many, else four (us, two | four: 18432 eigenvalues of 2048-row layers 601 | 764, 20000 of
+  // 500-row layers 160 | 187, 4700 of the ResNet-18 set 112 | 74, 11000 of the VGG-11 set 1082 | 985)
+  if (n_eigenvalues >= 16384) {
+    sp_bisect_kernel<2, 64><<<dim3((r_max + 31) / 32, n_layers), 64, smem, st>>>(d_layers, stride);
   } else if (r_max > 2048) {
-    // 64 KB of d and e^2 per CTA at 4096 rows: three CTAs per SM, so they have to be larger to fill it (2 x 4096: 2.60 -> 2.11 ms)
-    constexpr int per = 256 / 8;
-    sp_bisect_kernel<8, 13, 256><<<dim3((r_max + per - 1) / per, n_layers), 256, smem, st>>>(d_layers, stride);
+    // 64 KB of d and e^2 per CTA at 4096 rows: three CTAs per SM, so they are larger
+    sp_bisect_kernel<4, 128><<<dim3((r_max + 31) / 32, n_layers), 128, smem, st>>>(d_layers, stride);
   } else {
-    constexpr int per = kBisThreads / 8;
-    sp_bisect_kernel<8, 13><<<dim3((r_max + per - 1) / per, n_layers), kBisThreads, smem, st>>>(d_layers, stride);
+    sp_bisect_kernel<4, 64><<<dim3((r_max + 15) / 16, n_layers), 64, smem, st>>>(d_layers, stride);
   }
 }
 

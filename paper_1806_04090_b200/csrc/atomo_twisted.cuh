@@ -32,6 +32,7 @@ static __device__ __noinline__ double twisted_vector(const double* __restrict__ 
                                                      double* na, double* nb, double* z, int lane, int skip,
                                                      double* znorm2) {
   constexpr int kStep = 8;
+  bool dead = false;
   if (lane < 2) {
     const bool back = lane == 1;
     const int s = back ? -1 : 1;
@@ -63,27 +64,44 @@ static __device__ __noinline__ double twisted_vector(const double* __restrict__ 
       *n = pn;
       pm = p; p = pn; pe += s;
     }
+    dead = p == 0.0;
   }
-  __syncwarp();
-  // pivots in place: na <- D+ (from the last index down: a quotient needs the two minors before it), nb <- D- (upwards)
-  const int top = (r - 1) / 32 * 32;
+  // two zeros in a row (lambda a diagonal entry beside a zero off-diagonal one, to the last digit) end a sequence of minors: then
+  // the pivots themselves, a division per step
+  if (__any_sync(0xffffffffu, dead)) {
+    if (lane < 2) {
+      const bool back = lane == 1;
+      double D = 1.0;
+      for (int t = 0; t < r; ++t) {
+        const int i = back ? r - 1 - t : t;
+        const double ee = t == 0 ? 0.0 : e[back ? i : i - 1];
+        D = safe_pivot(d[i] - lambda - ee * ee / D);
+        (back ? nb : na)[i] = D;
+      }
+    }
+    __syncwarp();
+  } else {
+    __syncwarp();
+    // pivots in place: na <- D+ (from the last index down: a quotient needs the two minors before it), nb <- D- (upwards)
+    const int top = (r - 1) / 32 * 32;
 #pragma unroll 2
-  for (int i0 = top; i0 >= 0; i0 -= 32) {
-    const int i = i0 + lane;
-    const double p = na[min(i, r - 1)], q1 = na[min(max(i - 1, 0), r - 1)], q2 = na[min(max(i - 2, 0), r - 1)];
-    const double q = i == 0 ? 1.0 : (i - 1) % kStep == 0 && i > 1 ? q1 * minor_scale(q1, q2) : q1;
-    __syncwarp();
-    if (i < r) na[i] = safe_pivot(p / q);
-    __syncwarp();
-  }
+    for (int i0 = top; i0 >= 0; i0 -= 32) {
+      const int i = i0 + lane;
+      const double p = na[min(i, r - 1)], q1 = na[min(max(i - 1, 0), r - 1)], q2 = na[min(max(i - 2, 0), r - 1)];
+      const double q = i == 0 ? 1.0 : (i - 1) % kStep == 0 && i > 1 ? q1 * minor_scale(q1, q2) : q1;
+      __syncwarp();
+      if (i < r) na[i] = safe_pivot(p / q);
+      __syncwarp();
+    }
 #pragma unroll 2
-  for (int i0 = 0; i0 <= top; i0 += 32) {
-    const int i = i0 + lane, t = r - 1 - i;                    // (mirrored index)
-    const double p = nb[min(i, r - 1)], q1 = nb[min(i + 1, r - 1)], q2 = nb[min(i + 2, r - 1)];
-    const double q = t <= 0 ? 1.0 : (t - 1) % kStep == 0 && t > 1 ? q1 * minor_scale(q1, q2) : q1;
-    __syncwarp();
-    if (i < r) nb[i] = safe_pivot(p / q);
-    __syncwarp();
+    for (int i0 = 0; i0 <= top; i0 += 32) {
+      const int i = i0 + lane, t = r - 1 - i;                    // (mirrored index)
+      const double p = nb[min(i, r - 1)], q1 = nb[min(i + 1, r - 1)], q2 = nb[min(i + 2, r - 1)];
+      const double q = t <= 0 ? 1.0 : (t - 1) % kStep == 0 && t > 1 ? q1 * minor_scale(q1, q2) : q1;
+      __syncwarp();
+      if (i < r) nb[i] = safe_pivot(p / q);
+      __syncwarp();
+    }
   }
   // twist index: the (skip+1)-th smallest |gamma| (lowest index on ties).  skip > 0 for the later members of a group
   // of kept atoms with coinciding eigenvalues: z = gamma_k (T - lambda I)^{-1} e_k, so another k is another start
