@@ -297,6 +297,7 @@ int chase_room(atomo_ctx* ctx, int ctas) {
   if (known < 0) known = sp_chase_capacity(ctas);
   return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
+constexpr int64_t kI8Elements = (int64_t)1 << 26;             // elements from which layers of 513 .. 1024 rows take the integer Gram kernel
 int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
 bool bad_budget(double s) { return !(s > 0.0) || !std::isfinite(s); }
@@ -501,11 +502,13 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
 
   // ---- host descriptors, tiles, workspace carving (two passes: size, then pointers) ----
   std::vector<SpLayer> L(n_layers);
-  std::vector<int> tc_layers;
-  std::vector<TileRef> gram_tiles, gram_parts, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles;
+  std::vector<int> tc_layers, i8_layers;
+  std::vector<TileRef> gram_tiles, gram_parts, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles, i8_rows, i8_prep, i8_tiles;
   const int map_bytes = sp_tc_map_bytes();
   std::vector<uint8_t> maps_blob((size_t)n_layers * map_bytes, 0);
   int chol_panels = 0;
+  int64_t mid_elements = 0;                                  // of the layers with a short side of 513 .. 1024
+  for (int l = 0; l < n_layers; ++l) { const int r = std::min(layers[l].rows, layers[l].cols); if (r > 512 && r <= 1024) mid_elements += (int64_t)layers[l].rows * layers[l].cols; }
   int row_floats_max = 0, steps_max = 0, r_max = 0, rp_max = 0, r_max_tall = 0, k_cap_max = 1;
   for (int l = 0; l < n_layers; ++l) {
     SpLayer& d = L[l];
@@ -524,13 +527,17 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     r_max = std::max(r_max, d.r); rp_max = std::max(rp_max, d.rp);
     const int gt = (d.r + 63) / 64;
     d.tc = 0; d.gram_split = 1; d.gram_part_len = d.L;
-    // The tensor core's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
-    // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the
-    // fp32 FMA kernel, whose sums round to nearest (their Gram matrix is a small part of their cost)
-    if (ctx->tc_gram && ctx->tc_ok && !d.acc && d.r <= 1024 && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
+    // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
+    // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
+    // kernel, and above 512 those that the TF32 kernel cannot take, or all where they are many (with its digits, TF32 |
+    // integer, us: 20 layers of 1000 x 1200 241 | 259, one of 1024 x 4096 51 | 64, 40 of 520 x 8000 1081 | 767, 96 of 1024 x 4096 2818 | 2185)
+    if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && mid_elements < kI8Elements)) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
       d.tc = 1;
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
+    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && d.r > 512) {
+      d.tc = 2;
+      i8_layers.push_back(l);
     } else {
       d.gram_split = given ? 1 : sp_gram_split(d.r, d.L);
       d.gram_part_len = sp_gram_part(d.r, d.L);
@@ -624,6 +631,28 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       total += tiles_of(best) * L[best].gram_split;
       L[best].gram_split *= 2;
     }
+    // integer tiles likewise (at least 8 stages of 64 columns per part); their sums are exact in any number of parts
+    total = 0;
+    for (int l : i8_layers) { L[l].gram_split = sp_i8_min_split(L[l].L); total += tiles_of(l) * L[l].gram_split; }
+    for (;;) {
+      int best = -1;
+      for (int l : i8_layers) {
+        const int stages = sp_i8_stages(L[l].L) / L[l].gram_split;
+        if (stages >= 16 && total + tiles_of(l) * L[l].gram_split <= sms && (best < 0 || stages > sp_i8_stages(L[best].L) / L[best].gram_split)) best = l;
+      }
+      if (best < 0) break;
+      total += tiles_of(best) * L[best].gram_split;
+      L[best].gram_split *= 2;
+    }
+    for (int l : i8_layers) {
+      const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
+      for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
+        for (int c = 0; c < L[l].gram_split; ++c) i8_tiles.push_back({l, a, b, c});
+      int na = 0, nb = 0;
+      sp_i8_prep_tiles(L[l].r, L[l].L, L[l].tall, &na, &nb);
+      for (int a = 0; a < na; ++a) for (int b = 0; b < nb; ++b) (sp_i8_by_rows(L[l].L, L[l].tall) ? i8_rows : i8_prep).push_back({l, a, b, 0});
+    }
+    i8_prep.insert(i8_prep.begin(), i8_rows.begin(), i8_rows.end());
     for (int l : tc_layers) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
@@ -705,7 +734,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   }
   // the tables go to the table cache (device buffer tab_sp, host mirror `tables` with the same offsets), everything
   // the kernels write to the workspace
-  SpLayer* d_layers = nullptr; TileRef *d_gram = nullptr, *d_pairs = nullptr, *d_bp = nullptr, *d_chol = nullptr, *d_ref = nullptr, *d_tc = nullptr;
+  SpLayer* d_layers = nullptr; TileRef *d_gram = nullptr, *d_pairs = nullptr, *d_bp = nullptr, *d_chol = nullptr, *d_ref = nullptr, *d_tc = nullptr, *d_i8_prep = nullptr, *d_i8 = nullptr;
   uint8_t* d_maps = nullptr;
   uint32_t* d_flag = nullptr;
   ClusterCta* d_ctas = nullptr;
@@ -729,6 +758,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     d_chol = T.take<TileRef>(chol_ctas.size());
     d_ref = T.take<TileRef>(refine_tiles.size());
     d_tc = T.take<TileRef>(tc_tiles.size());
+    d_i8_prep = T.take<TileRef>(i8_prep.size());
+    d_i8 = T.take<TileRef>(i8_tiles.size());
     d_maps = T.take<uint8_t>(maps_blob.size());
     d_ctas = T.take<ClusterCta>(ctas.size());
     d_big = T.take<int>(big_layers.size());
@@ -765,10 +796,12 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.scale = A.take<float>(1);
       {
         const int tt = (d.r + sp_tc_tile() - 1) / sp_tc_tile();
-        d.gram_part = A.take<float>(d.tc && d.gram_split > 1
+        d.gram_part = A.take<float>(d.tc == 1 && d.gram_split > 1
                                         ? (size_t)tt * (tt + 1) / 2 * d.gram_split * sp_tc_tile() * sp_tc_tile() : 0);
       }
-      d.gram_sums = A.take<double>(d.tc ? 0 : (size_t)sp_gram_sums(d.r, d.gram_split));
+      d.gram_sums = A.take<double>(d.tc == 1 ? 0 : d.tc == 2 ? (size_t)sp_i8_sums(d.r, d.gram_split) : (size_t)sp_gram_sums(d.r, d.gram_split));
+      d.i8_ld = sp_i8_pitch(d.L);
+      d.i8_dig = A.take<int8_t>(d.tc == 2 ? (size_t)4 * d.r * d.i8_ld : 0);
       d.td_d = A.take<double>(d.tri ? d.rp : 0); d.td_e = A.take<double>(d.tri ? d.rp : 0);
       d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
@@ -803,6 +836,10 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       const int tf = (L[l].r + 63) / 64;
       L[l].gram_ticket = A.take<uint32_t>(L[l].gram_split > 1 ? (size_t)(L[l].tc ? tt * (tt + 1) / 2 : tf * (tf + 1) / 2) : 0);
     }
+    for (int l = 0; l < n_layers; ++l) {
+      L[l].i8_max = A.take<uint32_t>(L[l].tc == 2 ? (size_t)L[l].r : 0);
+      L[l].i8_rest = A.take<unsigned long long>(L[l].tc == 2 ? (size_t)L[l].r : 0);
+    }
     for (int l = 0; l < n_layers; ++l) L[l].X = A.take<float>(L[l].tri ? 0 : (size_t)L[l].rp * L[l].ldx);
     zero_beg = zb; zero_bytes = A.off - z0;
     for (int l = 0; l < n_layers; ++l) {
@@ -829,6 +866,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     }
     put(d_hdr_tmpl, tmpl.data(), tmpl.size() * sizeof(atomo_layer_header));
   }
+  for (int l : i8_layers)
+    if (sp_i8_make_map(maps_blob.data() + (size_t)l * map_bytes, L[l].i8_dig, L[l].r, L[l].L, L[l].i8_ld) != 0) return ATOMO_ERR_INVALID_ARG;
   put(d_layers, L.data(), L.size() * sizeof(SpLayer));
   put(d_gram, gram_tiles.data(), gram_tiles.size() * sizeof(TileRef));
   put(d_pairs, block_pairs.data(), block_pairs.size() * sizeof(TileRef));
@@ -836,6 +875,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   put(d_chol, chol_ctas.data(), chol_ctas.size() * sizeof(TileRef));
   put(d_ref, refine_tiles.data(), refine_tiles.size() * sizeof(TileRef));
   put(d_tc, tc_tiles.data(), tc_tiles.size() * sizeof(TileRef));
+  put(d_i8_prep, i8_prep.data(), i8_prep.size() * sizeof(TileRef));
+  put(d_i8, i8_tiles.data(), i8_tiles.size() * sizeof(TileRef));
   put(d_maps, maps_blob.data(), maps_blob.size());
   put(d_ctas, ctas.data(), ctas.size() * sizeof(ClusterCta));
   put(d_big, big_layers.data(), big_layers.size() * sizeof(int));
@@ -858,6 +899,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if (ctx->eig_mode == 0) launch_sp_init(d_layers, n_layers, nullptr, 0, st);   // the identity half of [A | I]
   launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), (int)gram_parts.size(), st);
   launch_sp_gram_tc(d_layers, d_maps, d_tc, (int)tc_tiles.size(), d_flag + 1, st);
+  launch_sp_gram_i8(d_layers, d_maps, d_i8_prep, (int)i8_rows.size(), (int)i8_prep.size(), d_i8, (int)i8_tiles.size(), d_flag + 1, st);
   launch_sp_scale(d_layers, n_layers, r_max, st);
   }
   if (!given && ctx->eig_mode != 0 && !tri_form) {

@@ -93,12 +93,15 @@ struct SpLayer {
   float* scale;                // 1 float: power-of-two scaling applied to A
   float* chol_dd;              // 32 x 32 + 32 floats: diagonal block of the current Cholesky panel, published by its owner
   float* dbg_short;            // r x r or nullptr
-  int tc;                      // Gram matrix came from the tensor-core kernel (see sp_scale_kernel)
+  int tc;                      // kernel of the Gram matrix: 0 FMA, 1 TF32 on tensor cores, 2 8-bit integers on tensor cores
   int gram_split;              // Gram matrix: CTAs per output tile (parts of the K range), 1 = no split
   float* gram_part;            // [tiles][gram_split][128 x 128] partial tiles (column-major) when gram_split > 1
   int gram_part_len;           // FMA kernel: length of a part of the K range
-  double* gram_sums;           // FMA kernel: [tiles][gram_split][16][threads that hold entries] partial tiles
+  double* gram_sums;           // FMA kernel: [tiles][gram_split][16][threads that hold entries] partial tiles; integer kernel: [tiles][gram_split][128 x 128]
   uint32_t* gram_ticket;       // [tiles] parts finished; zeroed per call
+  int8_t* i8_dig; int64_t i8_ld;   // integer kernel: [4][r][i8_ld] digits of the short-side vectors
+  uint32_t* i8_max;            // r: bits of the vectors' largest magnitudes; zeroed per call
+  unsigned long long* i8_rest; // r: what the digit pairs taken lack of the vectors' squares; zeroed per call
   int refine, refine_tiles;    // singular values from the projection norms; tiles along the long side
   float* row_inv;              // rp: 1 / norm of each short-side vector as stored in X
   float* refine_partials;      // [refine_tiles][rp] partial squared norms
@@ -205,6 +208,18 @@ int sp_tc_map_bytes();
 int sp_tc_tile();
 void launch_sp_gram_tc(const SpLayer* d_layers, const void* d_maps, const TileRef* d_tiles, int n_tiles, uint32_t* d_err,
                        cudaStream_t st);
+// integer Gram kernel (atomo_i8.cu)
+int sp_i8_configure();                                           // 0 if the kernel got its shared memory
+int64_t sp_i8_pitch(int len);                                    // bytes per vector and digit
+int sp_i8_stages(int len);
+int sp_i8_min_split(int len);                                    // fewest parts of the K range
+int64_t sp_i8_sums(int r, int split);                            // doubles for partial tiles
+bool sp_i8_by_rows(int len, bool tall);                           // digits in one pass over G
+void sp_i8_prep_tiles(int r, int len, bool tall, int* short_tiles, int* long_tiles);
+int sp_i8_make_map(void* out_map, const int8_t* digits, int r, int len, int64_t pitch);   // 0 on success
+// d_prep: n_prep tiles, the first n_rows of them of layers by rows
+void launch_sp_gram_i8(const SpLayer* d_layers, const void* d_maps, const TileRef* d_prep, int n_rows, int n_prep, const TileRef* d_tiles, int n_tiles,
+                       uint32_t* d_err, cudaStream_t st);
 int sp_bp_rows_per_tile();
 int sp_bp_cols_per_tile();
 int sp_bp_chunk_rows();

@@ -19,9 +19,8 @@
 //   warps 6-9   drain: TMEM -> registers, running sums in registers, at the end registers -> global
 // Every mbarrier wait is bounded; a wait that runs out sets an error word and the CTA leaves through
 // the common exit (TMEM is freed).
-#include <cuda.h>
-
 #include "atomo_kernels.cuh"
+#include "atomo_umma.cuh"
 
 namespace atomo {
 
@@ -33,31 +32,6 @@ constexpr int kTcStageBytes = 4 * kTcTileBytes;       // a_hi, a_lo, b_hi, b_lo
 constexpr int kTcThreads = 320;                    // TMA warp, MMA warp, 4 split warps, 4 drain warps
 constexpr int kTcSmemBytes = kTcStages * kTcStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr uint32_t kTcTmemCols = 256;               // two 128-column fp32 accumulators
-constexpr int kTcSpin = 1 << 20;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void tc_mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void tc_mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// bounded wait for the phase with the given parity; also gives up when another role has set the abort word (null: no other role)
-__device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_word) {
-  for (int it = 0; it < kTcSpin; ++it) {
-    uint32_t ok;
-    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if (abort_word != nullptr && (it & 63) == 63 && *abort_word) return false;
-  }
-  if (abort_word != nullptr) *abort_word = 1u;
-  return false;
-}
 __device__ __forceinline__ void tc_tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
@@ -80,10 +54,6 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t da, uint64_t db
 __device__ __forceinline__ float tf32_round(float x) {
   return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
 __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer* __restrict__ layers,
                                                                    const CUtensorMap* __restrict__ maps,
                                                                    const TileRef* __restrict__ tiles,
@@ -294,10 +264,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sp_gram_tc_kernel(const SpLayer
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static EncodeTiledFn g_encode_tiled = nullptr;
+EncodeTiledFn g_encode_tiled = nullptr;
 
 int sp_tc_configure() {
   if (g_encode_tiled == nullptr) {
@@ -308,6 +275,7 @@ int sp_tc_configure() {
     if (qres != cudaDriverEntryPointSuccess || fn == nullptr) return (int)cudaErrorNotSupported;
     g_encode_tiled = reinterpret_cast<EncodeTiledFn>(fn);
   }
+  if (sp_i8_configure() != 0) return (int)cudaErrorNotSupported;
   return (int)cudaFuncSetAttribute(sp_gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
 }
 
