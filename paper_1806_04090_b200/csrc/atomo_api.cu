@@ -812,8 +812,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.bd_UW = A.take<float>(on * rows * 2 * kBandWidth);
         d.bd_X = A.take<float>(on * rows * kBandWidth);
         d.bd_part = A.take<double>(on * sp_band_parts(band_form) * rows * kBandWidth);
-        d.bd_S = A.take<double>(on * 3 * kBandWidth * kBandWidth);
-        d.bd_G = A.take<double>(on * rows / 32 * 36); d.bd_M = A.take<double>(on * rows / 32 * 36);
+        d.bd_S = A.take<double>(on * 3 * 128);
+        d.bd_G = A.take<double>(on * rows / 32 * 36);
         d.bd_band = A.take<double>(on * d.r * (kBandWidth + 1));
         d.bd_T = A.take<double>(on * sp_band_steps(d.r) * kBandWidth * kBandWidth);
         d.bd_V2 = A.take<double>(on * d.r * sp_chase_row(d.r));

@@ -43,9 +43,14 @@ static_assert(kBw == 8, "the operand vectors are two float4");
 // U and W).  Twelve warps per SM: with sixteen the 128 registers do not hold a task.
 // (The sixteen products that update an entry are summed before they are added to it: added one by one they rounded the matrix
 // sixteen times per panel, and the singular values of 2000 x 2048 noise were off by 1.6e-7 instead of 5.4e-8.)
-// Bound: latency of the walk with few layers (a group of four columns takes a lone warp about 1000 cycles, its 200
-// multiply-adds alone would take 200), and the chain of a panel's small steps (Gram sums, 8 x 8 factorisation, U, T: 25 k
-// cycles).  Two layers of 4096 rows: 106 (one-stage reduction) -> 49.7 -> 25.9 ms; 96 of 1024: 29.4 -> 13.2 ms.
+// Bound: latency of the walk (with few layers 14 k cycles of a panel's 40 k at 1023 rows, 68 k of 100 k with two layers of 4096; a group
+// of four columns takes a lone warp about 1000 cycles, its 200 multiply-adds alone would take 200), and the chain of a panel's small
+// steps: own rows and first barrier 8 k, sums of the Gram matrix 2 k, 8 x 8 factorisation 3.5 k, U 2 .. 7 k (conversions), second
+// barrier 4 k, T and what follows from it 3.5 k.  Two layers of 4096 rows: 106 (one-stage reduction) -> 49.7 -> 25.8 -> 23.4 ms; 96 of
+// 1024: 29.4 -> 13.0 -> 12.7; one of 1023: 2.03 -> 1.71.  The last step is the chain's: with few layers the own rows are shared by all warps
+// of a CTA, eight lanes to a row (one warp took 8 k cycles), U^T U is added up like U^T A U instead of by every CTA, T is solved for
+// by columns in registers, a column per lane in the factorisation (6.1 k), barriers by release and acquire instead of fences.  Tried and
+// dropped: 32 or 64 tasks per strip (two of 4096 rows 26.3 and 32.1 ms, one of 1023 the same and 10 % slower).
 // The panel's QR is a Householder QR worked out on 8 x 8 matrices: the reflectors' norms and products follow from the panel's
 // Gram matrix (downdated as rows of R split off) and its first eight rows, and below those rows V = X K with an 8 x 8 matrix
 // K.  A column whose remainder is below 3e-8 of it is left alone (the fp32 panel has no more digits).  However inexact V is
@@ -71,6 +76,7 @@ struct BandShared {
   double K[8][8], vtop[8][8];     // K scaled to unit vectors; the reflectors' entries in the panel's first eight rows
   double M[36], G[36], sum[16][36];
   double s_part[16][64];          // the warps' parts of U^T A U
+  double m_part[16][40];          // ... and of U^T U
   double top[8][8];
   double Wc[8][8], Uc[8][8], Pc[8][8];   // W, U and A U of the next panel's pivot rows
   uint32_t fail;
@@ -89,25 +95,35 @@ __device__ __forceinline__ double band_scatter8(const double (&v)[8], int lane) 
   c += __shfl_xor_sync(0xffffffffu, c, 1);
   return c;
 }
-// the 36 dots of the columns of a 32 x 8 block, one row (a, b) per lane, to dst (lower triangle by rows).  (Out of line, as the
-// 8 x 8 factorisation below: a panel is a walk through the whole kernel, and what runs once per panel should stay small.)
-__device__ __noinline__ void band_gram32(const float4 a, const float4 b, double* __restrict__ dst, int lane) {
+// eight of the 36 dots (lower triangle by rows, number 8 BLK and on) of the columns of a 32 x 8 block, one row (a, b) per lane: the
+// lane ends with dot 8 BLK + lane / 4
+template <int BLK>
+__device__ __forceinline__ double band_dots(const float4 a, const float4 b, int lane) {
   const double d[8] = {(double)a.x, (double)a.y, (double)a.z, (double)a.w, (double)b.x, (double)b.y, (double)b.z, (double)b.w};
-  double acc[40];
+  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int e = 0;
 #pragma unroll
   for (int p = 0; p < 8; ++p)
 #pragma unroll
-    for (int q = 0; q <= p; ++q, ++e) acc[e] = d[p] * d[q];
+    for (int q = 0; q <= p; ++q, ++e) if (e / 8 == BLK) v[e % 8] = d[p] * d[q];
+  return band_scatter8(v, lane);
+}
+// (Out of line, as the 8 x 8 factorisation below: a panel is a walk through the whole kernel, and what runs once per panel should stay small.)
+__device__ __noinline__ double band_dots_of(int blk, const float4 a, const float4 b, int lane) {
+  switch (blk) {
+    case 0: return band_dots<0>(a, b, lane);
+    case 1: return band_dots<1>(a, b, lane);
+    case 2: return band_dots<2>(a, b, lane);
+    case 3: return band_dots<3>(a, b, lane);
+    default: return band_dots<4>(a, b, lane);
+  }
+}
+// all 36 of them by one warp, to dst
+__device__ __noinline__ void band_gram32(const float4 a, const float4 b, double* __restrict__ dst, int lane) {
+  const double x[5] = {band_dots<0>(a, b, lane), band_dots<1>(a, b, lane), band_dots<2>(a, b, lane), band_dots<3>(a, b, lane), band_dots<4>(a, b, lane)};
+  if ((lane & 3) == 0) {
 #pragma unroll
-  for (int q = 36; q < 40; ++q) acc[q] = 0.0;
-#pragma unroll
-  for (int e0 = 0; e0 < 40; e0 += 8) {
-    double v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = acc[e0 + q];
-    const double s = band_scatter8(v, lane);
-    if ((lane & 3) == 0 && e0 + (lane >> 2) < 36) dst[e0 + (lane >> 2)] = s;
+    for (int blk = 0; blk < 5; ++blk) if (blk * 8 + (lane >> 2) < 36) dst[blk * 8 + (lane >> 2)] = x[blk];
   }
 }
 
@@ -116,13 +132,14 @@ __device__ __noinline__ void band_gram32(const float4 a, const float4 b, double*
 __device__ __forceinline__ void band_barrier(uint32_t* ctr, uint32_t target, BandShared& sh, uint32_t* timeout_flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1u);
-    uint32_t polls = 0;
-    while (*(volatile uint32_t*)ctr < target && sh.fail == 0u) {
+    // (release and acquire at device scope; what the block's other threads did is ordered by the block barriers around them)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+    uint32_t polls = 0, seen;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(ctr) : "memory");
+      if (seen >= target || sh.fail != 0u) break;
       if (++polls > kBandPollLimit) { sh.fail = 1u; *timeout_flag = 1u; }
     }
-    __threadfence();
   }
   __syncwarp();                                              // (without it the polling thread's warp may stay divided past the barrier)
   __syncthreads();
@@ -149,56 +166,58 @@ __device__ __forceinline__ void band_sum36(const double* __restrict__ src, int f
   }
 }
 
-// Householder QR of the panel on its Gram matrix (lower triangle in sh.G) and first eight rows (sh.top), one warp.  Lane:
-// column l = lane % 8, rows lane / 8 and lane / 8 + 4.  Leaves R in sh.top, the unit reflectors' entries in the first eight rows
-// in sh.vtop (zero above the diagonal) and K, scaled likewise.
+// Householder QR of the panel on its Gram matrix (lower triangle in sh.G) and first eight rows (sh.top), one warp.  Lane l < 8
+// holds column l of the Gram matrix, of the rows and of K (the other lanes do the same on copies), so that what a step needs of
+// its own column is in registers and the pivot column's entries arrive while the norm's roots are taken.  Leaves R in sh.top, the unit
+// reflectors' entries in the first eight rows in sh.vtop (zero above the diagonal) and K, scaled likewise.
 __device__ __noinline__ void band_small_qr(BandShared& sh, const int n_ref, const int lane) {
   __syncwarp();
-  const int l = lane & 7, i0 = lane >> 3;
-  double top[2], g[2], k[2];
+  const int l = lane & 7;
+  double top[8], g[8], k[8];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int i = i0 + 4 * h;
-    top[h] = sh.top[i][l];
-    g[h] = sh.G[i >= l ? i * (i + 1) / 2 + l : l * (l + 1) / 2 + i];
-    k[h] = i == l ? 1.0 : 0.0;
+  for (int i = 0; i < 8; ++i) {
+    top[i] = sh.top[i][l];
+    g[i] = sh.G[i >= l ? i * (i + 1) / 2 + l : l * (l + 1) / 2 + i];
+    k[i] = i == l ? 1.0 : 0.0;
   }
   const double orig = sh.G[l * (l + 1) / 2 + l];             // squared norm of column l as given
-#pragma unroll 1
+#pragma unroll
   for (int t = 0; t < 8; ++t) {
-    const bool up = t >= 4;                                  // row t: register up of the lanes tl ..
-    const int tl = (t & 3) * 8;
-    const double g_of = up ? g[1] : g[0], top_of = up ? top[1] : top[0];
-    const double gt = __shfl_sync(0xffffffffu, g_of, tl + l), tt = __shfl_sync(0xffffffffu, top_of, tl + l);
-    const double nx2 = __shfl_sync(0xffffffffu, gt, t), x0 = __shfl_sync(0xffffffffu, tt, t), o = __shfl_sync(0xffffffffu, orig, t);
+    const double nx2 = __shfl_sync(0xffffffffu, g[t], t), x0 = __shfl_sync(0xffffffffu, top[t], t), o = __shfl_sync(0xffffffffu, orig, t);
+    double x[8], kt[8];                                      // the pivot column's entries below the diagonal, its column of K
+#pragma unroll
+    for (int i = t + 1; i < 8; ++i) x[i] = __shfl_sync(0xffffffffu, top[i], t);
+#pragma unroll
+    for (int i = 0; i <= t; ++i) kt[i] = __shfl_sync(0xffffffffu, k[i], t);
     double alpha = x0, beta = 0.0, un = 0.0;
     const bool act = t < n_ref && nx2 > 1.0e-290 && nx2 > 1.0e-15 * o;   // else H = I: a zero column, or no digits left
     if (act) {
       const double nx = nx2 * rsqrt(nx2);
       alpha = -copysign(nx, x0);
-      const double half = fma(fabs(x0), nx, nx2);            // v^T v / 2
-      un = rsqrt(2.0 * half);
+      un = rsqrt(2.0 * fma(fabs(x0), nx, nx2));              // 1 / ||v||
       beta = 2.0 * un * un;
     }
-    const double gl = l > t ? beta * (gt - alpha * tt) : 0.0;   // beta v^T x_l
+    x[t] = x0 - alpha;
+    const double gl = l > t ? beta * (g[t] - alpha * top[t]) : 0.0;   // beta v^T x_l
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = i0 + 4 * h;
-      const double xi = __shfl_sync(0xffffffffu, top[h], (lane & 24) + t), ki = __shfl_sync(0xffffffffu, k[h], (lane & 24) + t);
-      const double v = i > t ? xi : i == t ? x0 - alpha : 0.0;
-      if (l > t) { top[h] = fma(-gl, v, top[h]); k[h] = fma(-gl, ki, k[h]); }
-      if (l == t) {
-        sh.vtop[i][t] = v * un;
-        sh.K[i][t] = ki * un;
-        if (act) top[h] = i == t ? alpha : i > t ? 0.0 : top[h];
+    for (int i = t; i < 8; ++i) top[i] = fma(-gl, x[i], top[i]);
+#pragma unroll
+    for (int i = 0; i <= t; ++i) k[i] = fma(-gl, kt[i], k[i]);
+    if (lane == t) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        sh.vtop[i][t] = i < t ? 0.0 : x[i] * un;
+        sh.K[i][t] = i <= t ? kt[i] * un : 0.0;
+        if (act && i >= t) top[i] = i == t ? alpha : 0.0;
       }
     }
-    const double r_of = up ? top[1] : top[0], rl = __shfl_sync(0xffffffffu, r_of, tl + l);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) g[h] = fma(-__shfl_sync(0xffffffffu, r_of, tl + i0 + 4 * h), rl, g[h]);   // row t of R leaves the Gram matrix
+    for (int i = t + 1; i < 8; ++i) g[i] = fma(-__shfl_sync(0xffffffffu, top[t], i), top[t], g[i]);   // row t of R leaves the Gram matrix
   }
+  if (lane < 8) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) sh.top[i0 + 4 * h][l] = top[h];
+    for (int i = 0; i < 8; ++i) sh.top[i][l] = top[i];
+  }
 }
 
 }  // namespace
@@ -208,6 +227,7 @@ template <int THREADS, int MINB, int PARTS, int STAGES>
 __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* __restrict__ layers, const ClusterCta* __restrict__ ctas,
                                                                 uint32_t* __restrict__ timeout_flag) {
   constexpr int kWarps = THREADS / 32;
+  constexpr bool kSpread = PARTS >= 16;                      // few layers: a CTA has one or two half strips of its own
   extern __shared__ __align__(16) float band_smem[];
   __shared__ BandShared sh;
   const ClusterCta me = ctas[blockIdx.x];
@@ -218,7 +238,7 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   float* const A = L.A; const int64_t lda = L.lda; const int ld32 = (int)lda;           // lda is a multiple of the strip: whole strips may be read and written
   float* const gUW = L.bd_UW; float* const gX = L.bd_X;
   double* const gPart = L.bd_part; double* const gS = L.bd_S; double* const gB = L.bd_band;
-  double* const gG = L.bd_G; double* const gM = L.bd_M;
+  double* const gG = L.bd_G;
   float* const gV = L.td_V; const int64_t ldv = L.td_ldv;
   double* const gT = L.bd_T;
   float* const s_u = band_smem;                              // [r][8] this panel's U, by row
@@ -229,7 +249,55 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
   auto own_from = [&](int row) { const int h = row / 32; return h + ((g - h % G) % G + G) % G; };   // this CTA's first half strip, then every G-th
   for (int c = 0; c < r; c += kBw) {
     // ---- own rows: U and W of the panel before out, entries of this panel (columns c .. c+7) and the Gram matrix of those
-    // below the band; half a strip per warp ----
+    // below the band ----
+    if constexpr (kSpread) {                                 // eight lanes per row, all warps on the CTA's few half strips
+      const int h0 = own_from(c), n_own = h0 < 2 * n_strips ? (2 * n_strips - 1 - h0) / G + 1 : 0;
+      float* const s_x = s_ring;                             // [half strips of a round][32][8], the panel's entries (the ring is idle)
+      constexpr int kRound = kWarps * STAGES * kGroupFloats / 256;
+      for (int n0 = 0; n0 < n_own; n0 += kRound) {
+        const int n_now = min(kRound, n_own - n0);
+        for (int q = w; q < 8 * n_now; q += kWarps) {        // four rows
+          const int t = lane & 7, i = (h0 + (n0 + q / 8) * G) * 32 + q % 8 * 4 + (lane >> 3);
+          const bool in = i >= c && i < r;
+          float x = in && c + t < r ? __ldcg(A + (int64_t)(c + t) * lda + i) : 0.0f;
+          if (c > 0) {
+            double part[PARTS];
+#pragma unroll
+            for (int z = 0; z < PARTS; ++z) part[z] = in ? __ldcg(gPart + ((int64_t)z * n_strips * kStrip + i) * 8 + t) : 0.0;
+            double p = 0.0, z = 0.0;                         // the product A U: the parts added in order
+#pragma unroll
+            for (int q2 = 0; q2 < PARTS; ++q2) p += part[q2];
+            const float4* const us = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : r) * 8);   // (zeros past the end)
+            const float4 ua = us[0], ub = us[1];
+            const float uu[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
+            // W[i][t] = sum_s P[i][s] T[s][t] - 1/2 sum_s U[i][s] (T^T S T)[s][t]
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+              const double ps = __shfl_sync(0xffffffffu, p, (lane & 24) + s);
+              if (s <= t) z = fma(ps, sh.T[s][t], z);
+              z = fma((double)uu[s], sh.X[s][t], z);
+            }
+            const float ww = (float)z;
+            z = (double)x;
+#pragma unroll
+            for (int s = 0; s < 8; ++s) z -= fma((double)uu[s], sh.Wc[t][s], (double)__shfl_sync(0xffffffffu, ww, (lane & 24) + s) * sh.Uc[t][s]);
+            x = in && c + t < r ? (float)z : 0.0f;
+            gUW[(int64_t)i * 16 + t] = in ? s_u[(size_t)i * 8 + t] : 0.0f;
+            gUW[(int64_t)i * 16 + 8 + t] = ww;
+          }
+          gX[(int64_t)i * 8 + t] = x;
+          s_x[q * 32 + lane] = i < c + kBw ? 0.0f : x;
+        }
+        __syncthreads();
+        for (int q = w; q < 5 * n_now; q += kWarps) {        // eight of a half strip's dots
+          const float4* const src = reinterpret_cast<const float4*>(s_x + (q / 5) * 256 + lane * 8);
+          const double x = band_dots_of(q % 5, src[0], src[1], lane);
+          const int e = q % 5 * 8 + (lane >> 2);
+          if ((lane & 3) == 0 && e < 36) gG[(int64_t)(h0 + (n0 + q / 5) * G) * 36 + e] = x;
+        }
+        if (n0 + kRound < n_own) __syncthreads();
+      }
+    } else                                                   // half a strip per warp
     {
       for (int half = own_from(c) + w * G; half < 2 * n_strips; half += kWarps * G) {
         const int i = half * 32 + lane;
@@ -280,10 +348,10 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         band_gram32(lo, hi, gG + (int64_t)half * 36, lane);
       }
     }
-    // U^T A U is added up in one of three sets of 64 words in turn; the next panel's is cleared here: its last readers are
+    // U^T A U and U^T U are added up in one of three sets of 128 words in turn; the next panel's is cleared here: its last readers are
     // past the barrier before this one, its adders wait for the one after it
-    double* const s_sum = gS + c / kBw % 3 * 64;
-    if (g == 0 && tid < 64) { gS[(c / kBw + 1) % 3 * 64 + tid] = 0.0; if (c == 0) s_sum[tid] = 0.0; }
+    double* const s_sum = gS + c / kBw % 3 * 128;
+    if (g == 0 && tid < 128) { gS[(c / kBw + 1) % 3 * 128 + tid] = 0.0; if (c == 0) s_sum[tid] = 0.0; }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
     if (sh.fail) break;
@@ -334,6 +402,8 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
     const int per = ((m + PARTS - 1) / PARTS + 3) & ~3;      // columns per task, a multiple of the group
     __syncthreads();
     sh.s_part[w][lane] = sh.s_part[w][lane + 32] = 0.0;
+    sh.m_part[w][lane] = 0.0;
+    if (lane < 8) sh.m_part[w][lane + 32] = 0.0;
     __syncwarp();
     // tasks (strip, part), dealt to the warps of all CTAs
     for (int task = g + w * G; task < (n_strips - first_strip) * PARTS; task += kWarps * G) {
@@ -461,30 +531,37 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
         if ((lane & 3) == 0) sh.s_part[w][a * 8 + (lane >> 2)] += sum;
       }
     }
-    for (int half = own_from(row0) + w * G; half < 2 * n_strips; half += kWarps * G) {   // U^T U of the own half strips
+    constexpr int kPieces = kSpread ? 5 : 1;                 // U^T U of the own half strips, eight dots at a time or all 36
+    for (int q = w; ; q += kWarps) {
+      const int half = own_from(row0) + q / kPieces * G;
+      if (half >= 2 * n_strips) break;
       const int i = half * 32 + lane;
       const bool in = i >= row0 && i < r;
-      const float4* src = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : row0) * 8);
-      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-      band_gram32(in ? src[0] : zero, in ? src[1] : zero, gM + (int64_t)half * 36, lane);
+      const float4* src = reinterpret_cast<const float4*>(s_u + (size_t)(in ? i : r) * 8);
+      if (kSpread) {                                         // (in multiples of 2^-50 again)
+        const double x = band_dots_of(q % 5, src[0], src[1], lane);
+        if ((lane & 3) == 0) sh.m_part[w][q % 5 * 8 + (lane >> 2)] += (x + kFix) - kFix;
+      } else {
+        band_gram32(src[0], src[1], sh.sum[w], lane);
+        __syncwarp();
+        for (int e = lane; e < 36; e += 32) sh.m_part[w][e] += (sh.sum[w][e] + kFix) - kFix;
+        __syncwarp();
+      }
     }
     __syncthreads();
-    if (tid < 64) {
+    if (tid < 100) {
       double t = 0.0;
 #pragma unroll
-      for (int ww = 0; ww < kWarps; ++ww) t += sh.s_part[ww][tid];
+      for (int ww = 0; ww < kWarps; ++ww) t += tid < 64 ? sh.s_part[ww][tid] : sh.m_part[ww][tid - 64];
       atomicAdd(s_sum + tid, t);
     }
     arrivals += (uint32_t)G;
     band_barrier(L.bd_bar, arrivals, sh, timeout_flag);
-    // ---- T, T^T S T, W of the next panel's pivot rows (every CTA) ----
-    if (tid >= THREADS - 64) {
-      const int q = tid - (THREADS - 64);
-      sh.S[q / 8][q % 8] = __ldcg(s_sum + q);
-    }
-    band_sum36<THREADS>(gM, row0 / 32, 2 * n_strips, sh.sum, sh.M);
-    if (tid >= THREADS - 128 && tid < THREADS - 64) {         // the product's next pivot rows
-      const int q = tid - (THREADS - 128), i = row0 + q / 8;
+    // ---- T, T^T S T, W of the next panel's pivot rows (every CTA, one warp) ----
+    if (tid < 64) sh.S[tid / 8][tid % 8] = __ldcg(s_sum + tid);
+    else if (tid < 100) sh.M[tid - 64] = __ldcg(s_sum + tid);
+    else if (tid >= THREADS - 64) {                          // the product's next pivot rows
+      const int q = tid - (THREADS - 64), i = row0 + q / 8;
       double p = 0.0;
       if (i < r) {
         const double* src = gPart + (int64_t)i * 8 + q % 8;
@@ -495,45 +572,51 @@ __global__ void __launch_bounds__(THREADS, MINB) sp_band_kernel(const SpLayer* _
     }
     __syncthreads();
     if (w == 0) {
-      // T: tau_t in place t, -tau_t T[0:t, 0:t] M[0:t, t] above (lane: row)
-#pragma unroll 1
-      for (int t = 0; t < 8; ++t) {
-        const double* mt = sh.M + t * (t + 1) / 2;
-        const double tau = mt[t] > 0.5 ? 2.0 / mt[t] : 0.0;
-        double z0 = 0.0, z1 = 0.0;                           // (T is zero below its diagonal)
+      // T is the inverse of the upper triangle of U^T U with half its diagonal: lane t solves for column t from the diagonal up
+      if (lane < 8) {
+        double col[8];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) if (q < t && lane < 8) { if (q & 1) z1 = fma(sh.T[lane][q], mt[q], z1); else z0 = fma(sh.T[lane][q], mt[q], z0); }
-        if (lane < 8) sh.T[lane][t] = lane < t ? -tau * (z0 + z1) : lane == t ? tau : 0.0;
-        __syncwarp();
+        for (int q = 7; q >= 0; --q) {
+          double z = 0.0;
+#pragma unroll
+          for (int x = 7; x > q; --x) z = fma(sh.M[x * (x + 1) / 2 + q], col[x], z);
+          const double d = sh.M[q * (q + 1) / 2 + q], tau = d > 0.5 ? 2.0 / d : 0.0;
+          col[q] = q > lane ? 0.0 : q == lane ? tau : -tau * z;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sh.T[q][lane] = col[q];
       }
-    }
-    __syncthreads();
-    if (tid < 64) {
-      const int a = tid / 8, b = tid % 8;
-      double t = 0.0;
+      __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 8; ++q) t = fma(sh.S[a][q], sh.T[q][b], t);
-      sh.Y[a][b] = t;
-      if (g == 0) gT[(int64_t)(c / kBw) * 64 + tid] = sh.T[a][b];   // for the back-transformation, as the reflectors' rows below
-    }
-    __syncthreads();
-    if (tid < 64) {                                          // X = -1/2 T^T S T
-      const int a = tid / 8, b = tid % 8;
-      double t = 0.0;
+      for (int h = 0; h < 2; ++h) {
+        const int a = lane / 8 + 4 * h, b = lane % 8;
+        double t = 0.0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) t = fma(sh.T[q][a], sh.Y[q][b], t);
-      sh.X[a][b] = -0.5 * t;
-    }
-    __syncthreads();
-    if (tid < 64) {
-      const int a = tid / 8, t = tid % 8, i = row0 + a;
-      double z = 0.0;
-      if (i < r) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { z = fma(sh.Pc[a][q], sh.T[q][t], z); z = fma((double)s_u[(size_t)i * 8 + q], sh.X[q][t], z); }
+        for (int q = 0; q < 8; ++q) t = fma(sh.S[a][q], sh.T[q][b], t);
+        sh.Y[a][b] = t;
+        if (g == 0) gT[(int64_t)(c / kBw) * 64 + a * 8 + b] = sh.T[a][b];   // for the back-transformation, as the reflectors' rows below
       }
-      sh.Wc[a][t] = (double)(float)z;
-      sh.Uc[a][t] = i < r ? (double)s_u[(size_t)i * 8 + t] : 0.0;
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {                          // X = -1/2 T^T S T
+        const int a = lane / 8 + 4 * h, b = lane % 8;
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t = fma(sh.T[q][a], sh.Y[q][b], t);
+        sh.X[a][b] = -0.5 * t;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int a = lane / 8 + 4 * h, t = lane % 8, i = row0 + a;
+        double z = 0.0;
+        if (i < r) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) { z = fma(sh.Pc[a][q], sh.T[q][t], z); z = fma((double)s_u[(size_t)i * 8 + q], sh.X[q][t], z); }
+        }
+        sh.Wc[a][t] = (double)(float)z;
+        sh.Uc[a][t] = i < r ? (double)s_u[(size_t)i * 8 + t] : 0.0;
+      }
     }
     __syncthreads();
     // the reflectors' rows for the back-transformation (zero above row0 + t)

@@ -116,8 +116,8 @@ struct SpLayer {
   float* bd_UW;                // [rows padded to strips][16] U and W of the panel before
   float* bd_X;                 // [rows padded to strips][8] entries of the next panel
   double* bd_part;             // [parts][rows padded to strips][8] partial products
-  double* bd_S;                // [3][64] U^T A U of three panels in turn
-  double* bd_G; double* bd_M;  // [half strips][36] dots of the next panel's columns, of U's
+  double* bd_S;                // [3][128] U^T A U and U^T U of three panels in turn
+  double* bd_G;                // [half strips][36] dots of the next panel's columns
   double* bd_band;             // [r][9] the band, by column
   double* bd_T;                // [panels][64] T of the panels: Q1 is the product of I - U T U^T
   double* bd_V2;               // [r][sp_chase_row] reflectors of the chase, by sweep
