@@ -17,6 +17,7 @@
 //                                memory of one wave of resident CTAs
 //   ew_decode                  : a tile is put together in shared memory and leaves as one bulk copy, either format
 #include <algorithm>
+#include <type_traits>
 
 #include "atomo_kernels.cuh"
 
@@ -1071,7 +1072,8 @@ __global__ void __launch_bounds__(kEwDecThreads) ew_decode_kernel(const __grid_c
 // between barriers) and leaves once; explicit and compact payloads may be mixed.  Bound: HBM writes.  The payloads'
 // headers and table entries are fetched by one thread each, then the entries of all of them, as one sequence of up to
 // 2048 at a time, before the first is added: the chain of dependent loads is paid once per tile instead of once per
-// payload (88 us for eight payloads of 25.6 M elements at 1 % with a payload at a time).
+// payload (88 us for eight payloads of 25.6 M elements at 1 % with a payload at a time).  A window is instantiated for one, two, four or
+// eight entries per thread: with eight always, of which two were in use at 1 %, most instructions did nothing (73.6 -> 61.4 us).
 constexpr int kAvgThreads = 256, kAvgPer = 8, kAvgPayloads = 64;     // payloads per round: their ranges sit in shared memory
 struct AvgSource { const void* idx; const float* val; const uint32_t* sat_idx; uint32_t lo, sat_begin, n_sat, compact; float c; };
 template <int N>
@@ -1118,12 +1120,14 @@ __global__ void __launch_bounds__(kAvgThreads) ew_decode_average_kernel(const __
         if (off >= 0) s_tile[off] += __ldg(s.val + q);
       }
     };
-    for (uint32_t e0 = 0; e0 < total; e0 += kAvgThreads * kAvgPer) {
+    // a window of kPer entries per thread
+    auto window = [&](const uint32_t e0, auto per_tag) {
+      constexpr int kPer = decltype(per_tag)::value;
       // this thread's entries of the window: element, value, payload
-      uint32_t el[kAvgPer]; float vl[kAvgPer]; int pl[kAvgPer];
+      uint32_t el[kPer]; float vl[kPer]; int pl[kPer];
       int p = 0;
 #pragma unroll
-      for (int q = 0; q < kAvgPer; ++q) {
+      for (int q = 0; q < kPer; ++q) {
         const uint32_t e = e0 + (uint32_t)(q * kAvgThreads) + tid;
         el[q] = kEwTile; vl[q] = 0.0f; pl[q] = np;
         if (e < total) {
@@ -1141,13 +1145,20 @@ __global__ void __launch_bounds__(kAvgThreads) ew_decode_average_kernel(const __
           }
         }
       }
-      const uint32_t e_end = min(e0 + (uint32_t)(kAvgThreads * kAvgPer), total);
+      const uint32_t e_end = min(e0 + (uint32_t)(kAvgThreads * kPer), total);
       for (int pp = p_next; pp < np && s_begin[pp] < e_end; ++pp) {     // payload by payload, in array order
 #pragma unroll
-        for (int q = 0; q < kAvgPer; ++q) if (pl[q] == pp && el[q] < (uint32_t)kEwTile) s_tile[el[q]] += vl[q];
+        for (int q = 0; q < kPer; ++q) if (pl[q] == pp && el[q] < (uint32_t)kEwTile) s_tile[el[q]] += vl[q];
         if (s_begin[pp + 1] <= e_end) { add_saturated(pp); p_next = pp + 1; }
         __syncthreads();
       }
+    };
+    for (uint32_t e0 = 0; e0 < total; e0 += kAvgThreads * kAvgPer) {   // (uniform: as many entries per thread as the window has)
+      const uint32_t left_e = total - e0;
+      if (left_e <= kAvgThreads) window(e0, std::integral_constant<int, 1>{});
+      else if (left_e <= 2 * kAvgThreads) window(e0, std::integral_constant<int, 2>{});
+      else if (left_e <= 4 * kAvgThreads) window(e0, std::integral_constant<int, 4>{});
+      else window(e0, std::integral_constant<int, kAvgPer>{});
     }
     for (; p_next < np; ++p_next) if (s_src[p_next].n_sat) { add_saturated(p_next); __syncthreads(); }
   }
