@@ -62,6 +62,8 @@ struct atomo_ctx {
   int refine_min_short = 2048;       // layers with at least this short side get the sigma refinement pass
   bool tc_gram = true;               // Gram matrix on tcgen05 where the layer's layout allows it
   bool tc_ok = false;                // tensor-map entry point found
+  cudaStream_t side = nullptr;       // work beside the call's stream, which forks it and joins it again inside the call
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int eig_scheme = 3;                // eigen-solve: 0 = Jacobi, one launch per step, 1 = persistent (cooperative), 2 = clusters first, 3 = tridiagonal route first
   int tri_clusters = -1;             // co-resident clusters of the tridiagonal reduction (-1 = not asked yet, 0 = unavailable)
   int tri_big_ok = -1;               // two-stage tridiagonal reduction for short sides above 512 (-1 = not asked yet)
@@ -322,6 +324,9 @@ int atomo_create(atomo_ctx** out, int device) {
   if (e == 0) e = ew_configure();
   if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaFuncSetAttribute(max dynamic shared memory)");
   ctx->tc_ok = sp_tc_configure() == 0;
+  CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
+  CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
   ctx->configured = true;
   return ATOMO_OK;
 }
@@ -330,6 +335,9 @@ int atomo_destroy(atomo_ctx* ctx) {
   if (!ctx) return ATOMO_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
+  if (ctx->side) cudaStreamDestroy(ctx->side);
+  if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->ws) cudaFree(ctx->ws);
   if (ctx->ew_words) cudaFree(ctx->ew_words);
   table_free(ctx->tab_sp); table_free(ctx->tab_avg);
@@ -920,7 +928,10 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // layers in one cooperative launch.  A batch larger than the GPU is cut into such groups, launched one after
   // the other; a single layer with more block pairs than the GPU holds CTAs falls back to one launch per step.
   if (tri_form) {
-    if (n_clusters > 0) {
+    // small layers beside larger ones: their reduction (0.5 to 0.7 ms on up to 96 SMs) runs on a stream of the context's own next to the
+    // chase, which leaves most of the GPU idle; the call's stream waits for it before the eigenvalues
+    const bool beside = n_clusters > 0 && any_big;
+    if (n_clusters > 0 && !beside) {
       const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, d_flag + 1, st);
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(tridiagonal reduction)");
       ++n_eig_launch;
@@ -930,15 +941,25 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(band reduction)");
       ++n_eig_launch;
     }
-    for (size_t i = 0, n; i < big_layers.size(); i += n) {           // (sorted: layers of one class are neighbours)
+    if (beside) CK(cudaEventRecord(ctx->ev_fork, st));
+    int chase_err = 0;
+    for (size_t i = 0, n; i < big_layers.size() && chase_err == 0; i += n) {   // (sorted: layers of one class are neighbours)
       const int of = chase_class(L[big_layers[i]].r);
       n = 1;
       while (i + n < big_layers.size() && chase_class(L[big_layers[i + n]].r) == of) ++n;
       const int c = sp_chase_ctas(of, (int)n, of > 1024 ? chase_room(ctx, of / 256) : 0);
-      const int e = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
-      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(bulge chase)");
+      chase_err = launch_sp_chase(d_layers, d_big + i, (int)n, c, st);
       ++n_eig_launch;
     }
+    if (beside) {                                                    // (behind the chase in the order of launches: the longer one first)
+      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+      const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, d_flag + 1, ctx->side);
+      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+      CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
+      if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(tridiagonal reduction)");
+      ++n_eig_launch;
+    }
+    if (chase_err != 0) return fail_cuda(ctx, (cudaError_t)chase_err, "cudaLaunchKernelEx(bulge chase)");
     // the eigenvalues (bisection) are timed with the sampling stage.  No host wait on this route: a bounded wait of
     // the Gram kernel that ran out is reported by the sampling kernel in every layer's status word
     // (ATOMO_ERR_TIMEOUT, nothing kept)
@@ -1010,10 +1031,16 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // ---- S4: long-side vectors of the kept atoms ----
   stage_begin(ctx, ATOMO_STAGE_BACKPROJECT, st);
   if (tri_form) {                                                   // short-side vectors of the kept atoms
-    if (any_small) launch_sp_eigvec(d_layers, n_layers, rp_max_small, st);
+    if (any_small && any_big) {                                     // both kinds side by side, as their reductions
+      CK(cudaEventRecord(ctx->ev_fork, st));
+      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+      launch_sp_eigvec(d_layers, n_layers, rp_max_small, ctx->side);
+      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+    } else if (any_small) launch_sp_eigvec(d_layers, n_layers, rp_max_small, st);
     int rps = 0;
     for (int l : big_layers) rps |= L[l].rp <= 1024 ? 1 : L[l].rp <= 2048 ? 2 : 4;
     launch_sp_eigvec_big(d_layers, d_big, (int)big_layers.size(), rps, st);
+    if (any_small && any_big) CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
   }
   launch_sp_backproject(d_layers, d_bp, (int)bp_tiles.size(), std::max(r_max_tall, 1), st);
   launch_sp_finish_atoms(d_layers, n_layers, k_cap_max, st);

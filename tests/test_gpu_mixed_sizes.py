@@ -1,0 +1,60 @@
+"""Small and large layers in one call run partly side by side: what each yields must not depend on the company, on the stream, or on a
+replay from a graph."""
+import pytest
+import torch
+
+from paper_1806_04090_b200 import api
+
+pytestmark = pytest.mark.gpu
+
+
+def _layers():
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    return [torch.randn(m, n, device="cuda", generator=gen) for m, n in ((40, 90), (300, 500), (512, 700), (1100, 1300), (600, 650))]
+
+
+def _arrays(pay, n):
+    return [{k: v.copy() for k, v in pay.layer_arrays(l).items() if hasattr(v, "copy")} for l in range(n)]
+
+
+def test_small_layers_beside_large_ones():
+    G = _layers()
+    a = api.Atomo(0)
+    alone, _ = a.atomo_encode_spectral(G[:3], 3.0, seed=9, step=2, k_cap=24)
+    want = _arrays(alone, 3)
+    for stream in (torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.Stream()):
+        stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(stream):
+            pay, _ = a.atomo_encode_spectral(G, 3.0, seed=9, step=2, k_cap=24)
+            out = a.atomo_decode(pay)
+        stream.synchronize()
+        assert [h.status for h in pay.headers()[1]] == [0] * 5
+        for x, y in zip(want, _arrays(pay, 3)):
+            assert x.keys() == y.keys()
+            assert all((x[k] == y[k]).all() for k in x)
+        assert all(torch.isfinite(o).all() for o in out)
+    a.close()
+
+
+def test_replay_from_a_graph():
+    G = _layers()
+    a = api.Atomo(0)
+    shapes = [tuple(g.shape) for g in G]
+    buf = torch.zeros(api.payload_bytes_spectral(shapes, 24), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):                    # (the tables are uploaded on the stream that is captured later)
+        a.atomo_encode_spectral(G, 3.0, seed=9, step=2, k_cap=24, payload=buf)
+    torch.cuda.synchronize()
+    want = buf.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        a.atomo_encode_spectral(G, 3.0, seed=9, step=2, k_cap=24, payload=buf)
+    for _ in range(3):
+        buf.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(buf, want)
+    del graph
+    a.close()
