@@ -12,7 +12,7 @@
 //   (sp_finalize_sample_kernel sorts, solves Algorithm 1 and draws, as for the other routes)
 //   sp_eigvec_kernel          : for the kept atoms only: eigenvector of T by a twisted factorisation with one
 //                               Rayleigh-quotient correction, back-transformation u = Q z with the reflectors
-//                               (four at a time, fp32), normalised short-side vector into the payload; kept atoms with
+//                               (eight at a time, fp32), normalised short-side vector into the payload; kept atoms with
 //                               nearly equal eigenvalues are orthogonalised against each other at the end.
 //
 // Work per layer: about 2 r^3 fp64 flops for the reduction (full symmetric storage: matrix-vector product and
@@ -430,13 +430,21 @@ __global__ void __launch_bounds__(THREADS) sp_bisect_kernel(const SpLayer* __res
 // ---- vectors of the kept atoms --------------------------------------------------------------------------------
 constexpr int kVecThreads = 256;
 constexpr int kVecWarps = kVecThreads / 32;
-constexpr int kVecCtasPerLayer = 4;
-constexpr int kVecGroup = 4;          // reflectors applied together in the back-transformation
+constexpr int kVecCtasPerLayer = 4;   // at most
+constexpr int kVecGroup = 8;          // reflectors applied together in the back-transformation
 constexpr int kVecStages = 4;         // groups in flight between global and shared memory
 constexpr int kVecWork = 3;           // work vectors of the twisted factorisation per warp
 constexpr double kSameEig = 1.0e-9;   // scaled units (largest eigenvalue below 1): eigenvalues this close share a subspace
 
+// One warp per kept atom, the atoms dealt to the layer's CTAs in turn.  The reflectors go in groups of eight as I - U T U^T: T is the
+// inverse of the triangle that U^T U and a diagonal of 1/2 make (unit reflectors, H = I - 2 u u^T), worked out for all groups by the
+// warps that have no vector of T to solve for.  A lane owns columns 4 lane .. 4 lane + 3 of every 128; the groups stream through a ring of
+// kVecStages buffers filled by asynchronous copies, a row per warp, kVecStages - 1 groups ahead of use.
+// Bound: the serial recurrences of the vector of T, then the chain of a group (dots, sums over the lanes, T, update).  512 rows, three kept
+// atoms, four reflectors at a time with their products formed by every warp | now: ResNet-18 set 115 | 84 us
+// (170 with the factorisation that waited for its operands), 40 layers of 500 rows 146 | 87, one of 64 rows 18.6 | 14.6.
 __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer* __restrict__ layers) {
+  static_assert(kVecGroup == 8 && kVecWarps == 8, "a warp copies a row of a group");
   const SpLayer& L = layers[blockIdx.x];
   if (L.tri != 1) return;                                     // larger layers: sp_eigvec_big_kernel
   extern __shared__ __align__(16) unsigned char vec_smem[];
@@ -445,31 +453,37 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
   double* s_e = s_d + rp;                                     // [rp]
   double* s_work = s_e + rp;                                  // [warps][kVecWork][rp]
   float* s_ref = reinterpret_cast<float*>(s_work + (size_t)kVecWarps * kVecWork * rp);   // [kVecStages][kVecGroup][rp] ring of reflector groups
-  __shared__ float s_beta[kVecStages][kVecGroup];
+  float* s_t = s_ref + (size_t)kVecStages * kVecGroup * rp;   // [rp / 8][8][8] T of the groups
+  __shared__ float s_dots[kVecWarps][32];
+  __shared__ int s_next;                                      // groups whose T somebody has taken on
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  const uint32_t k = L.hdr->k;
+  const uint32_t k = L.hdr->k, n_ctas = gridDim.y;
   // the layer's pointers in registers (a field read through `layers` inside a loop is a global load each time)
   const float* const gV = L.td_V; const int ldv = L.td_ldv; const double* const gLam = L.lam64;
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
   const int nref = max(r - 2, 0);
   const int ngroups = (nref + kVecGroup - 1) / kVecGroup;
-  for (int i = tid; i < r; i += kVecThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
-  __syncthreads();
+  constexpr int kQuads = kTriMaxRp / 128;
+  if (blockIdx.y < k) {
+    for (int i = tid; i < r; i += kVecThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
+    if (tid == 0) s_next = 0;
+    __syncthreads();
+  }
   double* wa = s_work + (size_t)w * kVecWork * rp;
   double* wb = wa + rp;
   double* z = wb + rp;
-  constexpr int kCols = kTriCols;
-  for (uint32_t a0 = blockIdx.y * kVecWarps; a0 < k; a0 += kVecCtasPerLayer * kVecWarps) {
-    const uint32_t a = a0 + w;
+  bool have_t = false;
+  for (uint32_t a0 = blockIdx.y; a0 < k; a0 += n_ctas * kVecWarps) {
+    const uint32_t a = a0 + n_ctas * w;
     const bool have = a < k;
-    float zr[kCols];                                          // z[lane + 32 m]
+    float4 zr[kQuads];                                        // z[128 m + 4 lane ..]
 #pragma unroll
-    for (int m = 0; m < kCols; ++m) zr[m] = 0.0f;
+    for (int m = 0; m < kQuads; ++m) zr[m] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (have) {
       const int ei = gPerm[gIdx[a]];                          // index of the atom's eigenvalue (ascending order)
       double lambda = gLam[ei];
-      // earlier kept atoms with the same eigenvalue (to the accuracy of the bisection): each takes another twist index
+      // earlier kept atoms with the same eigenvalue (to the accuracy of the eigenvalues): each takes another twist index
       int skip = 0;
       for (uint32_t b = lane; b < a; b += 32) skip += fabs(gLam[gPerm[gIdx[b]]] - lambda) <= kSameEig ? 1 : 0;
       skip = (int)warp_sum((uint32_t)skip);
@@ -486,88 +500,166 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
       }
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
 #pragma unroll
-      for (int m = 0; m < kCols; ++m) { const int i = lane + 32 * m; zr[m] = i < r ? (float)(z[i] * inv) : 0.0f; }
+      for (int m = 0; m < kQuads; ++m) {
+        const int i = 128 * m + 4 * lane;
+        if (i < r) zr[m] = make_float4((float)(z[i] * inv), i + 1 < r ? (float)(z[i + 1] * inv) : 0.f, i + 2 < r ? (float)(z[i + 2] * inv) : 0.f,
+                                       i + 3 < r ? (float)(z[i + 3] * inv) : 0.f);
+      }
     }
-    // u = H_0 H_1 ... H_{r-3} z: the reflectors from the last to the first, kVecGroup at a time, in fp32 (an orthogonal
-    // map of a unit vector whose result is stored in fp32 anyway).  For a group applied in the order 0, 1, 2, 3:
-    // s_0 = beta_0 v_0.z,  s_i = beta_i (v_i.z - sum_{j<i} s_j v_i.v_j),  z -= sum s_i v_i.
-    __syncthreads();
-    // group gi holds the reflectors kk = nref-1 - 4 gi - q, q = 0..3 in the order of application.  The groups stream
-    // through a ring of kVecStages buffers filled by asynchronous copies, kVecStages - 1 groups ahead of use; warp w
-    // copies half of row q = w mod 4.
+    if (!have_t) {                                            // T of the groups, whoever is free
+      for (;;) {
+        int gi = 0;
+        if (lane == 0) gi = atomicAdd(&s_next, 1);
+        gi = __shfl_sync(0xffffffffu, gi, 0);
+        if (gi >= ngroups) break;
+        float dots[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) dots[e] = 0.0f;
+        for (int m = 8 * gi / 128; 128 * m < r; ++m) {
+          float u[8][4];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const int kk = 8 * gi + q, i = 128 * m + 4 * lane;
+            const float* src = gV + (int64_t)kk * ldv + i;    // (rows of ldv floats, whole float4)
+            const float4 v = kk < nref && i < r ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            u[q][0] = v.x; u[q][1] = i + 1 < r ? v.y : 0.f; u[q][2] = i + 2 < r ? v.z : 0.f; u[q][3] = i + 3 < r ? v.w : 0.f;
+          }
+          int e = 0;
+#pragma unroll
+          for (int x = 1; x < 8; ++x)
+#pragma unroll
+            for (int q = 0; q < x; ++q, ++e) dots[e] = fmaf(u[x][0], u[q][0], fmaf(u[x][1], u[q][1], fmaf(u[x][2], u[q][2], fmaf(u[x][3], u[q][3], dots[e]))));
+        }
+        // sums over the lanes: lane ends with pair `lane`
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const bool high = lane & o;
+#pragma unroll
+          for (int e = 0; e < o; ++e) {
+            const float keep = high ? dots[e + o] : dots[e], send = high ? dots[e] : dots[e + o];
+            dots[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        }
+        s_dots[w][lane] = dots[0];
+        __syncwarp();
+        if (lane < 8) {                                       // column `lane` of T, from the diagonal up
+          double col[8];
+#pragma unroll
+          for (int q = 7; q >= 0; --q) {
+            double t = 0.0;
+#pragma unroll
+            for (int x = 7; x > q; --x) t = fma((double)s_dots[w][x * (x - 1) / 2 + q], col[x], t);
+            col[q] = q > lane ? 0.0 : q == lane ? 2.0 : -2.0 * t;
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q) s_t[gi * 64 + q * 8 + lane] = (float)col[q];
+        }
+        __syncwarp();
+      }
+      have_t = true;
+    }
+    // u = H_0 H_1 ... H_{r-3} z, the groups from the last to the first, in fp32 (an orthogonal map of a unit vector whose result is
+    // stored in fp32 anyway): z -= U (T (U^T z))
     auto issue_group = [&](int gi) {
-      if (gi < ngroups) {
-        const int buf = gi % kVecStages;
-        const int q = w & (kVecGroup - 1);
-        const int kk = nref - 1 - kVecGroup * gi - q;
-        const float* srow = gV + (int64_t)max(kk, 0) * ldv;   // rows start on 16-byte boundaries (ldv is a multiple of 4)
-        float* drow = s_ref + ((size_t)buf * kVecGroup + q) * rp;
-        for (int i = 4 * ((w / kVecGroup) * 32 + lane); i < rp; i += 4 * 32 * (kVecWarps / kVecGroup)) {
-          const int bytes = kk >= 0 ? 4 * max(0, min(4, r - i)) : 0;   // the rest of the 16 bytes is filled with zeros
+      if (gi >= 0) {
+        const int kk = kVecGroup * gi + w;
+        const float* srow = gV + (int64_t)min(kk, max(nref - 1, 0)) * ldv;   // rows start on 16-byte boundaries (ldv is a multiple of 4)
+        float* drow = s_ref + ((size_t)(gi % kVecStages) * kVecGroup + w) * rp;
+        for (int i = 128 * (8 * gi / 128) + 4 * lane; i < rp; i += 128) {
+          const int bytes = kk < nref ? 4 * max(0, min(4, r - i)) : 0;   // the rest of the 16 bytes is filled with zeros
           const uint32_t dst = (uint32_t)__cvta_generic_to_shared(drow + i);
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(bytes ? srow + i : gV), "r"(bytes) : "memory");
         }
-        if (tid < kVecGroup) { const int kq = nref - 1 - kVecGroup * gi - tid; s_beta[buf][tid] = kq >= 0 ? 2.0f : 0.0f; }   // unit reflectors
       }
       asm volatile("cp.async.commit_group;" ::: "memory");    // one group per call, empty or not: the counting stays uniform
     };
-    for (int st = 0; st < kVecStages - 1; ++st) issue_group(st);
-    for (int gi = 0; gi < ngroups; ++gi) {
-      const int buf = gi % kVecStages;
+    for (int st = 0; st < kVecStages - 1; ++st) issue_group(ngroups - 1 - st);
+    for (int gi = ngroups - 1; gi >= 0; --gi) {
       asm volatile("cp.async.wait_group %0;" ::"n"(kVecStages - 2) : "memory");
-      __syncthreads();                                        // group gi has landed for everybody; the buffer of gi-1 is free
-      issue_group(gi + kVecStages - 1);
+      __syncthreads();                                        // group gi has landed for everybody; the buffer of gi + 1 is free
+      issue_group(gi - (kVecStages - 1));
       if (have) {
-        const float* v0 = s_ref + ((size_t)buf * kVecGroup + 0) * rp;
-        const float* v1 = v0 + rp; const float* v2 = v1 + rp; const float* v3 = v2 + rp;
-        // the group's four reflectors into registers first (64 loads in flight), then the arithmetic
-        float r0[kCols], r1[kCols], r2[kCols], r3[kCols];
+        const float* const ref = s_ref + (size_t)(gi % kVecStages) * kVecGroup * rp + 4 * lane;
+        const float4* const trow = reinterpret_cast<const float4*>(s_t + gi * 64 + (lane >> 2) * 8);
+        const float4 t0 = trow[0], t1 = trow[1];
+        const int m0 = 8 * gi / 128;                          // (rows of the group are zero before)
+        float4 u[8][kQuads];
+        float p[8];
 #pragma unroll
-        for (int m = 0; m < kCols; ++m) {
-          const int i = lane + 32 * m;
-          const bool in = 32 * m < rp;
-          r0[m] = in ? v0[i] : 0.0f; r1[m] = in ? v1[i] : 0.0f; r2[m] = in ? v2[i] : 0.0f; r3[m] = in ? v3[i] : 0.0f;
+        for (int q = 0; q < 8; ++q) p[q] = 0.0f;
+#pragma unroll
+        for (int m = 0; m < kQuads; ++m) {
+          if (m >= m0 && 128 * m < rp) {
+            const bool in = 128 * m + 4 * lane < rp;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              u[q][m] = in ? *reinterpret_cast<const float4*>(ref + q * rp + 128 * m) : make_float4(0.f, 0.f, 0.f, 0.f);
+              p[q] = fmaf(u[q][m].x, zr[m].x, fmaf(u[q][m].y, zr[m].y, fmaf(u[q][m].z, zr[m].z, fmaf(u[q][m].w, zr[m].w, p[q]))));
+            }
+          }
         }
-        float z0 = 0, z1 = 0, z2 = 0, z3 = 0, g10 = 0, g20 = 0, g21 = 0, g30 = 0, g31 = 0, g32 = 0;
+        // sums over the lanes: lane ends with dot lane / 4
+        float sum;
+        {
+          float b[4], c2[2];
+          const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
 #pragma unroll
-        for (int m = 0; m < kCols; ++m) {
-          const float zz = zr[m];
-          z0 = fmaf(r0[m], zz, z0); z1 = fmaf(r1[m], zz, z1); z2 = fmaf(r2[m], zz, z2); z3 = fmaf(r3[m], zz, z3);
-          g10 = fmaf(r1[m], r0[m], g10); g20 = fmaf(r2[m], r0[m], g20); g21 = fmaf(r2[m], r1[m], g21);
-          g30 = fmaf(r3[m], r0[m], g30); g31 = fmaf(r3[m], r1[m], g31); g32 = fmaf(r3[m], r2[m], g32);
+          for (int q = 0; q < 4; ++q) b[q] = (h4 ? p[q + 4] : p[q]) + __shfl_xor_sync(0xffffffffu, h4 ? p[q] : p[q + 4], 16);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) c2[q] = (h3 ? b[q + 2] : b[q]) + __shfl_xor_sync(0xffffffffu, h3 ? b[q] : b[q + 2], 8);
+          sum = (h2 ? c2[1] : c2[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c2[0] : c2[1], 4);
+          sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+          sum += __shfl_xor_sync(0xffffffffu, sum, 1);
         }
+        const float tt[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+        float ca = 0.0f, cb = 0.0f;                           // (T p)_{lane / 4}
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          z0 += __shfl_xor_sync(0xffffffffu, z0, o); z1 += __shfl_xor_sync(0xffffffffu, z1, o);
-          z2 += __shfl_xor_sync(0xffffffffu, z2, o); z3 += __shfl_xor_sync(0xffffffffu, z3, o);
-          g10 += __shfl_xor_sync(0xffffffffu, g10, o); g20 += __shfl_xor_sync(0xffffffffu, g20, o);
-          g21 += __shfl_xor_sync(0xffffffffu, g21, o); g30 += __shfl_xor_sync(0xffffffffu, g30, o);
-          g31 += __shfl_xor_sync(0xffffffffu, g31, o); g32 += __shfl_xor_sync(0xffffffffu, g32, o);
+        for (int q = 0; q < 8; q += 2) {
+          ca = fmaf(tt[q], __shfl_sync(0xffffffffu, sum, 4 * q), ca);
+          cb = fmaf(tt[q + 1], __shfl_sync(0xffffffffu, sum, 4 * q + 4), cb);
         }
-        const float c0 = s_beta[buf][0] * z0;
-        const float c1 = s_beta[buf][1] * (z1 - c0 * g10);
-        const float c2 = s_beta[buf][2] * (z2 - c0 * g20 - c1 * g21);
-        const float c3 = s_beta[buf][3] * (z3 - c0 * g30 - c1 * g31 - c2 * g32);
+        const float mine = ca + cb;
+        float c[8];
 #pragma unroll
-        for (int m = 0; m < kCols; ++m) zr[m] -= fmaf(c0, r0[m], fmaf(c1, r1[m], fmaf(c2, r2[m], c3 * r3[m])));
+        for (int q = 0; q < 8; ++q) c[q] = __shfl_sync(0xffffffffu, mine, 4 * q);
+#pragma unroll
+        for (int m = 0; m < kQuads; ++m) {
+          if (m >= m0 && 128 * m < rp) {
+            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              d.x = fmaf(c[q], u[q][m].x, d.x); d.y = fmaf(c[q], u[q][m].y, d.y);
+              d.z = fmaf(c[q], u[q][m].z, d.z); d.w = fmaf(c[q], u[q][m].w, d.w);
+            }
+            zr[m].x -= d.x; zr[m].y -= d.y; zr[m].z -= d.z; zr[m].w -= d.w;
+          }
+        }
       }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                          // the ring is free for the next atoms
     if (have) {
       float n2 = 0.0f;
 #pragma unroll
-      for (int m = 0; m < kCols; ++m) n2 = fmaf(zr[m], zr[m], n2);
+      for (int m = 0; m < kQuads; ++m) n2 = fmaf(zr[m].x, zr[m].x, fmaf(zr[m].y, zr[m].y, fmaf(zr[m].z, zr[m].z, fmaf(zr[m].w, zr[m].w, n2))));
       n2 = warp_sum(n2);
       const float inv = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
 #pragma unroll
-      for (int m = 0; m < kCols; ++m) { const int i = lane + 32 * m; if (i < r) gShort[(int64_t)a * r + i] = zr[m] * inv; }
+      for (int m = 0; m < kQuads; ++m) {
+        const int i = 128 * m + 4 * lane;
+        float* const dst = gShort + (int64_t)a * r + i;
+        if (i < r) dst[0] = zr[m].x * inv;
+        if (i + 1 < r) dst[1] = zr[m].y * inv;
+        if (i + 2 < r) dst[2] = zr[m].z * inv;
+        if (i + 3 < r) dst[3] = zr[m].w * inv;
+      }
     }
   }
   // the last CTA of the layer orthogonalises kept atoms whose eigenvalues nearly coincide (their vectors are
   // determined only as a subspace): modified Gram-Schmidt in payload order, one warp
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(L.vec_ticket, 1u) == (uint32_t)(kVecCtasPerLayer - 1) ? 1u : 0u;
+  if (tid == 0) s_last = atomicAdd(L.vec_ticket, 1u) == n_ctas - 1u ? 1u : 0u;
   __syncthreads();
   if (!s_last || w != 0 || k < 2) return;
   __threadfence();
@@ -600,7 +692,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
 
 // ---- host side ---------------------------------------------------------------------------------------------------
 static size_t vec_smem_bytes(int rp_max) {
-  return (size_t)(2 + kVecWork * kVecWarps) * rp_max * sizeof(double) + (size_t)kVecStages * kVecGroup * rp_max * sizeof(float);
+  return (size_t)(2 + kVecWork * kVecWarps) * rp_max * sizeof(double) + (size_t)(kVecStages * kVecGroup + 8) * rp_max * sizeof(float);
 }
 
 int sp_tridiag_max_rp() { return kTriMaxRp; }
@@ -666,7 +758,13 @@ void launch_sp_bisect(const SpLayer* d_layers, int n_layers, int r_max, int64_t 
 }
 
 void launch_sp_eigvec(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st) {
-  sp_eigvec_kernel<<<dim3(n_layers, kVecCtasPerLayer), kVecThreads, vec_smem_bytes(rp_max), st>>>(d_layers);
+  // CTAs per layer (a CTA has an SM to itself): as many as keep the launch within one wave (100 layers of 64 rows with eight atoms each, four
+  // CTAs | one: 56 | 44 us)
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int per = kVecCtasPerLayer;
+  while (per > 1 && n_layers * per > sms) per /= 2;
+  sp_eigvec_kernel<<<dim3(n_layers, per), kVecThreads, vec_smem_bytes(rp_max), st>>>(d_layers);
 }
 
 }  // namespace atomo
