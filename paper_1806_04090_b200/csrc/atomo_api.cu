@@ -619,39 +619,29 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   }
   for (int l = 0; l < n_layers; ++l) L[l].lam_ready = (cluster_form || tri_form || given) ? 1 : 0;
   if (given) { for (int l = 0; l < n_layers; ++l) L[l].refine = 0; refine_tiles.clear(); }
-  // tensor-core Gram tiles: while the batch has fewer CTAs than the GPU has SMs, the K range of the layers with the
-  // longest rows is split over 2 or 4 CTAs per tile (at least 16 stages of 32 columns per part)
+  // tensor-core Gram tiles: while the batch has fewer CTAs than the GPU has SMs, the K range of a layer's tiles is split into parts of
+  // at most `most` stages (TF32: 32 columns each, 16 at least; integers: 64 columns, 8 at least), the smallest `most` with which the
+  // parts of all layers are resident together.  (Doubling the longest layer's split as long as it fitted left one of the ResNet-18
+  // set's four largest layers with twice the others' stages: 83 -> 63 us.)
   {
     int sms = 148, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    auto tiles_of = [&](int l) { const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile(); return tt * (tt + 1) / 2; };
-    int total = 0;
-    for (int l : tc_layers) { L[l].gram_split = 1; total += tiles_of(l); }
-    for (;;) {
-      int best = -1;
-      for (int l : tc_layers) {
-        const int stages = (L[l].L + 31) / 32 / L[l].gram_split;
-        if (L[l].gram_split < 4 && stages >= 32 && total + tiles_of(l) * L[l].gram_split <= sms &&
-            (best < 0 || stages > (L[best].L + 31) / 32 / L[best].gram_split))
-          best = l;
+    auto tiles_of = [&](int l) { const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile(); return (int64_t)tt * (tt + 1) / 2; };
+    auto split = [&](const std::vector<int>& which, int least, auto stages_of, auto min_of) {
+      auto parts = [&](int l, int most) { return std::max(min_of(l), std::max(1, std::min((stages_of(l) + most - 1) / most, stages_of(l) / least))); };
+      int lo = least, hi = least;                              // (more stages per part: never more parts)
+      for (int l : which) hi = std::max(hi, stages_of(l));
+      while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        int64_t total = 0;
+        for (int l : which) total += tiles_of(l) * parts(l, mid);
+        if (total <= sms) hi = mid; else lo = mid + 1;
       }
-      if (best < 0) break;
-      total += tiles_of(best) * L[best].gram_split;
-      L[best].gram_split *= 2;
-    }
-    // integer tiles likewise (at least 8 stages of 64 columns per part); their sums are exact in any number of parts
-    total = 0;
-    for (int l : i8_layers) { L[l].gram_split = sp_i8_min_split(L[l].L); total += tiles_of(l) * L[l].gram_split; }
-    for (;;) {
-      int best = -1;
-      for (int l : i8_layers) {
-        const int stages = sp_i8_stages(L[l].L) / L[l].gram_split;
-        if (stages >= 16 && total + tiles_of(l) * L[l].gram_split <= sms && (best < 0 || stages > sp_i8_stages(L[best].L) / L[best].gram_split)) best = l;
-      }
-      if (best < 0) break;
-      total += tiles_of(best) * L[best].gram_split;
-      L[best].gram_split *= 2;
-    }
+      for (int l : which) L[l].gram_split = parts(l, lo);
+    };
+    split(tc_layers, 16, [&](int l) { return (L[l].L + 31) / 32; }, [](int) { return 1; });
+    // (the integer tiles' sums are exact in any number of parts)
+    split(i8_layers, 8, [&](int l) { return sp_i8_stages(L[l].L); }, [&](int l) { return sp_i8_min_split(L[l].L); });
     for (int l : i8_layers) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
