@@ -299,6 +299,7 @@ int chase_room(atomo_ctx* ctx, int ctas) {
   if (known < 0) known = sp_chase_capacity(ctas);
   return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
+constexpr int kI8Short = 16, kI8LongMin = 192, kI8LongMax = 1 << 16;   // shapes below 513 rows that take the integer Gram kernel instead of the FMA kernel
 constexpr int64_t kI8Elements = (int64_t)1 << 26;             // elements from which layers of 513 .. 1024 rows take the integer Gram kernel
 int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
@@ -537,13 +538,15 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     d.tc = 0; d.gram_split = 1; d.gram_part_len = d.L;
     // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
-    // kernel, and above 512 those that the TF32 kernel cannot take, or all where they are many (with its digits, TF32 |
+    // kernel, and below those that the TF32 kernel cannot take (FMA | integer with its digits, us: 129 x 4097 76 | 36, 500 x 777 69 | 32, 30 of
+    // 400 x 2001 625 | 168, 16384 x 18 145 | 70, 33 x 257 21 | 16, 64 x 65 9 | 23, hence the least length; the longest keep the FMA kernel's
+    // bounded number of parts), or of 513 to 1024 rows all where they are many (TF32 |
     // integer, us: 20 layers of 1000 x 1200 241 | 259, one of 1024 x 4096 51 | 64, 40 of 520 x 8000 1081 | 767, 96 of 1024 x 4096 2818 | 2185)
     if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && mid_elements < kI8Elements)) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
       d.tc = 1;
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
-    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && d.r > 512) {
+    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && (d.r > 512 || (d.r > kI8Short && d.L >= kI8LongMin && d.L <= kI8LongMax))) {
       d.tc = 2;
       i8_layers.push_back(l);
     } else {
@@ -642,13 +645,17 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     split(tc_layers, 16, [&](int l) { return (L[l].L + 31) / 32; }, [](int) { return 1; });
     // (the integer tiles' sums are exact in any number of parts)
     split(i8_layers, 8, [&](int l) { return sp_i8_stages(L[l].L); }, [&](int l) { return sp_i8_min_split(L[l].L); });
+    int64_t i8_row_count = 0;                                // (rows per CTA of the digits' kernel: one after the other, eight CTAs per SM)
+    for (int l : i8_layers) if (sp_i8_by_rows(L[l].L, L[l].tall)) i8_row_count += L[l].r;
+    const int row_step = (int)std::min<int64_t>(16, std::max<int64_t>(1, i8_row_count / (8 * sms)));
     for (int l : i8_layers) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
         for (int c = 0; c < L[l].gram_split; ++c) i8_tiles.push_back({l, a, b, c});
       int na = 0, nb = 0;
       sp_i8_prep_tiles(L[l].r, L[l].L, L[l].tall, &na, &nb);
-      for (int a = 0; a < na; ++a) for (int b = 0; b < nb; ++b) (sp_i8_by_rows(L[l].L, L[l].tall) ? i8_rows : i8_prep).push_back({l, a, b, 0});
+      if (sp_i8_by_rows(L[l].L, L[l].tall)) for (int a = 0; a < na; a += row_step) i8_rows.push_back({l, a, 0, row_step});
+      else for (int a = 0; a < na; ++a) for (int b = 0; b < nb; ++b) i8_prep.push_back({l, a, b, 0});
     }
     i8_prep.insert(i8_prep.begin(), i8_rows.begin(), i8_rows.end());
     for (int l : tc_layers) {

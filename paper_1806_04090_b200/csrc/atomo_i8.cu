@@ -1,5 +1,6 @@
-// Gram matrix of the short side on the 5th-generation tensor cores from 8-bit integers: layers with a short side above 1024, and above
-// 512 those that the TF32 kernel (atomo_tc.cu) cannot take (tall, or rows that do not start on 16-byte boundaries).
+// Gram matrix of the short side on the 5th-generation tensor cores from 8-bit integers: layers with a short side above 1024, all that the
+// TF32 kernel (atomo_tc.cu) cannot take (tall, or rows that do not start on 16-byte boundaries) but for very short or
+// narrow ones, and those of 513 to 1024 rows where a call has many elements of them.
 //
 //   sp_i8_row_kernel    vector i in units of 2^(E_i - 30), 2^E_i above its largest magnitude, rounded to integers, written as four
 //                       signed base-256 digits in four planes [digit][i][k], contiguous along the contraction whatever G's layout:
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(256) sp_i8_row_kernel(const SpLayer* __restric
   __shared__ uint32_t s_max[2][8];
   const TileRef ref = tiles[blockIdx.x];
   const SpLayer& L = layers[ref.layer];
-  const int i_lo = ref.a * kI8WideRows, i_hi = min(L.r, i_lo + kI8WideRows);
+  const int i_lo = ref.a, i_hi = min(L.r, ref.a + ref.c);      // (a few rows, one after the other)
   if (L.L <= 2048) i8_rows<2>(L, i_lo, i_hi, s_max);
   else if (L.L <= 4096) i8_rows<4>(L, i_lo, i_hi, s_max);
   else i8_rows<8>(L, i_lo, i_hi, s_max);
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kI8Threads, 1) sp_gram_i8_kernel(const SpLayer
           double sum[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) sum[j] = 0.0;
-#pragma unroll 2
+#pragma unroll 4
           for (int sp = 0; sp < n_split; ++sp) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) sum[j] += __ldcg(parts + ((int64_t)sp * kI8Tile + c0 + j) * kI8Tile);
@@ -429,10 +430,10 @@ int64_t sp_i8_sums(int r, int split) {
   return split > 1 ? tt * (tt + 1) / 2 * split * kI8Tile * kI8Tile : 0;
 }
 bool sp_i8_by_rows(int len, bool tall) { return !tall && len <= kI8RowLen; }
-// tiles of the layer's preparing kernels; by rows: one along the long side
+// tiles of the layer's preparing kernels (by rows: the rows themselves, which the caller groups)
 void sp_i8_prep_tiles(int r, int len, bool tall, int* short_tiles, int* long_tiles) {
   const int a = tall ? kI8TallCols : kI8WideRows, b = tall ? kI8TallRows : kI8WideCols;
-  *short_tiles = (r + a - 1) / a; *long_tiles = sp_i8_by_rows(len, tall) ? 1 : (len + b - 1) / b;
+  *short_tiles = sp_i8_by_rows(len, tall) ? r : (r + a - 1) / a; *long_tiles = sp_i8_by_rows(len, tall) ? 1 : (len + b - 1) / b;
 }
 // tensor map of the digits [4][r][pitch]: boxes of 64 columns x 128 vectors x 4 digits, 64-byte swizzle, zero fill outside
 int sp_i8_make_map(void* out_map /*CUtensorMap, host*/, const int8_t* digits, int r, int len, int64_t pitch) {

@@ -33,6 +33,7 @@ def _check(a, G):
 
 @pytest.mark.parametrize("m,n", [(513, 517), (640, 641), (1025, 1026), (1152, 1153), (1153, 2049), (1025, 8191), (1025, 8193),   # rows, two passes
                                  (700, 513), (1100, 1037), (3001, 641), (1153, 1025),                                        # columns
+                                 (17, 193), (129, 2049), (2047, 255), (16384, 18), (300, 65535),                             # narrow ones
                                  (520, 33001)])                                                                              # more columns than an accumulator holds
 def test_edges(atomo, m, n):
     gen = torch.Generator(device="cuda")
