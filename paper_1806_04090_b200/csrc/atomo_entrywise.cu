@@ -839,7 +839,12 @@ __device__ __forceinline__ int ew_vec_of(const EwVec (&vecs)[N], const int n, co
 // The one-kernel form.  Dynamic shared memory: [scratch: candidate slots, or list of large atoms, later the staging window]
 // [code bytes of the chunk] [list form: prefix words].  A chunk of at most kEwRegTiles tiles keeps its entries in
 // registers and draws its words before the barrier: nothing is read twice and no list is kept.
-template <int N>
+// kForm: what the chunks of the launch are, where they are all of one kind (64 registers hold any one of the kinds, but for the code of
+// all of them together a chunk's entries were spilled); kMixed asks each chunk.  Spilled bytes 368 | 76 .. 136; a pass,
+// us, one instance for all | by kind: 20 k elements 18.4 | 16.4, 1.5 M 23.8 | 21.9, 4 M at 10 % 45.0 | 43.0, 100 M at 10 % 343 | 338, 25.6 M by QSGD's budget
+// 109.6 | 106.5, three short vectors 20.3 | 18.6.
+enum { kMixed, kRegisters, kCandidates, kBigList };
+template <int N, int kForm>
 __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_constant__ EwBatch<N> B) {
   extern __shared__ __align__(16) uint32_t ew_smem[];
   __shared__ EwShared sh;
@@ -856,7 +861,8 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
   }
   if (tid == 0) v.chunk_status[c.index] = 0ull;            // ordered before its first use by the barrier after pass 1
   __syncthreads();
-  if (c.n_my <= kEwRegTiles && v.prob_out == nullptr && !v.candidates) {
+  if constexpr (kForm == kMixed || kForm == kRegisters)
+  if (kForm == kRegisters || (c.n_my <= kEwRegTiles && v.prob_out == nullptr && !v.candidates)) {
     float4 x[4];
     uint4 wd[4];
     const int unit = tid / kWarp;
@@ -884,7 +890,8 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
     ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
     return;
   }
-  if (v.candidates) {
+  if constexpr (kForm == kMixed || kForm == kCandidates)
+  if (kForm == kCandidates || v.candidates) {
     const uint32_t cand0 = (uint32_t)__cvta_generic_to_shared(scratch) + 4u * tid;
     EwCands cands{scratch, 0.0f, cand0, cand0};
     for (int i = tid; i < c.n_my * (kEwBlocks / 16); i += kEwThreads) reinterpret_cast<uint4*>(code)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -910,18 +917,20 @@ __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_c
     }
     return;
   }
-  EwBigList big{scratch, 0u, 0.0f, 0.0};
-  const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
-  c = ew_chunk(v, ew_opaque(blockIdx.x) - (uint32_t)v.cta0);
-  const float lo = big.lo;
-  const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
-    // (a barrier has passed since the pass)
-    return *(volatile uint32_t*)&sh.big_over == 0u && theta >= lo ? ew_round_list(v, c, big, theta, sh) : ew_round_memory(v, c, theta);
-  }, sh);
-  if (c.index == 0 && tid == 0) ew_store_state(v, S);
-  ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
-  __syncthreads();
-  ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
+  if constexpr (kForm == kMixed || kForm == kBigList) {
+    EwBigList big{scratch, 0u, 0.0f, 0.0};
+    const EwAcc first = ew_pass_big(v, c, B.s, big, sh);
+    c = ew_chunk(v, ew_opaque(blockIdx.x) - (uint32_t)v.cta0);
+    const float lo = big.lo;
+    const EwSolved S = ew_solve(v, c, B.s, first, [&](float theta) {
+      // (a barrier has passed since the pass)
+      return *(volatile uint32_t*)&sh.big_over == 0u && theta >= lo ? ew_round_list(v, c, big, theta, sh) : ew_round_memory(v, c, theta);
+    }, sh);
+    if (c.index == 0 && tid == 0) ew_store_state(v, S);
+    ew_decide_memory(v, c, ew_decide_of(S), B.key, B.kind_step, sh, code);
+    __syncthreads();
+    ew_pack(v, c, S, ew_arrivals(v, S), code, scratch, sh);
+  }
 }
 
 // The two-kernel form: the solve leaves its result in the state record; a CTA of the second kernel takes the next chunk of
@@ -1256,7 +1265,9 @@ constexpr int kEwPackTiles = 64;                    // tiles per chunk of the tw
 }  // namespace
 
 int ew_configure() {
-  const void* fns[] = {(const void*)ew_encode_kernel<1>, (const void*)ew_encode_kernel<kEwBatch>, (const void*)ew_sample_pack_kernel};
+  const void* fns[] = {(const void*)ew_encode_kernel<1, kMixed>, (const void*)ew_encode_kernel<1, kRegisters>, (const void*)ew_encode_kernel<1, kCandidates>,
+                       (const void*)ew_encode_kernel<1, kBigList>, (const void*)ew_encode_kernel<kEwBatch, kMixed>,
+                       (const void*)ew_encode_kernel<kEwBatch, kRegisters>, (const void*)ew_sample_pack_kernel};
   for (const void* f : fns) {
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEwMaxDyn);
     if (e != cudaSuccess) return (int)e;
@@ -1307,9 +1318,22 @@ int launch_ew_encode(EwBatch<N>& B, bool list, cudaStream_t st) {
   }
   B.scratch_words = (int)(ew_scratch_bytes(list) / sizeof(uint32_t));
   const size_t smem = ew_dyn_bytes((int)most, list);
-  if (!waits) { ew_encode_kernel<N><<<ctas, kEwThreads, smem, st>>>(B); return (int)cudaGetLastError(); }
+  // the instance for what the chunks are (a vector's chunks differ by one tile: those beside the bound may be of two kinds); calls
+  // with several vectors are either all short or mixed
+  bool all_reg = true, all_cand = true, all_big = true;
+  for (int i = 0; i < B.n; ++i) {
+    const EwVec& v = B.v[i];
+    const bool reg = v.prob_out == nullptr && !v.candidates;   // may keep short chunks in registers
+    all_reg &= reg && (v.n_tiles + v.n_ctas - 1) / v.n_ctas <= kEwRegTiles;
+    all_cand &= v.candidates != 0;
+    all_big &= !v.candidates && (!reg || v.n_tiles / v.n_ctas > kEwRegTiles);
+  }
+  const void* fn = (const void*)ew_encode_kernel<N, kMixed>;
+  if (all_reg) fn = (const void*)ew_encode_kernel<N, kRegisters>;
+  else if constexpr (N == 1) { if (all_cand) fn = (const void*)ew_encode_kernel<1, kCandidates>; else if (all_big) fn = (const void*)ew_encode_kernel<1, kBigList>; }
   void* args[] = {&B};
-  return (int)cudaLaunchCooperativeKernel((const void*)ew_encode_kernel<N>, dim3((unsigned)ctas), dim3(kEwThreads), args, smem, st);
+  if (!waits) return (int)cudaLaunchKernel(fn, dim3((unsigned)ctas), dim3(kEwThreads), args, smem, st);
+  return (int)cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctas), dim3(kEwThreads), args, smem, st);
 }
 template int launch_ew_encode<1>(EwBatch<1>&, bool, cudaStream_t);
 template int launch_ew_encode<kEwBatch>(EwBatch<kEwBatch>&, bool, cudaStream_t);
