@@ -121,7 +121,7 @@ typedef struct { float* sigma; float* prob; uint32_t* mask_words; float* short_v
 
 /* Stage timers (milliseconds of device time, CUDA events on the call's stream) filled while
  * profiling is on.  `launches[i]` counts the kernels of stage i in the last call.  On the
- * tridiagonal route EIG is the Householder reduction alone; the bisection for the eigenvalues
+ * tridiagonal route EIG is the Householder reduction alone; the kernel of the eigenvalues
  * is timed with SAMPLE and the vectors of the kept atoms with BACKPROJECT.  EW_REDUCE is the solve
  * kernel of vectors that take the two-kernel form; the one-kernel form is timed as EW_PACK.  */
 enum { ATOMO_STAGE_GRAM = 0, ATOMO_STAGE_EIG, ATOMO_STAGE_SAMPLE, ATOMO_STAGE_BACKPROJECT,
@@ -291,15 +291,17 @@ int atomo_set_eig_mode(atomo_ctx* ctx, int32_t mode);
  * turns into a visible error of the nuclear norm and thus of every p_i; the projection norm does not
  * have that floor.  It costs one more pass over G with twice the Gram matrix's arithmetic.              */
 int atomo_set_sigma_refinement(atomo_ctx* ctx, int32_t min_short_side);
-/* Gram matrix path: 1 (default) = tcgen05 tensor cores with the TF32 hi/lo split for layers with rows <= cols, a short
- * side of at most 1024, a 16-byte aligned base and ld % 4 == 0 (other layers take the fp32 FMA kernel); 0 = fp32 FMA
- * kernel always.  The tensor core accumulates in fp32 with truncation: at a short side of 1024 the probabilities then
- * sit within about 3e-6 of those of an exact decomposition (the few largest p_i; measured), with the FMA kernel within
+/* Gram matrix path: 1 (default) = tcgen05 tensor cores: a TF32 hi/lo split for layers with rows <= cols, a short side of at
+ * most 1024, a 16-byte aligned base and ld % 4 == 0; 8-bit integer digits (exact sums) for larger short sides, for other
+ * layouts (short side above 16, long side from 192; at most 65536 where the short side is at most 512) and, from 2^26 elements
+ * of them in a call, for all layers with a short side of 513 to 1024 (digits of at most 8 GiB per call); the fp32 FMA kernel for the rest.  0 = fp32 FMA
+ * kernel always.  The TF32 accumulator truncates: at a short side of 1024 the probabilities then
+ * sit within about 3e-6 of those of an exact decomposition (the few largest p_i; measured), with the other kernels within
  * about 5e-7.  A caller that needs every draw to agree with an fp64 computation outside a 1e-6 margin takes 0.    */
 int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores);
 /* Eigen-solver scheme (`enabled` = 0, 1, 2 or 3):
  * 3 (default) = the tridiagonal routes: the scaled Gram matrix of every layer is reduced to tridiagonal form by
- *     Householder reflectors, all eigenvalues come from bisection on Sturm counts, and eigenvectors are computed for the
+ *     Householder reflectors, all eigenvalues come from brackets of Sturm counts, and eigenvectors are computed for the
  *     kept atoms only (twisted factorisation, back-transformation with the reflectors): only the singular values of
  *     all atoms enter the probabilities, the vectors of atoms that are not kept are never formed.  Short sides up to
  *     512: the rows sit in the registers of the CTAs of a 16-CTA cluster and are exchanged through distributed shared

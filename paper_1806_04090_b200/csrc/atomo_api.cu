@@ -300,6 +300,7 @@ int chase_room(atomo_ctx* ctx, int ctas) {
   return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
 constexpr int kI8Short = 16, kI8LongMin = 192, kI8LongMax = 1 << 16;   // shapes below 513 rows that take the integer Gram kernel instead of the FMA kernel
+constexpr int64_t kI8Bytes = (int64_t)1 << 33;                // most that the digits of a call may take beside its gradients (beyond: the other kernels)
 constexpr int64_t kI8Elements = (int64_t)1 << 26;             // elements from which layers of 513 .. 1024 rows take the integer Gram kernel
 int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
@@ -516,6 +517,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   const int map_bytes = sp_tc_map_bytes();
   std::vector<uint8_t> maps_blob((size_t)n_layers * map_bytes, 0);
   int chol_panels = 0;
+  int64_t i8_bytes = 0;                                      // digits of the layers so far that take the integer Gram kernel
   int64_t mid_elements = 0;                                  // of the layers with a short side of 513 .. 1024
   for (int l = 0; l < n_layers; ++l) { const int r = std::min(layers[l].rows, layers[l].cols); if (r > 512 && r <= 1024) mid_elements += (int64_t)layers[l].rows * layers[l].cols; }
   int row_floats_max = 0, steps_max = 0, r_max = 0, rp_max = 0, r_max_tall = 0, k_cap_max = 1;
@@ -536,18 +538,21 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     r_max = std::max(r_max, d.r); rp_max = std::max(rp_max, d.rp);
     const int gt = (d.r + 63) / 64;
     d.tc = 0; d.gram_split = 1; d.gram_part_len = d.L;
+    const int64_t digits = 4 * (int64_t)d.r * sp_i8_pitch(d.L);
+    const bool digits_fit = i8_bytes + digits <= kI8Bytes;
     // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
     // kernel, and below those that the TF32 kernel cannot take (FMA | integer with its digits, us: 129 x 4097 76 | 36, 500 x 777 69 | 32, 30 of
     // 400 x 2001 625 | 168, 16384 x 18 145 | 70, 33 x 257 21 | 16, 64 x 65 9 | 23, hence the least length; the longest keep the FMA kernel's
     // bounded number of parts), or of 513 to 1024 rows all where they are many (TF32 |
     // integer, us: 20 layers of 1000 x 1200 241 | 259, one of 1024 x 4096 51 | 64, 40 of 520 x 8000 1081 | 767, 96 of 1024 x 4096 2818 | 2185)
-    if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && mid_elements < kI8Elements)) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
+    if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && (mid_elements < kI8Elements || !digits_fit))) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
       d.tc = 1;
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
-    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && (d.r > 512 || (d.r > kI8Short && d.L >= kI8LongMin && d.L <= kI8LongMax))) {
+    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || (d.r > kI8Short && d.L >= kI8LongMin && d.L <= kI8LongMax))) {
       d.tc = 2;
+      i8_bytes += digits;
       i8_layers.push_back(l);
     } else {
       d.gram_split = given ? 1 : sp_gram_split(d.r, d.L);
@@ -913,7 +918,9 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     const int e = launch_sp_cholesky_big(d_layers, d_chol, (int)chol_ctas.size(), chol_panels, st);
     if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(cholesky)");
   }
-  stage_end(ctx, ATOMO_STAGE_GRAM, st, 5);
+  const bool fma_large = gram_tiles.size() > gram_parts.size(), i8_two = i8_prep.size() > i8_rows.size();
+  stage_end(ctx, ATOMO_STAGE_GRAM, st, given ? 1 : 2 + (fma_large ? 1 : 0) + (gram_parts.empty() ? 0 : 1) + (tc_tiles.empty() ? 0 : 1) +
+                                           (i8_tiles.empty() ? 0 : 1) + (i8_rows.empty() ? 0 : 1) + (i8_two ? 2 : 0));
   CK(cudaGetLastError());
 
   // ---- S1: eigen-solver; the host reads a convergence flag once per sweep of the largest layer ----
@@ -957,7 +964,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       ++n_eig_launch;
     }
     if (chase_err != 0) return fail_cuda(ctx, (cudaError_t)chase_err, "cudaLaunchKernelEx(bulge chase)");
-    // the eigenvalues (bisection) are timed with the sampling stage.  No host wait on this route: a bounded wait of
+    // the eigenvalues are timed with the sampling stage.  No host wait on this route: a bounded wait of
     // the Gram kernel that ran out is reported by the sampling kernel in every layer's status word
     // (ATOMO_ERR_TIMEOUT, nothing kept)
   }

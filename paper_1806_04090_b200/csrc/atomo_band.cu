@@ -8,7 +8,7 @@
 //   sp_chase_kernel  B -> T = Q2^T B Q2 by bulge chasing, fp64, the band in shared memory (one CTA per layer up to a short
 //                    side of 1024, a cluster above), all sweeps in flight at once.
 //
-// Then the eigenvalues of T by bisection and vectors for the kept atoms only, as on the small route; a vector of T goes
+// Then the eigenvalues of T and vectors for the kept atoms only, as on the small route; a vector of T goes
 // through the chase's reflectors and then through the panels' (I - U T U^T, the columns of U as rows of td_V) in the vector
 // kernels of atomo_tridiag_big.cu.
 //

@@ -105,7 +105,7 @@ struct SpLayer {
   int refine, refine_tiles;    // singular values from the projection norms; tiles along the long side
   float* row_inv;              // rp: 1 / norm of each short-side vector as stored in X
   float* refine_partials;      // [refine_tiles][rp] partial squared norms
-  // tridiagonal route (short side <= 512): T = Q^T A Q, eigenvalues by bisection, vectors of the kept atoms only
+  // tridiagonal route (short side <= 512): T = Q^T A Q, its eigenvalues, vectors of the kept atoms only
   int tri;                     // this layer takes the tridiagonal route: 1 = registers of a cluster (rp <= 512), 2 = two stages, A in global memory
   double* td_d; double* td_e;  // rp each: diagonal and off-diagonal of T
   int td_ldv;                  // floats per row of td_V: r rounded up to a multiple of 4 (16-byte rows)
