@@ -342,6 +342,24 @@ def band_bytes(shapes):
     return float(sum(8.0 * (min(sh) - c) ** 2 for sh in shapes if min(sh) > 512 for c in range(8, min(sh), 8)))
 
 
+def gram_line(run, ms, peaks):
+    """Rate of the Gram stage: useful flop of one triangle of G G^T, and what the tensor cores issue for it."""
+    useful = sum(min(m, n) ** 2 * float(max(m, n)) for m, n in run.shapes)
+    mid = sum(m * n for m, n in run.shapes if 512 < min(m, n) <= 1024)
+    integer = mid >= 1 << 26 or any(min(m, n) > 1024 for m, n in run.shapes)      # which kernel takes most of the work
+    peak = peaks["bf16_tflops"] * (4.5 if integer else 1.1) / 2.25
+    products = 10.0 if integer else 3.0
+    line = {"kernel": "sp_gram_i8_kernel (tcgen05 kind::i8, ten digit products) with sp_i8_row_kernel" if integer else "sp_gram_tc_kernel (tcgen05, 3 x TF32)",
+            "ms_per_step": ms, "peak_tflops": peak,
+            "peak_source": f"{peaks['source']} bf16 burst x nominal {'4.5' if integer else '1.1'}/2.25",
+            "note": "useful = one triangle of G G^T, r^2 L flop; the stage also holds the digits, trace and scaling"}
+    if ms:
+        line["useful_tflops"] = useful / (ms * 1e-3) / 1e12
+        line["issued_frac"] = products * line["useful_tflops"] / peak
+        line["meets_50pct_target"] = line["issued_frac"] >= 0.5
+    return line
+
+
 def roofline_for(run, eig_ms_per_step, eig_launches_per_step, scheme, peaks, fma_peaks, step_ms):
     """Roofline of the dominant kernel of a spectral workload (the eigen stage)."""
     shapes = run.shapes
@@ -616,16 +634,7 @@ def run_ours(args):
         }
         if run.spectral:
             line["roofline"] = roofline_for(run, tot_ms["eig"] / stage_steps, tot_ln["eig"] / stage_steps, scheme, peaks, fma_peaks, ms_per_step)
-            gram_flops = sum(min(m, n) ** 2 * max(m, n) * 2.0 for m, n in run.shapes)      # useful flops, full square
-            tf32_peak = peaks["bf16_tflops"] * (1.1 / 2.25)
-            line["gram"] = {"kernel": "sp_gram_tc_kernel (tcgen05, 3 x TF32)", "ms_per_step": stage.get("gram"),
-                            "useful_tflops": gram_flops / 2 / (stage["gram"] * 1e-3) / 1e12 if stage.get("gram") else None,
-                            "tf32_peak_tflops": tf32_peak, "peak_source": f"{peaks['source']} bf16 burst x nominal 1.1/2.25",
-                            "note": "useful = one triangle of G G^T, r^2 L flop; the stage also holds trace and scaling"}
-            if line["gram"]["useful_tflops"]:
-                line["gram"]["useful_frac"] = line["gram"]["useful_tflops"] / tf32_peak
-                line["gram"]["issued_frac"] = 3.0 * line["gram"]["useful_tflops"] / tf32_peak
-                line["gram"]["meets_50pct_target"] = line["gram"]["issued_frac"] >= 0.5
+            line["gram"] = gram_line(run, stage.get("gram"), peaks)
         else:
             gbs = 12.0 * elems / (ms_per_step * 1e-3) / 1e9
             line["roofline"] = {"bound": "hbm", "kernel": "entry-wise path (ew_encode + ew_decode)", "achieved": gbs,

@@ -34,3 +34,16 @@ def test_algorithmic_work_of_the_reductions():
 def test_workload_text_names_the_config_and_budget():
     assert "c5" in bench.workload_text("c5", 4.0) and "s=4" in bench.workload_text("c5", 4.0)
     assert "1 % of the length" in bench.workload_text("c4", 0.01)
+
+
+def test_gram_line_names_the_kernel_and_what_it_issues():
+    class Run:
+        def __init__(self, shapes): self.shapes = shapes
+    peaks = {"bf16_tflops": 2250.0, "source": "nominal"}
+    tf32 = bench.gram_line(Run([(512, 4608)] * 4), 1.0, peaks)
+    assert "tf32" in tf32["kernel"].lower() and tf32["peak_tflops"] == 1100.0
+    assert abs(tf32["issued_frac"] - 3.0 * 4 * 512 ** 2 * 4608.0 / 1e-3 / 1e12 / 1100.0) < 1e-12
+    for shapes in ([(1024, 4096)] * 96, [(2048, 2048)]):
+        line = bench.gram_line(Run(shapes), 2.0, peaks)
+        assert "i8" in line["kernel"] and line["peak_tflops"] == 4500.0
+    assert "issued_frac" not in bench.gram_line(Run([(64, 64)]), None, peaks)
