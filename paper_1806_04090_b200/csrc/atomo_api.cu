@@ -1043,7 +1043,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     } else if (any_small) launch_sp_eigvec(d_layers, n_layers, rp_max_small, st);
     int rps = 0;
     for (int l : big_layers) rps |= L[l].rp <= 1024 ? 1 : L[l].rp <= 2048 ? 2 : 4;
-    launch_sp_eigvec_big(d_layers, d_big, (int)big_layers.size(), rps, st);
+    launch_sp_eigvec_big(d_layers, d_big, (int)big_layers.size(), rps, s, st);
     if (any_small && any_big) CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
   }
   launch_sp_backproject(d_layers, d_bp, (int)bp_tiles.size(), std::max(r_max_tall, 1), st);

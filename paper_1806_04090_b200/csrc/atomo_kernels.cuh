@@ -181,7 +181,7 @@ int launch_sp_chase(const SpLayer* d_layers, const int* d_list, int n, int ctas,
 int sp_configure_eigvec_big();                                    // 0 if available
 int sp_configure_bisect();                                        // 0 if the eigenvalue kernel got its shared memory
 // rps: which padded short sides are among them (bit 0: up to 1024, bit 1: up to 2048, bit 2: above)
-void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, cudaStream_t st);
+void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, double budget, cudaStream_t st);
 int launch_sp_cholesky(const SpLayer* d_layers, int n_layers, int rp_max, cudaStream_t st);
 int launch_sp_cholesky_big(const SpLayer* d_layers, const TileRef* d_ctas, int n_ctas, int max_panels, cudaStream_t st);
 int sp_cholesky_big_rows_per_cta();

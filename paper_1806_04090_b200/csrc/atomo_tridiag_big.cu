@@ -2,6 +2,7 @@
 // atomo_band.cu).  A vector of the tridiagonal T goes through the reflectors of the bulge chase and then through those of the
 // panels: u = Q1 Q2 z.
 #include <algorithm>
+#include <cmath>
 
 #include "atomo_kernels.cuh"
 #include "atomo_twisted.cuh"
@@ -18,7 +19,7 @@ namespace atomo {
 // 2.7e-8 instead of 1.0e-8 on 1024 x 4096 noise, its vectors orthogonal to 2.4e-7 instead of 4e-9: the eigenvector of the band
 // fills eight times as many entries as one of a one-stage T, and each of its reflectors rounds them.
 // Measured, before (a block barrier per sweep, four panel reflectors at a time, work vectors in global memory) | now: two layers of 4096 rows
-// 8.0 | 3.7 ms, nine of 2048 rows 2.23 | 1.30, 96 of 1024 rows 1.66 | 1.02, one of 1023 rows 0.54 | 0.33.  What bounds it now:
+// 8.0 | 3.7 ms, nine of 2048 rows 2.23 | 1.01, 96 of 1024 rows 1.66 | 1.02, one of 1023 rows 0.54 | 0.33.  What bounds it now:
 // the panels (sums over all warps and conversions to fp64: 3500 cycles each at 1024 rows, 8500 at 4096), then the sweeps of the chase
 // (290 and 640 cycles each).
 // Tried and dropped: what the moves bring fetched once per turn instead of a load per sweep (spills: 3.8 -> 4.5 ms); eight warps per atom up
@@ -315,11 +316,11 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
   vb_orthogonalise_equal(L, k, kVcCtas);
 }
 
-// BATCH atoms at a time, COLS columns per thread: up to a short side of 2048, or above
-template <int BATCH, int COLS>
-__global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLayer* __restrict__ layers,
+// BATCH atoms at a time (through the chase as many as THREADS has warps for), COLS columns per thread: up to a short side of 2048, or above
+template <int THREADS, int BATCH, int COLS, int DEPTH>
+__global__ void __launch_bounds__(THREADS, 1) sp_eigvec_big_kernel(const SpLayer* __restrict__ layers,
                                                                       const int* __restrict__ big_layers) {
-  constexpr int kRp = COLS * kVbThreads, kFew = kVbThreads * 8 / kRp;
+  constexpr int kRp = COLS * THREADS, kFew = THREADS * 8 / kRp, kWarps = THREADS / 32;
   const SpLayer& L = layers[big_layers[blockIdx.x]];
   if (L.rp <= kVcMaxRp || (L.rp <= kVbHalf) != (kRp <= kVbHalf)) return;   // another kernel's
   extern __shared__ __align__(16) unsigned char vb_smem[];
@@ -327,8 +328,8 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
   double* s_z = reinterpret_cast<double*>(vb_smem);            // [BATCH][rp]
   double* s_d = s_z + (size_t)BATCH * rp;                      // [rp], phase A
   double* s_e = s_d + rp;                                      // [rp]
-  __shared__ double s_ex[kVbWarps * (BATCH > 2 ? 8 * BATCH : 16)];   // what the warps exchange: in the chase's turns, in the panels' sums
-  double (*const s_edge)[kVbWarps][8] = reinterpret_cast<double (*)[kVbWarps][8]>(s_ex);
+  __shared__ double s_ex[kWarps * (BATCH > 2 ? 8 * BATCH : 16)];   // what the warps exchange: in the chase's turns, in the panels' sums
+  double (*const s_edge)[kWarps][8] = reinterpret_cast<double (*)[kWarps][8]>(s_ex);
   double (*const s_part)[8 * BATCH] = reinterpret_cast<double (*)[8 * BATCH]>(s_ex);
   __shared__ double s_tot[8 * BATCH];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
   double* const gZ = L.tb_z;
   const int nref = max(r - kBandWidth - 1, 0);
-  for (int i = tid; i < r; i += kVbThreads) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
+  for (int i = tid; i < r; i += THREADS) { s_d[i] = L.td_d[i]; s_e[i] = i + 1 < r ? L.td_e[i] : 0.0; }
   __syncthreads();
   // ---- (A) this CTA's atoms are a = cy, cy + n_ctas, ...; as many warps as there is room for work vectors beside T share them ----
   constexpr int kWork = kRp <= kVbHalf ? 2 : 1;
@@ -374,26 +375,26 @@ __global__ void __launch_bounds__(kVbThreads, 1) sp_eigvec_big_kernel(const SpLa
     const int nb = (int)min((uint32_t)BATCH, n_mine - b0);
     for (int b = 0; b < BATCH; ++b) {
       const double* src = gZ + (int64_t)(cy + (b0 + b) * n_ctas) * rp;
-      for (int i = tid; i < r; i += kVbThreads) s_z[(size_t)b * rp + i] = b < nb ? __ldcg(src + i) : 0.0;
+      for (int i = tid; i < r; i += THREADS) s_z[(size_t)b * rp + i] = b < nb ? __ldcg(src + i) : 0.0;
     }
     __syncthreads();
     // a run per thread: one or two atoms at a time
-    for (int b = 0; b < nb; b += kFew) vb_chase_back<kVbThreads, kFew, 4>(L.bd_V2, r, s_z + (size_t)b * rp, rp, nb - b, s_edge);
-    vb_apply_reflectors<kVbThreads, BATCH, COLS>(gV, ldv, L.bd_T, r, rp, nref, nb, s_z, s_part, s_tot);
+    for (int b = 0; b < nb; b += kFew) vb_chase_back<THREADS, kFew, DEPTH>(L.bd_V2, r, s_z + (size_t)b * rp, rp, nb - b, s_edge);
+    vb_apply_reflectors<THREADS, BATCH, COLS>(gV, ldv, L.bd_T, r, rp, nref, nb, s_z, s_part, s_tot);
     // normalise and file
     for (int b = 0; b < nb; ++b) {
       double n2 = 0.0;
-      for (int i = tid; i < r; i += kVbThreads) n2 = fma(s_z[(size_t)b * rp + i], s_z[(size_t)b * rp + i], n2);
+      for (int i = tid; i < r; i += THREADS) n2 = fma(s_z[(size_t)b * rp + i], s_z[(size_t)b * rp + i], n2);
       n2 = warp_sum(n2);
       __syncthreads();
       if (lane == 0) s_part[w][0] = n2;
       __syncthreads();
       double tot = 0.0;
 #pragma unroll
-      for (int ww = 0; ww < kVbWarps; ++ww) tot += s_part[ww][0];
+      for (int ww = 0; ww < kWarps; ++ww) tot += s_part[ww][0];
       const double inv = tot > 0.0 ? rsqrt(tot) : 0.0;
       float* dst = gShort + (int64_t)(cy + (b0 + b) * n_ctas) * r;
-      for (int i = tid; i < r; i += kVbThreads) dst[i] = (float)(s_z[(size_t)b * rp + i] * inv);
+      for (int i = tid; i < r; i += THREADS) dst[i] = (float)(s_z[(size_t)b * rp + i] * inv);
     }
     __syncthreads();
   }
@@ -410,14 +411,15 @@ size_t vc_smem_bytes() { return (size_t)kVcMaxRp * 5 * sizeof(double); }
 
 // 0 if the kernels got their shared memory
 int sp_configure_eigvec_big() {
-  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbBatch, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch>(kVbHalf)) != cudaSuccess;
-  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<2>(kMaxShort)) != cudaSuccess;
+  int bad = cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbThreads / 2, kVbBatch, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch>(kVbHalf)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbThreads, kVbBatch, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<kVbBatch>(kVbHalf)) != cudaSuccess;
+  bad |= cudaFuncSetAttribute(sp_eigvec_big_kernel<kVbThreads, 2, 8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vb_smem_bytes<2>(kMaxShort)) != cudaSuccess;
   bad |= cudaFuncSetAttribute(sp_eigvec_big_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vc_smem_bytes()) != cudaSuccess;
   if (bad) cudaGetLastError();
   return bad;
 }
 
-void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, cudaStream_t st) {
+void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, int rps, double budget, cudaStream_t st) {
   if (n_big <= 0) return;
   // layers up to a short side of 1024: a four-warp CTA per kept atom (each kernel's CTAs leave the others' layers at once)
   if (rps & 1) sp_eigvec_big_cta_kernel<<<dim3(n_big, kVcCtas), kVcThreads, vc_smem_bytes(), st>>>(d_layers, d_big);
@@ -427,8 +429,13 @@ void launch_sp_eigvec_big(const SpLayer* d_layers, const int* d_big, int n_big, 
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int per = 1;
   while (per < kVbMaxCtas && n_big * per * 2 <= sms) per *= 2;
-  if (rps & 2) sp_eigvec_big_kernel<kVbBatch, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<kVbBatch>(kVbHalf), st>>>(d_layers, d_big);
-  if (rps & 4) sp_eigvec_big_kernel<2, 8><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<2>(kMaxShort), st>>>(d_layers, d_big);
+  // up to a short side of 2048: one atom per CTA where the layer's CTAs are enough for the atoms to expect (the budget, and twice its root)
+  // -- eight warps with twice the registers, eight sweeps of reflectors ahead --, else two at once on sixteen warps (us, one | two at
+  // once: nine layers of 2048 rows at s = 2 1010 | 1183, one of 1100 at 6 448 | 500, ten of 1500 at 8 1325 | 991, 50 of 1200 at 7 2975 | 2580)
+  const bool alone = budget + 2.0 * std::sqrt(budget) + 1.0 <= (double)per;
+  if ((rps & 2) && alone) sp_eigvec_big_kernel<kVbThreads / 2, kVbBatch, 8, 8><<<dim3(n_big, per), kVbThreads / 2, vb_smem_bytes<kVbBatch>(kVbHalf), st>>>(d_layers, d_big);
+  if ((rps & 2) && !alone) sp_eigvec_big_kernel<kVbThreads, kVbBatch, 4, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<kVbBatch>(kVbHalf), st>>>(d_layers, d_big);
+  if (rps & 4) sp_eigvec_big_kernel<kVbThreads, 2, 8, 4><<<dim3(n_big, per), kVbThreads, vb_smem_bytes<2>(kMaxShort), st>>>(d_layers, d_big);
 }
 
 }  // namespace atomo
