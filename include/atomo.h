@@ -292,7 +292,8 @@ int atomo_set_eig_mode(atomo_ctx* ctx, int32_t mode);
  * have that floor.  It costs one more pass over G with twice the Gram matrix's arithmetic.              */
 int atomo_set_sigma_refinement(atomo_ctx* ctx, int32_t min_short_side);
 /* Gram matrix path: 1 (default) = tcgen05 tensor cores: a TF32 hi/lo split for layers with rows <= cols, a short side of at
- * most 1024, a 16-byte aligned base and ld % 4 == 0; 8-bit integer digits (exact sums) for larger short sides, for other
+ * most 1024, a 16-byte aligned base and ld % 4 == 0; 8-bit integer digits (entries to 2^-31 of their vector's largest, products to
+ * about 2^-26 of a typical sum; vectors with entries far above their others take all digit products, or fp32 products) for larger short sides, for other
  * layouts (short side above 16, long side from 192; at most 65536 where the short side is at most 512) and, from 2^26 elements
  * of them in a call, for all layers with a short side of 513 to 1024 (digits of at most 8 GiB per call); the fp32 FMA kernel for the rest.  0 = fp32 FMA
  * kernel always.  The TF32 accumulator truncates: at a short side of 1024 the probabilities then

@@ -537,7 +537,9 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     k_cap_max = std::max(k_cap_max, (int)d.k_cap);
     r_max = std::max(r_max, d.r); rp_max = std::max(rp_max, d.rp);
     const int gt = (d.r + 63) / 64;
-    d.tc = 0; d.gram_split = 1; d.gram_part_len = d.L;
+    d.tc = 0; d.gram_split = 1;
+    d.fma_split = given ? 1 : sp_gram_split(d.r, d.L);
+    d.gram_part_len = sp_gram_part(d.r, d.L);
     const int64_t digits = 4 * (int64_t)d.r * sp_i8_pitch(d.L);
     const bool digits_fit = i8_bytes + digits <= kI8Bytes;
     // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
@@ -555,9 +557,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       i8_bytes += digits;
       i8_layers.push_back(l);
     } else {
-      d.gram_split = given ? 1 : sp_gram_split(d.r, d.L);
-      d.gram_part_len = sp_gram_part(d.r, d.L);
-      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.gram_split; ++c) (d.r > 1024 ? gram_tiles : gram_parts).push_back({l, a, b, c});
+      for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.fma_split; ++c) (d.r > 1024 ? gram_tiles : gram_parts).push_back({l, a, b, c});
     }
     for (int p = 0; p < d.nb / 2; ++p) block_pairs.push_back({l, p, 0, 0});
     row_floats_max = std::max(row_floats_max, d.ldx); steps_max = std::max(steps_max, d.nb - 1);
@@ -746,7 +746,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // the kernels write to the workspace
   SpLayer* d_layers = nullptr; TileRef *d_gram = nullptr, *d_pairs = nullptr, *d_bp = nullptr, *d_chol = nullptr, *d_ref = nullptr, *d_tc = nullptr, *d_i8_prep = nullptr, *d_i8 = nullptr;
   uint8_t* d_maps = nullptr;
-  uint32_t* d_flag = nullptr;
+  uint32_t *d_flag = nullptr, *d_coarse = nullptr;
   ClusterCta* d_ctas = nullptr;
   int* d_big = nullptr;
   ClusterCta* d_band = nullptr;
@@ -809,7 +809,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
         d.gram_part = A.take<float>(d.tc == 1 && d.gram_split > 1
                                         ? (size_t)tt * (tt + 1) / 2 * d.gram_split * sp_tc_tile() * sp_tc_tile() : 0);
       }
-      d.gram_sums = A.take<double>(d.tc == 1 ? 0 : d.tc == 2 ? (size_t)sp_i8_sums(d.r, d.gram_split) : (size_t)sp_gram_sums(d.r, d.gram_split));
+      d.gram_sums = A.take<double>(d.tc == 1 ? 0 : (size_t)std::max(sp_gram_sums(d.r, d.fma_split), d.tc == 2 ? sp_i8_sums(d.r, d.gram_split) : 0));
       d.i8_ld = sp_i8_pitch(d.L);
       d.i8_dig = A.take<int8_t>(d.tc == 2 ? (size_t)4 * d.r * d.i8_ld : 0);
       d.td_d = A.take<double>(d.tri ? d.rp : 0); d.td_e = A.take<double>(d.tri ? d.rp : 0);
@@ -844,12 +844,14 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     for (int l = 0; l < n_layers; ++l) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       const int tf = (L[l].r + 63) / 64;
-      L[l].gram_ticket = A.take<uint32_t>(L[l].gram_split > 1 ? (size_t)(L[l].tc ? tt * (tt + 1) / 2 : tf * (tf + 1) / 2) : 0);
+      L[l].gram_ticket = A.take<uint32_t>(L[l].gram_split > 1 ? (size_t)(tt * (tt + 1) / 2) : 0);
+      L[l].fma_ticket = A.take<uint32_t>(L[l].tc != 1 && L[l].fma_split > 1 ? (size_t)(tf * (tf + 1) / 2) : 0);
     }
     for (int l = 0; l < n_layers; ++l) {
       L[l].i8_max = A.take<uint32_t>(L[l].tc == 2 ? (size_t)L[l].r : 0);
-      L[l].i8_rest = A.take<unsigned long long>(L[l].tc == 2 ? (size_t)L[l].r : 0);
+      L[l].i8_stat = A.take<I8Stat>(L[l].tc == 2 ? (size_t)L[l].r : 0);
     }
+    d_coarse = A.take<uint32_t>(1);
     for (int l = 0; l < n_layers; ++l) L[l].X = A.take<float>(L[l].tri ? 0 : (size_t)L[l].rp * L[l].ldx);
     zero_beg = zb; zero_bytes = A.off - z0;
     for (int l = 0; l < n_layers; ++l) {
@@ -909,7 +911,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if (ctx->eig_mode == 0) launch_sp_init(d_layers, n_layers, nullptr, 0, st);   // the identity half of [A | I]
   launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), (int)gram_parts.size(), st);
   launch_sp_gram_tc(d_layers, d_maps, d_tc, (int)tc_tiles.size(), d_flag + 1, st);
-  launch_sp_gram_i8(d_layers, d_maps, d_i8_prep, (int)i8_rows.size(), (int)i8_prep.size(), d_i8, (int)i8_tiles.size(), d_flag + 1, st);
+  launch_sp_gram_i8(d_layers, d_maps, d_i8_prep, (int)i8_rows.size(), (int)i8_prep.size(), d_i8, (int)i8_tiles.size(), d_flag + 1, d_coarse, st);
+  if (!i8_layers.empty()) launch_sp_gram_coarse(d_layers, n_layers, d_coarse, st);
   launch_sp_scale(d_layers, n_layers, r_max, st);
   }
   if (!given && ctx->eig_mode != 0 && !tri_form) {
@@ -920,7 +923,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   }
   const bool fma_large = gram_tiles.size() > gram_parts.size(), i8_two = i8_prep.size() > i8_rows.size();
   stage_end(ctx, ATOMO_STAGE_GRAM, st, given ? 1 : 2 + (fma_large ? 1 : 0) + (gram_parts.empty() ? 0 : 1) + (tc_tiles.empty() ? 0 : 1) +
-                                           (i8_tiles.empty() ? 0 : 1) + (i8_rows.empty() ? 0 : 1) + (i8_two ? 2 : 0));
+                                           (i8_tiles.empty() ? 0 : 2) + (i8_rows.empty() ? 0 : 1) + (i8_two ? 2 : 0));
   CK(cudaGetLastError());
 
   // ---- S1: eigen-solver; the host reads a convergence flag once per sweep of the largest layer ----

@@ -69,6 +69,15 @@ constexpr int kBandWidth = 8;         // sub-diagonals between the two stages of
 __host__ __device__ inline int64_t sp_chase_row(int r) { return (int64_t)((r + 255) / 256) * 256; }
 constexpr int kSmemRowsMaxRp = 4096;  // largest padded short side the shared-memory Jacobi kernel holds
 
+// what the digits of a short-side vector say of its range (integer Gram kernel; q = the entry in units of 2^(E - 30))
+struct I8Stat {
+  unsigned long long rest;     // what the digit pairs p + q <= 3 lack of the vector's square (signed, in units of 2^16)
+  unsigned long long square;   // sum of the squares of the leading digits (units of 2^(E - 6))
+  unsigned long long counts;   // entries other than zero << 32 | those of them below 2^(E - 9)
+};
+// more than a quarter of the entries that are not zero have fewer than 22 bits: the FMA kernel forms this vector's row of A
+__device__ __forceinline__ bool i8_coarse(const I8Stat& s) { return 4 * (s.counts & 0xffffffffull) > (s.counts >> 32); }
+
 struct SpLayer {
   const float* G; int rows, cols; int64_t ld;
   int r, L, tall;              // short side, long side, rows > cols
@@ -94,14 +103,14 @@ struct SpLayer {
   float* chol_dd;              // 32 x 32 + 32 floats: diagonal block of the current Cholesky panel, published by its owner
   float* dbg_short;            // r x r or nullptr
   int tc;                      // kernel of the Gram matrix: 0 FMA, 1 TF32 on tensor cores, 2 8-bit integers on tensor cores
-  int gram_split;              // Gram matrix: CTAs per output tile (parts of the K range), 1 = no split
+  int gram_split;              // Gram matrix on tensor cores: CTAs per output tile (parts of the K range), 1 = no split
   float* gram_part;            // [tiles][gram_split][128 x 128] partial tiles (column-major) when gram_split > 1
-  int gram_part_len;           // FMA kernel: length of a part of the K range
+  int fma_split, gram_part_len;   // FMA kernel: parts of the K range, length of a part
   double* gram_sums;           // FMA kernel: [tiles][gram_split][16][threads that hold entries] partial tiles; integer kernel: [tiles][gram_split][128 x 128]
-  uint32_t* gram_ticket;       // [tiles] parts finished; zeroed per call
+  uint32_t *gram_ticket, *fma_ticket;   // [tiles] parts finished; zeroed per call
   int8_t* i8_dig; int64_t i8_ld;   // integer kernel: [4][r][i8_ld] digits of the short-side vectors
   uint32_t* i8_max;            // r: bits of the vectors' largest magnitudes; zeroed per call
-  unsigned long long* i8_rest; // r: what the digit pairs taken lack of the vectors' squares; zeroed per call
+  I8Stat* i8_stat;             // r; zeroed per call
   int refine, refine_tiles;    // singular values from the projection norms; tiles along the long side
   float* row_inv;              // rp: 1 / norm of each short-side vector as stored in X
   float* refine_partials;      // [refine_tiles][rp] partial squared norms
@@ -140,6 +149,8 @@ int sp_gram_part(int r, int len);                                // FMA kernel: 
 int sp_gram_split(int r, int len);
 int64_t sp_gram_sums(int r, int split);
 void launch_sp_gram(const SpLayer* d_layers, const TileRef* d_tiles, int n_tiles, int n_parts, cudaStream_t st);
+// behind the integer kernel: the tiles of its layers that hold a vector too wide for its digits (d_coarse: whether there are any)
+void launch_sp_gram_coarse(const SpLayer* d_layers, int n_layers, const uint32_t* d_coarse, cudaStream_t st);
 void launch_sp_scale(const SpLayer* d_layers, int n_layers, int r_max, cudaStream_t st);   // trace, then scaling
 void launch_sp_load_svd(const SpLayer* d_layers, int n_layers, const float* const* d_sigma, const float* const* d_vecs,
                         cudaStream_t st);                                       // a decomposition given by the caller
@@ -219,7 +230,7 @@ void sp_i8_prep_tiles(int r, int len, bool tall, int* short_tiles, int* long_til
 int sp_i8_make_map(void* out_map, const int8_t* digits, int r, int len, int64_t pitch);   // 0 on success
 // d_prep: n_prep tiles, the first n_rows of them of layers by rows
 void launch_sp_gram_i8(const SpLayer* d_layers, const void* d_maps, const TileRef* d_prep, int n_rows, int n_prep, const TileRef* d_tiles, int n_tiles,
-                       uint32_t* d_err, cudaStream_t st);
+                       uint32_t* d_err, uint32_t* d_coarse, cudaStream_t st);
 int sp_bp_rows_per_tile();
 int sp_bp_cols_per_tile();
 int sp_bp_chunk_rows();

@@ -63,13 +63,13 @@ int64_t sp_gram_sums(int r, int split) {
 
 // kParts: short sides up to 1024, whose K range may be cut.  Larger layers have an instance of their own: with the code that adds
 // parts up in the same kernel, the loop took 6.9 ms on two layers of 4096 x 4096, without it 6.5.
+struct GramSmem {
+  __align__(16) float As[kGramK][kGramTile + 4], Bs[kGramK][kGramTile + 4];
+  bool last;
+};
 template <bool kParts>
-__global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict__ layers,
-                                                      const TileRef* __restrict__ tiles) {
-  __shared__ __align__(16) float As[kGramK][kGramTile + 4];
-  __shared__ __align__(16) float Bs[kGramK][kGramTile + 4];
-  const TileRef ref = tiles[blockIdx.x];
-  const SpLayer& L = layers[ref.layer];
+__device__ __forceinline__ void gram_tile(const SpLayer& L, const TileRef& ref, GramSmem& sm) {
+  float (&As)[kGramK][kGramTile + 4] = sm.As, (&Bs)[kGramK][kGramTile + 4] = sm.Bs;
   const int i0 = ref.a * kGramTile, j0 = ref.b * kGramTile;
   const bool diag = ref.a == ref.b;
   const float* __restrict__ G = L.G;
@@ -132,9 +132,8 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
   for (int p = 0; p < 4; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc64[p][q] += (double)acc[p][q];
-  __shared__ bool s_last;
-  if (kParts && L.gram_split > 1) {                           // the last part to finish adds them up, in order
-    const int n_split = L.gram_split;
+  if (kParts && L.fma_split > 1) {                            // the last part to finish adds them up, in order
+    const int n_split = L.fma_split;
     const int gt = (r + kGramTile - 1) / kGramTile, tile = ref.a * gt - ref.a * (ref.a - 1) / 2 + ref.b - ref.a;
     const int side = min((r + 3) / 4, 16), n_t = side * side; // threads whose 4 x 4 entries hold some of the matrix (short sides below 64: not all)
     const bool holds = ty < side && tx < side;
@@ -146,9 +145,9 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
     }
     __threadfence();
     __syncthreads();
-    if (t == 0) s_last = atomicAdd(L.gram_ticket + tile, 1u) == (uint32_t)(n_split - 1);
+    if (t == 0) sm.last = atomicAdd(L.fma_ticket + tile, 1u) == (uint32_t)(n_split - 1);
     __syncthreads();
-    if (!s_last) return;
+    if (!sm.last) return;
     __threadfence();
 #pragma unroll
     for (int e = 0; e < 16; ++e) acc64[e / 4][e % 4] = 0.0;
@@ -170,6 +169,41 @@ __global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict_
         if (!diag) L.A[(int64_t)j * lda + i] = v;
       }
     }
+}
+
+template <bool kParts>
+__global__ void __launch_bounds__(256) sp_gram_kernel(const SpLayer* __restrict__ layers, const TileRef* __restrict__ tiles) {
+  __shared__ GramSmem sm;
+  const TileRef ref = tiles[blockIdx.x];
+  gram_tile<kParts>(layers[ref.layer], ref, sm);
+}
+
+// The integer kernel's layers once more, where a vector's entries span more than its digits hold (i8_coarse): those tiles from fp32 products,
+// over what the integer kernel left there.  Every call with such layers launches it, and nearly always its CTAs read one word and leave:
+// four per SM deal the tiles of all layers among themselves, so that this costs a launch and no more.
+__global__ void __launch_bounds__(256) sp_gram_coarse_kernel(const SpLayer* __restrict__ layers, int n_layers, const uint32_t* __restrict__ coarse) {
+  __shared__ GramSmem sm;
+  if (*coarse == 0u) return;
+  const int t = threadIdx.x, grid = gridDim.x;
+  int turn = 0;                                                // the CTA that the next layer's first tile goes to
+  for (int l = 0; l < n_layers; ++l) {
+    const SpLayer& L = layers[l];
+    if (L.tc != 2) continue;
+    const int gt = (L.r + kGramTile - 1) / kGramTile, n = gt * (gt + 1) / 2 * L.fma_split;
+    for (int q = ((int)blockIdx.x + grid - turn) % grid; q < n; q += grid) {
+      TileRef ref{l, 0, q / L.fma_split, q % L.fma_split};
+      while (ref.b >= gt - ref.a) { ref.b -= gt - ref.a; ++ref.a; }
+      ref.b += ref.a;
+      const int i = (t < kGramTile ? ref.a : ref.b) * kGramTile + t % kGramTile;
+      if (__syncthreads_or(t < 2 * kGramTile && i < L.r && i8_coarse(L.i8_stat[i]))) gram_tile<true>(L, ref, sm);
+      __syncthreads();
+    }
+    turn = (turn + n) % grid;
+  }
+}
+
+void launch_sp_gram_coarse(const SpLayer* d_layers, int n_layers, const uint32_t* d_coarse, cudaStream_t st) {
+  sp_gram_coarse_kernel<<<kGramCtas, 256, 0, st>>>(d_layers, n_layers, d_coarse);
 }
 
 // d_tiles: n_tiles tiles, the last n_parts of them of short sides up to 1024 (or parts of such)

@@ -50,7 +50,7 @@ def test_leading_dimension_and_scales(atomo):
     rows = torch.exp2(torch.randint(-12, 12, (1030, 1), device="cuda", generator=gen).float())
     _check(atomo, (wide * rows).contiguous())                       # every vector has a unit of its own
     wide[7] = 0.0
-    wide[3, 5] = 3.0e4                                              # one entry outweighs its vector
+    wide[3, 5] = 3.0e4                                              # one entry outweighs its vector (how close such rows come: test_gpu_gram_range.py)
     _check(atomo, wide)
 
 
