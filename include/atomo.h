@@ -295,7 +295,7 @@ int atomo_set_sigma_refinement(atomo_ctx* ctx, int32_t min_short_side);
  * most 1024, a 16-byte aligned base and ld % 4 == 0; 8-bit integer digits (entries to 2^-31 of their vector's largest, products to
  * about 2^-26 of a typical sum; vectors with entries far above their others take all digit products, or fp32 products) for larger short sides, for other
  * layouts (short side above 16, long side from 192; at most 65536 where the short side is at most 512) and, from 2^26 elements
- * of them in a call, for all layers with a short side of 513 to 1024 (digits of at most 8 GiB per call); the fp32 FMA kernel for the rest.  0 = fp32 FMA
+ * of them in a call, for all layers with a short side of 513 to 1024 (layers whose digits take up to 8 GiB, one byte per byte of gradient; those of a call share up to 1 GiB, or what the largest layer takes); the fp32 FMA kernel for the rest.  0 = fp32 FMA
  * kernel always.  The TF32 accumulator truncates: at a short side of 1024 the probabilities then
  * sit within about 3e-6 of those of an exact decomposition (the few largest p_i; measured), with the other kernels within
  * about 5e-7.  A caller that needs every draw to agree with an fp64 computation outside a 1e-6 margin takes 0.    */
@@ -332,6 +332,10 @@ int atomo_set_tridiag_ctas(atomo_ctx* ctx, int32_t ctas_per_layer);
  * co-resident CTAs of the band reduction and `chase_clusters` clusters of the bulge chase (-1, the default: no limit).  With 0 of
  * either a batch that needs it takes scheme 2 as on a GPU that cannot place it.                                              */
 int atomo_limit_tridiag_route(atomo_ctx* ctx, int32_t band_ctas, int32_t chase_clusters);
+/* The context's workspace grows to at most `bytes` (-1, the default: no limit; what is allocated already stays).  A spectral encode
+ * that would need more does without the integer digits of its Gram matrices, as beside a GPU that is nearly full; one that needs
+ * more all the same, and any other call, returns ATOMO_ERR_CUDA with nothing launched.                                          */
+int atomo_limit_workspace(atomo_ctx* ctx, int64_t bytes);
 /* The scheme (0 to 3 as above) that the last atomo_encode_spectral() of this context actually ran; -1 before
  * the first call.  Host only.                                                                                */
 int atomo_last_eig_scheme(atomo_ctx* ctx);

@@ -33,7 +33,7 @@ EXPORTS = [
     "atomo_payload_read_headers", "atomo_payload_status", "atomo_set_profiling", "atomo_get_stage_times",
     "atomo_set_eig_params", "atomo_set_eig_mode", "atomo_set_sigma_refinement", "atomo_set_gram_path", "atomo_set_persistent_eig", "atomo_last_eig_scheme", "atomo_decode_spectral_static", "atomo_decode_average", "atomo_lq_budget",
     "atomo_payload_bytes_entrywise_compact", "atomo_set_entrywise_format", "atomo_get_stage_totals",
-    "atomo_set_tridiag_ctas", "atomo_limit_tridiag_route", "atomo_measure_fma_peak", "atomo_encode_spectral_from_svd", "atomo_get_table_uploads",
+    "atomo_set_tridiag_ctas", "atomo_limit_tridiag_route", "atomo_limit_workspace", "atomo_measure_fma_peak", "atomo_encode_spectral_from_svd", "atomo_get_table_uploads",
     "atomo_set_entrywise_launch",
     "atomo_get_entrywise_list_chunks",
 ]
@@ -122,6 +122,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.atomo_last_eig_scheme.argtypes = [vp]
     lib.atomo_set_tridiag_ctas.argtypes = [vp, i32]
     lib.atomo_limit_tridiag_route.argtypes = [vp, i32, i32]
+    lib.atomo_limit_workspace.argtypes = [vp, i64]
     lib.atomo_get_table_uploads.argtypes = [vp, ctypes.POINTER(i64), ctypes.POINTER(i64)]
     lib.atomo_encode_spectral_from_svd.argtypes = [vp, ctypes.POINTER(_Mat), i32, ctypes.POINTER(vp), ctypes.POINTER(vp),
                                                    ctypes.c_double, u64, u64, i32, vp, i64, ctypes.POINTER(_Debug), vp]
@@ -587,6 +588,10 @@ class Atomo:
     def limit_tridiag_route(self, band_ctas: int = -1, chase_clusters: int = -1):
         """Test hook: what the occupancy queries of the two-stage reduction count as at most (-1: as they are)."""
         self._check(self.lib.atomo_limit_tridiag_route(self._h, int(band_ctas), int(chase_clusters)), "atomo_limit_tridiag_route")
+
+    def limit_workspace(self, n_bytes: int = -1):
+        """Most that the context's workspace may grow to (-1: no limit); a spectral encode that needs more does without integer digits."""
+        self._check(self.lib.atomo_limit_workspace(self._h, int(n_bytes)), "atomo_limit_workspace")
 
     def last_eig_scheme(self) -> int:
         return int(self.lib.atomo_last_eig_scheme(self._h))

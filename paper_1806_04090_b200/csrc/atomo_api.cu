@@ -41,6 +41,7 @@ struct atomo_ctx {
   int64_t table_uploads = 0, table_reuses = 0;
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
+  int64_t ws_limit = -1;             // most that the workspace may grow to (-1: no limit)
   uint32_t* h_flag = nullptr;        // pinned: convergence flag / state mirror
   EwLqPart* h_lq = nullptr;          // pinned: results of the l_q sums, written by the GPU
   uint32_t* ew_words = nullptr;      // device: barrier counters of the entry-wise encode (zero between launches), the ticket of the l_q sums
@@ -175,11 +176,24 @@ void table_free(TableCache& tc) {
   tc = TableCache();
 }
 
-int ensure_ws(atomo_ctx* ctx, size_t bytes) {
+// optional: the caller can do with less, so that a workspace that does not fit beside what is allocated already is not even tried
+// (freeing the old one first, and waiting for the device, on every such call)
+int ensure_ws(atomo_ctx* ctx, size_t bytes, bool optional = false) {
   if (bytes <= ctx->ws_bytes) return ATOMO_OK;
+  const size_t limit = ctx->ws_limit < 0 ? SIZE_MAX : (size_t)ctx->ws_limit;
+  size_t free_bytes = 0, all_bytes = 0;
+  if (bytes > limit || (optional && cudaMemGetInfo(&free_bytes, &all_bytes) == cudaSuccess && bytes > free_bytes + ctx->ws_bytes)) {
+    ctx->err = "no room for a workspace of " + std::to_string(bytes) + " bytes";
+    return ATOMO_ERR_CUDA;
+  }
   if (ctx->ws) { CK(cudaDeviceSynchronize()); CK(cudaFree(ctx->ws)); ctx->ws = nullptr; ctx->ws_bytes = 0; }
-  const size_t want = bytes + bytes / 8 + (1 << 20);
-  CK(cudaMalloc(&ctx->ws, want));
+  size_t want = std::min(bytes + bytes / 8 + (1 << 20), limit);
+  cudaError_t e = cudaMalloc(&ctx->ws, want);
+  if (e == cudaErrorMemoryAllocation && want > bytes) {        // without the spare part, then
+    cudaGetLastError();
+    e = cudaMalloc(&ctx->ws, want = bytes);
+  }
+  if (e != cudaSuccess) { cudaGetLastError(); ctx->ws = nullptr; return fail_cuda(ctx, e, "cudaMalloc(workspace)"); }
   ctx->ws_bytes = want;
   return ATOMO_OK;
 }
@@ -300,7 +314,9 @@ int chase_room(atomo_ctx* ctx, int ctas) {
   return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
 constexpr int kI8Short = 16, kI8LongMin = 192, kI8LongMax = 1 << 16;   // shapes below 513 rows that take the integer Gram kernel instead of the FMA kernel
-constexpr int64_t kI8Bytes = (int64_t)1 << 33;                // most that the digits of a call may take beside its gradients (beyond: the other kernels)
+// digits of the integer Gram kernel, as many bytes as their gradients: layers whose own exceed kI8Bytes take the other kernels; the others' are
+// made and used in groups of layers, one behind the other in the same kI8Group bytes (96 layers of 1024 x 4096, two groups: 24 waves of CTAs as in one)
+constexpr int64_t kI8Bytes = (int64_t)1 << 33, kI8Group = (int64_t)1 << 30;
 constexpr int64_t kI8Elements = (int64_t)1 << 26;             // elements from which layers of 513 .. 1024 rows take the integer Gram kernel
 int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
@@ -466,6 +482,12 @@ int atomo_limit_tridiag_route(atomo_ctx* ctx, int32_t band_ctas, int32_t chase_c
   return ATOMO_OK;
 }
 
+int atomo_limit_workspace(atomo_ctx* ctx, int64_t bytes) {
+  if (!ctx || bytes < -1) return ATOMO_ERR_INVALID_ARG;
+  ctx->ws_limit = bytes;
+  return ATOMO_OK;
+}
+
 int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores) {
   if (!ctx) return ATOMO_ERR_INVALID_ARG;
   ctx->tc_gram = tensor_cores != 0;
@@ -485,10 +507,11 @@ int atomo_set_eig_mode(atomo_ctx* ctx, int32_t mode) {
 }
 
 // ==================================================================================================
-static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t n_layers, double s, uint64_t seed,
+// use_digits: whether layers may take the integer Gram kernel; comes back false, with nothing launched, if there is no room for their digits
+static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t n_layers, double s, uint64_t seed,
                                 uint64_t step, int32_t k_cap, void* payload, int64_t capacity_bytes,
                                 const atomo_debug* dbg, void* stream, const float* const* given_sigma,
-                                const float* const* given_short) {
+                                const float* const* given_short, bool& use_digits) {
   const bool given = given_sigma != nullptr;                   // the decomposition comes from the caller: S1 is skipped
   if (!ctx || !layers || n_layers <= 0 || k_cap <= 0 || !payload) return ATOMO_ERR_INVALID_ARG;
   if (bad_budget(s)) return ATOMO_ERR_BUDGET;
@@ -505,7 +528,6 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if ((int64_t)total > capacity_bytes) return ATOMO_ERR_CAPACITY;
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
-  stage_reset(ctx);
   const int max_sweeps = ctx->max_sweeps;
   uint8_t* pay = static_cast<uint8_t*>(payload);
   atomo_layer_header* d_hdr = reinterpret_cast<atomo_layer_header*>(pay + sizeof(atomo_payload_header));
@@ -513,11 +535,15 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // ---- host descriptors, tiles, workspace carving (two passes: size, then pointers) ----
   std::vector<SpLayer> L(n_layers);
   std::vector<int> tc_layers, i8_layers;
-  std::vector<TileRef> gram_tiles, gram_parts, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles, i8_rows, i8_prep, i8_tiles;
+  std::vector<int64_t> i8_at;                                // where a layer's digits start in its group's
+  std::vector<TileRef> gram_tiles, gram_parts, block_pairs, bp_tiles, chol_ctas, refine_tiles, tc_tiles, i8_prep, i8_tiles;
   const int map_bytes = sp_tc_map_bytes();
   std::vector<uint8_t> maps_blob((size_t)n_layers * map_bytes, 0);
   int chol_panels = 0;
-  int64_t i8_bytes = 0;                                      // digits of the layers so far that take the integer Gram kernel
+  // groups of layers that take the integer Gram kernel, by position in i8_layers; what the largest group's digits take
+  struct I8Group { int first, count, prep, n_rows, n_prep, tiles, n_tiles; };
+  std::vector<I8Group> i8_groups;
+  int64_t i8_bytes = 0, i8_room = 0;
   int64_t mid_elements = 0;                                  // of the layers with a short side of 513 .. 1024
   for (int l = 0; l < n_layers; ++l) { const int r = std::min(layers[l].rows, layers[l].cols); if (r > 512 && r <= 1024) mid_elements += (int64_t)layers[l].rows * layers[l].cols; }
   int row_floats_max = 0, steps_max = 0, r_max = 0, rp_max = 0, r_max_tall = 0, k_cap_max = 1;
@@ -541,7 +567,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     d.fma_split = given ? 1 : sp_gram_split(d.r, d.L);
     d.gram_part_len = sp_gram_part(d.r, d.L);
     const int64_t digits = 4 * (int64_t)d.r * sp_i8_pitch(d.L);
-    const bool digits_fit = i8_bytes + digits <= kI8Bytes;
+    const bool digits_fit = use_digits && digits <= kI8Bytes;
     // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
     // kernel, and below those that the TF32 kernel cannot take (FMA | integer with its digits, us: 129 x 4097 76 | 36, 500 x 777 69 | 32, 30 of
@@ -554,7 +580,11 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       tc_layers.push_back(l);
     } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || (d.r > kI8Short && d.L >= kI8LongMin && d.L <= kI8LongMax))) {
       d.tc = 2;
-      i8_bytes += digits;
+      if (i8_groups.empty() || i8_bytes + digits > kI8Group) { i8_groups.push_back({(int)i8_layers.size(), 0, 0, 0, 0, 0, 0}); i8_bytes = 0; }
+      ++i8_groups.back().count;
+      i8_at.push_back(i8_bytes);
+      i8_bytes += (digits + 255) / 256 * 256;
+      i8_room = std::max(i8_room, i8_bytes);
       i8_layers.push_back(l);
     } else {
       for (int a = 0; a < gt; ++a) for (int b = a; b < gt; ++b) for (int c = 0; c < d.fma_split; ++c) (d.r > 1024 ? gram_tiles : gram_parts).push_back({l, a, b, c});
@@ -648,21 +678,27 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       for (int l : which) L[l].gram_split = parts(l, lo);
     };
     split(tc_layers, 16, [&](int l) { return (L[l].L + 31) / 32; }, [](int) { return 1; });
-    // (the integer tiles' sums are exact in any number of parts)
-    split(i8_layers, 8, [&](int l) { return sp_i8_stages(L[l].L); }, [&](int l) { return sp_i8_min_split(L[l].L); });
-    int64_t i8_row_count = 0;                                // (rows per CTA of the digits' kernel: one after the other, eight CTAs per SM)
-    for (int l : i8_layers) if (sp_i8_by_rows(L[l].L, L[l].tall)) i8_row_count += L[l].r;
-    const int row_step = (int)std::min<int64_t>(16, std::max<int64_t>(1, i8_row_count / (8 * sms)));
-    for (int l : i8_layers) {
-      const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
-      for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
-        for (int c = 0; c < L[l].gram_split; ++c) i8_tiles.push_back({l, a, b, c});
-      int na = 0, nb = 0;
-      sp_i8_prep_tiles(L[l].r, L[l].L, L[l].tall, &na, &nb);
-      if (sp_i8_by_rows(L[l].L, L[l].tall)) for (int a = 0; a < na; a += row_step) i8_rows.push_back({l, a, 0, row_step});
-      else for (int a = 0; a < na; ++a) for (int b = 0; b < nb; ++b) i8_prep.push_back({l, a, b, 0});
+    for (I8Group& g : i8_groups) {
+      const std::vector<int> which(i8_layers.begin() + g.first, i8_layers.begin() + g.first + g.count);
+      split(which, 8, [&](int l) { return sp_i8_stages(L[l].L); }, [&](int l) { return sp_i8_min_split(L[l].L); });
+      int64_t i8_row_count = 0;                              // (rows per CTA of the digits' kernel: one after the other, eight CTAs per SM)
+      for (int l : which) if (sp_i8_by_rows(L[l].L, L[l].tall)) i8_row_count += L[l].r;
+      const int row_step = (int)std::min<int64_t>(16, std::max<int64_t>(1, i8_row_count / (8 * sms)));
+      std::vector<TileRef> two_pass;
+      g.prep = (int)i8_prep.size(); g.tiles = (int)i8_tiles.size();
+      for (int l : which) {
+        const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
+        for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
+          for (int c = 0; c < L[l].gram_split; ++c) i8_tiles.push_back({l, a, b, c});
+        int na = 0, nb = 0;
+        sp_i8_prep_tiles(L[l].r, L[l].L, L[l].tall, &na, &nb);
+        if (sp_i8_by_rows(L[l].L, L[l].tall)) for (int a = 0; a < na; a += row_step) i8_prep.push_back({l, a, 0, row_step});
+        else for (int a = 0; a < na; ++a) for (int b = 0; b < nb; ++b) two_pass.push_back({l, a, b, 0});
+      }
+      g.n_rows = (int)i8_prep.size() - g.prep;
+      i8_prep.insert(i8_prep.end(), two_pass.begin(), two_pass.end());
+      g.n_prep = (int)i8_prep.size() - g.prep; g.n_tiles = (int)i8_tiles.size() - g.tiles;
     }
-    i8_prep.insert(i8_prep.begin(), i8_rows.begin(), i8_rows.end());
     for (int l : tc_layers) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       for (int a = 0; a < tt; ++a) for (int b = a; b < tt; ++b)
@@ -788,6 +824,8 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   for (int pass = 0; pass < 2; ++pass) {
     Arena A(pass ? ctx->ws : nullptr);
     d_flag = A.take<uint32_t>(4);
+    int8_t* const digits = A.take<int8_t>((size_t)i8_room);
+    for (size_t q = 0; q < i8_layers.size(); ++q) L[i8_layers[q]].i8_dig = digits + i8_at[q];
     size_t dbg_atoms = 0, dbg_words = 0, dbg_sq = 0;
     for (int l = 0; l < n_layers; ++l) {
       SpLayer& d = L[l];
@@ -811,7 +849,6 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       }
       d.gram_sums = A.take<double>(d.tc == 1 ? 0 : (size_t)std::max(sp_gram_sums(d.r, d.fma_split), d.tc == 2 ? sp_i8_sums(d.r, d.gram_split) : 0));
       d.i8_ld = sp_i8_pitch(d.L);
-      d.i8_dig = A.take<int8_t>(d.tc == 2 ? (size_t)4 * d.r * d.i8_ld : 0);
       d.td_d = A.take<double>(d.tri ? d.rp : 0); d.td_e = A.take<double>(d.tri ? d.rp : 0);
       d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
@@ -861,9 +898,13 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       else { d.A = A.take<float>((size_t)d.r * d.r); d.lda = d.r; }
     }
     need = A.off + 256;
-    if (pass == 0) { const int rc = ensure_ws(ctx, need); if (rc != ATOMO_OK) return rc; }
+    if (pass == 0) {
+      const int rc = ensure_ws(ctx, need, i8_room > 0);
+      if (rc != ATOMO_OK) { use_digits = i8_room == 0; return rc; }
+    }
   }
 
+  stage_reset(ctx);
   // ---- tables (uploaded only if they changed since the last call), headers, zero-filled regions ----
   atomo_payload_header gh{};
   gh.magic = ATOMO_MAGIC; gh.version = ATOMO_VERSION; gh.kind = ATOMO_KIND_SPECTRAL; gh.n_layers = (uint32_t)n_layers;
@@ -911,7 +952,7 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if (ctx->eig_mode == 0) launch_sp_init(d_layers, n_layers, nullptr, 0, st);   // the identity half of [A | I]
   launch_sp_gram(d_layers, d_gram, (int)gram_tiles.size(), (int)gram_parts.size(), st);
   launch_sp_gram_tc(d_layers, d_maps, d_tc, (int)tc_tiles.size(), d_flag + 1, st);
-  launch_sp_gram_i8(d_layers, d_maps, d_i8_prep, (int)i8_rows.size(), (int)i8_prep.size(), d_i8, (int)i8_tiles.size(), d_flag + 1, d_coarse, st);
+  for (const I8Group& g : i8_groups) launch_sp_gram_i8(d_layers, d_maps, d_i8_prep + g.prep, g.n_rows, g.n_prep, d_i8 + g.tiles, g.n_tiles, d_flag + 1, d_coarse, st);
   if (!i8_layers.empty()) launch_sp_gram_coarse(d_layers, n_layers, d_coarse, st);
   launch_sp_scale(d_layers, n_layers, r_max, st);
   }
@@ -921,9 +962,11 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     const int e = launch_sp_cholesky_big(d_layers, d_chol, (int)chol_ctas.size(), chol_panels, st);
     if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchCooperativeKernel(cholesky)");
   }
-  const bool fma_large = gram_tiles.size() > gram_parts.size(), i8_two = i8_prep.size() > i8_rows.size();
+  const bool fma_large = gram_tiles.size() > gram_parts.size();
+  int i8_launches = i8_groups.empty() ? 0 : 1;
+  for (const I8Group& g : i8_groups) i8_launches += 1 + (g.n_rows > 0 ? 1 : 0) + (g.n_prep > g.n_rows ? 2 : 0);
   stage_end(ctx, ATOMO_STAGE_GRAM, st, given ? 1 : 2 + (fma_large ? 1 : 0) + (gram_parts.empty() ? 0 : 1) + (tc_tiles.empty() ? 0 : 1) +
-                                           (i8_tiles.empty() ? 0 : 2) + (i8_rows.empty() ? 0 : 1) + (i8_two ? 2 : 0));
+                                           i8_launches);
   CK(cudaGetLastError());
 
   // ---- S1: eigen-solver; the host reads a convergence flag once per sweep of the largest layer ----
@@ -1060,6 +1103,17 @@ static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     if (ctx->h_flag[2] != 0) { ctx->err = "a step barrier of the persistent eigen-solve ran out of polls"; return ATOMO_ERR_TIMEOUT; }
   }
   return ATOMO_OK;
+}
+
+static int encode_spectral_impl(atomo_ctx* ctx, const atomo_mat* layers, int32_t n_layers, double s, uint64_t seed,
+                                uint64_t step, int32_t k_cap, void* payload, int64_t capacity_bytes,
+                                const atomo_debug* dbg, void* stream, const float* const* given_sigma,
+                                const float* const* given_short) {
+  bool use_digits = true;
+  const int rc = encode_spectral_with(ctx, layers, n_layers, s, seed, step, k_cap, payload, capacity_bytes, dbg, stream, given_sigma, given_short, use_digits);
+  if (use_digits) return rc;
+  // beside a nearly full GPU: the Gram kernels that need no digits
+  return encode_spectral_with(ctx, layers, n_layers, s, seed, step, k_cap, payload, capacity_bytes, dbg, stream, given_sigma, given_short, use_digits);
 }
 
 int atomo_encode_spectral(atomo_ctx* ctx, const atomo_mat* layers, int32_t n_layers, double s, uint64_t seed,
