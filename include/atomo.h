@@ -294,11 +294,13 @@ int atomo_set_sigma_refinement(atomo_ctx* ctx, int32_t min_short_side);
 /* Gram matrix path: 1 (default) = tcgen05 tensor cores: a TF32 hi/lo split for layers with rows <= cols, a short side of at
  * most 1024, a 16-byte aligned base and ld % 4 == 0; 8-bit integer digits (entries to 2^-31 of their vector's largest, products to
  * about 2^-26 of a typical sum; vectors with entries far above their others take all digit products, or fp32 products) for larger short sides, for other
- * layouts (short side above 16, long side from 192; at most 65536 where the short side is at most 512) and, from 2^26 elements
+ * layouts (short side above 16 and a long side of a few hundred to 65536, the more layers of up to 64 rows in the call the longer) and, from 2^26 elements
  * of them in a call, for all layers with a short side of 513 to 1024 (layers whose digits take up to 8 GiB, one byte per byte of gradient; those of a call share up to 1 GiB, or what the largest layer takes); the fp32 FMA kernel for the rest.  0 = fp32 FMA
  * kernel always.  The TF32 accumulator truncates: at a short side of 1024 the probabilities then
  * sit within about 3e-6 of those of an exact decomposition (the few largest p_i; measured), with the other kernels within
- * about 5e-7.  A caller that needs every draw to agree with an fp64 computation outside a 1e-6 margin takes 0.    */
+ * about 5e-7.  A caller that needs every draw to agree with an fp64 computation outside a 1e-6 margin takes 0.
+ * Which kernel a layer takes, and in how many parts it sums, may depend on the other layers of the call, and with them the last
+ * digits of its singular values and vectors; the same call yields the same payload.                                          */
 int atomo_set_gram_path(atomo_ctx* ctx, int32_t tensor_cores);
 /* Eigen-solver scheme (`enabled` = 0, 1, 2 or 3):
  * 3 (default) = the tridiagonal routes: the scaled Gram matrix of every layer is reduced to tridiagonal form by

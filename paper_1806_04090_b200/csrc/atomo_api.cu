@@ -313,7 +313,24 @@ int chase_room(atomo_ctx* ctx, int ctas) {
   if (known < 0) known = sp_chase_capacity(ctas);
   return ctx->chase_limit >= 0 && ctas > 1 ? std::min(known, ctx->chase_limit) : known;
 }
-constexpr int kI8Short = 16, kI8LongMin = 192, kI8LongMax = 1 << 16;   // shapes below 513 rows that take the integer Gram kernel instead of the FMA kernel
+// Layers of up to 512 rows that the TF32 kernel cannot take: integer Gram kernel, or FMA kernel.  `narrow`: how many of them in the call have
+// up to 64 rows (one tile of either kernel).  The integer kernel costs two or three launches more and a CTA of 10 us per tile, the FMA kernel a walk
+// along the long side on one CTA up to 512 columns, on several from there.  A whole encode, FMA | integer, us:
+//   one layer: 17 x 193 95 | 99, 64 x 257 163 | 163, 17 x 321 103 | 99, 128 x 321 268 | 259, 17 x 513 119 | 98; tall 321 x 180 375 | 380, 401 x 128 274 | 268,
+//   401 x 64 170 | 172, 449 x 64 174 | 173
+//   20 layers: 48 x 257 149 | 153, 48 x 353 157 | 154; 50: 17 x 401 117 | 122, 17 x 513 133 | 123, 64 x 513 201 | 190
+//   100 layers: 128 x 321 774 | 769, 33 x 449 190 | 205, 33 x 513 216 | 212, 17 x 1201 180 | 208, 17 x 2401 204 | 208; tall 801 x 64 340 | 332,
+//   1601 x 64 415 | 431
+//   200 layers (the host's part of the call bounds the narrow ones): 33 x 801 334 | 362, 64 x 801 487 | 498, 64 x 1201 540 | 536, 17 x 2401 331 | 371,
+//   33 x 2401 463 | 406, 17 x 5001 489 | 376; 600: 17 x 2401 986 | 1068, 64 x 801 1234 | 1275, 64 x 2401 1602 | 1525
+// The longest keep the FMA kernel's bounded number of parts.
+bool i8_small(int r, int L, bool tall, int narrow) {
+  if (r <= 16 || L > 1 << 16) return false;
+  if (r > 64) return L >= (tall ? 400 : 320);
+  if (narrow <= 32) return L >= (tall ? 448 : 320);
+  if (narrow <= (r > 32 ? 128 : 64)) return L >= 512;
+  return r * L >= 1 << 16;
+}
 // digits of the integer Gram kernel, as many bytes as their gradients: layers whose own exceed kI8Bytes take the other kernels; the others' are
 // made and used in groups of layers, one behind the other in the same kI8Group bytes (96 layers of 1024 x 4096, two groups: 24 waves of CTAs as in one)
 constexpr int64_t kI8Bytes = (int64_t)1 << 33, kI8Group = (int64_t)1 << 30;
@@ -545,7 +562,13 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   std::vector<I8Group> i8_groups;
   int64_t i8_bytes = 0, i8_room = 0;
   int64_t mid_elements = 0;                                  // of the layers with a short side of 513 .. 1024
-  for (int l = 0; l < n_layers; ++l) { const int r = std::min(layers[l].rows, layers[l].cols); if (r > 512 && r <= 1024) mid_elements += (int64_t)layers[l].rows * layers[l].cols; }
+  int narrow = 0;                                            // see i8_small()
+  for (int l = 0; l < n_layers; ++l) {
+    const atomo_mat& m = layers[l];
+    const int r = std::min(m.rows, m.cols);
+    if (r > 512 && r <= 1024) mid_elements += (int64_t)m.rows * m.cols;
+    if (r > 16 && r <= 64 && !sp_tc_eligible(m.data, m.rows, m.cols, m.ld)) ++narrow;
+  }
   int row_floats_max = 0, steps_max = 0, r_max = 0, rp_max = 0, r_max_tall = 0, k_cap_max = 1;
   for (int l = 0; l < n_layers; ++l) {
     SpLayer& d = L[l];
@@ -570,15 +593,13 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     const bool digits_fit = use_digits && digits <= kI8Bytes;
     // The TF32 kernel's fp32 accumulation truncates, which perturbs sum(sigma) -- and with it the largest p_i -- by a few
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
-    // kernel, and below those that the TF32 kernel cannot take (FMA | integer with its digits, us: 129 x 4097 76 | 36, 500 x 777 69 | 32, 30 of
-    // 400 x 2001 625 | 168, 16384 x 18 145 | 70, 33 x 257 21 | 16, 64 x 65 9 | 23, hence the least length; the longest keep the FMA kernel's
-    // bounded number of parts), or of 513 to 1024 rows all where they are many (TF32 |
+    // kernel, and below those that the TF32 kernel cannot take (i8_small), or of 513 to 1024 rows all where they are many (TF32 |
     // integer, us: 20 layers of 1000 x 1200 241 | 259, one of 1024 x 4096 51 | 64, 40 of 520 x 8000 1081 | 767, 96 of 1024 x 4096 2818 | 2185)
     if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && (mid_elements < kI8Elements || !digits_fit))) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
       d.tc = 1;
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
-    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || (d.r > kI8Short && d.L >= kI8LongMin && d.L <= kI8LongMax))) {
+    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || i8_small(d.r, d.L, d.tall, narrow))) {
       d.tc = 2;
       if (i8_groups.empty() || i8_bytes + digits > kI8Group) { i8_groups.push_back({(int)i8_layers.size(), 0, 0, 0, 0, 0, 0}); i8_bytes = 0; }
       ++i8_groups.back().count;
