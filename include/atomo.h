@@ -13,7 +13,9 @@
  *   - Every pointer marked DEVICE is a CUDA device pointer owned by the caller; arrays of
  *     descriptors (atomo_mat, atomo_vec, pointer lists, shape lists) are HOST memory and are
  *     consumed before the call returns.
- *   - All work is enqueued on `stream` (a cudaStream_t passed as void*; NULL = default stream).
+ *   - All work is ordered on `stream` (a cudaStream_t passed as void*; NULL = default stream): a spectral encode of small and
+ *     large layers together puts some of it on a stream of the context, of the same priority, which forks from `stream` and joins
+ *     it again within the call.
  *     atomo_encode_spectral on the tridiagonal routes (eigen scheme 3, the default) never
  *     waits on the host: a bounded device-side wait that ran out shows as ATOMO_ERR_TIMEOUT in the layers' status
  *     words.  On the Jacobi routes it waits once, after it has enqueued all its work (the kernels' bounded waits

@@ -63,7 +63,9 @@ struct atomo_ctx {
   int refine_min_short = 2048;       // layers with at least this short side get the sigma refinement pass
   bool tc_gram = true;               // Gram matrix on tcgen05 where the layer's layout allows it
   bool tc_ok = false;                // tensor-map entry point found
-  cudaStream_t side = nullptr;       // work beside the call's stream, which forks it and joins it again inside the call
+  // work beside the call's stream, which forks it and joins it again inside the call: a stream per priority that calls came with, since a
+  // caller's work must not wait for less urgent work of others on its side stream
+  std::vector<std::pair<int, cudaStream_t>> sides;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int eig_scheme = 3;                // eigen-solve: 0 = Jacobi, one launch per step, 1 = persistent (cooperative), 2 = clusters first, 3 = tridiagonal route first
   int tri_clusters = -1;             // co-resident clusters of the tridiagonal reduction (-1 = not asked yet, 0 = unavailable)
@@ -337,6 +339,18 @@ constexpr int64_t kI8Bytes = (int64_t)1 << 33, kI8Group = (int64_t)1 << 30;
 constexpr int64_t kI8Elements = (int64_t)1 << 26;             // elements from which layers of 513 .. 1024 rows take the integer Gram kernel
 int chase_class(int r) { return r <= 1024 ? 1024 : r <= 2048 ? 2048 : 4096; }   // short sides that share a form of the chase
 
+// the context's side stream with the priority of st
+int side_stream(atomo_ctx* ctx, cudaStream_t st, cudaStream_t* out) {
+  int priority = 0;
+  CK(cudaStreamGetPriority(st, &priority));
+  for (auto& q : ctx->sides) if (q.first == priority) { *out = q.second; return ATOMO_OK; }
+  cudaStream_t s = nullptr;
+  CK(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, priority));
+  ctx->sides.emplace_back(priority, s);
+  *out = s;
+  return ATOMO_OK;
+}
+
 bool bad_budget(double s) { return !(s > 0.0) || !std::isfinite(s); }
 
 }  // namespace
@@ -359,7 +373,6 @@ int atomo_create(atomo_ctx** out, int device) {
   if (e == 0) e = ew_configure();
   if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaFuncSetAttribute(max dynamic shared memory)");
   ctx->tc_ok = sp_tc_configure() == 0;
-  CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
   ctx->configured = true;
@@ -370,7 +383,7 @@ int atomo_destroy(atomo_ctx* ctx) {
   if (!ctx) return ATOMO_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
-  if (ctx->side) cudaStreamDestroy(ctx->side);
+  for (auto& q : ctx->sides) cudaStreamDestroy(q.second);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->ws) cudaFree(ctx->ws);
@@ -998,6 +1011,8 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   // Persistent form: the block pairs of a group of whole layers are co-resident (one CTA per SM) and solve their
   // layers in one cooperative launch.  A batch larger than the GPU is cut into such groups, launched one after
   // the other; a single layer with more block pairs than the GPU holds CTAs falls back to one launch per step.
+  cudaStream_t side = nullptr;
+  if (tri_form && any_small && any_big) { const int rc = side_stream(ctx, st, &side); if (rc != ATOMO_OK) return rc; }
   if (tri_form) {
     // small layers beside larger ones: their reduction (0.5 to 0.7 ms on up to 96 SMs) runs on a stream of the context's own next to the
     // chase, which leaves most of the GPU idle; the call's stream waits for it before the eigenvalues
@@ -1023,9 +1038,9 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       ++n_eig_launch;
     }
     if (beside) {                                                    // (behind the chase in the order of launches: the longer one first)
-      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
-      const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, d_flag + 1, ctx->side);
-      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+      CK(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
+      const int e = launch_sp_tridiag(d_layers, d_ctas, n_clusters, d_flag + 1, side);
+      CK(cudaEventRecord(ctx->ev_join, side));
       CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
       if (e != 0) return fail_cuda(ctx, (cudaError_t)e, "cudaLaunchKernelEx(tridiagonal reduction)");
       ++n_eig_launch;
@@ -1104,9 +1119,9 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   if (tri_form) {                                                   // short-side vectors of the kept atoms
     if (any_small && any_big) {                                     // both kinds side by side, as their reductions
       CK(cudaEventRecord(ctx->ev_fork, st));
-      CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
-      launch_sp_eigvec(d_layers, n_layers, rp_max_small, ctx->side);
-      CK(cudaEventRecord(ctx->ev_join, ctx->side));
+      CK(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
+      launch_sp_eigvec(d_layers, n_layers, rp_max_small, side);
+      CK(cudaEventRecord(ctx->ev_join, side));
     } else if (any_small) launch_sp_eigvec(d_layers, n_layers, rp_max_small, st);
     int rps = 0;
     for (int l : big_layers) rps |= L[l].rp <= 1024 ? 1 : L[l].rp <= 2048 ? 2 : 4;

@@ -58,3 +58,34 @@ def test_replay_from_a_graph():
         assert torch.equal(buf, want)
     del graph
     a.close()
+
+
+@pytest.mark.parametrize("priority", [0, -1])
+def test_side_stream_has_the_callers_priority(priority):
+    from cuda.bindings import runtime as rt
+    G = _layers()
+    a = api.Atomo(0)
+    buf = torch.zeros(api.payload_bytes_spectral([tuple(g.shape) for g in G], 24), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream(priority=priority)
+    other = torch.cuda.Stream(priority=-1 - priority)
+    for st in (stream, other):                         # the context has seen calls of either kind (tables: see above)
+        st.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(st):
+            a.atomo_encode_spectral(G, 3.0, seed=9, step=2, k_cap=24, payload=buf)
+        torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=stream):
+        a.atomo_encode_spectral(G, 3.0, seed=9, step=2, k_cap=24, payload=buf)
+    raw = rt.cudaGraph_t(init_value=graph.raw_cuda_graph())
+    err, _, n = rt.cudaGraphGetNodes(raw, 0)
+    err, nodes, n = rt.cudaGraphGetNodes(raw, n)
+    seen = []
+    for node in nodes[:n]:
+        err, kind = rt.cudaGraphNodeGetType(node)
+        if kind == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel:
+            err, value = rt.cudaGraphKernelNodeGetAttribute(node, rt.cudaLaunchAttributeID.cudaLaunchAttributePriority)
+            assert err == rt.cudaError_t.cudaSuccess
+            seen.append(value.priority)
+    assert len(seen) >= 10 and set(seen) == {stream.priority}
+    del graph
+    a.close()
