@@ -325,9 +325,11 @@ int chase_room(atomo_ctx* ctx, int ctas) {
 //   1601 x 64 415 | 431
 //   200 layers (the host's part of the call bounds the narrow ones): 33 x 801 334 | 362, 64 x 801 487 | 498, 64 x 1201 540 | 536, 17 x 2401 331 | 371,
 //   33 x 2401 463 | 406, 17 x 5001 489 | 376; 600: 17 x 2401 986 | 1068, 64 x 801 1234 | 1275, 64 x 2401 1602 | 1525
-// The longest keep the FMA kernel's bounded number of parts.
-bool i8_small(int r, int L, bool tall, int narrow) {
+// beside: other layers of the call take the integer kernel, so that a few short ones cost it next to nothing, and the FMA kernel a launch of its own
+// (116 x 261 beside 789 x 1195 and 512 x 513, Gram stage: 147 | 125).  The longest keep the FMA kernel's bounded number of parts.
+bool i8_small(int r, int L, bool tall, int narrow, bool beside) {
   if (r <= 16 || L > 1 << 16) return false;
+  if (beside && narrow <= 32) return L >= 192;
   if (r > 64) return L >= (tall ? 400 : 320);
   if (narrow <= 32) return L >= (tall ? 448 : 320);
   if (narrow <= (r > 32 ? 128 : 64)) return L >= 512;
@@ -575,12 +577,22 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
   std::vector<I8Group> i8_groups;
   int64_t i8_bytes = 0, i8_room = 0;
   int64_t mid_elements = 0;                                  // of the layers with a short side of 513 .. 1024
-  int narrow = 0;                                            // see i8_small()
+  int narrow = 0;
+  bool beside = false;                                       // see i8_small()
   for (int l = 0; l < n_layers; ++l) {
     const atomo_mat& m = layers[l];
     const int r = std::min(m.rows, m.cols);
     if (r > 512 && r <= 1024) mid_elements += (int64_t)m.rows * m.cols;
     if (r > 16 && r <= 64 && !sp_tc_eligible(m.data, m.rows, m.cols, m.ld)) ++narrow;
+  }
+  auto tf32 = [&](const atomo_mat& m, bool fits) {
+    const int r = std::min(m.rows, m.cols);
+    return (r <= 512 || (r <= 1024 && (mid_elements < kI8Elements || !fits))) && sp_tc_eligible(m.data, m.rows, m.cols, m.ld);
+  };
+  for (int l = 0; l < n_layers && !beside; ++l) {
+    const atomo_mat& m = layers[l];
+    const int r = std::min(m.rows, m.cols);
+    beside = !tf32(m, true) && (r > 512 || i8_small(r, std::max(m.rows, m.cols), m.rows > m.cols, narrow, false));
   }
   int row_floats_max = 0, steps_max = 0, r_max = 0, rp_max = 0, r_max_tall = 0, k_cap_max = 1;
   for (int l = 0; l < n_layers; ++l) {
@@ -608,11 +620,11 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     // 1e-6 at a short side of 1024 and more above (measured 6e-6 at 4096): layers with a short side above 1024 take the integer
     // kernel, and below those that the TF32 kernel cannot take (i8_small), or of 513 to 1024 rows all where they are many (TF32 |
     // integer, us: 20 layers of 1000 x 1200 241 | 259, one of 1024 x 4096 51 | 64, 40 of 520 x 8000 1081 | 767, 96 of 1024 x 4096 2818 | 2185)
-    if (ctx->tc_gram && ctx->tc_ok && !d.acc && (d.r <= 512 || (d.r <= 1024 && (mid_elements < kI8Elements || !digits_fit))) && sp_tc_eligible(d.G, d.rows, d.cols, d.ld)) {
+    if (ctx->tc_gram && ctx->tc_ok && !d.acc && tf32(m, digits_fit)) {
       d.tc = 1;
       if (sp_tc_make_map(maps_blob.data() + (size_t)l * map_bytes, d.G, d.rows, d.cols, d.ld) != 0) return ATOMO_ERR_INVALID_ARG;
       tc_layers.push_back(l);
-    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || i8_small(d.r, d.L, d.tall, narrow))) {
+    } else if (ctx->tc_gram && ctx->tc_ok && !d.acc && !given && digits_fit && (d.r > 512 || i8_small(d.r, d.L, d.tall, narrow, beside))) {
       d.tc = 2;
       if (i8_groups.empty() || i8_bytes + digits > kI8Group) { i8_groups.push_back({(int)i8_layers.size(), 0, 0, 0, 0, 0, 0}); i8_bytes = 0; }
       ++i8_groups.back().count;

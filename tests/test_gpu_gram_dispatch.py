@@ -34,3 +34,22 @@ def test_kernel_by_size_and_number(r, length, count, rows, tall):
             # rounding A's entries to fp32 moves an eigenvalue by at most 2^-24 ||A||_F; the reduction and the sums by as much again, each
             assert np.abs(s ** 2 - lam).max() <= 4.0 * 2.0 ** -24 * np.linalg.norm(lam)
     a.close()
+
+
+# short layers go along where others take the integer kernel; many narrow ones do not
+@pytest.mark.parametrize("shape,count,launches", [((150, 193), 1, ROWS), ((150, 191), 1, ROWS + 1), ((33, 193), 32, ROWS), ((33, 191), 32, ROWS + 1), ((33, 193), 33, ROWS + 1),
+                                                  ((90, 193), 40, ROWS), ((16, 301), 1, ROWS + 1)])
+def test_short_layers_beside_others(shape, count, launches):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(sum(shape))
+    short, large = (torch.randn(*s, device="cuda", generator=gen) for s in (shape, (513, 701)))
+    a = api.Atomo(0)
+    a.set_profiling(True)
+    pay, dbg = a.atomo_encode_spectral([large] + [short] * count, 2.0, seed=3, step=0, k_cap=16, debug=True)
+    assert a.stage_times()[1]["gram"] == launches
+    assert all(h.status == 0 for h in pay.headers()[1])
+    for l, G in ((0, large), (1, short), (count, short)):
+        lam = torch.linalg.svdvals(G.double()).cpu().numpy() ** 2
+        s = dbg.layer_sigma(l, min(G.shape)).astype(np.float64)
+        assert np.abs(s ** 2 - lam).max() <= 4.0 * 2.0 ** -24 * np.linalg.norm(lam)
+    a.close()
