@@ -15,13 +15,11 @@ def atomo():
     a.close()
 
 
-# one CTA per atom and to spare; more atoms than CTAs although one each is expected (k varies); several atoms per CTA from the start
-@pytest.mark.parametrize("m,n,count,s", [(1025, 1030, 1, 5.0), (2047, 2048, 1, 8.0), (1100, 1200, 9, 3.0), (1100, 1200, 40, 6.0), (2048, 2060, 1, 60.0)])
-def test_vectors_of_either_form(atomo, m, n, count, s):
+def _check_vectors(atomo, m, n, count, s, seed, step):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(m + count)
     G = torch.randn(m, n, device="cuda", generator=gen)
-    pay, _ = atomo.atomo_encode_spectral([G] * count, s, 6, step=1, k_cap=128)
+    pay, _ = atomo.atomo_encode_spectral([G] * count, s, seed, step=step, k_cap=128)
     hdrs = pay.headers()
     A = G.double() @ G.double().T
     top = float(torch.linalg.eigvalsh(A)[-1])
@@ -41,3 +39,17 @@ def test_vectors_of_either_form(atomo, m, n, count, s):
         dots = U.T @ U
         assert float((dots - torch.eye(k, device="cuda")).abs().max()) <= 4e-7
     assert seen > 0
+    return [h.k for h in hdrs[1]]
+
+
+# one CTA per atom and to spare; several atoms per CTA from the start
+@pytest.mark.parametrize("m,n,count,s", [(1025, 1030, 1, 5.0), (2047, 2048, 1, 8.0), (1100, 1200, 9, 3.0), (1100, 1200, 40, 6.0), (2048, 2060, 1, 60.0)])
+def test_vectors_of_either_form(atomo, m, n, count, s):
+    _check_vectors(atomo, m, n, count, s, 6, 1)
+
+
+# a CTA per atom is expected (16 per layer for a budget of 9), and some layer keeps more atoms than that
+@pytest.mark.parametrize("m,n,step", [(1100, 1200, 26), (1601, 1700, 19)])
+def test_more_atoms_than_were_expected(atomo, m, n, step):
+    kept = _check_vectors(atomo, m, n, 9, 9.0, 6, step)
+    assert max(kept) > 16, kept
