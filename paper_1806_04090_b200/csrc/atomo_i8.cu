@@ -27,8 +27,9 @@
 // fp32 and the reduction, common to both); 1024 x 4096, TF32 kernel | this one: 1.35e-7 | 2.9e-8.  The TF32 kernel's accumulator
 // truncates, which is why the larger layers never took it.
 // An accumulator holds parts of up to 32768 columns (at most 49408 per column in magnitude, 2^31 in all).  A tile's columns are split
-// over several CTAs while the GPU has SMs left; the parts are integers, so that their sum does not depend on the split (the pass
-// ahead rounds its sum to weight 3 once per part: there the last bit of an entry of A may).
+// over several CTAs while the GPU has SMs left; the parts are integers of up to 2^36 per column, so that up to 131072 columns their sum in fp64 is exact and
+// does not depend on the split (the pass ahead rounds its sum to weight 3 once per part: there the last bit of an entry of A may).
+// Longer layers' parts are added with fp64 rounding, in their order: 2^-53 of the sum.
 //
 // One CTA per 128 x 128 tile of the upper triangle, all 512 columns of the tensor memory.
 //   warp 0      TMA producer: 64 columns of 128 vectors, four digits (32 KB a side, 64-byte swizzle), no multicast
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(kI8Threads, 1) sp_gram_i8_kernel(const SpLayer
       }
     }
     bool write_tile = ok;
-    if (ok && n_split > 1) {                                   // the last part to finish adds them up (integers: exact)
+    if (ok && n_split > 1) {                                   // the last part to finish adds them up, in order
       __threadfence();
       asm volatile("bar.sync 2, 128;" ::: "memory");
       if (tid == 64) *s_last = atomicAdd(L.gram_ticket + tile_id, 1u) == (uint32_t)(n_split - 1) ? 1u : 0u;

@@ -41,6 +41,19 @@ def test_edges(atomo, m, n):
     _check(atomo, torch.randn(m, n, device="cuda", generator=gen))
 
 
+@pytest.mark.parametrize("n", [131072, 150001])
+def test_parts_whose_sum_outgrows_53_bits(atomo, n):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    G = torch.randn(514, n, device="cuda", generator=gen)
+    G[:, : n // 2] *= 0.001
+    G[3] = G[2]                                                     # sums as large as the diagonal's off it
+    status, s = _sigma(atomo, torch.empty(514, n + 1, device="cuda")[:, 1:].copy_(G))
+    assert status == 0
+    lam = torch.linalg.eigvalsh(G.double() @ G.double().T).flip(0).cpu().numpy()
+    assert np.abs(s ** 2 - lam).max() <= 4.0 * 2.0 ** -24 * np.linalg.norm(lam)
+
+
 def test_leading_dimension_and_scales(atomo):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(1)
