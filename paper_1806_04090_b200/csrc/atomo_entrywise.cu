@@ -840,9 +840,9 @@ __device__ __forceinline__ int ew_vec_of(const EwVec (&vecs)[N], const int n, co
 // [code bytes of the chunk] [list form: prefix words].  A chunk of at most kEwRegTiles tiles keeps its entries in
 // registers and draws its words before the barrier: nothing is read twice and no list is kept.
 // kForm: what the chunks of the launch are, where they are all of one kind (64 registers hold any one of the kinds, but for the code of
-// all of them together a chunk's entries were spilled); kMixed asks each chunk.  Spilled bytes 368 | 76 .. 136; a pass,
-// us, one instance for all | by kind: 20 k elements 18.4 | 16.4, 1.5 M 23.8 | 21.9, 4 M at 10 % 45.0 | 43.0, 100 M at 10 % 343 | 338, 25.6 M by QSGD's budget
-// 109.6 | 106.5, three short vectors 20.3 | 18.6.
+// all of them together a chunk's entries were spilled); kMixed asks each chunk.  Spilled bytes 368 | 76 .. 136 for one vector, 504 | 76
+// for several (of different kinds: a network's layers still take the first).  An encode, us, one instance for all | by kind: 100 k elements 14.5 | 13.4, 600 k
+// 18.5 | 17.5, 1.5 M 18.8 | 17.3, 30 M at 10 % 75.8 | 72.5; within 3 % of each other: 3 M and 100 M at 10 %, 25.6 M, 60 M and 200 M at 1 % and less.
 enum { kMixed, kRegisters, kCandidates, kBigList };
 template <int N, int kForm>
 __global__ void __launch_bounds__(kEwThreads, 1) ew_encode_kernel(const __grid_constant__ EwBatch<N> B) {

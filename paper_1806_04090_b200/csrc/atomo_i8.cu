@@ -38,9 +38,9 @@
 // Every mbarrier wait is bounded; a wait that runs out sets an error word and the CTA leaves through the common exit (TMEM is freed).
 // Bound: the tensor cores (1430 cycles per stage of 64 columns, 1280 of them twenty MMAs of 128 x 128 x 32), and the last wave of CTAs
 // (1056 tiles of two layers of 4096 rows on 148 SMs).  Before (fp32 FMA kernel, or TF32) | now with the digits, us: two layers of
-// 4096 x 4096 6390 | 593, nine of 2048 x 2048 3646 | 429, 20 of 1000 x 1201 1174 | 260, 96 of 1024 x 4096 2818 | 2185.  The sums' way out
+// 4096 x 4096 6390 | 593, nine of 2048 x 2048 3646 | 429, 20 of 1000 x 1201 1174 | 260, 96 of 1024 x 4096 2818 | 2230.  The sums' way out
 // of the tensor memory took 31 k cycles per tile with 64-bit integer conversions and a store per entry and row, a third of that now.
-// The vectors' ranges cost the preparing kernel 3 % (96 layers 598 -> 616 us): the digits' squares and products by __dp4a on the words
+// The vectors' ranges and the second group cost 5 % (96 layers: digits 595 -> 645 us, this kernel 1523 -> 1586): the digits' squares and products by __dp4a on the words
 // that are written anyway (40 % with integer arithmetic per entry).
 #include <algorithm>
 
