@@ -727,7 +727,7 @@ __global__ void __launch_bounds__(kFinishThreads) sp_finish_atoms_kernel(const S
   }
   __syncthreads();
   const float sg = s_sg;
-  const float inv = sg > 0.f ? 1.0f / sg : 0.f;
+  const float inv = sg >= 1.17549435e-38f ? 1.0f / sg : 0.f;               // (a subnormal norm has no reciprocal: as zero)
   for (int j = threadIdx.x; j < len; j += kFinishThreads) out[j] *= inv;   // each thread rescales what it wrote itself
 }
 

@@ -68,3 +68,17 @@ def test_downstream_of_a_library_svd_at_1024(atomo, oracle):
     G = synth.c5_stress_layer(0, 0)
     U, sigma, Vt = np.linalg.svd(G.astype(np.float64), full_matrices=False)
     assert _downstream(atomo, oracle, G, U, sigma, Vt.T, 4.0, 11, 2, "1024 x 4096") == 1
+
+
+def test_atom_of_subnormal_norm(atomo):
+    """A given vector that meets the layer's rows in a subnormal entry only: its atom contributes nothing, and nothing that is not finite."""
+    import torch
+    G = torch.zeros(8, 64, device="cuda")
+    G[0] = torch.linspace(-2.0, 2.0, 64, device="cuda")
+    short = torch.eye(8, device="cuda")
+    short[1:, 0] = 1.0e-41
+    pay, _ = atomo.atomo_encode_spectral_from_svd([G], [torch.full((8,), 1.0, device="cuda")], [short], 8.0, 3, step=1, k_cap=8)
+    assert pay.headers()[1][0].status == 0 and pay.headers()[1][0].k == 8
+    assert np.isfinite(pay.layer_arrays(0)["V"]).all()
+    out = atomo.atomo_decode(pay)[0]
+    assert float((out - G).abs().max()) <= 2.0 ** -22 * 2.0
