@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) sp_tridiag_cluster_kernel(cons
     // the square root comes from the reciprocal square root; v^T v / 2 = ||x||^2 + |x_0| ||x||
     double alpha = 0.0, half = 0.0;
     v0 = 0.0;
-    if (nx2 > 1.0e-290) {                                     // below: treated as a zero column (H = I)
+    if (nx2 > 1.0e-140) {                                     // below: treated as a zero column (H = I), of a matrix of trace 1; beta^2 stays finite
       const double nx = nx2 * rsqrt(nx2);
       alpha = -copysign(nx, x0);
       v0 = x0 - alpha;
