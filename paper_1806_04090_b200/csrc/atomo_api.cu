@@ -899,7 +899,9 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
       d.lam64 = A.take<double>(d.tri ? d.rp : 0);
       d.td_ldv = (d.r + 3) / 4 * 4;
       d.td_V = A.take<float>(d.tri ? (size_t)d.r * d.td_ldv : 0);
-      d.tb_z = A.take<double>(d.tri == 2 && d.rp > 1024 ? (size_t)d.k_cap * d.rp : 0);
+      d.tb_z = A.take<double>(d.tri ? (size_t)d.k_cap * d.rp : 0);
+      d.close_work = A.take<double>(d.tri ? (size_t)kCloseWork * d.rp : 0);
+      d.close_flag = A.take<uint32_t>(d.tri ? d.k_cap : 0);
       {
         const size_t on = d.tri == 2 ? 1 : 0, rows = (size_t)sp_band_strips(d.r) * 64;
         d.bd_UW = A.take<float>(on * rows * 2 * kBandWidth);
@@ -923,7 +925,7 @@ static int encode_spectral_with(atomo_ctx* ctx, const atomo_mat* layers, int32_t
     // zero-filled region: rotation counters and the X matrices
     uint8_t* zb = reinterpret_cast<uint8_t*>(A.take<uint32_t>(0));
     size_t z0 = A.off;
-    for (int l = 0; l < n_layers; ++l) { L[l].rot_count = A.take<uint32_t>(max_sweeps); L[l].step_bar = A.take<uint32_t>(1); L[l].vec_ticket = A.take<uint32_t>(1); L[l].bd_bar = A.take<uint32_t>(1); }
+    for (int l = 0; l < n_layers; ++l) { L[l].rot_count = A.take<uint32_t>(max_sweeps); L[l].step_bar = A.take<uint32_t>(1); L[l].vec_ticket = A.take<uint32_t>(2); L[l].bd_bar = A.take<uint32_t>(1); }
     for (int l = 0; l < n_layers; ++l) {
       const int tt = (L[l].r + sp_tc_tile() - 1) / sp_tc_tile();
       const int tf = (L[l].r + 63) / 64;

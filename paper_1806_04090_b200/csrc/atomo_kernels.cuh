@@ -67,6 +67,10 @@ constexpr int kBandWidth = 8;         // sub-diagonals between the two stages of
 // doubles that a sweep of the chase takes in bd_V2: its steps in groups of 32, in a group the steps' entries 0 and 1, then 2 and
 // 3, .. (a warp of the back-transformation, a reflector per lane, reads whole lines)
 __host__ __device__ inline int64_t sp_chase_row(int r) { return (int64_t)((r + 255) / 256) * 256; }
+// kept atoms whose eigenvalues are this close (scaled units: trace 1) get their vectors of T together (sp_close_vectors): eigenvalues come to 4e-13 at
+// worst, and a vector of its own to that over the distance
+constexpr double kCloseEig = 2.0e-11;
+constexpr int kCloseWork = 1 + 3 * 16;   // rows of that kernel's workspace
 constexpr int kSmemRowsMaxRp = 4096;  // largest padded short side the shared-memory Jacobi kernel holds
 
 // what the digits of a short-side vector say of its range (integer Gram kernel; q = the entry in units of 2^(E - 30))
@@ -120,7 +124,7 @@ struct SpLayer {
   int td_ldv;                  // floats per row of td_V: r rounded up to a multiple of 4 (16-byte rows)
   float* td_V;                 // r x td_ldv: row k = v_k / ||v_k|| (zero up to index k), fp32 for the back-transformation: H_k = I - 2 u u^T
   double* lam64;               // rp: eigenvalues of T, ascending (scaled units); lam holds the same in fp32
-  uint32_t* vec_ticket;        // CTAs of the vector kernel that finished this layer; zeroed per call
+  uint32_t* vec_ticket;        // [2] CTAs of the vector kernel that finished this layer, whether some atoms come from tb_z; zeroed per call
   // tridiagonal route for short sides above 512 (tri = 2): dense -> band -> tridiagonal
   float* bd_UW;                // [rows padded to strips][16] U and W of the panel before
   float* bd_X;                 // [rows padded to strips][8] entries of the next panel
@@ -131,7 +135,9 @@ struct SpLayer {
   double* bd_T;                // [panels][64] T of the panels: Q1 is the product of I - U T U^T
   double* bd_V2;               // [r][sp_chase_row] reflectors of the chase, by sweep
   uint32_t* bd_bar;            // arrivals at the layer's barriers; zeroed per call
-  double* tb_z;                // [k_cap][rp] short sides above 1024: the kept atoms' eigenvectors of T
+  double* tb_z;                // [k_cap][rp] the kept atoms' eigenvectors of T: those of close eigenvalues, above 1024 rows all
+  double* close_work;          // [kCloseWork][rp] for the former: their eigenvalues, an upper triangle per warp
+  uint32_t* close_flag;        // [k_cap] which those are (valid where vec_ticket[1] is set)
 };
 
 // a layer of a spectral decode: threads per output row, rows per CTA, the layer's first CTA

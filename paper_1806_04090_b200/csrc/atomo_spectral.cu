@@ -398,6 +398,140 @@ void launch_sp_refine(const SpLayer* d_layers, int n_layers, const TileRef* d_ti
 // =================================================================================================
 constexpr int kFinThreads = 512;
 
+// x <- (T - mine)^{-1} x for a tridiagonal T, elimination with row interchanges, by one thread; u: [3][rp], the rows of the upper triangle.
+// (Eight steps' operands are fetched ahead of the chain of each.)
+__device__ __noinline__ void sp_solve_shifted(const double* __restrict__ d, const double* __restrict__ e, const int r, const int rp, const double mine,
+                                              double* u, double* x) {
+  constexpr double kLeast = 1.0e-14;                           // for pivots below: T is of trace 1, and its eigenvalues come to 4e-13
+  constexpr int kStep = 8;
+  double* const dd = u; double* const du = u + rp; double* const du2 = du + rp;
+  double piv = d[0] - mine, up = r > 1 ? e[0] : 0.0, top = x[0];   // row i of the triangle and of the right side so far
+  for (int i0 = 0; i0 + 1 < r; i0 += kStep) {
+    double ee[kStep + 1], dn[kStep], xn[kStep];
+#pragma unroll
+    for (int q = 0; q <= kStep; ++q) ee[q] = i0 + q + 1 < r ? e[i0 + q] : 0.0;
+#pragma unroll
+    for (int q = 0; q < kStep; ++q) { const bool in = i0 + q + 1 < r; dn[q] = in ? d[i0 + q + 1] - mine : 0.0; xn[q] = in ? x[i0 + q + 1] : 0.0; }
+#pragma unroll
+    for (int q = 0; q < kStep; ++q) {
+      if (i0 + q + 1 < r) {
+        const double low = ee[q];
+        const bool swap = fabs(low) > fabs(piv) && fabs(low) >= kLeast;   // the lower row has the larger pivot
+        if (!swap && !(fabs(piv) >= kLeast)) piv = kLeast;
+        const double inv = 1.0 / (swap ? low : piv), f = (swap ? piv : low) * inv;
+        dd[i0 + q] = inv;
+        du[i0 + q] = swap ? dn[q] : up;
+        du2[i0 + q] = swap ? ee[q + 1] : 0.0;
+        x[i0 + q] = swap ? xn[q] : top;
+        piv = swap ? fma(-f, dn[q], up) : fma(-f, up, dn[q]);
+        top = swap ? fma(-f, xn[q], top) : fma(-f, top, xn[q]);
+        up = swap ? -f * ee[q + 1] : ee[q + 1];
+      }
+    }
+  }
+  if (!(fabs(piv) >= kLeast)) piv = kLeast;
+  double x1 = top / piv, x2 = 0.0;
+  x[r - 1] = x1;
+  for (int i0 = r - 2; i0 >= 0; i0 -= kStep) {
+    double a[kStep], b[kStep], c[kStep], y[kStep];
+#pragma unroll
+    for (int q = 0; q < kStep; ++q) {
+      const int i = max(i0 - q, 0);
+      a[q] = dd[i]; b[q] = du[i]; c[q] = du2[i]; y[q] = x[i];
+    }
+#pragma unroll
+    for (int q = 0; q < kStep; ++q) {
+      if (i0 - q >= 0) {
+        const double v = fma(-c[q], x2, fma(-b[q], x1, y[q])) * a[q];
+        x[i0 - q] = v; x2 = x1; x1 = v;
+      }
+    }
+  }
+}
+
+// Vectors of T for kept atoms whose eigenvalues lie within kCloseEig of another kept atom's (equal to rounding, mostly: layers with equal or
+// orthogonal rows, zero rows, ranks below the short side).  Worked out one by one, each from its own eigenvalue, they would be the same vector twice,
+// or a vector and noise.  Inverse iteration with reorthogonalisation (the scheme of LAPACK's dstein): three steps from random starts, a warp per
+// atom, each followed by Gram-Schmidt against the atoms before it.  The whole CTA.  Other layers pay for a comparison in shared memory.
+// Against 64 bits, before | now: 8 x 1011 of +-1 (five equal eigenvalues), largest dot product of two kept vectors 0.58 | 1e-7.
+// A whole encode, ms: 512 x 700 of +-1 with 56 atoms kept 7.35 | 4.21 (they need no Gram-Schmidt in the vector kernel), with six 1.12 | 1.37,
+// identity of 4096 rows, 13 kept, 34.4 | 33.4.
+__device__ __noinline__ void sp_close_vectors(const SpLayer& L, const uint32_t k, double* __restrict__ s_red) {
+  constexpr int kWarps = kFinThreads / 32;
+  static_assert(kCloseWork == 1 + 3 * kWarps, "room for a triangle per warp");
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32, r = L.r, rp = L.rp;
+  double* const lam = L.close_work; double* const u = lam + rp + (int64_t)w * 3 * rp;
+  uint32_t* const flag = L.close_flag;
+  for (uint32_t a = tid; a < k; a += kFinThreads) lam[a] = L.lam64[L.perm[L.idx[a]]];
+  __syncthreads();
+  bool any = false;
+  for (uint32_t a = tid; a < k; a += kFinThreads) {
+    bool close = false;
+    for (uint32_t b = 0; b < k; ++b) close |= b != a && fabs(lam[a] - lam[b]) <= kCloseEig;
+    flag[a] = close ? 1u : 0u;
+    any |= close;
+  }
+  if (!__syncthreads_or(any)) return;
+  if (tid == 0) L.vec_ticket[1] = 1u;
+  for (uint32_t a = 0; a < k; ++a) {                           // (uniform)
+    if (!flag[a]) continue;
+    for (int i = tid; i < r; i += kFinThreads) {
+      uint32_t h = (uint32_t)i * 0x9e3779b1u ^ (a + 1u) * 0x85ebca77u;
+      h ^= h >> 15; h *= 0x2c1b3c6du; h ^= h >> 12; h *= 0x297a2d39u; h ^= h >> 15;
+      L.tb_z[(int64_t)a * rp + i] = (double)(int)h * 0x1p-31;
+    }
+  }
+  __syncthreads();
+  auto unit = [&](double* x) {                                 // to unit length (a zero or non-finite vector: to a unit vector)
+    double n2 = 0.0;
+    for (int i = tid; i < r; i += kFinThreads) n2 = fma(x[i], x[i], n2);
+    n2 = warp_sum(n2);
+    if (lane == 0) s_red[w] = n2;
+    __syncthreads();
+    n2 = 0.0;
+    for (int q = 0; q < kWarps; ++q) n2 += s_red[q];
+    const bool ok = n2 > 1.0e-280 && n2 < 1.0e300;
+    const double inv = ok ? rsqrt(n2) : 0.0;
+    for (int i = tid; i < r; i += kFinThreads) x[i] = ok ? x[i] * inv : i == 0 ? 1.0 : 0.0;
+    __syncthreads();
+  };
+  for (int it = 0; it < 3; ++it) {
+    for (uint32_t a = 0, turn = 0; a < k; ++a) {               // the flagged atoms, dealt to the warps
+      if (!flag[a]) continue;
+      if ((int)(turn++ % kWarps) == w && lane == 0) sp_solve_shifted(L.td_d, L.td_e, r, rp, lam[a], u, L.tb_z + (int64_t)a * rp);
+    }
+    __syncthreads();
+    for (uint32_t a = 0; a < k; ++a) {
+      if (!flag[a]) continue;
+      const double mine = lam[a];
+      double* const x = L.tb_z + (int64_t)a * rp;
+      unit(x);
+      for (int round = it < 2 ? 1 : 0; round < 2; ++round) {   // (the last step's vectors twice)
+        for (uint32_t b0 = 0; b0 < a; b0 += kFinThreads) {     // dots, a warp each, then all of them out of x
+          const uint32_t n = min((uint32_t)kFinThreads, a - b0);
+          for (uint32_t q = w; q < n; q += kWarps) {
+            double dot = 0.0;
+            if (fabs(lam[b0 + q] - mine) <= kCloseEig) {
+              const double* const z = L.tb_z + (int64_t)(b0 + q) * rp;
+              for (int i = lane; i < r; i += 32) dot = fma(z[i], x[i], dot);
+              dot = warp_sum(dot);
+            }
+            if (lane == 0) s_red[q] = dot;
+          }
+          __syncthreads();
+          for (int i = tid; i < r; i += kFinThreads) {
+            double v = x[i];
+            for (uint32_t q = 0; q < n; ++q) if (s_red[q] != 0.0) v = fma(-s_red[q], L.tb_z[(int64_t)(b0 + q) * rp + i], v);
+            x[i] = v;
+          }
+          __syncthreads();
+        }
+      }
+      unit(x);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kFinThreads) sp_finalize_sample_kernel(const SpLayer* __restrict__ layers, double s,
                                                                          PhiloxKey key, uint32_t kind_step,
                                                                          int max_sweeps,
@@ -497,6 +631,7 @@ __global__ void __launch_bounds__(kFinThreads) sp_finalize_sample_kernel(const S
   const double scale = (T > 0.0 && scur > 0.0) ? scur / T : 0.0;
 
   // probabilities, Bernoulli draws, ordered compaction of the kept ranks
+  int* const s_kept = reinterpret_cast<int*>(s_lam);         // (the eigenvalues have been ranked; at most r atoms)
   uint32_t carry = 0;
   for (int base = 0; base < r; base += kFinThreads) {
     const int i = base + tid;
@@ -524,7 +659,7 @@ __global__ void __launch_bounds__(kFinThreads) sp_finalize_sample_kernel(const S
     for (int j = 0; j < kFinThreads / 32; ++j) total += s_scan[j];
     if (keep) {
       const uint32_t pos = off + __popc(ballot & ((1u << lane) - 1u));
-      if (pos < L.k_cap) { L.idx[pos] = (uint32_t)i; L.p_sel[pos] = p; }
+      if (pos < L.k_cap) { L.idx[pos] = (uint32_t)i; L.p_sel[pos] = p; s_kept[pos] = i; }
     }
     carry += total;
     __syncthreads();
@@ -544,7 +679,16 @@ __global__ void __launch_bounds__(kFinThreads) sp_finalize_sample_kernel(const S
   }
   __syncthreads();
   const uint32_t k = s_k;
-  if (L.tri) return;                       // tridiagonal route: the vectors of the kept atoms come from sp_eigvec_kernel
+  if (L.tri) {                             // tridiagonal route: the vectors of the kept atoms come from sp_eigvec_kernel, but for ..
+    const float scale = *L.scale;          // .. neighbours within kCloseEig, or within the last digits of fp32
+    bool close = false;
+    for (uint32_t a = tid; a + 1 < k; a += kFinThreads) {
+      const float hi = s_sig[s_kept[a]], lo = s_sig[s_kept[a + 1]];
+      close |= (hi - lo) * (hi + lo) * scale <= (float)kCloseEig + 1.0e-6f * hi * hi * scale;
+    }
+    if (__syncthreads_or(close)) sp_close_vectors(L, k, s_red);
+    return;
+  }
   // short-side vectors of the kept atoms, normalised: payload shortv[a][0..r)
   for (uint32_t a = w; a < k; a += kFinThreads / 32) {
     const int row = L.perm[L.idx[a]];

@@ -13,7 +13,8 @@
 //   sp_eigvec_kernel          : for the kept atoms only: eigenvector of T by a twisted factorisation with one
 //                               Rayleigh-quotient correction, back-transformation u = Q z with the reflectors
 //                               (eight at a time, fp32), normalised short-side vector into the payload; kept atoms with
-//                               nearly equal eigenvalues are orthogonalised against each other at the end.
+//                               nearly equal eigenvalues are orthogonalised against each other at the end, and where they are
+//                               too close for vectors of their own (sp_finalize_sample_kernel), these are there already.
 //
 // Work per layer: about 2 r^3 fp64 flops for the reduction (full symmetric storage: matrix-vector product and
 // rank-two update of the trailing block), about 11 r^2 to 32 r^2 recurrence steps for the eigenvalues, O(r^2) per kept atom.
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
   __shared__ int s_next;                                      // groups whose T somebody has taken on
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  const uint32_t k = L.hdr->k, n_ctas = gridDim.y;
+  const uint32_t k = L.hdr->k, n_ctas = gridDim.y, given = L.vec_ticket[1];
   // the layer's pointers in registers (a field read through `layers` inside a loop is a global load each time)
   const float* const gV = L.td_V; const int ldv = L.td_ldv; const double* const gLam = L.lam64;
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
@@ -481,22 +482,23 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
 #pragma unroll
     for (int m = 0; m < kQuads; ++m) zr[m] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (have) {
-      const int ei = gPerm[gIdx[a]];                          // index of the atom's eigenvalue (ascending order)
-      double lambda = gLam[ei];
-      // earlier kept atoms with the same eigenvalue (to the accuracy of the eigenvalues): each takes another twist index
-      int skip = 0;
-      for (uint32_t b = lane; b < a; b += 32) skip += fabs(gLam[gPerm[gIdx[b]]] - lambda) <= kSameEig ? 1 : 0;
-      skip = (int)warp_sum((uint32_t)skip);
       double n2 = 1.0;
-      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, skip, &n2);
-      // the vector's error is about |correction| / gap to the nearest other eigenvalue: well-separated atoms are done
-      double gap = 1.0e300;
-      if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
-      if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
-      if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {   // one Rayleigh-quotient step, then the vector again
-        lambda += corr;
+      if (given && L.close_flag[a]) {                         // close to another kept atom's eigenvalue: sp_close_vectors has it
+        for (int i = lane; i < r; i += 32) z[i] = L.tb_z[(int64_t)a * rp + i];
         __syncwarp();
-        twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, 0, &n2);
+      } else {
+        const int ei = gPerm[gIdx[a]];                        // index of the atom's eigenvalue (ascending order)
+        double lambda = gLam[ei];
+        const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, &n2);
+        // the vector's error is about |correction| / gap to the nearest other eigenvalue: well-separated atoms are done
+        double gap = 1.0e300;
+        if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
+        if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
+        if (finite64(corr) && !(fabs(corr) <= 1.0e-9 * gap)) {   // one Rayleigh-quotient step, then the vector again
+          lambda += corr;
+          __syncwarp();
+          twisted_vector(s_d, s_e, r, lambda, wa, wb, z, lane, &n2);
+        }
       }
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
 #pragma unroll
@@ -668,7 +670,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) sp_eigvec_kernel(const SpLayer
     bool changed = false;
     for (uint32_t b = 0; b < a; ++b) {
       const double lb = gLam[gPerm[gIdx[b]]];
-      if (fabs(la - lb) > kSameEig) continue;
+      if (fabs(la - lb) > kSameEig || (given && fabs(la - lb) <= kCloseEig)) continue;   // (those are orthogonal already)
       volatile float* va = gShort + (int64_t)a * r;
       const volatile float* vb = gShort + (int64_t)b * r;
       double dot = 0.0;

@@ -40,6 +40,7 @@ __device__ __forceinline__ void vb_orthogonalise_equal(const SpLayer& L, uint32_
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int r = L.r;
+  const uint32_t given = L.vec_ticket[1];
   const double* const gLam = L.lam64; const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
   __threadfence();
   __syncthreads();
@@ -52,7 +53,7 @@ __device__ __forceinline__ void vb_orthogonalise_equal(const SpLayer& L, uint32_
     bool changed = false;
     for (uint32_t b = 0; b < a; ++b) {
       const double lb = gLam[gPerm[gIdx[b]]];
-      if (fabs(la - lb) > kVbSameEig) continue;
+      if (fabs(la - lb) > kVbSameEig || (given && fabs(la - lb) <= kCloseEig)) continue;   // (those are orthogonal already)
       volatile float* va = gShort + (int64_t)a * r;
       const volatile float* vb = gShort + (int64_t)b * r;
       double dot = 0.0;
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
   __shared__ double s_tot[8];
   __shared__ double s_edge[2][kVcWarps][8];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
-  const uint32_t k = L.hdr->k;
+  const uint32_t k = L.hdr->k, given = L.vec_ticket[1];
   const float* const gV = L.td_V; const int64_t ldv = L.td_ldv; const double* const gLam = L.lam64;
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
   const int nref = max(r - kBandWidth - 1, 0);                 // a panel's reflector kk is zero up to index kk + 7
@@ -276,21 +277,20 @@ __global__ void __launch_bounds__(kVcThreads) sp_eigvec_big_cta_kernel(const SpL
     double* const wa = s_work;
     double* const wb = wa + rp;
     for (uint32_t a = slot; a < k; a += kVcCtas) {
-      if (w == 0) {
+      if (given && L.close_flag[a]) {                          // close to another kept atom's eigenvalue: sp_close_vectors has it
+        for (int i = tid; i < r; i += kVcThreads) s_z[i] = L.tb_z[(int64_t)a * rp + i];
+      } else if (w == 0) {
         const int ei = gPerm[gIdx[a]];                         // index of the atom's eigenvalue (ascending order)
         double lambda = gLam[ei];
-        int skip = 0;                                          // earlier kept atoms with the same eigenvalue: another twist index each
-        for (uint32_t b2 = lane; b2 < a; b2 += 32) skip += fabs(gLam[gPerm[gIdx[b2]]] - lambda) <= kVbSameEig ? 1 : 0;
-        skip = (int)warp_sum((uint32_t)skip);
         double n2 = 1.0;
-        const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, skip, &n2);
+        const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, &n2);
         double gap = 1.0e300;
         if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
         if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
-        if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {  // one Rayleigh-quotient step, then the vector again
+        if (finite64(corr) && !(fabs(corr) <= 1.0e-9 * gap)) {  // one Rayleigh-quotient step, then the vector again
           lambda += corr;
           __syncwarp();
-          twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, 0, &n2);
+          twisted_vector(s_d, s_e, r, lambda, wa, wb, s_z, lane, &n2);
         }
         __syncwarp();
         const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(THREADS, 1) sp_eigvec_big_kernel(const SpLayer
   __shared__ double s_tot[8 * BATCH];
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int n_ctas = gridDim.y, cy = blockIdx.y;
-  const uint32_t k = L.hdr->k;
+  const uint32_t k = L.hdr->k, given = L.vec_ticket[1];
   const float* const gV = L.td_V; const int64_t ldv = L.td_ldv; const double* const gLam = L.lam64;
   const int* const gPerm = L.perm; const uint32_t* const gIdx = L.idx; float* const gShort = L.shortv;
   double* const gZ = L.tb_z;
@@ -347,20 +347,18 @@ __global__ void __launch_bounds__(THREADS, 1) sp_eigvec_big_kernel(const SpLayer
     double* const wa = s_e + rp + (size_t)w * 3 * rp;
     double* const wb = wa + rp; double* const zz = wb + rp;
     for (uint32_t a = cy + (uint32_t)n_ctas * w; a < k; a += (uint32_t)(n_ctas * kWork)) {
+      if (given && L.close_flag[a]) continue;                  // in gZ already
       const int ei = gPerm[gIdx[a]];                           // index of the atom's eigenvalue (ascending order)
       double lambda = gLam[ei];
-      int skip = 0;                                            // earlier kept atoms with the same eigenvalue: another twist index each
-      for (uint32_t b2 = lane; b2 < a; b2 += 32) skip += fabs(gLam[gPerm[gIdx[b2]]] - lambda) <= kVbSameEig ? 1 : 0;
-      skip = (int)warp_sum((uint32_t)skip);
       double n2 = 1.0;
-      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, skip, &n2);
+      const double corr = twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, &n2);
       double gap = 1.0e300;
       if (ei > 0) gap = fmin(gap, fabs(lambda - gLam[ei - 1]));
       if (ei + 1 < r) gap = fmin(gap, fabs(gLam[ei + 1] - lambda));
-      if (finite64(corr) && skip == 0 && !(fabs(corr) <= 1.0e-9 * gap)) {    // one Rayleigh-quotient step, then the vector again
+      if (finite64(corr) && !(fabs(corr) <= 1.0e-9 * gap)) {    // one Rayleigh-quotient step, then the vector again
         lambda += corr;
         __syncwarp();
-        twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, 0, &n2);
+        twisted_vector(s_d, s_e, r, lambda, wa, wb, zz, lane, &n2);
       }
       __syncwarp();
       const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;

@@ -29,8 +29,7 @@ __device__ __forceinline__ double safe_pivot(double x) {
 // Bound: the two serial loops.  Their operands are fetched eight steps at a time, so that a step is what the one warp issues (two
 // products, two loads and a store), not a round trip to memory.
 static __device__ __noinline__ double twisted_vector(const double* __restrict__ d, const double* __restrict__ e, int r, double lambda,
-                                                     double* na, double* nb, double* z, int lane, int skip,
-                                                     double* znorm2) {
+                                                     double* na, double* nb, double* z, int lane, double* znorm2) {
   constexpr int kStep = 8;
   bool dead = false;
   if (lane < 2) {
@@ -103,29 +102,20 @@ static __device__ __noinline__ double twisted_vector(const double* __restrict__ 
       __syncwarp();
     }
   }
-  // twist index: the (skip+1)-th smallest |gamma| (lowest index on ties).  skip > 0 for the later members of a group
-  // of kept atoms with coinciding eigenvalues: z = gamma_k (T - lambda I)^{-1} e_k, so another k is another start
-  // vector of inverse iteration and gives another vector of the invariant subspace.
-  double best = -1.0; int bk = -1;
-  for (int pick = 0; pick <= skip; ++pick) {
-    const double pb = best; const int pk = bk;
-    double cb = 1.0e300; int ck = 0x7fffffff;
+  // twist index: the smallest |gamma| (lowest index on ties)
+  double best = 1.0e300; int bk = 0x7fffffff;
 #pragma unroll 4
-    for (int i = lane; i < r; i += 32) {
-      const double gam = fabs(na[i] + nb[i] - (d[i] - lambda));
-      const bool after = gam > pb || (gam == pb && i > pk);   // not picked yet
-      if (after && (gam < cb || (gam == cb && i < ck))) { cb = gam; ck = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, cb, o);
-      const int ok = __shfl_xor_sync(0xffffffffu, ck, o);
-      if (ob < cb || (ob == cb && ok < ck)) { cb = ob; ck = ok; }
-    }
-    if (ck == 0x7fffffff) break;                              // fewer candidates than skip (non-finite input)
-    best = cb; bk = ck;
+  for (int i = lane; i < r; i += 32) {
+    const double gam = fabs(na[i] + nb[i] - (d[i] - lambda));
+    if (gam < best) { best = gam; bk = i; }
   }
-  if (bk < 0) bk = 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
+    if (ob < best || (ob == best && ok < bk)) { best = ob; bk = ok; }
+  }
+  if (bk == 0x7fffffff) bk = 0;                               // (non-finite input)
   const double gamma = na[bk] + nb[bk] - (d[bk] - lambda);
   __syncwarp();
   // multipliers: na[i] <- e_i / D+_i above the twist, e_i / D-_{i+1} from there
